@@ -173,21 +173,15 @@ int gcn_admm_dense_product_tn(gcn_admm* h, const float* A, const float* B, float
  * Same result as gcn_admm_propagate, for code that is not allowed to reserve device memory when it
  * calls: a real-time loop whose memory budget was fixed at start-up, a plug-in running inside
  * someone else's memory pool, a section between begin and end of a stream capture where cudaMalloc is
- * illegal.  gcn_admm_propagate stages x and the result in two padded matrices that it allocates and
- * frees on every call; this variant keeps those two matrices in an array compiled into the library
- * (32 MiB of device memory on every GPU that loads the library, held until the process ends), and
- * calls neither cudaMalloc nor cudaFree nor any allocating routine.
+ * illegal.  gcn_admm_propagate stages host buffers and may enlarge a workspace of the handle (the sums of
+ * long rows cut into items, for a matrix wider than every layer); this variant reads x and writes out
+ * where they are, walks those rows whole instead, and calls no allocating routine.
  *  - x and out are DEVICE pointers to n x width floats, original node order; out may not alias x.
  *  - its launches are counted by gcn_admm_launches but never timed by gcn_admm_profile (event
  *    creation reserves memory), whether profiling is on or off.
  *  - limit: n * (width rounded up to a multiple of 4) <= 4,194,304; larger sizes are refused with
  *    GCN_ADMM_ERR_ARG and a message naming the limit.
- *  - the first call on a device looks up the device address of the array (one runtime query, no
- *    allocation); make that first call before any stream capture begins.
- *  - the work is enqueued on the handle's stream and the call returns without synchronising.
- *  - all calls, from every handle, share the one array, which keeps whatever the last call left in
- *    it; each call overwrites all it later reads, so nothing needs clearing, but two calls whose
- *    kernels overlap on the GPU (different streams, different handles) race on it: serialise them. */
+ *  - the work is enqueued on the handle's stream and the call returns without synchronising. */
 int gcn_admm_propagate_static(gcn_admm* h, const float* x, int width, float* out);
 
 /* ---- index tables (Section 2; Appendix A first paragraph) ------------------------------------

@@ -190,6 +190,7 @@ struct gcn_admm {
   unsigned short* d_col_comm = nullptr;   // community of every stored column
   // rows too long for one warp, cut into items (see gcn_admm_host::LongRowTables)
   int4 *d_items = nullptr, *d_split = nullptr, *d_long_rows = nullptr;
+  int *d_item_row = nullptr, *d_row_done = nullptr;   // long row of every item; per long row a counter of finished items
   int n_items = 0, n_split = 0, n_long = 0, long_len = 0;
   float* item_sums = nullptr;             // n_items x max_ld
   size_t item_sums_elems = 0;
@@ -252,43 +253,87 @@ struct gcn_admm {
     char name[48];
     std::snprintf(name, sizeof name, "spmm@%d", ldx);
     Scope sc(this, name, 1, 4.0 * gi.nnz + 8.0 * n + 8.0 * (double)n * ldx, 2.0 * (double)gi.nnz * ldx);
-    // Long rows go as items unless the operand is wider than the item buffer was sized for (a
-    // caller's matrix wider than every layer): then they are walked whole, slower but the same sums.
-    const bool cut = n_items > 0 && (size_t)n_items * ldx <= item_sums_elems;
-    spmm_launch(d_row_ptr, d_col, d_dinv, d_row_order, (int)n, d_items, cut ? n_items : 0, cut ? long_len : INT_MAX, x, out, ldx);
-    if (cut) {
-      gk::k_spmm_long_rows<<<(unsigned)n_long, 64, 0, stream>>>(d_long_rows, reinterpret_cast<const float4*>(item_sums),
-                                                                reinterpret_cast<float4*>(out), ldx / 4);
+    spmm_tables<4, false>(gather_graph(ldx), x, out, ldx / 4);
+  }
+
+  // out = A~ x for dense n x width device matrices in the caller's row order, in vectors as wide as the width and
+  // both addresses allow.
+  void propagate_dense(const float* x, int width, float* out) {
+    char name[48];
+    std::snprintf(name, sizeof name, "spmm@%d", ldpad(width));
+    Scope sc(this, name, 1, 4.0 * gi.nnz + 8.0 * n + 8.0 * (double)n * width, 2.0 * (double)gi.nnz * width);
+    const GatherGraph g = gather_graph(ldpad(width));
+    const uintptr_t low = reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(out) | ((uintptr_t)width * sizeof(float));
+    if ((low & 15) == 0) spmm_tables<4, true>(g, x, out, width / 4);
+    else if ((low & 7) == 0) spmm_tables<2, true>(g, x, out, width / 2);
+    else spmm_tables<1, true>(g, x, out, width);
+  }
+
+  // The handle's graph for a propagation of ldw padded columns.  Long rows go as items unless the operand is
+  // wider than the item buffer (a caller's matrix wider than every layer, where nothing may be allocated): then
+  // they are walked whole, slower but the same sums.
+  struct GatherGraph {
+    const int *row_ptr, *col, *row_order, *perm;
+    const float* dinv;
+    const int4 *items, *rows;
+    const int* item_row;
+    int* row_done;
+    int n, n_items, n_long, long_len;
+  };
+  GatherGraph gather_graph(int ldw) const {
+    const bool cut = n_items > 0 && (size_t)n_items * ldw <= item_sums_elems;
+    return GatherGraph{d_row_ptr, d_col, d_row_order, d_perm, d_dinv, d_items, d_long_rows, d_item_row, d_row_done,
+                       (int)n, cut ? n_items : 0, cut ? n_long : 0, cut ? long_len : INT_MAX};
+  }
+  // Room for the items' sums at ldw padded columns (a workspace the handle keeps).
+  void grow_item_sums(int ldw) {
+    const size_t need = (size_t)n_items * ldw;
+    if (need <= item_sums_elems) return;
+    float* bigger = alloc<float>(need);   // the old one stays in `owned` until destroy: kernels in flight may hold it
+    item_sums = bigger;
+    item_sums_elems = need;
+  }
+
+  // The propagation kernels on a graph given by its tables (the handle's own, or a rank's local part of it); x and
+  // out have ldv vectors of VEC floats per row.
+  template <int VEC, bool MAPPED>
+  void spmm_tables(const GatherGraph& g, const float* xf, float* outf, int ldv) {
+    using T = typename gk::Vec<VEC>::T;
+    const T* x = reinterpret_cast<const T*>(xf);
+    T *out = reinterpret_cast<T*>(outf), *scratch = reinterpret_cast<T*>(item_sums);
+    const int ld4 = (int)cdiv((long long)ldv * VEC, 4);
+    const long long units = (long long)g.n + g.n_items;
+#define WIDE(NV4, UN)                                                                                                     \
+  gk::k_spmm_wide<VEC, 4 / VEC * (NV4), UN, MAPPED><<<(unsigned)cdiv(units * 32, 64), 64, 0, stream>>>( \
+      g.row_ptr, g.col, g.dinv, g.perm, g.items, g.n, g.n_items, g.long_len, x, out, ldv, scratch)
+#define SETS(CL, EP, UN)                                                                                                  \
+  gk::k_spmm_sets<VEC, 4 / VEC, CL, EP, UN, MAPPED><<<(unsigned)cdiv(units * ((CL) * (EP)), 128), 128, 0, stream>>>( \
+      g.row_ptr, g.col, g.dinv, g.perm, g.items, g.n, g.n_items, g.long_len, x, out, ldv, scratch, g.row_order, gk::ItemRows{g.rows, g.item_row, g.row_done})
+    // Sets of entries per row: as many as the warp holds while the grid is then still small (latency counts), fewer
+    // where the rows alone fill the chip several times over and the lanes of half-empty sets would only cost issue
+    // slots.  Lines between the measured sizes 0.2 / 1.4 / 20 M lanes (columns x rows); the rule reads the handle's n, so a
+    // rank's part of a graph is summed in the order of the whole.
+    const long long lanes = n * (ld4 <= 1 ? 1 : ld4 <= 2 ? 2 : ld4 <= 4 ? 4 : ld4 <= 8 ? 8 : 16);
+    if (ld4 <= 1) {
+      if (lanes <= 60000) SETS(1, 16, 4); else if (lanes <= 500000) SETS(1, 8, 4); else SETS(1, 4, 4);
+    } else if (ld4 <= 2) {
+      if (lanes <= 120000) SETS(2, 8, 4); else if (lanes <= 1000000) SETS(2, 4, 4); else SETS(2, 2, 4);
+    } else if (ld4 <= 4) {
+      if (lanes <= 240000) SETS(4, 8, 4); else SETS(4, 2, 4);
+    } else if (ld4 <= 8) {
+      if (lanes <= 480000) SETS(8, 4, 8); else SETS(8, 1, 8);
+    } else if (ld4 <= 16) {
+      if (lanes <= 960000) SETS(16, 2, 8); else SETS(16, 1, 8);
+    } else if (ld4 <= 32) WIDE(1, 4);
+    else WIDE(2, 2);   // two neighbours in flight per lane beat four (fewer registers, more warps): measured
+#undef WIDE
+#undef SETS
+    CU(cudaGetLastError());
+    if (ld4 > 16 && g.n_long > 0) {
+      gk::k_spmm_long_rows<T, MAPPED><<<(unsigned)g.n_long, 64, 0, stream>>>(g.rows, scratch, out, ldv, g.perm);
       CU(cudaGetLastError());
       ++launches;   // booked with the propagation it completes
     }
-  }
-
-  // The propagation kernel on a graph given by its tables (the handle's own, or a rank's local part of it):
-  // rows 0 .. nn-1 of out = A~ x, columns of `cl` index rows of x.  `order` lists the rows by falling length
-  // (used by the forms that put several rows in a warp).
-  void spmm_launch(const int* rp, const int* cl, const float* dv, const int* order, int nn, const int4* its, int items_used,
-                   int long_eff, const float* x, float* out, int ldx) {
-    const int ld4 = ldx / 4;
-    const float4* x4 = reinterpret_cast<const float4*>(x);
-    float4* o4 = reinterpret_cast<float4*>(out);
-    // 64-thread blocks: rows differ widely in length, small blocks keep the SMs evenly loaded.
-#define SPMM_CASE(G, V, UN)                                                                    \
-  {                                                                                            \
-    const long long threads = ((long long)nn + items_used) * (G);                              \
-    /* several rows per warp (G < 32): rows of equal length side by side */                     \
-    gk::k_spmm<G, V, UN, ((G) < 32)><<<(unsigned)cdiv(threads, 64), 64, 0, stream>>>(rp, cl, dv, x4, o4, nn, ld4, \
-        its, items_used, long_eff, reinterpret_cast<float4*>(item_sums), order);               \
-  }
-    if (ld4 <= 1) SPMM_CASE(1, 1, 4)
-    else if (ld4 <= 2) SPMM_CASE(2, 1, 4)
-    else if (ld4 <= 4) SPMM_CASE(4, 1, 8)
-    else if (ld4 <= 8) SPMM_CASE(8, 1, 8)
-    else if (ld4 <= 16) SPMM_CASE(16, 1, 8)
-    else if (ld4 <= 32) SPMM_CASE(32, 1, 4)
-    else SPMM_CASE(32, 2, 2)   // two neighbours in flight per lane beat four (fewer registers, more warps): measured
-#undef SPMM_CASE
-    CU(cudaGetLastError());
   }
 
   // C = A B.  B is handed over twice: row-major K x N (ldb) for the fp32-ALU kernels and K-major
@@ -987,6 +1032,12 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
       h->d_chunk_ptr_sorted = upload(h, sorted);
     }
     h->d_long_rows = reinterpret_cast<int4*>(upload(h, lt.rows));
+    std::vector<int> item_row(lt.items.size());
+    for (size_t r = 0; r < lt.rows.size(); ++r)
+      for (int k = 0; k < lt.rows[r].z; ++k) item_row[(size_t)(lt.rows[r].y + k)] = (int)r;
+    h->d_item_row = upload(h, item_row);
+    h->d_row_done = h->alloc<int>(lt.rows.size());
+    CU(cudaMemset(h->d_row_done, 0, std::max<size_t>(1, lt.rows.size()) * sizeof(int)));
   }
 
   const int L = n_layers;
@@ -1355,31 +1406,30 @@ int gcn_admm_predict(gcn_admm* h, float* logits, int* labels) {
 int gcn_admm_propagate(gcn_admm* h, const float* x, int width, float* out) {
   return guarded(h, [&] {
     if (!x || !out || width < 1 || width > kMaxWidth) throw Fail{GCN_ADMM_ERR_ARG, "bad argument"};
-    const int ldw = ldpad(width);
-    const size_t rows = (size_t)h->n;
     const bool dev_in = is_device_pointer(x), dev_out = is_device_pointer(out);
     if (dev_in != dev_out) throw Fail{GCN_ADMM_ERR_ARG, "x and out must both be host or both be device pointers"};
-    float *dense = nullptr, *a = nullptr, *b = nullptr;
+    h->grow_item_sums(ldpad(width));
+    if (dev_in) {
+      h->propagate_dense(x, width, out);
+      CU(cudaStreamSynchronize(h->stream));
+      return;
+    }
+    // host buffers: staged in two of the handle's scratch matrices (idle between calls), or, wider than those, in
+    // a pair allocated for the call
+    const size_t elems = (size_t)h->n * width, bytes = elems * sizeof(float);
+    const bool fits = width <= h->max_ld;
+    float *a = fits ? h->B0 : dalloc<float>(elems), *b = nullptr;
     try {
-      dense = dalloc<float>(rows * width);
-      a = dalloc<float>(rows * ldw);
-      b = dalloc<float>(rows * ldw);
-      CU(cudaMemcpyAsync(dense, x, rows * width * sizeof(float), dev_in ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
-                         h->stream));
-      gcn_admm::Scope sc(h, "permute_rows", 2, 16.0 * (double)h->n * width, 0.0);
-      gk::k_permute_rows<<<h->grid_for(h->n * ldw), 256, 0, h->stream>>>(dense, a, h->d_perm, h->n, width, ldw, 1);
-      CU(cudaGetLastError());
-      h->spmm(a, b, ldw);
-      gk::k_permute_rows<<<h->grid_for(h->n * ldw), 256, 0, h->stream>>>(b, dense, h->d_perm, h->n, width, ldw, 0);
-      CU(cudaGetLastError());
-      CU(cudaMemcpyAsync(out, dense, rows * width * sizeof(float), dev_out ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
-                         h->stream));
+      b = fits ? h->B1 : dalloc<float>(elems);
+      CU(cudaMemcpyAsync(a, x, bytes, cudaMemcpyHostToDevice, h->stream));
+      h->propagate_dense(a, width, b);
+      CU(cudaMemcpyAsync(out, b, bytes, cudaMemcpyDeviceToHost, h->stream));
       CU(cudaStreamSynchronize(h->stream));
     } catch (...) {
-      cudaFree(dense); cudaFree(a); cudaFree(b);
+      if (!fits) { cudaFree(a); cudaFree(b); }
       throw;
     }
-    cudaFree(dense); cudaFree(a); cudaFree(b);
+    if (!fits) { cudaFree(a); cudaFree(b); }
   });
 }
 
@@ -1453,53 +1503,20 @@ int gcn_admm_dense_product_tn(gcn_admm* h, const float* A, const float* B, float
 }
 
 // ---- propagation for callers that may not allocate ---------------------------------------------
-// The two padded staging matrices of gcn_admm_propagate live in one file-scope device array, so
-// this entry point reserves nothing at call time.  Every GPU that loads the library carries the
-// array (32 MiB) until the process exits.
-namespace {
-constexpr long long kStaticHalf = 4LL << 20;                       // floats per staging matrix
-static __device__ __align__(256) float g_propagate_scratch[2 * kStaticHalf];
-std::mutex g_scratch_mutex;
-float* g_scratch_addr[64] = {nullptr};
-
-// Device address of g_propagate_scratch on `device` (which must be current).  In host code the
-// array's name is only a handle for the runtime, never an address a kernel may be given.
-float* static_scratch(int device) {
-  if (device < 0 || device >= 64) throw Fail{GCN_ADMM_ERR_ARG, "device ordinal above 63"};
-  std::lock_guard<std::mutex> lock(g_scratch_mutex);
-  if (g_scratch_addr[device] == nullptr) {
-    float* ptr = nullptr;
-    CU(cudaGetSymbolAddress((void**)&ptr, g_propagate_scratch));
-    g_scratch_addr[device] = ptr;
-  }
-  return g_scratch_addr[device];
-}
-}  // namespace
-
 int gcn_admm_propagate_static(gcn_admm* h, const float* x, int width, float* out) {
   return guarded(h, [&] {
+    constexpr long long kStaticElems = 4LL << 20;
     if (!x || !out || width < 1 || width > kMaxWidth) throw Fail{GCN_ADMM_ERR_ARG, "bad argument"};
-    const int ldw = ldpad(width);
-    if ((long long)h->n * ldw > kStaticHalf)
-      throw Fail{GCN_ADMM_ERR_ARG, "n * padded width exceeds the static scratch of 4194304 floats per staging matrix"};
+    if ((long long)h->n * ldpad(width) > kStaticElems)
+      throw Fail{GCN_ADMM_ERR_ARG, "n * padded width exceeds the limit of 4194304 floats of this entry point"};
     if (!is_device_pointer(x) || !is_device_pointer(out))
       throw Fail{GCN_ADMM_ERR_ARG, "x and out must be device pointers"};
-    float* a = static_scratch(h->p.device);
-    float* b = a + kStaticHalf;
     struct Untimed {   // event creation reserves memory: launches here are counted, never timed
       gcn_admm* h; bool saved;
       explicit Untimed(gcn_admm* h_) : h(h_), saved(h_->profiling) { h->profiling = false; }
       ~Untimed() { h->profiling = saved; }
     } untimed(h);
-    {
-      gcn_admm::Scope sc(h, "permute_rows", 1, 8.0 * (double)h->n * width, 0.0);
-      gk::k_permute_rows<<<h->grid_for(h->n * ldw), 256, 0, h->stream>>>(x, a, h->d_perm, h->n, width, ldw, 1);
-      CU(cudaGetLastError());
-    }
-    h->spmm(a, b, ldw);
-    gcn_admm::Scope sc(h, "permute_rows", 1, 8.0 * (double)h->n * width, 0.0);
-    gk::k_permute_rows<<<h->grid_for(h->n * ldw), 256, 0, h->stream>>>(b, out, h->d_perm, h->n, width, ldw, 0);
-    CU(cudaGetLastError());
+    h->propagate_dense(x, width, out);
   });
 }
 
@@ -1633,7 +1650,8 @@ int gcn_admm_propagate_sharded(gcn_admm* h, int n_ranks, const float* x, int wid
         }
         if (n_own > 0) {
           gcn_admm::Scope sc(h, "spmm.sharded", 1, 0.0, 0.0);
-          h->spmm_launch(d_rp, d_cl, d_dv, d_order, n_own, nullptr, 0, INT_MAX, xl, b + (size_t)lo * ldw, ldw);
+          h->spmm_tables<4, false>(gcn_admm::GatherGraph{d_rp, d_cl, d_order, nullptr, d_dv, nullptr, nullptr, nullptr, nullptr, n_own, 0, 0, INT_MAX},
+                         xl, b + (size_t)lo * ldw, ldw / 4);
         }
         CU(cudaStreamSynchronize(h->stream));   // the host vectors of this rank go out of scope
       }

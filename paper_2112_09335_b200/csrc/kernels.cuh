@@ -69,120 +69,277 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
 
 // ------------------------------------------------------------------------------------------
 // Propagation  out = A~ x,  A~_ij = dinv_i dinv_j on the pattern of A + I (Problem 1).
-// G lanes share one row; each lane owns the float4 columns lane, lane+G, .. of a block of
-// G*V float4 columns; wider rows loop over column blocks.
-// A lane group walks its stored entries one after the other, so a row of thousands of entries
-// (row lengths follow a power law) would keep one warp busy long after the rest of the grid is
-// done.  Rows longer than `long_len` are therefore not handled as rows: they come as `n_items`
-// items {row, first entry, one past the last} (first in the grid), whose partial sums go to
-// `scratch` (one padded row per item) and are added up, in item order, by k_spmm_long_rows.
-// With ORDERED, rows are taken in the order `row_order` lists them (inside every community by falling
-// length): where several rows share a warp (narrow operands) its lane groups then walk rows of about the
-// same length and finish together (-20 % measured at 48 columns; at 256 columns, one row per warp, the
-// scattered order costs 13 %, so the caller passes no order there).
+// Two kernels: k_spmm_wide (a warp per row, more than 64 columns) and k_spmm_sets (narrower operands).
+// A warp walks its stored entries one after the other, so a row of thousands of entries (row lengths follow a
+// power law) would keep it busy long after the rest of the grid is done.  Rows longer than `long_len` are
+// therefore not handled as rows: they come as `n_items` items {row, first entry, one past the last} (first in
+// the grid), whose sums go to `scratch` (one row per item).  The row's items are then added up in
+// item order: by the last of them to finish (one counter per long row, left at zero), or by k_spmm_long_rows.
+// MAPPED: x and out are dense matrices in the caller's row order; node c's row is perm[c] (a 4-byte load in
+// parallel with that of its weight), so that no copy of the operand in community order and none back is made.
+// Values are moved in vectors of VEC floats: four wherever rows start on 16-byte boundaries (always inside the
+// library), fewer for a caller's matrix of odd width.
 // ------------------------------------------------------------------------------------------
-template <int G, int V, int UN, bool ORDERED>
-__global__ void __launch_bounds__(256)
-k_spmm(const int* __restrict__ row_ptr, const int* __restrict__ col, const float* __restrict__ dinv,
-       const float4* __restrict__ x, float4* __restrict__ out, int n, int ld4,
-       const int4* __restrict__ items, int n_items, int long_len, float4* __restrict__ scratch,
-       const int* __restrict__ row_order) {
+template <int VEC> struct Vec;
+template <> struct Vec<1> { using T = float; };
+template <> struct Vec<2> { using T = float2; };
+template <> struct Vec<4> { using T = float4; };
+
+__device__ __forceinline__ float vfma(float w, float x, float a) { return fmaf(w, x, a); }
+__device__ __forceinline__ float2 vfma(float w, float2 x, float2 a) { return make_float2(fmaf(w, x.x, a.x), fmaf(w, x.y, a.y)); }
+__device__ __forceinline__ float4 vfma(float w, float4 x, float4 a) {
+  return make_float4(fmaf(w, x.x, a.x), fmaf(w, x.y, a.y), fmaf(w, x.z, a.z), fmaf(w, x.w, a.w));
+}
+__device__ __forceinline__ float vscale(float w, float x) { return w * x; }
+__device__ __forceinline__ float2 vscale(float w, float2 x) { return make_float2(w * x.x, w * x.y); }
+__device__ __forceinline__ float4 vscale(float w, float4 x) { return make_float4(w * x.x, w * x.y, w * x.z, w * x.w); }
+__device__ __forceinline__ float vadd(float a, float b) { return a + b; }
+__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ float4 vadd(float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
+__device__ __forceinline__ float vxor(unsigned m, float a, int o) { return __shfl_xor_sync(m, a, o); }
+__device__ __forceinline__ float2 vxor(unsigned m, float2 a, int o) { return make_float2(vxor(m, a.x, o), vxor(m, a.y, o)); }
+__device__ __forceinline__ float4 vxor(unsigned m, float4 a, int o) {
+  return make_float4(vxor(m, a.x, o), vxor(m, a.y, o), vxor(m, a.z, o), vxor(m, a.w, o));
+}
+__device__ __forceinline__ void vzero(float& a) { a = 0.f; }
+__device__ __forceinline__ void vzero(float2& a) { a = make_float2(0.f, 0.f); }
+__device__ __forceinline__ void vzero(float4& a) { a = make_float4(0.f, 0.f, 0.f, 0.f); }
+
+// How the items of the long rows belong together: rows[r] = {row, first item, number of items}; item_row[k] = the entry
+// of `rows` item k belongs to; done: one zeroed counter per entry of `rows`.
+struct ItemRows {
+  const int4* rows;
+  const int* item_row;
+  int* done;
+};
+
+// Called by the G lanes (mask `gmask`, lane `gl`) that have just written item `unit`'s sums to scratch.
+template <typename T, int G>
+__device__ __forceinline__ void finish_item(const ItemRows& ir, int unit, T* __restrict__ row_out, const T* scratch, int ldv,
+                                            unsigned gmask, int gl) {
+  const int lr = ir.item_row[unit];
+  const int4 whole = ir.rows[lr];
+  __threadfence();
+  __syncwarp(gmask);
+  int done = 0;
+  if (gl == 0) done = atomicAdd(ir.done + lr, 1);
+  done = __shfl_sync(gmask, done, 0, G);
+  if (done + 1 < whole.z) return;
+  __threadfence();
+  for (int f = gl; f < ldv; f += G) {
+    T s;
+    vzero(s);
+#pragma unroll 4
+    for (int k = 0; k < whole.z; ++k) s = vadd(s, __ldcg(scratch + (long long)(whole.y + k) * ldv + f));
+    row_out[f] = s;
+  }
+  if (gl == 0) ir.done[lr] = 0;
+}
+
+// A warp per row, NV vectors per lane; wider rows loop over blocks of 32 NV vectors.  Lane t of a group of 32
+// stored entries holds column and weight of entry t, handed to the warp by shuffles.  UN neighbours in flight per
+// lane: the kernel is bound by the L2-to-SM traffic of the gathered rows, and by how the compiler orders its loads (the plain
+// loop measured faster than one that fetches columns ahead: 138 against 160 us at 128 columns on 169 k rows).
+template <int VEC, int NV, int UN, bool MAPPED>
+__global__ void __launch_bounds__(64, VEC == 4 ? 24 : 16)
+k_spmm_wide(const int* __restrict__ row_ptr, const int* __restrict__ col, const float* __restrict__ dinv,
+            const int* __restrict__ perm, const int4* __restrict__ items, int n, int n_items, int long_len,
+            const typename Vec<VEC>::T* __restrict__ x, typename Vec<VEC>::T* __restrict__ out, int ldv,
+            typename Vec<VEC>::T* __restrict__ scratch) {
+  using T = typename Vec<VEC>::T;
   const int lane = threadIdx.x & 31;
-  const int gl = lane & (G - 1);
-  const unsigned gmask = (G == 32) ? 0xffffffffu : (((1u << G) - 1u) << (lane & ~(G - 1)));
-  const long long unit = ((long long)blockIdx.x * blockDim.x + threadIdx.x) / G;
-  if (unit >= (long long)n + n_items) return;
-  long long row;
-  int rs, re;
-  float4* dst;
-  if (unit < n_items) {
+  const int unit = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+  if (unit >= n + n_items) return;
+  int row, rs, re;
+  T* dst;
+  const bool item = unit < n_items;
+  if (item) {
     const int4 it = items[unit];
     row = it.x; rs = it.y; re = it.z;
-    dst = scratch + unit * ld4;
+    dst = scratch + (long long)unit * ldv;
   } else {
     row = unit - n_items;
-    if (ORDERED) row = row_order[row];
     rs = row_ptr[row]; re = row_ptr[row + 1];
     if (re - rs > long_len) return;
-    dst = out + row * ld4;
+    dst = out + (long long)(MAPPED ? perm[row] : row) * ldv;
   }
   const float di = dinv[row];
-  for (int cb = 0; cb < ld4; cb += G * V) {
-    float4 acc[V];
+  for (int cb = 0; cb < ldv; cb += 32 * NV) {
+    T acc[NV];
 #pragma unroll
-    for (int v = 0; v < V; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
-    // Narrow operands (several rows per warp): a chunk of G entries costs three dependent load latencies
-    // (column, weight of that column, operand row) and moves little data, so the columns are fetched two
-    // chunks ahead and their weights one chunk ahead.  (At one row per warp the same prefetch was measured
-    // slower, and this kernel's load order is touchy there: the wide form keeps the plain loop.)
-    constexpr bool kAhead = G < 32;
-    int c_n = 0, c_n2 = 0;
-    float w_n = 0.f;
-    if (kAhead) {
-      if (rs + gl < re) c_n = col[rs + gl];
-      if (rs + G + gl < re) c_n2 = col[rs + G + gl];
-      if (rs + gl < re) w_n = dinv[c_n];
-    }
-    for (int base = rs; base < re; base += G) {
-      const int idx = base + gl;
-      int c = 0;
+    for (int v = 0; v < NV; ++v) vzero(acc[v]);
+    for (int base = rs; base < re; base += 32) {
+      int r = 0;
       float w = 0.f;
-      if (kAhead) {
-        c = c_n; w = w_n;
-        c_n = c_n2;
-        c_n2 = (idx + 2 * G < re) ? col[idx + 2 * G] : 0;
-        w_n = (idx + G < re) ? dinv[c_n] : 0.f;
-      } else if (idx < re) { c = col[idx]; w = dinv[c]; }
-      const int cnt = min(G, re - base);
+      if (base + lane < re) {
+        const int c = col[base + lane];
+        w = dinv[c];
+        r = MAPPED ? perm[c] : c;
+      }
+      const int cnt = min(32, re - base);
       for (int t = 0; t < cnt; t += UN) {
-        int cj[UN];
+        int rj[UN];
         float wj[UN];
 #pragma unroll
-        for (int u = 0; u < UN; ++u) {   // lanes past the row's end hold (column 0, weight 0)
-          cj[u] = __shfl_sync(gmask, c, (t + u) & (G - 1), G);
-          wj[u] = __shfl_sync(gmask, w, (t + u) & (G - 1), G);
-          if (t + u >= G) wj[u] = 0.f;
+        for (int u = 0; u < UN; ++u) {   // lanes past the row's end hold (row 0, weight 0)
+          rj[u] = __shfl_sync(0xffffffffu, r, (t + u) & 31);
+          wj[u] = __shfl_sync(0xffffffffu, w, (t + u) & 31);
         }
 #pragma unroll
-        for (int v = 0; v < V; ++v) {
-          const int f = cb + gl + G * v;
-          if (f < ld4) {
-            float4 xv[UN];
+        for (int v = 0; v < NV; ++v) {
+          const int f = cb + lane + 32 * v;
+          if (f < ldv) {
+            T xv[UN];
 #pragma unroll
-            for (int u = 0; u < UN; ++u) xv[u] = __ldg(x + (long long)cj[u] * ld4 + f);
+            for (int u = 0; u < UN; ++u) xv[u] = __ldg(x + (long long)rj[u] * ldv + f);
 #pragma unroll
-            for (int u = 0; u < UN; ++u) {
-              acc[v].x = fmaf(wj[u], xv[u].x, acc[v].x);
-              acc[v].y = fmaf(wj[u], xv[u].y, acc[v].y);
-              acc[v].z = fmaf(wj[u], xv[u].z, acc[v].z);
-              acc[v].w = fmaf(wj[u], xv[u].w, acc[v].w);
+            for (int u = 0; u < UN; ++u) acc[v] = vfma(wj[u], xv[u], acc[v]);
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      const int f = cb + lane + 32 * v;
+      if (f < ldv) dst[f] = vscale(di, acc[v]);
+    }
+  }
+}
+
+// Rows that k_spmm_wide handled as items (a kernel of its own: with finish_item at its end k_spmm_wide takes more
+// registers and was 4 % slower): out[row] = sum of the row's item sums, in item order, one block per row.
+template <typename T, bool MAPPED>
+__global__ void k_spmm_long_rows(const int4* __restrict__ rows, const T* __restrict__ scratch, T* __restrict__ out, int ldv,
+                                 const int* __restrict__ perm) {
+  const int4 r = rows[blockIdx.x];
+  const long long row = MAPPED ? perm[r.x] : r.x;
+  for (int f = threadIdx.x; f < ldv; f += blockDim.x) {
+    T s;
+    vzero(s);
+#pragma unroll 4
+    for (int k = 0; k < r.z; ++k) s = vadd(s, scratch[(long long)(r.y + k) * ldv + f]);
+    out[row * ldv + f] = s;
+  }
+}
+
+// Narrow operands.  G = CL * EP lanes share a row: CL of them side by side over its columns (NV vectors each), EP
+// such sets over its stored entries (entry e goes to set (e - first) mod EP), so that a row of k entries costs
+// k / EP dependent steps instead of k and a narrow row still fills the lanes of a warp; a shuffle tree adds the
+// sets at the end.  The order of a row's sum depends on EP alone: all layouts of a width agree bit for bit.
+// CL <= 4: every lane loads column and weight of its own entries (one word for the CL lanes of a set), one step
+// ahead of the operand rows.  CL >= 8: the G lanes load one entry each, columns two groups ahead and weights one,
+// and hand them to the sets by shuffles (with more lanes per set the repeated loads cost more than the shuffles).
+// Rows sharing a warp are taken by falling length.  Measured at 4 / 16 / 48 columns against one set per row:
+// 2.4 M rows, 126 M entries: 5.5 -> 1.1 ms, 2.2 -> 1.0, 2.7 -> 2.7; 13.8 k rows, 0.43 M entries: 293 -> 15 us, 85 -> 15, 37 -> 25.
+template <int VEC, int NV, int CL, int EP, int UN, bool MAPPED>
+__global__ void __launch_bounds__(128, CL >= 8 && VEC == 4 ? 10 : 8)
+k_spmm_sets(const int* __restrict__ row_ptr, const int* __restrict__ col, const float* __restrict__ dinv,
+            const int* __restrict__ perm, const int4* __restrict__ items, int n, int n_items, int long_len,
+            const typename Vec<VEC>::T* __restrict__ x, typename Vec<VEC>::T* __restrict__ out, int ldv,
+            typename Vec<VEC>::T* __restrict__ scratch, const int* __restrict__ row_order, const ItemRows ir) {
+  using T = typename Vec<VEC>::T;
+  constexpr int G = CL * EP;
+  static_assert(G <= 32, "a row is handled inside one warp");
+  static_assert(CL <= 4 || UN <= CL, "a group of G entries is CL steps of EP");
+  const int lane = threadIdx.x & 31, gl = lane & (G - 1), cl = gl & (CL - 1), set = gl / CL;
+  const unsigned gmask = G == 32 ? 0xffffffffu : (((1u << (G & 31)) - 1u) << (lane & ~(G - 1)));
+  const int unit = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) / G);
+  if (unit >= n + n_items) return;
+  int row, rs, re;
+  const bool item = unit < n_items;
+  if (item) {
+    const int4 it = items[unit];
+    row = it.x; rs = it.y; re = it.z;
+  } else {
+    row = unit - n_items;
+    if (G < 32) row = row_order[row];
+    rs = row_ptr[row]; re = row_ptr[row + 1];
+    if (re - rs > long_len) return;
+  }
+  const float di = dinv[row];
+  T* const row_out = out + (long long)(MAPPED ? perm[row] : row) * ldv;
+  T* const dst = item ? scratch + (long long)unit * ldv : row_out;
+  for (int cb = 0; cb < ldv; cb += CL * NV) {
+    T acc[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) vzero(acc[v]);
+    if constexpr (CL <= 4) {
+      int c[UN];
+#pragma unroll
+      for (int u = 0; u < UN; ++u) c[u] = (rs + set + u * EP < re) ? col[rs + set + u * EP] : -1;
+      for (int e = rs + set; e < re; e += EP * UN) {
+        float w[UN];
+        int r[UN];
+#pragma unroll
+        for (int u = 0; u < UN; ++u) {
+          w[u] = c[u] >= 0 ? dinv[c[u]] : 0.f;
+          r[u] = c[u] >= 0 ? (MAPPED ? perm[c[u]] : c[u]) : -1;
+        }
+        const int en = e + EP * UN;
+#pragma unroll
+        for (int u = 0; u < UN; ++u) c[u] = (en + u * EP < re) ? col[en + u * EP] : -1;
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+          const int f = cb + cl + CL * v;
+          if (f < ldv) {
+            T xv[UN];
+#pragma unroll
+            for (int u = 0; u < UN; ++u)
+              if (r[u] >= 0) xv[u] = __ldg(x + (long long)r[u] * ldv + f);
+#pragma unroll
+            for (int u = 0; u < UN; ++u)
+              if (r[u] >= 0) acc[v] = vfma(w[u], xv[u], acc[v]);
+          }
+        }
+      }
+    } else {
+      int c_n = rs + gl < re ? col[rs + gl] : -1, c_n2 = rs + G + gl < re ? col[rs + G + gl] : -1;
+      float w_n = c_n >= 0 ? dinv[c_n] : 0.f;
+      int r_n = c_n >= 0 ? (MAPPED ? perm[c_n] : c_n) : 0;
+      for (int base = rs; base < re; base += G) {
+        const float w = w_n;
+        const int r = r_n;
+        c_n = c_n2;
+        c_n2 = base + 2 * G + gl < re ? col[base + 2 * G + gl] : -1;
+        w_n = c_n >= 0 ? dinv[c_n] : 0.f;
+        r_n = c_n >= 0 ? (MAPPED ? perm[c_n] : c_n) : 0;
+        const int steps = (min(G, re - base) + EP - 1) / EP;
+        for (int t = 0; t < steps; t += UN) {
+          int rj[UN];
+          float wj[UN];
+#pragma unroll
+          for (int u = 0; u < UN; ++u) {   // lanes past the row's end hold (row 0, weight 0)
+            const int src = ((t + u) * EP + set) & (G - 1);
+            rj[u] = __shfl_sync(gmask, r, src, G);
+            wj[u] = __shfl_sync(gmask, w, src, G);
+          }
+#pragma unroll
+          for (int v = 0; v < NV; ++v) {
+            const int f = cb + cl + CL * v;
+            if (f < ldv) {
+              T xv[UN];
+#pragma unroll
+              for (int u = 0; u < UN; ++u) xv[u] = __ldg(x + (long long)rj[u] * ldv + f);
+#pragma unroll
+              for (int u = 0; u < UN; ++u) acc[v] = vfma(wj[u], xv[u], acc[v]);
             }
           }
         }
       }
     }
 #pragma unroll
-    for (int v = 0; v < V; ++v) {
-      const int f = cb + gl + G * v;
-      if (f < ld4)
-        dst[f] = make_float4(di * acc[v].x, di * acc[v].y, di * acc[v].z, di * acc[v].w);
+    for (int o = CL; o < G; o <<= 1)
+#pragma unroll
+      for (int v = 0; v < NV; ++v) acc[v] = vadd(acc[v], vxor(gmask, acc[v], o));
+    if (set == 0) {
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        const int f = cb + cl + CL * v;
+        if (f < ldv) dst[f] = vscale(di, acc[v]);
+      }
     }
   }
-}
-
-// Rows that k_spmm handled as items: out[row] = sum of the row's item sums, in item order.
-// rows[r] = {row, first item, number of items}; one block per row.
-__global__ void k_spmm_long_rows(const int4* __restrict__ rows, const float4* __restrict__ scratch,
-                                 float4* __restrict__ out, int ld4) {
-  const int4 r = rows[blockIdx.x];
-  for (int f = threadIdx.x; f < ld4; f += blockDim.x) {
-    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int k = 0; k < r.z; ++k) {
-      const float4 v = scratch[(long long)(r.y + k) * ld4 + f];
-      s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
-    }
-    out[(long long)r.x * ld4 + f] = s;
-  }
+  if (item) finish_item<T, G>(ir, unit, row_out, scratch, ldv, gmask, gl);
 }
 
 // ------------------------------------------------------------------------------------------
