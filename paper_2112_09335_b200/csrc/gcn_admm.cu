@@ -39,7 +39,7 @@ constexpr int kLogPasses = 256;
 constexpr int kSmCount = 148;
 constexpr long long kImageMinRows = 16384;   // row count from which the weight operand is pre-split
 constexpr int kZBlockRows = 32;      // rows per block of the hidden-layer gradient's closing sweep
-constexpr int kChunksPerGroup = 256; // chunks whose sums one block of k_reduce_chunks adds up
+constexpr int kChunkGroups = 512;    // groups the sums of a scoring sweep's chunks are first added up in, when there are more chunks
 constexpr int kCandZ = 4;           // theta candidates scored per sweep (2..4; steady-state searches close at trial 0..2)
 constexpr int kDefaultLongRow = 256;   // stored entries one warp walks before a row is cut into items
 
@@ -209,9 +209,12 @@ struct gcn_admm {
   float* part = nullptr;     // split partial sums of the transposed product
   size_t part_elems = 0;
   SearchCtl *ctl_w = nullptr, *ctl_z = nullptr;   // [L+1], [(L+1) * M]
-  double *sums_w = nullptr, *sums_z = nullptr, *obj = nullptr;
+  double *sums_z = nullptr, *obj = nullptr;
   double* red_part = nullptr;               // per-block partial sums awaiting their fixed-order reduction
-  int2* d_zblocks = nullptr;                // row blocks of at most kZBlockRows rows, none crossing a community
+  int4* d_zblocks = nullptr;                // row blocks of at most kZBlockRows rows, none crossing a community, and that community
+  unsigned *ticket = nullptr, *comm_tickets = nullptr;   // counters of finished blocks (one launch; per community), zero between launches
+  gk::GridBar* grid_bar = nullptr;          // meeting point of the cooperative launches (one at a time: one stream)
+  std::vector<float*> RN;                   // 2..L: derivative of phi_l at the new H_l, from the W_l update to that of Z_{l-1}
   int* d_comm_block_ptr = nullptr;          // [M+1] first row block of every community
   int n_zblocks = 0;
   int *n_active = nullptr, *status = nullptr, *d_pass = nullptr;
@@ -224,7 +227,6 @@ struct gcn_admm {
   double* z_chunk_part = nullptr;           // [chunk][M][candidates] sums of one sweep, per chunk of units
   double* z_group_part = nullptr;           // [group of chunks][M][candidates], chunks added in order
   int* chunk_counter = nullptr;             // hands the chunks out to the warps of a sweep
-  int n_groups = 0;
   double* split_scores = nullptr;           // [n_split][candidates] sums of the segments scored in pieces
   int *d_split_order = nullptr, *d_split_ptr = nullptr;   // split entries grouped by community
   cudaGraphExec_t pass_graph = nullptr;   // one pass of Algorithm 1, recorded once and replayed
@@ -405,21 +407,21 @@ struct gcn_admm {
     CU(cudaGetLastError());
   }
 
-  // out[Ka x ldp] = A^T B over `rows` rows, through split partial sums reduced in a fixed order.
+  // A^T B over `rows` rows as split partial sums in `part` (added up in a fixed order by finish_grad); returns their number.
   // Whether P^T R runs on the tensor cores (that form can also build a hidden layer's R itself).
   bool tn_on_tensor_cores(long long rows) const { return p.tensor_cores != 0 && rows >= 4096; }
 
   // With `zres` (tensor-core form only) B holds pre-activations H and the operand is
   // h > 0 ? nu (h - z) : 0, formed while staging: the residual matrix is never stored.
-  void gemm_tn(const float* A, int lda, const float* B, int ldb, float* out, int ldp, long long rows, int Ka,
-               int Nb, const float* zres = nullptr, float nu = 0.f) {
+  int gemm_tn(const float* A, int lda, const float* B, int ldb, int ldp, long long rows, int Ka, int Nb,
+              const float* zres = nullptr, float nu = 0.f) {
     int splits = 1;
     long long rps = rows;
     char name[48];
     if (zres && !tn_on_tensor_cores(rows)) throw Fail{GCN_ADMM_ERR_ARG, "fused residual needs the tensor-core product"};
     if (tn_on_tensor_cores(rows)) {
       std::snprintf(name, sizeof name, zres ? "gemm_tn_tc.resid@%dx%d" : "gemm_tn_tc@%dx%d", Ka, Nb);
-      Scope sc(this, name, 2, 4.0 * ((double)rows * (lda + (zres ? 2 : 1) * ldb) + (double)Ka * ldp), 2.0 * (double)rows * Ka * Nb);
+      Scope sc(this, name, 1, 4.0 * ((double)rows * (lda + (zres ? 2 : 1) * ldb) + (double)Ka * ldp), 2.0 * (double)rows * Ka * Nb);
       const int nt_tn = Nb <= 16 ? 16 : Nb <= 32 ? 32 : Nb <= 48 ? 48 : Nb <= 64 ? 64 : Nb <= 128 ? 128 : 256;
       const int nb_groups = (int)cdiv(Nb, nt_tn);
       const int groups = (int)cdiv(Ka, gtc::kBlockM);
@@ -454,13 +456,10 @@ struct gcn_admm {
       else TN_TC(256)
 #undef TN_TC
       CU(cudaGetLastError());
-      const long long elems_tc = (long long)Ka * ldp;
-      gk::k_reduce_splits<<<(unsigned)cdiv(elems_tc, 256), 256, 0, stream>>>(part, out, elems_tc, splits);
-      CU(cudaGetLastError());
-      return;
+      return splits;
     }
     std::snprintf(name, sizeof name, "gemm_tn@%dx%d", Ka, Nb);
-    Scope sc(this, name, 2, 4.0 * ((double)rows * (lda + ldb) + (double)Ka * ldp), 2.0 * (double)rows * Ka * Nb);
+    Scope sc(this, name, 1, 4.0 * ((double)rows * (lda + ldb) + (double)Ka * ldp), 2.0 * (double)rows * Ka * Nb);
 #define TN_CASE(BM, BN, BK, TM, TN)                                                             \
   {                                                                                             \
     const long long tiles = cdiv(Ka, BM) * cdiv(ldp, BN);                                        \
@@ -477,9 +476,41 @@ struct gcn_admm {
     else TN_CASE(128, 8, 16, 4, 1)
 #undef TN_CASE
     CU(cudaGetLastError());
-    const long long elems = (long long)Ka * ldp;
-    gk::k_reduce_splits<<<(unsigned)cdiv(elems, 256), 256, 0, stream>>>(part, out, elems, splits);
+    return splits;
+  }
+
+  // grad (and grad_t) from the `splits` partial sums gemm_tn left in `part`; with `ctl` the start of the W_l search too.
+  void finish_grad(int splits, int Ka, int Nb, int ldp, float* out, float* out_t, int ldt, const float* w, SearchCtl* ctl) {
+    Scope sc(this, "finish_grad", 1, 4.0 * (double)Ka * ldp * (splits + (w ? 3 : 1)), 0.0);
+    const long long col_blocks = cdiv(ldp, 32);
+    if (splits >= 16)
+      gk::k_finish_grad<8><<<(unsigned)(col_blocks * Ka), 256, 0, stream>>>(part, splits, Ka, Nb, ldp, out, out_t, ldt, w, red_part,
+                                                                            ticket, ctl, p.bt_shrink, p.bt_growth, status);
+    else
+      gk::k_finish_grad<1><<<(unsigned)(col_blocks * cdiv(Ka, 8)), 256, 0, stream>>>(part, splits, Ka, Nb, ldp, out, out_t, ldt, w, red_part,
+                                                                                     ticket, ctl, p.bt_shrink, p.bt_growth, status);
     CU(cudaGetLastError());
+  }
+
+  // Blocks of `kernel` that fit the device at once (looked up once per kernel and shared-memory size): the grid of a
+  // cooperative or persistent launch.
+  std::map<std::pair<const void*, size_t>, int> resident_cache;
+  int resident_blocks(const void* kernel, int threads, size_t smem) {
+    auto it = resident_cache.find({kernel, smem});
+    if (it != resident_cache.end()) return it->second;
+    if (smem > 48 * 1024) CU(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    int per_sm = 0;
+    CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem));
+    if (per_sm < 1) throw Fail{GCN_ADMM_ERR_CUDA, "a kernel does not fit the device"};
+    return resident_cache[{kernel, smem}] = per_sm * kSmCount;
+  }
+  template <typename T> struct Same { using type = T; };   // keeps a parameter out of template deduction
+  template <typename... Args>
+  void launch_together(void (*kernel)(Args...), long long blocks_wanted, int threads, size_t smem, typename Same<Args>::type... args) {
+    const void* f = reinterpret_cast<const void*>(kernel);
+    const int grid = (int)std::max<long long>(1, std::min<long long>(blocks_wanted, resident_blocks(f, threads, smem)));
+    void* argv[] = {const_cast<void*>(static_cast<const void*>(&args))...};
+    CU(cudaLaunchCooperativeKernel(f, dim3((unsigned)grid), dim3((unsigned)threads), argv, smem, stream));
   }
 
   void resid(int l, float* R) {   // derivative of phi_l with respect to H_l, at the stored H_l
@@ -493,244 +524,187 @@ struct gcn_admm {
     CU(cudaGetLastError());
   }
 
-  int n_passes(int cand) const { return (p.bt_max_trials + cand - 1) / cand; }
-
   long long z_per_pass() const { return (long long)std::max(L - 1, 0) * M; }
+  gk::DecisionLog log_w(int l) const { return gk::DecisionLog{log_trial_w, log_q_w, d_pass, L, l - 1, kLogPasses}; }
+  gk::DecisionLog log_z(int l) const {
+    return gk::DecisionLog{log_trial_z, log_q_z, d_pass, z_per_pass(), (long long)(l - 1) * M, kLogPasses};
+  }
 
-  void begin_log_pass() {
+  // A single block family is about to run: everything else is logged as "not run".
+  void clear_log_pass() {
     const long long zc = z_per_pass();
     Scope sc(this, "small", zc > 0 ? 2 : 1, 0.0, 0.0);
     gk::k_log_clear<<<1, 64, 0, stream>>>(log_trial_w, d_pass, L, kLogPasses);
     if (zc > 0) gk::k_log_clear<<<grid_for(zc), 256, 0, stream>>>(log_trial_z, d_pass, zc, kLogPasses);
     CU(cudaGetLastError());
   }
-  void end_log_pass() {
-    Scope sc(this, "small", 1, 0.0, 0.0);
-    gk::k_pass_advance<<<1, 1, 0, stream>>>(d_pass);
-    CU(cudaGetLastError());
-    ++log_count;
-  }
 
   // ---- W_l block (Section 3.1) --------------------------------------------------------
-  void update_W(int l) {
+  // resid_next: also leave the derivative of phi_l at the new H_l in RN[l] (what the Z_{l-1} update starts from).
+  void update_W(int l, bool resid_next) {
     Range range("gcn_admm: W block");
     const int Kp = C[l - 1], Cn = C[l], ldc = ld[l];
     const long long n4 = n * ldc / 4;
     SearchCtl* ctl = ctl_w + l;
+    int splits;
     if (l < L && tn_on_tensor_cores(n)) {                               // grad = P_l^T R_l, R_l formed inside the product
-      gemm_tn(P[l], ld[l - 1], H[l], ldc, grad, ldc, n, Kp, Cn, Z[l], p.nu);
+      splits = gemm_tn(P[l], ld[l - 1], H[l], ldc, ldc, n, Kp, Cn, Z[l], p.nu);
     } else {
       resid(l, B0);                                                     // R_l
-      gemm_tn(P[l], ld[l - 1], B0, ldc, grad, ldc, n, Kp, Cn);          // grad = P_l^T R_l
+      splits = gemm_tn(P[l], ld[l - 1], B0, ldc, ldc, n, Kp, Cn);       // grad = P_l^T R_l
     }
-    {
-      Scope sc(this, "small", 3, 0.0, 0.0);
-      gk::k_transpose_small<<<(unsigned)cdiv((long long)Kp * Cn, 256), 256, 0, stream>>>(grad, ldc, grad_t, ld[l - 1], Kp, Cn);
-      gk::k_two_sumsq<<<1, 1024, 0, stream>>>(grad, W[l], (long long)Kp * ldc, sums_w);
-      gk::k_search_begin<<<1, 32, 0, stream>>>(ctl, sums_w, p.bt_shrink, p.bt_growth, status);
-      CU(cudaGetLastError());
-    }
+    finish_grad(splits, Kp, Cn, ldc, grad, grad_t, ld[l - 1], W[l], ctl);
     gemm_nn(P[l], ld[l - 1], grad, ldc, grad_t, ld[l - 1], B1, ldc, n, Cn, Kp, &ctl->done);   // D = P_l grad
-    gk::DecideArgs a{};
-    a.growth = p.bt_growth;
-    a.max_trials = p.bt_max_trials;
-    a.cand = gk::kCand;
-    const int score_grid = grid_for(n4);   // every block of a scoring sweep leaves its sums in red_part
-    if (l == L) {
-      {
-        Scope sc(this, "score_w_out", 1, 32.0 * n4, 0.0);
-        gk::k_score_w_out<<<score_grid, 256, 0, stream>>>((const float4*)B1, (const float4*)B0, n4, ctl, red_part);
-      }
-      a.mode = 1;
-      a.quad_coef = 0.5 * p.rho;
-      a.last_pass = 1;
-      Scope sc(this, "small", 1, 0.0, 0.0);
-      gk::k_search_decide_w<<<1, 256, 0, stream>>>(ctl, red_part, score_grid, 2, a, status);
-    } else {
-      a.mode = 0;
-      a.scale = 0.5 * p.nu;
-      const int passes = n_passes(gk::kCand);
-      for (int ps = 0; ps < passes; ++ps) {
-        {   // passes after the first almost always find the search finished and return at once
-          Scope sc(this, ps == 0 ? "score_w_hidden" : "score_w_hidden.retry", 1, ps == 0 ? 48.0 * n4 : 0.0, 0.0);
-          gk::k_score_w_hidden<<<score_grid, 256, 0, stream>>>((const float4*)H[l], (const float4*)B1,
-                                                               (const float4*)Z[l], n4, ctl, red_part);
-        }
-        a.last_pass = (ps == passes - 1);
-        Scope sc(this, "small", 1, 0.0, 0.0);
-        gk::k_search_decide_w<<<1, 256, 0, stream>>>(ctl, red_part, score_grid, gk::kCand, a, status);
-      }
-    }
-    CU(cudaGetLastError());
-    {
-      Scope sc(this, "small", 2, 0.0, 0.0);
-      gk::k_log_decisions<<<1, 32, 0, stream>>>(ctl, 1, log_trial_w, log_q_w, d_pass, L, l - 1, kLogPasses);
-      gk::k_apply_w<<<(unsigned)cdiv((long long)Kp * Cn, 256), 256, 0, stream>>>(W[l], Wt[l], grad, Kp, Cn, ldc,
-                                                                               ld[l - 1], ctl);
-    }
-    Scope sc(this, "axpy_h", 1, 48.0 * n4, 0.0);
-    gk::k_axpy_ctl<<<grid_for(n4), 256, 0, stream>>>((float4*)H[l], (const float4*)B1, n4, ctl);   // H_l at W^{k+1}
-    CU(cudaGetLastError());
+    gk::SearchW a{};
+    a.H = (float4*)H[l]; a.D = (const float4*)B1; a.Z = (const float4*)Z[l]; a.U = (const float4*)U; a.R = (const float4*)B0;
+    a.Rn = resid_next ? (float4*)RN[l] : nullptr;
+    a.n4 = n4;
+    a.coef = l == L ? p.rho : p.nu;
+    a.W = W[l]; a.Wt = Wt[l]; a.grad = grad;
+    a.rows = Kp; a.cols = Cn; a.ldw = ldc; a.ldwt = ld[l - 1];
+    a.ctl = ctl; a.partial = red_part; a.bar = grid_bar; a.status = status; a.err = tc_error;
+    a.a.growth = p.bt_growth;
+    a.a.max_trials = p.bt_max_trials;
+    a.a.cand = gk::kCand;
+    a.a.mode = l == L ? 1 : 0;
+    a.a.scale = 0.5 * p.nu;
+    a.a.quad_coef = 0.5 * p.rho;
+    a.log = log_w(l);
+    // scoring reads three arrays (two for the last layer), the move reads two and writes one, the residual reads one or two and writes one
+    const double arrays = (l == L ? 2 : 3) + 3 + (resid_next ? (l == L ? 3 : 2) : 0);
+    Scope sc(this, l == L ? "search_w_out" : "search_w_hidden", 1, 16.0 * arrays * n4, 0.0);
+    launch_together(l == L ? gk::k_search_w<true> : gk::k_search_w<false>, cdiv(n4, 256), 256, 0, a);
   }
 
   // ---- Z_{l,m}, l < L, every community (Appendix A, Eq. 5/6 and 8-10) ------------------
-  void update_Z_hidden(int l) {
+  // resid_ready: RN[l+1] holds the derivative of phi_{l+1} at the stored H_{l+1}.
+  void update_Z_hidden(int l, bool resid_ready) {
     Range range("gcn_admm: hidden Z blocks");
     const int ldl = ld[l], ldn = ld[l + 1];
     SearchCtl* ctl = ctl_z + (size_t)l * M;
-    resid(l + 1, B0);                                                    // R'_{l+1}
-    spmm(B0, B1, ldn);                                                   // S = A~ R'
+    float* const Rn = RN[l + 1];
+    if (!resid_ready) resid(l + 1, Rn);                                  // R'_{l+1}
+    spmm(Rn, B1, ldn);                                                   // S = A~ R'
     gemm_nn(B1, ldn, Wt[l + 1], ldl, W[l + 1], ldn, B2, ldl, n, C[l], C[l + 1]);        // S W_{l+1}^T
-    CU(cudaMemsetAsync(n_active, 0, sizeof(int), stream));
     {
       Scope sc(this, "zgrad_finish", 1, 16.0 * 4.0 * (double)n * (ldl / 4), 0.0);
-      gk::k_zgrad_finish<<<(unsigned)n_zblocks, 256, 0, stream>>>((float4*)B2, (const float4*)Z[l], (const float4*)H[l],
-                                                                 ldl / 4, d_zblocks, p.nu, red_part);
-    }
-    const bool out = (l + 1 == L);
-    const int per = out ? 2 : kCandZ;
-    {
-      Scope sc(this, "small", 1, 0.0, 0.0);
-      gk::k_search_begin_z<<<(unsigned)cdiv((long long)M * 32, 128), 128, 0, stream>>>(
-          ctl, M, red_part, d_comm_block_ptr, sums_z, p.bt_shrink, p.bt_growth, n_active, status);
+      gk::k_zgrad_finish<<<(unsigned)n_zblocks, 256, 0, stream>>>(
+          (float4*)B2, (const float4*)Z[l], (const float4*)H[l], ldl / 4, d_zblocks, p.nu, red_part, d_comm_block_ptr, comm_tickets, ctl, sums_z,
+          p.bt_shrink, p.bt_growth, n_active, status);
       CU(cudaGetLastError());
     }
     gemm_nn(B2, ldl, W[l + 1], ldn, Wt[l + 1], ldl, B1, ldn, n, C[l + 1], C[l]);         // T = G W_{l+1}
-    gk::DecideArgs a{};
-    a.growth = p.bt_growth;
-    a.max_trials = p.bt_max_trials;
-    a.cand = kCandZ;
-    a.own_nu = p.nu;
-    const int ld4 = ldn / 4;
-    const int warps = 8;
-    const size_t smem = (size_t)warps * M * per * sizeof(double);
-    const int use_smem = smem <= 96 * 1024;
-    const size_t dyn = use_smem ? smem : 0;
-    // after a sweep: the chunks' sums are added group by group, in chunk order (first stage of the ordered sum)
-    int groups_used = 0;   // groups of chunks the last sweep filled (the chunk table depends on the kernel)
-    auto reduce_chunks = [&](int chunks) {
-      groups_used = (int)cdiv(chunks, kChunksPerGroup);
-      gk::k_reduce_chunks<<<(unsigned)groups_used, 256, 0, stream>>>(z_chunk_part, chunks, kChunksPerGroup, M * per,
-                                                                     z_group_part, n_active);
-      ++launches;
-    };
-#define SCORE_Z_U(V, OUT, UNZ)                                                                                 \
-  {                                                                                                       \
-    const size_t dynv = dyn + (size_t)warps * 2 * (V) * 32 * sizeof(float4);   /* per-warp copy of the row's a, b */ \
-    if (dynv > 48 * 1024)                                                                                 \
-      CU(cudaFuncSetAttribute(gk::k_score_z<V, OUT, UNZ, kCandZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dynv)); \
-    int occ = 1;                                                                                          \
-    CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, gk::k_score_z<V, OUT, UNZ, kCandZ>, warps * 32, dynv));     \
-    const unsigned grid = (unsigned)std::min<long long>(cdiv(n_chunks, warps), (long long)kSmCount * std::max(occ, 1)); \
-    CU(cudaMemsetAsync(chunk_counter, 0, sizeof(int), stream));                                           \
-    gk::k_score_z<V, OUT, UNZ, kCandZ><<<grid, warps * 32, dynv, stream>>>(d_row_ptr, d_col, d_col_comm, d_dinv,       \
-        (const float4*)B1, (const float4*)H[l + 1], (const float4*)Z[l + 1], (const float4*)B0, ld4, (int)n, ctl, M, \
-        z_chunk_part, n_active, use_smem, d_chunk_ptr, n_chunks, chunk_counter, d_items, n_items, long_len,      \
-        reinterpret_cast<float4*>(item_sums), nullptr);                                                         \
-    reduce_chunks(n_chunks);                                                                              \
-    if (n_split > 0) {                                                                                    \
-      gk::k_score_z_split<V, OUT, kCandZ><<<(unsigned)cdiv(n_split, warps), warps * 32, 0, stream>>>(d_split, n_split, d_dinv, \
-          reinterpret_cast<const float4*>(item_sums), (const float4*)H[l + 1], (const float4*)Z[l + 1], (const float4*)B0, \
-          ld4, ctl, split_scores, n_active);                                                              \
-      ++launches;                                                                                         \
-    }                                                                                                     \
-  }
-#define SCORE_Z_ANY(OUT)                        \
-  {                                             \
-    if (ld4 <= 32) SCORE_Z_U(1, OUT, 4)         \
-    else if (ld4 <= 64) SCORE_Z_U(2, OUT, 4)    \
-    else if (ld4 <= 128) SCORE_Z_U(4, OUT, 4)   \
-    else SCORE_Z_U(8, OUT, 4)                   \
-  }
-    auto decide = [&](const gk::DecideArgs& args) {
-      Scope sc(this, "small", 1, 0.0, 0.0);
-      gk::k_search_decide_z<<<(unsigned)cdiv((long long)M * 32, 128), 128, 0, stream>>>(
-          ctl, M, z_group_part, groups_used, per, split_scores, d_split_order, d_split_ptr, sums_z, args, n_active, status);
+
+    const bool out = (l + 1 == L);
+    const int per = out ? 2 : kCandZ, ld4 = ldn / 4, warps = 8;
+    gk::SearchZ a{};
+    a.ctl = ctl; a.n_comm = M;
+    a.chunk_part = z_chunk_part; a.chunk_counter = chunk_counter; a.group_part = z_group_part;
+    a.split = d_split; a.n_split = n_split; a.split_scores = split_scores; a.split_order = d_split_order; a.split_ptr = d_split_ptr;
+    a.own = sums_z; a.n_active = n_active; a.status = status; a.err = tc_error; a.bar = grid_bar;
+    a.a.growth = p.bt_growth;
+    a.a.max_trials = p.bt_max_trials;
+    a.a.cand = kCandZ;
+    a.a.own_nu = p.nu;
+    a.a.mode = out ? 1 : 0;
+    a.a.scale = 0.5 * p.nu;
+    a.a.quad_coef = 0.5 * p.rho;
+    a.log = log_z(l);
+    a.Z = (float4*)Z[l]; a.G = (const float4*)B2; a.ldz4 = ldl / 4; a.row_comm = d_row_comm;
+    // few chunks: a warp per community adds them up directly; many: group by group first (one more meeting of the grid)
+    auto with_groups = [&](int chunks) {
+      gk::SearchZ b = a;
+      b.per_group = (int)cdiv(chunks, kChunkGroups);
+      b.n_groups = chunks > kChunkGroups ? (int)cdiv(chunks, b.per_group) : 0;
+      return b;
     };
     char zname[48];
     std::snprintf(zname, sizeof zname, out ? "score_z_out@%d" : "score_z_hidden@%d", ldn);
-    const std::string zretry = std::string(zname) + ".retry";
-    const double zbytes = 6.0 * gi.nnz + 8.0 * n +
-                          4.0 * (double)n * ldn * (out ? 2 : 3);
-    if (out) {
+    const double score_bytes = 6.0 * gi.nnz + 8.0 * n + 4.0 * (double)n * ldn * (out ? 2 : 3), score_flops = 2.0 * (double)gi.nnz * ldn;
+    const double move_bytes = 12.0 * (double)n * ldl;
+    const float4 *T = (const float4*)B1, *Hn = (const float4*)H[l + 1], *Zn = (const float4*)Z[l + 1], *R4 = (const float4*)Rn;
+    float4* const scratch = reinterpret_cast<float4*>(item_sums);
+    // closing, further sweeps and the move: as many blocks as the move can use
+    const long long move_blocks = cdiv(n * (ldl / 4), 256);
+#define SCORE_PART(G)                                                                                                       \
+  if (ld4 <= (G) && (size_t)(32 / (G)) * warps * M * 2 * sizeof(double) <= 96 * 1024) {                                     \
+    const size_t smem = (size_t)(32 / (G)) * warps * M * 2 * sizeof(double);                                                \
+    const auto kernel = gk::k_score_z_out_part<(G), 4>;                                                                     \
+    const int grid = (int)std::min<long long>(cdiv(n_chunks_sorted, warps), resident_blocks((const void*)kernel, warps * 32, smem)); \
+    {                                                                                                                       \
+      Scope sc(this, zname, 1, score_bytes, score_flops);                                                                   \
+      kernel<<<grid, warps * 32, smem, stream>>>(d_row_ptr, d_col, d_col_comm, d_dinv, T, R4, ld4, ctl, M, z_chunk_part, n_active, \
+                                                 d_chunk_ptr_sorted, n_chunks_sorted, chunk_counter, d_items, n_items, long_len, \
+                                                 scratch, d_row_order);                                                     \
+      CU(cudaGetLastError());                                                                                               \
+    }                                                                                                                       \
+    Scope sc(this, "close_z", 1, move_bytes, 0.0);                                                                          \
+    launch_together(gk::k_close_z<1, true, 4, kCandZ>, move_blocks, warps * 32, 0, d_row_ptr, d_col, d_col_comm, d_dinv, T, Hn, Zn, R4, \
+                    ld4, (int)n, 0, d_chunk_ptr_sorted, n_chunks_sorted, d_items, n_items, long_len, scratch,               \
+                    with_groups(n_chunks_sorted));                                                                          \
+    return;                                                                                                                 \
+  }
+    if (out) {   // narrow output layer: several rows per warp
+      SCORE_PART(4)
+      SCORE_PART(8)
+      SCORE_PART(16)
+    }
+#undef SCORE_PART
+    const size_t sums = (size_t)warps * M * per * sizeof(double);
+    const int use_smem = sums <= 96 * 1024;
+    auto score = [&](auto kernel, auto close, int V) {
+      const size_t smem = (size_t)warps * 2 * V * 32 * sizeof(float4) + (use_smem ? sums + (size_t)M * sizeof(float4) : 0);
+      const int grid = (int)std::min<long long>(cdiv(n_chunks, warps), resident_blocks((const void*)kernel, warps * 32, smem));
       {
-        Scope sc(this, zname, 1, zbytes, 2.0 * (double)gi.nnz * ldn);
-        const size_t smem_h = (size_t)2 * warps * M * 2 * sizeof(double);
-        if (ld4 <= 16 && smem_h <= 96 * 1024) {   // narrow output layer: two rows per warp (see k_score_z_out_half)
-          if (smem_h > 48 * 1024)
-            CU(cudaFuncSetAttribute(gk::k_score_z_out_half<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_h));
-          int occ = 1;
-          CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, gk::k_score_z_out_half<4>, warps * 32, smem_h));
-          const unsigned grid = (unsigned)std::min<long long>(cdiv(n_chunks_sorted, warps), (long long)kSmCount * std::max(occ, 1));
-          CU(cudaMemsetAsync(chunk_counter, 0, sizeof(int), stream));
-          gk::k_score_z_out_half<4><<<grid, warps * 32, smem_h, stream>>>(d_row_ptr, d_col, d_col_comm, d_dinv,
-              (const float4*)B1, (const float4*)B0, ld4, (int)n, ctl, M, z_chunk_part, n_active, d_chunk_ptr_sorted, n_chunks_sorted,
-              chunk_counter, d_items, n_items, long_len, reinterpret_cast<float4*>(item_sums), d_row_order);
-          reduce_chunks(n_chunks_sorted);
-          if (n_split > 0) {
-            gk::k_score_z_split<1, true, kCandZ><<<(unsigned)cdiv(n_split, warps), warps * 32, 0, stream>>>(d_split, n_split, d_dinv,
-                reinterpret_cast<const float4*>(item_sums), (const float4*)H[l + 1], (const float4*)Z[l + 1], (const float4*)B0,
-                ld4, ctl, split_scores, n_active);
-            ++launches;
-          }
-        } else {
-          SCORE_Z_ANY(true)
-        }
+        Scope sc(this, zname, 1, score_bytes, score_flops);
+        kernel<<<grid, warps * 32, smem, stream>>>(d_row_ptr, d_col, d_col_comm, d_dinv, T, Hn, Zn, R4, ld4, ctl, M, z_chunk_part, n_active,
+                                                   use_smem, d_chunk_ptr, n_chunks, chunk_counter, d_items, n_items, long_len, scratch);
+        CU(cudaGetLastError());
       }
-      a.mode = 1;
-      a.quad_coef = 0.5 * p.rho;
-      a.last_pass = 1;
-      decide(a);
-    } else {
-      a.mode = 0;
-      a.scale = 0.5 * p.nu;
-      const int passes = n_passes(kCandZ);
-      for (int ps = 0; ps < passes; ++ps) {
-        {   // later passes touch only the segments of communities still searching
-          Scope sc(this, ps == 0 ? zname : zretry.c_str(), 1, ps == 0 ? zbytes : 0.0,
-                   ps == 0 ? 2.0 * (double)gi.nnz * ldn : 0.0);
-          SCORE_Z_ANY(false)
-        }
-        a.last_pass = (ps == passes - 1);
-        decide(a);
-      }
-    }
-#undef SCORE_Z_ANY
-#undef SCORE_Z_U
-    CU(cudaGetLastError());
-    {
-      Scope sc(this, "small", 1, 0.0, 0.0);
-      gk::k_log_decisions<<<(unsigned)cdiv(M, 128), 128, 0, stream>>>(ctl, M, log_trial_z, log_q_z, d_pass, z_per_pass(),
-                                                                      (long long)(l - 1) * M, kLogPasses);
-    }
-    Scope sc(this, "apply_z", 1, 12.0 * (double)n * ldl, 0.0);
-    gk::k_apply_z<<<grid_for(n * (ldl / 4)), 256, 0, stream>>>((float4*)Z[l], (const float4*)B2, ldl / 4, n, d_row_comm, ctl);
-    CU(cudaGetLastError());
+      Scope sc(this, "close_z", 1, move_bytes, 0.0);
+      launch_together(close, move_blocks, warps * 32, smem, d_row_ptr, d_col, d_col_comm, d_dinv, T, Hn, Zn, R4, ld4, (int)n,
+                      use_smem, d_chunk_ptr, n_chunks, d_items, n_items, long_len, scratch, with_groups(n_chunks));
+    };
+#define SCORE_Z(V)                                                                                           \
+  {                                                                                                          \
+    if (out) score(gk::k_score_z<V, true, 4, kCandZ>, gk::k_close_z<V, true, 4, kCandZ>, V);                 \
+    else score(gk::k_score_z<V, false, 4, kCandZ>, gk::k_close_z<V, false, 4, kCandZ>, V);                   \
+  }
+    if (ld4 <= 32) SCORE_Z(1)
+    else if (ld4 <= 64) SCORE_Z(2)
+    else if (ld4 <= 128) SCORE_Z(4)
+    else SCORE_Z(8)
+#undef SCORE_Z
   }
 
   // ---- Z_L (Eq. 7) and, in the same sweep, the dual as printed in Eq. 3 -----------------
-  void update_output(bool dual_now, bool update_z) {
+  // end_pass: this is the last block family of a pass (the pass counter of the log moves on).
+  void update_output(bool dual_now, bool update_z, bool end_pass) {
     Range range("gcn_admm: output layer and dual");
-    const int warps = 8;
     Scope sc(this, "output_rows", 1, 4.0 * (double)n * ld[L] * (3 + (update_z ? 1 : 0) + (dual_now ? 1 : 0)), 0.0);
-    // rows without a loss term: closed form, plain sweep; training rows: one warp each (FISTA)
-    gk::k_output_plain<<<grid_for(n * (ld[L] / 4)), 256, 0, stream>>>((float4*)Z[L], (float4*)U, (const float4*)H[L],
-                                                                      ld[L] / 4, n, d_train, p.rho, dual_now ? 1 : 0,
-                                                                      update_z ? 1 : 0);
+    gk::OutputArgs a{};
+    a.Z = Z[L]; a.U = U; a.H = H[L];
+    a.ld = ld[L]; a.C = C[L]; a.n = n;
+    a.train = d_train; a.rows = d_train_rows; a.y = d_y; a.n_train = n_train; a.momentum = d_fista_momentum;
+    a.rho = p.rho; a.loss_scale = p.loss_scale; a.iters = p.fista_iters;
+    a.dual_now = dual_now ? 1 : 0; a.update_z = update_z ? 1 : 0;
+    a.advance = end_pass ? d_pass : nullptr;
+    const int plain_blocks = grid_for(n * (ld[L] / 4));
+#define OUTPUT(LPR, CPL)                                                        \
+  {                                                                             \
+    a.train_blocks = (int)cdiv((long long)n_train * (LPR), 256);                \
+    gk::k_output<LPR, CPL><<<(unsigned)(a.train_blocks + plain_blocks), 256, 0, stream>>>(a); \
+  }
+    if (C[L] <= 4) OUTPUT(4, 1)
+    else if (C[L] <= 8) OUTPUT(4, 2)
+    else if (C[L] <= 16) OUTPUT(8, 2)
+    else if (C[L] <= 32) OUTPUT(8, 4)
+    else if (C[L] <= 48) OUTPUT(8, 6)
+    else if (C[L] <= 64) OUTPUT(8, 8)
+    else if (C[L] <= 96) OUTPUT(16, 6)
+    else OUTPUT(16, 8)
+#undef OUTPUT
     CU(cudaGetLastError());
-    if (n_train > 0) {
-#define OUTPUT_ROWS(CPL)                                                                                          \
-  gk::k_output_rows<CPL><<<(unsigned)cdiv(n_train, warps), warps * 32, 0, stream>>>(                              \
-      Z[L], U, H[L], ld[L], C[L], n_train, d_y, d_train, p.rho, p.loss_scale, p.fista_iters, dual_now ? 1 : 0,    \
-      update_z ? 1 : 0, d_train_rows, d_fista_momentum);
-      if (C[L] <= 32) OUTPUT_ROWS(1)
-      else if (C[L] <= 64) OUTPUT_ROWS(2)
-      else if (C[L] <= 96) OUTPUT_ROWS(3)
-      else OUTPUT_ROWS(4)
-#undef OUTPUT_ROWS
-      CU(cudaGetLastError());
-      ++launches;
-    }
   }
 
   void dual_from_stored() {   // U + rho (Z_L - H_L) with H_L = A~ Z_{L-1} W_L of the stored iterates
@@ -761,31 +735,29 @@ struct gcn_admm {
   // W_1, Z_1, .., W_L, Z_L, U, each reading the latest value of every other block.
   void iterate_sequential() {
     if (!fresh) refresh();
-    begin_log_pass();
     for (int l = 1; l <= L; ++l) {
       if (l >= 2) {   // Z_{l-1} has just moved: P_l and H_l follow it (H_{l+1} still matches the untouched Z_l)
         spmm(Z[l - 1], P[l], ld[l - 1]);
         gemm_nn(P[l], ld[l - 1], W[l], ld[l], Wt[l], ld[l - 1], H[l], ld[l], n, C[l], C[l - 1]);
       }
-      update_W(l);
-      if (l < L) update_Z_hidden(l);
-      else update_output(false, true);
+      update_W(l, false);
+      if (l < L) update_Z_hidden(l, false);
+      else update_output(false, true, true);
     }
     refresh(true);
     dual_from_stored();
-    end_log_pass();
+    ++log_count;
   }
 
   void iterate() {   // Algorithm 1, one pass
     if (p.schedule == 1) { iterate_sequential(); return; }
     if (!fresh) refresh();
-    begin_log_pass();
-    for (int l = 1; l <= L; ++l) update_W(l);
-    for (int l = 1; l < L; ++l) update_Z_hidden(l);
-    update_output(p.dual_mode == 0, true);
+    for (int l = 1; l <= L; ++l) update_W(l, l >= 2);
+    for (int l = 1; l < L; ++l) update_Z_hidden(l, true);
+    update_output(p.dual_mode == 0, true, true);
     refresh(true);
     if (p.dual_mode != 0) dual_from_stored();
-    end_log_pass();
+    ++log_count;
   }
 
   // logits of Problem 1's forward pass with the stored W, left in B0 (N x ld_L)
@@ -808,7 +780,9 @@ struct gcn_admm {
     CU(cudaStreamSynchronize(stream));
     if (t != 0) {
       CU(cudaMemsetAsync(tc_error, 0, sizeof(int), stream));
-      throw Fail{GCN_ADMM_ERR_CUDA, "a tensor-core product gave up waiting on its pipeline"};
+      CU(cudaMemsetAsync(grid_bar, 0, sizeof(gk::GridBar), stream));
+      throw Fail{GCN_ADMM_ERR_CUDA, t & gk::kErrGridBarrier ? "a step-size search gave up waiting for the rest of its grid"
+                                                            : "a tensor-core product gave up waiting on its pipeline"};
     }
     if (s & 1) {
       CU(cudaMemsetAsync(status, 0, sizeof(int), stream));
@@ -1005,7 +979,7 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
       const long long n_units = (long long)lt.items.size() + n;
       const long long warps_guess = (long long)kSmCount * 3 * 8;
       // few enough chunks that their sums (M x candidates doubles each) stay small next to the entries they cover
-      const long long target = std::max<long long>({64, std::min<long long>(1024, (long long)g.nnz / (warps_guess * 16)), 16LL * n_comm});
+      const long long target = std::max<long long>({64, std::min<long long>(1024, (long long)g.nnz / (warps_guess * 4)), 2LL * n_comm});
       auto build_chunks = [&](const int* order) {
         std::vector<int> cp;
         cp.push_back(0);
@@ -1044,7 +1018,7 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
   const size_t rows = (size_t)n;
   h->W.assign(L + 1, nullptr); h->Wt.assign(L + 1, nullptr); h->Z.assign(L + 1, nullptr);
   h->P.assign(L + 1, nullptr); h->H.assign(L + 1, nullptr);
-  size_t grad_elems = 1, grad_t_elems = 1;
+  size_t grad_elems = 1, grad_t_elems = 1, grad_blocks = 1;   // grad_blocks: most blocks of a finish_grad launch
   h->part_elems = 1;
   for (int l = 1; l <= L; ++l) {
     h->W[l] = h->alloc<float>((size_t)h->C[l - 1] * h->ld[l]);
@@ -1054,6 +1028,7 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
     h->H[l] = h->alloc<float>(rows * h->ld[l]);
     const size_t ge = (size_t)h->C[l - 1] * h->ld[l];
     grad_elems = std::max(grad_elems, ge);
+    grad_blocks = std::max(grad_blocks, (size_t)h->C[l - 1] * (size_t)cdiv(h->ld[l], 32));
     grad_t_elems = std::max(grad_t_elems, (size_t)h->C[l] * h->ld[l - 1]);
     h->part_elems = std::max(h->part_elems, ge * 4 * kSmCount);
   }
@@ -1065,6 +1040,8 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
   h->B0 = h->alloc<float>(rows * h->max_ld);
   h->B1 = h->alloc<float>(rows * h->max_ld);
   h->B2 = h->alloc<float>(rows * h->max_ld);
+  h->RN.assign(L + 1, nullptr);
+  for (int l = 2; l <= L; ++l) h->RN[l] = l == L ? h->B0 : h->alloc<float>(rows * h->ld[l]);   // R_L is turned into its new value in place
   h->item_sums_elems = std::max<size_t>(1, (size_t)h->n_items * h->max_ld);
   h->item_sums = h->alloc<float>(h->item_sums_elems);
   h->grad = h->alloc<float>(grad_elems);
@@ -1077,16 +1054,15 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
   h->part = h->alloc<float>(h->part_elems);
   h->ctl_w = h->alloc<SearchCtl>(L + 1);
   h->ctl_z = h->alloc<SearchCtl>((size_t)(L + 1) * n_comm);
-  h->sums_w = h->alloc<double>(2);
   h->sums_z = h->alloc<double>((size_t)3 * n_comm);
   h->obj = h->alloc<double>(8);
   {   // row blocks of the hidden-layer gradient's closing sweep, cut at community boundaries
-    std::vector<int2> zb;
+    std::vector<int4> zb;
     std::vector<int> cbp((size_t)n_comm + 1, 0);
     for (int m = 0; m < n_comm; ++m) {
       cbp[m] = (int)zb.size();
       for (int r = g.comm_ptr[m]; r < g.comm_ptr[m + 1]; r += kZBlockRows)
-        zb.push_back(make_int2(r, std::min(r + kZBlockRows, g.comm_ptr[m + 1])));
+        zb.push_back(make_int4(r, std::min(r + kZBlockRows, g.comm_ptr[m + 1]), m, 0));
     }
     cbp[n_comm] = (int)zb.size();
     h->n_zblocks = (int)zb.size();
@@ -1094,12 +1070,18 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
     h->d_comm_block_ptr = upload(h, cbp);
   }
   const int max_chunks = std::max(h->n_chunks, h->n_chunks_sorted);
-  h->n_groups = (int)cdiv(max_chunks, kChunksPerGroup);
   h->z_chunk_part = h->alloc<double>((size_t)max_chunks * n_comm * gk::kCand);
-  h->z_group_part = h->alloc<double>((size_t)h->n_groups * n_comm * gk::kCand);
+  h->z_group_part = h->alloc<double>((size_t)kChunkGroups * n_comm * gk::kCand);
   h->chunk_counter = h->alloc<int>(1);
+  CU(cudaMemset(h->chunk_counter, 0, sizeof(int)));
+  h->ticket = h->alloc<unsigned>(1);
+  CU(cudaMemset(h->ticket, 0, sizeof(unsigned)));
+  h->comm_tickets = h->alloc<unsigned>(n_comm);
+  CU(cudaMemset(h->comm_tickets, 0, n_comm * sizeof(unsigned)));
+  h->grid_bar = h->alloc<gk::GridBar>(1);
+  CU(cudaMemset(h->grid_bar, 0, sizeof(gk::GridBar)));
   h->red_part = h->alloc<double>(std::max<size_t>({(size_t)kSmCount * 8 * gk::kCand, (size_t)h->n_zblocks * 3,
-                                                   (size_t)cdiv(n, 8) * 2}));
+                                                   (size_t)cdiv(n, 8) * 2, grad_blocks * 2}));
   h->n_active = h->alloc<int>(1);
   h->status = h->alloc<int>(1);
   h->d_pass = h->alloc<int>(1);
@@ -1311,19 +1293,19 @@ int gcn_admm_step_block(gcn_admm* h, int phase, int layer) {
     if (!h->fresh) h->refresh();
     h->log_count = 0;
     CU(cudaMemsetAsync(h->d_pass, 0, sizeof(int), h->stream));
-    h->begin_log_pass();
+    h->clear_log_pass();
     if (phase == GCN_ADMM_PHASE_W) {
-      h->update_W(layer);
+      h->update_W(layer, false);
     } else if (phase == GCN_ADMM_PHASE_Z) {
-      if (layer < L) h->update_Z_hidden(layer);
-      else h->update_output(false, true);
+      if (layer < L) h->update_Z_hidden(layer, false);
+      else h->update_output(false, true, false);
       h->fresh = false;
     } else if (phase == GCN_ADMM_PHASE_U) {
       h->dual_from_stored();
     } else {
       throw Fail{GCN_ADMM_ERR_ARG, "unknown phase"};
     }
-    h->end_log_pass();
+    h->log_count = 1;
   });
 }
 
@@ -1488,7 +1470,8 @@ int gcn_admm_dense_product_tn(gcn_admm* h, const float* A, const float* B, float
       CU(cudaMemcpy2DAsync(a, (size_t)lda * 4, A, (size_t)ka * 4, (size_t)ka * 4, (size_t)rows, cudaMemcpyDeviceToDevice, h->stream));
       CU(cudaMemcpy2DAsync(b, (size_t)ldb * 4, B, (size_t)nb * 4, (size_t)nb * 4, (size_t)rows, cudaMemcpyDeviceToDevice, h->stream));
       h->p.tensor_cores = tensor_cores;
-      h->gemm_tn(a, lda, b, ldb, c, ldp, rows, ka, nb);
+      const int splits = h->gemm_tn(a, lda, b, ldb, ldp, rows, ka, nb);
+      h->finish_grad(splits, ka, nb, ldp, c, nullptr, 0, nullptr, nullptr);
       h->p.tensor_cores = saved;
       CU(cudaMemcpy2DAsync(C, (size_t)nb * 4, c, (size_t)ldp * 4, (size_t)nb * 4, (size_t)ka, cudaMemcpyDeviceToDevice, h->stream));
       CU(cudaStreamSynchronize(h->stream));

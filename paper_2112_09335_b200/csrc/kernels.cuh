@@ -614,126 +614,87 @@ k_gemm_tn(const float* __restrict__ A, int lda, const float* __restrict__ B, int
   }
 }
 
-// grad[e] = sum over splits of part[s][e], summed in fp64 in split order (fixed order).
-__global__ void k_reduce_splits(const float* __restrict__ part, float* __restrict__ grad, long long elems,
-                                int splits) {
-  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= elems) return;
-  double s = 0.0;
-  for (int k = 0; k < splits; ++k) s += (double)part[(long long)k * elems + e];
-  grad[e] = (float)s;
-}
-
-// out[0] = sum a^2, out[1] = sum b^2 over `elems` floats (one block, fixed order).
-__global__ void k_two_sumsq(const float* __restrict__ a, const float* __restrict__ b, long long elems,
-                            double* __restrict__ out) {
-  __shared__ double sh[32];
-  double sa = 0.0, sb = 0.0;
-  for (long long e = threadIdx.x; e < elems; e += blockDim.x) {
-    const double x = a[e], y = b[e];
-    sa += x * x;
-    sb += y * y;
-  }
-  sa = block_sum(sa, sh);
-  sb = block_sum(sb, sh);
-  if (threadIdx.x == 0) { out[0] = sa; out[1] = sb; }
-}
-
 // ------------------------------------------------------------------------------------------
 // Residuals with respect to the pre-activation H (derivatives of phi, Section 3):
 //   hidden layer  R = nu (f(H) - Z) * f'(H)
 //   last layer    R = -(U + rho (Z - H))
 // ------------------------------------------------------------------------------------------
+__device__ __forceinline__ float4 resid_hidden(const float4& h, const float4& z, float nu) {
+  return make_float4(h.x > 0.f ? nu * (h.x - z.x) : 0.f, h.y > 0.f ? nu * (h.y - z.y) : 0.f,
+                     h.z > 0.f ? nu * (h.z - z.z) : 0.f, h.w > 0.f ? nu * (h.w - z.w) : 0.f);
+}
+__device__ __forceinline__ float4 resid_out(const float4& h, const float4& z, const float4& u, float rho) {
+  return make_float4(-(u.x + rho * (z.x - h.x)), -(u.y + rho * (z.y - h.y)), -(u.z + rho * (z.z - h.z)), -(u.w + rho * (z.w - h.w)));
+}
+
 __global__ void k_resid_hidden(const float4* __restrict__ H, const float4* __restrict__ Z,
                                float4* __restrict__ R, long long n4, float nu) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n4;
-       i += (long long)gridDim.x * blockDim.x) {
-    const float4 h = H[i], z = Z[i];
-    float4 r;
-    r.x = h.x > 0.f ? nu * (h.x - z.x) : 0.f;
-    r.y = h.y > 0.f ? nu * (h.y - z.y) : 0.f;
-    r.z = h.z > 0.f ? nu * (h.z - z.z) : 0.f;
-    r.w = h.w > 0.f ? nu * (h.w - z.w) : 0.f;
-    R[i] = r;
-  }
+       i += (long long)gridDim.x * blockDim.x)
+    R[i] = resid_hidden(H[i], Z[i], nu);
 }
 
 __global__ void k_resid_out(const float4* __restrict__ H, const float4* __restrict__ Z,
                             const float4* __restrict__ U, float4* __restrict__ R, long long n4, float rho) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n4;
-       i += (long long)gridDim.x * blockDim.x) {
-    const float4 h = H[i], z = Z[i], u = U[i];
-    float4 r;
-    r.x = -(u.x + rho * (z.x - h.x));
-    r.y = -(u.y + rho * (z.y - h.y));
-    r.z = -(u.z + rho * (z.z - h.z));
-    r.w = -(u.w + rho * (z.w - h.w));
-    R[i] = r;
-  }
+       i += (long long)gridDim.x * blockDim.x)
+    R[i] = resid_out(H[i], Z[i], U[i], rho);
 }
 
 // ------------------------------------------------------------------------------------------
-// Step-size search of a W block (Section 3.1).  Along W - grad/t the pre-activation is
-// H - D/t with D = P grad, so every candidate is scored from H, D, Z without another product.
+// Step-size searches (Section 3.1 for W, Eq. 9 for Z).  A search is one cooperative launch: score candidates, add the
+// blocks' sums up in a fixed order, decide, score again while a search is open, then move the block.  As separate
+// launches (ten sweeps of scoring and decision, nine of which usually found nothing to do) this was half of the
+// kernels of a pass and, on graphs of a few thousand nodes, most of its time.
 // ------------------------------------------------------------------------------------------
-// Every block leaves its sums in `partial` (kCand, resp. 2, doubles per block); k_search_decide_w adds the
-// blocks up in a fixed order, so a decision does not depend on how the blocks were scheduled.
-// hidden layer: sum_j = sum ( (z - f(h - d/t_j))^2 - (z - f(h))^2 )   (times nu/2 at decision time)
-__global__ void __launch_bounds__(256)
-k_score_w_hidden(const float4* __restrict__ H, const float4* __restrict__ D, const float4* __restrict__ Z,
-                 long long n4, const SearchCtl* __restrict__ ctl, double* __restrict__ partial) {
-  if (ctl->done) return;
-  __shared__ double sh[32];
-  float inv[kCand];
-#pragma unroll
-  for (int j = 0; j < kCand; ++j) inv[j] = ctl->inv_cand[j];
-  double s[kCand];
-#pragma unroll
-  for (int j = 0; j < kCand; ++j) s[j] = 0.0;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n4;
-       i += (long long)gridDim.x * blockDim.x) {
-    const float4 h4 = H[i], d4 = D[i], z4 = Z[i];
-    const float h[4] = {h4.x, h4.y, h4.z, h4.w}, d[4] = {d4.x, d4.y, d4.z, d4.w},
-                z[4] = {z4.x, z4.y, z4.z, z4.w};
-    float part[kCand];
-#pragma unroll
-    for (int j = 0; j < kCand; ++j) part[j] = 0.f;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const float pos = fmaxf(h[c], 0.f), neg = fmaxf(-h[c], 0.f);
-      const float e2 = 2.f * (z[c] - pos);
-#pragma unroll
-      for (int j = 0; j < kCand; ++j) {
-        const float df = relu_drop(d[c], inv[j], neg, pos);
-        part[j] = fmaf(df, e2 + df, part[j]);   // e1^2 - e0^2 = (e1 - e0)(e1 + e0), e1 - e0 = df
-      }
+// Grid-wide rendezvous of a cooperative launch (all blocks resident).  Every wait is bounded by elapsed clocks (a few
+// seconds); one that runs out raises *err and every block leaves the kernel.
+struct GridBar {
+  unsigned arrived, generation;
+};
+constexpr int kErrGridBarrier = 2;
+constexpr long long kGridWaitClocks = 1LL << 33;
+
+__device__ __forceinline__ unsigned load_acquire(const unsigned* p) {
+  unsigned v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void store_release(unsigned* p, unsigned v) {
+  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+// Waits until every block of the grid has arrived; the last one to arrive runs `last` (with all its threads) before
+// the others are let go.  What blocks wrote before the call is visible to `last`, and what `last` wrote to everyone after it.
+// False when the wait ran out (the same in every thread of the block).
+template <typename F>
+__device__ __forceinline__ bool grid_meet(GridBar* bar, int* err, F&& last) {
+  __shared__ int s_last, s_ok;
+  __syncthreads();
+  unsigned gen = 0;
+  if (threadIdx.x == 0) {
+    gen = load_acquire(&bar->generation);
+    __threadfence();
+    s_last = atomicAdd(&bar->arrived, 1u) == gridDim.x - 1;
+    s_ok = 1;
+  }
+  __syncthreads();
+  if (s_last) {
+    __threadfence();
+    last();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      bar->arrived = 0;
+      __threadfence();
+      store_release(&bar->generation, gen + 1);
     }
-#pragma unroll
-    for (int j = 0; j < kCand; ++j) s[j] += (double)part[j];
+  } else if (threadIdx.x == 0) {
+    const long long t0 = clock64();
+    while (load_acquire(&bar->generation) == gen)
+      if (clock64() - t0 > kGridWaitClocks) { s_ok = 0; atomicOr(err, kErrGridBarrier); break; }
   }
-#pragma unroll
-  for (int j = 0; j < kCand; ++j) {
-    const double v = block_sum(s[j], sh);
-    if (threadIdx.x == 0) partial[(size_t)blockIdx.x * kCand + j] = v;
-  }
-}
-
-// last layer: phi_L(t) - phi_L = -(1/t) <D, R> + (rho / 2t^2) ||D||^2 ; sums <D,R> and ||D||^2
-__global__ void __launch_bounds__(256)
-k_score_w_out(const float4* __restrict__ D, const float4* __restrict__ R, long long n4,
-              const SearchCtl* __restrict__ ctl, double* __restrict__ partial) {
-  if (ctl->done) return;
-  __shared__ double sh[32];
-  double s1 = 0.0, s2 = 0.0;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n4;
-       i += (long long)gridDim.x * blockDim.x) {
-    const float4 d = D[i], r = R[i];
-    s1 += (double)(d.x * r.x + d.y * r.y + d.z * r.z + d.w * r.w);
-    s2 += (double)(d.x * d.x + d.y * d.y + d.z * d.z + d.w * d.w);
-  }
-  s1 = block_sum(s1, sh);
-  s2 = block_sum(s2, sh);
-  if (threadIdx.x == 0) { partial[(size_t)blockIdx.x * 2] = s1; partial[(size_t)blockIdx.x * 2 + 1] = s2; }
+  __syncthreads();
+  return s_ok != 0;
 }
 
 __device__ __forceinline__ void set_candidates(SearchCtl* c, double growth) {
@@ -764,32 +725,6 @@ __device__ __forceinline__ void begin_one(SearchCtl* c, double gg, double xx, do
   if (n_active) atomicAdd(n_active, 1);
 }
 
-// Starts the search of a W block: sums[0] = ||grad||^2, sums[1] = ||W||^2.
-__global__ void k_search_begin(SearchCtl* ctl, const double* __restrict__ sums, double shrink, double growth,
-                               int* __restrict__ status) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) begin_one(ctl, sums[0], sums[1], shrink, growth, nullptr, status);
-}
-
-// Starts the searches of the `count` communities of a hidden layer, one warp each.  k_zgrad_finish left
-// three sums per row block in `partial`; the blocks of community i are block_ptr[i] .. block_ptr[i+1]-1
-// and are added up in a fixed order (lane-strided, then the shuffle tree).  sums[i*3 + ..] receives
-// { ||G_i||^2, ||Z_i||^2, <Z_i - f(H_i), G_i> }.
-__global__ void k_search_begin_z(SearchCtl* ctl, int count, const double* __restrict__ partial,
-                                 const int* __restrict__ block_ptr, double* __restrict__ sums, double shrink,
-                                 double growth, int* __restrict__ n_active, int* __restrict__ status) {
-  const int lane = threadIdx.x & 31;
-  const int i = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  if (i >= count) return;
-  double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-  for (int b = block_ptr[i] + lane; b < block_ptr[i + 1]; b += 32) {
-    s0 += partial[(size_t)b * 3]; s1 += partial[(size_t)b * 3 + 1]; s2 += partial[(size_t)b * 3 + 2];
-  }
-  s0 = warp_sum(s0); s1 = warp_sum(s1); s2 = warp_sum(s2);
-  if (lane != 0) return;
-  sums[i * 3] = s0; sums[i * 3 + 1] = s1; sums[i * 3 + 2] = s2;
-  begin_one(ctl + i, s0, s1, shrink, growth, n_active, status);
-}
-
 // One decision per search.  mode 0: `cand` sums of a scoring pass, delta_j = scale * sum[j]
 // plus the quadratic own term; mode 1: closed form, delta(t) = -lin/t + quad/t^2, all trials at once.
 //   own term (Z blocks only): -(nu/t) sag + (nu/2t^2) sgg with sag = <Z - f(H), G>, sgg = gg
@@ -801,7 +736,6 @@ struct DecideArgs {
   double scale;      // multiplies the scored sums (nu/2)
   double quad_coef;  // closed form: delta = -sum[0]/t + quad_coef * sum[1] / t^2
   double own_nu;     // nu when the block has a quadratic own term, else 0
-  int last_pass;     // this is the final pass: mark exhausted searches
 };
 
 __device__ __forceinline__ bool accept(SearchCtl* c, double delta, double t, int trial) {
@@ -849,7 +783,7 @@ __device__ __forceinline__ bool decide_one(SearchCtl* c, const double* __restric
   if (!finite) atomicOr(status, 1);
   if (ok) { if (n_active) atomicSub(n_active, 1); return false; }
   c->pass += 1;
-  if (a.last_pass || c->pass * a.cand >= a.max_trials) {
+  if (c->pass * a.cand >= a.max_trials) {
     c->done = 1; c->trial = -2; c->inv_step = 0.f;
     if (n_active) atomicSub(n_active, 1);
     return false;
@@ -859,82 +793,192 @@ __device__ __forceinline__ bool decide_one(SearchCtl* c, const double* __restric
   return true;
 }
 
-// Sums of a scoring sweep, first stage: group g adds the chunks g*per_group .. (g+1)*per_group - 1 in chunk
-// order, value by value (width = communities x sums per community): group_part[g][v] = sum_ch chunk_part[ch][v].
-__global__ void k_reduce_chunks(const double* __restrict__ chunk_part, int n_chunks, int per_group, int width,
-                                double* __restrict__ group_part, const int* __restrict__ n_active) {
-  if (*n_active <= 0) return;
-  const int c0 = blockIdx.x * per_group, c1 = min(n_chunks, c0 + per_group);
-  for (int v = threadIdx.x; v < width; v += blockDim.x) {
-    double s = 0.0;
-    for (int ch = c0; ch < c1; ++ch) s += chunk_part[(size_t)ch * width + v];
-    group_part[(size_t)blockIdx.x * width + v] = s;
-  }
-}
-
-// Decisions of the `count` communities of a hidden layer, one warp each.  k_reduce_chunks left the sweep's
-// sums in block_part[(b*count + i)*per + j], b < n_blocks; they are added in a fixed order (lane-strided
-// over b, then the shuffle tree), together with the sums of the segments scored in pieces
-// (split_scores, in the order split_order lists those of community i: split_ptr[i] .. split_ptr[i+1]-1).
-// own[i*3 + 2] = <Z_i - f(H_i), G_i>.
-__global__ void k_search_decide_z(SearchCtl* ctl, int count, const double* __restrict__ block_part, int n_blocks,
-                                  int per, const double* __restrict__ split_scores,
-                                  const int* __restrict__ split_order, const int* __restrict__ split_ptr,
-                                  const double* __restrict__ own, DecideArgs a, int* __restrict__ n_active,
-                                  int* __restrict__ status) {
-  const int lane = threadIdx.x & 31;
-  const int i = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  if (i >= count) return;
-  SearchCtl* c = ctl + i;
-  if (c->done) return;
-  double s[kCand];
-#pragma unroll
-  for (int j = 0; j < kCand; ++j) s[j] = 0.0;
-  for (int b = lane; b < n_blocks; b += 32)
-#pragma unroll
-    for (int j = 0; j < kCand; ++j)
-      if (j < per) s[j] += block_part[((size_t)b * count + i) * per + j];
-  for (int k = split_ptr[i] + lane; k < split_ptr[i + 1]; k += 32) {
-    const size_t at = (size_t)split_order[k] * per;
-#pragma unroll
-    for (int j = 0; j < kCand; ++j)
-      if (j < per) s[j] += split_scores[at + j];
-  }
-#pragma unroll
-  for (int j = 0; j < kCand; ++j) s[j] = warp_sum(s[j]);
-  if (lane != 0) return;
-  decide_one(c, s, own[i * 3 + 2], a, n_active, status);
-}
-
-// Decision of a W block: the `n_part` blocks of the scoring kernel left `per` sums each in `partial`;
-// they are added in a fixed order (thread-strided, then the block tree) before the decision is taken.
-// One block of 256 threads.
-__global__ void __launch_bounds__(256)
-k_search_decide_w(SearchCtl* c, const double* __restrict__ partial, int n_part, int per, DecideArgs a,
-                  int* __restrict__ status) {
-  if (c->done) return;
-  __shared__ double sh[32];
-  __shared__ double total[kCand];
-  for (int j = 0; j < per; ++j) {
-    double s = 0.0;
-    for (int b = threadIdx.x; b < n_part; b += blockDim.x) s += partial[(size_t)b * per + j];
-    s = block_sum(s, sh);
-    if (threadIdx.x == 0) total[j] = s;
-  }
-  if (threadIdx.x == 0) decide_one(c, total, 0.0, a, nullptr, status);
-}
-
 // The decision log is a ring of `ring` passes; the slot in use is *pass mod ring, with the pass counter
 // kept on the device so that a recorded launch sequence stays valid from one pass to the next.
-// Copies the decision of each search into the slot of the current pass.
-__global__ void k_log_decisions(const SearchCtl* __restrict__ ctl, int count, int* __restrict__ trial_base,
-                                double* __restrict__ q_base, const int* __restrict__ pass, long long per_pass,
-                                long long offset, int ring) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= count) return;
-  const long long at = (long long)(*pass % ring) * per_pass + offset + i;
-  trial_base[at] = ctl[i].trial;
-  q_base[at] = ctl[i].q;
+struct DecisionLog {
+  int* trial;
+  double* q;
+  const int* pass;
+  long long per_pass, offset;   // entries of a pass, first entry of this block family
+  int ring;
+};
+__device__ __forceinline__ void log_decision(const DecisionLog& lg, int i, const SearchCtl* c) {
+  const long long at = (long long)(*lg.pass % lg.ring) * lg.per_pass + lg.offset + i;
+  lg.trial[at] = c->trial;
+  lg.q[at] = c->q;
+}
+
+// Weight gradient from its split partial sums, and the start of the W_l search, in one launch:
+//   grad[e] = sum over splits of part[s][e] (fp64, in split order), its transpose, ||grad||^2, ||W||^2.
+// A block owns 32 columns of 8 / SG rows; with many splits SG = 8 threads share an element, each adding its own run of
+// consecutive splits.  The last block to finish adds the blocks' sums of squares in block order and starts the search.
+// W = NULL: only the sum over the splits.
+template <int SG>
+__global__ void __launch_bounds__(256)
+k_finish_grad(const float* __restrict__ part, int splits, int rows, int cols, int ldp, float* __restrict__ grad,
+              float* __restrict__ grad_t, int ldt, const float* __restrict__ W, double* partial, unsigned* ticket,
+              SearchCtl* ctl, double shrink, double growth, int* status) {
+  constexpr int ROWS = 8 / SG;
+  __shared__ double sh[32], s_part[SG][ROWS][32];
+  __shared__ int s_last;
+  const int x = threadIdx.x & 31, y = (threadIdx.x >> 5) % ROWS, sg = (threadIdx.x >> 5) / ROWS;
+  const int col_blocks = (ldp + 31) / 32;
+  const int c = (int)(blockIdx.x % col_blocks) * 32 + x;
+  const int r = (int)(blockIdx.x / col_blocks) * ROWS + y;
+  const bool in = r < rows && c < ldp;
+  const long long elems = (long long)rows * ldp, e = (long long)r * ldp + c;
+  double s = 0.0;
+  if (in) {
+    const int k1 = (int)((long long)splits * (sg + 1) / SG);
+#pragma unroll 8
+    for (int k = (int)((long long)splits * sg / SG); k < k1; ++k) s += (double)part[k * elems + e];
+  }
+  if (SG > 1) {
+    s_part[sg][y][x] = s;
+    __syncthreads();
+    if (sg == 0)
+#pragma unroll
+      for (int k = 1; k < SG; ++k) s += s_part[k][y][x];
+  }
+  double gg = 0.0, ww = 0.0;
+  if (in && sg == 0) {
+    const float g = (float)s;
+    grad[e] = g;
+    if (W != nullptr) {
+      if (c < cols) grad_t[(long long)c * ldt + r] = g;
+      const double w = W[e];
+      gg = (double)g * (double)g;
+      ww = w * w;
+    }
+  }
+  if (W == nullptr) return;
+  gg = block_sum(gg, sh);
+  ww = block_sum(ww, sh);
+  if (threadIdx.x == 0) {
+    partial[2 * (size_t)blockIdx.x] = gg;
+    partial[2 * (size_t)blockIdx.x + 1] = ww;
+    __threadfence();
+    s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  gg = ww = 0.0;
+  for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x) {
+    gg += __ldcg(partial + 2 * (size_t)b);
+    ww += __ldcg(partial + 2 * (size_t)b + 1);
+  }
+  gg = block_sum(gg, sh);
+  ww = block_sum(ww, sh);
+  if (threadIdx.x == 0) {
+    *ticket = 0;
+    begin_one(ctl, gg, ww, shrink, growth, nullptr, status);
+  }
+}
+
+// Search and move of a W block.  Along W - grad/t the pre-activation is H - D/t with D = P grad, so every candidate is
+// scored from H, D, Z without another product:
+//   hidden layer: sum_j = sum ( (z - f(h - d/t_j))^2 - (z - f(h))^2 )   (times nu/2 at decision time), kCand trials a sweep
+//   last layer:   phi_L(t) - phi_L = -(1/t) <D, R> + (rho / 2t^2) ||D||^2 : two sums decide every trial
+// Then W <- W - grad/tau (and its transpose), H <- H - D/tau and, where Rn is given, the derivative of phi_l at the new
+// H, which the gradient of Z_{l-1} starts from (formed here it costs one array less than in a sweep of its own).
+struct SearchW {
+  float4* H;
+  const float4 *D, *Z, *U, *R;      // R: residual at the old H (last layer); U: last layer, for Rn
+  float4* Rn;
+  long long n4;
+  float coef;                       // nu (hidden) or rho (last layer)
+  float *W, *Wt;
+  const float* grad;
+  int rows, cols, ldw, ldwt;
+  SearchCtl* ctl;
+  double* partial;                  // kCand (2) per block
+  GridBar* bar;
+  int *status, *err;
+  DecideArgs a;
+  DecisionLog log;
+};
+template <bool OUT>
+__global__ void __launch_bounds__(256, 4)
+k_search_w(const SearchW p) {
+  constexpr int PER = OUT ? 2 : kCand;
+  __shared__ double sh[32], total[kCand];
+  SearchCtl* const ctl = p.ctl;
+  const long long first = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
+  if (ctl->done) {                  // skipped: the same in every block
+    if (first == 0) log_decision(p.log, 0, ctl);
+  } else {
+    bool open = true;
+    while (open) {
+      double s[PER];
+#pragma unroll
+      for (int j = 0; j < PER; ++j) s[j] = 0.0;
+      if (OUT) {
+        for (long long i = first; i < p.n4; i += stride) {
+          const float4 d = p.D[i], r = p.R[i];
+          s[0] += (double)(d.x * r.x + d.y * r.y + d.z * r.z + d.w * r.w);
+          s[1] += (double)(d.x * d.x + d.y * d.y + d.z * d.z + d.w * d.w);
+        }
+      } else {
+        float inv[kCand];
+#pragma unroll
+        for (int j = 0; j < kCand; ++j) inv[j] = __ldcg(&ctl->inv_cand[j]);
+        for (long long i = first; i < p.n4; i += stride) {
+          const float4 h4 = p.H[i], d4 = p.D[i], z4 = p.Z[i];
+          const float h[4] = {h4.x, h4.y, h4.z, h4.w}, d[4] = {d4.x, d4.y, d4.z, d4.w}, z[4] = {z4.x, z4.y, z4.z, z4.w};
+          float part[kCand];
+#pragma unroll
+          for (int j = 0; j < kCand; ++j) part[j] = 0.f;
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            const float pos = fmaxf(h[c], 0.f), neg = fmaxf(-h[c], 0.f);
+            const float e2 = 2.f * (z[c] - pos);
+#pragma unroll
+            for (int j = 0; j < kCand; ++j) {
+              const float df = relu_drop(d[c], inv[j], neg, pos);
+              part[j] = fmaf(df, e2 + df, part[j]);   // e1^2 - e0^2 = (e1 - e0)(e1 + e0), e1 - e0 = df
+            }
+          }
+#pragma unroll
+          for (int j = 0; j < kCand; ++j) s[j % PER] += (double)part[j];
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < PER; ++j) {
+        const double v = block_sum(s[j], sh);
+        if (threadIdx.x == 0) p.partial[(size_t)blockIdx.x * PER + j] = v;
+      }
+      const bool ok = grid_meet(p.bar, p.err, [&] {
+        for (int j = 0; j < PER; ++j) {
+          double t = 0.0;
+          for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x) t += __ldcg(p.partial + (size_t)b * PER + j);
+          t = block_sum(t, sh);
+          if (threadIdx.x == 0) total[j] = t;
+        }
+        if (threadIdx.x == 0 && !decide_one(ctl, total, 0.0, p.a, nullptr, p.status)) log_decision(p.log, 0, ctl);
+      });
+      if (!ok) return;
+      open = __ldcg(&ctl->done) == 0;
+    }
+  }
+  const float step = __ldcg(&ctl->inv_step);
+  if (step != 0.f)
+    for (long long e = first; e < (long long)p.rows * p.cols; e += stride) {
+      const int r = (int)(e / p.cols), c = (int)(e - (long long)r * p.cols);
+      const float w = fmaf(-p.grad[(long long)r * p.ldw + c], step, p.W[(long long)r * p.ldw + c]);
+      p.W[(long long)r * p.ldw + c] = w;
+      p.Wt[(long long)c * p.ldwt + r] = w;
+    }
+  if (step == 0.f && p.Rn == nullptr) return;
+  for (long long i = first; i < p.n4; i += stride) {
+    float4 h = p.H[i];
+    if (step != 0.f) {
+      const float4 d = p.D[i];
+      h.x = fmaf(-step, d.x, h.x); h.y = fmaf(-step, d.y, h.y); h.z = fmaf(-step, d.z, h.z); h.w = fmaf(-step, d.w, h.w);
+      p.H[i] = h;
+    }
+    if (p.Rn != nullptr) p.Rn[i] = OUT ? resid_out(h, p.Z[i], p.U[i], p.coef) : resid_hidden(h, p.Z[i], p.coef);
+  }
 }
 
 // Marks every entry of the current pass's slot as "not run".
@@ -945,47 +989,22 @@ __global__ void k_log_clear(int* __restrict__ trial_base, const int* __restrict_
     trial_base[at0 + i] = -3;
 }
 
-__global__ void k_pass_advance(int* __restrict__ pass) { *pass += 1; }
-
-// W <- W - grad / tau (and its transpose copy), C_prev x C matrices with padded leading dimensions.
-__global__ void k_apply_w(float* __restrict__ W, float* __restrict__ Wt, const float* __restrict__ grad,
-                          int rows, int cols, int ldw, int ldwt, const SearchCtl* __restrict__ ctl) {
-  const float s = ctl->inv_step;
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= rows * cols) return;
-  const int r = e / cols, c = e % cols;
-  const float w = fmaf(-grad[r * ldw + c], s, W[r * ldw + c]);
-  W[r * ldw + c] = w;
-  Wt[c * ldwt + r] = w;
-}
-
-// Y <- Y - s X with s = ctl->inv_step (H <- H - D/tau).
-__global__ void k_axpy_ctl(float4* __restrict__ Y, const float4* __restrict__ X, long long n4,
-                           const SearchCtl* __restrict__ ctl) {
-  const float s = ctl->inv_step;
-  if (s == 0.f) return;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n4;
-       i += (long long)gridDim.x * blockDim.x) {
-    float4 y = Y[i];
-    const float4 x = X[i];
-    y.x = fmaf(-s, x.x, y.x); y.y = fmaf(-s, x.y, y.y); y.z = fmaf(-s, x.z, y.z); y.w = fmaf(-s, x.w, y.w);
-    Y[i] = y;
-  }
-}
-
 // ------------------------------------------------------------------------------------------
 // Hidden Z blocks (Appendix A).  The gradient of psi_m with respect to Z_{l,m} is the rows V_m of
 //   G = nu (Z_l - f(H_l)) + (A~ R') W_{l+1}^T ,
-// R' the residual of layer l+1 at the new W.  k_zgrad_finish adds the first term to the product and
-// leaves, per row block, partial[b*3 + ..] = { ||G||^2, ||Z_l||^2, <Z_l - f(H_l), G> } over the block's
-// rows.  blocks[b] = {first row, one past the last}: a block never crosses a community boundary, so
-// the sums of a community are the sums of its blocks, added in a fixed order by k_search_begin_z.
+// R' the residual of layer l+1 at the new W.  k_zgrad_finish adds the first term to the product and forms, per
+// community, { ||G||^2, ||Z_l||^2, <Z_l - f(H_l), G> }.  blocks[b] = {first row, one past the last, community, 0}: a
+// block never crosses a community boundary and leaves the sums of its rows in partial[b*3 + ..]; the last block of a
+// community to finish (tickets[m], left at zero) adds the community's blocks block_ptr[m] .. block_ptr[m+1]-1 up in a
+// fixed order and starts its search.
 // ------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256)
 k_zgrad_finish(float4* __restrict__ G, const float4* __restrict__ Z, const float4* __restrict__ H, int ld4,
-               const int2* __restrict__ blocks, float nu, double* __restrict__ partial) {
+               const int4* __restrict__ blocks, float nu, double* partial, const int* __restrict__ block_ptr, unsigned* tickets,
+               SearchCtl* ctl, double* __restrict__ sums, double shrink, double growth, int* n_active, int* status) {
   __shared__ double sh[32];
-  const int2 rb = blocks[blockIdx.x];
+  __shared__ int s_last;
+  const int4 rb = blocks[blockIdx.x];
   double sgg = 0.0, szz = 0.0, sag = 0.0;
   const long long e0 = (long long)rb.x * ld4, e1 = (long long)rb.y * ld4;
   for (long long e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
@@ -999,8 +1018,24 @@ k_zgrad_finish(float4* __restrict__ G, const float4* __restrict__ Z, const float
     sag += (double)(ax * g.x + ay * g.y + az * g.z + aw * g.w);
   }
   sgg = block_sum(sgg, sh); szz = block_sum(szz, sh); sag = block_sum(sag, sh);
+  const int m = rb.z, b0 = block_ptr[m], b1 = block_ptr[m + 1];
   if (threadIdx.x == 0) {
     partial[(size_t)blockIdx.x * 3] = sgg; partial[(size_t)blockIdx.x * 3 + 1] = szz; partial[(size_t)blockIdx.x * 3 + 2] = sag;
+    __threadfence();
+    s_last = atomicAdd(tickets + m, 1u) == (unsigned)(b1 - b0) - 1u;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  sgg = szz = sag = 0.0;
+  for (int b = b0 + threadIdx.x; b < b1; b += blockDim.x) {
+    sgg += __ldcg(partial + (size_t)b * 3); szz += __ldcg(partial + (size_t)b * 3 + 1); sag += __ldcg(partial + (size_t)b * 3 + 2);
+  }
+  sgg = block_sum(sgg, sh); szz = block_sum(szz, sh); sag = block_sum(sag, sh);
+  if (threadIdx.x == 0) {
+    tickets[m] = 0;
+    sums[m * 3] = sgg; sums[m * 3 + 1] = szz; sums[m * 3 + 2] = sag;
+    begin_one(ctl + m, sgg, szz, shrink, growth, n_active, status);
   }
 }
 
@@ -1054,16 +1089,12 @@ __device__ __forceinline__ float4 twice_error(const float4& h, const float4& z) 
 
 // Scores one finished K_m[i] (k, still without the factor di) against the row's a, b:
 // OUT: a = R'; else a = h and b = twice_error(h, z).  The sums (2 when OUT, else NC) go to `slots`:
-// how = 0 added by plain stores (the slots belong to this warp), 1 added atomically, 2 stored.
-__device__ __forceinline__ void put_sum(double* dst, float r, int how) {
-  if (how == 0) *dst += (double)r;
-  else if (how == 1) atomicAdd(dst, (double)r);
-  else *dst = (double)r;
-}
+// add: added to what is there (the slots belong to this warp), else stored.
+__device__ __forceinline__ void put_sum(double* dst, float r, bool add) { *dst = add ? *dst + (double)r : (double)r; }
 template <int V, bool OUT, int NC>
 __device__ __forceinline__ void score_segment(const float4 (&k)[V], float di, const float4 (&a)[V],
-                                              const float4 (&b)[V], const SearchCtl* __restrict__ ctl,
-                                              int cur, int lane, double* slots, int how) {
+                                              const float4 (&b)[V], const float* inv_cand, int lane, double* slots,
+                                              bool add) {
   if (OUT) {
     float p1 = 0.f, p2 = 0.f;
 #pragma unroll
@@ -1073,12 +1104,12 @@ __device__ __forceinline__ void score_segment(const float4 (&k)[V], float di, co
       p2 += kx * kx + ky * ky + kz * kz + kw * kw;
     }
     const float r = warp_sum2(p1, p2, lane);
-    if ((lane & 15) == 0) put_sum(slots + (lane >> 4), r, how);
+    if ((lane & 15) == 0) put_sum(slots + (lane >> 4), r, add);
   } else {
     static_assert(NC >= 2 && NC <= 4, "two to four candidates per sweep");
     float inv[NC], part[NC];
 #pragma unroll
-    for (int j = 0; j < NC; ++j) { inv[j] = di * ctl[cur].inv_cand[j]; part[j] = 0.f; }   // K_m[i] = di * k
+    for (int j = 0; j < NC; ++j) { inv[j] = di * inv_cand[j]; part[j] = 0.f; }   // K_m[i] = di * k
 #pragma unroll
     for (int v = 0; v < V; ++v) {
       const float kk[4] = {k[v].x, k[v].y, k[v].z, k[v].w};
@@ -1096,37 +1127,153 @@ __device__ __forceinline__ void score_segment(const float4 (&k)[V], float di, co
     }
     if constexpr (NC >= 3) {
       const float r = warp_sum4(part[0], part[1], part[2], NC == 4 ? part[NC - 1] : 0.f, lane);
-      if ((lane & 7) == 0 && (lane >> 3) < NC) put_sum(slots + (lane >> 3), r, how);
+      if ((lane & 7) == 0 && (lane >> 3) < NC) put_sum(slots + (lane >> 3), r, add);
     } else {
       const float r = warp_sum2(part[0], part[1], lane);
-      if ((lane & 15) == 0) put_sum(slots + (lane >> 4), r, how);
+      if ((lane & 15) == 0) put_sum(slots + (lane >> 4), r, add);
     }
   }
 }
 
+// What the search of a hidden layer's Z blocks needs beside the scoring kernel's own operands.
+struct SearchZ {
+  SearchCtl* ctl;                    // one per community
+  int n_comm;
+  double* chunk_part;                // [chunk][community][sums] of a sweep
+  int* chunk_counter;                // hands the chunks out; left at zero
+  double* group_part;                // [group of chunks][community][sums], used when n_groups > 0
+  int n_groups, per_group;
+  const int4* split;                 // segments scored in pieces: {row, community, first item, number of items}
+  int n_split;
+  double* split_scores;
+  const int *split_order, *split_ptr;   // their order by community
+  const double* own;                 // [community][3] from k_zgrad_finish; [2] = <Z - f(H), G>
+  int *n_active, *status, *err;
+  GridBar* bar;
+  DecideArgs a;
+  DecisionLog log;
+  float4* Z;                         // the block that moves, its gradient, their width, community of every row
+  const float4* G;
+  int ldz4;
+  const int* row_comm;
+};
+
+// Closes a sweep.  Segments that were scored in pieces: K_m[i] = sum of the pieces (item order), then scored like any
+// other, one warp each.  With many chunks their sums are first added group by group, in chunk order.  Then one warp per
+// community adds up its groups (or chunks; lane-strided, then the shuffle tree) and its split segments in table order,
+// and takes the decision.  No sum depends on which warp scored which chunk.
+template <int V, bool OUT, int NC>
+__device__ __forceinline__ bool close_sweep(const SearchZ& p, int n_chunks, const float* __restrict__ dinv, const float4* scratch,
+                                            const float4* __restrict__ Hn, const float4* __restrict__ Zn,
+                                            const float4* __restrict__ Rn, int ld4) {
+  constexpr int PER = OUT ? 2 : NC;
+  const int lane = threadIdx.x & 31;
+  const int gwarp = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), n_warps = (int)((gridDim.x * blockDim.x) >> 5);
+  const auto nothing = [] {};
+  if (blockIdx.x == 0 && threadIdx.x == 0) *p.chunk_counter = 0;
+  if (p.n_split > 0 || p.n_groups > 0) {
+    for (int s = gwarp; s < p.n_split; s += n_warps) {
+      const int4 sp = p.split[s];
+      if (p.ctl[sp.y].done) continue;
+      float4 a[V], b[V], k[V];
+#pragma unroll
+      for (int v = 0; v < V; ++v) {
+        const int f = lane + 32 * v;
+        a[v] = b[v] = k[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (f < ld4) {
+          if (OUT) a[v] = Rn[(long long)sp.x * ld4 + f];
+          else { a[v] = Hn[(long long)sp.x * ld4 + f]; b[v] = twice_error(a[v], Zn[(long long)sp.x * ld4 + f]); }
+          for (int q = 0; q < sp.w; ++q) k[v] = vadd(k[v], __ldcg(scratch + (long long)(sp.z + q) * ld4 + f));
+        }
+      }
+      score_segment<V, OUT, NC>(k, dinv[sp.x], a, b, p.ctl[sp.y].inv_cand, lane, p.split_scores + (size_t)s * PER, false);
+    }
+    const int width = p.n_comm * PER;
+    for (int g = blockIdx.x; g < p.n_groups; g += gridDim.x) {
+      const int c1 = min(n_chunks, (g + 1) * p.per_group);
+      for (int v = threadIdx.x; v < width; v += blockDim.x) {
+        double s = 0.0;
+#pragma unroll 8
+        for (int ch = g * p.per_group; ch < c1; ++ch) s += __ldcg(p.chunk_part + (size_t)ch * width + v);
+        p.group_part[(size_t)g * width + v] = s;
+      }
+    }
+    if (!grid_meet(p.bar, p.err, nothing)) return false;
+  }
+  const double* const parts = p.n_groups > 0 ? p.group_part : p.chunk_part;
+  const int n_parts = p.n_groups > 0 ? p.n_groups : n_chunks;
+  for (int i = gwarp; i < p.n_comm; i += n_warps) {
+    SearchCtl* c = p.ctl + i;
+    if (c->done) continue;
+    double s[PER];
+#pragma unroll
+    for (int j = 0; j < PER; ++j) s[j] = 0.0;
+    for (int b = lane; b < n_parts; b += 32)
+#pragma unroll
+      for (int j = 0; j < PER; ++j) s[j] += __ldcg(parts + ((size_t)b * p.n_comm + i) * PER + j);
+    for (int k = p.split_ptr[i] + lane; k < p.split_ptr[i + 1]; k += 32) {
+      const size_t at = (size_t)p.split_order[k] * PER;
+#pragma unroll
+      for (int j = 0; j < PER; ++j) s[j] += __ldcg(p.split_scores + at + j);
+    }
+#pragma unroll
+    for (int j = 0; j < PER; ++j) s[j] = warp_sum(s[j]);
+    if (lane == 0) decide_one(c, s, p.own[i * 3 + 2], p.a, p.n_active, p.status);
+  }
+  return grid_meet(p.bar, p.err, nothing);
+}
+
+// After the last sweep: the decisions go to the log and every block moves, Z_l[i,:] <- Z_l[i,:] - G[i,:] / theta_{comm(i)} (Eq. 10).
+__device__ __forceinline__ void move_blocks(const SearchZ& p, long long n) {
+  const long long first = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
+  for (long long i = first; i < p.n_comm; i += stride) log_decision(p.log, (int)i, p.ctl + i);
+  // four elements per thread in flight: the kernel holds few warps (its scoring loop takes the registers)
+  const long long total = n * p.ldz4;   // below 2^32
+  for (long long e0 = first; e0 < total; e0 += 4 * stride) {
+    float s[4];
+    float4 g[4], z[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const long long e = e0 + k * stride;
+      s[k] = 0.f;
+      if (e < total) {
+        s[k] = p.ctl[p.row_comm[(unsigned)e / (unsigned)p.ldz4]].inv_step;
+        g[k] = __ldcs(p.G + e);
+        z[k] = p.Z[e];
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (s[k] != 0.f) p.Z[e0 + k * stride] = vfma(-s[k], g[k], z[k]);
+  }
+}
+
+// One sweep over all chunks by the warps of the grid.  Dynamic shared memory: per warp the row's a, b (2 V float4 per
+// lane; parked there during the walk so that the registers hold gathered rows instead), the candidates of every community
+// (one float4; negative when its search is closed), then the per-warp sums; the last two only with use_smem.
 template <int V, bool OUT, int UN, int NC>
-__global__ void __launch_bounds__(256, (V <= 1 ? 4 : V <= 2 ? 3 : 1))
-k_score_z(const int* __restrict__ row_ptr, const int* __restrict__ col,
+__device__ __forceinline__ void score_sweep(const int* __restrict__ row_ptr, const int* __restrict__ col,
           const unsigned short* __restrict__ col_comm, const float* __restrict__ dinv,
           const float4* __restrict__ T, const float4* __restrict__ Hn, const float4* __restrict__ Zn,
-          const float4* __restrict__ Rn, int ld4, int n, const SearchCtl* __restrict__ ctl, int n_comm,
-          double* __restrict__ chunk_part, const int* __restrict__ n_active, int use_smem,
-          const int* __restrict__ chunk_ptr, int n_chunks, int* __restrict__ chunk_counter,
-          const int4* __restrict__ items, int n_items, int long_len, float4* __restrict__ scratch,
-          const int* __restrict__ row_order) {
-  if (*n_active <= 0) return;
+          const float4* __restrict__ Rn, int ld4, const SearchCtl* ctl, int n_comm, double* chunk_part, int use_smem,
+          const int* __restrict__ chunk_ptr, int n_chunks, int* chunk_counter,
+          const int4* __restrict__ items, int n_items, int long_len, float4* scratch) {
   constexpr int PER = OUT ? 2 : NC;
-  // dynamic shared memory: per warp the row's a, b (2 V float4 per lane; parked there during the
-  // walk so that the registers hold gathered rows instead), then the per-warp sums
   extern __shared__ float4 s_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int warps_per_block = blockDim.x >> 5;
   float4* row_ab = s_raw + (size_t)warp * (2 * V * 32) + lane;
-  double* s_acc = reinterpret_cast<double*>(s_raw + (size_t)warps_per_block * (2 * V * 32));
+  float4* const s_cand = s_raw + (size_t)warps_per_block * (2 * V * 32);
+  double* s_acc = reinterpret_cast<double*>(s_cand + n_comm);
   double* mine = nullptr;   // the sums of the chunk in hand, [community][PER]
   if (use_smem) {
     for (int i = threadIdx.x; i < warps_per_block * n_comm * PER; i += blockDim.x) s_acc[i] = 0.0;
     mine = s_acc + (size_t)warp * n_comm * PER;
+    for (int m = threadIdx.x; m < n_comm; m += blockDim.x) {   // written by other blocks in a sweep after the first: not through L1
+      const SearchCtl* c = ctl + m;
+      s_cand[m] = __ldcg(&c->done) ? make_float4(-1.f, 0.f, 0.f, 0.f)
+                                   : make_float4(__ldcg(c->inv_cand), __ldcg(c->inv_cand + 1), __ldcg(c->inv_cand + 2), __ldcg(c->inv_cand + 3));
+    }
   }
   __syncthreads();
   const float4* __restrict__ T_lane = T + lane;   // rows of T are addressed by 32-bit float4 offsets (n * ld4 < 2^32)
@@ -1138,7 +1285,7 @@ k_score_z(const int* __restrict__ row_ptr, const int* __restrict__ col,
   // lengths follow a power law and the time a chunk takes depends on what its rows find in L2, so any
   // static deal leaves most warps waiting for the unlucky ones.  A chunk is scored by one warp, units in
   // order, and its sums go to chunk_part[chunk][community][PER]; they are added up in chunk order
-  // afterwards (k_reduce_chunks, k_search_decide_z), so no sum depends on which warp took which chunk.
+  // afterwards (close_sweep), so no sum depends on which warp took which chunk.
   // With room in shared memory the chunk's sums are kept there and copied out at the end of the chunk;
   // otherwise (too many communities) the warp adds into the chunk's slice of chunk_part directly.
   for (;;) {
@@ -1161,7 +1308,7 @@ k_score_z(const int* __restrict__ row_ptr, const int* __restrict__ col,
       const int u = unit_base + lane;
       if (u < n_items) my_unit = items[u];
       else {
-        const int r = row_order != nullptr ? row_order[u - n_items] : u - n_items;
+        const int r = u - n_items;
         my_unit = make_int4(r, row_ptr[r], row_ptr[r + 1], -1);
         if (my_unit.z - my_unit.y > long_len) my_unit.z = my_unit.y;   // walked as items
       }
@@ -1219,7 +1366,8 @@ k_score_z(const int* __restrict__ row_ptr, const int* __restrict__ col,
         a[v] = row_ab[32 * v];
         b[v] = OUT ? a[v] : row_ab[32 * (V + v)];
       }
-      score_segment<V, OUT, NC>(k, di, a, b, ctl, cur, lane, mine + cur * PER, 0);
+      score_segment<V, OUT, NC>(k, di, a, b, use_smem ? reinterpret_cast<const float*>(s_cand + cur) : ctl[cur].inv_cand, lane,
+                                mine + cur * PER, true);
     };
 
     // column and community of a chunk are fetched while the chunk before it is walked; the two
@@ -1235,7 +1383,7 @@ k_score_z(const int* __restrict__ row_ptr, const int* __restrict__ col,
       bool live = false;      // the entry's community is still searching: its row of T is gathered
       if (valid) {
         const float wc = dinv[c];
-        live = !ctl[m].done;
+        live = use_smem ? s_cand[m].x >= 0.f : __ldcg(&ctl[m].done) == 0;
         if (live) { w = wc; off = (unsigned)c * (unsigned)ld4; }
       }
       // entries of one community are contiguous: bit t of `chg` says that entry t opens a new
@@ -1296,45 +1444,82 @@ k_score_z(const int* __restrict__ row_ptr, const int* __restrict__ col,
   }
 }
 
-// The output-layer form of k_score_z (OUT = true) for rows of at most 16 float4 (C_L <= 64), two
-// units per warp: each half-warp walks its own row or item, 16 stored entries per chunk.  With 12 of
-// 32 lanes carrying columns (47 classes) the full-warp form spends most of its issue slots on lanes
-// that hold nothing; here every instruction of the walk serves two rows.  Control flow is kept the
-// same for both halves (loop bounds are the larger of the two, a half that has run out holds weight 0
-// and no segment start), shuffles use width 16, and only the closing of a segment is a divergent
-// branch, inside which nothing is exchanged beyond the half's own 16 lanes.  Sums go to one array
-// per half-warp (the halves may close segments of the same community at the same time).
-// Dynamic shared memory: 2 x warps x n_comm x 2 doubles (the caller uses k_score_z when that does not fit).
-template <int UN>
+template <int V, bool OUT, int UN, int NC>
+__global__ void __launch_bounds__(256, (V <= 1 ? 4 : V <= 2 ? 3 : 1))
+k_score_z(const int* __restrict__ row_ptr, const int* __restrict__ col,
+          const unsigned short* __restrict__ col_comm, const float* __restrict__ dinv,
+          const float4* __restrict__ T, const float4* __restrict__ Hn, const float4* __restrict__ Zn,
+          const float4* __restrict__ Rn, int ld4, const SearchCtl* __restrict__ ctl, int n_comm,
+          double* __restrict__ chunk_part, const int* __restrict__ n_active, int use_smem,
+          const int* __restrict__ chunk_ptr, int n_chunks, int* __restrict__ chunk_counter,
+          const int4* __restrict__ items, int n_items, int long_len, float4* __restrict__ scratch) {
+  if (*n_active <= 0) return;
+  score_sweep<V, OUT, UN, NC>(row_ptr, col, col_comm, dinv, T, Hn, Zn, Rn, ld4, ctl, n_comm, chunk_part, use_smem, chunk_ptr, n_chunks,
+                              chunk_counter, items, n_items, long_len, scratch);
+}
+
+// The rest of the search, cooperative: closes the sweep that k_score_z (or k_score_z_out_part) has just made, makes and
+// closes further ones while a community is still searching (hidden layers), and moves the blocks.  The first sweep has a
+// kernel of its own because, compiled together with this one, its walk spills registers (2.4 M rows x 256: 14.9 against 13.6 ms).
+template <int V, bool OUT, int UN, int NC>
+__global__ void __launch_bounds__(256, (OUT ? 4 : V <= 2 ? 3 : 1))
+k_close_z(const int* __restrict__ row_ptr, const int* __restrict__ col,
+          const unsigned short* __restrict__ col_comm, const float* __restrict__ dinv,
+          const float4* __restrict__ T, const float4* __restrict__ Hn, const float4* __restrict__ Zn,
+          const float4* __restrict__ Rn, int ld4, int n, int use_smem, const int* __restrict__ chunk_ptr, int n_chunks,
+          const int4* __restrict__ items, int n_items, int long_len, float4* scratch, const SearchZ sz) {
+  if (__ldcg(sz.n_active) > 0) {
+    for (;;) {
+      if (!close_sweep<V, OUT, NC>(sz, n_chunks, dinv, scratch, Hn, Zn, Rn, ld4)) return;
+      if (OUT || __ldcg(sz.n_active) <= 0) break;   // changes only between the meetings of close_sweep
+      score_sweep<V, OUT, UN, NC>(row_ptr, col, col_comm, dinv, T, Hn, Zn, Rn, ld4, sz.ctl, sz.n_comm, sz.chunk_part, use_smem, chunk_ptr,
+                                  n_chunks, sz.chunk_counter, items, n_items, long_len, scratch);
+      if (!grid_meet(sz.bar, sz.err, [] {})) return;
+    }
+  }
+  move_blocks(sz, n);
+}
+
+// The output-layer form of k_score_z (OUT = true) for rows of at most G float4 (G = 4, 8, 16: C_L <= 16, 32, 64): 32 / G
+// units per warp, each group of G lanes walking its own row or item, G stored entries per chunk.  With 12 of 32 lanes
+// carrying columns (47 classes), or one (3 classes), the full-warp form spends most of its issue slots on lanes that hold
+// nothing and walks one row where the warp could walk eight.  Control flow is kept the same for all groups (loop bounds
+// are the largest of them, a group that has run out holds weight 0 and no segment start), shuffles use width G, and only
+// the closing of a segment is a divergent branch, inside which nothing is exchanged beyond the group's own lanes.  Sums go to one
+// array per group (groups may close segments of the same community at the same time).
+// Dynamic shared memory: (32 / G) x warps x n_comm x 2 doubles (the caller takes a larger G, then k_score_z, when that
+// does not fit).
+template <int G, int UN>
 __global__ void __launch_bounds__(256, 4)
-k_score_z_out_half(const int* __restrict__ row_ptr, const int* __restrict__ col,
+k_score_z_out_part(const int* __restrict__ row_ptr, const int* __restrict__ col,
                    const unsigned short* __restrict__ col_comm, const float* __restrict__ dinv,
-                   const float4* __restrict__ T, const float4* __restrict__ Rn, int ld4, int n,
+                   const float4* __restrict__ T, const float4* __restrict__ Rn, int ld4,
                    const SearchCtl* __restrict__ ctl, int n_comm, double* __restrict__ chunk_part,
                    const int* __restrict__ n_active, const int* __restrict__ chunk_ptr, int n_chunks,
                    int* __restrict__ chunk_counter,
                    const int4* __restrict__ items, int n_items, int long_len, float4* __restrict__ scratch,
                    const int* __restrict__ row_order) {
   if (*n_active <= 0) return;
-  static_assert(16 % UN == 0, "UN divides the chunk");
-  extern __shared__ double s_half[];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, half = lane >> 4, hl = lane & 15;
+  static_assert(G % UN == 0, "UN divides the chunk");
+  constexpr int GROUPS = 32 / G;
+  extern __shared__ double s_part[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, grp = lane / G, gl = lane & (G - 1);
   const int warps_per_block = blockDim.x >> 5;
-  const unsigned hmask = 0xffffu << (16 * half);
-  for (int i = threadIdx.x; i < 2 * warps_per_block * n_comm * 2; i += blockDim.x) s_half[i] = 0.0;
-  double* const mine = s_half + (size_t)(2 * warp + half) * n_comm * 2;   // the half-warp's sums of the chunk in hand
+  constexpr unsigned kGroupMask = G == 32 ? 0xffffffffu : ((1u << G) - 1u);
+  const unsigned gmask = kGroupMask << (G * grp);
+  for (int i = threadIdx.x; i < GROUPS * warps_per_block * n_comm * 2; i += blockDim.x) s_part[i] = 0.0;
+  double* const mine = s_part + (size_t)(GROUPS * warp + grp) * n_comm * 2;   // the group's sums of the chunk in hand
   __syncthreads();
-  const bool in_row = hl < ld4;
-  const float4* __restrict__ T_lane = T + hl;
+  const bool in_row = gl < ld4;
+  const float4* __restrict__ T_lane = T + gl;
   for (;;) {   // chunks from a global counter, their sums to chunk_part: see k_score_z
     int ch = 0;
     if (lane == 0) ch = atomicAdd(chunk_counter, 1);
     ch = __shfl_sync(0xffffffffu, ch, 0);
     if (ch >= n_chunks) break;
     const int chunk_end = chunk_ptr[ch + 1];
-  for (int unit_base = chunk_ptr[ch]; unit_base < chunk_end; unit_base += 4) {
-    for (int pair = 0; pair < 2; ++pair) {
-      const int unit = unit_base + 2 * pair + half;
+    for (int unit0 = chunk_ptr[ch]; unit0 < chunk_end; unit0 += GROUPS) {
+      const int unit = unit0 + grp;
       int row = 0, rs = 0, re = 0;
       bool piece = false;
       if (unit < chunk_end) {
@@ -1349,38 +1534,39 @@ k_score_z_out_half(const int* __restrict__ row_ptr, const int* __restrict__ col,
         }
       }
       float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (in_row && !piece && re > rs) a = Rn[(long long)row * ld4 + hl];
+      if (in_row && !piece && re > rs) a = Rn[(long long)row * ld4 + gl];
       const float di = dinv[row];
       float4 k = make_float4(0.f, 0.f, 0.f, 0.f);
       int cur = -1;
       bool cur_on = false;
 
-      auto finish_segment = [&]() {   // called by one half at a time: exchanges stay inside hmask
+      auto finish_segment = [&]() {   // called by one group at a time: exchanges stay inside gmask
         if (!cur_on) return;
         if (piece) {
-          if (in_row) scratch[(long long)unit * ld4 + hl] = k;
+          if (in_row) scratch[(long long)unit * ld4 + gl] = k;
           return;
         }
         const float kx = di * k.x, ky = di * k.y, kz = di * k.z, kw = di * k.w;
         const float p1 = kx * a.x + ky * a.y + kz * a.z + kw * a.w;
         const float p2 = kx * kx + ky * ky + kz * kz + kw * kw;
-        const bool up8 = hl & 8;
-        float c = (up8 ? p2 : p1) + __shfl_xor_sync(hmask, up8 ? p1 : p2, 8, 16);
-        c += __shfl_xor_sync(hmask, c, 4, 16);
-        c += __shfl_xor_sync(hmask, c, 2, 16);
-        c += __shfl_xor_sync(hmask, c, 1, 16);
-        if ((hl & 7) == 0) put_sum(mine + cur * 2 + (hl >> 3), c, 0);
+        const bool up = gl & (G / 2);
+        float c = (up ? p2 : p1) + __shfl_xor_sync(gmask, up ? p1 : p2, G / 2, G);
+#pragma unroll
+        for (int o = G / 4; o > 0; o >>= 1) c += __shfl_xor_sync(gmask, c, o, G);
+        if ((gl & (G / 2 - 1)) == 0) put_sum(mine + cur * 2 + (up ? 1 : 0), c, true);
       };
 
       const int len = re - rs;
-      const int len_max = max(len, __shfl_xor_sync(0xffffffffu, len, 16));
+      int len_max = len;
+#pragma unroll
+      for (int o = G; o < 32; o <<= 1) len_max = max(len_max, __shfl_xor_sync(0xffffffffu, len_max, o));
       int c_next = 0, m_next = -1;   // fetched one chunk ahead, as in k_score_z
-      if (rs + hl < re) { c_next = col[rs + hl]; m_next = col_comm[rs + hl]; }
-      for (int o = 0; o < len_max; o += 16) {
-        const int idx = rs + o + hl;
+      if (rs + gl < re) { c_next = col[rs + gl]; m_next = col_comm[rs + gl]; }
+      for (int o = 0; o < len_max; o += G) {
+        const int idx = rs + o + gl;
         const bool valid = idx < re;
         const int c = c_next, m = m_next;
-        if (idx + 16 < re) { c_next = col[idx + 16]; m_next = col_comm[idx + 16]; }
+        if (idx + G < re) { c_next = col[idx + G]; m_next = col_comm[idx + G]; }
         else m_next = -1;
         unsigned off = 0u;
         float w = 0.f;
@@ -1390,16 +1576,16 @@ k_score_z_out_half(const int* __restrict__ row_ptr, const int* __restrict__ col,
           live = !ctl[m].done;
           if (live) { w = wc; off = (unsigned)c * (unsigned)ld4; }
         }
-        int mprev = __shfl_up_sync(0xffffffffu, m, 1, 16);
-        if (hl == 0) mprev = cur;
-        unsigned chg = (__ballot_sync(0xffffffffu, valid && m != mprev) >> (16 * half)) & 0xffffu;
-        const unsigned on_both = __ballot_sync(0xffffffffu, live);
-        unsigned on = (on_both >> (16 * half)) & 0xffffu;
-        const int cnt_max = min(16, len_max - o);
-        if (on_both == 0u) {   // neither half has anything to gather in this chunk
-          if (chg != 0u) {     // per half: an open segment ends at the chunk's first entry
+        int mprev = __shfl_up_sync(0xffffffffu, m, 1, G);
+        if (gl == 0) mprev = cur;
+        unsigned chg = (__ballot_sync(0xffffffffu, valid && m != mprev) >> (G * grp)) & kGroupMask;
+        const unsigned on_all = __ballot_sync(0xffffffffu, live);
+        unsigned on = (on_all >> (G * grp)) & kGroupMask;
+        const int cnt_max = min(G, len_max - o);
+        if (on_all == 0u) {   // no group has anything to gather in this chunk
+          if (chg != 0u) {    // per group: an open segment ends at the chunk's first entry
             finish_segment();
-            cur = __shfl_sync(hmask, m, min(16, len - o) - 1, 16);
+            cur = __shfl_sync(gmask, m, min(G, len - o) - 1, G);
             cur_on = false;
           }
           continue;
@@ -1409,8 +1595,8 @@ k_score_z_out_half(const int* __restrict__ row_ptr, const int* __restrict__ col,
           float wj[UN];
 #pragma unroll
           for (int u = 0; u < UN; ++u) {
-            oj[u] = __shfl_sync(0xffffffffu, off, t + u, 16);
-            wj[u] = __shfl_sync(0xffffffffu, w, t + u, 16);
+            oj[u] = __shfl_sync(0xffffffffu, off, t + u, G);
+            wj[u] = __shfl_sync(0xffffffffu, w, t + u, G);
           }
           float4 xv[UN];   // set and read under the same condition
 #pragma unroll
@@ -1418,172 +1604,129 @@ k_score_z_out_half(const int* __restrict__ row_ptr, const int* __restrict__ col,
             if (((on >> u) & 1u) && in_row) xv[u] = __ldg(T_lane + oj[u]);
 #pragma unroll
           for (int u = 0; u < UN; ++u) {
-            if ((chg >> u) & 1u) {                        // uniform within the half
+            if ((chg >> u) & 1u) {                        // uniform within the group
               finish_segment();
               cur = col_comm[rs + o + t + u];
               cur_on = (on >> u) & 1u;
               k = make_float4(0.f, 0.f, 0.f, 0.f);
             }
-            if (((on >> u) & 1u) && in_row) {
-              k.x = fmaf(wj[u], xv[u].x, k.x); k.y = fmaf(wj[u], xv[u].y, k.y);
-              k.z = fmaf(wj[u], xv[u].z, k.z); k.w = fmaf(wj[u], xv[u].w, k.w);
-            }
+            if (((on >> u) & 1u) && in_row) k = vfma(wj[u], xv[u], k);
           }
         }
       }
       finish_segment();
       __syncwarp();
     }
-  }
-    // the chunk's sums: lower half-warp first, then the upper one
-    double* const lo = s_half + (size_t)(2 * warp) * n_comm * 2;
-    double* const hi = lo + (size_t)n_comm * 2;
+    // the chunk's sums, group after group
+    double* const warp_sums = s_part + (size_t)(GROUPS * warp) * n_comm * 2;
     double* const out_part = chunk_part + (size_t)ch * n_comm * 2;
-    for (int i = lane; i < n_comm * 2; i += 32) { out_part[i] = lo[i] + hi[i]; lo[i] = 0.0; hi[i] = 0.0; }
+    for (int i = lane; i < n_comm * 2; i += 32) {
+      double t = 0.0;
+#pragma unroll
+      for (int g = 0; g < GROUPS; ++g) { t += warp_sums[(size_t)g * n_comm * 2 + i]; warp_sums[(size_t)g * n_comm * 2 + i] = 0.0; }
+      out_part[i] = t;
+    }
     __syncwarp();
   }
 }
 
-// Segments that k_score_z handled in pieces: K_m[i] = sum of the pieces (item order), then scored
-// as above.  split[s] = {row, community, first item, number of items}; one warp per entry, whose sums
-// go to split_scores[s*PER ..] (PER = 2 when OUT, else NC); k_search_decide_z adds them in table order.
-template <int V, bool OUT, int NC>
-__global__ void __launch_bounds__(256)
-k_score_z_split(const int4* __restrict__ split, int n_split, const float* __restrict__ dinv,
-                const float4* __restrict__ scratch, const float4* __restrict__ Hn, const float4* __restrict__ Zn,
-                const float4* __restrict__ Rn, int ld4, const SearchCtl* __restrict__ ctl,
-                double* __restrict__ split_scores, const int* __restrict__ n_active) {
-  if (*n_active <= 0) return;
-  const int lane = threadIdx.x & 31;
-  const int s = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  if (s >= n_split) return;
-  const int4 sp = split[s];
-  if (ctl[sp.y].done) return;
-  float4 a[V], b[V], k[V];
-#pragma unroll
-  for (int v = 0; v < V; ++v) {
-    const int f = lane + 32 * v;
-    a[v] = b[v] = k[v] = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (f < ld4) {
-      if (OUT) a[v] = Rn[(long long)sp.x * ld4 + f];
-      else { a[v] = Hn[(long long)sp.x * ld4 + f]; b[v] = twice_error(a[v], Zn[(long long)sp.x * ld4 + f]); }
-      for (int q = 0; q < sp.w; ++q) {
-        const float4 t = scratch[(long long)(sp.z + q) * ld4 + f];
-        k[v].x += t.x; k[v].y += t.y; k[v].z += t.z; k[v].w += t.w;
-      }
-    }
-  }
-  score_segment<V, OUT, NC>(k, dinv[sp.x], a, b, ctl, sp.y, lane, split_scores + (size_t)s * (OUT ? 2 : NC), 2);
-}
-
-// The rows of Eq. 7 without a loss term (not in the training set) have the closed form
-// z = q - u / rho; with dual_now, U <- u + rho (z_old - q) first (Eq. 3 as printed).  Plain
-// elementwise sweep; training rows are skipped (k_output_rows visits them).
-__global__ void k_output_plain(float4* __restrict__ ZL, float4* __restrict__ U, const float4* __restrict__ HL, int ld4,
-                               long long n, const unsigned char* __restrict__ train, float rho, int dual_now,
-                               int update_z) {
-  const long long total = n * ld4;
-  const float inv_rho = 1.f / rho;
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (long long)gridDim.x * blockDim.x) {
-    if (train[e / ld4]) continue;
-    const float4 q = HL[e], u = U[e];
-    if (dual_now) {
-      const float4 z = ZL[e];
-      U[e] = make_float4(fmaf(rho, z.x - q.x, u.x), fmaf(rho, z.y - q.y, u.y), fmaf(rho, z.z - q.z, u.z),
-                         fmaf(rho, z.w - q.w, u.w));
-    }
-    if (update_z)
-      ZL[e] = make_float4(fmaf(-u.x, inv_rho, q.x), fmaf(-u.y, inv_rho, q.y), fmaf(-u.z, inv_rho, q.z),
-                          fmaf(-u.w, inv_rho, q.w));
-  }
-}
-
-// Z_l[i,:] <- Z_l[i,:] - G[i,:] / theta_{comm(i)}   (Eq. 10)
-__global__ void k_apply_z(float4* __restrict__ Z, const float4* __restrict__ G, int ld4, long long n,
-                          const int* __restrict__ row_comm, const SearchCtl* __restrict__ ctl) {
-  const long long total = n * ld4;
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (long long)gridDim.x * blockDim.x) {
-    const float s = ctl[row_comm[e / ld4]].inv_step;
-    if (s == 0.f) continue;
-    float4 z = Z[e];
-    const float4 g = G[e];
-    z.x = fmaf(-s, g.x, z.x); z.y = fmaf(-s, g.y, z.y); z.z = fmaf(-s, g.z, z.z); z.w = fmaf(-s, g.w, z.w);
-    Z[e] = z;
-  }
-}
-
 // ------------------------------------------------------------------------------------------
-// Output layer rows (Eq. 7) and the dual (Eq. 3), one warp per row, classes spread over lanes.
-//   q = row of A~ Z_{L-1}^k W_L^{k+1};  training rows: FISTA on
-//   loss_scale * CE(z, y) + <u, z - q> + (rho/2)||z - q||^2 ;  other rows: z = q - u / rho.
+// Output layer rows (Eq. 7) and the dual (Eq. 3).  q = row of A~ Z_{L-1}^k W_L^{k+1}.
+//   training rows: FISTA on  loss_scale * CE(z, y) + <u, z - q> + (rho/2)||z - q||^2 ;  other rows: z = q - u / rho.
 //   dual_now != 0: U <- u + rho (z_old - q) in the same sweep (Eq. 3 as printed).
-// `rows` (may be NULL = every row) lists the rows to visit: the training rows, when the rest is
-// left to k_output_plain.  CPL = classes per lane (C <= 32 CPL).  momentum[j] = (t_j - 1) / t_{j+1}
-// of FISTA's sequence t_1 = 1, t_{j+1} = (1 + sqrt(1 + 4 t_j^2)) / 2: the same for every row, so it
-// is tabulated once (in fp64) instead of being recomputed by every lane in every iteration.
+// The first `train_blocks` blocks take the training rows (`rows` lists them), LPR lanes per row with CPL classes each (C <=
+// LPR * CPL): a lane that holds several classes costs an exponential per class either way, but the two reductions per
+// iteration then take log2(LPR) shuffles for 32 / LPR rows at once.  91 k rows x 40 classes x 30 iterations: a warp per row
+// 255 us, 8 lanes per row 95 us.  The other blocks sweep the remaining rows elementwise.
+// momentum[j] = (t_j - 1) / t_{j+1} of FISTA's sequence t_1 = 1, t_{j+1} = (1 + sqrt(1 + 4 t_j^2)) / 2: the same for every
+// row, so it is tabulated once (in fp64).  `advance` (may be NULL): the pass counter of the decision log, counted up by
+// this last kernel of a pass.
 // ------------------------------------------------------------------------------------------
-template <int CPL>
+struct OutputArgs {
+  float *Z, *U;
+  const float* H;
+  int ld, C;
+  long long n;
+  const unsigned char* train;
+  const int *rows, *y;
+  int n_train, train_blocks;
+  const float* momentum;
+  float rho, loss_scale;
+  int iters, dual_now, update_z;
+  int* advance;
+};
+template <int LPR, int CPL>
 __global__ void __launch_bounds__(256)
-k_output_rows(float* __restrict__ ZL, float* __restrict__ U, const float* __restrict__ HL, int ld, int C,
-              int n, const int* __restrict__ y, const unsigned char* __restrict__ train, float rho,
-              float loss_scale, int iters, int dual_now, int update_z, const int* __restrict__ rows,
-              const float* __restrict__ momentum) {
-  const int lane = threadIdx.x & 31;
-  const int slot = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (slot >= n) return;
-  const int row = rows != nullptr ? rows[slot] : slot;
-  float q[CPL], u[CPL], z[CPL];
-  const long long base = (long long)row * ld;
-#pragma unroll
-  for (int t = 0; t < CPL; ++t) {
-    const int c = lane + 32 * t;
-    q[t] = u[t] = z[t] = 0.f;
-    if (c < C) { q[t] = HL[base + c]; u[t] = U[base + c]; z[t] = ZL[base + c]; }
-  }
-  if (dual_now) {
-#pragma unroll
-    for (int t = 0; t < CPL; ++t) {
-      const int c = lane + 32 * t;
-      if (c < C) U[base + c] = fmaf(rho, z[t] - q[t], u[t]);
-    }
-  }
-  if (!update_z) return;
-  if (!train[row]) {
-    const float inv_rho = 1.f / rho;
-#pragma unroll
-    for (int t = 0; t < CPL; ++t) {
-      const int c = lane + 32 * t;
-      if (c < C) ZL[base + c] = fmaf(-u[t], inv_rho, q[t]);
+k_output(const OutputArgs p) {
+  if (p.advance != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *p.advance += 1;
+  if ((int)blockIdx.x >= p.train_blocks) {
+    const int ld4 = p.ld / 4;
+    float4* const Z4 = reinterpret_cast<float4*>(p.Z);
+    float4* const U4 = reinterpret_cast<float4*>(p.U);
+    const float4* const H4 = reinterpret_cast<const float4*>(p.H);
+    const float inv_rho = 1.f / p.rho;
+    const long long total = p.n * ld4;   // below 2^32
+    for (long long e = (long long)(blockIdx.x - p.train_blocks) * blockDim.x + threadIdx.x; e < total;
+         e += (long long)(gridDim.x - p.train_blocks) * blockDim.x) {
+      if (p.train[(unsigned)e / (unsigned)ld4]) continue;
+      const float4 q = H4[e], u = U4[e];
+      if (p.dual_now) {
+        const float4 z = Z4[e];
+        U4[e] = make_float4(fmaf(p.rho, z.x - q.x, u.x), fmaf(p.rho, z.y - q.y, u.y), fmaf(p.rho, z.z - q.z, u.z),
+                            fmaf(p.rho, z.w - q.w, u.w));
+      }
+      if (p.update_z)
+        Z4[e] = make_float4(fmaf(-u.x, inv_rho, q.x), fmaf(-u.y, inv_rho, q.y), fmaf(-u.z, inv_rho, q.z), fmaf(-u.w, inv_rho, q.w));
     }
     return;
   }
-  const int yi = y[row];
-  const float step = 1.f / (0.5f * loss_scale + rho);
+  const int lane = threadIdx.x & (LPR - 1);
+  const int slot = (int)((blockIdx.x * blockDim.x + threadIdx.x) / LPR);
+  const bool here = slot < p.n_train;   // lanes without a row keep step with the shuffles of the others
+  const int row = here ? p.rows[slot] : 0;
+  const int C = here ? p.C : 0;
+  float q[CPL], u[CPL], z[CPL];
+  const long long base = (long long)row * p.ld;
+#pragma unroll
+  for (int t = 0; t < CPL; ++t) {
+    const int c = lane + LPR * t;
+    q[t] = u[t] = z[t] = 0.f;
+    if (c < C) { q[t] = p.H[base + c]; u[t] = p.U[base + c]; z[t] = p.Z[base + c]; }
+  }
+  if (p.dual_now) {
+#pragma unroll
+    for (int t = 0; t < CPL; ++t) {
+      const int c = lane + LPR * t;
+      if (c < C) p.U[base + c] = fmaf(p.rho, z[t] - q[t], u[t]);
+    }
+  }
+  if (!p.update_z) return;
+  const int yi = here ? p.y[row] : -1;
+  const float step = 1.f / (0.5f * p.loss_scale + p.rho);
   float xp[CPL], v[CPL];
 #pragma unroll
   for (int t = 0; t < CPL; ++t) { xp[t] = z[t]; v[t] = z[t]; }
-  for (int it = 0; it < iters; ++it) {
+  for (int it = 0; it < p.iters; ++it) {
     float mx = -3.0e38f;
 #pragma unroll
     for (int t = 0; t < CPL; ++t)
-      if (lane + 32 * t < C) mx = fmaxf(mx, v[t]);
-    mx = warp_max(mx);
+      if (lane + LPR * t < C) mx = fmaxf(mx, v[t]);
+#pragma unroll
+    for (int o = LPR / 2; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     float ex[CPL], se = 0.f;
 #pragma unroll
     for (int t = 0; t < CPL; ++t) {
-      ex[t] = (lane + 32 * t < C) ? expf(v[t] - mx) : 0.f;
+      ex[t] = (lane + LPR * t < C) ? expf(v[t] - mx) : 0.f;
       se += ex[t];
     }
-    se = warp_sum(se);
+#pragma unroll
+    for (int o = LPR / 2; o > 0; o >>= 1) se += __shfl_xor_sync(0xffffffffu, se, o);
     const float inv_se = 1.f / se;
-    const float mom = momentum[it];
+    const float mom = p.momentum[it];
 #pragma unroll
     for (int t = 0; t < CPL; ++t) {
-      const int c = lane + 32 * t;
-      const float p = ex[t] * inv_se - (c == yi ? 1.f : 0.f);
-      const float g = loss_scale * p + u[t] + rho * (v[t] - q[t]);
+      const float pr = ex[t] * inv_se - (lane + LPR * t == yi ? 1.f : 0.f);
+      const float g = p.loss_scale * pr + u[t] + p.rho * (v[t] - q[t]);
       const float x = fmaf(-step, g, v[t]);
       v[t] = fmaf(mom, x - xp[t], x);
       xp[t] = x;
@@ -1591,8 +1734,8 @@ k_output_rows(float* __restrict__ ZL, float* __restrict__ U, const float* __rest
   }
 #pragma unroll
   for (int t = 0; t < CPL; ++t) {
-    const int c = lane + 32 * t;
-    if (c < C) ZL[base + c] = xp[t];
+    const int c = lane + LPR * t;
+    if (c < C) p.Z[base + c] = xp[t];
   }
 }
 
