@@ -20,6 +20,7 @@
 #include "gemm_tc.cuh"
 #include "graph_index.hpp"
 #include "kernels.cuh"
+#include "memory.hpp"
 #include "shard_plan.hpp"
 
 using gcn_admm_host::GraphIndex;
@@ -41,6 +42,8 @@ constexpr long long kImageMinRows = 16384;   // row count from which the weight 
 constexpr int kZBlockRows = 32;      // rows per block of the hidden-layer gradient's closing sweep
 constexpr int kChunkGroups = 512;    // groups the sums of a scoring sweep's chunks are first added up in, when there are more chunks
 constexpr int kCandZ = 4;           // theta candidates scored per sweep (2..4; steady-state searches close at trial 0..2)
+constexpr size_t kDirectBytes = (size_t)256 << 10;   // matrices up to this size cross the bus inside the permuting kernel (one copy and its latency less)
+constexpr int kMaxCommNarrow = 384;            // communities whose sums k_score_z_out_part<16> holds in shared memory (96 KB)
 constexpr int kDefaultLongRow = 256;   // stored entries one warp walks before a row is cut into items
 
 thread_local std::string g_create_error;
@@ -182,9 +185,10 @@ struct gcn_admm {
   std::vector<int> C, ld;   // widths C_0..C_L and their padded leading dimensions
   int max_ld = 0;
   GraphIndex gi;
-  std::vector<void*> owned;  // every device allocation, for destroy
+  std::vector<gcn_admm_mem::Slab> slabs;   // device memory: one slab for everything, more only for workspaces that grow
+  gcn_admm_mem::Stage stage;               // page-locked staging of host buffers
 
-  int *d_row_ptr = nullptr, *d_col = nullptr, *d_row_comm = nullptr, *d_perm = nullptr;
+  int *d_row_ptr = nullptr, *d_col = nullptr, *d_row_comm = nullptr, *d_perm = nullptr, *d_inv = nullptr;
   int* d_y = nullptr;
   float* d_dinv = nullptr;
   unsigned short* d_col_comm = nullptr;   // community of every stored column
@@ -203,13 +207,14 @@ struct gcn_admm {
   float *B0 = nullptr, *B1 = nullptr, *B2 = nullptr;   // N x max_ld scratch
   float* grad = nullptr;     // max over l of C_{l-1} x ld_l
   float* grad_t = nullptr;   // its transpose, C_l x ld_{l-1} (K-major operand of the tensor-core product)
-  int* tc_error = nullptr;   // raised by a tensor-core product whose bounded wait ran out
+  int* tc_error = nullptr;   // &report->error: raised by a tensor-core product (1) or a search (2) whose bounded wait ran out
   uint8_t* b_image = nullptr;   // split weight operand in the staged layout (see gtc::k_split_b)
   size_t b_image_bytes = 0;
   float* part = nullptr;     // split partial sums of the transposed product
   size_t part_elems = 0;
   SearchCtl *ctl_w = nullptr, *ctl_z = nullptr;   // [L+1], [(L+1) * M]
-  double *sums_z = nullptr, *obj = nullptr;
+  double* sums_z = nullptr;
+  gk::Report* report = nullptr;             // objective sums and error flags
   double* red_part = nullptr;               // per-block partial sums awaiting their fixed-order reduction
   int4* d_zblocks = nullptr;                // row blocks of at most kZBlockRows rows, none crossing a community, and that community
   unsigned *ticket = nullptr, *comm_tickets = nullptr;   // counters of finished blocks (one launch; per community), zero between launches
@@ -217,7 +222,7 @@ struct gcn_admm {
   std::vector<float*> RN;                   // 2..L: derivative of phi_l at the new H_l, from the W_l update to that of Z_{l-1}
   int* d_comm_block_ptr = nullptr;          // [M+1] first row block of every community
   int n_zblocks = 0;
-  int *n_active = nullptr, *status = nullptr, *d_pass = nullptr;
+  int *n_active = nullptr, *status = nullptr, *d_pass = nullptr;   // status = &report->status
   // Z scoring: units in chunks of about equally many stored entries, dealt to the warps of the grid in a fixed order
   int* d_chunk_ptr = nullptr;
   int* d_row_order = nullptr;               // rows per community by falling length: the order of the kernels that put several rows in a warp
@@ -240,11 +245,51 @@ struct gcn_admm {
   gcn_admm_host::ShardPlan shard_plan;      // last plan asked for (host only)
   std::vector<int> shard_ranges;
 
+  // Device memory is asked for first and cut from one slab by commit(): tables to upload (staged in one stream of copies),
+  // then what starts at zero, then the rest.  The sources must live until commit() returns.
+  enum Start { kTable, kZero, kPlain };
+  struct Want {
+    void** slot;
+    size_t bytes;
+    const void* src;
+    Start start;
+  };
+  std::vector<Want> wants;
   template <typename T>
-  T* alloc(size_t count) {
-    T* p_ = dalloc<T>(count);
-    owned.push_back(p_);
-    return p_;
+  void want(T*& slot, size_t count, Start start = kPlain) {
+    wants.push_back(Want{reinterpret_cast<void**>(&slot), std::max<size_t>(count, 1) * sizeof(T), nullptr, start});
+  }
+  template <typename T, typename V>
+  void want_table(T*& slot, const V& v) {
+    static_assert(sizeof(T) == sizeof(typename V::value_type), "a table is uploaded as it is");
+    wants.push_back(Want{reinterpret_cast<void**>(&slot), std::max<size_t>(v.size(), 1) * sizeof(T), v.empty() ? nullptr : v.data(), kTable});
+  }
+  char* take_slab(size_t bytes) {
+    gcn_admm_mem::Slab slab;
+    const cudaError_t e = gcn_admm_mem::Pool::get().take(p.device, bytes, &slab);
+    if (e != cudaSuccess)
+      throw Fail{e == cudaErrorMemoryAllocation ? GCN_ADMM_ERR_ALLOC : GCN_ADMM_ERR_CUDA, std::string("cudaMalloc: ") + cudaGetErrorString(e)};
+    slabs.push_back(slab);
+    return slab.base;
+  }
+  void commit() {
+    std::stable_sort(wants.begin(), wants.end(), [](const Want& a, const Want& b) { return a.start < b.start; });
+    size_t total = 0, zero_begin = 0, zero_end = 0;
+    std::vector<size_t> at;
+    for (const Want& w : wants) {
+      if (w.start == kZero && zero_end == 0) zero_begin = total;
+      at.push_back(total);
+      total += (w.bytes + 255) / 256 * 256;
+      if (w.start == kZero) zero_end = total;
+    }
+    char* const base = take_slab(total);
+    for (size_t k = 0; k < wants.size(); ++k) {
+      *wants[k].slot = base + at[k];
+      if (wants[k].start == kTable && wants[k].src) CU(stage.put(base + at[k], wants[k].src, wants[k].bytes, stream));
+    }
+    CU(stage.flush(stream));
+    if (zero_end > zero_begin) CU(cudaMemsetAsync(base + zero_begin, 0, zero_end - zero_begin, stream));
+    wants.clear();
   }
   int grid_for(long long work_items, int per_block = 256) const {
     return (int)std::max<long long>(1, std::min<long long>(cdiv(work_items, per_block), (long long)kSmCount * 8));
@@ -291,8 +336,7 @@ struct gcn_admm {
   void grow_item_sums(int ldw) {
     const size_t need = (size_t)n_items * ldw;
     if (need <= item_sums_elems) return;
-    float* bigger = alloc<float>(need);   // the old one stays in `owned` until destroy: kernels in flight may hold it
-    item_sums = bigger;
+    item_sums = reinterpret_cast<float*>(take_slab(need * sizeof(float)));   // the old one stays until destroy: kernels in flight may hold it
     item_sums_elems = need;
   }
 
@@ -773,51 +817,100 @@ struct gcn_admm {
     }
   }
 
-  void check_status() {
-    int s = 0, t = 0;
-    CU(cudaMemcpyAsync(&s, status, sizeof(int), cudaMemcpyDeviceToHost, stream));
-    CU(cudaMemcpyAsync(&t, tc_error, sizeof(int), cudaMemcpyDeviceToHost, stream));
-    CU(cudaStreamSynchronize(stream));
-    if (t != 0) {
-      CU(cudaMemsetAsync(tc_error, 0, sizeof(int), stream));
+  // Reported numbers and error flags, read back together.
+  gk::Report read_report() {
+    gk::Report r;
+    CU(stage.get(&r, report, sizeof r, sizeof r, 1, stream));
+    return r;
+  }
+  void check(const gk::Report& r) {
+    if (r.error != 0) {
+      CU(cudaMemsetAsync(&report->error, 0, sizeof(int), stream));
       CU(cudaMemsetAsync(grid_bar, 0, sizeof(gk::GridBar), stream));
-      throw Fail{GCN_ADMM_ERR_CUDA, t & gk::kErrGridBarrier ? "a step-size search gave up waiting for the rest of its grid"
-                                                            : "a tensor-core product gave up waiting on its pipeline"};
+      throw Fail{GCN_ADMM_ERR_CUDA, r.error & gk::kErrGridBarrier ? "a step-size search gave up waiting for the rest of its grid"
+                                                                  : "a tensor-core product gave up waiting on its pipeline"};
     }
-    if (s & 1) {
-      CU(cudaMemsetAsync(status, 0, sizeof(int), stream));
+    if (r.status & 1) {
+      CU(cudaMemsetAsync(&report->status, 0, sizeof(int), stream));
       throw Fail{GCN_ADMM_ERR_NONFINITE, "a non-finite value reached a step-size decision"};
     }
   }
+  void check_status() { check(read_report()); }
 
-  // rows in the caller's order (dense, width c) <-> internal (community order, padded)
+  // rows in the caller's order (dense, width c) <-> internal (community order, padded).  Small matrices are written to and
+  // read from the staging buffer by the permuting kernel itself.
   void rows_to_host(const float* dev, int c, float* host_out) {
-    float* dense = B2;
-    Scope sc(this, "permute_rows", 1, 8.0 * (double)n * c, 0.0);
-    gk::k_permute_rows<<<grid_for(n * ldpad(c)), 256, 0, stream>>>(dev, dense, d_perm, n, c, ldpad(c), 0);
-    CU(cudaGetLastError());
-    CU(cudaMemcpyAsync(host_out, dense, sizeof(float) * n * c, cudaMemcpyDeviceToHost, stream));
-    CU(cudaStreamSynchronize(stream));
+    const size_t bytes = sizeof(float) * (size_t)n * c;
+    const bool small = bytes <= kDirectBytes;
+    char* near_host = nullptr;
+    if (small) CU(stage.enter(stream, &near_host));
+    float* dense = small ? reinterpret_cast<float*>(near_host) : B2;
+    {
+      Scope sc(this, "permute_rows", 1, 8.0 * (double)n * c, 0.0);
+      gk::k_permute_rows<<<grid_for(n * ldpad(c)), 256, 0, stream>>>(dev, dense, d_inv, n, c, ldpad(c), 0);
+      CU(cudaGetLastError());
+    }
+    if (small) {
+      CU(stage.leave(stream));
+      CU(cudaStreamSynchronize(stream));
+      std::memcpy(host_out, near_host, bytes);
+    } else {
+      CU(stage.get(host_out, dense, bytes, bytes, 1, stream));
+    }
   }
   void rows_from_host(const float* host_in, int c, float* dev) {
-    float* dense = B2;
-    CU(cudaMemcpyAsync(dense, host_in, sizeof(float) * n * c, cudaMemcpyHostToDevice, stream));
-    Scope sc(this, "permute_rows", 1, 8.0 * (double)n * c, 0.0);
-    gk::k_permute_rows<<<grid_for(n * ldpad(c)), 256, 0, stream>>>(dense, dev, d_perm, n, c, ldpad(c), 1);
-    CU(cudaGetLastError());
-    CU(cudaStreamSynchronize(stream));
+    const size_t bytes = sizeof(float) * (size_t)n * c;
+    const bool small = bytes <= kDirectBytes;
+    char* near_host = nullptr;
+    const float* dense = B2;
+    if (small) {
+      CU(stage.enter(stream, &near_host));
+      std::memcpy(near_host, host_in, bytes);
+      dense = reinterpret_cast<const float*>(near_host);
+    } else {
+      CU(stage.put(B2, host_in, bytes, stream));
+      CU(stage.flush(stream));
+    }
+    {
+      Scope sc(this, "permute_rows", 1, 8.0 * (double)n * c, 0.0);
+      gk::k_permute_rows<<<grid_for(n * ldpad(c)), 256, 0, stream>>>(dense, dev, d_inv, n, c, ldpad(c), 1);
+      CU(cudaGetLastError());
+    }
+    if (small) CU(stage.leave(stream));
+    else CU(stage.finish(stream));
   }
+  // W_l and its transpose from a dense host matrix, through the gradient's buffer.
   void upload_weight(int l, const float* host_w) {
     const int r = C[l - 1], c = C[l];
-    std::vector<float> w((size_t)r * ld[l], 0.f), wt((size_t)c * ld[l - 1], 0.f);
-    for (int i = 0; i < r; ++i)
-      for (int j = 0; j < c; ++j) {
-        w[(size_t)i * ld[l] + j] = host_w[(size_t)i * c + j];
-        wt[(size_t)j * ld[l - 1] + i] = host_w[(size_t)i * c + j];
-      }
-    CU(cudaMemcpyAsync(W[l], w.data(), w.size() * sizeof(float), cudaMemcpyHostToDevice, stream));
-    CU(cudaMemcpyAsync(Wt[l], wt.data(), wt.size() * sizeof(float), cudaMemcpyHostToDevice, stream));
-    CU(cudaStreamSynchronize(stream));
+    CU(stage.put(grad, host_w, sizeof(float) * (size_t)r * c, stream));
+    CU(stage.finish(stream));
+    const long long cells = std::max((long long)r * ld[l], (long long)c * ld[l - 1]);
+    gk::k_load_weight<<<grid_for(cells), 256, 0, stream>>>(grad, r, c, W[l], ld[l], Wt[l], ld[l - 1]);
+    CU(cudaGetLastError());
+  }
+  // Step parameters (t_prev) of `count` searches in a row, to and from the host.
+  void take_steps(const SearchCtl* ctl, double* values, int count) {
+    for (int k = 0; k < count; k += (int)(gcn_admm_mem::kSlot / sizeof(double))) {
+      const int now = std::min(count - k, (int)(gcn_admm_mem::kSlot / sizeof(double)));
+      char* near_host = nullptr;
+      CU(stage.enter(stream, &near_host));
+      gk::k_take_steps<<<(unsigned)cdiv(now, 256), 256, 0, stream>>>(ctl + k, reinterpret_cast<double*>(near_host), now);
+      CU(cudaGetLastError());
+      CU(stage.leave(stream));
+      CU(cudaStreamSynchronize(stream));
+      std::memcpy(values + k, near_host, sizeof(double) * now);
+    }
+  }
+  void put_steps(SearchCtl* ctl, const double* values, int count) {
+    for (int k = 0; k < count; k += (int)(gcn_admm_mem::kSlot / sizeof(double))) {
+      const int now = std::min(count - k, (int)(gcn_admm_mem::kSlot / sizeof(double)));
+      char* near_host = nullptr;
+      CU(stage.enter(stream, &near_host));
+      std::memcpy(near_host, values + k, sizeof(double) * now);
+      gk::k_put_steps<<<(unsigned)cdiv(now, 256), 256, 0, stream>>>(ctl + k, reinterpret_cast<const double*>(near_host), now);
+      CU(cudaGetLastError());
+      CU(stage.leave(stream));
+    }
   }
 };
 
@@ -847,12 +940,15 @@ int guarded(gcn_admm* h, F&& body) {
 // it lives on the device.
 template <typename T>
 struct HostView {
-  std::vector<T> copy;
+  gcn_admm_host::Table<T> copy;
   const T* ptr = nullptr;
-  HostView(const T* p, size_t count) {
+  HostView(gcn_admm* h, const T* p, size_t count) {
     if (count > 0 && is_device_pointer(p)) {
       copy.resize(count);
-      CU(cudaMemcpy(copy.data(), p, count * sizeof(T), cudaMemcpyDeviceToHost));
+      CU(cudaSetDevice(h->p.device));
+      CU(cudaDeviceSynchronize());   // whatever fills the buffer, on whichever stream
+      CU(h->stage.open());
+      CU(h->stage.get(copy.data(), p, count * sizeof(T), count * sizeof(T), 1, h->stream));
       ptr = copy.data();
     } else {
       ptr = p;
@@ -861,13 +957,6 @@ struct HostView {
   const T* data() const { return ptr; }
   const T& operator[](size_t i) const { return ptr[i]; }
 };
-
-template <typename T, typename A>
-T* upload(gcn_admm* h, const std::vector<T, A>& v) {
-  T* d = h->alloc<T>(v.size());
-  if (!v.empty()) CU(cudaMemcpy(d, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice));
-  return d;
-}
 
 void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* col_idx, const float* X, const int* y,
                  const unsigned char* train_mask, int n_layers, const int* widths, int n_comm, const int* community) {
@@ -891,141 +980,140 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
       throw Fail{GCN_ADMM_ERR_WIDTHS, "n x layer width exceeds 2^34 elements"};
 
   // host copies of the graph-side inputs, then the index tables
-  HostView<long long> rp(row_ptr, (size_t)n + 1);
+  h->stream = static_cast<cudaStream_t>(p.stream);
+  HostView<long long> rp(h, row_ptr, (size_t)n + 1);
   if (rp[n] < 0 || rp[0] != 0) throw Fail{GCN_ADMM_ERR_GRAPH, "row_ptr must start at 0 and be ascending"};
-  HostView<int> ci(col_idx, (size_t)rp[n]);
-  HostView<int> comm(community, (size_t)n);
-  HostView<int> yy(y, (size_t)n);
-  HostView<unsigned char> tm(train_mask, (size_t)n);
+  HostView<int> ci(h, col_idx, (size_t)rp[n]);
+  HostView<int> comm(h, community, (size_t)n);
+  HostView<int> yy(h, y, (size_t)n);
+  HostView<unsigned char> tm(h, train_mask, (size_t)n);
   std::string msg;
   const int rc = gcn_admm_host::build_graph_index(n, rp.data(), ci.data(), n_comm, comm.data(), h->gi, msg);
   if (rc == gcn_admm_host::IDX_BAD_GRAPH) throw Fail{GCN_ADMM_ERR_GRAPH, msg};
   if (rc == gcn_admm_host::IDX_BAD_COMMUNITY) throw Fail{GCN_ADMM_ERR_COMMUNITY, msg};
-  { std::vector<long long>().swap(rp.copy); std::vector<int>().swap(ci.copy); }
+  { gcn_admm_host::Table<long long>().swap(rp.copy); gcn_admm_host::Table<int>().swap(ci.copy); }
   const GraphIndex& g = h->gi;
-  std::vector<int> y_new(n);
-  std::vector<unsigned char> t_new(n);
-  h->n_train = 0;
+  gcn_admm_host::Table<int> y_new;
+  gcn_admm_host::Table<unsigned char> t_new;
+  y_new.resize((size_t)n);
+  t_new.resize((size_t)n);
+  int bad_label = 0, n_train = 0;
+#pragma omp parallel for schedule(static) reduction(| : bad_label) reduction(+ : n_train) if (n > 20000)
   for (long long i = 0; i < n; ++i) {
-    y_new[i] = yy[g.perm[i]];
-    t_new[i] = tm[g.perm[i]] ? 1 : 0;
-    h->n_train += t_new[i];
-    if (t_new[i] && (y_new[i] < 0 || y_new[i] >= h->C[n_layers]))
-      throw Fail{GCN_ADMM_ERR_WIDTHS, "a training label lies outside 0..C_L-1"};
-    if (y_new[i] < 0 || y_new[i] >= h->C[n_layers]) y_new[i] = 0;
+    const bool in = yy[g.perm[i]] >= 0 && yy[g.perm[i]] < h->C[n_layers];
+    t_new[(size_t)i] = tm[g.perm[i]] ? 1 : 0;
+    n_train += t_new[(size_t)i];
+    bad_label |= t_new[(size_t)i] && !in;
+    y_new[(size_t)i] = in ? yy[g.perm[i]] : 0;
   }
+  h->n_train = n_train;
+  if (bad_label) throw Fail{GCN_ADMM_ERR_WIDTHS, "a training label lies outside 0..C_L-1"};
   // all host-side validation is done; from here on a CUDA device is required
   int dev_count = 0;
   CU(cudaGetDeviceCount(&dev_count));
   if (p.device < 0 || p.device >= dev_count) throw Fail{GCN_ADMM_ERR_CUDA, "no such CUDA device"};
   CU(cudaSetDevice(p.device));
-  h->stream = static_cast<cudaStream_t>(p.stream);
-  h->d_row_ptr = upload(h, g.row_ptr);
-  h->d_col = upload(h, g.col);
-  h->d_row_comm = upload(h, g.row_comm);
-  h->d_perm = upload(h, g.perm);
-  h->d_dinv = upload(h, g.dinv);
-  h->d_col_comm = upload(h, g.col_comm);
-  { gcn_admm_host::Table<unsigned short>().swap(h->gi.col_comm); }   // needed on the device only
-  h->d_y = upload(h, y_new);
-  h->d_train = upload(h, t_new);
+  CU(h->stage.open());
+  h->want_table(h->d_row_ptr, g.row_ptr);
+  h->want_table(h->d_col, g.col);
+  h->want_table(h->d_row_comm, g.row_comm);
+  h->want_table(h->d_perm, g.perm);
+  h->want_table(h->d_inv, g.inv);
+  h->want_table(h->d_dinv, g.dinv);
+  h->want_table(h->d_col_comm, g.col_comm);
+  h->want_table(h->d_y, y_new);
+  h->want_table(h->d_train, t_new);
+  std::vector<int> tr;
+  tr.reserve((size_t)h->n_train);
+  for (long long i = 0; i < n; ++i)
+    if (t_new[(size_t)i]) tr.push_back((int)i);
+  h->want_table(h->d_train_rows, tr);
+  std::vector<float> mom((size_t)std::max(p.fista_iters, 1), 0.f);
   {
-    std::vector<int> tr;
-    tr.reserve((size_t)h->n_train);
-    for (long long i = 0; i < n; ++i)
-      if (t_new[i]) tr.push_back((int)i);
-    h->d_train_rows = upload(h, tr);
-  }
-  {
-    std::vector<float> mom((size_t)std::max(p.fista_iters, 1), 0.f);
     double t = 1.0;
     for (int j = 0; j < p.fista_iters; ++j) {
       const double tn = 0.5 * (1.0 + std::sqrt(1.0 + 4.0 * t * t));
       mom[(size_t)j] = (float)((t - 1.0) / tn);
       t = tn;
     }
-    h->d_fista_momentum = upload(h, mom);
   }
+  h->want_table(h->d_fista_momentum, mom);
+  h->long_len = p.long_row > 0 ? p.long_row : kDefaultLongRow;
+  gcn_admm_host::LongRowTables lt;
+  gcn_admm_host::build_long_row_tables(g, h->long_len, lt);
+  h->n_items = (int)lt.items.size();
+  h->n_split = (int)lt.split.size();
+  h->n_long = (int)lt.rows.size();
+  h->want_table(h->d_items, lt.items);
+  h->want_table(h->d_split, lt.split);
+  h->want_table(h->d_long_rows, lt.rows);
+  std::vector<int> item_row(lt.items.size());
+  for (size_t r = 0; r < lt.rows.size(); ++r)
+    for (int k = 0; k < lt.rows[r].z; ++k) item_row[(size_t)(lt.rows[r].y + k)] = (int)r;
+  h->want_table(h->d_item_row, item_row);
+  h->want(h->d_row_done, lt.rows.size(), gcn_admm::kZero);
+  // split entries grouped by community (stable), for the ordered sums of the Z search
+  std::vector<int> split_ptr((size_t)n_comm + 1, 0), split_order(lt.split.size());
+  for (const auto& q : lt.split) ++split_ptr[(size_t)q.y + 1];
+  for (int m = 0; m < n_comm; ++m) split_ptr[m + 1] += split_ptr[m];
   {
-    h->long_len = p.long_row > 0 ? p.long_row : kDefaultLongRow;
-    gcn_admm_host::LongRowTables lt;
-    gcn_admm_host::build_long_row_tables(g, h->long_len, lt);
-    static_assert(sizeof(gcn_admm_host::Quad) == sizeof(int4), "tables are uploaded as int4");
-    h->n_items = (int)lt.items.size();
-    h->n_split = (int)lt.split.size();
-    h->n_long = (int)lt.rows.size();
-    h->d_items = reinterpret_cast<int4*>(upload(h, lt.items));
-    h->d_split = reinterpret_cast<int4*>(upload(h, lt.split));
-    {   // split entries grouped by community (stable), for the ordered sums of k_search_decide_z
-      std::vector<int> sptr((size_t)n_comm + 1, 0), order(lt.split.size());
-      for (const auto& q : lt.split) ++sptr[(size_t)q.y + 1];
-      for (int m = 0; m < n_comm; ++m) sptr[m + 1] += sptr[m];
-      std::vector<int> at(sptr.begin(), sptr.end() - 1);
-      for (size_t k = 0; k < lt.split.size(); ++k) order[(size_t)at[lt.split[k].y]++] = (int)k;
-      h->d_split_order = upload(h, order);
-      h->d_split_ptr = upload(h, sptr);
-      h->split_scores = h->alloc<double>(std::max<size_t>(1, lt.split.size() * gk::kCand));
-    }
-    std::vector<int> row_order((size_t)n);
-    for (long long i = 0; i < n; ++i) row_order[(size_t)i] = (int)i;
-#pragma omp parallel for schedule(dynamic, 1)
-    for (int m = 0; m < n_comm; ++m)   // inside a community: longest rows first, ties by row id
-      std::stable_sort(row_order.begin() + g.comm_ptr[m], row_order.begin() + g.comm_ptr[m + 1], [&](int a, int b) {
-        return g.row_ptr[a + 1] - g.row_ptr[a] > g.row_ptr[b + 1] - g.row_ptr[b];
-      });
-    h->d_row_order = upload(h, row_order);
-    {   // chunks of units (items first, then rows) holding about the same number of stored entries each,
-        // once for rows in storage order and once for rows in the sorted order
-      const long long n_units = (long long)lt.items.size() + n;
-      const long long warps_guess = (long long)kSmCount * 3 * 8;
-      // few enough chunks that their sums (M x candidates doubles each) stay small next to the entries they cover
-      const long long target = std::max<long long>({64, std::min<long long>(1024, (long long)g.nnz / (warps_guess * 4)), 2LL * n_comm});
-      auto build_chunks = [&](const int* order) {
-        std::vector<int> cp;
-        cp.push_back(0);
-        long long in_chunk = 0;
-        for (long long u = 0; u < n_units; ++u) {
-          long long len;
-          if (u < (long long)lt.items.size()) len = lt.items[(size_t)u].z - lt.items[(size_t)u].y;
-          else {
-            const long long k = u - (long long)lt.items.size();
-            const long long r = order ? order[k] : k;
-            len = g.row_ptr[r + 1] - g.row_ptr[r];
-            if (len > h->long_len) len = 0;                 // walked as items
-          }
-          in_chunk += len + 2;                              // a unit costs a little even when it is short
-          if (in_chunk >= target) { cp.push_back((int)(u + 1)); in_chunk = 0; }
-        }
-        if (cp.back() != (int)n_units) cp.push_back((int)n_units);
-        return cp;
-      };
-      const std::vector<int> plain = build_chunks(nullptr), sorted = build_chunks(row_order.data());
-      h->n_chunks = (int)plain.size() - 1;
-      h->d_chunk_ptr = upload(h, plain);
-      h->n_chunks_sorted = (int)sorted.size() - 1;
-      h->d_chunk_ptr_sorted = upload(h, sorted);
-    }
-    h->d_long_rows = reinterpret_cast<int4*>(upload(h, lt.rows));
-    std::vector<int> item_row(lt.items.size());
-    for (size_t r = 0; r < lt.rows.size(); ++r)
-      for (int k = 0; k < lt.rows[r].z; ++k) item_row[(size_t)(lt.rows[r].y + k)] = (int)r;
-    h->d_item_row = upload(h, item_row);
-    h->d_row_done = h->alloc<int>(lt.rows.size());
-    CU(cudaMemset(h->d_row_done, 0, std::max<size_t>(1, lt.rows.size()) * sizeof(int)));
+    std::vector<int> at(split_ptr.begin(), split_ptr.end() - 1);
+    for (size_t k = 0; k < lt.split.size(); ++k) split_order[(size_t)at[lt.split[k].y]++] = (int)k;
   }
+  h->want_table(h->d_split_order, split_order);
+  h->want_table(h->d_split_ptr, split_ptr);
+  h->want(h->split_scores, lt.split.size() * gk::kCand);
+  gcn_admm_host::Table<int> row_order;
+  gcn_admm_host::order_rows_by_length(g, row_order);
+  h->want_table(h->d_row_order, row_order);
+  // chunks of units (items first, then rows) holding about the same number of stored entries each: for rows in storage
+  // order (whole-warp scoring) and for rows by falling length (several rows per warp: output layers of at most 64 classes)
+  std::vector<int> chunks_plain, chunks_sorted;
+  {
+    const long long n_units = (long long)lt.items.size() + n;
+    const long long warps_guess = (long long)kSmCount * 3 * 8;
+    // few enough chunks that their sums (M x candidates doubles each) stay small next to the entries they cover
+    const long long target = std::max<long long>({64, std::min<long long>(1024, (long long)g.nnz / (warps_guess * 4)), 2LL * n_comm});
+    auto build_chunks = [&](const int* order) {
+      std::vector<int> cp;
+      cp.push_back(0);
+      long long in_chunk = 0;
+      for (long long u = 0; u < n_units; ++u) {
+        long long len;
+        if (u < (long long)lt.items.size()) len = lt.items[(size_t)u].z - lt.items[(size_t)u].y;
+        else {
+          const long long k = u - (long long)lt.items.size();
+          const long long r = order ? order[k] : k;
+          len = g.row_ptr[r + 1] - g.row_ptr[r];
+          if (len > h->long_len) len = 0;                 // walked as items
+        }
+        in_chunk += len + 2;                              // a unit costs a little even when it is short
+        if (in_chunk >= target) { cp.push_back((int)(u + 1)); in_chunk = 0; }
+      }
+      if (cp.back() != (int)n_units) cp.push_back((int)n_units);
+      return cp;
+    };
+    const bool narrow_out = n_layers >= 2 && h->ld[n_layers] <= 64;
+    if (n_layers >= 3 || !narrow_out || n_comm > kMaxCommNarrow) chunks_plain = build_chunks(nullptr);
+    if (narrow_out) chunks_sorted = build_chunks(row_order.data());
+    h->n_chunks = std::max(0, (int)chunks_plain.size() - 1);
+    h->n_chunks_sorted = std::max(0, (int)chunks_sorted.size() - 1);
+  }
+  h->want_table(h->d_chunk_ptr, chunks_plain);
+  h->want_table(h->d_chunk_ptr_sorted, chunks_sorted);
 
   const int L = n_layers;
   const size_t rows = (size_t)n;
   h->W.assign(L + 1, nullptr); h->Wt.assign(L + 1, nullptr); h->Z.assign(L + 1, nullptr);
-  h->P.assign(L + 1, nullptr); h->H.assign(L + 1, nullptr);
+  h->P.assign(L + 1, nullptr); h->H.assign(L + 1, nullptr); h->RN.assign(L + 1, nullptr);
   size_t grad_elems = 1, grad_t_elems = 1, grad_blocks = 1;   // grad_blocks: most blocks of a finish_grad launch
   h->part_elems = 1;
   for (int l = 1; l <= L; ++l) {
-    h->W[l] = h->alloc<float>((size_t)h->C[l - 1] * h->ld[l]);
-    h->Wt[l] = h->alloc<float>((size_t)h->C[l] * h->ld[l - 1]);
-    h->Z[l] = h->alloc<float>(rows * h->ld[l]);
-    h->P[l] = h->alloc<float>(rows * h->ld[l - 1]);
-    h->H[l] = h->alloc<float>(rows * h->ld[l]);
+    h->want(h->W[l], (size_t)h->C[l - 1] * h->ld[l]);
+    h->want(h->Wt[l], (size_t)h->C[l] * h->ld[l - 1]);
+    h->want(h->Z[l], rows * h->ld[l]);
+    h->want(h->P[l], rows * h->ld[l - 1]);
+    h->want(h->H[l], rows * h->ld[l]);
     const size_t ge = (size_t)h->C[l - 1] * h->ld[l];
     grad_elems = std::max(grad_elems, ge);
     grad_blocks = std::max(grad_blocks, (size_t)h->C[l - 1] * (size_t)cdiv(h->ld[l], 32));
@@ -1036,99 +1124,71 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
     h->part_elems = std::max(h->part_elems, (size_t)h->C[l - 1] * h->ld[l] * (size_t)(cdiv(n, 2048) + kSmCount));
   h->part_elems = std::min<size_t>(h->part_elems, (size_t)256 << 20);   // at most 1 GB of partial sums
   h->part_elems = std::max(h->part_elems, grad_elems);
-  h->U = h->alloc<float>(rows * h->ld[L]);
-  h->B0 = h->alloc<float>(rows * h->max_ld);
-  h->B1 = h->alloc<float>(rows * h->max_ld);
-  h->B2 = h->alloc<float>(rows * h->max_ld);
-  h->RN.assign(L + 1, nullptr);
-  for (int l = 2; l <= L; ++l) h->RN[l] = l == L ? h->B0 : h->alloc<float>(rows * h->ld[l]);   // R_L is turned into its new value in place
+  h->want(h->U, rows * h->ld[L], gcn_admm::kZero);
+  h->want(h->B0, rows * h->max_ld);
+  h->want(h->B1, rows * h->max_ld);
+  h->want(h->B2, rows * h->max_ld);
+  for (int l = 2; l < L; ++l) h->want(h->RN[l], rows * h->ld[l]);
   h->item_sums_elems = std::max<size_t>(1, (size_t)h->n_items * h->max_ld);
-  h->item_sums = h->alloc<float>(h->item_sums_elems);
-  h->grad = h->alloc<float>(grad_elems);
-  h->grad_t = h->alloc<float>(grad_t_elems);
-  h->tc_error = h->alloc<int>(1);
+  h->want(h->item_sums, h->item_sums_elems);
+  h->want(h->grad, grad_elems);
+  h->want(h->grad_t, grad_t_elems, gcn_admm::kZero);
   h->b_image_bytes = (size_t)16 << 20;   // e.g. 1024 columns x 2048 K
-  h->b_image = h->alloc<uint8_t>(h->b_image_bytes);
-  CU(cudaMemset(h->tc_error, 0, sizeof(int)));
-  CU(cudaMemset(h->grad_t, 0, grad_t_elems * sizeof(float)));
-  h->part = h->alloc<float>(h->part_elems);
-  h->ctl_w = h->alloc<SearchCtl>(L + 1);
-  h->ctl_z = h->alloc<SearchCtl>((size_t)(L + 1) * n_comm);
-  h->sums_z = h->alloc<double>((size_t)3 * n_comm);
-  h->obj = h->alloc<double>(8);
-  {   // row blocks of the hidden-layer gradient's closing sweep, cut at community boundaries
-    std::vector<int4> zb;
-    std::vector<int> cbp((size_t)n_comm + 1, 0);
-    for (int m = 0; m < n_comm; ++m) {
-      cbp[m] = (int)zb.size();
-      for (int r = g.comm_ptr[m]; r < g.comm_ptr[m + 1]; r += kZBlockRows)
-        zb.push_back(make_int4(r, std::min(r + kZBlockRows, g.comm_ptr[m + 1]), m, 0));
-    }
-    cbp[n_comm] = (int)zb.size();
-    h->n_zblocks = (int)zb.size();
-    h->d_zblocks = upload(h, zb);
-    h->d_comm_block_ptr = upload(h, cbp);
+  h->want(h->b_image, h->b_image_bytes);
+  h->want(h->part, h->part_elems);
+  std::vector<SearchCtl> cw(L + 1), cz((size_t)(L + 1) * n_comm);
+  std::memset(cw.data(), 0, cw.size() * sizeof(SearchCtl));
+  std::memset(cz.data(), 0, cz.size() * sizeof(SearchCtl));
+  for (auto& c : cw) { c.t_prev = p.tau0; c.done = 1; c.trial = -3; }
+  for (auto& c : cz) { c.t_prev = p.theta0; c.done = 1; c.trial = -3; }
+  h->want_table(h->ctl_w, cw);
+  h->want_table(h->ctl_z, cz);
+  h->want(h->sums_z, (size_t)3 * n_comm);
+  h->want(h->report, 1, gcn_admm::kZero);
+  // row blocks of the hidden-layer gradient's closing sweep, cut at community boundaries
+  std::vector<int4> zb;
+  std::vector<int> cbp((size_t)n_comm + 1, 0);
+  for (int m = 0; m < n_comm; ++m) {
+    cbp[m] = (int)zb.size();
+    for (int r = g.comm_ptr[m]; r < g.comm_ptr[m + 1]; r += kZBlockRows)
+      zb.push_back(make_int4(r, std::min(r + kZBlockRows, g.comm_ptr[m + 1]), m, 0));
   }
-  const int max_chunks = std::max(h->n_chunks, h->n_chunks_sorted);
-  h->z_chunk_part = h->alloc<double>((size_t)max_chunks * n_comm * gk::kCand);
-  h->z_group_part = h->alloc<double>((size_t)kChunkGroups * n_comm * gk::kCand);
-  h->chunk_counter = h->alloc<int>(1);
-  CU(cudaMemset(h->chunk_counter, 0, sizeof(int)));
-  h->ticket = h->alloc<unsigned>(1);
-  CU(cudaMemset(h->ticket, 0, sizeof(unsigned)));
-  h->comm_tickets = h->alloc<unsigned>(n_comm);
-  CU(cudaMemset(h->comm_tickets, 0, n_comm * sizeof(unsigned)));
-  h->grid_bar = h->alloc<gk::GridBar>(1);
-  CU(cudaMemset(h->grid_bar, 0, sizeof(gk::GridBar)));
-  h->red_part = h->alloc<double>(std::max<size_t>({(size_t)kSmCount * 8 * gk::kCand, (size_t)h->n_zblocks * 3,
-                                                   (size_t)cdiv(n, 8) * 2, grad_blocks * 2}));
-  h->n_active = h->alloc<int>(1);
-  h->status = h->alloc<int>(1);
-  h->d_pass = h->alloc<int>(1);
-  CU(cudaMemset(h->d_pass, 0, sizeof(int)));
-  h->log_trial_w = h->alloc<int>((size_t)kLogPasses * L);
-  h->log_q_w = h->alloc<double>((size_t)kLogPasses * L);
-  h->log_trial_z = h->alloc<int>((size_t)kLogPasses * std::max(L - 1, 0) * n_comm);
-  h->log_q_z = h->alloc<double>((size_t)kLogPasses * std::max(L - 1, 0) * n_comm);
-  CU(cudaMemset(h->status, 0, sizeof(int)));
-  CU(cudaMemset(h->n_active, 0, sizeof(int)));
-  CU(cudaMemset(h->U, 0, rows * h->ld[L] * sizeof(float)));
-
-  {
-    std::vector<SearchCtl> cw(L + 1), cz((size_t)(L + 1) * n_comm);
-    std::memset(cw.data(), 0, cw.size() * sizeof(SearchCtl));
-    std::memset(cz.data(), 0, cz.size() * sizeof(SearchCtl));
-    for (auto& c : cw) { c.t_prev = p.tau0; c.done = 1; c.trial = -3; }
-    for (auto& c : cz) { c.t_prev = p.theta0; c.done = 1; c.trial = -3; }
-    CU(cudaMemcpy(h->ctl_w, cw.data(), cw.size() * sizeof(SearchCtl), cudaMemcpyHostToDevice));
-    CU(cudaMemcpy(h->ctl_z, cz.data(), cz.size() * sizeof(SearchCtl), cudaMemcpyHostToDevice));
-  }
+  cbp[n_comm] = (int)zb.size();
+  h->n_zblocks = (int)zb.size();
+  h->want_table(h->d_zblocks, zb);
+  h->want_table(h->d_comm_block_ptr, cbp);
+  h->want(h->z_chunk_part, (size_t)std::max(h->n_chunks, h->n_chunks_sorted) * n_comm * gk::kCand);
+  h->want(h->z_group_part, (size_t)kChunkGroups * n_comm * gk::kCand);
+  h->want(h->chunk_counter, 1, gcn_admm::kZero);
+  h->want(h->ticket, 1, gcn_admm::kZero);
+  h->want(h->comm_tickets, n_comm, gcn_admm::kZero);
+  h->want(h->grid_bar, 1, gcn_admm::kZero);
+  h->want(h->red_part, std::max<size_t>({(size_t)kSmCount * 8 * gk::kCand, (size_t)h->n_zblocks * 3,
+                                         (size_t)cdiv(n, 8) * 2, grad_blocks * 2}));
+  h->want(h->n_active, 1, gcn_admm::kZero);
+  h->want(h->d_pass, 1, gcn_admm::kZero);
+  h->want(h->log_trial_w, (size_t)kLogPasses * L);
+  h->want(h->log_q_w, (size_t)kLogPasses * L);
+  h->want(h->log_trial_z, (size_t)kLogPasses * std::max(L - 1, 0) * n_comm);
+  h->want(h->log_q_z, (size_t)kLogPasses * std::max(L - 1, 0) * n_comm);
+  h->commit();
+  { gcn_admm_host::Table<unsigned short>().swap(h->gi.col_comm); }   // needed on the device only
+  if (L >= 2) h->RN[L] = h->B0;   // R_L is turned into its new value in place
+  h->status = &h->report->status;
+  h->tc_error = &h->report->error;
 
   // Z_0 in community order, then P_1 = A~ Z_0 (Z_0 never changes, so neither does P_1)
   {
-    float* dense = nullptr;
     const bool on_device = is_device_pointer(X);
-    if (!on_device) {
-      dense = dalloc<float>(rows * h->C[0]);
-      cudaError_t e = cudaMemcpy(dense, X, rows * h->C[0] * sizeof(float), cudaMemcpyHostToDevice);
-      if (e != cudaSuccess) { cudaFree(dense); throw Fail{GCN_ADMM_ERR_CUDA, cudaGetErrorString(e)}; }
-    }
-    float* x_pad = nullptr;
-    try {
-      x_pad = dalloc<float>(rows * h->ld[0]);
+    if (on_device) CU(cudaDeviceSynchronize());
+    else CU(h->stage.put(h->B0, X, rows * h->C[0] * sizeof(float), h->stream));
+    CU(h->stage.flush(h->stream));
+    {
       gcn_admm::Scope sc(h, "permute_rows", 1, 8.0 * (double)n * h->C[0], 0.0);
-      gk::k_permute_rows<<<h->grid_for(n * h->ld[0]), 256, 0, h->stream>>>(on_device ? X : dense, x_pad, h->d_perm, n,
-                                                                           h->C[0], h->ld[0], 1);
+      gk::k_permute_rows<<<h->grid_for(n * h->ld[0]), 256, 0, h->stream>>>(on_device ? X : h->B0, h->B1, h->d_inv, n, h->C[0], h->ld[0], 1);
       CU(cudaGetLastError());
-      h->spmm(x_pad, h->P[1], h->ld[0]);
-      CU(cudaStreamSynchronize(h->stream));
-    } catch (...) {
-      if (dense) cudaFree(dense);
-      if (x_pad) cudaFree(x_pad);
-      throw;
     }
-    if (dense) cudaFree(dense);
-    cudaFree(x_pad);
+    h->spmm(h->B1, h->P[1], h->ld[0]);
   }
 
   for (int l = 1; l <= L; ++l) {
@@ -1158,6 +1218,7 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
     }
   }
   h->fresh = true;
+  CU(h->stage.finish(h->stream));
   CU(cudaStreamSynchronize(h->stream));
 }
 
@@ -1232,7 +1293,8 @@ void gcn_admm_destroy(gcn_admm* h) {
     h->collect_profile();
     if (h->pass_graph) cudaGraphExecDestroy(h->pass_graph);
     for (cudaEvent_t e : h->event_pool) cudaEventDestroy(e);
-    for (void* q : h->owned) cudaFree(q);
+    for (const gcn_admm_mem::Slab& q : h->slabs) gcn_admm_mem::Pool::get().give(q);
+    h->stage.close();
   }
   cudaGetLastError();
   delete h;
@@ -1315,14 +1377,15 @@ int gcn_admm_objective(gcn_admm* h, double out[6]) {
     if (!h->fresh) h->refresh();
     const int L = h->L;
     cudaStream_t s = h->stream;
-    CU(cudaMemsetAsync(h->obj, 0, 8 * sizeof(double), s));
+    double* const obj = h->report->obj;
+    CU(cudaMemsetAsync(obj, 0, 8 * sizeof(double), s));
     // every sum: per-block partials, then one block adds them in a fixed order
     for (int l = 1; l < L; ++l) {
       const long long n4 = h->n * h->ld[l] / 4;
       gcn_admm::Scope sc(h, "objective_sums", 2, 32.0 * n4, 0.0);
       const int grid = h->grid_for(n4);
       gk::k_sum_hidden_penalty<<<grid, 256, 0, s>>>((const float4*)h->Z[l], (const float4*)h->H[l], n4, h->red_part);
-      gk::k_add_partials<<<1, 256, 0, s>>>(h->red_part, grid, 1, h->obj + 2);
+      gk::k_add_partials<<<1, 256, 0, s>>>(h->red_part, grid, 1, obj + 2);
     }
     const long long n4 = h->n * h->ld[L] / 4;
     const int warps = 8;
@@ -1332,23 +1395,22 @@ int gcn_admm_objective(gcn_admm* h, double out[6]) {
       const int grid = h->grid_for(n4);
       gk::k_sum_constraint<<<grid, 256, 0, s>>>((const float4*)h->Z[L], (const float4*)h->H[L], (const float4*)h->U, n4,
                                                 h->red_part);
-      gk::k_add_partials<<<1, 256, 0, s>>>(h->red_part, grid, 2, h->obj + 3);
+      gk::k_add_partials<<<1, 256, 0, s>>>(h->red_part, grid, 2, obj + 3);
       gk::k_row_loss_argmax<<<row_blocks, warps * 32, 0, s>>>(h->Z[L], nullptr, h->ld[L], h->C[L], (int)h->n, h->d_y,
-                                                              h->d_train, nullptr, h->red_part);
-      gk::k_add_partials<<<1, 256, 0, s>>>(h->red_part, row_blocks, 2, h->obj);      // obj[0] = cross-entropy sum
+                                                              h->d_train, nullptr, nullptr, h->red_part);
+      gk::k_add_partials<<<1, 256, 0, s>>>(h->red_part, row_blocks, 2, obj);      // obj[0] = cross-entropy sum
       CU(cudaGetLastError());
     }
     h->forward_logits();
     {
       gcn_admm::Scope sc_obj(h, "objective_sums", 2, 4.0 * (double)h->n * h->ld[L], 0.0);
       gk::k_row_loss_argmax<<<row_blocks, warps * 32, 0, s>>>(nullptr, h->B0, h->ld[L], h->C[L], (int)h->n, h->d_y,
-                                                              h->d_train, nullptr, h->red_part);
-      gk::k_add_partials<<<1, 256, 0, s>>>(h->red_part, row_blocks, 2, h->obj + 5);  // obj[6] = correct training rows
+                                                              h->d_train, nullptr, nullptr, h->red_part);
+      gk::k_add_partials<<<1, 256, 0, s>>>(h->red_part, row_blocks, 2, obj + 5);  // obj[6] = correct training rows
       CU(cudaGetLastError());
     }
-    double v[8];
-    CU(cudaMemcpyAsync(v, h->obj, 8 * sizeof(double), cudaMemcpyDeviceToHost, s));
-    CU(cudaStreamSynchronize(s));
+    const gk::Report report = h->read_report();
+    const double* const v = report.obj;
     const double R = h->p.loss_scale * v[0];
     const double pen = 0.5 * h->p.nu * v[2];
     const double ur = v[3];
@@ -1356,7 +1418,7 @@ int gcn_admm_objective(gcn_admm* h, double out[6]) {
     out[0] = R + pen + ur + rr;
     out[1] = R; out[2] = pen; out[3] = ur; out[4] = rr;
     out[5] = h->n_train > 0 ? v[6] / h->n_train : 0.0;
-    h->check_status();
+    h->check(report);
   });
 }
 
@@ -1371,14 +1433,13 @@ int gcn_admm_predict(gcn_admm* h, float* logits, int* labels) {
     if (labels) {
       const int warps = 8;
       int* d_lab = reinterpret_cast<int*>(h->B1);
-      gcn_admm::Scope sc(h, "row_argmax", 1, 4.0 * (double)h->n * h->ld[L], 0.0);
-      gk::k_row_loss_argmax<<<(unsigned)cdiv(h->n, warps), warps * 32, 0, h->stream>>>(
-          nullptr, h->B0, h->ld[L], h->C[L], (int)h->n, h->d_y, h->d_train, d_lab, h->red_part);
-      CU(cudaGetLastError());
-      std::vector<int> lab(h->n);
-      CU(cudaMemcpyAsync(lab.data(), d_lab, sizeof(int) * h->n, cudaMemcpyDeviceToHost, h->stream));
-      CU(cudaStreamSynchronize(h->stream));
-      for (long long i = 0; i < h->n; ++i) labels[h->gi.perm[i]] = lab[i];
+      {
+        gcn_admm::Scope sc(h, "row_argmax", 1, 4.0 * (double)h->n * h->ld[L], 0.0);
+        gk::k_row_loss_argmax<<<(unsigned)cdiv(h->n, warps), warps * 32, 0, h->stream>>>(
+            nullptr, h->B0, h->ld[L], h->C[L], (int)h->n, h->d_y, h->d_train, d_lab, h->d_perm, h->red_part);
+        CU(cudaGetLastError());
+      }
+      CU(h->stage.get(labels, d_lab, sizeof(int) * h->n, sizeof(int) * h->n, 1, h->stream));
     }
     if (logits) h->rows_to_host(h->B0, h->C[L], logits);
     CU(cudaStreamSynchronize(h->stream));
@@ -1403,9 +1464,11 @@ int gcn_admm_propagate(gcn_admm* h, const float* x, int width, float* out) {
     float *a = fits ? h->B0 : dalloc<float>(elems), *b = nullptr;
     try {
       b = fits ? h->B1 : dalloc<float>(elems);
-      CU(cudaMemcpyAsync(a, x, bytes, cudaMemcpyHostToDevice, h->stream));
+      CU(h->stage.put(a, x, bytes, h->stream));
+      CU(h->stage.flush(h->stream));
       h->propagate_dense(a, width, b);
-      CU(cudaMemcpyAsync(out, b, bytes, cudaMemcpyDeviceToHost, h->stream));
+      CU(h->stage.get(out, b, bytes, bytes, 1, h->stream));
+      CU(h->stage.finish(h->stream));
       CU(cudaStreamSynchronize(h->stream));
     } catch (...) {
       if (!fits) { cudaFree(a); cudaFree(b); }
@@ -1577,7 +1640,7 @@ int gcn_admm_propagate_sharded(gcn_admm* h, int n_ranks, const float* x, int wid
       float* b = static_cast<float*>(take(rows * ldw * sizeof(float)));
       CU(cudaMemcpyAsync(dense, x, rows * width * sizeof(float), dev_in ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
                          h->stream));
-      gk::k_permute_rows<<<h->grid_for(h->n * ldw), 256, 0, h->stream>>>(dense, a, h->d_perm, h->n, width, ldw, 1);
+      gk::k_permute_rows<<<h->grid_for(h->n * ldw), 256, 0, h->stream>>>(dense, a, h->d_inv, h->n, width, ldw, 1);
       CU(cudaGetLastError());
       for (int r = 0; r < R; ++r) {
         const int lo = plan.row_begin[r], hi = plan.row_begin[r + 1], n_own = hi - lo;
@@ -1638,7 +1701,7 @@ int gcn_admm_propagate_sharded(gcn_admm* h, int n_ranks, const float* x, int wid
         }
         CU(cudaStreamSynchronize(h->stream));   // the host vectors of this rank go out of scope
       }
-      gk::k_permute_rows<<<h->grid_for(h->n * ldw), 256, 0, h->stream>>>(b, dense, h->d_perm, h->n, width, ldw, 0);
+      gk::k_permute_rows<<<h->grid_for(h->n * ldw), 256, 0, h->stream>>>(b, dense, h->d_inv, h->n, width, ldw, 0);
       CU(cudaGetLastError());
       h->launches += 2;   // the two row permutations
       CU(cudaMemcpyAsync(out, dense, rows * width * sizeof(float), dev_out ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
@@ -1663,11 +1726,7 @@ int gcn_admm_get_state(gcn_admm* h, int which, int layer, void* out) {
     if (which == GCN_ADMM_ST_W) {
       need_layer(1, L);
       const int r = h->C[layer - 1], c = h->C[layer], ldw = h->ld[layer];
-      std::vector<float> w((size_t)r * ldw);
-      CU(cudaMemcpyAsync(w.data(), h->W[layer], w.size() * sizeof(float), cudaMemcpyDeviceToHost, h->stream));
-      CU(cudaStreamSynchronize(h->stream));
-      float* o = static_cast<float*>(out);
-      for (int i = 0; i < r; ++i) std::memcpy(o + (size_t)i * c, w.data() + (size_t)i * ldw, c * sizeof(float));
+      CU(h->stage.get(out, h->W[layer], sizeof(float) * c, sizeof(float) * ldw, r, h->stream));
     } else if (which == GCN_ADMM_ST_Z) {
       need_layer(1, L);
       h->rows_to_host(h->Z[layer], h->C[layer], static_cast<float*>(out));
@@ -1675,17 +1734,10 @@ int gcn_admm_get_state(gcn_admm* h, int which, int layer, void* out) {
       h->rows_to_host(h->U, h->C[L], static_cast<float*>(out));
     } else if (which == GCN_ADMM_ST_TAU) {
       need_layer(1, L);
-      SearchCtl c;
-      CU(cudaMemcpyAsync(&c, h->ctl_w + layer, sizeof(c), cudaMemcpyDeviceToHost, h->stream));
-      CU(cudaStreamSynchronize(h->stream));
-      *static_cast<double*>(out) = c.t_prev;
+      h->take_steps(h->ctl_w + layer, static_cast<double*>(out), 1);
     } else if (which == GCN_ADMM_ST_THETA) {
       need_layer(1, L - 1);
-      std::vector<SearchCtl> c(h->M);
-      CU(cudaMemcpyAsync(c.data(), h->ctl_z + (size_t)layer * h->M, c.size() * sizeof(SearchCtl), cudaMemcpyDeviceToHost,
-                         h->stream));
-      CU(cudaStreamSynchronize(h->stream));
-      for (int m = 0; m < h->M; ++m) static_cast<double*>(out)[m] = c[m].t_prev;
+      h->take_steps(h->ctl_z + (size_t)layer * h->M, static_cast<double*>(out), h->M);
     } else if (which == GCN_ADMM_ST_PIPELINE_FLAG) {
       CU(cudaMemcpyAsync(out, h->tc_error, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
       CU(cudaStreamSynchronize(h->stream));
@@ -1716,17 +1768,13 @@ int gcn_admm_set_state(gcn_admm* h, int which, int layer, const void* in) {
       need_layer(1, L);
       const double t = *static_cast<const double*>(in);
       if (!(t > 0.0)) throw Fail{GCN_ADMM_ERR_ARG, "tau must be positive"};
-      CU(cudaMemcpyAsync(&h->ctl_w[layer].t_prev, &t, sizeof(double), cudaMemcpyHostToDevice, h->stream));
-      CU(cudaStreamSynchronize(h->stream));
+      h->put_steps(h->ctl_w + layer, &t, 1);
     } else if (which == GCN_ADMM_ST_THETA) {
       need_layer(1, L - 1);
       const double* t = static_cast<const double*>(in);
-      for (int m = 0; m < h->M; ++m) {
+      for (int m = 0; m < h->M; ++m)
         if (!(t[m] > 0.0)) throw Fail{GCN_ADMM_ERR_ARG, "theta must be positive"};
-        CU(cudaMemcpyAsync(&h->ctl_z[(size_t)layer * h->M + m].t_prev, t + m, sizeof(double), cudaMemcpyHostToDevice,
-                           h->stream));
-      }
-      CU(cudaStreamSynchronize(h->stream));
+      h->put_steps(h->ctl_z + (size_t)layer * h->M, t, h->M);
     } else if (which == GCN_ADMM_ST_PIPELINE_FLAG) {
       CU(cudaMemcpyAsync(h->tc_error, in, sizeof(int), cudaMemcpyHostToDevice, h->stream));
       CU(cudaStreamSynchronize(h->stream));

@@ -320,6 +320,25 @@ inline void build_long_row_tables(const GraphIndex& g, int limit, LongRowTables&
   }
 }
 
+// Rows of every community by falling number of stored entries, ties by row id: a counting sort per community.
+inline void order_rows_by_length(const GraphIndex& g, Table<int>& order) {
+  order.resize((std::size_t)g.n);
+#pragma omp parallel
+  {
+    std::vector<int> at;
+#pragma omp for schedule(dynamic, 1)
+    for (int m = 0; m < g.n_comm; ++m) {
+      const int lo = g.comm_ptr[m], hi = g.comm_ptr[m + 1];
+      int longest = 0;
+      for (int i = lo; i < hi; ++i) longest = std::max(longest, g.row_ptr[i + 1] - g.row_ptr[i]);
+      at.assign((std::size_t)longest + 2, 0);
+      for (int i = lo; i < hi; ++i) ++at[(std::size_t)(longest - (g.row_ptr[i + 1] - g.row_ptr[i])) + 1];
+      for (int k = 0; k <= longest; ++k) at[(std::size_t)k + 1] += at[(std::size_t)k];
+      for (int i = lo; i < hi; ++i) order[(std::size_t)(lo + at[(std::size_t)(longest - (g.row_ptr[i + 1] - g.row_ptr[i]))]++)] = i;
+    }
+  }
+}
+
 // First-order neighbour rows of community m: new ids outside V_m adjacent to V_m, ascending.
 inline std::vector<int> halo1_of(const GraphIndex& g, int m) {
   std::vector<int> out;

@@ -27,6 +27,13 @@ struct SearchCtl {
   float inv_cand[kCand];  // 1/t of the candidates of the current pass
 };
 
+// Numbers and flags the host reads back together.
+struct Report {
+  double obj[8];
+  int status;    // bit 0: a NaN or an infinity reached a step-size decision
+  int error;     // a bounded wait ran out: 1 in a tensor-core product, kErrGridBarrier in a search
+};
+
 __device__ __forceinline__ float relu(float x) { return x > 0.f ? x : 0.f; }
 
 // relu(h) - relu(h - s) without forming h - s when both sides are active, so that a step s far
@@ -1791,13 +1798,13 @@ k_add_partials(const double* __restrict__ partial, int n_part, int per, double* 
 }
 
 // Per row: cross-entropy of the row of Zrows with its label (training rows only); argmax of the row of
-// `logits` (lowest index on ties) to labels[row]; whether a training row's argmax equals its label.
+// `logits` (lowest index on ties) to labels[perm[row]], the caller's order; whether a training row's argmax equals its label.
 // One warp per row; partial[2b] = the block's cross-entropy sum, partial[2b+1] = its count of hits,
 // rows added in row order.  Either of Zrows / logits may be NULL.
 __global__ void __launch_bounds__(256)
 k_row_loss_argmax(const float* __restrict__ Zrows, const float* __restrict__ logits, int ld, int C, int n,
                   const int* __restrict__ y, const unsigned char* __restrict__ train,
-                  int* __restrict__ labels, double* __restrict__ partial) {
+                  int* __restrict__ labels, const int* __restrict__ perm, double* __restrict__ partial) {
   __shared__ double s_loss[8], s_hit[8];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int row = blockIdx.x * (blockDim.x >> 5) + warp;
@@ -1827,7 +1834,7 @@ k_row_loss_argmax(const float* __restrict__ Zrows, const float* __restrict__ log
         const int oa = __shfl_xor_sync(0xffffffffu, arg, o);
         if (ob > best || (ob == best && oa < arg)) { best = ob; arg = oa; }
       }
-      if (lane == 0 && labels) labels[row] = arg;
+      if (lane == 0 && labels) labels[perm[row]] = arg;
       if (tr && arg == y[row]) hit = 1.0;
     }
   }
@@ -1873,14 +1880,29 @@ __global__ void k_transpose_small(const float* __restrict__ src, int lds, float*
   dst[c * ldd + r] = src[r * lds + c];
 }
 
-__global__ void k_fill_int(int* __restrict__ p, long long count, int value) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < count;
-       i += (long long)gridDim.x * blockDim.x)
-    p[i] = value;
+// W (rows x cols, leading dimension ldw) and its transpose from a dense matrix; padding columns become zero.
+__global__ void k_load_weight(const float* __restrict__ src, int rows, int cols, float* __restrict__ W, int ldw,
+                              float* __restrict__ Wt, int ldwt) {
+  const long long first = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
+  for (long long i = first; i < (long long)rows * ldw; i += stride) {
+    const long long r = i / ldw, c = i - r * ldw;
+    W[i] = c < cols ? src[r * cols + c] : 0.f;
+  }
+  for (long long i = first; i < (long long)cols * ldwt; i += stride) {
+    const long long c = i / ldwt, r = i - c * ldwt;
+    Wt[i] = r < rows ? src[r * cols + c] : 0.f;
+  }
 }
 
-// Row gather / scatter between the caller's dense layout (original order, width C) and the
-// internal one (community order, leading dimension ld).  to_internal != 0: dst[new] = src[perm[new]].
+__global__ void k_put_steps(SearchCtl* __restrict__ ctl, const double* __restrict__ values, int count) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < count) ctl[i].t_prev = values[i];
+}
+__global__ void k_take_steps(const SearchCtl* __restrict__ ctl, double* __restrict__ values, int count) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < count) values[i] = ctl[i].t_prev;
+}
+
 // dst[r] = src[rows[r]] for padded rows of ld4 float4: the staging copy of the rows a rank does not own
 // (what a receive from their owners would deliver) behind its own rows.
 __global__ void k_gather_rows(const float4* __restrict__ src, const int* __restrict__ rows, float4* __restrict__ dst,
@@ -1892,16 +1914,31 @@ __global__ void k_gather_rows(const float4* __restrict__ src, const int* __restr
   }
 }
 
-__global__ void k_permute_rows(const float* __restrict__ src, float* __restrict__ dst, const int* __restrict__ perm,
-                               long long n, int C, int ld, int to_internal) {
-  const long long total = n * ld;
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (long long)gridDim.x * blockDim.x) {
-    const long long r = e / ld;
-    const int c = (int)(e % ld);
-    if (to_internal) dst[e] = (c < C) ? src[(long long)perm[r] * C + c] : 0.f;
-    else if (c < C) dst[(long long)perm[r] * C + c] = src[e];
+// Row gather / scatter between the caller's dense layout (original order, width C) and the internal one (community order,
+// leading dimension ld, padding columns zero).  `inv`: original id -> new id.  Both directions walk the caller's matrix in
+// its order, so that it can lie in host memory (reads and writes over the bus are then whole lines); the scattered side is
+// the device's own.
+template <typename I>
+__device__ __forceinline__ void permute_rows(const float* __restrict__ src, float* __restrict__ dst, const int* __restrict__ inv,
+                                             I n, I C, I ld, int to_internal) {
+  const I first = (I)blockIdx.x * blockDim.x + threadIdx.x, stride = (I)gridDim.x * blockDim.x;
+  if (to_internal) {
+    for (I e = first; e < n * ld; e += stride) {
+      const I r = e / ld, c = e - r * ld;
+      dst[(long long)inv[r] * ld + c] = c < C ? src[(long long)r * C + c] : 0.f;
+    }
+  } else {
+    for (I e = first; e < n * C; e += stride) {
+      const I r = e / C, c = e - r * C;
+      dst[e] = src[(long long)inv[r] * ld + c];
+    }
   }
+}
+__global__ void k_permute_rows(const float* __restrict__ src, float* __restrict__ dst, const int* __restrict__ inv,
+                               long long n, int C, int ld, int to_internal) {
+  if (n * ld + (long long)gridDim.x * blockDim.x < (1LL << 32))   // 32-bit divisions
+    permute_rows<unsigned>(src, dst, inv, (unsigned)n, (unsigned)C, (unsigned)ld, to_internal);
+  else permute_rows<long long>(src, dst, inv, n, C, ld, to_internal);
 }
 
 }  // namespace gk

@@ -1,0 +1,284 @@
+// Memory of a handle: one device slab that all its matrices and tables are cut from, and a page-locked staging
+// buffer through which host buffers are copied in both directions.
+//
+// A handle has about sixty device buffers.  Allocated one by one they cost 5 ms to create and 2 ms to free on a quiet
+// machine, more than the twenty passes of a small training run, and ten times that where other processes use the
+// driver too.  Copies between the device and pageable host memory go through the driver's own staging on one core at
+// 5-10 GB/s; here several cores fill or drain one part of the staging buffer while the copy engine works on the next.
+//
+// Slabs and staging buffers of destroyed handles are kept for later ones up to a fixed amount (kIdleSlabBytes,
+// kIdleStages; the oldest go first), under a lock, and only after the work that used them has finished; the rest goes back
+// to the driver at once, everything at exit or when an allocation fails.
+#pragma once
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cstddef>
+#include <cstring>
+#include <mutex>
+#include <vector>
+
+namespace gcn_admm_mem {
+
+constexpr std::size_t kIdleSlabBytes = (std::size_t)3 << 30;     // device memory kept for later handles, all devices together
+constexpr std::size_t kIdleStages = 4;
+constexpr std::size_t kSlot = (std::size_t)4 << 20;               // a staging buffer is kSlots parts of this size
+constexpr int kSlots = 3;
+
+struct Slab {
+  int device = 0;
+  char* base = nullptr;
+  std::size_t size = 0;
+};
+
+class Pool {
+ public:
+  static Pool& get() {
+    static Pool pool;
+    return pool;
+  }
+  // A slab of at least `bytes` on the current device (`device`).
+  cudaError_t take(int device, std::size_t bytes, Slab* out) {
+    const std::size_t grain = (std::size_t)2 << 20;
+    bytes = (bytes + grain - 1) / grain * grain;
+    {
+      std::lock_guard<std::mutex> lock(mutex_);
+      auto best = idle_.end();
+      for (auto it = idle_.begin(); it != idle_.end(); ++it)
+        if (it->device == device && it->size >= bytes && it->size <= 2 * bytes + 8 * grain && (best == idle_.end() || it->size < best->size))
+          best = it;
+      if (best != idle_.end()) {
+        *out = *best;
+        idle_bytes_ -= best->size;
+        idle_.erase(best);
+        return cudaSuccess;
+      }
+    }
+    void* p = nullptr;
+    cudaError_t e = cudaMalloc(&p, bytes);
+    if (e == cudaErrorMemoryAllocation) {
+      cudaGetLastError();
+      trim(device);
+      e = cudaMalloc(&p, bytes);
+    }
+    if (e == cudaSuccess) *out = Slab{device, static_cast<char*>(p), bytes};
+    return e;
+  }
+  // The slab's device is current and no work uses the slab any more.
+  void give(const Slab& s) {
+    if (!s.base) return;
+    std::vector<Slab> out;   // the oldest make room; their work has finished too
+    {
+      std::lock_guard<std::mutex> lock(mutex_);
+      if (s.size <= kIdleSlabBytes) {
+        while (idle_bytes_ + s.size > kIdleSlabBytes) {
+          out.push_back(idle_.front());
+          idle_bytes_ -= idle_.front().size;
+          idle_.erase(idle_.begin());
+        }
+        idle_bytes_ += s.size;
+        idle_.push_back(s);
+      } else {
+        out.push_back(s);
+      }
+    }
+    for (const Slab& o : out) cudaFree(o.base);
+  }
+  char* take_stage() {
+    {
+      std::lock_guard<std::mutex> lock(mutex_);
+      if (!stages_.empty()) {
+        char* p = stages_.back();
+        stages_.pop_back();
+        return p;
+      }
+    }
+    void* p = nullptr;
+    if (cudaHostAlloc(&p, kSlot * kSlots, cudaHostAllocPortable) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    return static_cast<char*>(p);
+  }
+  void give_stage(char* p) {
+    if (!p) return;
+    {
+      std::lock_guard<std::mutex> lock(mutex_);
+      if (stages_.size() < kIdleStages) { stages_.push_back(p); return; }
+    }
+    cudaFreeHost(p);
+  }
+  ~Pool() {   // at exit the driver may already be gone: its error is of no consequence then
+    for (const Slab& s : idle_) cudaFree(s.base);
+    for (char* p : stages_) cudaFreeHost(p);
+  }
+
+ private:
+  void trim(int device) {
+    std::vector<Slab> out;
+    {
+      std::lock_guard<std::mutex> lock(mutex_);
+      for (auto it = idle_.begin(); it != idle_.end();)
+        if (it->device == device) { out.push_back(*it); idle_bytes_ -= it->size; it = idle_.erase(it); }
+        else ++it;
+    }
+    for (const Slab& s : out) cudaFree(s.base);
+  }
+  std::mutex mutex_;
+  std::vector<Slab> idle_;
+  std::size_t idle_bytes_ = 0;
+  std::vector<char*> stages_;
+};
+
+// memcpy by several threads where it pays (a core moves about 10 GB/s, less into pages that are touched first here).
+inline void copy_bytes(void* dst, const void* src, std::size_t bytes) {
+  constexpr std::size_t kPiece = (std::size_t)256 << 10;
+  if (bytes < 4 * kPiece) { std::memcpy(dst, src, bytes); return; }
+  const long long pieces = (long long)((bytes + kPiece - 1) / kPiece);
+#pragma omp parallel for schedule(static) num_threads(8)
+  for (long long i = 0; i < pieces; ++i) {
+    const std::size_t at = (std::size_t)i * kPiece;
+    std::memcpy(static_cast<char*>(dst) + at, static_cast<const char*>(src) + at, std::min(kPiece, bytes - at));
+  }
+}
+
+// Is `p` host memory the copy engine can reach by itself (page-locked)?
+inline bool page_locked(const void* p) {
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) { cudaGetLastError(); return false; }
+  return a.type == cudaMemoryTypeHost;
+}
+
+// The staging buffer of one handle.  Copies are enqueued on the handle's stream; kSlots parts take turns, each with an
+// event after its last use.
+class Stage {
+ public:
+  cudaError_t open() {
+    if (base_) return cudaSuccess;
+    base_ = Pool::get().take_stage();
+    if (!base_) return cudaErrorMemoryAllocation;
+    for (cudaEvent_t& e : used_) {
+      const cudaError_t err = cudaEventCreateWithFlags(&e, cudaEventDisableTiming);
+      if (err != cudaSuccess) return err;
+    }
+    return cudaSuccess;
+  }
+  // Nothing is in flight any more.
+  void close() {
+    for (cudaEvent_t& e : used_)
+      if (e) { cudaEventDestroy(e); e = nullptr; }
+    Pool::get().give_stage(base_);
+    base_ = nullptr;
+  }
+
+  // Host -> device.  Small pieces whose destinations follow each other (up to `slack` bytes apart) leave as one copy; flush()
+  // sends the last one.  The source may be reused after finish().
+  cudaError_t put(void* dst, const void* src, std::size_t bytes, cudaStream_t stream) {
+    if (bytes == 0) return cudaSuccess;
+    if (bytes >= kSlot / 4 && page_locked(src)) {
+      if (const cudaError_t e = flush(stream)) return e;
+      direct_ = true;
+      return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, stream);
+    }
+    constexpr std::ptrdiff_t slack = 256;
+    char* d = static_cast<char*>(dst);
+    const char* s = static_cast<const char*>(src);
+    while (bytes > 0) {
+      const std::ptrdiff_t gap = d - (run_dst_ + run_);
+      if (run_ == 0 || gap < 0 || gap > slack || run_ + (std::size_t)gap >= kSlot) {
+        if (const cudaError_t e = flush(stream)) return e;
+        if (const cudaError_t e = cudaEventSynchronize(used_[slot_])) return e;
+        run_dst_ = d;
+      } else if (gap > 0) {
+        std::memset(part() + run_, 0, (std::size_t)gap);   // alignment gap between two tables of the slab
+        run_ += (std::size_t)gap;
+      }
+      const std::size_t now = std::min(bytes, kSlot - run_);
+      copy_bytes(part() + run_, s, now);
+      run_ += now; d += now; s += now; bytes -= now;
+      if (run_ == kSlot)
+        if (const cudaError_t e = flush(stream)) return e;
+    }
+    return cudaSuccess;
+  }
+  // Ends an upload: sends what is left and waits where a source is still being read in place.
+  cudaError_t finish(cudaStream_t stream) {
+    if (const cudaError_t e = flush(stream)) return e;
+    if (!direct_) return cudaSuccess;
+    direct_ = false;
+    return cudaStreamSynchronize(stream);
+  }
+  cudaError_t flush(cudaStream_t stream) {
+    if (run_ == 0) return cudaSuccess;
+    cudaError_t e = cudaMemcpyAsync(run_dst_, part(), run_, cudaMemcpyHostToDevice, stream);
+    if (e == cudaSuccess) e = cudaEventRecord(used_[slot_], stream);
+    run_ = 0;
+    slot_ = (slot_ + 1) % kSlots;
+    return e;
+  }
+
+  // A part of the buffer that kernels may read (after the host has filled it) or write: valid until leave().
+  // At most kSlot bytes.
+  cudaError_t enter(cudaStream_t stream, char** out) {
+    if (const cudaError_t e = flush(stream)) return e;
+    if (const cudaError_t e = cudaEventSynchronize(used_[slot_])) return e;
+    *out = part();
+    return cudaSuccess;
+  }
+  cudaError_t leave(cudaStream_t stream) {
+    const cudaError_t e = cudaEventRecord(used_[slot_], stream);
+    slot_ = (slot_ + 1) % kSlots;
+    return e;
+  }
+
+  // Device -> host: `rows` rows of `width` bytes, `pitch` bytes apart on the device, dense on the host.  Returns with the
+  // host buffer filled.
+  cudaError_t get(void* dst, const void* src, std::size_t width, std::size_t pitch, std::size_t rows, cudaStream_t stream) {
+    if (width == 0 || rows == 0) return cudaSuccess;
+    if (const cudaError_t e = flush(stream)) return e;
+    if (width == pitch) { width *= rows; pitch = width; rows = 1; }
+    if (width * rows >= kSlot / 4 && page_locked(dst)) {
+      const cudaError_t e = rows == 1 ? cudaMemcpyAsync(dst, src, width, cudaMemcpyDeviceToHost, stream)
+                                      : cudaMemcpy2DAsync(dst, width, src, pitch, width, rows, cudaMemcpyDeviceToHost, stream);
+      return e ? e : cudaStreamSynchronize(stream);
+    }
+    // pieces of at most a slot: whole rows, or parts of one row when a row is longer than that
+    const std::size_t rows_at_once = std::max<std::size_t>(1, kSlot / width);
+    const std::size_t per_row = rows == 1 ? (width + kSlot - 1) / kSlot : 1;
+    if (rows > 1 && width > kSlot) {
+      for (std::size_t r = 0; r < rows; ++r)
+        if (const cudaError_t e = get(static_cast<char*>(dst) + r * width, static_cast<const char*>(src) + r * pitch, width, width, 1, stream)) return e;
+      return cudaSuccess;
+    }
+    const std::size_t pieces = rows == 1 ? per_row : (rows + rows_at_once - 1) / rows_at_once;
+    auto begin = [&](std::size_t i) -> cudaError_t {
+      char* to = base_ + (std::size_t)((slot_ + i) % kSlots) * kSlot;
+      cudaError_t e = cudaEventSynchronize(used_[(slot_ + i) % kSlots]);
+      if (e != cudaSuccess) return e;
+      if (rows == 1) e = cudaMemcpyAsync(to, static_cast<const char*>(src) + i * kSlot, std::min(kSlot, width - i * kSlot), cudaMemcpyDeviceToHost, stream);
+      else e = cudaMemcpy2DAsync(to, width, static_cast<const char*>(src) + i * rows_at_once * pitch, pitch, width,
+                                 std::min(rows_at_once, rows - i * rows_at_once), cudaMemcpyDeviceToHost, stream);
+      return e ? e : cudaEventRecord(used_[(slot_ + i) % kSlots], stream);
+    };
+    for (std::size_t i = 0; i < std::min<std::size_t>(pieces, kSlots - 1); ++i)
+      if (const cudaError_t e = begin(i)) return e;
+    for (std::size_t i = 0; i < pieces; ++i) {
+      if (i + kSlots - 1 < pieces)
+        if (const cudaError_t e = begin(i + kSlots - 1)) return e;
+      if (const cudaError_t e = cudaEventSynchronize(used_[(slot_ + i) % kSlots])) return e;
+      const std::size_t at = rows == 1 ? i * kSlot : i * rows_at_once * width;
+      const std::size_t len = rows == 1 ? std::min(kSlot, width - at) : std::min(rows_at_once, rows - i * rows_at_once) * width;
+      copy_bytes(static_cast<char*>(dst) + at, base_ + (std::size_t)((slot_ + i) % kSlots) * kSlot, len);
+    }
+    slot_ = (int)((slot_ + pieces) % kSlots);
+    return cudaSuccess;
+  }
+
+ private:
+  char* part() { return base_ + (std::size_t)slot_ * kSlot; }
+  char* base_ = nullptr;
+  cudaEvent_t used_[kSlots] = {};
+  int slot_ = 0;
+  char* run_dst_ = nullptr;   // destination of the run being filled and its length so far
+  std::size_t run_ = 0;
+  bool direct_ = false;       // a page-locked source is being read by the copy engine
+};
+
+}  // namespace gcn_admm_mem
