@@ -349,8 +349,10 @@ struct gcn_admm {
     T *out = reinterpret_cast<T*>(outf), *scratch = reinterpret_cast<T*>(item_sums);
     const int ld4 = (int)cdiv((long long)ldv * VEC, 4);
     const long long units = (long long)g.n + g.n_items;
-#define WIDE(NV4, UN)                                                                                                     \
-  gk::k_spmm_wide<VEC, 4 / VEC * (NV4), UN, MAPPED><<<(unsigned)cdiv(units * 32, 64), 64, 0, stream>>>( \
+#define WIDE(NV4, UN, SLICED)                                                                                             \
+  gk::k_spmm_wide<VEC, 4 / VEC * (NV4), UN, MAPPED, SLICED>                                                               \
+      <<<dim3((unsigned)cdiv(units * 32, 64), (unsigned)std::min<long long>(32768, cdiv(ld4, 32 * (NV4))),                \
+              (unsigned)cdiv(ld4, 32768LL * 32 * (NV4))), 64, 0, stream>>>(                                               \
       g.row_ptr, g.col, g.dinv, g.perm, g.items, g.n, g.n_items, g.long_len, x, out, ldv, scratch)
 #define SETS(CL, EP, UN)                                                                                                  \
   gk::k_spmm_sets<VEC, 4 / VEC, CL, EP, UN, MAPPED><<<(unsigned)cdiv(units * ((CL) * (EP)), 128), 128, 0, stream>>>( \
@@ -370,8 +372,9 @@ struct gcn_admm {
       if (lanes <= 480000) SETS(8, 4, 8); else SETS(8, 1, 8);
     } else if (ld4 <= 16) {
       if (lanes <= 960000) SETS(16, 2, 8); else SETS(16, 1, 8);
-    } else if (ld4 <= 32) WIDE(1, 4);
-    else WIDE(2, 2);   // two neighbours in flight per lane beat four (fewer registers, more warps): measured
+    } else if (ld4 <= 32) WIDE(1, 4, false);
+    else if (ld4 > 64) WIDE(2, 2, true);
+    else WIDE(2, 2, false);   // two neighbours in flight per lane beat four (fewer registers, more warps): measured
 #undef WIDE
 #undef SETS
     CU(cudaGetLastError());
@@ -526,12 +529,12 @@ struct gcn_admm {
   // grad (and grad_t) from the `splits` partial sums gemm_tn left in `part`; with `ctl` the start of the W_l search too.
   void finish_grad(int splits, int Ka, int Nb, int ldp, float* out, float* out_t, int ldt, const float* w, SearchCtl* ctl) {
     Scope sc(this, "finish_grad", 1, 4.0 * (double)Ka * ldp * (splits + (w ? 3 : 1)), 0.0);
-    const long long col_blocks = cdiv(ldp, 32);
+    const long long elems = (long long)Ka * ldp;
     if (splits >= 16)
-      gk::k_finish_grad<8><<<(unsigned)(col_blocks * Ka), 256, 0, stream>>>(part, splits, Ka, Nb, ldp, out, out_t, ldt, w, red_part,
+      gk::k_finish_grad<8><<<(unsigned)cdiv(elems, 32), 256, 0, stream>>>(part, splits, Ka, Nb, ldp, out, out_t, ldt, w, red_part,
                                                                             ticket, ctl, p.bt_shrink, p.bt_growth, status);
     else
-      gk::k_finish_grad<1><<<(unsigned)(col_blocks * cdiv(Ka, 8)), 256, 0, stream>>>(part, splits, Ka, Nb, ldp, out, out_t, ldt, w, red_part,
+      gk::k_finish_grad<1><<<(unsigned)cdiv(elems, 256), 256, 0, stream>>>(part, splits, Ka, Nb, ldp, out, out_t, ldt, w, red_part,
                                                                                      ticket, ctl, p.bt_shrink, p.bt_growth, status);
     CU(cudaGetLastError());
   }
@@ -1116,7 +1119,7 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
     h->want(h->H[l], rows * h->ld[l]);
     const size_t ge = (size_t)h->C[l - 1] * h->ld[l];
     grad_elems = std::max(grad_elems, ge);
-    grad_blocks = std::max(grad_blocks, (size_t)h->C[l - 1] * (size_t)cdiv(h->ld[l], 32));
+    grad_blocks = std::max(grad_blocks, (size_t)cdiv((long long)ge, 32));
     grad_t_elems = std::max(grad_t_elems, (size_t)h->C[l] * h->ld[l - 1]);
     h->part_elems = std::max(h->part_elems, ge * 4 * kSmCount);
   }

@@ -61,17 +61,48 @@ __device__ __forceinline__ float warp_max(float v) {
   return v;
 }
 
-// Sum of `v` over the block; valid in thread 0.  `sh` holds >= 32 doubles.
+// Sums of N values over the block (up to 8 warps), valid in thread 0: all of them in one round, since a round costs two
+// barriers and the shuffle latencies whether it carries one value or four.  `sh` holds N * 8 doubles.
+template <int N>
+__device__ __forceinline__ void block_sums(double (&v)[N], double* sh) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int j = 0; j < N; ++j) v[j] += __shfl_xor_sync(0xffffffffu, v[j], o);
+  __syncthreads();
+  if (lane == 0)
+#pragma unroll
+    for (int j = 0; j < N; ++j) sh[j * 8 + w] = v[j];
+  __syncthreads();
+  if (w == 0) {
+#pragma unroll
+    for (int j = 0; j < N; ++j) v[j] = lane < nw ? sh[j * 8 + lane] : 0.0;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+      for (int j = 0; j < N; ++j) v[j] += __shfl_xor_sync(0xffffffffu, v[j], o);
+  }
+}
 __device__ __forceinline__ double block_sum(double v, double* sh) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  v = warp_sum(v);
+  double a[1] = {v};
+  block_sums(a, sh);
+  return a[0];
+}
+
+// Sums over the `count` blocks that left N values each in partial[b * N + ..], by one block: warp j adds value j, lanes strided,
+// then the shuffle tree.  total[0 .. N-1] (shared memory) is valid after the barrier at the end.
+template <int N>
+__device__ __forceinline__ void add_block_sums(const double* partial, int count, double* total) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  for (int j = w; j < N; j += nw) {
+    double t = 0.0;
+#pragma unroll 4
+    for (int b = lane; b < count; b += 32) t += __ldcg(partial + (size_t)b * N + j);
+    t = warp_sum(t);
+    if (lane == 0) total[j] = t;
+  }
   __syncthreads();
-  if (lane == 0) sh[w] = v;
-  __syncthreads();
-  const int nw = (blockDim.x + 31) >> 5;
-  v = (threadIdx.x < nw) ? sh[threadIdx.x] : 0.0;
-  if (w == 0) v = warp_sum(v);
-  return v;
 }
 
 // ------------------------------------------------------------------------------------------
@@ -143,11 +174,13 @@ __device__ __forceinline__ void finish_item(const ItemRows& ir, int unit, T* __r
   if (gl == 0) ir.done[lr] = 0;
 }
 
-// A warp per row, NV vectors per lane; wider rows loop over blocks of 32 NV vectors.  Lane t of a group of 32
+// A warp per row, NV vectors per lane.  SLICED: operands of more than 32 NV vectors, a warp per row and block of columns
+// (blockIdx.y and, past the limit of that, .z): more warps, and one slice of the operand at a time is what L2 has to hold
+// (1000 columns on 14 k rows 195 -> 142 us).  Lane t of a group of 32
 // stored entries holds column and weight of entry t, handed to the warp by shuffles.  UN neighbours in flight per
 // lane: the kernel is bound by the L2-to-SM traffic of the gathered rows, and by how the compiler orders its loads (the plain
 // loop measured faster than one that fetches columns ahead: 138 against 160 us at 128 columns on 169 k rows).
-template <int VEC, int NV, int UN, bool MAPPED>
+template <int VEC, int NV, int UN, bool MAPPED, bool SLICED>
 __global__ void __launch_bounds__(64, VEC == 4 ? 24 : 16)
 k_spmm_wide(const int* __restrict__ row_ptr, const int* __restrict__ col, const float* __restrict__ dinv,
             const int* __restrict__ perm, const int4* __restrict__ items, int n, int n_items, int long_len,
@@ -155,6 +188,9 @@ k_spmm_wide(const int* __restrict__ row_ptr, const int* __restrict__ col, const 
             typename Vec<VEC>::T* __restrict__ scratch) {
   using T = typename Vec<VEC>::T;
   const int lane = threadIdx.x & 31;
+  const int off = SLICED ? (blockIdx.y + gridDim.y * blockIdx.z) * (32 * NV) : 0;
+  const int wv = SLICED ? min(32 * NV, ldv - off) : ldv;   // this block's columns
+  if (SLICED) { x += off; out += off; scratch += off; }
   const int unit = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   if (unit >= n + n_items) return;
   int row, rs, re;
@@ -171,7 +207,8 @@ k_spmm_wide(const int* __restrict__ row_ptr, const int* __restrict__ col, const 
     dst = out + (long long)(MAPPED ? perm[row] : row) * ldv;
   }
   const float di = dinv[row];
-  for (int cb = 0; cb < ldv; cb += 32 * NV) {
+  // One turn only, but the compiler is not to know: it then issues all loads of a step before the first sum (+20 % at 256 columns).
+  for (int cb = 0; cb < wv; cb += 32 * NV) {
     T acc[NV];
 #pragma unroll
     for (int v = 0; v < NV; ++v) vzero(acc[v]);
@@ -195,7 +232,7 @@ k_spmm_wide(const int* __restrict__ row_ptr, const int* __restrict__ col, const 
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
           const int f = cb + lane + 32 * v;
-          if (f < ldv) {
+          if (f < wv) {
             T xv[UN];
 #pragma unroll
             for (int u = 0; u < UN; ++u) xv[u] = __ldg(x + (long long)rj[u] * ldv + f);
@@ -208,7 +245,7 @@ k_spmm_wide(const int* __restrict__ row_ptr, const int* __restrict__ col, const 
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
       const int f = cb + lane + 32 * v;
-      if (f < ldv) dst[f] = vscale(di, acc[v]);
+      if (f < wv) dst[f] = vscale(di, acc[v]);
     }
   }
 }
@@ -745,59 +782,72 @@ struct DecideArgs {
   double own_nu;     // nu when the block has a quadratic own term, else 0
 };
 
-__device__ __forceinline__ bool accept(SearchCtl* c, double delta, double t, int trial) {
-  const double need = c->gg / (2.0 * t);
-  if (delta <= -need) {          // f(x+) - f(x) <= -||g||^2 / (2t); false for NaN
-    c->t_prev = t;
-    c->q = -delta / need;
-    c->inv_step = (float)(1.0 / t);
-    c->trial = trial;
-    c->done = 1;
-    return true;
-  }
-  return false;
-}
-
-// Decision of one open search from the sums of the pass just scored.  Returns true when the search
-// goes on to another pass (its candidates are then already set).
-__device__ __forceinline__ bool decide_one(SearchCtl* c, const double* __restrict__ sums, double sag,
-                                           const DecideArgs& a, int* __restrict__ n_active,
-                                           int* __restrict__ status) {
-  if (a.mode == 1) {
-    double t = c->t_base;
-    const double lin = sums[0], quad = a.quad_coef * sums[1];
-    bool ok = false;
-    for (int trial = 0; trial < a.max_trials && !ok; ++trial) {
-      const double delta = -lin / t + quad / (t * t) - a.own_nu * sag / t + 0.5 * a.own_nu * c->gg / (t * t);
-      ok = accept(c, delta, t, trial);
-      t *= a.growth;
+// Decision of one open search from the sums of the sweep just scored, by the 32 lanes of a warp (sums, sag the same in
+// all): lane j tries the j-th trial, t = t_base * growth^j, and the first lane whose trial meets the condition
+// f(x+) - f(x) <= -||g||^2 / (2t) has its trial accepted.  The fp64 divisions of a trial are a chain of several hundred
+// clocks; one after the other they were most of a small search.  Returns true when the search goes on to another sweep
+// (its candidates are then already set).
+__device__ __forceinline__ bool decide_one(SearchCtl* c, const double* sums, double sag, const DecideArgs& a, int* n_active,
+                                           int* status) {
+  const int lane = threadIdx.x & 31;
+  const double gg = c->gg, t_base = c->t_base;
+  const int first = a.mode == 1 ? 0 : c->pass * a.cand;
+  const int tries = min(a.mode == 1 ? a.max_trials : a.cand, a.max_trials - first);
+  const double lin = a.mode == 1 ? sums[0] : 0.0, quad = a.mode == 1 ? a.quad_coef * sums[1] : 0.0;
+  double t = t_base;
+  for (int j = 0; j < (lane < tries ? lane : 0); ++j) t *= a.growth;
+  int found = -1;
+  double delta = 0.0, need = 1.0;
+  bool finite = true;
+  for (int base = 0; base < tries && found < 0; base += 32) {
+    const int j = base + lane;
+    bool pass = false;
+    if (j < tries) {
+      const double own = 0.5 * a.own_nu * gg / (t * t) - a.own_nu * sag / t;
+      if (a.mode == 1) delta = -lin / t + quad / (t * t) + own;
+      else {
+        const double sum = sums[j & (kCand - 1)];
+        finite = sum == sum;
+        delta = a.scale * sum + own;
+      }
+      need = gg / (2.0 * t);
+      pass = delta <= -need;         // false for NaN
     }
-    if (!ok) { c->done = 1; c->trial = -2; c->inv_step = 0.f; if (!(lin == lin && quad == quad)) atomicOr(status, 1); }
-    if (n_active) atomicSub(n_active, 1);
-    return false;
+    const unsigned hits = __ballot_sync(0xffffffffu, pass);
+    if (hits != 0u) found = base + __ffs((int)hits) - 1;
+    else if (base + 32 < tries)
+      for (int k = 0; k < 32; ++k) t *= a.growth;
   }
-  double t = c->t_base;
-  bool ok = false, finite = true;
-  for (int j = 0; j < a.cand && !ok; ++j) {
-    const int trial = c->pass * a.cand + j;
-    if (trial >= a.max_trials) break;
-    const double sum = sums[j];
-    finite = finite && (sum == sum);
-    const double delta = a.scale * sum - a.own_nu * sag / t + 0.5 * a.own_nu * c->gg / (t * t);
-    ok = accept(c, delta, t, trial);
-    t *= a.growth;
+  if (a.mode == 1) finite = lin == lin && quad == quad;
+  // trials behind the accepted one are not looked at: their sums may be anything
+  const unsigned bad = __ballot_sync(0xffffffffu, !finite);
+  const bool nonfinite = a.mode == 1 ? (bad != 0u && found < 0) : (bad & (found < 0 ? 0xffffffffu : (2u << (found & 31)) - 1u)) != 0u;
+  bool goes_on = false;
+  if (found >= 0) {
+    if (lane == (found & 31)) {
+      c->t_prev = t;
+      c->q = -delta / need;
+      c->inv_step = (float)(1.0 / t);
+      c->trial = first + found;
+      c->done = 1;
+    }
+  } else {
+    goes_on = a.mode == 0 && first + a.cand < a.max_trials;
+    double next = t_base;
+    if (goes_on)
+      for (int j = 0; j < a.cand; ++j) next *= a.growth;
+    if (lane == 0) {
+      if (a.mode == 0) c->pass += 1;
+      if (goes_on) { c->t_base = next; set_candidates(c, a.growth); }
+      else { c->done = 1; c->trial = -2; c->inv_step = 0.f; }
+    }
   }
-  if (!finite) atomicOr(status, 1);
-  if (ok) { if (n_active) atomicSub(n_active, 1); return false; }
-  c->pass += 1;
-  if (c->pass * a.cand >= a.max_trials) {
-    c->done = 1; c->trial = -2; c->inv_step = 0.f;
-    if (n_active) atomicSub(n_active, 1);
-    return false;
+  if (lane == 0) {
+    if (nonfinite) atomicOr(status, 1);
+    if (!goes_on && n_active) atomicSub(n_active, 1);
   }
-  c->t_base = t;
-  set_candidates(c, a.growth);
-  return true;
+  __syncwarp();
+  return goes_on;
 }
 
 // The decision log is a ring of `ring` passes; the slot in use is *pass mod ring, with the pass counter
@@ -817,69 +867,66 @@ __device__ __forceinline__ void log_decision(const DecisionLog& lg, int i, const
 
 // Weight gradient from its split partial sums, and the start of the W_l search, in one launch:
 //   grad[e] = sum over splits of part[s][e] (fp64, in split order), its transpose, ||grad||^2, ||W||^2.
-// A block owns 32 columns of 8 / SG rows; with many splits SG = 8 threads share an element, each adding its own run of
-// consecutive splits.  The last block to finish adds the blocks' sums of squares in block order and starts the search.
+// A block owns 256 / SG elements; with many splits SG = 8 threads share an element, each adding its own run of consecutive
+// splits.  The last block to finish adds the blocks' sums of squares up in block order and starts the search.
 // W = NULL: only the sum over the splits.
 template <int SG>
 __global__ void __launch_bounds__(256)
 k_finish_grad(const float* __restrict__ part, int splits, int rows, int cols, int ldp, float* __restrict__ grad,
               float* __restrict__ grad_t, int ldt, const float* __restrict__ W, double* partial, unsigned* ticket,
               SearchCtl* ctl, double shrink, double growth, int* status) {
-  constexpr int ROWS = 8 / SG;
-  __shared__ double sh[32], s_part[SG][ROWS][32];
+  constexpr int ELEMS = 256 / SG;
+  __shared__ double sh[16], s_part[SG][ELEMS];
   __shared__ int s_last;
-  const int x = threadIdx.x & 31, y = (threadIdx.x >> 5) % ROWS, sg = (threadIdx.x >> 5) / ROWS;
-  const int col_blocks = (ldp + 31) / 32;
-  const int c = (int)(blockIdx.x % col_blocks) * 32 + x;
-  const int r = (int)(blockIdx.x / col_blocks) * ROWS + y;
-  const bool in = r < rows && c < ldp;
-  const long long elems = (long long)rows * ldp, e = (long long)r * ldp + c;
+  const int x = threadIdx.x % ELEMS, sg = threadIdx.x / ELEMS;
+  const long long elems = (long long)rows * ldp, e = (long long)blockIdx.x * ELEMS + x;
+  const bool in = e < elems;
   double s = 0.0;
+  float w = 0.f;
   if (in) {
+    if (W != nullptr && sg == 0) w = W[e];
     const int k1 = (int)((long long)splits * (sg + 1) / SG);
 #pragma unroll 8
     for (int k = (int)((long long)splits * sg / SG); k < k1; ++k) s += (double)part[k * elems + e];
   }
   if (SG > 1) {
-    s_part[sg][y][x] = s;
+    s_part[sg][x] = s;
     __syncthreads();
     if (sg == 0)
 #pragma unroll
-      for (int k = 1; k < SG; ++k) s += s_part[k][y][x];
+      for (int k = 1; k < SG; ++k) s += s_part[k][x];
   }
-  double gg = 0.0, ww = 0.0;
+  double sq[2] = {0.0, 0.0};   // of grad, of W
   if (in && sg == 0) {
     const float g = (float)s;
     grad[e] = g;
     if (W != nullptr) {
+      const int r = (int)(e / ldp), c = (int)(e - (long long)r * ldp);
       if (c < cols) grad_t[(long long)c * ldt + r] = g;
-      const double w = W[e];
-      gg = (double)g * (double)g;
-      ww = w * w;
+      sq[0] = (double)g * (double)g;
+      sq[1] = (double)w * (double)w;
     }
   }
   if (W == nullptr) return;
-  gg = block_sum(gg, sh);
-  ww = block_sum(ww, sh);
+  block_sums(sq, sh);
   if (threadIdx.x == 0) {
-    partial[2 * (size_t)blockIdx.x] = gg;
-    partial[2 * (size_t)blockIdx.x + 1] = ww;
+    partial[2 * (size_t)blockIdx.x] = sq[0];
+    partial[2 * (size_t)blockIdx.x + 1] = sq[1];
     __threadfence();
     s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
   }
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  gg = ww = 0.0;
+  sq[0] = sq[1] = 0.0;
   for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x) {
-    gg += __ldcg(partial + 2 * (size_t)b);
-    ww += __ldcg(partial + 2 * (size_t)b + 1);
+    sq[0] += __ldcg(partial + 2 * (size_t)b);
+    sq[1] += __ldcg(partial + 2 * (size_t)b + 1);
   }
-  gg = block_sum(gg, sh);
-  ww = block_sum(ww, sh);
+  block_sums(sq, sh);
   if (threadIdx.x == 0) {
     *ticket = 0;
-    begin_one(ctl, gg, ww, shrink, growth, nullptr, status);
+    begin_one(ctl, sq[0], sq[1], shrink, growth, nullptr, status);
   }
 }
 
@@ -909,7 +956,7 @@ template <bool OUT>
 __global__ void __launch_bounds__(256, 4)
 k_search_w(const SearchW p) {
   constexpr int PER = OUT ? 2 : kCand;
-  __shared__ double sh[32], total[kCand];
+  __shared__ double sh[PER * 8], total[PER];
   SearchCtl* const ctl = p.ctl;
   const long long first = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
   if (ctl->done) {                  // skipped: the same in every block
@@ -950,19 +997,13 @@ k_search_w(const SearchW p) {
           for (int j = 0; j < kCand; ++j) s[j % PER] += (double)part[j];
         }
       }
+      block_sums(s, sh);
+      if (threadIdx.x == 0)
 #pragma unroll
-      for (int j = 0; j < PER; ++j) {
-        const double v = block_sum(s[j], sh);
-        if (threadIdx.x == 0) p.partial[(size_t)blockIdx.x * PER + j] = v;
-      }
+        for (int j = 0; j < PER; ++j) p.partial[(size_t)blockIdx.x * PER + j] = s[j];
       const bool ok = grid_meet(p.bar, p.err, [&] {
-        for (int j = 0; j < PER; ++j) {
-          double t = 0.0;
-          for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x) t += __ldcg(p.partial + (size_t)b * PER + j);
-          t = block_sum(t, sh);
-          if (threadIdx.x == 0) total[j] = t;
-        }
-        if (threadIdx.x == 0 && !decide_one(ctl, total, 0.0, p.a, nullptr, p.status)) log_decision(p.log, 0, ctl);
+        add_block_sums<PER>(p.partial, (int)gridDim.x, total);
+        if (threadIdx.x < 32 && !decide_one(ctl, total, 0.0, p.a, nullptr, p.status) && threadIdx.x == 0) log_decision(p.log, 0, ctl);
       });
       if (!ok) return;
       open = __ldcg(&ctl->done) == 0;
@@ -1009,10 +1050,10 @@ __global__ void __launch_bounds__(256)
 k_zgrad_finish(float4* __restrict__ G, const float4* __restrict__ Z, const float4* __restrict__ H, int ld4,
                const int4* __restrict__ blocks, float nu, double* partial, const int* __restrict__ block_ptr, unsigned* tickets,
                SearchCtl* ctl, double* __restrict__ sums, double shrink, double growth, int* n_active, int* status) {
-  __shared__ double sh[32];
+  __shared__ double sh[24];
   __shared__ int s_last;
   const int4 rb = blocks[blockIdx.x];
-  double sgg = 0.0, szz = 0.0, sag = 0.0;
+  double t[3] = {0.0, 0.0, 0.0};
   const long long e0 = (long long)rb.x * ld4, e1 = (long long)rb.y * ld4;
   for (long long e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
     const float4 z = Z[e], h = H[e];
@@ -1020,29 +1061,32 @@ k_zgrad_finish(float4* __restrict__ G, const float4* __restrict__ Z, const float
     const float ax = z.x - relu(h.x), ay = z.y - relu(h.y), az = z.z - relu(h.z), aw = z.w - relu(h.w);
     g.x = fmaf(nu, ax, g.x); g.y = fmaf(nu, ay, g.y); g.z = fmaf(nu, az, g.z); g.w = fmaf(nu, aw, g.w);
     G[e] = g;
-    sgg += (double)(g.x * g.x + g.y * g.y + g.z * g.z + g.w * g.w);
-    szz += (double)(z.x * z.x + z.y * z.y + z.z * z.z + z.w * z.w);
-    sag += (double)(ax * g.x + ay * g.y + az * g.z + aw * g.w);
+    t[0] += (double)(g.x * g.x + g.y * g.y + g.z * g.z + g.w * g.w);
+    t[1] += (double)(z.x * z.x + z.y * z.y + z.z * z.z + z.w * z.w);
+    t[2] += (double)(ax * g.x + ay * g.y + az * g.z + aw * g.w);
   }
-  sgg = block_sum(sgg, sh); szz = block_sum(szz, sh); sag = block_sum(sag, sh);
+  block_sums(t, sh);
   const int m = rb.z, b0 = block_ptr[m], b1 = block_ptr[m + 1];
   if (threadIdx.x == 0) {
-    partial[(size_t)blockIdx.x * 3] = sgg; partial[(size_t)blockIdx.x * 3 + 1] = szz; partial[(size_t)blockIdx.x * 3 + 2] = sag;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) partial[(size_t)blockIdx.x * 3 + j] = t[j];
     __threadfence();
     s_last = atomicAdd(tickets + m, 1u) == (unsigned)(b1 - b0) - 1u;
   }
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  sgg = szz = sag = 0.0;
-  for (int b = b0 + threadIdx.x; b < b1; b += blockDim.x) {
-    sgg += __ldcg(partial + (size_t)b * 3); szz += __ldcg(partial + (size_t)b * 3 + 1); sag += __ldcg(partial + (size_t)b * 3 + 2);
-  }
-  sgg = block_sum(sgg, sh); szz = block_sum(szz, sh); sag = block_sum(sag, sh);
+#pragma unroll
+  for (int j = 0; j < 3; ++j) t[j] = 0.0;
+  for (int b = b0 + threadIdx.x; b < b1; b += blockDim.x)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) t[j] += __ldcg(partial + (size_t)b * 3 + j);
+  block_sums(t, sh);
   if (threadIdx.x == 0) {
     tickets[m] = 0;
-    sums[m * 3] = sgg; sums[m * 3 + 1] = szz; sums[m * 3 + 2] = sag;
-    begin_one(ctl + m, sgg, szz, shrink, growth, n_active, status);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) sums[m * 3 + j] = t[j];
+    begin_one(ctl + m, t[0], t[1], shrink, growth, n_active, status);
   }
 }
 
@@ -1225,7 +1269,7 @@ __device__ __forceinline__ bool close_sweep(const SearchZ& p, int n_chunks, cons
     }
 #pragma unroll
     for (int j = 0; j < PER; ++j) s[j] = warp_sum(s[j]);
-    if (lane == 0) decide_one(c, s, p.own[i * 3 + 2], p.a, p.n_active, p.status);
+    decide_one(c, s, p.own[i * 3 + 2], p.a, p.n_active, p.status);
   }
   return grid_meet(p.bar, p.err, nothing);
 }
@@ -1687,6 +1731,10 @@ k_output(const OutputArgs p) {
     }
     return;
   }
+  constexpr int kTable = 128;          // iterations whose momentum is kept in shared memory
+  __shared__ float s_mom[kTable];
+  for (int k = threadIdx.x; k < min(p.iters, kTable); k += blockDim.x) s_mom[k] = p.momentum[k];
+  __syncthreads();
   const int lane = threadIdx.x & (LPR - 1);
   const int slot = (int)((blockIdx.x * blockDim.x + threadIdx.x) / LPR);
   const bool here = slot < p.n_train;   // lanes without a row keep step with the shuffles of the others
@@ -1729,7 +1777,7 @@ k_output(const OutputArgs p) {
 #pragma unroll
     for (int o = LPR / 2; o > 0; o >>= 1) se += __shfl_xor_sync(0xffffffffu, se, o);
     const float inv_se = 1.f / se;
-    const float mom = p.momentum[it];
+    const float mom = it < kTable ? s_mom[it] : p.momentum[it];
 #pragma unroll
     for (int t = 0; t < CPL; ++t) {
       const float pr = ex[t] * inv_se - (lane + LPR * t == yi ? 1.f : 0.f);
