@@ -43,7 +43,6 @@ constexpr int kZBlockRows = 32;      // rows per block of the hidden-layer gradi
 constexpr int kChunkGroups = 512;    // groups the sums of a scoring sweep's chunks are first added up in, when there are more chunks
 constexpr int kCandZ = 4;           // theta candidates scored per sweep (2..4; steady-state searches close at trial 0..2)
 constexpr size_t kDirectBytes = (size_t)256 << 10;   // matrices up to this size cross the bus inside the permuting kernel (one copy and its latency less)
-constexpr int kMaxCommNarrow = 384;            // communities whose sums k_score_z_out_part<16> holds in shared memory (96 KB)
 constexpr int kDefaultLongRow = 256;   // stored entries one warp walks before a row is cut into items
 
 thread_local std::string g_create_error;
@@ -226,8 +225,12 @@ struct gcn_admm {
   // Z scoring: units in chunks of about equally many stored entries, dealt to the warps of the grid in a fixed order
   int* d_chunk_ptr = nullptr;
   int* d_row_order = nullptr;               // rows per community by falling length: the order of the kernels that put several rows in a warp
-  int* d_chunk_ptr_sorted = nullptr;        // chunk table of the units in that order
-  int n_chunks_sorted = 0;
+  // closed-form search of the last hidden layer (gcn_admm_host::SegmentTables)
+  gk::SegRef* d_segs = nullptr;
+  gk::SegChunk* d_seg_chunks = nullptr;
+  int *d_slot_ptr = nullptr, *comm_done = nullptr, *split_done = nullptr;
+  double* slots = nullptr;
+  int n_seg_chunks = 0;
   int n_chunks = 0;
   double* z_chunk_part = nullptr;           // [chunk][M][candidates] sums of one sweep, per chunk of units
   double* z_group_part = nullptr;           // [group of chunks][M][candidates], chunks added in order
@@ -640,88 +643,84 @@ struct gcn_admm {
           p.bt_shrink, p.bt_growth, n_active, status);
       CU(cudaGetLastError());
     }
+    const int ld4 = ldn / 4, warps = 8;
+    const double move_bytes = 12.0 * (double)n * ldl;
+    char zname[48];
+    float4* const scratch = reinterpret_cast<float4*>(item_sums);
+    gk::DecideArgs decide{};
+    decide.growth = p.bt_growth;
+    decide.max_trials = p.bt_max_trials;
+    decide.own_nu = p.nu;
+    if (l + 1 == L) {   // closed form
+      gemm_nn(B2, ldl, W[L], ldn, Wt[L], ldl, B0, ldn, n, C[L], C[l]);   // T = G W_L; S stays in B1, R' is not needed any more
+      decide.mode = 1;
+      decide.quad_coef = 0.5 * p.rho;
+      gk::SearchOut a{};
+      a.segs = d_segs; a.chunks = d_seg_chunks; a.n_chunks = n_seg_chunks; a.chunk_counter = chunk_counter;
+      a.slot_ptr = d_slot_ptr; a.slots = slots; a.comm_done = comm_done; a.split_done = split_done; a.items = d_items; a.split = d_split;
+      a.ctl = ctl; a.own = sums_z; a.n_active = n_active; a.status = status; a.a = decide;
+      // one wave of chunks: the longest segment is the critical path, so long ones get a whole warp
+      a.share_from = ld4 <= 4 ? 24 : n_seg_chunks <= 2 * kSmCount * 24 ? 64 : INT_MAX;
+      std::snprintf(zname, sizeof zname, "search_z_out@%d", ldn);
+      {
+        Scope sc(this, zname, 1, 4.0 * gi.nnz + 12.0 * n + 8.0 * (double)n * ldn, 2.0 * (double)gi.nnz * ldn);
+#define SEARCH_OUT(CL)                                                                                                      \
+  {                                                                                                                         \
+    const auto kernel = gk::k_search_z_out<CL>;                                                                             \
+    const int grid = (int)std::min<long long>(cdiv(n_seg_chunks, warps), resident_blocks((const void*)kernel, warps * 32, 0)); \
+    kernel<<<grid, warps * 32, 0, stream>>>(d_col, d_dinv, (const float4*)B0, (const float4*)B1, ld4, scratch, a);          \
+  }
+        if (ld4 <= 1) SEARCH_OUT(1)
+        else if (ld4 <= 2) SEARCH_OUT(2)
+        else if (ld4 <= 4) SEARCH_OUT(4)
+        else if (ld4 <= 8) SEARCH_OUT(8)
+        else if (ld4 <= 16) SEARCH_OUT(16)
+        else SEARCH_OUT(32)
+#undef SEARCH_OUT
+        CU(cudaGetLastError());
+      }
+      Scope sc(this, "move_z", 1, move_bytes, 0.0);
+      gk::k_move_z<<<grid_for(n * (ldl / 4)), 256, 0, stream>>>((float4*)Z[l], (const float4*)B2, ldl / 4, n, d_row_comm, ctl, M, log_z(l),
+                                                                chunk_counter);
+      CU(cudaGetLastError());
+      return;
+    }
     gemm_nn(B2, ldl, W[l + 1], ldn, Wt[l + 1], ldl, B1, ldn, n, C[l + 1], C[l]);         // T = G W_{l+1}
-
-    const bool out = (l + 1 == L);
-    const int per = out ? 2 : kCandZ, ld4 = ldn / 4, warps = 8;
+    decide.cand = kCandZ;
+    decide.scale = 0.5 * p.nu;
     gk::SearchZ a{};
     a.ctl = ctl; a.n_comm = M;
     a.chunk_part = z_chunk_part; a.chunk_counter = chunk_counter; a.group_part = z_group_part;
+    // few chunks: a warp per community adds them up directly; many: group by group first (one more meeting of the grid)
+    a.per_group = (int)cdiv(n_chunks, kChunkGroups);
+    a.n_groups = n_chunks > kChunkGroups ? (int)cdiv(n_chunks, a.per_group) : 0;
     a.split = d_split; a.n_split = n_split; a.split_scores = split_scores; a.split_order = d_split_order; a.split_ptr = d_split_ptr;
     a.own = sums_z; a.n_active = n_active; a.status = status; a.err = tc_error; a.bar = grid_bar;
-    a.a.growth = p.bt_growth;
-    a.a.max_trials = p.bt_max_trials;
-    a.a.cand = kCandZ;
-    a.a.own_nu = p.nu;
-    a.a.mode = out ? 1 : 0;
-    a.a.scale = 0.5 * p.nu;
-    a.a.quad_coef = 0.5 * p.rho;
+    a.a = decide;
     a.log = log_z(l);
     a.Z = (float4*)Z[l]; a.G = (const float4*)B2; a.ldz4 = ldl / 4; a.row_comm = d_row_comm;
-    // few chunks: a warp per community adds them up directly; many: group by group first (one more meeting of the grid)
-    auto with_groups = [&](int chunks) {
-      gk::SearchZ b = a;
-      b.per_group = (int)cdiv(chunks, kChunkGroups);
-      b.n_groups = chunks > kChunkGroups ? (int)cdiv(chunks, b.per_group) : 0;
-      return b;
-    };
-    char zname[48];
-    std::snprintf(zname, sizeof zname, out ? "score_z_out@%d" : "score_z_hidden@%d", ldn);
-    const double score_bytes = 6.0 * gi.nnz + 8.0 * n + 4.0 * (double)n * ldn * (out ? 2 : 3), score_flops = 2.0 * (double)gi.nnz * ldn;
-    const double move_bytes = 12.0 * (double)n * ldl;
-    const float4 *T = (const float4*)B1, *Hn = (const float4*)H[l + 1], *Zn = (const float4*)Z[l + 1], *R4 = (const float4*)Rn;
-    float4* const scratch = reinterpret_cast<float4*>(item_sums);
-    // closing, further sweeps and the move: as many blocks as the move can use
-    const long long move_blocks = cdiv(n * (ldl / 4), 256);
-#define SCORE_PART(G)                                                                                                       \
-  if (ld4 <= (G) && (size_t)(32 / (G)) * warps * M * 2 * sizeof(double) <= 96 * 1024) {                                     \
-    const size_t smem = (size_t)(32 / (G)) * warps * M * 2 * sizeof(double);                                                \
-    const auto kernel = gk::k_score_z_out_part<(G), 4>;                                                                     \
-    const int grid = (int)std::min<long long>(cdiv(n_chunks_sorted, warps), resident_blocks((const void*)kernel, warps * 32, smem)); \
-    {                                                                                                                       \
-      Scope sc(this, zname, 1, score_bytes, score_flops);                                                                   \
-      kernel<<<grid, warps * 32, smem, stream>>>(d_row_ptr, d_col, d_col_comm, d_dinv, T, R4, ld4, ctl, M, z_chunk_part, n_active, \
-                                                 d_chunk_ptr_sorted, n_chunks_sorted, chunk_counter, d_items, n_items, long_len, \
-                                                 scratch, d_row_order);                                                     \
-      CU(cudaGetLastError());                                                                                               \
-    }                                                                                                                       \
-    Scope sc(this, "close_z", 1, move_bytes, 0.0);                                                                          \
-    launch_together(gk::k_close_z<1, true, 4, kCandZ>, move_blocks, warps * 32, 0, d_row_ptr, d_col, d_col_comm, d_dinv, T, Hn, Zn, R4, \
-                    ld4, (int)n, 0, d_chunk_ptr_sorted, n_chunks_sorted, d_items, n_items, long_len, scratch,               \
-                    with_groups(n_chunks_sorted));                                                                          \
-    return;                                                                                                                 \
-  }
-    if (out) {   // narrow output layer: several rows per warp
-      SCORE_PART(4)
-      SCORE_PART(8)
-      SCORE_PART(16)
-    }
-#undef SCORE_PART
-    const size_t sums = (size_t)warps * M * per * sizeof(double);
+    std::snprintf(zname, sizeof zname, "score_z_hidden@%d", ldn);
+    const float4 *T = (const float4*)B1, *Hn = (const float4*)H[l + 1], *Zn = (const float4*)Z[l + 1];
+    const size_t sums = (size_t)warps * M * kCandZ * sizeof(double);
     const int use_smem = sums <= 96 * 1024;
     auto score = [&](auto kernel, auto close, int V) {
       const size_t smem = (size_t)warps * 2 * V * 32 * sizeof(float4) + (use_smem ? sums + (size_t)M * sizeof(float4) : 0);
       const int grid = (int)std::min<long long>(cdiv(n_chunks, warps), resident_blocks((const void*)kernel, warps * 32, smem));
       {
-        Scope sc(this, zname, 1, score_bytes, score_flops);
-        kernel<<<grid, warps * 32, smem, stream>>>(d_row_ptr, d_col, d_col_comm, d_dinv, T, Hn, Zn, R4, ld4, ctl, M, z_chunk_part, n_active,
+        Scope sc(this, zname, 1, 6.0 * gi.nnz + 8.0 * n + 12.0 * (double)n * ldn, 2.0 * (double)gi.nnz * ldn);
+        kernel<<<grid, warps * 32, smem, stream>>>(d_row_ptr, d_col, d_col_comm, d_dinv, T, Hn, Zn, ld4, ctl, M, z_chunk_part, n_active,
                                                    use_smem, d_chunk_ptr, n_chunks, chunk_counter, d_items, n_items, long_len, scratch);
         CU(cudaGetLastError());
       }
+      // closing, further sweeps and the move: as many blocks as the move can use
       Scope sc(this, "close_z", 1, move_bytes, 0.0);
-      launch_together(close, move_blocks, warps * 32, smem, d_row_ptr, d_col, d_col_comm, d_dinv, T, Hn, Zn, R4, ld4, (int)n,
-                      use_smem, d_chunk_ptr, n_chunks, d_items, n_items, long_len, scratch, with_groups(n_chunks));
+      launch_together(close, cdiv(n * (ldl / 4), 256), warps * 32, smem, d_row_ptr, d_col, d_col_comm, d_dinv, T, Hn, Zn, ld4, (int)n,
+                      use_smem, d_chunk_ptr, n_chunks, d_items, n_items, long_len, scratch, a);
     };
-#define SCORE_Z(V)                                                                                           \
-  {                                                                                                          \
-    if (out) score(gk::k_score_z<V, true, 4, kCandZ>, gk::k_close_z<V, true, 4, kCandZ>, V);                 \
-    else score(gk::k_score_z<V, false, 4, kCandZ>, gk::k_close_z<V, false, 4, kCandZ>, V);                   \
-  }
-    if (ld4 <= 32) SCORE_Z(1)
-    else if (ld4 <= 64) SCORE_Z(2)
-    else if (ld4 <= 128) SCORE_Z(4)
-    else SCORE_Z(8)
-#undef SCORE_Z
+    if (ld4 <= 32) score(gk::k_score_z<1, 4, kCandZ>, gk::k_close_z<1, 4, kCandZ>, 1);
+    else if (ld4 <= 64) score(gk::k_score_z<2, 4, kCandZ>, gk::k_close_z<2, 4, kCandZ>, 2);
+    else if (ld4 <= 128) score(gk::k_score_z<4, 4, kCandZ>, gk::k_close_z<4, 4, kCandZ>, 4);
+    else score(gk::k_score_z<8, 4, kCandZ>, gk::k_close_z<8, 4, kCandZ>, 8);
   }
 
   // ---- Z_L (Eq. 7) and, in the same sweep, the dual as printed in Eq. 3 -----------------
@@ -1069,41 +1068,46 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
   gcn_admm_host::Table<int> row_order;
   gcn_admm_host::order_rows_by_length(g, row_order);
   h->want_table(h->d_row_order, row_order);
-  // chunks of units (items first, then rows) holding about the same number of stored entries each: for rows in storage
-  // order (whole-warp scoring) and for rows by falling length (several rows per warp: output layers of at most 64 classes)
-  std::vector<int> chunks_plain, chunks_sorted;
-  {
+  // work lists of the two forms of the Z search: the closed form's segments by community (at least two layers), and chunks
+  // of units (items first, then rows) holding about the same number of stored entries each (at least three layers)
+  gcn_admm_host::SegmentTables seg;
+  std::vector<int> chunks;
+  const long long warps_guess = (long long)kSmCount * 3 * 8;
+  if (n_layers >= 2) {
+    // a chunk per warp and a few more; rows of the plain sums in chunks of about 8 KB
+    const long long target = std::max<long long>(32, std::min<long long>(1024, (long long)g.nnz / (warps_guess * 2)));
+    gcn_admm_host::build_segment_tables(g, h->long_len, lt, target, std::max(1, 2048 / h->ld[n_layers]), seg);
+    static_assert(sizeof(gcn_admm_host::SegRef) == sizeof(gk::SegRef) && sizeof(gcn_admm_host::SegChunk) == sizeof(gk::SegChunk),
+                  "tables are uploaded as they are");
+    h->n_seg_chunks = (int)seg.chunks.size();
+    h->want_table(h->d_segs, seg.segs);
+    h->want_table(h->d_seg_chunks, seg.chunks);
+    h->want_table(h->d_slot_ptr, seg.slot_ptr);
+    h->want(h->slots, 2 * (size_t)seg.slot_ptr.back());
+    h->want(h->comm_done, n_comm, gcn_admm::kZero);
+    h->want(h->split_done, lt.split.size(), gcn_admm::kZero);
+  }
+  if (n_layers >= 3) {
     const long long n_units = (long long)lt.items.size() + n;
-    const long long warps_guess = (long long)kSmCount * 3 * 8;
     // few enough chunks that their sums (M x candidates doubles each) stay small next to the entries they cover
     const long long target = std::max<long long>({64, std::min<long long>(1024, (long long)g.nnz / (warps_guess * 4)), 2LL * n_comm});
-    auto build_chunks = [&](const int* order) {
-      std::vector<int> cp;
-      cp.push_back(0);
-      long long in_chunk = 0;
-      for (long long u = 0; u < n_units; ++u) {
-        long long len;
-        if (u < (long long)lt.items.size()) len = lt.items[(size_t)u].z - lt.items[(size_t)u].y;
-        else {
-          const long long k = u - (long long)lt.items.size();
-          const long long r = order ? order[k] : k;
-          len = g.row_ptr[r + 1] - g.row_ptr[r];
-          if (len > h->long_len) len = 0;                 // walked as items
-        }
-        in_chunk += len + 2;                              // a unit costs a little even when it is short
-        if (in_chunk >= target) { cp.push_back((int)(u + 1)); in_chunk = 0; }
+    chunks.push_back(0);
+    long long in_chunk = 0;
+    for (long long u = 0; u < n_units; ++u) {
+      long long len;
+      if (u < (long long)lt.items.size()) len = lt.items[(size_t)u].z - lt.items[(size_t)u].y;
+      else {
+        const long long r = u - (long long)lt.items.size();
+        len = g.row_ptr[r + 1] - g.row_ptr[r];
+        if (len > h->long_len) len = 0;                 // walked as items
       }
-      if (cp.back() != (int)n_units) cp.push_back((int)n_units);
-      return cp;
-    };
-    const bool narrow_out = n_layers >= 2 && h->ld[n_layers] <= 64;
-    if (n_layers >= 3 || !narrow_out || n_comm > kMaxCommNarrow) chunks_plain = build_chunks(nullptr);
-    if (narrow_out) chunks_sorted = build_chunks(row_order.data());
-    h->n_chunks = std::max(0, (int)chunks_plain.size() - 1);
-    h->n_chunks_sorted = std::max(0, (int)chunks_sorted.size() - 1);
+      in_chunk += len + 2;                              // a unit costs a little even when it is short
+      if (in_chunk >= target) { chunks.push_back((int)(u + 1)); in_chunk = 0; }
+    }
+    if (chunks.back() != (int)n_units) chunks.push_back((int)n_units);
   }
-  h->want_table(h->d_chunk_ptr, chunks_plain);
-  h->want_table(h->d_chunk_ptr_sorted, chunks_sorted);
+  h->n_chunks = std::max(0, (int)chunks.size() - 1);
+  h->want_table(h->d_chunk_ptr, chunks);
 
   const int L = n_layers;
   const size_t rows = (size_t)n;
@@ -1160,7 +1164,7 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
   h->n_zblocks = (int)zb.size();
   h->want_table(h->d_zblocks, zb);
   h->want_table(h->d_comm_block_ptr, cbp);
-  h->want(h->z_chunk_part, (size_t)std::max(h->n_chunks, h->n_chunks_sorted) * n_comm * gk::kCand);
+  h->want(h->z_chunk_part, (size_t)h->n_chunks * n_comm * gk::kCand);
   h->want(h->z_group_part, (size_t)kChunkGroups * n_comm * gk::kCand);
   h->want(h->chunk_counter, 1, gcn_admm::kZero);
   h->want(h->ticket, 1, gcn_admm::kZero);

@@ -339,6 +339,101 @@ inline void order_rows_by_length(const GraphIndex& g, Table<int>& order) {
   }
 }
 
+// ------------------------------------------------------------------------------------------
+// The segments of all rows by the community of their columns, for the closed-form search of the last hidden layer, which
+// needs the sum of ||K_m[i]||^2 over the segments (i, m) of a community and nothing else of the row.  Inside a community
+// segments go by falling length, so that a chunk of them is walked without divergence; segments longer than `limit` are left
+// to the pieces of build_long_row_tables.
+//   segs[k]   = {first entry, dinv of its row}
+//   chunks[c] = {first, count, length, community, slot}: length > 0: segments first .. first + count - 1 of that length; 0: rows
+//               first .. first + count - 1 of the community; -1: item `first` (a piece of split segment `count`)
+// Pieces first, then community after community (what the warps gather at a time is then the rows of one or two communities),
+// then the rows.  Every chunk has a slot of its own, except that the pieces of a split segment share one;
+// slot_ptr[m] .. slot_ptr[m+1] - 1 are those of community m.
+// ------------------------------------------------------------------------------------------
+struct SegRef { int begin; float dinv; };
+struct SegChunk { int first, count, length, comm, slot; };
+struct SegmentTables {
+  Table<SegRef> segs;
+  std::vector<SegChunk> chunks;
+  std::vector<int> slot_ptr;
+};
+
+inline void build_segment_tables(const GraphIndex& g, int limit, const LongRowTables& lt, long long target, long long rows_per_chunk,
+                                 SegmentTables& t) {
+  const int M = g.n_comm;
+  int longest = 1;
+#pragma omp parallel for schedule(static) reduction(max : longest)
+  for (long long i = 0; i < g.n; ++i)
+    for (int s = g.seg_row_ptr[i]; s < g.seg_row_ptr[i + 1]; ++s) {
+      const int len = g.seg_begin[s + 1] - g.seg_begin[s];
+      if (len <= limit) longest = std::max(longest, len);
+    }
+  const long long bins = (long long)M * longest;   // bin (m, longest - len): community-major, falling length
+  int slices = 1;
+#ifdef _OPENMP
+  slices = (int)std::max<long long>(1, std::min<long long>({(long long)omp_get_max_threads(), (long long)(16 << 20) / bins, g.n / 512}));
+#endif
+  std::vector<long long> hist((std::size_t)(slices * bins), 0);
+  const auto bin_of = [&](int s, int len) { return (long long)g.seg_comm[s] * longest + (longest - len); };
+#pragma omp parallel for schedule(static, 1)
+  for (int k = 0; k < slices; ++k) {
+    long long* const mine = hist.data() + (std::size_t)k * bins;
+    for (long long i = g.n * k / slices; i < g.n * (k + 1) / slices; ++i)
+      for (int s = g.seg_row_ptr[i]; s < g.seg_row_ptr[i + 1]; ++s) {
+        const int len = g.seg_begin[s + 1] - g.seg_begin[s];
+        if (len <= limit) ++mine[bin_of(s, len)];
+      }
+  }
+  std::vector<long long> bin_ptr((std::size_t)bins + 1, 0);
+  long long at = 0;
+  for (long long b = 0; b < bins; ++b) {
+    bin_ptr[(std::size_t)b] = at;
+    for (int k = 0; k < slices; ++k) {
+      const long long here = hist[(std::size_t)(k * bins + b)];
+      hist[(std::size_t)(k * bins + b)] = at;
+      at += here;
+    }
+  }
+  bin_ptr[(std::size_t)bins] = at;
+  t.segs.resize((std::size_t)at);
+#pragma omp parallel for schedule(static, 1)
+  for (int k = 0; k < slices; ++k) {
+    long long* const mine = hist.data() + (std::size_t)k * bins;
+    for (long long i = g.n * k / slices; i < g.n * (k + 1) / slices; ++i)
+      for (int s = g.seg_row_ptr[i]; s < g.seg_row_ptr[i + 1]; ++s) {
+        const int len = g.seg_begin[s + 1] - g.seg_begin[s];
+        if (len <= limit) t.segs[(std::size_t)mine[bin_of(s, len)]++] = SegRef{g.seg_begin[s], g.dinv[(std::size_t)i]};
+      }
+  }
+  t.chunks.clear();
+  t.slot_ptr.assign((std::size_t)M + 1, 0);
+  std::vector<SegChunk> rows;
+  std::vector<int> split_slot(lt.split.size());
+  std::vector<std::vector<int>> split_of((std::size_t)M);
+  for (std::size_t k = 0; k < lt.split.size(); ++k) split_of[(std::size_t)lt.split[k].y].push_back((int)k);
+  int slot = 0;
+  for (int m = 0; m < M; ++m) {
+    t.slot_ptr[(std::size_t)m] = slot;
+    for (int k : split_of[(std::size_t)m]) split_slot[(std::size_t)k] = slot++;
+    for (long long b = (long long)m * longest; b < (long long)(m + 1) * longest; ++b) {
+      const int len = longest - (int)(b % longest);
+      const long long step = std::max<long long>(1, target / (len + 1));
+      for (long long f = bin_ptr[(std::size_t)b]; f < bin_ptr[(std::size_t)b + 1]; f += step)
+        t.chunks.push_back(SegChunk{(int)f, (int)std::min(step, bin_ptr[(std::size_t)b + 1] - f), len, m, slot++});
+    }
+    for (int r = g.comm_ptr[m]; r < g.comm_ptr[m + 1]; r += (int)rows_per_chunk)
+      rows.push_back(SegChunk{r, (int)std::min<long long>(rows_per_chunk, g.comm_ptr[m + 1] - r), 0, m, slot++});
+  }
+  t.slot_ptr[(std::size_t)M] = slot;
+  t.chunks.insert(t.chunks.end(), rows.begin(), rows.end());
+  std::vector<SegChunk> pieces;
+  for (std::size_t k = 0; k < lt.split.size(); ++k)
+    for (int q = 0; q < lt.split[k].w; ++q)
+      pieces.push_back(SegChunk{lt.split[k].z + q, (int)k, -1, lt.split[k].y, split_slot[k]});
+  t.chunks.insert(t.chunks.begin(), pieces.begin(), pieces.end());
+}
+
 // First-order neighbour rows of community m: new ids outside V_m adjacent to V_m, ascending.
 inline std::vector<int> halo1_of(const GraphIndex& g, int m) {
   std::vector<int> out;

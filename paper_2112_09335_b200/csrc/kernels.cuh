@@ -1119,11 +1119,11 @@ __device__ __forceinline__ float warp_sum2(float v0, float v1, int lane) {
 // which is non-zero on V_m and its first-order neighbour rows only.  A warp owns row i and walks
 // its stored entries once; col_comm gives the community of every entry, entries of one community
 // are contiguous (ascending columns), and at every change of community the finished K_m[i] is scored:
-//   OUT = false (layer l+1 < L, ReLU):  per community, sum_c (z - f(h - k/t_j))^2 - (z - f(h))^2 for j < NC
+//   per community, sum_c (z - f(h - k/t_j))^2 - (z - f(h))^2 for j < NC
 //                                        (NC = candidates scored per sweep, 2..4: a candidate costs two
 //                                        instructions per element, and a search that needs more trials
 //                                        than one sweep scores is served by a further sweep)
-//   OUT = true  (layer l+1 = L):        sums <k, R'> and ||k||^2 per community   (closed form)
+// (Layer l+1 = L is linear and has a search of its own, k_search_z_out.)
 // Sums are kept per warp in shared memory (no atomics on the hot path) and leave the kernel per chunk of
 // units (see the scheduling note in the kernel).  V = float4 columns per lane (width <= 128 V).
 // Persistent grid.
@@ -1139,24 +1139,14 @@ __device__ __forceinline__ float4 twice_error(const float4& h, const float4& z) 
 }
 
 // Scores one finished K_m[i] (k, still without the factor di) against the row's a, b:
-// OUT: a = R'; else a = h and b = twice_error(h, z).  The sums (2 when OUT, else NC) go to `slots`:
+// a = h and b = twice_error(h, z).  The NC sums go to `slots`:
 // add: added to what is there (the slots belong to this warp), else stored.
 __device__ __forceinline__ void put_sum(double* dst, float r, bool add) { *dst = add ? *dst + (double)r : (double)r; }
-template <int V, bool OUT, int NC>
+template <int V, int NC>
 __device__ __forceinline__ void score_segment(const float4 (&k)[V], float di, const float4 (&a)[V],
                                               const float4 (&b)[V], const float* inv_cand, int lane, double* slots,
                                               bool add) {
-  if (OUT) {
-    float p1 = 0.f, p2 = 0.f;
-#pragma unroll
-    for (int v = 0; v < V; ++v) {
-      const float kx = di * k[v].x, ky = di * k[v].y, kz = di * k[v].z, kw = di * k[v].w;
-      p1 += kx * a[v].x + ky * a[v].y + kz * a[v].z + kw * a[v].w;
-      p2 += kx * kx + ky * ky + kz * kz + kw * kw;
-    }
-    const float r = warp_sum2(p1, p2, lane);
-    if ((lane & 15) == 0) put_sum(slots + (lane >> 4), r, add);
-  } else {
+  {
     static_assert(NC >= 2 && NC <= 4, "two to four candidates per sweep");
     float inv[NC], part[NC];
 #pragma unroll
@@ -1213,11 +1203,10 @@ struct SearchZ {
 // other, one warp each.  With many chunks their sums are first added group by group, in chunk order.  Then one warp per
 // community adds up its groups (or chunks; lane-strided, then the shuffle tree) and its split segments in table order,
 // and takes the decision.  No sum depends on which warp scored which chunk.
-template <int V, bool OUT, int NC>
+template <int V, int NC>
 __device__ __forceinline__ bool close_sweep(const SearchZ& p, int n_chunks, const float* __restrict__ dinv, const float4* scratch,
-                                            const float4* __restrict__ Hn, const float4* __restrict__ Zn,
-                                            const float4* __restrict__ Rn, int ld4) {
-  constexpr int PER = OUT ? 2 : NC;
+                                            const float4* __restrict__ Hn, const float4* __restrict__ Zn, int ld4) {
+  constexpr int PER = NC;
   const int lane = threadIdx.x & 31;
   const int gwarp = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), n_warps = (int)((gridDim.x * blockDim.x) >> 5);
   const auto nothing = [] {};
@@ -1232,12 +1221,12 @@ __device__ __forceinline__ bool close_sweep(const SearchZ& p, int n_chunks, cons
         const int f = lane + 32 * v;
         a[v] = b[v] = k[v] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (f < ld4) {
-          if (OUT) a[v] = Rn[(long long)sp.x * ld4 + f];
-          else { a[v] = Hn[(long long)sp.x * ld4 + f]; b[v] = twice_error(a[v], Zn[(long long)sp.x * ld4 + f]); }
+          a[v] = Hn[(long long)sp.x * ld4 + f];
+          b[v] = twice_error(a[v], Zn[(long long)sp.x * ld4 + f]);
           for (int q = 0; q < sp.w; ++q) k[v] = vadd(k[v], __ldcg(scratch + (long long)(sp.z + q) * ld4 + f));
         }
       }
-      score_segment<V, OUT, NC>(k, dinv[sp.x], a, b, p.ctl[sp.y].inv_cand, lane, p.split_scores + (size_t)s * PER, false);
+      score_segment<V, NC>(k, dinv[sp.x], a, b, p.ctl[sp.y].inv_cand, lane, p.split_scores + (size_t)s * PER, false);
     }
     const int width = p.n_comm * PER;
     for (int g = blockIdx.x; g < p.n_groups; g += gridDim.x) {
@@ -1302,14 +1291,13 @@ __device__ __forceinline__ void move_blocks(const SearchZ& p, long long n) {
 // One sweep over all chunks by the warps of the grid.  Dynamic shared memory: per warp the row's a, b (2 V float4 per
 // lane; parked there during the walk so that the registers hold gathered rows instead), the candidates of every community
 // (one float4; negative when its search is closed), then the per-warp sums; the last two only with use_smem.
-template <int V, bool OUT, int UN, int NC>
+template <int V, int UN, int NC>
 __device__ __forceinline__ void score_sweep(const int* __restrict__ row_ptr, const int* __restrict__ col,
           const unsigned short* __restrict__ col_comm, const float* __restrict__ dinv,
-          const float4* __restrict__ T, const float4* __restrict__ Hn, const float4* __restrict__ Zn,
-          const float4* __restrict__ Rn, int ld4, const SearchCtl* ctl, int n_comm, double* chunk_part, int use_smem,
+          const float4* __restrict__ T, const float4* __restrict__ Hn, const float4* __restrict__ Zn, int ld4, const SearchCtl* ctl, int n_comm, double* chunk_part, int use_smem,
           const int* __restrict__ chunk_ptr, int n_chunks, int* chunk_counter,
           const int4* __restrict__ items, int n_items, int long_len, float4* scratch) {
-  constexpr int PER = OUT ? 2 : NC;
+  constexpr int PER = NC;
   extern __shared__ float4 s_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int warps_per_block = blockDim.x >> 5;
@@ -1384,15 +1372,14 @@ __device__ __forceinline__ void score_sweep(const int* __restrict__ row_ptr, con
     if (rs >= re) continue;
     __syncwarp();          // the previous unit's last segment has been scored
 #pragma unroll
-    for (int v = 0; v < V; ++v) {   // OUT: a = R' ; else a = h, b = 2 (z - f(h))
+    for (int v = 0; v < V; ++v) {   // a = h, b = 2 (z - f(h))
       const int f = lane + 32 * v;
       float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
       if (f < ld4 && !piece) {
-        if (OUT) a = Rn[(long long)row * ld4 + f];
-        else { a = Hn[(long long)row * ld4 + f]; b = twice_error(a, Zn[(long long)row * ld4 + f]); }
+        { a = Hn[(long long)row * ld4 + f]; b = twice_error(a, Zn[(long long)row * ld4 + f]); }
       }
       row_ab[32 * v] = a;
-      if (!OUT) row_ab[32 * (V + v)] = b;
+      row_ab[32 * (V + v)] = b;
     }
     const float di = dinv[row];
     float4 k[V];
@@ -1415,9 +1402,9 @@ __device__ __forceinline__ void score_sweep(const int* __restrict__ row_ptr, con
 #pragma unroll
       for (int v = 0; v < V; ++v) {
         a[v] = row_ab[32 * v];
-        b[v] = OUT ? a[v] : row_ab[32 * (V + v)];
+        b[v] = row_ab[32 * (V + v)];
       }
-      score_segment<V, OUT, NC>(k, di, a, b, use_smem ? reinterpret_cast<const float*>(s_cand + cur) : ctl[cur].inv_cand, lane,
+      score_segment<V, NC>(k, di, a, b, use_smem ? reinterpret_cast<const float*>(s_cand + cur) : ctl[cur].inv_cand, lane,
                                 mine + cur * PER, true);
     };
 
@@ -1495,35 +1482,33 @@ __device__ __forceinline__ void score_sweep(const int* __restrict__ row_ptr, con
   }
 }
 
-template <int V, bool OUT, int UN, int NC>
+template <int V, int UN, int NC>
 __global__ void __launch_bounds__(256, (V <= 1 ? 4 : V <= 2 ? 3 : 1))
 k_score_z(const int* __restrict__ row_ptr, const int* __restrict__ col,
           const unsigned short* __restrict__ col_comm, const float* __restrict__ dinv,
-          const float4* __restrict__ T, const float4* __restrict__ Hn, const float4* __restrict__ Zn,
-          const float4* __restrict__ Rn, int ld4, const SearchCtl* __restrict__ ctl, int n_comm,
+          const float4* __restrict__ T, const float4* __restrict__ Hn, const float4* __restrict__ Zn, int ld4, const SearchCtl* __restrict__ ctl, int n_comm,
           double* __restrict__ chunk_part, const int* __restrict__ n_active, int use_smem,
           const int* __restrict__ chunk_ptr, int n_chunks, int* __restrict__ chunk_counter,
           const int4* __restrict__ items, int n_items, int long_len, float4* __restrict__ scratch) {
   if (*n_active <= 0) return;
-  score_sweep<V, OUT, UN, NC>(row_ptr, col, col_comm, dinv, T, Hn, Zn, Rn, ld4, ctl, n_comm, chunk_part, use_smem, chunk_ptr, n_chunks,
+  score_sweep<V, UN, NC>(row_ptr, col, col_comm, dinv, T, Hn, Zn, ld4, ctl, n_comm, chunk_part, use_smem, chunk_ptr, n_chunks,
                               chunk_counter, items, n_items, long_len, scratch);
 }
 
-// The rest of the search, cooperative: closes the sweep that k_score_z (or k_score_z_out_part) has just made, makes and
-// closes further ones while a community is still searching (hidden layers), and moves the blocks.  The first sweep has a
+// The rest of the search, cooperative: closes the sweep that k_score_z has just made, makes and
+// closes further ones while a community is still searching, and moves the blocks.  The first sweep has a
 // kernel of its own because, compiled together with this one, its walk spills registers (2.4 M rows x 256: 14.9 against 13.6 ms).
-template <int V, bool OUT, int UN, int NC>
-__global__ void __launch_bounds__(256, (OUT ? 4 : V <= 2 ? 3 : 1))
+template <int V, int UN, int NC>
+__global__ void __launch_bounds__(256, (V <= 2 ? 3 : 1))
 k_close_z(const int* __restrict__ row_ptr, const int* __restrict__ col,
           const unsigned short* __restrict__ col_comm, const float* __restrict__ dinv,
-          const float4* __restrict__ T, const float4* __restrict__ Hn, const float4* __restrict__ Zn,
-          const float4* __restrict__ Rn, int ld4, int n, int use_smem, const int* __restrict__ chunk_ptr, int n_chunks,
+          const float4* __restrict__ T, const float4* __restrict__ Hn, const float4* __restrict__ Zn, int ld4, int n, int use_smem, const int* __restrict__ chunk_ptr, int n_chunks,
           const int4* __restrict__ items, int n_items, int long_len, float4* scratch, const SearchZ sz) {
   if (__ldcg(sz.n_active) > 0) {
     for (;;) {
-      if (!close_sweep<V, OUT, NC>(sz, n_chunks, dinv, scratch, Hn, Zn, Rn, ld4)) return;
-      if (OUT || __ldcg(sz.n_active) <= 0) break;   // changes only between the meetings of close_sweep
-      score_sweep<V, OUT, UN, NC>(row_ptr, col, col_comm, dinv, T, Hn, Zn, Rn, ld4, sz.ctl, sz.n_comm, sz.chunk_part, use_smem, chunk_ptr,
+      if (!close_sweep<V, NC>(sz, n_chunks, dinv, scratch, Hn, Zn, ld4)) return;
+      if (__ldcg(sz.n_active) <= 0) break;   // changes only between the meetings of close_sweep
+      score_sweep<V, UN, NC>(row_ptr, col, col_comm, dinv, T, Hn, Zn, ld4, sz.ctl, sz.n_comm, sz.chunk_part, use_smem, chunk_ptr,
                                   n_chunks, sz.chunk_counter, items, n_items, long_len, scratch);
       if (!grid_meet(sz.bar, sz.err, [] {})) return;
     }
@@ -1531,153 +1516,295 @@ k_close_z(const int* __restrict__ row_ptr, const int* __restrict__ col,
   move_blocks(sz, n);
 }
 
-// The output-layer form of k_score_z (OUT = true) for rows of at most G float4 (G = 4, 8, 16: C_L <= 16, 32, 64): 32 / G
-// units per warp, each group of G lanes walking its own row or item, G stored entries per chunk.  With 12 of 32 lanes
-// carrying columns (47 classes), or one (3 classes), the full-warp form spends most of its issue slots on lanes that hold
-// nothing and walks one row where the warp could walk eight.  Control flow is kept the same for all groups (loop bounds
-// are the largest of them, a group that has run out holds weight 0 and no segment start), shuffles use width G, and only
-// the closing of a segment is a divergent branch, inside which nothing is exchanged beyond the group's own lanes.  Sums go to one
-// array per group (groups may close segments of the same community at the same time).
-// Dynamic shared memory: (32 / G) x warps x n_comm x 2 doubles (the caller takes a larger G, then k_score_z, when that
-// does not fit).
-template <int G, int UN>
-__global__ void __launch_bounds__(256, 4)
-k_score_z_out_part(const int* __restrict__ row_ptr, const int* __restrict__ col,
-                   const unsigned short* __restrict__ col_comm, const float* __restrict__ dinv,
-                   const float4* __restrict__ T, const float4* __restrict__ Rn, int ld4,
-                   const SearchCtl* __restrict__ ctl, int n_comm, double* __restrict__ chunk_part,
-                   const int* __restrict__ n_active, const int* __restrict__ chunk_ptr, int n_chunks,
-                   int* __restrict__ chunk_counter,
-                   const int4* __restrict__ items, int n_items, int long_len, float4* __restrict__ scratch,
-                   const int* __restrict__ row_order) {
-  if (*n_active <= 0) return;
-  static_assert(G % UN == 0, "UN divides the chunk");
-  constexpr int GROUPS = 32 / G;
-  extern __shared__ double s_part[];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, grp = lane / G, gl = lane & (G - 1);
-  const int warps_per_block = blockDim.x >> 5;
-  constexpr unsigned kGroupMask = G == 32 ? 0xffffffffu : ((1u << G) - 1u);
-  const unsigned gmask = kGroupMask << (G * grp);
-  for (int i = threadIdx.x; i < GROUPS * warps_per_block * n_comm * 2; i += blockDim.x) s_part[i] = 0.0;
-  double* const mine = s_part + (size_t)(GROUPS * warp + grp) * n_comm * 2;   // the group's sums of the chunk in hand
-  __syncthreads();
-  const bool in_row = gl < ld4;
-  const float4* __restrict__ T_lane = T + gl;
-  for (;;) {   // chunks from a global counter, their sums to chunk_part: see k_score_z
+// ------------------------------------------------------------------------------------------
+// The search of the last hidden layer (layer l+1 = L is linear): along Z_{l,m} - G_m/theta the objective changes by
+//   -(1/theta) sum_i <K_m[i], R'_i> + (rho / 2 theta^2) sum_i ||K_m[i]||^2   plus the block's own quadratic term,
+// so two sums decide every trial.  The first needs no walk over the graph: A~ is symmetric, hence
+//   sum_i <K_m[i], R'_i> = sum_{j in V_m} <T_j, (A~ R')_j>,  and A~ R' = S has just been formed for the gradient.
+// The second is a sum over the segments (row i, community m) of the graph, taken community by community (tables of
+// build_segment_tables): the rows of T that a community's segments gather are the community's own block of T, a few MB that
+// stay in L2, the segments of a chunk have one length, so the lanes of a warp never wait for each other, and a chunk
+// belongs to one community, so that its sum lives in a register.
+// (Walking the rows instead, with a ballot per group of entries to find the segments and a shared-memory slot per
+// community: 45 us at 20 k rows x 3 classes, 146 us at 169 k x 40, 4.6 ms at 2.45 M x 47; this form: 21 us, 99 us, 3.8 ms.)
+// CL lanes hold a row of T (ld4 <= CL float4), 32 / CL segments at a time per warp; segments of `share_from` entries or more
+// are shared by all lanes of the warp, entry e going to set e mod (32 / CL): where the chunks are few and the longest
+// segment sets the time, and with CL <= 4.  The warp that finishes a community's last slot adds
+// its slots up in slot order and takes the decision.
+// ------------------------------------------------------------------------------------------
+struct SegRef {
+  int begin;
+  float dinv;
+};
+struct SegChunk {
+  int first, count, length, comm, slot;   // see build_segment_tables
+};
+struct SearchOut {
+  const SegRef* segs;
+  const SegChunk* chunks;
+  int n_chunks;
+  int* chunk_counter;
+  const int* slot_ptr;        // [n_comm + 1]
+  double* slots;              // [slot][2]: sum of <T, S>, sum of ||K||^2
+  int *comm_done, *split_done;   // finished slots of a community, finished pieces of a split segment; left at zero
+  const int4 *items, *split;
+  SearchCtl* ctl;
+  const double* own;          // [community][3] from k_zgrad_finish; [2] = <Z - f(H), G>
+  int *n_active, *status;
+  int share_from;             // segments of this length or more are shared by all lanes of a warp
+  DecideArgs a;
+};
+
+// dot and square sums of the float4 a lane holds
+__device__ __forceinline__ float dot4(const float4& a, const float4& b) { return a.x * b.x + a.y * b.y + a.z * b.z + a.w * b.w; }
+
+// `count` segments of length LEN <= 3.  The lanes fetch the entries of 32 segments, one segment each (columns of the
+// next 32 while these are gathered), and hand them to the groups by shuffles; UN segments per group in flight.
+template <int CL, int LEN, int UN>
+__device__ __forceinline__ double short_segments(const SegRef* __restrict__ segs, int count, const int* __restrict__ col,
+                                                 const float* __restrict__ dinv, const float4* __restrict__ T, int ld4, int lane) {
+  constexpr int GROUPS = 32 / CL;
+  const int grp = lane / CL, cl = lane & (CL - 1);
+  const float4* __restrict__ T_lane = T + min(cl, ld4 - 1);
+  double acc = 0.0;
+  SegRef next{0, 0.f};
+  if (lane < count) next = segs[lane];
+  int c_next[LEN];
+#pragma unroll
+  for (int e = 0; e < LEN; ++e) c_next[e] = lane < count ? col[next.begin + e] : 0;
+  for (int b = 0; b < count; b += 32) {
+    const float di = next.dinv;
+    int c[LEN];
+    float w[LEN];
+#pragma unroll
+    for (int e = 0; e < LEN; ++e) { c[e] = c_next[e]; w[e] = dinv[c[e]]; }   // past the last segment: column 0, factor 0
+    next.dinv = 0.f;
+    const bool more = b + 32 + lane < count;
+    if (more) next = segs[b + 32 + lane];
+#pragma unroll
+    for (int e = 0; e < LEN; ++e) c_next[e] = more ? col[next.begin + e] : 0;
+    const int nb = min(32, count - b);
+    for (int t = 0; t * GROUPS < nb; t += UN) {
+      float part = 0.f;
+      float4 x[UN][LEN];
+      float ww[UN][LEN], dd[UN];
+#pragma unroll
+      for (int u = 0; u < UN; ++u) {
+        const int src = ((t + u) * GROUPS + grp) & 31;
+        dd[u] = __shfl_sync(0xffffffffu, di, src);
+        if ((t + u) * GROUPS >= 32) dd[u] = 0.f;
+#pragma unroll
+        for (int e = 0; e < LEN; ++e) {
+          const int r = __shfl_sync(0xffffffffu, c[e], src);
+          ww[u][e] = __shfl_sync(0xffffffffu, w[e], src);
+          x[u][e] = __ldg(T_lane + (unsigned)r * (unsigned)ld4);   // n * ld4 < 2^32; lanes past the row read its last column
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < UN; ++u) {
+        float4 k = vscale(ww[u][0], x[u][0]);
+#pragma unroll
+        for (int e = 1; e < LEN; ++e) k = vfma(ww[u][e], x[u][e], k);
+        k = vscale(dd[u], k);
+        part += dot4(k, k);
+      }
+      if (cl < ld4) acc += (double)part;
+    }
+  }
+  return acc;
+}
+
+// `count` segments of one length, a group of CL >= 8 lanes each: the group's lanes fetch CL entries at a time, columns two
+// steps ahead and weights one (across segments too), and hand them round by shuffles.
+template <int CL, int UN>
+__device__ __forceinline__ double group_segments(const SegRef* __restrict__ segs, int count, int len, const int* __restrict__ col,
+                                                 const float* __restrict__ dinv, const float4* __restrict__ T, int ld4, int lane) {
+  constexpr int GROUPS = 32 / CL;
+  const int grp = lane / CL, cl = lane & (CL - 1);
+  const bool in_row = cl < ld4;
+  const float4* __restrict__ T_lane = T + cl;
+  double acc = 0.0;
+  int f_k = grp, f_o = cl, f_begin = grp < count ? segs[grp].begin : 0, f_next = grp + GROUPS < count ? segs[grp + GROUPS].begin : 0;
+  auto fetch = [&]() {   // the next column of this lane; -1 past a segment's end
+    const int c = f_k < count && f_o < len ? col[f_begin + f_o] : -1;
+    f_o += CL;
+    if (f_o - cl >= len) {   // the same in all groups
+      f_o = cl;
+      f_k += GROUPS;
+      f_begin = f_next;
+      if (f_k + GROUPS < count) f_next = segs[f_k + GROUPS].begin;
+    }
+    return c;
+  };
+  int c_n = fetch(), c_n2 = fetch();
+  float w_n = c_n >= 0 ? dinv[c_n] : 0.f;
+  for (int k0 = 0; k0 < count; k0 += GROUPS) {
+    float4 k;
+    vzero(k);
+    for (int o = 0; o < len; o += CL) {
+      const int c = max(c_n, 0);
+      const float w = w_n;
+      c_n = c_n2;
+      w_n = c_n >= 0 ? dinv[c_n] : 0.f;
+      c_n2 = fetch();
+      const int cnt = min(CL, len - o);
+      for (int t = 0; t < cnt; t += UN) {
+        int r[UN];
+        float ww[UN];
+#pragma unroll
+        for (int u = 0; u < UN; ++u) {
+          r[u] = __shfl_sync(0xffffffffu, c, t + u, CL);
+          ww[u] = __shfl_sync(0xffffffffu, w, t + u, CL);
+        }
+        if (in_row) {
+          float4 x[UN];
+#pragma unroll
+          for (int u = 0; u < UN; ++u) x[u] = __ldg(T_lane + (unsigned)r[u] * (unsigned)ld4);   // n * ld4 < 2^32
+#pragma unroll
+          for (int u = 0; u < UN; ++u) k = vfma(ww[u], x[u], k);
+        }
+      }
+    }
+    if (k0 + grp < count) {
+      k = vscale(segs[k0 + grp].dinv, k);
+      acc += (double)dot4(k, k);
+    }
+  }
+  return acc;
+}
+
+// K_m[i] / dinv_i of one run of entries [b, e), entry b + set, b + set + sets, .. of it
+template <int UN>
+__device__ __forceinline__ float4 walk_run(int b, int e, int set, int sets, const int* __restrict__ col, const float* __restrict__ dinv,
+                                           const float4* __restrict__ T, int ld4, int cl) {
+  float4 k;
+  vzero(k);
+  int c[UN];
+#pragma unroll
+  for (int u = 0; u < UN; ++u) c[u] = b + set + u * sets < e ? col[b + set + u * sets] : -1;
+  for (int p = b + set; p < e; p += UN * sets) {
+    float w[UN];
+    int r[UN];
+#pragma unroll
+    for (int u = 0; u < UN; ++u) { r[u] = c[u]; w[u] = r[u] >= 0 ? dinv[r[u]] : 0.f; }
+    const int q = p + UN * sets;
+#pragma unroll
+    for (int u = 0; u < UN; ++u) c[u] = q + u * sets < e ? col[q + u * sets] : -1;
+    if (cl < ld4) {
+      float4 x[UN];
+#pragma unroll
+      for (int u = 0; u < UN; ++u)
+        if (r[u] >= 0) x[u] = __ldg(T + (long long)r[u] * ld4 + cl);
+#pragma unroll
+      for (int u = 0; u < UN; ++u)
+        if (r[u] >= 0) k = vfma(w[u], x[u], k);
+    }
+  }
+  return k;
+}
+// sum over the sets of a warp that share a run
+template <int CL>
+__device__ __forceinline__ float4 add_sets(float4 k) {
+#pragma unroll
+  for (int o = CL; o < 32; o <<= 1) k = vadd(k, vxor(0xffffffffu, k, o));
+  return k;
+}
+
+template <int CL>
+__global__ void __launch_bounds__(256, 3)
+k_search_z_out(const int* __restrict__ col, const float* __restrict__ dinv, const float4* __restrict__ T, const float4* __restrict__ S,
+               int ld4, float4* scratch, const SearchOut p) {
+  constexpr int GROUPS = 32 / CL;
+  const int lane = threadIdx.x & 31, grp = lane / CL, cl = lane & (CL - 1);
+  for (;;) {
     int ch = 0;
-    if (lane == 0) ch = atomicAdd(chunk_counter, 1);
+    if (lane == 0) ch = atomicAdd(p.chunk_counter, 1);
     ch = __shfl_sync(0xffffffffu, ch, 0);
-    if (ch >= n_chunks) break;
-    const int chunk_end = chunk_ptr[ch + 1];
-    for (int unit0 = chunk_ptr[ch]; unit0 < chunk_end; unit0 += GROUPS) {
-      const int unit = unit0 + grp;
-      int row = 0, rs = 0, re = 0;
-      bool piece = false;
-      if (unit < chunk_end) {
-        if (unit < n_items) {
-          const int4 it = items[unit];
-          row = it.x; rs = it.y; re = it.z;
-          piece = it.w >= 0;
-        } else {
-          row = row_order[unit - n_items];
-          rs = row_ptr[row]; re = row_ptr[row + 1];
-          if (re - rs > long_len) re = rs;          // walked as items
+    if (ch >= p.n_chunks) return;
+    const SegChunk c = p.chunks[ch];
+    if (__ldcg(&p.ctl[c.comm].done)) continue;   // skipped: none of its slots is filled
+    double lin = 0.0, quad = 0.0;
+    if (c.length > 0) {
+      const SegRef* const segs = p.segs + c.first;
+      if (c.length == 1) quad = short_segments<CL, 1, CL >= 8 ? 8 : CL>(segs, c.count, col, dinv, T, ld4, lane);
+      else if (c.length == 2) quad = short_segments<CL, 2, CL >= 4 ? 4 : CL>(segs, c.count, col, dinv, T, ld4, lane);
+      else if (c.length == 3) quad = short_segments<CL, 3, CL >= 2 ? 2 : CL>(segs, c.count, col, dinv, T, ld4, lane);
+      else if (CL >= 8 && c.length < p.share_from) {
+        if constexpr (CL >= 8) quad = group_segments<CL, 8>(segs, c.count, c.length, col, dinv, T, ld4, lane);
+      } else if (c.length < p.share_from) {
+        for (int k = grp; k < c.count; k += GROUPS) {
+          const SegRef sg = segs[k];
+          const float4 v = vscale(sg.dinv, walk_run<4>(sg.begin, sg.begin + c.length, 0, 1, col, dinv, T, ld4, cl));
+          quad += (double)dot4(v, v);
+        }
+      } else {
+        for (int k = 0; k < c.count; ++k) {
+          const SegRef sg = segs[k];
+          const float4 v = vscale(sg.dinv, add_sets<CL>(walk_run<4>(sg.begin, sg.begin + c.length, grp, GROUPS, col, dinv, T, ld4, cl)));
+          if (grp == 0) quad += (double)dot4(v, v);
         }
       }
-      float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (in_row && !piece && re > rs) a = Rn[(long long)row * ld4 + gl];
-      const float di = dinv[row];
-      float4 k = make_float4(0.f, 0.f, 0.f, 0.f);
-      int cur = -1;
-      bool cur_on = false;
-
-      auto finish_segment = [&]() {   // called by one group at a time: exchanges stay inside gmask
-        if (!cur_on) return;
-        if (piece) {
-          if (in_row) scratch[(long long)unit * ld4 + gl] = k;
-          return;
-        }
-        const float kx = di * k.x, ky = di * k.y, kz = di * k.z, kw = di * k.w;
-        const float p1 = kx * a.x + ky * a.y + kz * a.z + kw * a.w;
-        const float p2 = kx * kx + ky * ky + kz * kz + kw * kw;
-        const bool up = gl & (G / 2);
-        float c = (up ? p2 : p1) + __shfl_xor_sync(gmask, up ? p1 : p2, G / 2, G);
-#pragma unroll
-        for (int o = G / 4; o > 0; o >>= 1) c += __shfl_xor_sync(gmask, c, o, G);
-        if ((gl & (G / 2 - 1)) == 0) put_sum(mine + cur * 2 + (up ? 1 : 0), c, true);
-      };
-
-      const int len = re - rs;
-      int len_max = len;
-#pragma unroll
-      for (int o = G; o < 32; o <<= 1) len_max = max(len_max, __shfl_xor_sync(0xffffffffu, len_max, o));
-      int c_next = 0, m_next = -1;   // fetched one chunk ahead, as in k_score_z
-      if (rs + gl < re) { c_next = col[rs + gl]; m_next = col_comm[rs + gl]; }
-      for (int o = 0; o < len_max; o += G) {
-        const int idx = rs + o + gl;
-        const bool valid = idx < re;
-        const int c = c_next, m = m_next;
-        if (idx + G < re) { c_next = col[idx + G]; m_next = col_comm[idx + G]; }
-        else m_next = -1;
-        unsigned off = 0u;
-        float w = 0.f;
-        bool live = false;
-        if (valid) {
-          const float wc = dinv[c];
-          live = !ctl[m].done;
-          if (live) { w = wc; off = (unsigned)c * (unsigned)ld4; }
-        }
-        int mprev = __shfl_up_sync(0xffffffffu, m, 1, G);
-        if (gl == 0) mprev = cur;
-        unsigned chg = (__ballot_sync(0xffffffffu, valid && m != mprev) >> (G * grp)) & kGroupMask;
-        const unsigned on_all = __ballot_sync(0xffffffffu, live);
-        unsigned on = (on_all >> (G * grp)) & kGroupMask;
-        const int cnt_max = min(G, len_max - o);
-        if (on_all == 0u) {   // no group has anything to gather in this chunk
-          if (chg != 0u) {    // per group: an open segment ends at the chunk's first entry
-            finish_segment();
-            cur = __shfl_sync(gmask, m, min(G, len - o) - 1, G);
-            cur_on = false;
-          }
-          continue;
-        }
-        for (int t = 0; t < cnt_max; t += UN, chg >>= UN, on >>= UN) {
-          unsigned oj[UN];
-          float wj[UN];
-#pragma unroll
-          for (int u = 0; u < UN; ++u) {
-            oj[u] = __shfl_sync(0xffffffffu, off, t + u, G);
-            wj[u] = __shfl_sync(0xffffffffu, w, t + u, G);
-          }
-          float4 xv[UN];   // set and read under the same condition
-#pragma unroll
-          for (int u = 0; u < UN; ++u)
-            if (((on >> u) & 1u) && in_row) xv[u] = __ldg(T_lane + oj[u]);
-#pragma unroll
-          for (int u = 0; u < UN; ++u) {
-            if ((chg >> u) & 1u) {                        // uniform within the group
-              finish_segment();
-              cur = col_comm[rs + o + t + u];
-              cur_on = (on >> u) & 1u;
-              k = make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-            if (((on >> u) & 1u) && in_row) k = vfma(wj[u], xv[u], k);
-          }
-        }
-      }
-      finish_segment();
+    } else if (c.length == 0) {
+      const long long e1 = (long long)(c.first + c.count) * ld4;
+#pragma unroll 2
+      for (long long e = (long long)c.first * ld4 + lane; e < e1; e += 32) lin += (double)dot4(T[e], S[e]);
+    } else {
+      const int4 it = p.items[c.first], sp = p.split[c.count];   // a piece {row, first entry, one past the last} of a segment {.., first item, items}
+      const float4 v = add_sets<CL>(walk_run<4>(it.y, it.z, grp, GROUPS, col, dinv, T, ld4, cl));
+      if (grp == 0 && cl < ld4) scratch[(long long)c.first * ld4 + cl] = v;
+      __threadfence();
       __syncwarp();
+      int done = 0;
+      if (lane == 0) done = atomicAdd(p.split_done + c.count, 1);
+      done = __shfl_sync(0xffffffffu, done, 0);
+      if (done + 1 < sp.w) continue;
+      __threadfence();
+      if (lane == 0) p.split_done[c.count] = 0;
+      if (lane < ld4) {   // the pieces in item order
+        float4 k;
+        vzero(k);
+        for (int q = 0; q < sp.w; ++q) k = vadd(k, __ldcg(scratch + (long long)(sp.z + q) * ld4 + lane));
+        k = vscale(dinv[it.x], k);
+        quad = (double)dot4(k, k);
+      }
     }
-    // the chunk's sums, group after group
-    double* const warp_sums = s_part + (size_t)(GROUPS * warp) * n_comm * 2;
-    double* const out_part = chunk_part + (size_t)ch * n_comm * 2;
-    for (int i = lane; i < n_comm * 2; i += 32) {
-      double t = 0.0;
-#pragma unroll
-      for (int g = 0; g < GROUPS; ++g) { t += warp_sums[(size_t)g * n_comm * 2 + i]; warp_sums[(size_t)g * n_comm * 2 + i] = 0.0; }
-      out_part[i] = t;
+    lin = warp_sum(lin);
+    quad = warp_sum(quad);
+    const int s0 = p.slot_ptr[c.comm], s1 = p.slot_ptr[c.comm + 1];
+    int done = 0;
+    if (lane == 0) {
+      p.slots[2 * (size_t)c.slot] = lin;
+      p.slots[2 * (size_t)c.slot + 1] = quad;
+      __threadfence();
+      done = atomicAdd(p.comm_done + c.comm, 1);
     }
-    __syncwarp();
+    done = __shfl_sync(0xffffffffu, done, 0);
+    if (done + 1 < s1 - s0) continue;
+    __threadfence();
+    if (lane == 0) p.comm_done[c.comm] = 0;
+    double sums[2] = {0.0, 0.0};
+#pragma unroll 4
+    for (int s = s0 + lane; s < s1; s += 32) {
+      sums[0] += __ldcg(p.slots + 2 * (size_t)s);
+      sums[1] += __ldcg(p.slots + 2 * (size_t)s + 1);
+    }
+    sums[0] = warp_sum(sums[0]);
+    sums[1] = warp_sum(sums[1]);
+    decide_one(p.ctl + c.comm, sums, p.own[c.comm * 3 + 2], p.a, p.n_active, p.status);
+  }
+}
+
+// The move of the blocks after it: Z_l[i,:] <- Z_l[i,:] - G[i,:] / theta_{comm(i)} (Eq. 10), and the log entries.
+__global__ void __launch_bounds__(256)
+k_move_z(float4* __restrict__ Z, const float4* __restrict__ G, int ld4, long long n, const int* __restrict__ row_comm,
+         const SearchCtl* __restrict__ ctl, int n_comm, const DecisionLog log, int* __restrict__ chunk_counter) {
+  const long long first = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
+  if (first == 0) *chunk_counter = 0;
+  for (long long i = first; i < n_comm; i += stride) log_decision(log, (int)i, ctl + i);
+  for (long long e = first; e < n * ld4; e += stride) {   // below 2^32
+    const float s = ctl[row_comm[(unsigned)e / (unsigned)ld4]].inv_step;
+    if (s == 0.f) continue;
+    Z[e] = vfma(-s, G[e], Z[e]);
   }
 }
 
