@@ -43,6 +43,7 @@ constexpr int kZBlockRows = 32;      // rows per block of the hidden-layer gradi
 constexpr int kChunkGroups = 512;    // groups the sums of a scoring sweep's chunks are first added up in, when there are more chunks
 constexpr int kCandZ = 4;           // theta candidates scored per sweep (2..4; steady-state searches close at trial 0..2)
 constexpr size_t kDirectBytes = (size_t)256 << 10;   // matrices up to this size cross the bus inside the permuting kernel (one copy and its latency less)
+constexpr long long kSmallProblem = 1LL << 27;   // nodes x widest layer: below it launch gaps show in a pass
 constexpr int kDefaultLongRow = 256;   // stored entries one warp walks before a row is cut into items
 
 thread_local std::string g_create_error;
@@ -216,11 +217,13 @@ struct gcn_admm {
   gk::Report* report = nullptr;             // objective sums and error flags
   double* red_part = nullptr;               // per-block partial sums awaiting their fixed-order reduction
   int4* d_zblocks = nullptr;                // row blocks of at most kZBlockRows rows, none crossing a community, and that community
-  unsigned *ticket = nullptr, *comm_tickets = nullptr;   // counters of finished blocks (one launch; per community), zero between launches
+  unsigned *ticket = nullptr, *tile_tickets = nullptr, *comm_tickets = nullptr;   // counters of finished blocks (one launch; per community), zero between launches
   gk::GridBar* grid_bar = nullptr;          // meeting point of the cooperative launches (one at a time: one stream)
   std::vector<float*> RN;                   // 2..L: derivative of phi_l at the new H_l, from the W_l update to that of Z_{l-1}
   int* d_comm_block_ptr = nullptr;          // [M+1] first row block of every community
   int n_zblocks = 0;
+  int *d_h1_age = nullptr, *skip_h1 = nullptr;   // see k_end_pass
+  float* DL = nullptr;       // P_L grad_L
   int *n_active = nullptr, *status = nullptr, *d_pass = nullptr;   // status = &report->status
   // Z scoring: units in chunks of about equally many stored entries, dealt to the warps of the grid in a fixed order
   int* d_chunk_ptr = nullptr;
@@ -238,6 +241,7 @@ struct gcn_admm {
   double* split_scores = nullptr;           // [n_split][candidates] sums of the segments scored in pieces
   int *d_split_order = nullptr, *d_split_ptr = nullptr;   // split entries grouped by community
   cudaGraphExec_t pass_graph = nullptr;   // one pass of Algorithm 1, recorded once and replayed
+  long long single_passes = 0;            // passes launched without it
   int *log_trial_w = nullptr, *log_trial_z = nullptr;
   double *log_q_w = nullptr, *log_q_z = nullptr;
   long long log_count = 0;
@@ -411,21 +415,27 @@ struct gcn_admm {
     dim3 grid((unsigned)std::max(1, std::min(tiles, kSmCount / groups)), (unsigned)groups);                    \
     if ((p.tensor_cores == 2 || Mr >= kImageMinRows) && image_bytes <= b_image_bytes) {                        \
       const long long work = (long long)groups * cdiv(K, gtc::kChunkK) * (NT) * 8;                             \
-      gtc::k_split_b<<<(unsigned)std::min<long long>(cdiv(work, 256), 4 * kSmCount), 256, 0, stream>>>(Bk, ldbk, N, K, NT, b_image); \
+      gtc::k_split_b<<<(unsigned)std::min<long long>(cdiv(work, 256), 4 * kSmCount), 256, 0, stream>>>(Bk, ldbk, N, K, NT, b_image, skip); \
       ++launches;                                                                                              \
       /* up to 128 columns: A tiles by tensor copies into a ring of their own (at 256 columns shared memory    \
          leaves no room for it, and the form measured no faster there) */                                      \
       if ((NT) <= 128 && make_a_tile_map(A, Mr, lda, &tmap)) {                                                 \
         const size_t smem_ring = gtc::WsCfg<NT>::kSmemRing;                                                    \
         CU(cudaFuncSetAttribute(gtc::k_gemm_tc_ws<NT, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_ring)); \
-        gtc::k_gemm_tc_ws<NT, true, true><<<grid, gtc::WsCfg<NT>::kThreads + 32, smem_ring, stream>>>(A, lda, Bk, ldbk, Cm, ldc, (int)Mr, N, K, skip, tc_error, b_image, tmap); \
+        gtc::k_gemm_tc_ws<NT, true, true><<<grid, gtc::WsCfg<NT>::kThreads + 32, smem_ring, stream>>>(A, lda, Bk, ldbk, Cm, ldc, (int)Mr, N, K, skip, tc_error, b_image, tmap, nullptr, nullptr); \
       } else {                                                                                                 \
         CU(cudaFuncSetAttribute(gtc::k_gemm_tc_ws<NT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
-        gtc::k_gemm_tc_ws<NT, true><<<grid, gtc::WsCfg<NT>::kThreads, smem, stream>>>(A, lda, Bk, ldbk, Cm, ldc, (int)Mr, N, K, skip, tc_error, b_image, tmap); \
+        gtc::k_gemm_tc_ws<NT, true><<<grid, gtc::WsCfg<NT>::kThreads, smem, stream>>>(A, lda, Bk, ldbk, Cm, ldc, (int)Mr, N, K, skip, tc_error, b_image, tmap, nullptr, nullptr); \
       }                                                                                                        \
     } else {                                                                                                   \
+      /* few row tiles and a long reduction: several CTAs share a tile's K chunks, at least four chunks each          \
+         (2.7 k rows, K = 1433, 16 columns: 34 -> 13 us) */                                                       \
+      const int kc = (int)cdiv(K, gtc::kChunkK);                                                               \
+      const int ways = (int)std::max<long long>(1, std::min<long long>({kSmCount / ((long long)tiles * groups), kc / 4, \
+                                                                        (long long)(part_elems / ((size_t)Mr * ldc))})); \
+      grid.z = (unsigned)ways;                                                                                 \
       CU(cudaFuncSetAttribute(gtc::k_gemm_tc_ws<NT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
-      gtc::k_gemm_tc_ws<NT, false><<<grid, gtc::WsCfg<NT>::kThreads, smem, stream>>>(A, lda, Bk, ldbk, Cm, ldc, (int)Mr, N, K, skip, tc_error, nullptr, tmap); \
+      gtc::k_gemm_tc_ws<NT, false><<<grid, gtc::WsCfg<NT>::kThreads, smem, stream>>>(A, lda, Bk, ldbk, Cm, ldc, (int)Mr, N, K, skip, tc_error, nullptr, tmap, part, tile_tickets); \
     }                                                                                                          \
   }
       if (N <= 16) TC_WS(16)
@@ -591,28 +601,30 @@ struct gcn_admm {
 
   // ---- W_l block (Section 3.1) --------------------------------------------------------
   // resid_next: also leave the derivative of phi_l at the new H_l in RN[l] (what the Z_{l-1} update starts from).
+  // The last layer works in matrices of its own width (RN[L], DL), so that its chain can run beside the others' (see Lane).
   void update_W(int l, bool resid_next) {
     Range range("gcn_admm: W block");
     const int Kp = C[l - 1], Cn = C[l], ldc = ld[l];
     const long long n4 = n * ldc / 4;
     SearchCtl* ctl = ctl_w + l;
+    float *const R = l == L ? RN[L] : B0, *const D = l == L ? DL : B1;
     int splits;
     if (l < L && tn_on_tensor_cores(n)) {                               // grad = P_l^T R_l, R_l formed inside the product
       splits = gemm_tn(P[l], ld[l - 1], H[l], ldc, ldc, n, Kp, Cn, Z[l], p.nu);
     } else {
-      resid(l, B0);                                                     // R_l
-      splits = gemm_tn(P[l], ld[l - 1], B0, ldc, ldc, n, Kp, Cn);       // grad = P_l^T R_l
+      resid(l, R);                                                      // R_l
+      splits = gemm_tn(P[l], ld[l - 1], R, ldc, ldc, n, Kp, Cn);        // grad = P_l^T R_l
     }
     finish_grad(splits, Kp, Cn, ldc, grad, grad_t, ld[l - 1], W[l], ctl);
-    gemm_nn(P[l], ld[l - 1], grad, ldc, grad_t, ld[l - 1], B1, ldc, n, Cn, Kp, &ctl->done);   // D = P_l grad
+    gemm_nn(P[l], ld[l - 1], grad, ldc, grad_t, ld[l - 1], D, ldc, n, Cn, Kp, &ctl->done);   // D = P_l grad
     gk::SearchW a{};
-    a.H = (float4*)H[l]; a.D = (const float4*)B1; a.Z = (const float4*)Z[l]; a.U = (const float4*)U; a.R = (const float4*)B0;
+    a.H = (float4*)H[l]; a.D = (const float4*)D; a.Z = (const float4*)Z[l]; a.U = (const float4*)U; a.R = (const float4*)R;
     a.Rn = resid_next ? (float4*)RN[l] : nullptr;
     a.n4 = n4;
     a.coef = l == L ? p.rho : p.nu;
     a.W = W[l]; a.Wt = Wt[l]; a.grad = grad;
     a.rows = Kp; a.cols = Cn; a.ldw = ldc; a.ldwt = ld[l - 1];
-    a.ctl = ctl; a.partial = red_part; a.bar = grid_bar; a.status = status; a.err = tc_error;
+    a.ctl = ctl; a.partial = red_part; a.bar = grid_bar; a.ticket = ticket; a.status = status; a.err = tc_error;
     a.a.growth = p.bt_growth;
     a.a.max_trials = p.bt_max_trials;
     a.a.cand = gk::kCand;
@@ -620,10 +632,20 @@ struct gcn_admm {
     a.a.scale = 0.5 * p.nu;
     a.a.quad_coef = 0.5 * p.rho;
     a.log = log_w(l);
-    // scoring reads three arrays (two for the last layer), the move reads two and writes one, the residual reads one or two and writes one
-    const double arrays = (l == L ? 2 : 3) + 3 + (resid_next ? (l == L ? 3 : 2) : 0);
-    Scope sc(this, l == L ? "search_w_out" : "search_w_hidden", 1, 16.0 * arrays * n4, 0.0);
-    launch_together(l == L ? gk::k_search_w<true> : gk::k_search_w<false>, cdiv(n4, 256), 256, 0, a);
+    // the move reads two arrays and writes one; the next residual reads one more (two for the last layer) and writes one
+    if (l == L) {
+      {
+        Scope sc(this, "score_w_out", 1, 32.0 * n4, 0.0);
+        gk::k_score_w_out<<<grid_for(n4), 256, 0, stream>>>(a);
+        CU(cudaGetLastError());
+      }
+      Scope sc(this, "move_w_out", 1, 16.0 * (3 + (resid_next ? 3 : 0)) * n4, 0.0);
+      gk::k_move_w_out<<<grid_for(n4), 256, 0, stream>>>(a);
+      CU(cudaGetLastError());
+    } else {
+      Scope sc(this, "search_w_hidden", 1, 16.0 * (6 + (resid_next ? 2 : 0)) * n4, 0.0);
+      launch_together(gk::k_search_w_hidden, cdiv(n4, 256), 256, 0, a);
+    }
   }
 
   // ---- Z_{l,m}, l < L, every community (Appendix A, Eq. 5/6 and 8-10) ------------------
@@ -652,7 +674,7 @@ struct gcn_admm {
     decide.max_trials = p.bt_max_trials;
     decide.own_nu = p.nu;
     if (l + 1 == L) {   // closed form
-      gemm_nn(B2, ldl, W[L], ldn, Wt[L], ldl, B0, ldn, n, C[L], C[l]);   // T = G W_L; S stays in B1, R' is not needed any more
+      gemm_nn(B2, ldl, W[L], ldn, Wt[L], ldl, B0, ldn, n, C[L], C[l]);   // T = G W_L; S stays in B1
       decide.mode = 1;
       decide.quad_coef = 0.5 * p.rho;
       gk::SearchOut a{};
@@ -724,8 +746,7 @@ struct gcn_admm {
   }
 
   // ---- Z_L (Eq. 7) and, in the same sweep, the dual as printed in Eq. 3 -----------------
-  // end_pass: this is the last block family of a pass (the pass counter of the log moves on).
-  void update_output(bool dual_now, bool update_z, bool end_pass) {
+  void update_output(bool dual_now, bool update_z) {
     Range range("gcn_admm: output layer and dual");
     Scope sc(this, "output_rows", 1, 4.0 * (double)n * ld[L] * (3 + (update_z ? 1 : 0) + (dual_now ? 1 : 0)), 0.0);
     gk::OutputArgs a{};
@@ -734,7 +755,6 @@ struct gcn_admm {
     a.train = d_train; a.rows = d_train_rows; a.y = d_y; a.n_train = n_train; a.momentum = d_fista_momentum;
     a.rho = p.rho; a.loss_scale = p.loss_scale; a.iters = p.fista_iters;
     a.dual_now = dual_now ? 1 : 0; a.update_z = update_z ? 1 : 0;
-    a.advance = end_pass ? d_pass : nullptr;
     const int plain_blocks = grid_for(n * (ld[L] / 4));
 #define OUTPUT(LPR, CPL)                                                        \
   {                                                                             \
@@ -764,17 +784,30 @@ struct gcn_admm {
   // keep_h1: the caller knows that H_1 already is P_1 W_1.  After a pass it is: P_1 never changes and
   // the W_1 step left H_1 - D/tau = P_1 (W_1 - grad/tau) behind, so the product is skipped; to keep
   // rounding from piling up over many passes it is still formed afresh every kH1RefreshEvery passes.
+  // A recorded pass launches the product every time and lets the device decide (*skip_h1, kept by k_end_pass).
   static constexpr int kH1RefreshEvery = 16;
   int h1_age = 0;
   bool capturing = false;
   void refresh(bool keep_h1 = false) {
     Range range("gcn_admm: refresh P_l, H_l");
     for (int l = 2; l <= L; ++l) spmm(Z[l - 1], P[l], ld[l - 1]);
-    const bool skip_h1 = keep_h1 && !capturing && h1_age + 1 < kH1RefreshEvery;
-    h1_age = skip_h1 ? h1_age + 1 : 0;
-    for (int l = skip_h1 ? 2 : 1; l <= L; ++l)
-      gemm_nn(P[l], ld[l - 1], W[l], ld[l], Wt[l], ld[l - 1], H[l], ld[l], n, C[l], C[l - 1]);
+    refresh_H1(keep_h1);
+    for (int l = 2; l <= L; ++l) refresh_H(l);
     fresh = true;
+  }
+  void refresh_H(int l, const int* skip = nullptr) {
+    gemm_nn(P[l], ld[l - 1], W[l], ld[l], Wt[l], ld[l - 1], H[l], ld[l], n, C[l], C[l - 1], skip);
+  }
+  void refresh_H1(bool keep_h1) {
+    const bool skip = keep_h1 && !capturing && h1_age + 1 < kH1RefreshEvery;
+    h1_age = skip ? h1_age + 1 : 0;
+    if (!skip) refresh_H(1, keep_h1 && capturing ? skip_h1 : nullptr);
+  }
+  void end_pass() {
+    Scope sc(this, "small", 1, 0.0, 0.0);
+    gk::k_end_pass<<<1, 1, 0, stream>>>(d_pass, d_h1_age, skip_h1, kH1RefreshEvery);
+    CU(cudaGetLastError());
+    ++log_count;
   }
 
   // The serial schedule of Section 4.1: the same block updates, one after the other in the order
@@ -788,22 +821,88 @@ struct gcn_admm {
       }
       update_W(l, false);
       if (l < L) update_Z_hidden(l, false);
-      else update_output(false, true, true);
+      else update_output(false, true);
     }
     refresh(true);
     dual_from_stored();
-    ++log_count;
+    end_pass();
+  }
+
+  // A second line of launches for what does not depend on the hidden layers: the W_L update and the output layer's rows read
+  // iterate k only (Jacobi), so on a graph too small to fill the chip they run beside W_1 .. W_{L-1} and Z_1 .. Z_{L-1} instead
+  // of between them.  It has a stream, the scratch of the products and sums, and matrices of the last layer's width of its own.
+  struct Lane {
+    cudaStream_t stream = nullptr;
+    float *part = nullptr, *grad = nullptr, *grad_t = nullptr;
+    size_t part_elems = 0;
+    uint8_t* b_image = nullptr;
+    double* red_part = nullptr;
+    unsigned *ticket = nullptr, *tile_tickets = nullptr;
+    cudaEvent_t begun = nullptr, w_done = nullptr, out_done = nullptr, done = nullptr;
+  } side;
+  bool two_lanes = false;
+  void swap_lane() {   // launches go to the other line until the next call
+    std::swap(stream, side.stream);
+    std::swap(part, side.part);
+    std::swap(part_elems, side.part_elems);
+    std::swap(grad, side.grad);
+    std::swap(grad_t, side.grad_t);
+    std::swap(b_image, side.b_image);
+    std::swap(red_part, side.red_part);
+    std::swap(ticket, side.ticket);
+    std::swap(tile_tickets, side.tile_tickets);
+  }
+
+  template <typename F>
+  void on_side(F&& launches_there) {
+    swap_lane();
+    try {
+      launches_there();
+    } catch (...) {
+      swap_lane();
+      throw;
+    }
+    swap_lane();
   }
 
   void iterate() {   // Algorithm 1, one pass
     if (p.schedule == 1) { iterate_sequential(); return; }
     if (!fresh) refresh();
-    for (int l = 1; l <= L; ++l) update_W(l, l >= 2);
-    for (int l = 1; l < L; ++l) update_Z_hidden(l, true);
-    update_output(p.dual_mode == 0, true, true);
-    refresh(true);
+    if (!two_lanes || profiling) {
+      for (int l = 1; l <= L; ++l) update_W(l, l >= 2);
+      for (int l = 1; l < L; ++l) update_Z_hidden(l, true);
+      update_output(p.dual_mode == 0, true);
+      refresh(true);
+    } else {
+      CU(cudaEventRecord(side.begun, stream));
+      CU(cudaStreamWaitEvent(side.stream, side.begun, 0));
+      on_side([&] {
+        update_W(L, true);
+        CU(cudaEventRecord(side.w_done, stream));
+        update_output(p.dual_mode == 0, true);
+        CU(cudaEventRecord(side.out_done, stream));
+      });
+      for (int l = 1; l < L; ++l) update_W(l, l >= 2);
+      for (int l = 1; l < L; ++l) {
+        if (l == L - 1) CU(cudaStreamWaitEvent(stream, side.w_done, 0));
+        update_Z_hidden(l, true);
+      }
+      CU(cudaEventRecord(side.begun, stream));
+      CU(cudaStreamWaitEvent(side.stream, side.begun, 0));
+      on_side([&] {
+        refresh_H1(true);
+        end_pass();
+        CU(cudaEventRecord(side.done, stream));
+      });
+      for (int l = 2; l <= L; ++l) spmm(Z[l - 1], P[l], ld[l - 1]);
+      CU(cudaStreamWaitEvent(stream, side.out_done, 0));   // its rows of H_L have been read
+      for (int l = 2; l <= L; ++l) refresh_H(l);
+      CU(cudaStreamWaitEvent(stream, side.done, 0));
+      if (p.dual_mode != 0) dual_from_stored();
+      return;
+    }
     if (p.dual_mode != 0) dual_from_stored();
-    ++log_count;
+    end_pass();
   }
 
   // logits of Problem 1's forward pass with the stored W, left in B0 (N x ld_L)
@@ -1135,7 +1234,24 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
   h->want(h->B0, rows * h->max_ld);
   h->want(h->B1, rows * h->max_ld);
   h->want(h->B2, rows * h->max_ld);
-  for (int l = 2; l < L; ++l) h->want(h->RN[l], rows * h->ld[l]);
+  for (int l = 2; l <= L; ++l) h->want(h->RN[l], rows * h->ld[l]);   // R_L is turned into its new value in place
+  if (L == 1) h->want(h->RN[1], rows * h->ld[1]);
+  h->want(h->DL, rows * h->ld[L]);
+  // a second line of launches where a pass is short enough for it to matter (the sizes that are recorded as graphs)
+  h->two_lanes = L >= 2 && n * (long long)h->max_ld < kSmallProblem;
+  if (h->two_lanes) {
+    const size_t ge = (size_t)h->C[L - 1] * h->ld[L];
+    h->side.part_elems = std::max<size_t>(ge, std::min<size_t>(std::max(ge * 4 * kSmCount, ge * (size_t)(cdiv(n, 2048) + kSmCount)), (size_t)64 << 20));
+    h->want(h->side.part, h->side.part_elems);
+    h->want(h->side.grad, ge);
+    h->want(h->side.grad_t, (size_t)h->C[L] * h->ld[L - 1], gcn_admm::kZero);
+    h->want(h->side.b_image, (size_t)16 << 20);
+    h->want(h->side.red_part, std::max<size_t>((size_t)kSmCount * 8 * gk::kCand, (size_t)cdiv((long long)ge, 32) * 2));
+    h->want(h->side.ticket, 1, gcn_admm::kZero);
+    h->want(h->side.tile_tickets, kSmCount, gcn_admm::kZero);
+    CU(gcn_admm_mem::Pool::get().take_stream(p.device, &h->side.stream));
+    for (cudaEvent_t* e : {&h->side.begun, &h->side.w_done, &h->side.out_done, &h->side.done}) CU(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
+  }
   h->item_sums_elems = std::max<size_t>(1, (size_t)h->n_items * h->max_ld);
   h->want(h->item_sums, h->item_sums_elems);
   h->want(h->grad, grad_elems);
@@ -1168,19 +1284,21 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
   h->want(h->z_group_part, (size_t)kChunkGroups * n_comm * gk::kCand);
   h->want(h->chunk_counter, 1, gcn_admm::kZero);
   h->want(h->ticket, 1, gcn_admm::kZero);
+  h->want(h->tile_tickets, kSmCount, gcn_admm::kZero);
   h->want(h->comm_tickets, n_comm, gcn_admm::kZero);
   h->want(h->grid_bar, 1, gcn_admm::kZero);
   h->want(h->red_part, std::max<size_t>({(size_t)kSmCount * 8 * gk::kCand, (size_t)h->n_zblocks * 3,
                                          (size_t)cdiv(n, 8) * 2, grad_blocks * 2}));
   h->want(h->n_active, 1, gcn_admm::kZero);
   h->want(h->d_pass, 1, gcn_admm::kZero);
+  h->want(h->d_h1_age, 1, gcn_admm::kZero);
+  h->want(h->skip_h1, 1, gcn_admm::kZero);
   h->want(h->log_trial_w, (size_t)kLogPasses * L);
   h->want(h->log_q_w, (size_t)kLogPasses * L);
   h->want(h->log_trial_z, (size_t)kLogPasses * std::max(L - 1, 0) * n_comm);
   h->want(h->log_q_z, (size_t)kLogPasses * std::max(L - 1, 0) * n_comm);
   h->commit();
   { gcn_admm_host::Table<unsigned short>().swap(h->gi.col_comm); }   // needed on the device only
-  if (L >= 2) h->RN[L] = h->B0;   // R_L is turned into its new value in place
   h->status = &h->report->status;
   h->tc_error = &h->report->error;
 
@@ -1299,6 +1417,12 @@ void gcn_admm_destroy(gcn_admm* h) {
     cudaStreamSynchronize(h->stream);
     h->collect_profile();
     if (h->pass_graph) cudaGraphExecDestroy(h->pass_graph);
+    if (h->side.stream) {
+      cudaStreamSynchronize(h->side.stream);
+      gcn_admm_mem::Pool::get().give_stream(h->p.device, h->side.stream);
+    }
+    for (cudaEvent_t e : {h->side.begun, h->side.w_done, h->side.out_done, h->side.done})
+      if (e) cudaEventDestroy(e);
     for (cudaEvent_t e : h->event_pool) cudaEventDestroy(e);
     for (const gcn_admm_mem::Slab& q : h->slabs) gcn_admm_mem::Pool::get().give(q);
     h->stage.close();
@@ -1317,10 +1441,13 @@ int gcn_admm_step(gcn_admm* h, int n_iters) {
     // A pass is a fixed sequence of launches (every decision is taken on the device), so on a stream
     // that can be captured it is recorded once and replayed: the small workloads are launch-bound.
     // use_graph 1: always; 2: only where a pass is short enough for launch overhead to matter
-    const bool wanted = h->p.use_graph == 1 || (h->p.use_graph == 2 && h->n * (long long)h->max_ld < (1LL << 27));
-    const bool replay = wanted && h->stream != nullptr && !h->profiling && n_iters >= 2;
+    const bool wanted = h->p.use_graph == 1 || (h->p.use_graph == 2 && h->n * (long long)h->max_ld < kSmallProblem);
+    // single passes are recorded once a few of them have been asked for: a loop that looks at the result after each
+    const bool replay = wanted && h->stream != nullptr && !h->profiling && n_iters >= 1 &&
+                        (n_iters >= 2 || h->pass_graph != nullptr || h->single_passes >= 2);
     if (!replay) {
       for (int k = 0; k < n_iters; ++k) h->iterate();
+      h->single_passes += n_iters;
       return;
     }
     if (!h->fresh) h->refresh();
@@ -1367,7 +1494,7 @@ int gcn_admm_step_block(gcn_admm* h, int phase, int layer) {
       h->update_W(layer, false);
     } else if (phase == GCN_ADMM_PHASE_Z) {
       if (layer < L) h->update_Z_hidden(layer, false);
-      else h->update_output(false, true, false);
+      else h->update_output(false, true);
       h->fresh = false;
     } else if (phase == GCN_ADMM_PHASE_U) {
       h->dual_from_stored();

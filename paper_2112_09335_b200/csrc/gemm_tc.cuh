@@ -171,7 +171,9 @@ struct WsCfg {
 // of 2 * NT * 128 bytes at block index g * chunks + kc.  With it (IMG = true) a stage's B tiles arrive
 // by one bulk copy issued by one thread, and the producers stage A only; without it they load, split
 // and store B again for every 128-row tile.
-__global__ void k_split_b(const float* __restrict__ Bk, int ldbk, int N, int K, int nt, uint8_t* __restrict__ image) {
+__global__ void k_split_b(const float* __restrict__ Bk, int ldbk, int N, int K, int nt, uint8_t* __restrict__ image,
+                          const int* __restrict__ skip) {
+  if (skip != nullptr && *skip) return;
   const int kc_count = (K + kChunkK - 1) / kChunkK;
   const int groups = (N + nt - 1) / nt;
   const long long total = (long long)groups * kc_count * nt * 8;
@@ -205,7 +207,7 @@ template <int NT, bool IMG, bool TMA = false>
 __global__ void __launch_bounds__(WsCfg<NT>::kThreads + (TMA ? 32 : 0), 1)
 k_gemm_tc_ws(const float* __restrict__ A, int lda, const float* __restrict__ Bk, int ldbk, float* __restrict__ C, int ldc,
              int M, int N, int K, const int* __restrict__ skip, int* __restrict__ error_flag,
-             const uint8_t* __restrict__ b_image, const __grid_constant__ CUtensorMap tmap_a) {
+             const uint8_t* __restrict__ b_image, const __grid_constant__ CUtensorMap tmap_a, float* partial, unsigned* tickets) {
   static_assert(!TMA || IMG, "the tensor-copy form stages no B tile");
   using Cfg = WsCfg<NT>;
   constexpr int S = TMA ? Cfg::kLoStages : Cfg::kStagesWs;   // stages of the ring the producers fill
@@ -219,7 +221,7 @@ k_gemm_tc_ws(const float* __restrict__ A, int lda, const float* __restrict__ Bk,
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t bars[2 * S + 4 + 2 * R];      // full[S], empty[S], acc_full[2], acc_empty[2], raw_full[R], raw_empty[R]
   __shared__ uint32_t tmem_base_slot;
-  __shared__ int abort_flag;
+  __shared__ int abort_flag, last_part;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t smem_base = smem_u32(smem);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -251,7 +253,10 @@ k_gemm_tc_ws(const float* __restrict__ A, int lda, const float* __restrict__ Bk,
   const uint32_t tmem_base = tmem_base_slot;
   volatile int* abortp = &abort_flag;
 
-  const int kc_count = (K + kChunkK - 1) / kChunkK;
+  const int kc_all = (K + kChunkK - 1) / kChunkK;
+  // gridDim.z CTAs share a tile's reduction (few row tiles, many K chunks): this one walks chunks kc0 .. kc0 + kc_count - 1
+  const int kc0 = (int)((long long)kc_all * blockIdx.z / gridDim.z);
+  const int kc_count = (int)((long long)kc_all * (blockIdx.z + 1) / gridDim.z) - kc0;
   const int n_tiles = (M + kBlockM - 1) / kBlockM;
   const int my_tiles = (n_tiles > (int)blockIdx.x) ? (n_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
   const int total = my_tiles * kc_count;
@@ -268,7 +273,7 @@ k_gemm_tc_ws(const float* __restrict__ A, int lda, const float* __restrict__ Bk,
     long long ld_row0 = (long long)blockIdx.x * kBlockM;
     auto load_chunk = [&](float4* pa, float4* pb) {
       if (ld_j >= total) return;
-      const int k0 = ld_kc * kChunkK + ld_c16 * 4;
+      const int k0 = (kc0 + ld_kc) * kChunkK + ld_c16 * 4;
       const long long row0 = ld_row0;
       ++ld_j;
       if (++ld_kc == kc_count) { ld_kc = 0; ld_row0 += (long long)gridDim.x * kBlockM; }
@@ -359,7 +364,7 @@ k_gemm_tc_ws(const float* __restrict__ A, int lda, const float* __restrict__ Bk,
           // the stage is free (its MMAs have retired): fetch both B tiles of this chunk with one bulk copy
           // that reports its bytes to the stage's full barrier; this thread's own arrival comes below
           const uint32_t bytes = 2u * (uint32_t)Cfg::kBTile;
-          const uint8_t* src = b_image + ((size_t)blockIdx.y * kc_count + (size_t)st_kc) * bytes;
+          const uint8_t* src = b_image + ((size_t)blockIdx.y * kc_all + (size_t)(kc0 + st_kc)) * bytes;
           const uint32_t dst = smem_base + (uint32_t)stage * Cfg::kStage + 2u * kATileBytes;
           asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar_full + 8 * stage), "r"(bytes) : "memory");
           asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
@@ -378,7 +383,7 @@ k_gemm_tc_ws(const float* __restrict__ A, int lda, const float* __restrict__ Bk,
     // ---------------- copies (tensor-copy form only): A tile and weight tiles of chunk j as soon as slot j mod R is free ----------------
     if (lane == 0) {
       const uint32_t b_bytes = 2u * (uint32_t)Cfg::kBTile;
-      const uint8_t* const b_src = b_image + (size_t)blockIdx.y * kc_count * b_bytes;
+      const uint8_t* const b_src = b_image + ((size_t)blockIdx.y * kc_all + (size_t)kc0) * b_bytes;
       int kc = 0, tile = blockIdx.x, slot = 0;
       uint32_t empty_parity = 1;   // a fresh barrier passes a wait on parity 1
       for (int j = 0; j < total; ++j) {
@@ -387,7 +392,7 @@ k_gemm_tc_ws(const float* __restrict__ A, int lda, const float* __restrict__ Bk,
         const uint32_t raw_bar = bar_raw_full + 8 * slot;
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(raw_bar), "r"((uint32_t)kATileBytes + b_bytes) : "memory");
         asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-                     ::"r"(dst_a), "l"(&tmap_a), "r"(kc * kChunkK), "r"(tile * kBlockM), "r"(raw_bar)
+                     ::"r"(dst_a), "l"(&tmap_a), "r"((kc0 + kc) * kChunkK), "r"(tile * kBlockM), "r"(raw_bar)
                      : "memory");
         asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                      ::"r"(dst_a + (uint32_t)kATileBytes), "l"(b_src + (size_t)kc * b_bytes), "r"(b_bytes), "r"(raw_bar)
@@ -456,6 +461,7 @@ k_gemm_tc_ws(const float* __restrict__ A, int lda, const float* __restrict__ Bk,
     constexpr int ROWS_PER_STORE = 32 / SLOTS;
     const int turn = (warp - 8) >> 2;                  // which of the quarter's two warps this is
     uint8_t* tbuf = smem + kRingBytes + (size_t)(warp - 8) * 4096;
+    float* const dst = gridDim.z == 1 ? C : partial + (size_t)blockIdx.z * M * ldc;
     for (int tile_i = 0; tile_i < my_tiles; ++tile_i) {
       const int set = tile_i % SETS;
       if (!__all_sync(0xffffffffu, mbar_wait_abortable(bar_acc_full + 8 * set, (tile_i / SETS) & 1, abortp))) break;
@@ -487,12 +493,36 @@ k_gemm_tc_ws(const float* __restrict__ A, int lda, const float* __restrict__ Bk,
         for (int i = 0; i < SLOTS; ++i) {
           const int r = i * ROWS_PER_STORE + lane / SLOTS;
           const float4 val = *reinterpret_cast<const float4*>(tbuf + r * 128 + ((c4 ^ (r & (SLOTS - 1))) * 16));
-          if (row0 + r < M && col < ldc) *reinterpret_cast<float4*>(C + (row0 + r) * ldc + col) = val;
+          if (row0 + r < M && col < ldc) *reinterpret_cast<float4*>(dst + (row0 + r) * ldc + col) = val;
         }
         __syncwarp();
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       mbar_arrive_warp(bar_acc_empty + 8 * set);
+      if (gridDim.z > 1) {   // the last CTA of the tile adds the parts up, in order of their K ranges
+        constexpr int kEpiThreads = Cfg::kEpiWarps * 32;
+        const int et = tid - 256;
+        const int tile = blockIdx.x + tile_i * gridDim.x;
+        __threadfence();
+        asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory");
+        if (et == 0) last_part = atomicAdd(tickets + tile * gridDim.y + blockIdx.y, 1u) == gridDim.z - 1;
+        asm volatile("bar.sync 1, %0;" ::"n"(kEpiThreads) : "memory");
+        if (last_part) {
+          __threadfence();
+          if (et == 0) tickets[tile * gridDim.y + blockIdx.y] = 0;
+          for (int i = et; i < kBlockM * (NT / 4); i += kEpiThreads) {
+            const long long r = (long long)tile * kBlockM + i / (NT / 4);
+            const int col = n0 + (i % (NT / 4)) * 4;
+            if (r >= M || col >= ldc) continue;
+            float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (unsigned z = 0; z < gridDim.z; ++z) {
+              const float4 v = __ldcg(reinterpret_cast<const float4*>(partial + ((size_t)z * M + r) * ldc + col));
+              sum.x += v.x; sum.y += v.y; sum.z += v.z; sum.w += v.w;
+            }
+            *reinterpret_cast<float4*>(C + r * ldc + col) = sum;
+          }
+        }
+      }
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");

@@ -932,8 +932,10 @@ k_finish_grad(const float* __restrict__ part, int splits, int rows, int cols, in
 
 // Search and move of a W block.  Along W - grad/t the pre-activation is H - D/t with D = P grad, so every candidate is
 // scored from H, D, Z without another product:
-//   hidden layer: sum_j = sum ( (z - f(h - d/t_j))^2 - (z - f(h))^2 )   (times nu/2 at decision time), kCand trials a sweep
-//   last layer:   phi_L(t) - phi_L = -(1/t) <D, R> + (rho / 2t^2) ||D||^2 : two sums decide every trial
+//   hidden layer: sum_j = sum ( (z - f(h - d/t_j))^2 - (z - f(h))^2 )   (times nu/2 at decision time), kCand trials a sweep;
+//                 one cooperative launch, k_search_w_hidden
+//   last layer:   phi_L(t) - phi_L = -(1/t) <D, R> + (rho / 2t^2) ||D||^2 : two sums decide every trial, taken by the last
+//                 block of k_score_w_out; k_move_w_out follows (ordinary launches: this chain runs beside the hidden layers')
 // Then W <- W - grad/tau (and its transpose), H <- H - D/tau and, where Rn is given, the derivative of phi_l at the new
 // H, which the gradient of Z_{l-1} starts from (formed here it costs one array less than in a sweep of its own).
 struct SearchW {
@@ -948,71 +950,18 @@ struct SearchW {
   SearchCtl* ctl;
   double* partial;                  // kCand (2) per block
   GridBar* bar;
+  unsigned* ticket;
   int *status, *err;
   DecideArgs a;
   DecisionLog log;
 };
+
 template <bool OUT>
-__global__ void __launch_bounds__(256, 4)
-k_search_w(const SearchW p) {
-  constexpr int PER = OUT ? 2 : kCand;
-  __shared__ double sh[PER * 8], total[PER];
-  SearchCtl* const ctl = p.ctl;
+__device__ __forceinline__ void move_w(const SearchW& p, float step) {
   const long long first = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
-  if (ctl->done) {                  // skipped: the same in every block
-    if (first == 0) log_decision(p.log, 0, ctl);
-  } else {
-    bool open = true;
-    while (open) {
-      double s[PER];
-#pragma unroll
-      for (int j = 0; j < PER; ++j) s[j] = 0.0;
-      if (OUT) {
-        for (long long i = first; i < p.n4; i += stride) {
-          const float4 d = p.D[i], r = p.R[i];
-          s[0] += (double)(d.x * r.x + d.y * r.y + d.z * r.z + d.w * r.w);
-          s[1] += (double)(d.x * d.x + d.y * d.y + d.z * d.z + d.w * d.w);
-        }
-      } else {
-        float inv[kCand];
-#pragma unroll
-        for (int j = 0; j < kCand; ++j) inv[j] = __ldcg(&ctl->inv_cand[j]);
-        for (long long i = first; i < p.n4; i += stride) {
-          const float4 h4 = p.H[i], d4 = p.D[i], z4 = p.Z[i];
-          const float h[4] = {h4.x, h4.y, h4.z, h4.w}, d[4] = {d4.x, d4.y, d4.z, d4.w}, z[4] = {z4.x, z4.y, z4.z, z4.w};
-          float part[kCand];
-#pragma unroll
-          for (int j = 0; j < kCand; ++j) part[j] = 0.f;
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            const float pos = fmaxf(h[c], 0.f), neg = fmaxf(-h[c], 0.f);
-            const float e2 = 2.f * (z[c] - pos);
-#pragma unroll
-            for (int j = 0; j < kCand; ++j) {
-              const float df = relu_drop(d[c], inv[j], neg, pos);
-              part[j] = fmaf(df, e2 + df, part[j]);   // e1^2 - e0^2 = (e1 - e0)(e1 + e0), e1 - e0 = df
-            }
-          }
-#pragma unroll
-          for (int j = 0; j < kCand; ++j) s[j % PER] += (double)part[j];
-        }
-      }
-      block_sums(s, sh);
-      if (threadIdx.x == 0)
-#pragma unroll
-        for (int j = 0; j < PER; ++j) p.partial[(size_t)blockIdx.x * PER + j] = s[j];
-      const bool ok = grid_meet(p.bar, p.err, [&] {
-        add_block_sums<PER>(p.partial, (int)gridDim.x, total);
-        if (threadIdx.x < 32 && !decide_one(ctl, total, 0.0, p.a, nullptr, p.status) && threadIdx.x == 0) log_decision(p.log, 0, ctl);
-      });
-      if (!ok) return;
-      open = __ldcg(&ctl->done) == 0;
-    }
-  }
-  const float step = __ldcg(&ctl->inv_step);
   if (step != 0.f)
-    for (long long e = first; e < (long long)p.rows * p.cols; e += stride) {
-      const int r = (int)(e / p.cols), c = (int)(e - (long long)r * p.cols);
+    for (long long e = first; e < (long long)p.rows * p.cols; e += stride) {   // a weight matrix: below 2^32
+      const int r = (int)((unsigned)e / (unsigned)p.cols), c = (int)((unsigned)e - (unsigned)r * (unsigned)p.cols);
       const float w = fmaf(-p.grad[(long long)r * p.ldw + c], step, p.W[(long long)r * p.ldw + c]);
       p.W[(long long)r * p.ldw + c] = w;
       p.Wt[(long long)c * p.ldwt + r] = w;
@@ -1021,12 +970,106 @@ k_search_w(const SearchW p) {
   for (long long i = first; i < p.n4; i += stride) {
     float4 h = p.H[i];
     if (step != 0.f) {
-      const float4 d = p.D[i];
-      h.x = fmaf(-step, d.x, h.x); h.y = fmaf(-step, d.y, h.y); h.z = fmaf(-step, d.z, h.z); h.w = fmaf(-step, d.w, h.w);
+      h = vfma(-step, p.D[i], h);
       p.H[i] = h;
     }
     if (p.Rn != nullptr) p.Rn[i] = OUT ? resid_out(h, p.Z[i], p.U[i], p.coef) : resid_hidden(h, p.Z[i], p.coef);
   }
+}
+
+__global__ void __launch_bounds__(256, 4)
+k_search_w_hidden(const SearchW p) {
+  __shared__ double sh[kCand * 8], total[kCand];
+  SearchCtl* const ctl = p.ctl;
+  const long long first = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
+  if (ctl->done) {                  // skipped: the same in every block
+    if (first == 0) log_decision(p.log, 0, ctl);
+  } else {
+    bool open = true;
+    while (open) {
+      double s[kCand];
+#pragma unroll
+      for (int j = 0; j < kCand; ++j) s[j] = 0.0;
+      float inv[kCand];
+#pragma unroll
+      for (int j = 0; j < kCand; ++j) inv[j] = __ldcg(&ctl->inv_cand[j]);
+      for (long long i = first; i < p.n4; i += stride) {
+        const float4 h4 = p.H[i], d4 = p.D[i], z4 = p.Z[i];
+        const float h[4] = {h4.x, h4.y, h4.z, h4.w}, d[4] = {d4.x, d4.y, d4.z, d4.w}, z[4] = {z4.x, z4.y, z4.z, z4.w};
+        float part[kCand];
+#pragma unroll
+        for (int j = 0; j < kCand; ++j) part[j] = 0.f;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const float pos = fmaxf(h[c], 0.f), neg = fmaxf(-h[c], 0.f);
+          const float e2 = 2.f * (z[c] - pos);
+#pragma unroll
+          for (int j = 0; j < kCand; ++j) {
+            const float df = relu_drop(d[c], inv[j], neg, pos);
+            part[j] = fmaf(df, e2 + df, part[j]);   // e1^2 - e0^2 = (e1 - e0)(e1 + e0), e1 - e0 = df
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < kCand; ++j) s[j] += (double)part[j];
+      }
+      block_sums(s, sh);
+      if (threadIdx.x == 0)
+#pragma unroll
+        for (int j = 0; j < kCand; ++j) p.partial[(size_t)blockIdx.x * kCand + j] = s[j];
+      const bool ok = grid_meet(p.bar, p.err, [&] {
+        add_block_sums<kCand>(p.partial, (int)gridDim.x, total);
+        if (threadIdx.x < 32 && !decide_one(ctl, total, 0.0, p.a, nullptr, p.status) && threadIdx.x == 0) log_decision(p.log, 0, ctl);
+      });
+      if (!ok) return;
+      open = __ldcg(&ctl->done) == 0;
+    }
+  }
+  move_w<false>(p, __ldcg(&ctl->inv_step));
+}
+
+__global__ void __launch_bounds__(256)
+k_score_w_out(const SearchW p) {
+  __shared__ double sh[16], total[2];
+  __shared__ int s_last;
+  if (p.ctl->done) {                // skipped: the same in every block
+    if (blockIdx.x == 0 && threadIdx.x == 0) log_decision(p.log, 0, p.ctl);
+    return;
+  }
+  double s[2] = {0.0, 0.0};
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < p.n4; i += (long long)gridDim.x * blockDim.x) {
+    const float4 d = p.D[i], r = p.R[i];
+    s[0] += (double)(d.x * r.x + d.y * r.y + d.z * r.z + d.w * r.w);
+    s[1] += (double)(d.x * d.x + d.y * d.y + d.z * d.z + d.w * d.w);
+  }
+  block_sums(s, sh);
+  if (threadIdx.x == 0) {
+    p.partial[(size_t)blockIdx.x * 2] = s[0];
+    p.partial[(size_t)blockIdx.x * 2 + 1] = s[1];
+    __threadfence();
+    s_last = atomicAdd(p.ticket, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  add_block_sums<2>(p.partial, (int)gridDim.x, total);
+  if (threadIdx.x >= 32) return;
+  decide_one(p.ctl, total, 0.0, p.a, nullptr, p.status);
+  if (threadIdx.x == 0) {
+    *p.ticket = 0;
+    log_decision(p.log, 0, p.ctl);
+  }
+}
+
+__global__ void __launch_bounds__(256)
+k_move_w_out(const SearchW p) { move_w<true>(p, p.ctl->inv_step); }
+
+// The end of a pass: the pass counter of the log moves on, and with it the count of passes since H_1 was last formed afresh
+// (*skip_h1 = 1 while H_1, which the W_1 update keeps equal to P_1 W_1 up to rounding, need not be).
+__global__ void k_end_pass(int* __restrict__ pass, int* __restrict__ h1_age, int* __restrict__ skip_h1, int every) {
+  *pass += 1;
+  const int age = *skip_h1 ? *h1_age + 1 : 0;   // the pass that has just ended formed H_1 unless *skip_h1 said not to
+  *h1_age = age;
+  *skip_h1 = age + 1 < every;
 }
 
 // Marks every entry of the current pass's slot as "not run".
@@ -1817,8 +1860,7 @@ k_move_z(float4* __restrict__ Z, const float4* __restrict__ G, int ld4, long lon
 // iteration then take log2(LPR) shuffles for 32 / LPR rows at once.  91 k rows x 40 classes x 30 iterations: a warp per row
 // 255 us, 8 lanes per row 95 us.  The other blocks sweep the remaining rows elementwise.
 // momentum[j] = (t_j - 1) / t_{j+1} of FISTA's sequence t_1 = 1, t_{j+1} = (1 + sqrt(1 + 4 t_j^2)) / 2: the same for every
-// row, so it is tabulated once (in fp64).  `advance` (may be NULL): the pass counter of the decision log, counted up by
-// this last kernel of a pass.
+// row, so it is tabulated once (in fp64).
 // ------------------------------------------------------------------------------------------
 struct OutputArgs {
   float *Z, *U;
@@ -1831,12 +1873,10 @@ struct OutputArgs {
   const float* momentum;
   float rho, loss_scale;
   int iters, dual_now, update_z;
-  int* advance;
 };
 template <int LPR, int CPL>
 __global__ void __launch_bounds__(256)
 k_output(const OutputArgs p) {
-  if (p.advance != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *p.advance += 1;
   if ((int)blockIdx.x >= p.train_blocks) {
     const int ld4 = p.ld / 4;
     float4* const Z4 = reinterpret_cast<float4*>(p.Z);

@@ -6,7 +6,7 @@
 // driver too.  Copies between the device and pageable host memory go through the driver's own staging on one core at
 // 5-10 GB/s; here several cores fill or drain one part of the staging buffer while the copy engine works on the next.
 //
-// Slabs and staging buffers of destroyed handles are kept for later ones up to a fixed amount (kIdleSlabBytes,
+// Slabs, staging buffers and streams of destroyed handles are kept for later ones up to a fixed amount (kIdleSlabBytes,
 // kIdleStages; the oldest go first), under a lock, and only after the work that used them has finished; the rest goes back
 // to the driver at once, everything at exit or when an allocation fails.
 #pragma once
@@ -16,6 +16,7 @@
 #include <cstddef>
 #include <cstring>
 #include <mutex>
+#include <utility>
 #include <vector>
 
 namespace gcn_admm_mem {
@@ -105,9 +106,30 @@ class Pool {
     }
     cudaFreeHost(p);
   }
+  // A non-blocking stream of the current device (`device`); given back when nothing is in flight on it.
+  cudaError_t take_stream(int device, cudaStream_t* out) {
+    {
+      std::lock_guard<std::mutex> lock(mutex_);
+      for (auto it = streams_.begin(); it != streams_.end(); ++it)
+        if (it->first == device) {
+          *out = it->second;
+          streams_.erase(it);
+          return cudaSuccess;
+        }
+    }
+    return cudaStreamCreateWithFlags(out, cudaStreamNonBlocking);
+  }
+  void give_stream(int device, cudaStream_t s) {
+    {
+      std::lock_guard<std::mutex> lock(mutex_);
+      if (streams_.size() < kIdleStages) { streams_.push_back({device, s}); return; }
+    }
+    cudaStreamDestroy(s);
+  }
   ~Pool() {   // at exit the driver may already be gone: its error is of no consequence then
     for (const Slab& s : idle_) cudaFree(s.base);
     for (char* p : stages_) cudaFreeHost(p);
+    for (const auto& s : streams_) cudaStreamDestroy(s.second);
   }
 
  private:
@@ -125,6 +147,7 @@ class Pool {
   std::vector<Slab> idle_;
   std::size_t idle_bytes_ = 0;
   std::vector<char*> stages_;
+  std::vector<std::pair<int, cudaStream_t>> streams_;
 };
 
 // memcpy by several threads where it pays (a core moves about 10 GB/s, less into pages that are touched first here).
