@@ -208,7 +208,8 @@ struct gcn_admm {
   float* grad = nullptr;     // max over l of C_{l-1} x ld_l
   float* grad_t = nullptr;   // its transpose, C_l x ld_{l-1} (K-major operand of the tensor-core product)
   int* tc_error = nullptr;   // &report->error: raised by a tensor-core product (1) or a search (2) whose bounded wait ran out
-  uint8_t* b_image = nullptr;   // split weight operand in the staged layout (see gtc::k_split_b)
+  uint8_t* b_image = nullptr;   // split operand of a product without a kept image (see gtc::k_split_b)
+  std::vector<gtc::Image> img_H, img_G, img_D;   // 1..L: kept images of W_l for P_l W_l, of W_l for S W_l^T, of the gradient for P_l grad
   size_t b_image_bytes = 0;
   float* part = nullptr;     // split partial sums of the transposed product
   size_t part_elems = 0;
@@ -392,64 +393,84 @@ struct gcn_admm {
     }
   }
 
-  // C = A B.  B is handed over twice: row-major K x N (ldb) for the fp32-ALU kernels and K-major
-  // N x K (Bk, ldbk; may be NULL) for the tensor-core kernel, which is used whenever it applies
-  // (K capped at 2048 because its accumulator error grows with K, about 2.5e-9 K of the magnitude).
+  // Whether C = A B with these sizes runs on the tensor cores (K capped at 2048 because the accumulator error grows with K,
+  // about 2.5e-9 K of the magnitude), and how: columns per group, and whether B is taken from an image of the staged layout.
+  bool on_tensor_cores(long long Mr, int K) const { return p.tensor_cores && K >= 8 && K <= 2048 && Mr >= 512; }
+  int group_width(long long Mr, int N, int K, int lda) const {
+    if (N <= 16) return 16;
+    if (N <= 32) return 32;
+    if (N <= 48) return 48;
+    if (N <= 64) return 64;
+    if (N <= 128) return 128;
+    // 129..256 columns with a short reduction (K <= 128: a tile has at most four chunks of MMAs, so the epilogue
+    // that the single accumulator set of the 256-column form leaves uncovered dominates): two groups of 128 columns
+    // in the tensor-copy form instead, whose two accumulator sets put the epilogue under the next tile's MMAs
+    // (measured on 1.2 M rows: 0.372 -> 0.326 ms at K = 47, 0.560 -> 0.463 at 100, 0.518 -> 0.456 at 128; no gain at 256)
+    return K <= 128 && lda >= gtc::kChunkK && Mr >= kImageMinRows ? 128 : 256;
+  }
+  // With many row tiles the producers would split the same weights again for every tile; with at most one tile per CTA, or
+  // with few chunks, that costs nothing (13.8 k rows, 767 x 1000, three tiles per CTA: 130 -> 98 us; 10 x 1000: no gain).
+  bool takes_image(long long Mr, int N, int K, int nt) const {
+    return p.tensor_cores == 2 || Mr >= kImageMinRows || (K >= 128 && cdiv(Mr, gtc::kBlockM) > kSmCount / cdiv(N, nt));
+  }
+  static size_t image_bytes(int N, int K, int nt) { return (size_t)cdiv(N, nt) * cdiv(K, gtc::kChunkK) * 2 * nt * gtc::kChunkK * 4; }
+  // Asks for a kept image of the operand of an n x K by K x N product, where that product takes one.
+  void want_image(gtc::Image& im, int N, int K, int lda) {
+    im = gtc::Image{nullptr, group_width(n, N, K, lda), (int)cdiv(K, gtc::kChunkK)};
+    if (on_tensor_cores(n, K) && takes_image(n, N, K, im.nt)) want(im.data, image_bytes(N, K, im.nt), kZero);
+  }
+
+  // C = A B.  B is handed over twice: row-major K x N (ldb) for the fp32-ALU kernels and K-major N x K (Bk, ldbk; may be
+  // NULL) for the tensor-core kernel, which is used whenever it applies; `kept`: its image, where one is kept.
   void gemm_nn(const float* A, int lda, const float* B, int ldb, const float* Bk, int ldbk, float* Cm, int ldc,
-               long long Mr, int N, int K, const int* skip = nullptr) {
+               long long Mr, int N, int K, const gtc::Image* kept = nullptr, const int* skip = nullptr) {
     char name[48];
-    if (p.tensor_cores && Bk != nullptr && K >= 8 && K <= 2048 && Mr >= 512) {
+    if (Bk != nullptr && on_tensor_cores(Mr, K)) {
       std::snprintf(name, sizeof name, "gemm_tc@%dx%d", K, N);
       Scope sc(this, name, 1, 4.0 * ((double)Mr * (lda + ldc) + (double)K * ldb), 2.0 * (double)Mr * N * K);
-      const int tiles = (int)cdiv(Mr, gtc::kBlockM);
+      const int tiles = (int)cdiv(Mr, gtc::kBlockM), nt = group_width(Mr, N, K, lda), groups = (int)cdiv(N, nt), kc = (int)cdiv(K, gtc::kChunkK);
+      dim3 grid((unsigned)std::max(1, std::min(tiles, kSmCount / groups)), (unsigned)groups);
       CUtensorMap tmap;
       std::memset(&tmap, 0, sizeof tmap);
-      // With many row tiles the weight operand is split once into an image of the staged layout and
-      // fetched by bulk copies; with few (launch-bound problems) the extra launch costs more than the
-      // producers' repeated work.  tensor_cores = 2 takes the image at every size.
-#define TC_WS(NT)                                                                                              \
-  {                                                                                                            \
-    const size_t smem = gtc::WsCfg<NT>::kSmem;                                                                 \
-    const int groups = (int)cdiv(N, NT);                                                                       \
-    const size_t image_bytes = (size_t)groups * cdiv(K, gtc::kChunkK) * 2 * (NT) * gtc::kChunkK * 4;            \
-    dim3 grid((unsigned)std::max(1, std::min(tiles, kSmCount / groups)), (unsigned)groups);                    \
-    if ((p.tensor_cores == 2 || Mr >= kImageMinRows) && image_bytes <= b_image_bytes) {                        \
-      const long long work = (long long)groups * cdiv(K, gtc::kChunkK) * (NT) * 8;                             \
-      gtc::k_split_b<<<(unsigned)std::min<long long>(cdiv(work, 256), 4 * kSmCount), 256, 0, stream>>>(Bk, ldbk, N, K, NT, b_image, skip); \
-      ++launches;                                                                                              \
-      /* up to 128 columns: A tiles by tensor copies into a ring of their own (at 256 columns shared memory    \
-         leaves no room for it, and the form measured no faster there) */                                      \
-      if ((NT) <= 128 && make_a_tile_map(A, Mr, lda, &tmap)) {                                                 \
-        const size_t smem_ring = gtc::WsCfg<NT>::kSmemRing;                                                    \
-        CU(cudaFuncSetAttribute(gtc::k_gemm_tc_ws<NT, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_ring)); \
-        gtc::k_gemm_tc_ws<NT, true, true><<<grid, gtc::WsCfg<NT>::kThreads + 32, smem_ring, stream>>>(A, lda, Bk, ldbk, Cm, ldc, (int)Mr, N, K, skip, tc_error, b_image, tmap, nullptr, nullptr); \
-      } else {                                                                                                 \
-        CU(cudaFuncSetAttribute(gtc::k_gemm_tc_ws<NT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
-        gtc::k_gemm_tc_ws<NT, true><<<grid, gtc::WsCfg<NT>::kThreads, smem, stream>>>(A, lda, Bk, ldbk, Cm, ldc, (int)Mr, N, K, skip, tc_error, b_image, tmap, nullptr, nullptr); \
-      }                                                                                                        \
-    } else {                                                                                                   \
-      /* few row tiles and a long reduction: several CTAs share a tile's K chunks, at least four chunks each          \
-         (2.7 k rows, K = 1433, 16 columns: 34 -> 13 us) */                                                       \
-      const int kc = (int)cdiv(K, gtc::kChunkK);                                                               \
-      const int ways = (int)std::max<long long>(1, std::min<long long>({kSmCount / ((long long)tiles * groups), kc / 4, \
-                                                                        (long long)(part_elems / ((size_t)Mr * ldc))})); \
-      grid.z = (unsigned)ways;                                                                                 \
-      CU(cudaFuncSetAttribute(gtc::k_gemm_tc_ws<NT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
-      gtc::k_gemm_tc_ws<NT, false><<<grid, gtc::WsCfg<NT>::kThreads, smem, stream>>>(A, lda, Bk, ldbk, Cm, ldc, (int)Mr, N, K, skip, tc_error, nullptr, tmap, part, tile_tickets); \
-    }                                                                                                          \
-  }
-      if (N <= 16) TC_WS(16)
-      else if (N <= 32) TC_WS(32)
-      else if (N <= 48) TC_WS(48)
-      else if (N <= 64) TC_WS(64)
-      else if (N <= 128) TC_WS(128)
-      // 129..256 columns with a short reduction (K <= 128: a tile has at most four chunks of MMAs, so the epilogue
-      // that the single accumulator set of the 256-column form leaves uncovered dominates): two groups of 128 columns
-      // in the tensor-copy form instead, whose two accumulator sets put the epilogue under the next tile's MMAs
-      // (measured on 1.2 M rows: 0.372 -> 0.326 ms at K = 47, 0.560 -> 0.463 at 100, 0.518 -> 0.456 at 128; no gain at 256)
-      else if (K <= 128 && lda >= gtc::kChunkK && Mr >= kImageMinRows) TC_WS(128)
-      else TC_WS(256)
-#undef TC_WS
+      const uint8_t* image = nullptr;
+      if (takes_image(Mr, N, K, nt)) {
+        if (kept != nullptr && kept->data != nullptr) image = kept->data;
+        else if (image_bytes(N, K, nt) <= b_image_bytes) {
+          gtc::k_split_b<<<(unsigned)std::min<long long>(cdiv((long long)groups * kc * nt * 8, 256), 4 * kSmCount), 256, 0, stream>>>(Bk, ldbk, N, K, nt, b_image);
+          CU(cudaGetLastError());
+          ++launches;
+          image = b_image;
+        }
+      }
+      // few row tiles and a long reduction: several CTAs share a tile's K chunks, at least four chunks each
+      // (2.7 k rows, K = 1433, 16 columns: 34 -> 13 us)
+      if (image == nullptr)
+        grid.z = (unsigned)std::max<long long>(1, std::min<long long>({kSmCount / ((long long)tiles * groups), kc / 4,
+                                                                       (long long)(part_elems / ((size_t)Mr * ldc))}));
+      // an image and up to 128 columns: A tiles by tensor copies into a ring of their own (at 256 columns shared memory
+      // leaves no room for it, and the form measured no faster there)
+      const bool copies = image != nullptr && nt <= 128 && make_a_tile_map(A, Mr, lda, &tmap);
+      auto launch = [&](auto kernel, int threads, size_t smem) {
+        CU(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        kernel<<<grid, threads, smem, stream>>>(A, lda, Bk, ldbk, Cm, ldc, (int)Mr, N, K, skip, tc_error, image, tmap, part, tile_tickets);
+      };
+      auto with_width = [&](auto width) {
+        constexpr int NT = decltype(width)::value;
+        using Cfg = gtc::WsCfg<NT>;
+        if constexpr (NT <= 128) {
+          if (copies) { launch(gtc::k_gemm_tc_ws<NT, true, true>, Cfg::kThreads + 32, Cfg::kSmemRing); return; }
+        }
+        if (image != nullptr) launch(gtc::k_gemm_tc_ws<NT, true, false>, Cfg::kThreads, Cfg::kSmem);
+        else launch(gtc::k_gemm_tc_ws<NT, false, false>, Cfg::kThreads, Cfg::kSmem);
+      };
+      switch (nt) {
+        case 16: with_width(std::integral_constant<int, 16>()); break;
+        case 32: with_width(std::integral_constant<int, 32>()); break;
+        case 48: with_width(std::integral_constant<int, 48>()); break;
+        case 64: with_width(std::integral_constant<int, 64>()); break;
+        case 128: with_width(std::integral_constant<int, 128>()); break;
+        default: with_width(std::integral_constant<int, 256>());
+      }
       CU(cudaGetLastError());
       return;
     }
@@ -540,15 +561,16 @@ struct gcn_admm {
   }
 
   // grad (and grad_t) from the `splits` partial sums gemm_tn left in `part`; with `ctl` the start of the W_l search too.
-  void finish_grad(int splits, int Ka, int Nb, int ldp, float* out, float* out_t, int ldt, const float* w, SearchCtl* ctl) {
+  void finish_grad(int splits, int Ka, int Nb, int ldp, float* out, float* out_t, int ldt, const float* w, SearchCtl* ctl,
+                   const gtc::Image& image) {
     Scope sc(this, "finish_grad", 1, 4.0 * (double)Ka * ldp * (splits + (w ? 3 : 1)), 0.0);
     const long long elems = (long long)Ka * ldp;
     if (splits >= 16)
       gk::k_finish_grad<8><<<(unsigned)cdiv(elems, 32), 256, 0, stream>>>(part, splits, Ka, Nb, ldp, out, out_t, ldt, w, red_part,
-                                                                            ticket, ctl, p.bt_shrink, p.bt_growth, status);
+                                                                            ticket, ctl, p.bt_shrink, p.bt_growth, status, image);
     else
       gk::k_finish_grad<1><<<(unsigned)cdiv(elems, 256), 256, 0, stream>>>(part, splits, Ka, Nb, ldp, out, out_t, ldt, w, red_part,
-                                                                                     ticket, ctl, p.bt_shrink, p.bt_growth, status);
+                                                                                     ticket, ctl, p.bt_shrink, p.bt_growth, status, image);
     CU(cudaGetLastError());
   }
 
@@ -615,14 +637,14 @@ struct gcn_admm {
       resid(l, R);                                                      // R_l
       splits = gemm_tn(P[l], ld[l - 1], R, ldc, ldc, n, Kp, Cn);        // grad = P_l^T R_l
     }
-    finish_grad(splits, Kp, Cn, ldc, grad, grad_t, ld[l - 1], W[l], ctl);
-    gemm_nn(P[l], ld[l - 1], grad, ldc, grad_t, ld[l - 1], D, ldc, n, Cn, Kp, &ctl->done);   // D = P_l grad
+    finish_grad(splits, Kp, Cn, ldc, grad, grad_t, ld[l - 1], W[l], ctl, img_D[l]);
+    gemm_nn(P[l], ld[l - 1], grad, ldc, grad_t, ld[l - 1], D, ldc, n, Cn, Kp, &img_D[l], &ctl->done);   // D = P_l grad
     gk::SearchW a{};
     a.H = (float4*)H[l]; a.D = (const float4*)D; a.Z = (const float4*)Z[l]; a.U = (const float4*)U; a.R = (const float4*)R;
     a.Rn = resid_next ? (float4*)RN[l] : nullptr;
     a.n4 = n4;
     a.coef = l == L ? p.rho : p.nu;
-    a.W = W[l]; a.Wt = Wt[l]; a.grad = grad;
+    a.W = W[l]; a.Wt = Wt[l]; a.image = img_H[l]; a.image_t = img_G[l]; a.grad = grad;
     a.rows = Kp; a.cols = Cn; a.ldw = ldc; a.ldwt = ld[l - 1];
     a.ctl = ctl; a.partial = red_part; a.bar = grid_bar; a.ticket = ticket; a.status = status; a.err = tc_error;
     a.a.growth = p.bt_growth;
@@ -657,7 +679,7 @@ struct gcn_admm {
     float* const Rn = RN[l + 1];
     if (!resid_ready) resid(l + 1, Rn);                                  // R'_{l+1}
     spmm(Rn, B1, ldn);                                                   // S = A~ R'
-    gemm_nn(B1, ldn, Wt[l + 1], ldl, W[l + 1], ldn, B2, ldl, n, C[l], C[l + 1]);        // S W_{l+1}^T
+    gemm_nn(B1, ldn, Wt[l + 1], ldl, W[l + 1], ldn, B2, ldl, n, C[l], C[l + 1], &img_G[l + 1]);        // S W_{l+1}^T
     {
       Scope sc(this, "zgrad_finish", 1, 16.0 * 4.0 * (double)n * (ldl / 4), 0.0);
       gk::k_zgrad_finish<<<(unsigned)n_zblocks, 256, 0, stream>>>(
@@ -674,7 +696,7 @@ struct gcn_admm {
     decide.max_trials = p.bt_max_trials;
     decide.own_nu = p.nu;
     if (l + 1 == L) {   // closed form
-      gemm_nn(B2, ldl, W[L], ldn, Wt[L], ldl, B0, ldn, n, C[L], C[l]);   // T = G W_L; S stays in B1
+      gemm_nn(B2, ldl, W[L], ldn, Wt[L], ldl, B0, ldn, n, C[L], C[l], &img_H[L]);   // T = G W_L; S stays in B1
       decide.mode = 1;
       decide.quad_coef = 0.5 * p.rho;
       gk::SearchOut a{};
@@ -707,7 +729,7 @@ struct gcn_admm {
       CU(cudaGetLastError());
       return;
     }
-    gemm_nn(B2, ldl, W[l + 1], ldn, Wt[l + 1], ldl, B1, ldn, n, C[l + 1], C[l]);         // T = G W_{l+1}
+    gemm_nn(B2, ldl, W[l + 1], ldn, Wt[l + 1], ldl, B1, ldn, n, C[l + 1], C[l], &img_H[l + 1]);         // T = G W_{l+1}
     decide.cand = kCandZ;
     decide.scale = 0.5 * p.nu;
     gk::SearchZ a{};
@@ -796,7 +818,7 @@ struct gcn_admm {
     fresh = true;
   }
   void refresh_H(int l, const int* skip = nullptr) {
-    gemm_nn(P[l], ld[l - 1], W[l], ld[l], Wt[l], ld[l - 1], H[l], ld[l], n, C[l], C[l - 1], skip);
+    gemm_nn(P[l], ld[l - 1], W[l], ld[l], Wt[l], ld[l - 1], H[l], ld[l], n, C[l], C[l - 1], &img_H[l], skip);
   }
   void refresh_H1(bool keep_h1) {
     const bool skip = keep_h1 && !capturing && h1_age + 1 < kH1RefreshEvery;
@@ -817,7 +839,7 @@ struct gcn_admm {
     for (int l = 1; l <= L; ++l) {
       if (l >= 2) {   // Z_{l-1} has just moved: P_l and H_l follow it (H_{l+1} still matches the untouched Z_l)
         spmm(Z[l - 1], P[l], ld[l - 1]);
-        gemm_nn(P[l], ld[l - 1], W[l], ld[l], Wt[l], ld[l - 1], H[l], ld[l], n, C[l], C[l - 1]);
+        refresh_H(l);
       }
       update_W(l, false);
       if (l < L) update_Z_hidden(l, false);
@@ -835,7 +857,6 @@ struct gcn_admm {
     cudaStream_t stream = nullptr;
     float *part = nullptr, *grad = nullptr, *grad_t = nullptr;
     size_t part_elems = 0;
-    uint8_t* b_image = nullptr;
     double* red_part = nullptr;
     unsigned *ticket = nullptr, *tile_tickets = nullptr;
     cudaEvent_t begun = nullptr, w_done = nullptr, out_done = nullptr, done = nullptr;
@@ -847,7 +868,6 @@ struct gcn_admm {
     std::swap(part_elems, side.part_elems);
     std::swap(grad, side.grad);
     std::swap(grad_t, side.grad_t);
-    std::swap(b_image, side.b_image);
     std::swap(red_part, side.red_part);
     std::swap(ticket, side.ticket);
     std::swap(tile_tickets, side.tile_tickets);
@@ -907,14 +927,14 @@ struct gcn_admm {
 
   // logits of Problem 1's forward pass with the stored W, left in B0 (N x ld_L)
   void forward_logits() {
-    gemm_nn(P[1], ld[0], W[1], ld[1], Wt[1], ld[0], B0, ld[1], n, C[1], C[0]);
+    gemm_nn(P[1], ld[0], W[1], ld[1], Wt[1], ld[0], B0, ld[1], n, C[1], C[0], &img_H[1]);
     for (int l = 1; l < L; ++l) {
       const long long n4 = n * ld[l] / 4;
       Scope sc(this, "relu", 1, 32.0 * n4, 0.0);
       gk::k_relu_inplace<<<grid_for(n4), 256, 0, stream>>>((float4*)B0, n4);
       CU(cudaGetLastError());
       spmm(B0, B1, ld[l]);
-      gemm_nn(B1, ld[l], W[l + 1], ld[l + 1], Wt[l + 1], ld[l], B0, ld[l + 1], n, C[l + 1], C[l]);
+      gemm_nn(B1, ld[l], W[l + 1], ld[l + 1], Wt[l + 1], ld[l], B0, ld[l + 1], n, C[l + 1], C[l], &img_H[l + 1]);
     }
   }
 
@@ -986,7 +1006,7 @@ struct gcn_admm {
     CU(stage.put(grad, host_w, sizeof(float) * (size_t)r * c, stream));
     CU(stage.finish(stream));
     const long long cells = std::max((long long)r * ld[l], (long long)c * ld[l - 1]);
-    gk::k_load_weight<<<grid_for(cells), 256, 0, stream>>>(grad, r, c, W[l], ld[l], Wt[l], ld[l - 1]);
+    gk::k_load_weight<<<grid_for(cells), 256, 0, stream>>>(grad, r, c, W[l], ld[l], Wt[l], ld[l - 1], img_H[l], img_G[l]);
     CU(cudaGetLastError());
   }
   // Step parameters (t_prev) of `count` searches in a row, to and from the host.
@@ -1245,7 +1265,6 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
     h->want(h->side.part, h->side.part_elems);
     h->want(h->side.grad, ge);
     h->want(h->side.grad_t, (size_t)h->C[L] * h->ld[L - 1], gcn_admm::kZero);
-    h->want(h->side.b_image, (size_t)16 << 20);
     h->want(h->side.red_part, std::max<size_t>((size_t)kSmCount * 8 * gk::kCand, (size_t)cdiv((long long)ge, 32) * 2));
     h->want(h->side.ticket, 1, gcn_admm::kZero);
     h->want(h->side.tile_tickets, kSmCount, gcn_admm::kZero);
@@ -1258,6 +1277,12 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
   h->want(h->grad_t, grad_t_elems, gcn_admm::kZero);
   h->b_image_bytes = (size_t)16 << 20;   // e.g. 1024 columns x 2048 K
   h->want(h->b_image, h->b_image_bytes);
+  h->img_H.assign(L + 1, gtc::Image{nullptr, 16, 1}); h->img_G = h->img_D = h->img_H;
+  for (int l = 1; l <= L; ++l) {
+    h->want_image(h->img_H[l], h->C[l], h->C[l - 1], h->ld[l - 1]);
+    h->want_image(h->img_D[l], h->C[l], h->C[l - 1], h->ld[l - 1]);
+    if (l >= 2) h->want_image(h->img_G[l], h->C[l - 1], h->C[l], h->ld[l]);
+  }
   h->want(h->part, h->part_elems);
   std::vector<SearchCtl> cw(L + 1), cz((size_t)(L + 1) * n_comm);
   std::memset(cw.data(), 0, cw.size() * sizeof(SearchCtl));
@@ -1332,7 +1357,7 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
   // initial residuals are exactly zero
   for (int l = 1; l <= L; ++l) {
     if (l >= 2) h->spmm(h->Z[l - 1], h->P[l], h->ld[l - 1]);
-    h->gemm_nn(h->P[l], h->ld[l - 1], h->W[l], h->ld[l], h->Wt[l], h->ld[l - 1], h->H[l], h->ld[l], n, h->C[l], h->C[l - 1]);
+    h->refresh_H(l);
     const size_t bytes = rows * h->ld[l] * sizeof(float);
     CU(cudaMemcpyAsync(h->Z[l], h->H[l], bytes, cudaMemcpyDeviceToDevice, h->stream));
     if (l < L) {
@@ -1668,7 +1693,7 @@ int gcn_admm_dense_product_tn(gcn_admm* h, const float* A, const float* B, float
       CU(cudaMemcpy2DAsync(b, (size_t)ldb * 4, B, (size_t)nb * 4, (size_t)nb * 4, (size_t)rows, cudaMemcpyDeviceToDevice, h->stream));
       h->p.tensor_cores = tensor_cores;
       const int splits = h->gemm_tn(a, lda, b, ldb, ldp, rows, ka, nb);
-      h->finish_grad(splits, ka, nb, ldp, c, nullptr, 0, nullptr, nullptr);
+      h->finish_grad(splits, ka, nb, ldp, c, nullptr, 0, nullptr, nullptr, gtc::Image{nullptr, 16, 1});
       h->p.tensor_cores = saved;
       CU(cudaMemcpy2DAsync(C, (size_t)nb * 4, c, (size_t)ldp * 4, (size_t)nb * 4, (size_t)ka, cudaMemcpyDeviceToDevice, h->stream));
       CU(cudaStreamSynchronize(h->stream));

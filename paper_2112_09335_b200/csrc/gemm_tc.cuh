@@ -171,9 +171,7 @@ struct WsCfg {
 // of 2 * NT * 128 bytes at block index g * chunks + kc.  With it (IMG = true) a stage's B tiles arrive
 // by one bulk copy issued by one thread, and the producers stage A only; without it they load, split
 // and store B again for every 128-row tile.
-__global__ void k_split_b(const float* __restrict__ Bk, int ldbk, int N, int K, int nt, uint8_t* __restrict__ image,
-                          const int* __restrict__ skip) {
-  if (skip != nullptr && *skip) return;
+__global__ void k_split_b(const float* __restrict__ Bk, int ldbk, int N, int K, int nt, uint8_t* __restrict__ image) {
   const int kc_count = (K + kChunkK - 1) / kChunkK;
   const int groups = (N + nt - 1) / nt;
   const long long total = (long long)groups * kc_count * nt * 8;
@@ -191,6 +189,23 @@ __global__ void k_split_b(const float* __restrict__ Bk, int ldbk, int N, int K, 
     *reinterpret_cast<float4*>(dst) = h;
     *reinterpret_cast<float4*>(dst + (size_t)nt * kChunkK * 4) = l;
   }
+}
+
+// Such an image kept up to date by whoever writes the operand (the weights and their gradients: a launch of k_split_b and
+// its gap before every product otherwise, 4 us each).  nt: column group width, kc: K chunks; data = NULL: no image is kept.
+// The padding of the image is zero from the start and never written.
+struct Image {
+  uint8_t* data;
+  int nt, kc;
+};
+__device__ __forceinline__ void put_split(const Image& im, int n, int k, float x) {
+  if (im.data == nullptr) return;
+  const int g = n / im.nt, r = n - g * im.nt, c = k / kChunkK, kk = k - c * kChunkK;
+  uint8_t* const at = im.data + (size_t)(g * im.kc + c) * (size_t)(2 * im.nt * kChunkK * 4) + swz(r, kk >> 2) + (kk & 3) * 4;
+  float h, l;
+  split_tf32(x, h, l);
+  *reinterpret_cast<float*>(at) = h;
+  *reinterpret_cast<float*>(at + (size_t)im.nt * kChunkK * 4) = l;
 }
 
 // TMA = true (needs IMG): the A operand is not loaded by the producers at all.  One more warp (its lane 0)

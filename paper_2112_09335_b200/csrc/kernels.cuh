@@ -8,6 +8,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "gemm_tc.cuh"
+
 namespace gk {
 
 constexpr int kCand = 4;        // step-size candidates scored per pass
@@ -866,7 +868,7 @@ __device__ __forceinline__ void log_decision(const DecisionLog& lg, int i, const
 }
 
 // Weight gradient from its split partial sums, and the start of the W_l search, in one launch:
-//   grad[e] = sum over splits of part[s][e] (fp64, in split order), its transpose, ||grad||^2, ||W||^2.
+//   grad[e] = sum over splits of part[s][e] (fp64, in split order), its transpose and its image for P grad, ||grad||^2, ||W||^2.
 // A block owns 256 / SG elements; with many splits SG = 8 threads share an element, each adding its own run of consecutive
 // splits.  The last block to finish adds the blocks' sums of squares up in block order and starts the search.
 // W = NULL: only the sum over the splits.
@@ -874,7 +876,7 @@ template <int SG>
 __global__ void __launch_bounds__(256)
 k_finish_grad(const float* __restrict__ part, int splits, int rows, int cols, int ldp, float* __restrict__ grad,
               float* __restrict__ grad_t, int ldt, const float* __restrict__ W, double* partial, unsigned* ticket,
-              SearchCtl* ctl, double shrink, double growth, int* status) {
+              SearchCtl* ctl, double shrink, double growth, int* status, const gtc::Image image) {
   constexpr int ELEMS = 256 / SG;
   __shared__ double sh[16], s_part[SG][ELEMS];
   __shared__ int s_last;
@@ -902,7 +904,10 @@ k_finish_grad(const float* __restrict__ part, int splits, int rows, int cols, in
     grad[e] = g;
     if (W != nullptr) {
       const int r = (int)(e / ldp), c = (int)(e - (long long)r * ldp);
-      if (c < cols) grad_t[(long long)c * ldt + r] = g;
+      if (c < cols) {
+        grad_t[(long long)c * ldt + r] = g;
+        gtc::put_split(image, c, r, g);
+      }
       sq[0] = (double)g * (double)g;
       sq[1] = (double)w * (double)w;
     }
@@ -945,6 +950,7 @@ struct SearchW {
   long long n4;
   float coef;                       // nu (hidden) or rho (last layer)
   float *W, *Wt;
+  gtc::Image image, image_t;        // of W as the operand of P W and of S W^T
   const float* grad;
   int rows, cols, ldw, ldwt;
   SearchCtl* ctl;
@@ -965,6 +971,8 @@ __device__ __forceinline__ void move_w(const SearchW& p, float step) {
       const float w = fmaf(-p.grad[(long long)r * p.ldw + c], step, p.W[(long long)r * p.ldw + c]);
       p.W[(long long)r * p.ldw + c] = w;
       p.Wt[(long long)c * p.ldwt + r] = w;
+      gtc::put_split(p.image, c, r, w);
+      gtc::put_split(p.image_t, r, c, w);
     }
   if (step == 0.f && p.Rn == nullptr) return;
   for (long long i = first; i < p.n4; i += stride) {
@@ -2095,13 +2103,18 @@ __global__ void k_transpose_small(const float* __restrict__ src, int lds, float*
   dst[c * ldd + r] = src[r * lds + c];
 }
 
-// W (rows x cols, leading dimension ldw) and its transpose from a dense matrix; padding columns become zero.
+// W (rows x cols, leading dimension ldw), its transpose and its images from a dense matrix; padding columns become zero.
 __global__ void k_load_weight(const float* __restrict__ src, int rows, int cols, float* __restrict__ W, int ldw,
-                              float* __restrict__ Wt, int ldwt) {
+                              float* __restrict__ Wt, int ldwt, const gtc::Image image, const gtc::Image image_t) {
   const long long first = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
   for (long long i = first; i < (long long)rows * ldw; i += stride) {
     const long long r = i / ldw, c = i - r * ldw;
-    W[i] = c < cols ? src[r * cols + c] : 0.f;
+    const float w = c < cols ? src[r * cols + c] : 0.f;
+    W[i] = w;
+    if (c < cols) {
+      gtc::put_split(image, (int)c, (int)r, w);
+      gtc::put_split(image_t, (int)r, (int)c, w);
+    }
   }
   for (long long i = first; i < (long long)cols * ldwt; i += stride) {
     const long long c = i / ldwt, r = i - c * ldwt;
