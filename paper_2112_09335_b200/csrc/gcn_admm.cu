@@ -304,11 +304,12 @@ struct gcn_admm {
   }
 
   // ---- launches -----------------------------------------------------------------------
-  void spmm(const float* x, float* out, int ldx) {
+  void spmm(const float* x, float* out, int ldx, bool relu = false) {
     char name[48];
     std::snprintf(name, sizeof name, "spmm@%d", ldx);
     Scope sc(this, name, 1, 4.0 * gi.nnz + 8.0 * n + 8.0 * (double)n * ldx, 2.0 * (double)gi.nnz * ldx);
-    spmm_tables<4, false>(gather_graph(ldx), x, out, ldx / 4);
+    if (relu) spmm_tables<4, false, true>(gather_graph(ldx), x, out, ldx / 4);
+    else spmm_tables<4, false>(gather_graph(ldx), x, out, ldx / 4);
   }
 
   // out = A~ x for dense n x width device matrices in the caller's row order, in vectors as wide as the width and
@@ -350,7 +351,7 @@ struct gcn_admm {
 
   // The propagation kernels on a graph given by its tables (the handle's own, or a rank's local part of it); x and
   // out have ldv vectors of VEC floats per row.
-  template <int VEC, bool MAPPED>
+  template <int VEC, bool MAPPED, bool RELU = false>
   void spmm_tables(const GatherGraph& g, const float* xf, float* outf, int ldv) {
     using T = typename gk::Vec<VEC>::T;
     const T* x = reinterpret_cast<const T*>(xf);
@@ -358,12 +359,12 @@ struct gcn_admm {
     const int ld4 = (int)cdiv((long long)ldv * VEC, 4);
     const long long units = (long long)g.n + g.n_items;
 #define WIDE(NV4, UN, SLICED)                                                                                             \
-  gk::k_spmm_wide<VEC, 4 / VEC * (NV4), UN, MAPPED, SLICED>                                                               \
+  gk::k_spmm_wide<VEC, 4 / VEC * (NV4), UN, MAPPED, SLICED, RELU>                                                               \
       <<<dim3((unsigned)cdiv(units * 32, 64), (unsigned)std::min<long long>(32768, cdiv(ld4, 32 * (NV4))),                \
               (unsigned)cdiv(ld4, 32768LL * 32 * (NV4))), 64, 0, stream>>>(                                               \
       g.row_ptr, g.col, g.dinv, g.perm, g.items, g.n, g.n_items, g.long_len, x, out, ldv, scratch)
 #define SETS(CL, EP, UN)                                                                                                  \
-  gk::k_spmm_sets<VEC, 4 / VEC, CL, EP, UN, MAPPED><<<(unsigned)cdiv(units * ((CL) * (EP)), 128), 128, 0, stream>>>( \
+  gk::k_spmm_sets<VEC, 4 / VEC, CL, EP, UN, MAPPED, RELU><<<(unsigned)cdiv(units * ((CL) * (EP)), 128), 128, 0, stream>>>( \
       g.row_ptr, g.col, g.dinv, g.perm, g.items, g.n, g.n_items, g.long_len, x, out, ldv, scratch, g.row_order, gk::ItemRows{g.rows, g.item_row, g.row_done})
     // Sets of entries per row: as many as the warp holds while the grid is then still small (latency counts), fewer
     // where the rows alone fill the chip several times over and the lanes of half-empty sets would only cost issue
@@ -569,7 +570,7 @@ struct gcn_admm {
       gk::k_finish_grad<8><<<(unsigned)cdiv(elems, 32), 256, 0, stream>>>(part, splits, Ka, Nb, ldp, out, out_t, ldt, w, red_part,
                                                                             ticket, ctl, p.bt_shrink, p.bt_growth, status, image);
     else
-      gk::k_finish_grad<1><<<(unsigned)cdiv(elems, 256), 256, 0, stream>>>(part, splits, Ka, Nb, ldp, out, out_t, ldt, w, red_part,
+      gk::k_finish_grad<1><<<(unsigned)(cdiv(Ka, 32) * cdiv(ldp, 32)), 256, 0, stream>>>(part, splits, Ka, Nb, ldp, out, out_t, ldt, w, red_part,
                                                                                      ticket, ctl, p.bt_shrink, p.bt_growth, status, image);
     CU(cudaGetLastError());
   }
@@ -925,17 +926,20 @@ struct gcn_admm {
     end_pass();
   }
 
-  // logits of Problem 1's forward pass with the stored W, left in B0 (N x ld_L)
-  void forward_logits() {
-    gemm_nn(P[1], ld[0], W[1], ld[1], Wt[1], ld[0], B0, ld[1], n, C[1], C[0], &img_H[1]);
-    for (int l = 1; l < L; ++l) {
-      const long long n4 = n * ld[l] / 4;
-      Scope sc(this, "relu", 1, 32.0 * n4, 0.0);
-      gk::k_relu_inplace<<<grid_for(n4), 256, 0, stream>>>((float4*)B0, n4);
-      CU(cudaGetLastError());
-      spmm(B0, B1, ld[l]);
-      gemm_nn(B1, ld[l], W[l + 1], ld[l + 1], Wt[l + 1], ld[l], B0, ld[l + 1], n, C[l + 1], C[l], &img_H[l + 1]);
+  // Logits of Problem 1's forward pass with the stored W (N x ld_L, in B0 unless they are H_1).  The first layer's product is
+  // H_1 itself while the stored matrices agree; activations are taken as the rows are gathered.
+  const float* forward_logits() {
+    const float* h = H[1];
+    if (!fresh) {
+      gemm_nn(P[1], ld[0], W[1], ld[1], Wt[1], ld[0], B0, ld[1], n, C[1], C[0], &img_H[1]);
+      h = B0;
     }
+    for (int l = 1; l < L; ++l) {
+      spmm(h, B1, ld[l], true);
+      gemm_nn(B1, ld[l], W[l + 1], ld[l + 1], Wt[l + 1], ld[l], B0, ld[l + 1], n, C[l + 1], C[l], &img_H[l + 1]);
+      h = B0;
+    }
+    return h;
   }
 
   // Reported numbers and error flags, read back together.
@@ -1560,10 +1564,10 @@ int gcn_admm_objective(gcn_admm* h, double out[6]) {
       gk::k_add_partials<<<1, 256, 0, s>>>(h->red_part, row_blocks, 2, obj);      // obj[0] = cross-entropy sum
       CU(cudaGetLastError());
     }
-    h->forward_logits();
+    const float* const logits = h->forward_logits();
     {
       gcn_admm::Scope sc_obj(h, "objective_sums", 2, 4.0 * (double)h->n * h->ld[L], 0.0);
-      gk::k_row_loss_argmax<<<row_blocks, warps * 32, 0, s>>>(nullptr, h->B0, h->ld[L], h->C[L], (int)h->n, h->d_y,
+      gk::k_row_loss_argmax<<<row_blocks, warps * 32, 0, s>>>(nullptr, logits, h->ld[L], h->C[L], (int)h->n, h->d_y,
                                                               h->d_train, nullptr, nullptr, h->red_part);
       gk::k_add_partials<<<1, 256, 0, s>>>(h->red_part, row_blocks, 2, obj + 5);  // obj[6] = correct training rows
       CU(cudaGetLastError());
@@ -1588,19 +1592,19 @@ int gcn_admm_weights(gcn_admm* h, int layer, float* out) {
 int gcn_admm_predict(gcn_admm* h, float* logits, int* labels) {
   return guarded(h, [&] {
     const int L = h->L;
-    h->forward_logits();
+    const float* const z = h->forward_logits();
     if (labels) {
       const int warps = 8;
       int* d_lab = reinterpret_cast<int*>(h->B1);
       {
         gcn_admm::Scope sc(h, "row_argmax", 1, 4.0 * (double)h->n * h->ld[L], 0.0);
         gk::k_row_loss_argmax<<<(unsigned)cdiv(h->n, warps), warps * 32, 0, h->stream>>>(
-            nullptr, h->B0, h->ld[L], h->C[L], (int)h->n, h->d_y, h->d_train, d_lab, h->d_perm, h->red_part);
+            nullptr, z, h->ld[L], h->C[L], (int)h->n, h->d_y, h->d_train, d_lab, h->d_perm, h->red_part);
         CU(cudaGetLastError());
       }
       CU(h->stage.get(labels, d_lab, sizeof(int) * h->n, sizeof(int) * h->n, 1, h->stream));
     }
-    if (logits) h->rows_to_host(h->B0, h->C[L], logits);
+    if (logits) h->rows_to_host(z, h->C[L], logits);
     CU(cudaStreamSynchronize(h->stream));
   });
 }

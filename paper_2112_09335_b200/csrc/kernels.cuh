@@ -117,6 +117,7 @@ __device__ __forceinline__ void add_block_sums(const double* partial, int count,
 // item order: by the last of them to finish (one counter per long row, left at zero), or by k_spmm_long_rows.
 // MAPPED: x and out are dense matrices in the caller's row order; node c's row is perm[c] (a 4-byte load in
 // parallel with that of its weight), so that no copy of the operand in community order and none back is made.
+// RELU: out = A~ max(x, 0), so that a forward pass needs no sweep for its activations.
 // Values are moved in vectors of VEC floats: four wherever rows start on 16-byte boundaries (always inside the
 // library), fewer for a caller's matrix of odd width.
 // ------------------------------------------------------------------------------------------
@@ -141,6 +142,9 @@ __device__ __forceinline__ float2 vxor(unsigned m, float2 a, int o) { return mak
 __device__ __forceinline__ float4 vxor(unsigned m, float4 a, int o) {
   return make_float4(vxor(m, a.x, o), vxor(m, a.y, o), vxor(m, a.z, o), vxor(m, a.w, o));
 }
+__device__ __forceinline__ float vrelu(float a) { return relu(a); }
+__device__ __forceinline__ float2 vrelu(float2 a) { return make_float2(relu(a.x), relu(a.y)); }
+__device__ __forceinline__ float4 vrelu(float4 a) { return make_float4(relu(a.x), relu(a.y), relu(a.z), relu(a.w)); }
 __device__ __forceinline__ void vzero(float& a) { a = 0.f; }
 __device__ __forceinline__ void vzero(float2& a) { a = make_float2(0.f, 0.f); }
 __device__ __forceinline__ void vzero(float4& a) { a = make_float4(0.f, 0.f, 0.f, 0.f); }
@@ -182,7 +186,7 @@ __device__ __forceinline__ void finish_item(const ItemRows& ir, int unit, T* __r
 // stored entries holds column and weight of entry t, handed to the warp by shuffles.  UN neighbours in flight per
 // lane: the kernel is bound by the L2-to-SM traffic of the gathered rows, and by how the compiler orders its loads (the plain
 // loop measured faster than one that fetches columns ahead: 138 against 160 us at 128 columns on 169 k rows).
-template <int VEC, int NV, int UN, bool MAPPED, bool SLICED>
+template <int VEC, int NV, int UN, bool MAPPED, bool SLICED, bool RELU>
 __global__ void __launch_bounds__(64, VEC == 4 ? 24 : 16)
 k_spmm_wide(const int* __restrict__ row_ptr, const int* __restrict__ col, const float* __restrict__ dinv,
             const int* __restrict__ perm, const int4* __restrict__ items, int n, int n_items, int long_len,
@@ -239,7 +243,7 @@ k_spmm_wide(const int* __restrict__ row_ptr, const int* __restrict__ col, const 
 #pragma unroll
             for (int u = 0; u < UN; ++u) xv[u] = __ldg(x + (long long)rj[u] * ldv + f);
 #pragma unroll
-            for (int u = 0; u < UN; ++u) acc[v] = vfma(wj[u], xv[u], acc[v]);
+            for (int u = 0; u < UN; ++u) acc[v] = vfma(wj[u], RELU ? vrelu(xv[u]) : xv[u], acc[v]);
           }
         }
       }
@@ -277,7 +281,7 @@ __global__ void k_spmm_long_rows(const int4* __restrict__ rows, const T* __restr
 // and hand them to the sets by shuffles (with more lanes per set the repeated loads cost more than the shuffles).
 // Rows sharing a warp are taken by falling length.  Measured at 4 / 16 / 48 columns against one set per row:
 // 2.4 M rows, 126 M entries: 5.5 -> 1.1 ms, 2.2 -> 1.0, 2.7 -> 2.7; 13.8 k rows, 0.43 M entries: 293 -> 15 us, 85 -> 15, 37 -> 25.
-template <int VEC, int NV, int CL, int EP, int UN, bool MAPPED>
+template <int VEC, int NV, int CL, int EP, int UN, bool MAPPED, bool RELU>
 __global__ void __launch_bounds__(128, CL >= 8 && VEC == 4 ? 10 : 8)
 k_spmm_sets(const int* __restrict__ row_ptr, const int* __restrict__ col, const float* __restrict__ dinv,
             const int* __restrict__ perm, const int4* __restrict__ items, int n, int n_items, int long_len,
@@ -334,7 +338,7 @@ k_spmm_sets(const int* __restrict__ row_ptr, const int* __restrict__ col, const 
               if (r[u] >= 0) xv[u] = __ldg(x + (long long)r[u] * ldv + f);
 #pragma unroll
             for (int u = 0; u < UN; ++u)
-              if (r[u] >= 0) acc[v] = vfma(w[u], xv[u], acc[v]);
+              if (r[u] >= 0) acc[v] = vfma(w[u], RELU ? vrelu(xv[u]) : xv[u], acc[v]);
           }
         }
       }
@@ -367,7 +371,7 @@ k_spmm_sets(const int* __restrict__ row_ptr, const int* __restrict__ col, const 
 #pragma unroll
               for (int u = 0; u < UN; ++u) xv[u] = __ldg(x + (long long)rj[u] * ldv + f);
 #pragma unroll
-              for (int u = 0; u < UN; ++u) acc[v] = vfma(wj[u], xv[u], acc[v]);
+              for (int u = 0; u < UN; ++u) acc[v] = vfma(wj[u], RELU ? vrelu(xv[u]) : xv[u], acc[v]);
             }
           }
         }
@@ -867,49 +871,88 @@ __device__ __forceinline__ void log_decision(const DecisionLog& lg, int i, const
   lg.q[at] = c->q;
 }
 
+// Weight matrices are written in two orders at once (themselves and their transpose, an image for either): in tiles of 32 x
+// 32 that turn through shared memory, because a column of single floats costs a memory sector per element.  `value(r, c)` is called once per element of the tile, padding columns included, and gives its new value; t may be
+// NULL.  Blocks of 256 threads, all of them.
+using WeightTile = float[32][33];
+template <typename F>
+__device__ __forceinline__ void weight_tile(int tile, int rows, int cols, int padded, WeightTile& turn, float* __restrict__ t, int ldt,
+                                            const gtc::Image& image, const gtc::Image& image_t, F&& value) {
+  const int x = threadIdx.x & 31, y = threadIdx.x >> 5, col_tiles = (padded + 31) / 32;
+  const int r0 = tile / col_tiles * 32, c0 = tile % col_tiles * 32;
+  __syncthreads();   // the tile before this one has been read
+#pragma unroll
+  for (int k = 0; k < 32; k += 8) {
+    const int r = r0 + y + k, c = c0 + x;
+    if (r < rows && c < padded) {
+      const float v = value(r, c);
+      turn[y + k][x] = v;
+      if (c < cols) gtc::put_split(image_t, r, c, v);
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < 32; k += 8) {
+    const int r = r0 + x, c = c0 + y + k;
+    if (r < rows && c < cols) {
+      const float v = turn[x][y + k];
+      if (t != nullptr) t[(long long)c * ldt + r] = v;
+      gtc::put_split(image, c, r, v);
+    }
+  }
+}
+
 // Weight gradient from its split partial sums, and the start of the W_l search, in one launch:
 //   grad[e] = sum over splits of part[s][e] (fp64, in split order), its transpose and its image for P grad, ||grad||^2, ||W||^2.
-// A block owns 256 / SG elements; with many splits SG = 8 threads share an element, each adding its own run of consecutive
-// splits.  The last block to finish adds the blocks' sums of squares up in block order and starts the search.
-// W = NULL: only the sum over the splits.
+// SG = 1: a block owns a tile of 32 x 32 elements (grid: tiles over rows x ldp).  SG = 8 (many splits): 32 consecutive elements,
+// eight threads per element, each adding its own run of consecutive splits.  The last block to finish adds the
+// blocks' sums of squares up in block order and starts the search.  W = NULL: only the sum over the splits.
 template <int SG>
 __global__ void __launch_bounds__(256)
 k_finish_grad(const float* __restrict__ part, int splits, int rows, int cols, int ldp, float* __restrict__ grad,
               float* __restrict__ grad_t, int ldt, const float* __restrict__ W, double* partial, unsigned* ticket,
               SearchCtl* ctl, double shrink, double growth, int* status, const gtc::Image image) {
-  constexpr int ELEMS = 256 / SG;
-  __shared__ double sh[16], s_part[SG][ELEMS];
+  __shared__ double sh[16], s_part[SG == 1 ? 1 : SG][32];
+  __shared__ WeightTile turn;
   __shared__ int s_last;
-  const int x = threadIdx.x % ELEMS, sg = threadIdx.x / ELEMS;
-  const long long elems = (long long)rows * ldp, e = (long long)blockIdx.x * ELEMS + x;
-  const bool in = e < elems;
-  double s = 0.0;
-  float w = 0.f;
-  if (in) {
-    if (W != nullptr && sg == 0) w = W[e];
-    const int k1 = (int)((long long)splits * (sg + 1) / SG);
+  const long long elems = (long long)rows * ldp;
+  double sq[2] = {0.0, 0.0};   // of grad, of W
+  const auto sum_splits = [&](long long e, int k0, int k1) {
+    double s = 0.0;
 #pragma unroll 8
-    for (int k = (int)((long long)splits * sg / SG); k < k1; ++k) s += (double)part[k * elems + e];
-  }
-  if (SG > 1) {
+    for (int k = k0; k < k1; ++k) s += (double)part[k * elems + e];
+    return s;
+  };
+  if (SG == 1) {
+    weight_tile((int)blockIdx.x, rows, cols, ldp, turn, W != nullptr ? grad_t : nullptr, ldt, image, gtc::Image{nullptr, 16, 1}, [&](int r, int c) {
+      const long long e = (long long)r * ldp + c;
+      const float g = (float)sum_splits(e, 0, splits);
+      grad[e] = g;
+      if (W != nullptr) { const double w = W[e]; sq[0] += (double)g * (double)g; sq[1] += w * w; }
+      return g;
+    });
+  } else {
+    const int x = threadIdx.x & 31, sg = threadIdx.x >> 5;
+    const long long e = (long long)blockIdx.x * 32 + x;
+    const bool in = e < elems;
+    const float w = in && W != nullptr && sg == 0 ? W[e] : 0.f;
+    double s = in ? sum_splits(e, (int)((long long)splits * sg / SG), (int)((long long)splits * (sg + 1) / SG)) : 0.0;
     s_part[sg][x] = s;
     __syncthreads();
-    if (sg == 0)
+    if (in && sg == 0) {
 #pragma unroll
       for (int k = 1; k < SG; ++k) s += s_part[k][x];
-  }
-  double sq[2] = {0.0, 0.0};   // of grad, of W
-  if (in && sg == 0) {
-    const float g = (float)s;
-    grad[e] = g;
-    if (W != nullptr) {
-      const int r = (int)(e / ldp), c = (int)(e - (long long)r * ldp);
-      if (c < cols) {
-        grad_t[(long long)c * ldt + r] = g;
-        gtc::put_split(image, c, r, g);
+      const float g = (float)s;
+      grad[e] = g;
+      if (W != nullptr) {
+        const int r = (int)(e / ldp), c = (int)(e - (long long)r * ldp);
+        if (c < cols) {
+          grad_t[(long long)c * ldt + r] = g;
+          gtc::put_split(image, c, r, g);
+        }
+        sq[0] = (double)g * (double)g;
+        sq[1] = (double)w * (double)w;
       }
-      sq[0] = (double)g * (double)g;
-      sq[1] = (double)w * (double)w;
     }
   }
   if (W == nullptr) return;
@@ -965,15 +1008,17 @@ struct SearchW {
 template <bool OUT>
 __device__ __forceinline__ void move_w(const SearchW& p, float step) {
   const long long first = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
-  if (step != 0.f)
-    for (long long e = first; e < (long long)p.rows * p.cols; e += stride) {   // a weight matrix: below 2^32
-      const int r = (int)((unsigned)e / (unsigned)p.cols), c = (int)((unsigned)e - (unsigned)r * (unsigned)p.cols);
-      const float w = fmaf(-p.grad[(long long)r * p.ldw + c], step, p.W[(long long)r * p.ldw + c]);
-      p.W[(long long)r * p.ldw + c] = w;
-      p.Wt[(long long)c * p.ldwt + r] = w;
-      gtc::put_split(p.image, c, r, w);
-      gtc::put_split(p.image_t, r, c, w);
-    }
+  if (step != 0.f) {
+    __shared__ WeightTile turn;
+    const int tiles = ((p.rows + 31) / 32) * ((p.cols + 31) / 32);
+    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x)
+      weight_tile(tile, p.rows, p.cols, p.cols, turn, p.Wt, p.ldwt, p.image, p.image_t, [&](int r, int c) {
+        const long long e = (long long)r * p.ldw + c;
+        const float w = fmaf(-p.grad[e], step, p.W[e]);
+        p.W[e] = w;
+        return w;
+      });
+  }
   if (step == 0.f && p.Rn == nullptr) return;
   for (long long i = first; i < p.n4; i += stride) {
     float4 h = p.H[i];
