@@ -349,6 +349,41 @@ struct gcn_admm {
     item_sums_elems = need;
   }
 
+  template <typename T> struct Same { using type = T; };   // keeps a parameter out of template deduction
+  // Launch of a kernel that waits for its predecessor on the stream itself (gtc::enter_kernel), where the grid is short, so
+  // that the launch is a good part of its time.  In a pass that is a wave or less: waiting blocks hold their SMs' threads
+  // against what still runs there and against the other line of launches (without the bound 13.8 k rows lost 3 %, 169 k
+  // 1 %).  A propagation on its own has nothing beside it (2.7 k rows, 16 columns, call after call: 6.1 -> 4.0 us).  The first
+  // kernel after a wait for the other line's event takes the ordinary dependency on both.
+  template <typename... Args>
+  void launch(void (*kernel)(Args...), dim3 grid, int threads, size_t smem, typename Same<Args>::type... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute behind{};
+    behind.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    behind.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &behind;
+    cfg.numAttrs = joined || (long long)grid.x * grid.y * grid.z > (in_pass ? 4 : 32) * kSmCount ? 0 : 1;
+    joined = false;
+    CU(cudaLaunchKernelEx(&cfg, kernel, args...));
+  }
+  // The ordinary launch, for kernels without that wait: the products (with it 13.8 k rows lost 3 % of a pass), the wide gathers
+  // and the sweeps over the graph (their loads are ordered worse behind it: 2.4 M rows at 256 columns lost 20 %).
+  template <typename... Args>
+  void launch_alone(void (*kernel)(Args...), dim3 grid, int threads, size_t smem, typename Same<Args>::type... args) {
+    joined = true;
+    launch(kernel, grid, threads, smem, args...);
+  }
+  bool joined = false;   // the next launch takes the ordinary dependency
+  bool in_pass = true;   // false: a propagation on its own
+  void join(cudaStream_t waiting, cudaEvent_t e) {
+    CU(cudaStreamWaitEvent(waiting, e, 0));
+    joined = true;
+  }
+
   // The propagation kernels on a graph given by its tables (the handle's own, or a rank's local part of it); x and
   // out have ldv vectors of VEC floats per row.
   template <int VEC, bool MAPPED, bool RELU = false>
@@ -358,13 +393,13 @@ struct gcn_admm {
     T *out = reinterpret_cast<T*>(outf), *scratch = reinterpret_cast<T*>(item_sums);
     const int ld4 = (int)cdiv((long long)ldv * VEC, 4);
     const long long units = (long long)g.n + g.n_items;
+    in_pass = !MAPPED;   // the caller's matrices: a call of its own
 #define WIDE(NV4, UN, SLICED)                                                                                             \
-  gk::k_spmm_wide<VEC, 4 / VEC * (NV4), UN, MAPPED, SLICED, RELU>                                                               \
-      <<<dim3((unsigned)cdiv(units * 32, 64), (unsigned)std::min<long long>(32768, cdiv(ld4, 32 * (NV4))),                \
-              (unsigned)cdiv(ld4, 32768LL * 32 * (NV4))), 64, 0, stream>>>(                                               \
+  launch_alone(gk::k_spmm_wide<VEC, 4 / VEC * (NV4), UN, MAPPED, SLICED, RELU>, dim3((unsigned)cdiv(units * 32, 64), (unsigned)std::min<long long>(32768, cdiv(ld4, 32 * (NV4))),                \
+              (unsigned)cdiv(ld4, 32768LL * 32 * (NV4))), 64, 0,                                                \
       g.row_ptr, g.col, g.dinv, g.perm, g.items, g.n, g.n_items, g.long_len, x, out, ldv, scratch)
 #define SETS(CL, EP, UN)                                                                                                  \
-  gk::k_spmm_sets<VEC, 4 / VEC, CL, EP, UN, MAPPED, RELU><<<(unsigned)cdiv(units * ((CL) * (EP)), 128), 128, 0, stream>>>( \
+  launch(gk::k_spmm_sets<VEC, 4 / VEC, CL, EP, UN, MAPPED, RELU>, (unsigned)cdiv(units * ((CL) * (EP)), 128), 128, 0,  \
       g.row_ptr, g.col, g.dinv, g.perm, g.items, g.n, g.n_items, g.long_len, x, out, ldv, scratch, g.row_order, gk::ItemRows{g.rows, g.item_row, g.row_done})
     // Sets of entries per row: as many as the warp holds while the grid is then still small (latency counts), fewer
     // where the rows alone fill the chip several times over and the lanes of half-empty sets would only cost issue
@@ -386,9 +421,10 @@ struct gcn_admm {
     else WIDE(2, 2, false);   // two neighbours in flight per lane beat four (fewer registers, more warps): measured
 #undef WIDE
 #undef SETS
+    in_pass = true;
     CU(cudaGetLastError());
     if (ld4 > 16 && g.n_long > 0) {
-      gk::k_spmm_long_rows<T, MAPPED><<<(unsigned)g.n_long, 64, 0, stream>>>(g.rows, scratch, out, ldv, g.perm);
+      launch(gk::k_spmm_long_rows<T, MAPPED>, (unsigned)g.n_long, 64, 0, g.rows, scratch, out, ldv, g.perm);
       CU(cudaGetLastError());
       ++launches;   // booked with the propagation it completes
     }
@@ -451,18 +487,18 @@ struct gcn_admm {
       // an image and up to 128 columns: A tiles by tensor copies into a ring of their own (at 256 columns shared memory
       // leaves no room for it, and the form measured no faster there)
       const bool copies = image != nullptr && nt <= 128 && make_a_tile_map(A, Mr, lda, &tmap);
-      auto launch = [&](auto kernel, int threads, size_t smem) {
+      auto run = [&](auto kernel, int threads, size_t smem) {
         CU(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        kernel<<<grid, threads, smem, stream>>>(A, lda, Bk, ldbk, Cm, ldc, (int)Mr, N, K, skip, tc_error, image, tmap, part, tile_tickets);
+        launch_alone(kernel, grid, threads, smem, A, lda, Bk, ldbk, Cm, ldc, (int)Mr, N, K, skip, tc_error, image, tmap, part, tile_tickets);
       };
       auto with_width = [&](auto width) {
         constexpr int NT = decltype(width)::value;
         using Cfg = gtc::WsCfg<NT>;
         if constexpr (NT <= 128) {
-          if (copies) { launch(gtc::k_gemm_tc_ws<NT, true, true>, Cfg::kThreads + 32, Cfg::kSmemRing); return; }
+          if (copies) { run(gtc::k_gemm_tc_ws<NT, true, true>, Cfg::kThreads + 32, Cfg::kSmemRing); return; }
         }
-        if (image != nullptr) launch(gtc::k_gemm_tc_ws<NT, true, false>, Cfg::kThreads, Cfg::kSmem);
-        else launch(gtc::k_gemm_tc_ws<NT, false, false>, Cfg::kThreads, Cfg::kSmem);
+        if (image != nullptr) run(gtc::k_gemm_tc_ws<NT, true, false>, Cfg::kThreads, Cfg::kSmem);
+        else run(gtc::k_gemm_tc_ws<NT, false, false>, Cfg::kThreads, Cfg::kSmem);
       };
       switch (nt) {
         case 16: with_width(std::integral_constant<int, 16>()); break;
@@ -480,7 +516,7 @@ struct gcn_admm {
 #define NN_CASE(BM, BN, BK, TM, TN)                                                             \
   {                                                                                             \
     dim3 grid((unsigned)cdiv(Mr, BM), (unsigned)cdiv(ldc, BN));                                  \
-    gk::k_gemm_nn<BM, BN, BK, TM, TN><<<grid, (BM / TM) * (BN / TN), 0, stream>>>(A, lda, B, ldb, Cm, ldc, (int)Mr, N, K, skip); \
+    launch_alone(gk::k_gemm_nn<BM, BN, BK, TM, TN>, grid, (BM / TM) * (BN / TN), 0, A, lda, B, ldb, Cm, ldc, (int)Mr, N, K, skip); \
   }
     if (N > 64) NN_CASE(128, 128, 16, 8, 8)
     else if (N > 16) NN_CASE(128, 64, 16, 8, 4)
@@ -524,10 +560,10 @@ struct gcn_admm {
     dim3 grid((unsigned)groups, (unsigned)splits, (unsigned)nb_groups);                                        \
     if (zres) {                                                                                                \
       CU(cudaFuncSetAttribute(gtc::k_gemm_tn_tc<NT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
-      gtc::k_gemm_tn_tc<NT, true><<<grid, gtc::kTnThreads, smem, stream>>>(A, lda, B, ldb, part, ldp, rows, rps, Ka, Nb, tc_error, zres, nu); \
+      launch_alone(gtc::k_gemm_tn_tc<NT, true>, grid, gtc::kTnThreads, smem, A, lda, B, ldb, part, ldp, rows, rps, Ka, Nb, tc_error, zres, nu); \
     } else {                                                                                                   \
       CU(cudaFuncSetAttribute(gtc::k_gemm_tn_tc<NT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
-      gtc::k_gemm_tn_tc<NT, false><<<grid, gtc::kTnThreads, smem, stream>>>(A, lda, B, ldb, part, ldp, rows, rps, Ka, Nb, tc_error, nullptr, 0.f); \
+      launch_alone(gtc::k_gemm_tn_tc<NT, false>, grid, gtc::kTnThreads, smem, A, lda, B, ldb, part, ldp, rows, rps, Ka, Nb, tc_error, nullptr, 0.f); \
     }                                                                                                          \
   }
       if (Nb <= 16) TN_TC(16)
@@ -550,7 +586,7 @@ struct gcn_admm {
     rps = cdiv(rows, splits);                                                                    \
     splits = (int)cdiv(rows, rps);                                                               \
     dim3 grid((unsigned)cdiv(Ka, BM), (unsigned)cdiv(ldp, BN), (unsigned)splits);                \
-    gk::k_gemm_tn<BM, BN, BK, TM, TN><<<grid, (BM / TM) * (BN / TN), 0, stream>>>(A, lda, B, ldb, part, ldp, rows, rps, Ka, Nb); \
+    launch_alone(gk::k_gemm_tn<BM, BN, BK, TM, TN>, grid, (BM / TM) * (BN / TN), 0, A, lda, B, ldb, part, ldp, rows, rps, Ka, Nb); \
   }
     if (Nb > 64) TN_CASE(128, 128, 16, 8, 8)
     else if (Nb > 16) TN_CASE(128, 64, 16, 8, 4)
@@ -567,10 +603,10 @@ struct gcn_admm {
     Scope sc(this, "finish_grad", 1, 4.0 * (double)Ka * ldp * (splits + (w ? 3 : 1)), 0.0);
     const long long elems = (long long)Ka * ldp;
     if (splits >= 16)
-      gk::k_finish_grad<8><<<(unsigned)cdiv(elems, 32), 256, 0, stream>>>(part, splits, Ka, Nb, ldp, out, out_t, ldt, w, red_part,
+      launch(gk::k_finish_grad<8>, (unsigned)cdiv(elems, 32), 256, 0, part, splits, Ka, Nb, ldp, out, out_t, ldt, w, red_part,
                                                                             ticket, ctl, p.bt_shrink, p.bt_growth, status, image);
     else
-      gk::k_finish_grad<1><<<(unsigned)(cdiv(Ka, 32) * cdiv(ldp, 32)), 256, 0, stream>>>(part, splits, Ka, Nb, ldp, out, out_t, ldt, w, red_part,
+      launch(gk::k_finish_grad<1>, (unsigned)(cdiv(Ka, 32) * cdiv(ldp, 32)), 256, 0, part, splits, Ka, Nb, ldp, out, out_t, ldt, w, red_part,
                                                                                      ticket, ctl, p.bt_shrink, p.bt_growth, status, image);
     CU(cudaGetLastError());
   }
@@ -587,7 +623,6 @@ struct gcn_admm {
     if (per_sm < 1) throw Fail{GCN_ADMM_ERR_CUDA, "a kernel does not fit the device"};
     return resident_cache[{kernel, smem}] = per_sm * kSmCount;
   }
-  template <typename T> struct Same { using type = T; };   // keeps a parameter out of template deduction
   template <typename... Args>
   void launch_together(void (*kernel)(Args...), long long blocks_wanted, int threads, size_t smem, typename Same<Args>::type... args) {
     const void* f = reinterpret_cast<const void*>(kernel);
@@ -600,9 +635,9 @@ struct gcn_admm {
     const long long n4 = n * ld[l] / 4;
     Scope sc(this, l < L ? "resid_hidden" : "resid_out", 1, 16.0 * n4 * (l < L ? 3 : 4), 0.0);
     if (l < L)
-      gk::k_resid_hidden<<<grid_for(n4), 256, 0, stream>>>((const float4*)H[l], (const float4*)Z[l], (float4*)R, n4, p.nu);
+      launch(gk::k_resid_hidden, grid_for(n4), 256, 0, (const float4*)H[l], (const float4*)Z[l], (float4*)R, n4, p.nu);
     else
-      gk::k_resid_out<<<grid_for(n4), 256, 0, stream>>>((const float4*)H[l], (const float4*)Z[l], (const float4*)U,
+      launch(gk::k_resid_out, grid_for(n4), 256, 0, (const float4*)H[l], (const float4*)Z[l], (const float4*)U,
                                                         (float4*)R, n4, p.rho);
     CU(cudaGetLastError());
   }
@@ -659,11 +694,11 @@ struct gcn_admm {
     if (l == L) {
       {
         Scope sc(this, "score_w_out", 1, 32.0 * n4, 0.0);
-        gk::k_score_w_out<<<grid_for(n4), 256, 0, stream>>>(a);
+        launch(gk::k_score_w_out, grid_for(n4), 256, 0, a);
         CU(cudaGetLastError());
       }
       Scope sc(this, "move_w_out", 1, 16.0 * (3 + (resid_next ? 3 : 0)) * n4, 0.0);
-      gk::k_move_w_out<<<grid_for(n4), 256, 0, stream>>>(a);
+      launch(gk::k_move_w_out, grid_for(n4), 256, 0, a);
       CU(cudaGetLastError());
     } else {
       Scope sc(this, "search_w_hidden", 1, 16.0 * (6 + (resid_next ? 2 : 0)) * n4, 0.0);
@@ -683,8 +718,7 @@ struct gcn_admm {
     gemm_nn(B1, ldn, Wt[l + 1], ldl, W[l + 1], ldn, B2, ldl, n, C[l], C[l + 1], &img_G[l + 1]);        // S W_{l+1}^T
     {
       Scope sc(this, "zgrad_finish", 1, 16.0 * 4.0 * (double)n * (ldl / 4), 0.0);
-      gk::k_zgrad_finish<<<(unsigned)n_zblocks, 256, 0, stream>>>(
-          (float4*)B2, (const float4*)Z[l], (const float4*)H[l], ldl / 4, d_zblocks, p.nu, red_part, d_comm_block_ptr, comm_tickets, ctl, sums_z,
+      launch(gk::k_zgrad_finish, (unsigned)n_zblocks, 256, 0, (float4*)B2, (const float4*)Z[l], (const float4*)H[l], ldl / 4, d_zblocks, p.nu, red_part, d_comm_block_ptr, comm_tickets, ctl, sums_z,
           p.bt_shrink, p.bt_growth, n_active, status);
       CU(cudaGetLastError());
     }
@@ -713,7 +747,7 @@ struct gcn_admm {
   {                                                                                                                         \
     const auto kernel = gk::k_search_z_out<CL>;                                                                             \
     const int grid = (int)std::min<long long>(cdiv(n_seg_chunks, warps), resident_blocks((const void*)kernel, warps * 32, 0)); \
-    kernel<<<grid, warps * 32, 0, stream>>>(d_col, d_dinv, (const float4*)B0, (const float4*)B1, ld4, scratch, a);          \
+    launch_alone(kernel, grid, warps * 32, 0, d_col, d_dinv, (const float4*)B0, (const float4*)B1, ld4, scratch, a);          \
   }
         if (ld4 <= 1) SEARCH_OUT(1)
         else if (ld4 <= 2) SEARCH_OUT(2)
@@ -725,7 +759,7 @@ struct gcn_admm {
         CU(cudaGetLastError());
       }
       Scope sc(this, "move_z", 1, move_bytes, 0.0);
-      gk::k_move_z<<<grid_for(n * (ldl / 4)), 256, 0, stream>>>((float4*)Z[l], (const float4*)B2, ldl / 4, n, d_row_comm, ctl, M, log_z(l),
+      launch(gk::k_move_z, grid_for(n * (ldl / 4)), 256, 0, (float4*)Z[l], (const float4*)B2, ldl / 4, n, d_row_comm, ctl, M, log_z(l),
                                                                 chunk_counter);
       CU(cudaGetLastError());
       return;
@@ -753,8 +787,8 @@ struct gcn_admm {
       const int grid = (int)std::min<long long>(cdiv(n_chunks, warps), resident_blocks((const void*)kernel, warps * 32, smem));
       {
         Scope sc(this, zname, 1, 6.0 * gi.nnz + 8.0 * n + 12.0 * (double)n * ldn, 2.0 * (double)gi.nnz * ldn);
-        kernel<<<grid, warps * 32, smem, stream>>>(d_row_ptr, d_col, d_col_comm, d_dinv, T, Hn, Zn, ld4, ctl, M, z_chunk_part, n_active,
-                                                   use_smem, d_chunk_ptr, n_chunks, chunk_counter, d_items, n_items, long_len, scratch);
+        launch_alone(kernel, grid, warps * 32, smem, d_row_ptr, d_col, d_col_comm, d_dinv, T, Hn, Zn, ld4, ctl, M, z_chunk_part, n_active,
+               use_smem, d_chunk_ptr, n_chunks, chunk_counter, d_items, n_items, long_len, scratch);
         CU(cudaGetLastError());
       }
       // closing, further sweeps and the move: as many blocks as the move can use
@@ -782,7 +816,7 @@ struct gcn_admm {
 #define OUTPUT(LPR, CPL)                                                        \
   {                                                                             \
     a.train_blocks = (int)cdiv((long long)n_train * (LPR), 256);                \
-    gk::k_output<LPR, CPL><<<(unsigned)(a.train_blocks + plain_blocks), 256, 0, stream>>>(a); \
+    launch(gk::k_output<LPR, CPL>, (unsigned)(a.train_blocks + plain_blocks), 256, 0, a); \
   }
     if (C[L] <= 4) OUTPUT(4, 1)
     else if (C[L] <= 8) OUTPUT(4, 2)
@@ -799,7 +833,7 @@ struct gcn_admm {
   void dual_from_stored() {   // U + rho (Z_L - H_L) with H_L = A~ Z_{L-1} W_L of the stored iterates
     const long long n4 = n * ld[L] / 4;
     Scope sc(this, "dual", 1, 64.0 * n4, 0.0);
-    gk::k_dual<<<grid_for(n4), 256, 0, stream>>>((float4*)U, (const float4*)Z[L], (const float4*)H[L], n4, p.rho);
+    launch(gk::k_dual, grid_for(n4), 256, 0, (float4*)U, (const float4*)Z[L], (const float4*)H[L], n4, p.rho);
     CU(cudaGetLastError());
   }
 
@@ -828,7 +862,7 @@ struct gcn_admm {
   }
   void end_pass() {
     Scope sc(this, "small", 1, 0.0, 0.0);
-    gk::k_end_pass<<<1, 1, 0, stream>>>(d_pass, d_h1_age, skip_h1, kH1RefreshEvery);
+    launch(gk::k_end_pass, 1, 1, 0, d_pass, d_h1_age, skip_h1, kH1RefreshEvery);
     CU(cudaGetLastError());
     ++log_count;
   }
@@ -896,7 +930,7 @@ struct gcn_admm {
       refresh(true);
     } else {
       CU(cudaEventRecord(side.begun, stream));
-      CU(cudaStreamWaitEvent(side.stream, side.begun, 0));
+      join(side.stream, side.begun);
       on_side([&] {
         update_W(L, true);
         CU(cudaEventRecord(side.w_done, stream));
@@ -905,20 +939,20 @@ struct gcn_admm {
       });
       for (int l = 1; l < L; ++l) update_W(l, l >= 2);
       for (int l = 1; l < L; ++l) {
-        if (l == L - 1) CU(cudaStreamWaitEvent(stream, side.w_done, 0));
+        if (l == L - 1) join(stream, side.w_done);
         update_Z_hidden(l, true);
       }
       CU(cudaEventRecord(side.begun, stream));
-      CU(cudaStreamWaitEvent(side.stream, side.begun, 0));
+      join(side.stream, side.begun);
       on_side([&] {
         refresh_H1(true);
         end_pass();
         CU(cudaEventRecord(side.done, stream));
       });
       for (int l = 2; l <= L; ++l) spmm(Z[l - 1], P[l], ld[l - 1]);
-      CU(cudaStreamWaitEvent(stream, side.out_done, 0));   // its rows of H_L have been read
+      join(stream, side.out_done);   // its rows of H_L have been read
       for (int l = 2; l <= L; ++l) refresh_H(l);
-      CU(cudaStreamWaitEvent(stream, side.done, 0));
+      join(stream, side.done);
       if (p.dual_mode != 0) dual_from_stored();
       return;
     }

@@ -38,6 +38,15 @@ constexpr int kChunkK = 32;                 // floats per K chunk (128 bytes)
 constexpr int kATileBytes = kBlockM * kChunkK * 4;     // 16 KiB, one of hi / lo
 constexpr long long kWaitClocks = 1LL << 31;   // bound of every mbarrier wait, in SM clocks (about a second)
 
+// First statement of a kernel that may be launched with programmatic serialisation: its grid may start while the one before
+// it on the stream still runs, waits here until that one is complete and its writes are seen, and only then lets the grid
+// behind it start in turn, so each kernel still follows all the ones before it.  What overlaps is the launch, one to two
+// microseconds.  Launched in the ordinary way both instructions do nothing.
+__device__ __forceinline__ void enter_kernel() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {

@@ -261,6 +261,7 @@ k_spmm_wide(const int* __restrict__ row_ptr, const int* __restrict__ col, const 
 template <typename T, bool MAPPED>
 __global__ void k_spmm_long_rows(const int4* __restrict__ rows, const T* __restrict__ scratch, T* __restrict__ out, int ldv,
                                  const int* __restrict__ perm) {
+  gtc::enter_kernel();
   const int4 r = rows[blockIdx.x];
   const long long row = MAPPED ? perm[r.x] : r.x;
   for (int f = threadIdx.x; f < ldv; f += blockDim.x) {
@@ -287,6 +288,7 @@ k_spmm_sets(const int* __restrict__ row_ptr, const int* __restrict__ col, const 
             const int* __restrict__ perm, const int4* __restrict__ items, int n, int n_items, int long_len,
             const typename Vec<VEC>::T* __restrict__ x, typename Vec<VEC>::T* __restrict__ out, int ldv,
             typename Vec<VEC>::T* __restrict__ scratch, const int* __restrict__ row_order, const ItemRows ir) {
+  gtc::enter_kernel();
   using T = typename Vec<VEC>::T;
   constexpr int G = CL * EP;
   static_assert(G <= 32, "a row is handled inside one warp");
@@ -679,6 +681,7 @@ __device__ __forceinline__ float4 resid_out(const float4& h, const float4& z, co
 
 __global__ void k_resid_hidden(const float4* __restrict__ H, const float4* __restrict__ Z,
                                float4* __restrict__ R, long long n4, float nu) {
+  gtc::enter_kernel();
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n4;
        i += (long long)gridDim.x * blockDim.x)
     R[i] = resid_hidden(H[i], Z[i], nu);
@@ -686,6 +689,7 @@ __global__ void k_resid_hidden(const float4* __restrict__ H, const float4* __res
 
 __global__ void k_resid_out(const float4* __restrict__ H, const float4* __restrict__ Z,
                             const float4* __restrict__ U, float4* __restrict__ R, long long n4, float rho) {
+  gtc::enter_kernel();
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n4;
        i += (long long)gridDim.x * blockDim.x)
     R[i] = resid_out(H[i], Z[i], U[i], rho);
@@ -872,8 +876,9 @@ __device__ __forceinline__ void log_decision(const DecisionLog& lg, int i, const
 }
 
 // Weight matrices are written in two orders at once (themselves and their transpose, an image for either): in tiles of 32 x
-// 32 that turn through shared memory, because a column of single floats costs a memory sector per element.  `value(r, c)` is called once per element of the tile, padding columns included, and gives its new value; t may be
-// NULL.  Blocks of 256 threads, all of them.
+// 32 that turn through shared memory, because a column of single floats costs a memory sector per element.
+// `value(r, c)` is called once per element of the tile, padding columns included, and gives its new value; t may be NULL.
+// Blocks of 256 threads, all of them.
 using WeightTile = float[32][33];
 template <typename F>
 __device__ __forceinline__ void weight_tile(int tile, int rows, int cols, int padded, WeightTile& turn, float* __restrict__ t, int ldt,
@@ -912,6 +917,7 @@ __global__ void __launch_bounds__(256)
 k_finish_grad(const float* __restrict__ part, int splits, int rows, int cols, int ldp, float* __restrict__ grad,
               float* __restrict__ grad_t, int ldt, const float* __restrict__ W, double* partial, unsigned* ticket,
               SearchCtl* ctl, double shrink, double growth, int* status, const gtc::Image image) {
+  gtc::enter_kernel();
   __shared__ double sh[16], s_part[SG == 1 ? 1 : SG][32];
   __shared__ WeightTile turn;
   __shared__ int s_last;
@@ -1082,6 +1088,7 @@ k_search_w_hidden(const SearchW p) {
 
 __global__ void __launch_bounds__(256)
 k_score_w_out(const SearchW p) {
+  gtc::enter_kernel();
   __shared__ double sh[16], total[2];
   __shared__ int s_last;
   if (p.ctl->done) {                // skipped: the same in every block
@@ -1114,11 +1121,15 @@ k_score_w_out(const SearchW p) {
 }
 
 __global__ void __launch_bounds__(256)
-k_move_w_out(const SearchW p) { move_w<true>(p, p.ctl->inv_step); }
+k_move_w_out(const SearchW p) {
+  gtc::enter_kernel();
+  move_w<true>(p, p.ctl->inv_step);
+}
 
 // The end of a pass: the pass counter of the log moves on, and with it the count of passes since H_1 was last formed afresh
 // (*skip_h1 = 1 while H_1, which the W_1 update keeps equal to P_1 W_1 up to rounding, need not be).
 __global__ void k_end_pass(int* __restrict__ pass, int* __restrict__ h1_age, int* __restrict__ skip_h1, int every) {
+  gtc::enter_kernel();
   *pass += 1;
   const int age = *skip_h1 ? *h1_age + 1 : 0;   // the pass that has just ended formed H_1 unless *skip_h1 said not to
   *h1_age = age;
@@ -1146,6 +1157,7 @@ __global__ void __launch_bounds__(256)
 k_zgrad_finish(float4* __restrict__ G, const float4* __restrict__ Z, const float4* __restrict__ H, int ld4,
                const int4* __restrict__ blocks, float nu, double* partial, const int* __restrict__ block_ptr, unsigned* tickets,
                SearchCtl* ctl, double* __restrict__ sums, double shrink, double growth, int* n_active, int* status) {
+  gtc::enter_kernel();
   __shared__ double sh[24];
   __shared__ int s_last;
   const int4 rb = blocks[blockIdx.x];
@@ -1894,6 +1906,7 @@ k_search_z_out(const int* __restrict__ col, const float* __restrict__ dinv, cons
 __global__ void __launch_bounds__(256)
 k_move_z(float4* __restrict__ Z, const float4* __restrict__ G, int ld4, long long n, const int* __restrict__ row_comm,
          const SearchCtl* __restrict__ ctl, int n_comm, const DecisionLog log, int* __restrict__ chunk_counter) {
+  gtc::enter_kernel();
   const long long first = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
   if (first == 0) *chunk_counter = 0;
   for (long long i = first; i < n_comm; i += stride) log_decision(log, (int)i, ctl + i);
@@ -1930,6 +1943,7 @@ struct OutputArgs {
 template <int LPR, int CPL>
 __global__ void __launch_bounds__(256)
 k_output(const OutputArgs p) {
+  gtc::enter_kernel();
   if ((int)blockIdx.x >= p.train_blocks) {
     const int ld4 = p.ld / 4;
     float4* const Z4 = reinterpret_cast<float4*>(p.Z);
@@ -2129,6 +2143,7 @@ __global__ void k_relu_inplace(float4* __restrict__ Y, long long n4) {
 // U <- U + rho (Z - H)
 __global__ void k_dual(float4* __restrict__ U, const float4* __restrict__ Z, const float4* __restrict__ H,
                        long long n4, float rho) {
+  gtc::enter_kernel();
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n4;
        i += (long long)gridDim.x * blockDim.x) {
     float4 u = U[i];
