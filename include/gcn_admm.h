@@ -57,14 +57,16 @@ enum {
  *  dual_mode       0: Eq. 3 as printed (Z_L^k, Z_{L-1}^k, W_L^{k+1}); 1: the k+1 iterates
  *  tensor_cores    1: dense products with 8 <= K <= 2048 and at least 512 rows run on the tensor cores as an
  *                  error-compensated TF32 product (three passes, fp32 accumulation, relative error of a few
- *                  1e-7 of sum |a||b|); products of 16384 rows or more first split the weight operand once
- *                  into the staged layout and fetch it with bulk copies (smaller ones re-split it per row
- *                  tile, which is cheaper than another launch), and with at most 128 output columns they also
+ *                  1e-7 of sum |a||b|); products of 16384 rows or more (or with several row tiles per SM
+ *                  and K >= 128) take the weight operand from an image of the staged layout, kept by the
+ *                  kernels that write the weights, and fetch it with bulk copies (smaller ones split it per
+ *                  row tile), and with at most 128 output columns they also
  *                  fetch the tiles of the row operand by tensor copies (products with 129 to 256 output columns
  *                  and K <= 128 run in that form as two groups of 128 columns); 2: the same kernels, pre-split
  *                  at every size; 0: fp32 FMA kernels everywhere
  *  use_graph       1: gcn_admm_step records one pass as a CUDA graph on first use and replays it (only when
- *                  the handle's stream is not the default stream and profiling is off); 2: the same, but
+ *                  the handle's stream is not the default stream and profiling is off; for calls of one
+ *                  pass from the third on); 2: the same, but
  *                  only for problems small enough for launch gaps to show (N x widest layer < 2^27);
  *                  0: plain launches
  *  schedule        0: Algorithm 1 (every W_l, then every Z_{l,m}, then U; Jacobi inside a pass);

@@ -1237,9 +1237,9 @@ __device__ __forceinline__ float warp_sum2(float v0, float v1, int lane) {
 // Persistent grid.
 //
 // Rows longer than `long_len` come as `n_items` items {row, first entry, one past the last, split}
-// (see k_spmm): an item of whole community segments (split < 0) is scored like a short row; an
+// (see k_spmm_wide): an item of whole community segments (split < 0) is scored like a short row; an
 // item that is one piece of a segment too long for one warp only leaves its part of K_m[i],
-// unscaled, in `scratch` (one padded row per item), and k_score_z_split scores the sum of the pieces.
+// unscaled, in `scratch` (one padded row per item), and k_close_z scores the sum of the pieces.
 
 // 2 (z - f(h)): twice the row's current error, formed once per row and reused by every segment.
 __device__ __forceinline__ float4 twice_error(const float4& h, const float4& z) {
