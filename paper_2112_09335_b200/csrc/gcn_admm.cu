@@ -821,7 +821,9 @@ struct gcn_admm {
     if (C[L] <= 4) OUTPUT(4, 1)
     else if (C[L] <= 8) OUTPUT(4, 2)
     else if (C[L] <= 16) OUTPUT(8, 2)
+    else if (C[L] <= 24) OUTPUT(8, 3)
     else if (C[L] <= 32) OUTPUT(8, 4)
+    else if (C[L] <= 40) OUTPUT(8, 5)
     else if (C[L] <= 48) OUTPUT(8, 6)
     else if (C[L] <= 64) OUTPUT(8, 8)
     else if (C[L] <= 96) OUTPUT(16, 6)
@@ -960,8 +962,18 @@ struct gcn_admm {
     end_pass();
   }
 
-  // Logits of Problem 1's forward pass with the stored W (N x ld_L, in B0 unless they are H_1).  The first layer's product is
-  // H_1 itself while the stored matrices agree; activations are taken as the rows are gathered.
+  void relu(const float* x, float* out, int ldx) {
+    const long long n4 = n * ldx / 4;
+    Scope sc(this, "relu", 1, 32.0 * n4, 0.0);
+    gk::k_relu<<<grid_for(n4), 256, 0, stream>>>((const float4*)x, (float4*)out, n4);
+    CU(cudaGetLastError());
+  }
+
+  // Logits of Problem 1's forward pass with the stored W (N x ld_L, in H_1, B0 or B1; B2 is free).  The first layer's product
+  // is H_1 itself while the stored matrices agree.  A (f(H) W) = (A f(H)) W: where the next layer is so much narrower that the
+  // gathered bytes it saves outweigh a sweep for f(H), the product comes first and its few columns are propagated.  A gather
+  // moves its entries at two to three times the sweep's rate; the line leaves that margin (13.8 k rows of 31 entries, 1000 to
+  // 10 columns: objective 275 -> 152 us; 2.45 M rows of 51, 256 to 47: 25 -> 19 ms).  Else activations are taken as the rows are gathered.
   const float* forward_logits() {
     const float* h = H[1];
     if (!fresh) {
@@ -969,9 +981,16 @@ struct gcn_admm {
       h = B0;
     }
     for (int l = 1; l < L; ++l) {
-      spmm(h, B1, ld[l], true);
-      gemm_nn(B1, ld[l], W[l + 1], ld[l + 1], Wt[l + 1], ld[l], B0, ld[l + 1], n, C[l + 1], C[l], &img_H[l + 1]);
-      h = B0;
+      float *const out = h == B0 ? B1 : B0, *const mid = out == B0 ? B1 : B0;
+      if (gi.nnz * (long long)(ld[l] - ld[l + 1]) >= 8 * n * ld[l]) {
+        relu(h, B2, ld[l]);
+        gemm_nn(B2, ld[l], W[l + 1], ld[l + 1], Wt[l + 1], ld[l], mid, ld[l + 1], n, C[l + 1], C[l], &img_H[l + 1]);
+        spmm(mid, out, ld[l + 1]);
+      } else {
+        spmm(h, B2, ld[l], true);
+        gemm_nn(B2, ld[l], W[l + 1], ld[l + 1], Wt[l + 1], ld[l], out, ld[l + 1], n, C[l + 1], C[l], &img_H[l + 1]);
+      }
+      h = out;
     }
     return h;
   }
@@ -1396,14 +1415,8 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
   for (int l = 1; l <= L; ++l) {
     if (l >= 2) h->spmm(h->Z[l - 1], h->P[l], h->ld[l - 1]);
     h->refresh_H(l);
-    const size_t bytes = rows * h->ld[l] * sizeof(float);
-    CU(cudaMemcpyAsync(h->Z[l], h->H[l], bytes, cudaMemcpyDeviceToDevice, h->stream));
-    if (l < L) {
-      const long long n4 = n * h->ld[l] / 4;
-      gcn_admm::Scope sc(h, "relu", 1, 32.0 * n4, 0.0);
-      gk::k_relu_inplace<<<h->grid_for(n4), 256, 0, h->stream>>>((float4*)h->Z[l], n4);
-      CU(cudaGetLastError());
-    }
+    if (l < L) h->relu(h->H[l], h->Z[l], h->ld[l]);
+    else CU(cudaMemcpyAsync(h->Z[l], h->H[l], rows * h->ld[l] * sizeof(float), cudaMemcpyDeviceToDevice, h->stream));
   }
   h->fresh = true;
   CU(h->stage.finish(h->stream));
@@ -1629,7 +1642,7 @@ int gcn_admm_predict(gcn_admm* h, float* logits, int* labels) {
     const float* const z = h->forward_logits();
     if (labels) {
       const int warps = 8;
-      int* d_lab = reinterpret_cast<int*>(h->B1);
+      int* d_lab = reinterpret_cast<int*>(h->B2);
       {
         gcn_admm::Scope sc(h, "row_argmax", 1, 4.0 * (double)h->n * h->ld[L], 0.0);
         gk::k_row_loss_argmax<<<(unsigned)cdiv(h->n, warps), warps * 32, 0, h->stream>>>(

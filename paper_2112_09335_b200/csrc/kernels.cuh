@@ -2130,11 +2130,11 @@ k_row_loss_argmax(const float* __restrict__ Zrows, const float* __restrict__ log
   }
 }
 
-// Y = relu(Y) in place.
-__global__ void k_relu_inplace(float4* __restrict__ Y, long long n4) {
+// Y = relu(X).
+__global__ void k_relu(const float4* __restrict__ X, float4* __restrict__ Y, long long n4) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n4;
        i += (long long)gridDim.x * blockDim.x) {
-    float4 y = Y[i];
+    float4 y = X[i];
     y.x = relu(y.x); y.y = relu(y.y); y.z = relu(y.z); y.w = relu(y.w);
     Y[i] = y;
   }

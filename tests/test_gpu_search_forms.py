@@ -10,7 +10,7 @@ from test_gpu_edge_cases import run_pair
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("classes", [1, 4, 5, 8, 9, 16, 17, 32, 33, 48, 49, 64, 65, 96, 97, 128])
+@pytest.mark.parametrize("classes", [1, 4, 5, 8, 9, 16, 17, 24, 25, 32, 33, 40, 41, 48, 49, 64, 65, 96, 97, 128])
 def test_output_widths(classes):
     run_pair(tiny_problem(20 + classes, n=90, widths=(6, 9, classes), n_comm=3), n_it=3)
 
