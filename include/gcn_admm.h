@@ -250,10 +250,12 @@ int gcn_admm_propagate_sharded(gcn_admm* h, int n_ranks, const float* x, int wid
  *  GCN_ADMM_ST_U      layer ignored float n x C_L
  *  GCN_ADMM_ST_TAU    layer 1..L   double [1]
  *  GCN_ADMM_ST_THETA  layer 1..L-1 double [M]
- *  GCN_ADMM_ST_PIPELINE_FLAG  layer ignored, int [1]: non-zero once a tensor-core product has given up one of
- *                     its bounded waits.  The next call that synchronises (objective, decisions, dense
- *                     products) then returns GCN_ADMM_ERR_CUDA once and clears the flag; the handle stays
- *                     usable.  Writable so that this path can be exercised without a failing kernel. */
+ *  GCN_ADMM_ST_PIPELINE_FLAG  layer ignored, int [1]: non-zero once a tensor-core product or a step-size
+ *                     search has given up one of its bounded waits.  The searches of later launches are then left out,
+ *                     and the next objective, decisions or dense product returns GCN_ADMM_ERR_CUDA once, clears the flag
+ *                     and zeroes the counters that kernels hand to each other.  The iterates are those of an
+ *                     incomplete pass: write W, Z, U, tau and theta back from a checkpoint and go on; the handle
+ *                     stays usable.  Writable so that this path can be exercised without a failing kernel. */
 enum { GCN_ADMM_ST_W = 0, GCN_ADMM_ST_Z, GCN_ADMM_ST_U, GCN_ADMM_ST_TAU, GCN_ADMM_ST_THETA, GCN_ADMM_ST_PIPELINE_FLAG };
 int gcn_admm_get_state(gcn_admm* h, int which, int layer, void* out);
 int gcn_admm_set_state(gcn_admm* h, int which, int layer, const void* in);

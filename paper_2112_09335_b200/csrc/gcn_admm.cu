@@ -263,6 +263,13 @@ struct gcn_admm {
     Start start;
   };
   std::vector<Want> wants;
+  // Counters that every complete launch leaves at zero for the next one, and their sizes: zeroed by check() after one that gave up.
+  std::vector<std::pair<void**, size_t>> counters;
+  template <typename T>
+  void want_counter(T*& slot, size_t count) {
+    want(slot, count, kZero);
+    counters.push_back({reinterpret_cast<void**>(&slot), std::max<size_t>(count, 1) * sizeof(T)});
+  }
   template <typename T>
   void want(T*& slot, size_t count, Start start = kPlain) {
     wants.push_back(Want{reinterpret_cast<void**>(&slot), std::max<size_t>(count, 1) * sizeof(T), nullptr, start});
@@ -1002,9 +1009,11 @@ struct gcn_admm {
     return r;
   }
   void check(const gk::Report& r) {
-    if (r.error != 0) {
+    if (r.error != 0) {   // a launch gave up and others may have left early: counters and products from scratch
       CU(cudaMemsetAsync(&report->error, 0, sizeof(int), stream));
-      CU(cudaMemsetAsync(grid_bar, 0, sizeof(gk::GridBar), stream));
+      CU(cudaMemsetAsync(&report->status, 0, sizeof(int), stream));   // decisions since then may have read anything
+      for (const auto& c : counters) CU(cudaMemsetAsync(*c.first, 0, c.second, stream));
+      fresh = false;
       throw Fail{GCN_ADMM_ERR_CUDA, r.error & gk::kErrGridBarrier ? "a step-size search gave up waiting for the rest of its grid"
                                                                   : "a tensor-core product gave up waiting on its pipeline"};
     }
@@ -1229,7 +1238,7 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
   for (size_t r = 0; r < lt.rows.size(); ++r)
     for (int k = 0; k < lt.rows[r].z; ++k) item_row[(size_t)(lt.rows[r].y + k)] = (int)r;
   h->want_table(h->d_item_row, item_row);
-  h->want(h->d_row_done, lt.rows.size(), gcn_admm::kZero);
+  h->want_counter(h->d_row_done, lt.rows.size());
   // split entries grouped by community (stable), for the ordered sums of the Z search
   std::vector<int> split_ptr((size_t)n_comm + 1, 0), split_order(lt.split.size());
   for (const auto& q : lt.split) ++split_ptr[(size_t)q.y + 1];
@@ -1260,8 +1269,8 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
     h->want_table(h->d_seg_chunks, seg.chunks);
     h->want_table(h->d_slot_ptr, seg.slot_ptr);
     h->want(h->slots, 2 * (size_t)seg.slot_ptr.back());
-    h->want(h->comm_done, n_comm, gcn_admm::kZero);
-    h->want(h->split_done, lt.split.size(), gcn_admm::kZero);
+    h->want_counter(h->comm_done, n_comm);
+    h->want_counter(h->split_done, lt.split.size());
   }
   if (n_layers >= 3) {
     const long long n_units = (long long)lt.items.size() + n;
@@ -1323,8 +1332,8 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
     h->want(h->side.grad, ge);
     h->want(h->side.grad_t, (size_t)h->C[L] * h->ld[L - 1], gcn_admm::kZero);
     h->want(h->side.red_part, std::max<size_t>((size_t)kSmCount * 8 * gk::kCand, (size_t)cdiv((long long)ge, 32) * 2));
-    h->want(h->side.ticket, 1, gcn_admm::kZero);
-    h->want(h->side.tile_tickets, kSmCount, gcn_admm::kZero);
+    h->want_counter(h->side.ticket, 1);
+    h->want_counter(h->side.tile_tickets, kSmCount);
     CU(gcn_admm_mem::Pool::get().take_stream(p.device, &h->side.stream));
     for (cudaEvent_t* e : {&h->side.begun, &h->side.w_done, &h->side.out_done, &h->side.done}) CU(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
   }
@@ -1364,14 +1373,14 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
   h->want_table(h->d_comm_block_ptr, cbp);
   h->want(h->z_chunk_part, (size_t)h->n_chunks * n_comm * gk::kCand);
   h->want(h->z_group_part, (size_t)kChunkGroups * n_comm * gk::kCand);
-  h->want(h->chunk_counter, 1, gcn_admm::kZero);
-  h->want(h->ticket, 1, gcn_admm::kZero);
-  h->want(h->tile_tickets, kSmCount, gcn_admm::kZero);
-  h->want(h->comm_tickets, n_comm, gcn_admm::kZero);
-  h->want(h->grid_bar, 1, gcn_admm::kZero);
+  h->want_counter(h->chunk_counter, 1);
+  h->want_counter(h->ticket, 1);
+  h->want_counter(h->tile_tickets, kSmCount);
+  h->want_counter(h->comm_tickets, n_comm);
+  h->want_counter(h->grid_bar, 1);
   h->want(h->red_part, std::max<size_t>({(size_t)kSmCount * 8 * gk::kCand, (size_t)h->n_zblocks * 3,
                                          (size_t)cdiv(n, 8) * 2, grad_blocks * 2}));
-  h->want(h->n_active, 1, gcn_admm::kZero);
+  h->want_counter(h->n_active, 1);
   h->want(h->d_pass, 1, gcn_admm::kZero);
   h->want(h->d_h1_age, 1, gcn_admm::kZero);
   h->want(h->skip_h1, 1, gcn_admm::kZero);

@@ -702,7 +702,9 @@ __global__ void k_resid_out(const float4* __restrict__ H, const float4* __restri
 // kernels of a pass and, on graphs of a few thousand nodes, most of its time.
 // ------------------------------------------------------------------------------------------
 // Grid-wide rendezvous of a cooperative launch (all blocks resident).  Every wait is bounded by elapsed clocks (a few
-// seconds); one that runs out raises *err and every block leaves the kernel.
+// seconds); one that runs out raises *err and every block leaves the kernel.  A launch that finds *err raised (by itself or by
+// any launch before it) leaves at once: the counters between launches, this one among them, may then hold anything until the
+// host has seen the flag and zeroed them.
 struct GridBar {
   unsigned arrived, generation;
 };
@@ -744,8 +746,10 @@ __device__ __forceinline__ bool grid_meet(GridBar* bar, int* err, F&& last) {
     }
   } else if (threadIdx.x == 0) {
     const long long t0 = clock64();
-    while (load_acquire(&bar->generation) == gen)
+    for (unsigned i = 1; load_acquire(&bar->generation) == gen; ++i) {
+      if ((i & 63u) == 0u && __ldcg(err) != 0) { s_ok = 0; break; }   // others have left or will not come
       if (clock64() - t0 > kGridWaitClocks) { s_ok = 0; atomicOr(err, kErrGridBarrier); break; }
+    }
   }
   __syncthreads();
   return s_ok != 0;
@@ -1041,6 +1045,7 @@ k_search_w_hidden(const SearchW p) {
   __shared__ double sh[kCand * 8], total[kCand];
   SearchCtl* const ctl = p.ctl;
   const long long first = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
+  if (__ldcg(p.err) != 0) return;   // see GridBar
   if (ctl->done) {                  // skipped: the same in every block
     if (first == 0) log_decision(p.log, 0, ctl);
   } else {
@@ -1606,16 +1611,19 @@ k_score_z(const int* __restrict__ row_ptr, const int* __restrict__ col,
 // The rest of the search, cooperative: closes the sweep that k_score_z has just made, makes and
 // closes further ones while a community is still searching, and moves the blocks.  The first sweep has a
 // kernel of its own because, compiled together with this one, its walk spills registers (2.4 M rows x 256: 14.9 against 13.6 ms).
+// The searches of a launch start together, so the sweep that scores the last of max_trials is the last one: *n_active alone
+// would not end the loop where a launch before this one gave up and left it too high.
 template <int V, int UN, int NC>
 __global__ void __launch_bounds__(256, (V <= 2 ? 3 : 1))
 k_close_z(const int* __restrict__ row_ptr, const int* __restrict__ col,
           const unsigned short* __restrict__ col_comm, const float* __restrict__ dinv,
           const float4* __restrict__ T, const float4* __restrict__ Hn, const float4* __restrict__ Zn, int ld4, int n, int use_smem, const int* __restrict__ chunk_ptr, int n_chunks,
           const int4* __restrict__ items, int n_items, int long_len, float4* scratch, const SearchZ sz) {
+  if (__ldcg(sz.err) != 0) return;   // see GridBar
   if (__ldcg(sz.n_active) > 0) {
-    for (;;) {
+    for (int scored = sz.a.cand;; scored += sz.a.cand) {
       if (!close_sweep<V, NC>(sz, n_chunks, dinv, scratch, Hn, Zn, ld4)) return;
-      if (__ldcg(sz.n_active) <= 0) break;   // changes only between the meetings of close_sweep
+      if (__ldcg(sz.n_active) <= 0 || scored >= sz.a.max_trials) break;   // *n_active changes only between the meetings of close_sweep
       score_sweep<V, UN, NC>(row_ptr, col, col_comm, dinv, T, Hn, Zn, ld4, sz.ctl, sz.n_comm, sz.chunk_part, use_smem, chunk_ptr,
                                   n_chunks, sz.chunk_counter, items, n_items, long_len, scratch);
       if (!grid_meet(sz.bar, sz.err, [] {})) return;
