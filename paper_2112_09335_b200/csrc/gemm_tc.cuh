@@ -151,6 +151,20 @@ __device__ __forceinline__ bool mbar_wait_abortable(uint32_t bar, uint32_t parit
   return false;
 }
 
+// Whether all `threads` threads that meet at named barrier 1 hold a true `ok`: the same answer in each of them.
+__device__ __forceinline__ bool all_agree(bool ok, int threads) {
+  uint32_t all;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 p, %1, 0;\n\t"
+      "bar.red.and.pred q, 1, %2, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(all)
+      : "r"((uint32_t)ok), "r"(threads)
+      : "memory");
+  return all != 0u;
+}
+
 template <int NT>
 struct WsCfg {
   static constexpr int kSets = NT > 128 ? 1 : 2;                        // accumulator sets (main + correction each)
@@ -488,7 +502,10 @@ k_gemm_tc_ws(const float* __restrict__ A, int lda, const float* __restrict__ Bk,
     float* const dst = gridDim.z == 1 ? C : partial + (size_t)blockIdx.z * M * ldc;
     for (int tile_i = 0; tile_i < my_tiles; ++tile_i) {
       const int set = tile_i % SETS;
-      if (!__all_sync(0xffffffffu, mbar_wait_abortable(bar_acc_full + 8 * set, (tile_i / SETS) & 1, abortp))) break;
+      bool ok = __all_sync(0xffffffffu, mbar_wait_abortable(bar_acc_full + 8 * set, (tile_i / SETS) & 1, abortp));
+      // The parts of a tile are added up behind named barriers without a bound of their own: all of these warps come to them or none.
+      if (gridDim.z > 1) ok = all_agree(ok, Cfg::kEpiWarps * 32);
+      if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const long long row0 = (long long)(blockIdx.x + tile_i * gridDim.x) * kBlockM + quarter * 32;
 #pragma unroll 1
@@ -764,7 +781,7 @@ k_gemm_tn_tc(const float* __restrict__ A, int lda, const float* __restrict__ B, 
   // ---------------- epilogue: warps 0-3, one tensor-memory lane (= column of A) per thread ----------------
   if (warp < 4) {
     bool ok = true;
-    if (total > 0) ok = mbar_wait_abortable(bar_acc, 0, abortp);
+    if (total > 0) ok = __all_sync(0xffffffffu, mbar_wait_abortable(bar_acc, 0, abortp));   // the loads below are the whole warp's
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const int ka = ka0 + warp * 32 + lane;
     float* dst = part + ((long long)blockIdx.y * Ka + ka) * ldp;
