@@ -37,6 +37,7 @@ constexpr int kBlockM = 128;
 constexpr int kChunkK = 32;                 // floats per K chunk (128 bytes)
 constexpr int kATileBytes = kBlockM * kChunkK * 4;     // 16 KiB, one of hi / lo
 constexpr long long kWaitClocks = 1LL << 31;   // bound of every mbarrier wait, in SM clocks (about a second)
+constexpr long long kDrainClocks = 1LL << 22;  // bound of the waits of a block that has given up for what it still has in flight
 
 // First statement of a kernel that may be launched with programmatic serialisation: its grid may start while the one before
 // it on the stream still runs, waits here until that one is complete and its writes are seen, and only then lets the grid
@@ -165,6 +166,31 @@ __device__ __forceinline__ bool all_agree(bool ok, int threads) {
   return all != 0u;
 }
 
+// A block that gives up (abort flag raised, all roles past the closing barrier) still owns what it has started: bulk copies into its
+// shared memory and MMAs on its tensor memory.  It waits for them, with a bound again, before it lets go of either.
+__device__ __forceinline__ void drain_wait(uint32_t bar, uint32_t parity) {
+  const long long t0 = clock64();
+  uint32_t ok = 0;
+  while (!ok && clock64() - t0 < kDrainClocks)
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+}
+// Copies: `started` of them, number i reporting to barrier i mod `slots` (a stage some producer never filled has no such end:
+// the bound covers it).  By one thread.
+__device__ __noinline__ void drain_copies(uint32_t bars, int slots, int started) {
+  for (int i = max(0, started - slots); i < started; ++i) drain_wait(bars + 8 * (i % slots), (uint32_t)(i / slots) & 1u);
+}
+// MMAs: by the thread that issued them, on a barrier nothing else uses.
+__device__ __noinline__ void drain_mmas(uint32_t bar) {
+  mma_commit(bar);
+  drain_wait(bar, 0);
+}
+
 template <int NT>
 struct WsCfg {
   static constexpr int kSets = NT > 128 ? 1 : 2;                        // accumulator sets (main + correction each)
@@ -257,9 +283,9 @@ k_gemm_tc_ws(const float* __restrict__ A, int lda, const float* __restrict__ Bk,
   if (skip != nullptr && *skip) return;
 
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t bars[2 * S + 4 + 2 * R];      // full[S], empty[S], acc_full[2], acc_empty[2], raw_full[R], raw_empty[R]
+  __shared__ __align__(8) uint64_t bars[2 * S + 5 + 2 * R];      // full[S], empty[S], acc_full[2], acc_empty[2], raw_full[R], raw_empty[R], drain
   __shared__ uint32_t tmem_base_slot;
-  __shared__ int abort_flag, last_part;
+  __shared__ int abort_flag, last_part, copies;   // copies: chunks whose bulk copies have been started
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t smem_base = smem_u32(smem);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -276,7 +302,8 @@ k_gemm_tc_ws(const float* __restrict__ A, int lda, const float* __restrict__ Bk,
     for (int s = 0; s < S; ++s) { mbar_init(bar_full + 8 * s, 8); mbar_init(bar_empty + 8 * s, 1); }   // full: one arrival per producer warp
     for (int r = 0; r < R; ++r) { mbar_init(bar_raw_full + 8 * r, 1); mbar_init(bar_raw_empty + 8 * r, 1); }
     for (int a = 0; a < 2; ++a) { mbar_init(bar_acc_full + 8 * a, 1); mbar_init(bar_acc_empty + 8 * a, Cfg::kEpiWarps); }
-    abort_flag = 0;
+    mbar_init(bar_raw_empty + 8 * R, 1);
+    abort_flag = copies = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == Cfg::kMmaWarp) {
@@ -408,6 +435,7 @@ k_gemm_tc_ws(const float* __restrict__ A, int lda, const float* __restrict__ Bk,
           asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                        ::"r"(dst), "l"(src), "r"(bytes), "r"(bar_full + 8 * stage)
                        : "memory");
+          copies = j + 1;
         }
         if (++st_kc == kc_count) st_kc = 0;
         store_chunk(stage, ra[d], rb[d]);
@@ -435,6 +463,7 @@ k_gemm_tc_ws(const float* __restrict__ A, int lda, const float* __restrict__ Bk,
         asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                      ::"r"(dst_a + (uint32_t)kATileBytes), "l"(b_src + (size_t)kc * b_bytes), "r"(b_bytes), "r"(raw_bar)
                      : "memory");
+        copies = j + 1;
         if (++kc == kc_count) { kc = 0; tile += gridDim.x; }
         if (++slot == R) { slot = 0; empty_parity ^= 1u; }
       }
@@ -568,7 +597,14 @@ k_gemm_tc_ws(const float* __restrict__ A, int lda, const float* __restrict__ Bk,
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (tid == 0 && abort_flag) atomicExch(error_flag, 1);
+  if (abort_flag) {
+    if (tid == 0) {
+      atomicOr(error_flag, 1);
+      if (IMG) drain_copies(TMA ? bar_raw_full : bar_full, TMA ? R : S, copies);
+    }
+    if (tid == Cfg::kMmaWarp * 32) drain_mmas(bar_raw_empty + 8 * R);
+    __syncthreads();
+  }
   if (warp == Cfg::kMmaWarp) {
     __syncwarp();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(Cfg::kTmemCols) : "memory");
@@ -634,7 +670,7 @@ k_gemm_tn_tc(const float* __restrict__ A, int lda, const float* __restrict__ B, 
   static_assert(NT % 16 == 0 && NT <= 256, "NT");
 
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t bars[2 * S + 1];       // full[S], empty[S], acc_full
+  __shared__ __align__(8) uint64_t bars[2 * S + 2];       // full[S], empty[S], acc_full, drain
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -645,6 +681,7 @@ k_gemm_tn_tc(const float* __restrict__ A, int lda, const float* __restrict__ B, 
   if (tid == 0) {
     for (int s = 0; s < S; ++s) { mbar_init(bar_full + 8 * s, 8); mbar_init(bar_empty + 8 * s, 1); }   // full: one arrival per producer warp
     mbar_init(bar_acc, 1);
+    mbar_init(bar_acc + 8, 1);
     abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -812,7 +849,11 @@ k_gemm_tn_tc(const float* __restrict__ A, int lda, const float* __restrict__ B, 
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (tid == 0 && abort_flag) atomicExch(error_flag, 1);
+  if (abort_flag) {
+    if (tid == 0) atomicOr(error_flag, 1);
+    if (tid == 8 * 32) drain_mmas(bar_acc + 8);
+    __syncthreads();
+  }
   if (warp == 8) {
     __syncwarp();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(Cfg::kTmemCols) : "memory");
