@@ -113,6 +113,17 @@ bool make_a_tile_map(const float* A, long long rows, int ld, CUtensorMap* map) {
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Lets `kernel` be launched on the current device (`device`) with `smem` bytes of dynamic shared memory.  The limit belongs to the
+// function, not to a handle, and handles of other sizes are stepped in between: it is only ever raised.
+void allow_shared(int device, const void* kernel, size_t smem) {
+  static std::mutex mutex;
+  static std::map<std::pair<int, const void*>, size_t> most;
+  std::lock_guard<std::mutex> lock(mutex);
+  size_t& limit = most[{device, kernel}];
+  limit = std::max(limit, smem);
+  if (limit > 48 * 1024) CU(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit));
+}
+
 bool is_device_pointer(const void* p) {
   cudaPointerAttributes a;
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
@@ -624,7 +635,7 @@ struct gcn_admm {
   int resident_blocks(const void* kernel, int threads, size_t smem) {
     auto it = resident_cache.find({kernel, smem});
     if (it != resident_cache.end()) return it->second;
-    if (smem > 48 * 1024) CU(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    allow_shared(p.device, kernel, smem);
     int per_sm = 0;
     CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem));
     if (per_sm < 1) throw Fail{GCN_ADMM_ERR_CUDA, "a kernel does not fit the device"};

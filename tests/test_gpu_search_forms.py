@@ -5,6 +5,7 @@ import numpy as np
 import pytest
 
 from conftest import tiny_problem
+from paper_2112_09335_b200 import binding
 from test_gpu_edge_cases import run_pair
 
 pytestmark = pytest.mark.gpu
@@ -28,3 +29,31 @@ def test_many_chunks_and_a_search_of_several_sweeps():
 @pytest.mark.parametrize("n", [900, 1100, 5000])
 def test_few_and_many_splits_of_the_weight_gradient(n):
     run_pair(tiny_problem(62, n=n, widths=(33, 9, 4), n_comm=4, p=3.0 / n), n_it=2)
+
+
+@pytest.mark.parametrize("width,more,fewer", [(130, 200, 130), (300, 80, 61), (520, 9, 5)])
+def test_handles_with_different_shared_memory_needs(width, more, fewer):
+    """The scoring of layer 1 takes 8 warps x (2 V x 512 B + 32 B per community) + 16 B per community of dynamic shared memory
+    (V = 2, 4, 8 at these widths of layer 2), above 48 KB for both handles of a pair.  The limit a launch is held to belongs to
+    the kernel: the handle with fewer communities, stepped in between, must not lower it for the other."""
+    def steps(handles):
+        for _ in range(2):
+            for g in handles:
+                g.step(1)
+        return [[g.get_state(binding.ST_Z, 1), g.weights(2)] for g in handles]
+
+    def make(n_comm):
+        pr = tiny_problem(63, n=800, widths=(5, 6, width, 3), n_comm=n_comm, p=0.01)
+        return binding.GcnAdmm(pr["n"], pr["row_ptr"], pr["col_idx"], pr["X"].astype(np.float32), pr["y"], pr["mask"], pr["widths"],
+                               pr["n_comm"], pr["community"], [w.astype(np.float32) for w in pr["W"]], nu=0.05, rho=0.08, use_graph=0)
+    a, b = make(more), make(fewer)
+    alone = steps([a])
+    a.destroy()
+    alone += steps([b])
+    b.destroy()
+    pair = [make(more), make(fewer)]
+    together = steps(pair)
+    for g in pair:
+        g.destroy()
+    for got, want in zip(together, alone):
+        assert all(np.array_equal(x, y) for x, y in zip(got, want))
