@@ -148,7 +148,16 @@ int gcn_admm_weights(gcn_admm* h, int layer, float* out);
  * (row argmax, ties to the lowest class).  Either may be NULL.  Host pointers, original order. */
 int gcn_admm_predict(gcn_admm* h, float* logits, int* labels);
 
+/* Frees the handle after its work has finished.  Device memory and page-locked staging memory of destroyed handles stay
+ * with the process for later handles (their allocation costs more than a small training run): device slabs up to 3 GB over
+ * all devices, four staging buffers of 12 MB and four streams.  What is idle goes back to the driver when an allocation of
+ * this library fails, by the call below, and at exit. */
 void gcn_admm_destroy(gcn_admm* h);
+
+/* Gives all memory and streams that destroyed handles have left idle back to the driver, on every device: for a process
+ * whose other code needs them (another library's allocator cannot ask for them by itself).  Live handles are untouched;
+ * may be called from any thread. */
+void gcn_admm_release_idle(void);
 
 /* Text of the last error of this handle (or of the last failed create when h is NULL). */
 const char* gcn_admm_last_error(const gcn_admm* h);

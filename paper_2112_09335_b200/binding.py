@@ -1,7 +1,7 @@
 """ctypes binding of ``libgcn_admm.so``: argument marshalling only.
 
 Every function of ``include/gcn_admm.h`` has a counterpart of the same name on ``GcnAdmm``
-(without the ``gcn_admm_`` prefix).  Nothing is computed here; the library must have been built
+(without the ``gcn_admm_`` prefix; ``release_idle``, which takes no handle, is a function of this module).  Nothing is computed here; the library must have been built
 (``python -m paper_2112_09335_b200.build``) or loading fails with an error -- there is no fallback.
 """
 from __future__ import annotations
@@ -16,7 +16,7 @@ LIB_PATH = os.path.join(HERE, "libgcn_admm.so")
 
 EXPORTS = [
     "gcn_admm_default_params", "gcn_admm_create", "gcn_admm_step", "gcn_admm_objective", "gcn_admm_weights",
-    "gcn_admm_predict", "gcn_admm_destroy", "gcn_admm_last_error", "gcn_admm_propagate", "gcn_admm_index",
+    "gcn_admm_predict", "gcn_admm_destroy", "gcn_admm_release_idle", "gcn_admm_last_error", "gcn_admm_propagate", "gcn_admm_index",
     "gcn_admm_get_state", "gcn_admm_set_state", "gcn_admm_step_block", "gcn_admm_decisions",
     "gcn_admm_launches", "gcn_admm_profile", "gcn_admm_profile_read", "gcn_admm_propagate_static", "gcn_admm_dense_product", "gcn_admm_dense_product_tn",
     "gcn_admm_shard_plan", "gcn_admm_propagate_sharded",
@@ -63,6 +63,8 @@ def load():
     lib.gcn_admm_predict.argtypes = [vp, vp, vp]
     lib.gcn_admm_destroy.argtypes = [vp]
     lib.gcn_admm_destroy.restype = None
+    lib.gcn_admm_release_idle.argtypes = []
+    lib.gcn_admm_release_idle.restype = None
     lib.gcn_admm_last_error.argtypes = [vp]
     lib.gcn_admm_last_error.restype = C.c_char_p
     lib.gcn_admm_propagate.argtypes = [vp, vp, i32, vp]
@@ -96,6 +98,11 @@ def default_params() -> Params:
     p = Params()
     load().gcn_admm_default_params(C.byref(p))
     return p
+
+
+def release_idle():
+    """Gives device and page-locked memory that destroyed handles have left idle back to the driver."""
+    load().gcn_admm_release_idle()
 
 
 class GcnAdmm:

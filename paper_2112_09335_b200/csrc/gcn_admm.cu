@@ -75,7 +75,9 @@ struct Fail {
 template <typename T>
 T* dalloc(size_t count) {
   void* p = nullptr;
-  cudaError_t e = cudaMalloc(&p, std::max<size_t>(count, 1) * sizeof(T));
+  int device = 0;
+  cudaError_t e = cudaGetDevice(&device);
+  if (e == cudaSuccess) e = gcn_admm_mem::Pool::get().allocate(device, std::max<size_t>(count, 1) * sizeof(T), &p);
   if (e != cudaSuccess)
     throw Fail{e == cudaErrorMemoryAllocation ? GCN_ADMM_ERR_ALLOC : GCN_ADMM_ERR_CUDA,
                std::string("cudaMalloc: ") + cudaGetErrorString(e)};
@@ -1525,6 +1527,11 @@ void gcn_admm_destroy(gcn_admm* h) {
   }
   cudaGetLastError();
   delete h;
+}
+
+void gcn_admm_release_idle(void) {
+  gcn_admm_mem::Pool::get().release();
+  cudaGetLastError();
 }
 
 const char* gcn_admm_last_error(const gcn_admm* h) { return h ? h->err.c_str() : g_create_error.c_str(); }

@@ -8,7 +8,8 @@
 //
 // Slabs, staging buffers and streams of destroyed handles are kept for later ones up to a fixed amount (kIdleSlabBytes,
 // kIdleStages; the oldest go first), under a lock, and only after the work that used them has finished; the rest goes back
-// to the driver at once, everything at exit or when an allocation fails.
+// to the driver at once, the idle slabs of a device when an allocation of the library fails there, and everything when the
+// caller asks for it (gcn_admm_release_idle) and at exit.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -56,13 +57,17 @@ class Pool {
       }
     }
     void* p = nullptr;
-    cudaError_t e = cudaMalloc(&p, bytes);
-    if (e == cudaErrorMemoryAllocation) {
-      cudaGetLastError();
-      trim(device);
-      e = cudaMalloc(&p, bytes);
-    }
+    const cudaError_t e = allocate(device, bytes, &p);
     if (e == cudaSuccess) *out = Slab{device, static_cast<char*>(p), bytes};
+    return e;
+  }
+  // cudaMalloc on the current device (`device`); where that fails, once more without the idle slabs.
+  cudaError_t allocate(int device, std::size_t bytes, void** out) {
+    cudaError_t e = cudaMalloc(out, bytes);
+    if (e == cudaErrorMemoryAllocation && release_slabs(device)) {
+      cudaGetLastError();
+      e = cudaMalloc(out, bytes);
+    }
     return e;
   }
   // The slab's device is current and no work uses the slab any more.
@@ -126,22 +131,34 @@ class Pool {
     }
     cudaStreamDestroy(s);
   }
-  ~Pool() {   // at exit the driver may already be gone: its error is of no consequence then
-    for (const Slab& s : idle_) cudaFree(s.base);
-    for (char* p : stages_) cudaFreeHost(p);
-    for (const auto& s : streams_) cudaStreamDestroy(s.second);
+  // Gives everything idle back to the driver.
+  void release() {
+    release_slabs(kAnyDevice);
+    std::vector<char*> stages;
+    std::vector<std::pair<int, cudaStream_t>> streams;
+    {
+      std::lock_guard<std::mutex> lock(mutex_);
+      stages.swap(stages_);
+      streams.swap(streams_);
+    }
+    for (char* p : stages) cudaFreeHost(p);
+    for (const auto& s : streams) cudaStreamDestroy(s.second);
   }
+  ~Pool() { release(); }   // at exit the driver may already be gone: its error is of no consequence then
 
  private:
-  void trim(int device) {
+  static constexpr int kAnyDevice = -1;
+  // Whether there was anything to give back.
+  bool release_slabs(int device) {
     std::vector<Slab> out;
     {
       std::lock_guard<std::mutex> lock(mutex_);
       for (auto it = idle_.begin(); it != idle_.end();)
-        if (it->device == device) { out.push_back(*it); idle_bytes_ -= it->size; it = idle_.erase(it); }
+        if (device == kAnyDevice || it->device == device) { out.push_back(*it); idle_bytes_ -= it->size; it = idle_.erase(it); }
         else ++it;
     }
     for (const Slab& s : out) cudaFree(s.base);
+    return !out.empty();
   }
   std::mutex mutex_;
   std::vector<Slab> idle_;

@@ -66,3 +66,34 @@ def test_handles_on_recycled_memory_and_from_threads():
     for t in threads:
         t.join()
     assert not bad
+
+
+def test_idle_memory_goes_back_on_request():
+    """A destroyed handle's slab stays with the process until release_idle(); a live handle keeps its own."""
+    import torch
+    small, big = tiny_problem(73, n=300, widths=(7, 11, 4), n_comm=3), tiny_problem(74, n=5000, widths=(7, 4000, 4), n_comm=3, p=6e-4)
+
+    def free():
+        torch.cuda.synchronize()
+        return torch.cuda.mem_get_info()[0]
+
+    for pr in (big, small):                         # kernels and the streams of two handles are loaded and made
+        g = handle(pr)
+        g.step(2)
+        g.destroy()
+    binding.release_idle()
+    before = free()
+    live = handle(small)
+    live.step(2)
+    want = live.get_state(binding.ST_U)
+    g = handle(big)
+    g.step(2)
+    g.destroy()
+    slab = 5000 * 4000 * 4 * 5                       # a good part of it: Z_1, H_1 and three scratch matrices
+    assert free() < before - slab
+    binding.release_idle()
+    assert free() > before - (32 << 20)              # the live handle's own slab and what the driver rounds up
+    assert np.array_equal(live.get_state(binding.ST_U), want)
+    live.step(1)
+    assert np.isfinite(live.objective()).all()
+    live.destroy()
