@@ -12,6 +12,7 @@
 // caller asks for it (gcn_admm_release_idle) and at exit.
 #pragma once
 #include <cuda_runtime.h>
+#include <omp.h>
 
 #include <algorithm>
 #include <cstddef>
@@ -167,12 +168,13 @@ class Pool {
   std::vector<std::pair<int, cudaStream_t>> streams_;
 };
 
-// memcpy by several threads where it pays (a core moves about 10 GB/s, less into pages that are touched first here).
+// memcpy by several threads where it pays (a core moves about 10 GB/s, less into pages that are touched first here): at most
+// eight, and no more than the caller allows OpenMP (OMP_NUM_THREADS, omp_set_num_threads).
 inline void copy_bytes(void* dst, const void* src, std::size_t bytes) {
   constexpr std::size_t kPiece = (std::size_t)256 << 10;
   if (bytes < 4 * kPiece) { std::memcpy(dst, src, bytes); return; }
   const long long pieces = (long long)((bytes + kPiece - 1) / kPiece);
-#pragma omp parallel for schedule(static) num_threads(8)
+#pragma omp parallel for schedule(static) num_threads(std::min(8, omp_get_max_threads()))
   for (long long i = 0; i < pieces; ++i) {
     const std::size_t at = (std::size_t)i * kPiece;
     std::memcpy(static_cast<char*>(dst) + at, static_cast<const char*>(src) + at, std::min(kPiece, bytes - at));

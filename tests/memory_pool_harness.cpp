@@ -1,8 +1,9 @@
-// Host-only program for test_memory_pool.py: the pool of memory.hpp on a stand-in for the CUDA runtime whose device memory is
+// Host-only program for test_memory_pool.py: with an argument, the threads of the process after a copy of that many bytes; else the pool of memory.hpp on a stand-in for the CUDA runtime whose device memory is
 // a byte count with a limit.
 #include <cstdio>
 #include <cstdlib>
 #include <map>
+#include <vector>
 
 #include "memory.hpp"
 
@@ -29,7 +30,19 @@ cudaError_t CUDARTAPI cudaGetLastError() { return cudaSuccess; }
 #define NEED(c) \
   if (!(c)) { std::printf("line %d: %s\n", __LINE__, #c); return 1; }
 
-int main() {
+static int threads_after_copy(std::size_t bytes) {
+  std::vector<char> from(bytes, 7), to(bytes);
+  gcn_admm_mem::copy_bytes(to.data(), from.data(), bytes);
+  int n = -1;
+  char line[256];
+  std::FILE* f = std::fopen("/proc/self/status", "r");
+  while (f && std::fgets(line, sizeof line, f)) std::sscanf(line, "Threads: %d", &n);
+  if (f) std::fclose(f);
+  return to == from ? n : -1;
+}
+
+int main(int argc, char** argv) {
+  if (argc > 1) { std::printf("%d\n", threads_after_copy(std::strtoull(argv[1], nullptr, 10))); return 0; }
   using namespace gcn_admm_mem;
   constexpr std::size_t GB = (std::size_t)1 << 30;
   Pool& pool = Pool::get();
