@@ -198,7 +198,7 @@ struct gcn_admm {
   std::vector<int> C, ld;   // widths C_0..C_L and their padded leading dimensions
   int max_ld = 0;
   GraphIndex gi;
-  std::vector<gcn_admm_mem::Slab> slabs;   // device memory: one slab for everything, more only for workspaces that grow
+  gcn_admm_mem::Slab slab;                 // device memory: everything but wide_sums
   gcn_admm_mem::Stage stage;               // page-locked staging of host buffers
 
   int *d_row_ptr = nullptr, *d_col = nullptr, *d_row_comm = nullptr, *d_perm = nullptr, *d_inv = nullptr;
@@ -211,6 +211,7 @@ struct gcn_admm {
   int n_items = 0, n_split = 0, n_long = 0, long_len = 0;
   float* item_sums = nullptr;             // n_items x max_ld
   size_t item_sums_elems = 0;
+  gcn_admm_mem::Slab wide_sums;           // the same for the widest matrix gcn_admm_propagate was given, where that is wider than every layer
   unsigned char* d_train = nullptr;
   int* d_train_rows = nullptr;            // new ids of the training rows, ascending
   float* d_fista_momentum = nullptr;      // (t_j - 1) / t_{j+1}, j = 1..fista_iters
@@ -292,13 +293,12 @@ struct gcn_admm {
     static_assert(sizeof(T) == sizeof(typename V::value_type), "a table is uploaded as it is");
     wants.push_back(Want{reinterpret_cast<void**>(&slot), std::max<size_t>(v.size(), 1) * sizeof(T), v.empty() ? nullptr : v.data(), kTable});
   }
-  char* take_slab(size_t bytes) {
+  gcn_admm_mem::Slab take_slab(size_t bytes) {
     gcn_admm_mem::Slab slab;
     const cudaError_t e = gcn_admm_mem::Pool::get().take(p.device, bytes, &slab);
     if (e != cudaSuccess)
       throw Fail{e == cudaErrorMemoryAllocation ? GCN_ADMM_ERR_ALLOC : GCN_ADMM_ERR_CUDA, std::string("cudaMalloc: ") + cudaGetErrorString(e)};
-    slabs.push_back(slab);
-    return slab.base;
+    return slab;
   }
   void commit() {
     std::stable_sort(wants.begin(), wants.end(), [](const Want& a, const Want& b) { return a.start < b.start; });
@@ -310,7 +310,8 @@ struct gcn_admm {
       total += (w.bytes + 255) / 256 * 256;
       if (w.start == kZero) zero_end = total;
     }
-    char* const base = take_slab(total);
+    slab = take_slab(total);
+    char* const base = slab.base;
     for (size_t k = 0; k < wants.size(); ++k) {
       *wants[k].slot = base + at[k];
       if (wants[k].start == kTable && wants[k].src) CU(stage.put(base + at[k], wants[k].src, wants[k].bytes, stream));
@@ -333,12 +334,12 @@ struct gcn_admm {
   }
 
   // out = A~ x for dense n x width device matrices in the caller's row order, in vectors as wide as the width and
-  // both addresses allow.
-  void propagate_dense(const float* x, int width, float* out) {
+  // both addresses allow.  `wide`: long rows may go through wide_sums; the caller then waits for the result.
+  void propagate_dense(const float* x, int width, float* out, bool wide) {
     char name[48];
     std::snprintf(name, sizeof name, "spmm@%d", ldpad(width));
     Scope sc(this, name, 1, 4.0 * gi.nnz + 8.0 * n + 8.0 * (double)n * width, 2.0 * (double)gi.nnz * width);
-    const GatherGraph g = gather_graph(ldpad(width));
+    const GatherGraph g = gather_graph(ldpad(width), wide);
     const uintptr_t low = reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(out) | ((uintptr_t)width * sizeof(float));
     if ((low & 15) == 0) spmm_tables<4, true>(g, x, out, width / 4);
     else if ((low & 7) == 0) spmm_tables<2, true>(g, x, out, width / 2);
@@ -355,18 +356,24 @@ struct gcn_admm {
     const int* item_row;
     int* row_done;
     int n, n_items, n_long, long_len;
+    float* item_sums;
   };
-  GatherGraph gather_graph(int ldw) const {
-    const bool cut = n_items > 0 && (size_t)n_items * ldw <= item_sums_elems;
-    return GatherGraph{d_row_ptr, d_col, d_row_order, d_perm, d_dinv, d_items, d_long_rows, d_item_row, d_row_done,
-                       (int)n, cut ? n_items : 0, cut ? n_long : 0, cut ? long_len : INT_MAX};
-  }
-  // Room for the items' sums at ldw padded columns (a workspace the handle keeps).
-  void grow_item_sums(int ldw) {
+  GatherGraph gather_graph(int ldw, bool wide = false) const {
     const size_t need = (size_t)n_items * ldw;
-    if (need <= item_sums_elems) return;
-    item_sums = reinterpret_cast<float*>(take_slab(need * sizeof(float)));   // the old one stays until destroy: kernels in flight may hold it
-    item_sums_elems = need;
+    float* const room = need <= item_sums_elems ? item_sums : wide && need * sizeof(float) <= wide_sums.size ? reinterpret_cast<float*>(wide_sums.base) : nullptr;
+    const bool cut = n_items > 0 && room != nullptr;
+    return GatherGraph{d_row_ptr, d_col, d_row_order, d_perm, d_dinv, d_items, d_long_rows, d_item_row, d_row_done,
+                       (int)n, cut ? n_items : 0, cut ? n_long : 0, cut ? long_len : INT_MAX, room};
+  }
+  // Room for the items' sums at ldw padded columns.  Passes, recorded ones too, and callers under capture hold item_sums, which
+  // therefore stays what it is; wide_sums serves calls that wait for their result, so a larger one may take its place.
+  void grow_wide_sums(int ldw) {
+    const size_t need = (size_t)n_items * ldw;
+    if (need <= item_sums_elems || need * sizeof(float) <= wide_sums.size) return;
+    CU(cudaStreamSynchronize(stream));
+    gcn_admm_mem::Pool::get().give(wide_sums);
+    wide_sums = gcn_admm_mem::Slab{};
+    wide_sums = take_slab(need * sizeof(float));
   }
 
   template <typename T> struct Same { using type = T; };   // keeps a parameter out of template deduction
@@ -410,7 +417,7 @@ struct gcn_admm {
   void spmm_tables(const GatherGraph& g, const float* xf, float* outf, int ldv) {
     using T = typename gk::Vec<VEC>::T;
     const T* x = reinterpret_cast<const T*>(xf);
-    T *out = reinterpret_cast<T*>(outf), *scratch = reinterpret_cast<T*>(item_sums);
+    T *out = reinterpret_cast<T*>(outf), *scratch = reinterpret_cast<T*>(g.item_sums);
     const int ld4 = (int)cdiv((long long)ldv * VEC, 4);
     const long long units = (long long)g.n + g.n_items;
     in_pass = !MAPPED;   // the caller's matrices: a call of its own
@@ -1522,7 +1529,7 @@ void gcn_admm_destroy(gcn_admm* h) {
     for (cudaEvent_t e : {h->side.begun, h->side.w_done, h->side.out_done, h->side.done})
       if (e) cudaEventDestroy(e);
     for (cudaEvent_t e : h->event_pool) cudaEventDestroy(e);
-    for (const gcn_admm_mem::Slab& q : h->slabs) gcn_admm_mem::Pool::get().give(q);
+    for (const gcn_admm_mem::Slab& q : {h->slab, h->wide_sums}) gcn_admm_mem::Pool::get().give(q);
     h->stage.close();
   }
   cudaGetLastError();
@@ -1688,9 +1695,9 @@ int gcn_admm_propagate(gcn_admm* h, const float* x, int width, float* out) {
     if (!x || !out || width < 1 || width > kMaxWidth) throw Fail{GCN_ADMM_ERR_ARG, "bad argument"};
     const bool dev_in = is_device_pointer(x), dev_out = is_device_pointer(out);
     if (dev_in != dev_out) throw Fail{GCN_ADMM_ERR_ARG, "x and out must both be host or both be device pointers"};
-    h->grow_item_sums(ldpad(width));
+    h->grow_wide_sums(ldpad(width));
     if (dev_in) {
-      h->propagate_dense(x, width, out);
+      h->propagate_dense(x, width, out, true);
       CU(cudaStreamSynchronize(h->stream));
       return;
     }
@@ -1703,7 +1710,7 @@ int gcn_admm_propagate(gcn_admm* h, const float* x, int width, float* out) {
       b = fits ? h->B1 : dalloc<float>(elems);
       CU(h->stage.put(a, x, bytes, h->stream));
       CU(h->stage.flush(h->stream));
-      h->propagate_dense(a, width, b);
+      h->propagate_dense(a, width, b, true);
       CU(h->stage.get(out, b, bytes, bytes, 1, h->stream));
       CU(h->stage.finish(h->stream));
       CU(cudaStreamSynchronize(h->stream));
@@ -1799,7 +1806,7 @@ int gcn_admm_propagate_static(gcn_admm* h, const float* x, int width, float* out
       explicit Untimed(gcn_admm* h_) : h(h_), saved(h_->profiling) { h->profiling = false; }
       ~Untimed() { h->profiling = saved; }
     } untimed(h);
-    h->propagate_dense(x, width, out);
+    h->propagate_dense(x, width, out, false);
   });
 }
 
@@ -1933,7 +1940,7 @@ int gcn_admm_propagate_sharded(gcn_admm* h, int n_ranks, const float* x, int wid
         }
         if (n_own > 0) {
           gcn_admm::Scope sc(h, "spmm.sharded", 1, 0.0, 0.0);
-          h->spmm_tables<4, false>(gcn_admm::GatherGraph{d_rp, d_cl, d_order, nullptr, d_dv, nullptr, nullptr, nullptr, nullptr, n_own, 0, 0, INT_MAX},
+          h->spmm_tables<4, false>(gcn_admm::GatherGraph{d_rp, d_cl, d_order, nullptr, d_dv, nullptr, nullptr, nullptr, nullptr, n_own, 0, 0, INT_MAX, nullptr},
                          xl, b + (size_t)lo * ldw, ldw / 4);
         }
         CU(cudaStreamSynchronize(h->stream));   // the host vectors of this rank go out of scope

@@ -4,6 +4,7 @@ segments of the Z scoring), and the results must still match the fp64 oracle and
 import numpy as np
 import pytest
 
+from conftest import tiny_problem
 from oracle import gcn_admm_oracle as orc
 from paper_2112_09335_b200 import binding, inputs
 from parity_utils import forced_from, make_oracle, relerr
@@ -86,3 +87,47 @@ def test_ten_iterations_with_cut_rows(case, schedule):
         assert relerr(g.get_state(binding.ST_U), o.U) <= 1e-3
     finally:
         g.destroy()
+
+
+def test_workspace_of_wide_propagations():
+    """Matrices wider than every layer, one wider than the other: the handle keeps one workspace for the items' sums, of the
+    widest, and the call that may not allocate gives the same bits before and after it has grown."""
+    import torch
+
+    def check(n):
+        """Device memory of the handle after the wide calls less that before them, and the workspace's size."""
+        pr = tiny_problem(91, n=n, widths=(6, 9, 4), n_comm=1, p=20.0 / n)
+        lengths = np.diff(pr["row_ptr"]) + 1
+        items = int(((lengths + 3) // 4)[lengths > 4].sum())
+        At = orc.normalized_adjacency(n, pr["row_ptr"], pr["col_idx"])
+        g = binding.GcnAdmm(n, pr["row_ptr"], pr["col_idx"], pr["X"].astype(np.float32), pr["y"], pr["mask"], pr["widths"],
+                            pr["n_comm"], pr["community"], [w.astype(np.float32) for w in pr["W"]], long_row=4)
+        try:
+            x = np.random.default_rng(5).standard_normal((n, 1000)).astype(np.float32)
+            want, scale = At @ x.astype(np.float64), abs(At) @ np.abs(x).astype(np.float64) + 1e-30
+            y = [torch.zeros(n, width, device="cuda") for width in (1000, 1400, 2000)]
+            for t in y:
+                t[:, :1000] = torch.from_numpy(x)
+            out, before, after = torch.empty(n, 2000, device="cuda"), torch.empty(n, 1000, device="cuda"), torch.empty(n, 1000, device="cuda")
+            torch.cuda.synchronize()
+            g.propagate_static(y[0].data_ptr(), 1000, before.data_ptr())
+            binding.release_idle()
+            torch.cuda.synchronize()
+            free = torch.cuda.mem_get_info()[0]
+            got = []
+            for t in y:
+                g.propagate(t.data_ptr(), t.shape[1], out.data_ptr())
+                got.append(out.reshape(-1)[:t.numel()].reshape(t.shape)[:, :1000].cpu().numpy())
+            binding.release_idle()
+            grown = free - torch.cuda.mem_get_info()[0]
+            g.propagate_static(y[0].data_ptr(), 1000, after.data_ptr())
+            torch.cuda.synchronize()
+            assert torch.equal(before, after)
+            assert all(np.max(np.abs(a - want) / scale) < 1e-6 for a in got)
+            return grown, items * 2000 * 4
+        finally:
+            g.destroy()
+
+    check(300)                                       # loads the kernels
+    grown, workspace = check(3000)
+    assert workspace <= grown <= 1.25 * workspace    # (1000 + 1400) / 2000 more with all three kept; the driver takes some MB of its own
