@@ -222,9 +222,7 @@ struct gcn_admm {
   float* grad = nullptr;     // max over l of C_{l-1} x ld_l
   float* grad_t = nullptr;   // its transpose, C_l x ld_{l-1} (K-major operand of the tensor-core product)
   int* tc_error = nullptr;   // &report->error: raised by a tensor-core product (1) or a search (2) whose bounded wait ran out
-  uint8_t* b_image = nullptr;   // split operand of a product without a kept image (see gtc::k_split_b)
   std::vector<gtc::Image> img_H, img_G, img_D;   // 1..L: kept images of W_l for P_l W_l, of W_l for S W_l^T, of the gradient for P_l grad
-  size_t b_image_bytes = 0;
   float* part = nullptr;     // split partial sums of the transposed product
   size_t part_elems = 0;
   SearchCtl *ctl_w = nullptr, *ctl_z = nullptr;   // [L+1], [(L+1) * M]
@@ -485,7 +483,7 @@ struct gcn_admm {
   }
 
   // C = A B.  B is handed over twice: row-major K x N (ldb) for the fp32-ALU kernels and K-major N x K (Bk, ldbk; may be
-  // NULL) for the tensor-core kernel, which is used whenever it applies; `kept`: its image, where one is kept.
+  // NULL) for the tensor-core kernel, which is used whenever it applies; `kept`: its image, where the product takes one.
   void gemm_nn(const float* A, int lda, const float* B, int ldb, const float* Bk, int ldbk, float* Cm, int ldc,
                long long Mr, int N, int K, const gtc::Image* kept = nullptr, const int* skip = nullptr) {
     char name[48];
@@ -496,16 +494,7 @@ struct gcn_admm {
       dim3 grid((unsigned)std::max(1, std::min(tiles, kSmCount / groups)), (unsigned)groups);
       CUtensorMap tmap;
       std::memset(&tmap, 0, sizeof tmap);
-      const uint8_t* image = nullptr;
-      if (takes_image(Mr, N, K, nt)) {
-        if (kept != nullptr && kept->data != nullptr) image = kept->data;
-        else if (image_bytes(N, K, nt) <= b_image_bytes) {
-          gtc::k_split_b<<<(unsigned)std::min<long long>(cdiv((long long)groups * kc * nt * 8, 256), 4 * kSmCount), 256, 0, stream>>>(Bk, ldbk, N, K, nt, b_image);
-          CU(cudaGetLastError());
-          ++launches;
-          image = b_image;
-        }
-      }
+      const uint8_t* const image = takes_image(Mr, N, K, nt) && kept != nullptr ? kept->data : nullptr;
       // few row tiles and a long reduction: several CTAs share a tile's K chunks, at least four chunks each
       // (2.7 k rows, K = 1433, 16 columns: 34 -> 13 us)
       if (image == nullptr)
@@ -1361,8 +1350,6 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
   h->want(h->item_sums, h->item_sums_elems);
   h->want(h->grad, grad_elems);
   h->want(h->grad_t, grad_t_elems, gcn_admm::kZero);
-  h->b_image_bytes = (size_t)16 << 20;   // e.g. 1024 columns x 2048 K
-  h->want(h->b_image, h->b_image_bytes);
   h->img_H.assign(L + 1, gtc::Image{nullptr, 16, 1}); h->img_G = h->img_D = h->img_H;
   for (int l = 1; l <= L; ++l) {
     h->want_image(h->img_H[l], h->C[l], h->C[l - 1], h->ld[l - 1]);
@@ -1730,6 +1717,7 @@ int gcn_admm_dense_product(gcn_admm* h, const float* A, const float* B, float* C
       throw Fail{GCN_ADMM_ERR_ARG, "A, B and C must be device pointers"};
     const int lda = ldpad(k), ldb = ldpad(n), ldc = ldpad(n), ldbk = ldpad(k);
     float *a = nullptr, *b = nullptr, *bk = nullptr, *c = nullptr;
+    gtc::Image image{nullptr, 16, 1};
     const int saved = h->p.tensor_cores;
     try {
       a = dalloc<float>((size_t)m * lda);
@@ -1744,16 +1732,24 @@ int gcn_admm_dense_product(gcn_admm* h, const float* A, const float* B, float* C
       gk::k_transpose_small<<<(unsigned)cdiv((long long)k * n, 256), 256, 0, h->stream>>>(b, ldb, bk, ldbk, k, n);
       CU(cudaGetLastError());
       h->p.tensor_cores = tensor_cores;
-      h->gemm_nn(a, lda, b, ldb, tensor_cores ? bk : nullptr, ldbk, c, ldc, m, n, k);
+      const int nt = h->group_width(m, n, k, lda);
+      if (h->on_tensor_cores(m, k) && h->takes_image(m, n, k, nt)) {
+        const long long units = cdiv(n, nt) * cdiv(k, gtc::kChunkK) * nt * 8;   // threads of k_split_b
+        image = gtc::Image{dalloc<uint8_t>(gcn_admm::image_bytes(n, k, nt)), nt, (int)cdiv(k, gtc::kChunkK)};
+        gtc::k_split_b<<<(unsigned)std::min<long long>(cdiv(units, 256), 4 * kSmCount), 256, 0, h->stream>>>(bk, ldbk, n, k, nt, image.data);
+        CU(cudaGetLastError());
+        ++h->launches;
+      }
+      h->gemm_nn(a, lda, b, ldb, tensor_cores ? bk : nullptr, ldbk, c, ldc, m, n, k, &image);
       h->p.tensor_cores = saved;
       CU(cudaMemcpy2DAsync(C, (size_t)n * 4, c, (size_t)ldc * 4, (size_t)n * 4, (size_t)m, cudaMemcpyDeviceToDevice, h->stream));
       CU(cudaStreamSynchronize(h->stream));
     } catch (...) {
       h->p.tensor_cores = saved;
-      cudaFree(a); cudaFree(b); cudaFree(bk); cudaFree(c);
+      cudaFree(a); cudaFree(b); cudaFree(bk); cudaFree(c); cudaFree(image.data);
       throw;
     }
-    cudaFree(a); cudaFree(b); cudaFree(bk); cudaFree(c);
+    cudaFree(a); cudaFree(b); cudaFree(bk); cudaFree(c); cudaFree(image.data);
     h->check_status();
   });
 }

@@ -1,0 +1,36 @@
+"""Device memory of a handle against what its arrays need."""
+import numpy as np
+import pytest
+
+from conftest import tiny_problem
+from paper_2112_09335_b200 import binding
+
+pytestmark = pytest.mark.gpu
+
+MB = 1 << 20
+
+
+def handle(pr, **kw):
+    return binding.GcnAdmm(pr["n"], pr["row_ptr"], pr["col_idx"], pr["X"].astype(np.float32), pr["y"], pr["mask"], pr["widths"],
+                           pr["n_comm"], pr["community"], [w.astype(np.float32) for w in pr["W"]], **kw)
+
+
+def memory_of(make, count=1):
+    """Device memory that `count` handles hold, after a first round has loaded kernels and made streams."""
+    import torch
+    for _ in range(2):
+        binding.release_idle()
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        made = [make() for _ in range(count)]
+        torch.cuda.synchronize()
+        used = free - torch.cuda.mem_get_info()[0]
+        for g in made:
+            g.destroy()
+    binding.release_idle()
+    return used
+
+
+def test_small_handles_take_little():
+    pr = tiny_problem(75, n=200, widths=(6, 9, 4), n_comm=3)
+    assert memory_of(lambda: handle(pr), count=8) <= 8 * 4 * MB      # a slab of 2 MB each, and as much again for the driver
