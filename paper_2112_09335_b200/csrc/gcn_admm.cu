@@ -232,11 +232,10 @@ struct gcn_admm {
   int4* d_zblocks = nullptr;                // row blocks of at most kZBlockRows rows, none crossing a community, and that community
   unsigned *ticket = nullptr, *tile_tickets = nullptr, *comm_tickets = nullptr;   // counters of finished blocks (one launch; per community), zero between launches
   gk::GridBar* grid_bar = nullptr;          // meeting point of the cooperative launches (one at a time: one stream)
-  std::vector<float*> RN;                   // 2..L: derivative of phi_l at the new H_l, from the W_l update to that of Z_{l-1}
   int* d_comm_block_ptr = nullptr;          // [M+1] first row block of every community
   int n_zblocks = 0;
   int *d_h1_age = nullptr, *skip_h1 = nullptr;   // see k_end_pass
-  float* DL = nullptr;       // P_L grad_L
+  float *RL = nullptr, *DL = nullptr;       // the last layer's R and P grad, where its chain runs beside the hidden layers' (see Lane)
   int *n_active = nullptr, *status = nullptr, *d_pass = nullptr;   // status = &report->status
   // Z scoring: units in chunks of about equally many stored entries, dealt to the warps of the grid in a fixed order
   int* d_chunk_ptr = nullptr;
@@ -674,14 +673,15 @@ struct gcn_admm {
   }
 
   // ---- W_l block (Section 3.1) --------------------------------------------------------
-  // resid_next: also leave the derivative of phi_l at the new H_l in RN[l] (what the Z_{l-1} update starts from).
-  // The last layer works in matrices of its own width (RN[L], DL), so that its chain can run beside the others' (see Lane).
+  // Where R_l is formed and, turned into its value at the new H_l, handed from the W_l update to that of Z_{l-1}.
+  float* resid_of(int l) const { return l == L && RL != nullptr ? RL : B0; }
+  // resid_next: also leave the derivative of phi_l at the new H_l in resid_of(l) (what the Z_{l-1} update starts from).
   void update_W(int l, bool resid_next) {
     Range range("gcn_admm: W block");
     const int Kp = C[l - 1], Cn = C[l], ldc = ld[l];
     const long long n4 = n * ldc / 4;
     SearchCtl* ctl = ctl_w + l;
-    float *const R = l == L ? RN[L] : B0, *const D = l == L ? DL : B1;
+    float *const R = resid_of(l), *const D = l == L && DL != nullptr ? DL : B1;
     int splits;
     if (l < L && tn_on_tensor_cores(n)) {                               // grad = P_l^T R_l, R_l formed inside the product
       splits = gemm_tn(P[l], ld[l - 1], H[l], ldc, ldc, n, Kp, Cn, Z[l], p.nu);
@@ -693,7 +693,7 @@ struct gcn_admm {
     gemm_nn(P[l], ld[l - 1], grad, ldc, grad_t, ld[l - 1], D, ldc, n, Cn, Kp, &img_D[l], &ctl->done);   // D = P_l grad
     gk::SearchW a{};
     a.H = (float4*)H[l]; a.D = (const float4*)D; a.Z = (const float4*)Z[l]; a.U = (const float4*)U; a.R = (const float4*)R;
-    a.Rn = resid_next ? (float4*)RN[l] : nullptr;
+    a.Rn = resid_next ? (float4*)R : nullptr;
     a.n4 = n4;
     a.coef = l == L ? p.rho : p.nu;
     a.W = W[l]; a.Wt = Wt[l]; a.image = img_H[l]; a.image_t = img_G[l]; a.grad = grad;
@@ -723,12 +723,12 @@ struct gcn_admm {
   }
 
   // ---- Z_{l,m}, l < L, every community (Appendix A, Eq. 5/6 and 8-10) ------------------
-  // resid_ready: RN[l+1] holds the derivative of phi_{l+1} at the stored H_{l+1}.
+  // resid_ready: resid_of(l + 1) holds the derivative of phi_{l+1} at the stored H_{l+1}.
   void update_Z_hidden(int l, bool resid_ready) {
     Range range("gcn_admm: hidden Z blocks");
     const int ldl = ld[l], ldn = ld[l + 1];
     SearchCtl* ctl = ctl_z + (size_t)l * M;
-    float* const Rn = RN[l + 1];
+    float* const Rn = resid_of(l + 1);
     if (!resid_ready) resid(l + 1, Rn);                                  // R'_{l+1}
     spmm(Rn, B1, ldn);                                                   // S = A~ R'
     gemm_nn(B1, ldn, Wt[l + 1], ldl, W[l + 1], ldn, B2, ldl, n, C[l], C[l + 1], &img_G[l + 1]);        // S W_{l+1}^T
@@ -938,12 +938,16 @@ struct gcn_admm {
     swap_lane();
   }
 
-  void iterate() {   // Algorithm 1, one pass
+  // Algorithm 1, one pass.  Z_{l-1} follows W_l directly, so that one matrix carries R_l from one to the other whatever the depth:
+  // the W updates after it read P (not yet formed again), H, Z and U of other layers, none of which it writes.
+  void iterate() {
     if (p.schedule == 1) { iterate_sequential(); return; }
     if (!fresh) refresh();
     if (!two_lanes || profiling) {
-      for (int l = 1; l <= L; ++l) update_W(l, l >= 2);
-      for (int l = 1; l < L; ++l) update_Z_hidden(l, true);
+      for (int l = 1; l <= L; ++l) {
+        update_W(l, l >= 2);
+        if (l >= 2) update_Z_hidden(l - 1, true);
+      }
       update_output(p.dual_mode == 0, true);
       refresh(true);
     } else {
@@ -955,11 +959,12 @@ struct gcn_admm {
         update_output(p.dual_mode == 0, true);
         CU(cudaEventRecord(side.out_done, stream));
       });
-      for (int l = 1; l < L; ++l) update_W(l, l >= 2);
       for (int l = 1; l < L; ++l) {
-        if (l == L - 1) join(stream, side.w_done);
-        update_Z_hidden(l, true);
+        update_W(l, l >= 2);
+        if (l >= 2) update_Z_hidden(l - 1, true);
       }
+      join(stream, side.w_done);
+      update_Z_hidden(L - 1, true);
       CU(cudaEventRecord(side.begun, stream));
       join(side.stream, side.begun);
       on_side([&] {
@@ -1306,7 +1311,7 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
   const int L = n_layers;
   const size_t rows = (size_t)n;
   h->W.assign(L + 1, nullptr); h->Wt.assign(L + 1, nullptr); h->Z.assign(L + 1, nullptr);
-  h->P.assign(L + 1, nullptr); h->H.assign(L + 1, nullptr); h->RN.assign(L + 1, nullptr);
+  h->P.assign(L + 1, nullptr); h->H.assign(L + 1, nullptr);
   size_t grad_elems = 1, grad_t_elems = 1, grad_blocks = 1;   // grad_blocks: most blocks of a finish_grad launch
   h->part_elems = 1;
   for (int l = 1; l <= L; ++l) {
@@ -1329,13 +1334,12 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
   h->want(h->B0, rows * h->max_ld);
   h->want(h->B1, rows * h->max_ld);
   h->want(h->B2, rows * h->max_ld);
-  for (int l = 2; l <= L; ++l) h->want(h->RN[l], rows * h->ld[l]);   // R_L is turned into its new value in place
-  if (L == 1) h->want(h->RN[1], rows * h->ld[1]);
-  h->want(h->DL, rows * h->ld[L]);
   // a second line of launches where a pass is short enough for it to matter (the sizes that are recorded as graphs)
   h->two_lanes = L >= 2 && n * (long long)h->max_ld < kSmallProblem;
   if (h->two_lanes) {
     const size_t ge = (size_t)h->C[L - 1] * h->ld[L];
+    h->want(h->RL, rows * h->ld[L]);
+    h->want(h->DL, rows * h->ld[L]);
     h->side.part_elems = std::max<size_t>(ge, std::min<size_t>(std::max(ge * 4 * kSmCount, ge * (size_t)(cdiv(n, 2048) + kSmCount)), (size_t)64 << 20));
     h->want(h->side.part, h->side.part_elems);
     h->want(h->side.grad, ge);

@@ -34,3 +34,17 @@ def memory_of(make, count=1):
 def test_small_handles_take_little():
     pr = tiny_problem(75, n=200, widths=(6, 9, 4), n_comm=3)
     assert memory_of(lambda: handle(pr), count=8) <= 8 * 4 * MB      # a slab of 2 MB each, and as much again for the driver
+
+
+def test_depth_costs_the_state_of_a_layer_and_no_more():
+    """Six layers: Z, H and P of each, U, three scratch matrices of the widest, two of the last layer's width, the weights, the
+    gradient and its split sums (4 x 148 of the largest, and of the last layer for its own line of launches)."""
+    n, widths = 8000, (16, 256, 256, 256, 256, 256, 8)
+    pr = tiny_problem(76, n=n, widths=widths, n_comm=3, p=5.0 / n)
+    ld, L = [(w + 3) // 4 * 4 for w in widths], len(widths) - 1
+    rows = sum(ld[1:]) * 2 + sum(ld[:-1]) + 3 * max(ld) + 3 * ld[-1]
+    weights = sum(a * b for a, b in zip(ld, ld[1:]))
+    split = 4 * 148 * (256 * 256 + 256 * 8)
+    arrays = 4 * (n * rows + 2 * weights + 2 * 256 * 256 + split)
+    # tables of 48 k stored entries, and rounding; a matrix of 256 columns more per hidden layer would be 33 MB
+    assert memory_of(lambda: handle(pr)) <= arrays + 12 * MB
