@@ -41,7 +41,6 @@ constexpr int kSmCount = 148;
 constexpr long long kImageMinRows = 16384;   // row count from which the weight operand is pre-split
 constexpr int kZBlockRows = 32;      // rows per block of the hidden-layer gradient's closing sweep
 constexpr int kChunkGroups = 512;    // groups the sums of a scoring sweep's chunks are first added up in, when there are more chunks
-constexpr int kCandZ = 4;           // theta candidates scored per sweep (2..4; steady-state searches close at trial 0..2)
 constexpr size_t kDirectBytes = (size_t)256 << 10;   // matrices up to this size cross the bus inside the permuting kernel (one copy and its latency less)
 constexpr long long kSmallProblem = 1LL << 27;   // nodes x widest layer: below it launch gaps show in a pass
 constexpr int kDefaultLongRow = 256;   // stored entries one warp walks before a row is cut into items
@@ -781,7 +780,7 @@ struct gcn_admm {
       return;
     }
     gemm_nn(B2, ldl, W[l + 1], ldn, Wt[l + 1], ldl, B1, ldn, n, C[l + 1], C[l], &img_H[l + 1]);         // T = G W_{l+1}
-    decide.cand = kCandZ;
+    decide.cand = gk::kCand;   // steady-state searches close at trial 0..2
     decide.scale = 0.5 * p.nu;
     gk::SearchZ a{};
     a.ctl = ctl; a.n_comm = M;
@@ -796,7 +795,7 @@ struct gcn_admm {
     a.Z = (float4*)Z[l]; a.G = (const float4*)B2; a.ldz4 = ldl / 4; a.row_comm = d_row_comm;
     std::snprintf(zname, sizeof zname, "score_z_hidden@%d", ldn);
     const float4 *T = (const float4*)B1, *Hn = (const float4*)H[l + 1], *Zn = (const float4*)Z[l + 1];
-    const size_t sums = (size_t)warps * M * kCandZ * sizeof(double);
+    const size_t sums = (size_t)warps * M * gk::kCand * sizeof(double);
     const int use_smem = sums <= 96 * 1024;
     auto score = [&](auto kernel, auto close, int V) {
       const size_t smem = (size_t)warps * 2 * V * 32 * sizeof(float4) + (use_smem ? sums + (size_t)M * sizeof(float4) : 0);
@@ -812,10 +811,10 @@ struct gcn_admm {
       launch_together(close, cdiv(n * (ldl / 4), 256), warps * 32, smem, d_row_ptr, d_col, d_col_comm, d_dinv, T, Hn, Zn, ld4, (int)n,
                       use_smem, d_chunk_ptr, n_chunks, d_items, n_items, long_len, scratch, a);
     };
-    if (ld4 <= 32) score(gk::k_score_z<1, 4, kCandZ>, gk::k_close_z<1, 4, kCandZ>, 1);
-    else if (ld4 <= 64) score(gk::k_score_z<2, 4, kCandZ>, gk::k_close_z<2, 4, kCandZ>, 2);
-    else if (ld4 <= 128) score(gk::k_score_z<4, 4, kCandZ>, gk::k_close_z<4, 4, kCandZ>, 4);
-    else score(gk::k_score_z<8, 4, kCandZ>, gk::k_close_z<8, 4, kCandZ>, 8);
+    if (ld4 <= 32) score(gk::k_score_z<1, 4>, gk::k_close_z<1, 4>, 1);
+    else if (ld4 <= 64) score(gk::k_score_z<2, 4>, gk::k_close_z<2, 4>, 2);
+    else if (ld4 <= 128) score(gk::k_score_z<4, 4>, gk::k_close_z<4, 4>, 4);
+    else score(gk::k_score_z<8, 4>, gk::k_close_z<8, 4>, 8);
   }
 
   // ---- Z_L (Eq. 7) and, in the same sweep, the dual as printed in Eq. 3 -----------------

@@ -1203,23 +1203,13 @@ k_zgrad_finish(float4* __restrict__ G, const float4* __restrict__ Z, const float
   }
 }
 
-// Warp-wide sums of 4 (or 2) per-lane values with 6 (5) shuffles: lane 8*j (16*j) ends up holding
-// the total of value j.
+// Warp-wide sums of 4 per-lane values with 6 shuffles: lane 8*j ends up holding the total of value j.
 __device__ __forceinline__ float warp_sum4(float v0, float v1, float v2, float v3, int lane) {
   const bool up16 = lane & 16, up8 = lane & 8;
   const float r0 = __shfl_xor_sync(0xffffffffu, up16 ? v0 : v2, 16);
   const float r1 = __shfl_xor_sync(0xffffffffu, up16 ? v1 : v3, 16);
   const float a = (up16 ? v2 : v0) + r0, b = (up16 ? v3 : v1) + r1;
   float c = (up8 ? b : a) + __shfl_xor_sync(0xffffffffu, up8 ? a : b, 8);
-  c += __shfl_xor_sync(0xffffffffu, c, 4);
-  c += __shfl_xor_sync(0xffffffffu, c, 2);
-  c += __shfl_xor_sync(0xffffffffu, c, 1);
-  return c;
-}
-__device__ __forceinline__ float warp_sum2(float v0, float v1, int lane) {
-  const bool up16 = lane & 16;
-  float c = (up16 ? v1 : v0) + __shfl_xor_sync(0xffffffffu, up16 ? v0 : v1, 16);
-  c += __shfl_xor_sync(0xffffffffu, c, 8);
   c += __shfl_xor_sync(0xffffffffu, c, 4);
   c += __shfl_xor_sync(0xffffffffu, c, 2);
   c += __shfl_xor_sync(0xffffffffu, c, 1);
@@ -1232,10 +1222,11 @@ __device__ __forceinline__ float warp_sum2(float v0, float v1, int lane) {
 // which is non-zero on V_m and its first-order neighbour rows only.  A warp owns row i and walks
 // its stored entries once; col_comm gives the community of every entry, entries of one community
 // are contiguous (ascending columns), and at every change of community the finished K_m[i] is scored:
-//   per community, sum_c (z - f(h - k/t_j))^2 - (z - f(h))^2 for j < NC
-//                                        (NC = candidates scored per sweep, 2..4: a candidate costs two
-//                                        instructions per element, and a search that needs more trials
-//                                        than one sweep scores is served by a further sweep)
+//   per community, sum_c (z - f(h - k/t_j))^2 - (z - f(h))^2 for j < kCand
+//                                        (a candidate costs two instructions per element, and a search
+//                                        that needs more trials than one sweep scores is served by a
+//                                        further sweep; two or three per sweep gained 8 % of the first
+//                                        sweep at most and brought later ones back)
 // (Layer l+1 = L is linear and has a search of its own, k_search_z_out.)
 // Sums are kept per warp in shared memory (no atomics on the hot path) and leave the kernel per chunk of
 // units (see the scheduling note in the kernel).  V = float4 columns per lane (width <= 128 V).
@@ -1252,41 +1243,34 @@ __device__ __forceinline__ float4 twice_error(const float4& h, const float4& z) 
 }
 
 // Scores one finished K_m[i] (k, still without the factor di) against the row's a, b:
-// a = h and b = twice_error(h, z).  The NC sums go to `slots`:
+// a = h and b = twice_error(h, z).  The kCand sums go to `slots`:
 // add: added to what is there (the slots belong to this warp), else stored.
 __device__ __forceinline__ void put_sum(double* dst, float r, bool add) { *dst = add ? *dst + (double)r : (double)r; }
-template <int V, int NC>
+template <int V>
 __device__ __forceinline__ void score_segment(const float4 (&k)[V], float di, const float4 (&a)[V],
                                               const float4 (&b)[V], const float* inv_cand, int lane, double* slots,
                                               bool add) {
-  {
-    static_assert(NC >= 2 && NC <= 4, "two to four candidates per sweep");
-    float inv[NC], part[NC];
+  static_assert(kCand == 4, "warp_sum4 and the float4 of a community's candidates hold four");
+  float inv[kCand], part[kCand];
 #pragma unroll
-    for (int j = 0; j < NC; ++j) { inv[j] = di * inv_cand[j]; part[j] = 0.f; }   // K_m[i] = di * k
+  for (int j = 0; j < kCand; ++j) { inv[j] = di * inv_cand[j]; part[j] = 0.f; }   // K_m[i] = di * k
 #pragma unroll
-    for (int v = 0; v < V; ++v) {
-      const float kk[4] = {k[v].x, k[v].y, k[v].z, k[v].w};
-      const float hh[4] = {a[v].x, a[v].y, a[v].z, a[v].w};
-      const float ee[4] = {b[v].x, b[v].y, b[v].z, b[v].w};   // 2 (z - f(h)), see twice_error
+  for (int v = 0; v < V; ++v) {
+    const float kk[4] = {k[v].x, k[v].y, k[v].z, k[v].w};
+    const float hh[4] = {a[v].x, a[v].y, a[v].z, a[v].w};
+    const float ee[4] = {b[v].x, b[v].y, b[v].z, b[v].w};   // 2 (z - f(h)), see twice_error
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const float pos = fmaxf(hh[c], 0.f), neg = fmaxf(-hh[c], 0.f);
+    for (int c = 0; c < 4; ++c) {
+      const float pos = fmaxf(hh[c], 0.f), neg = fmaxf(-hh[c], 0.f);
 #pragma unroll
-        for (int j = 0; j < NC; ++j) {
-          const float df = relu_drop(kk[c], inv[j], neg, pos);
-          part[j] = fmaf(df, ee[c] + df, part[j]);   // e1^2 - e0^2 = df (2 e0 + df)
-        }
+      for (int j = 0; j < kCand; ++j) {
+        const float df = relu_drop(kk[c], inv[j], neg, pos);
+        part[j] = fmaf(df, ee[c] + df, part[j]);   // e1^2 - e0^2 = df (2 e0 + df)
       }
     }
-    if constexpr (NC >= 3) {
-      const float r = warp_sum4(part[0], part[1], part[2], NC == 4 ? part[NC - 1] : 0.f, lane);
-      if ((lane & 7) == 0 && (lane >> 3) < NC) put_sum(slots + (lane >> 3), r, add);
-    } else {
-      const float r = warp_sum2(part[0], part[1], lane);
-      if ((lane & 15) == 0) put_sum(slots + (lane >> 4), r, add);
-    }
   }
+  const float r = warp_sum4(part[0], part[1], part[2], part[3], lane);
+  if ((lane & 7) == 0) put_sum(slots + (lane >> 3), r, add);
 }
 
 // What the search of a hidden layer's Z blocks needs beside the scoring kernel's own operands.
@@ -1316,10 +1300,10 @@ struct SearchZ {
 // other, one warp each.  With many chunks their sums are first added group by group, in chunk order.  Then one warp per
 // community adds up its groups (or chunks; lane-strided, then the shuffle tree) and its split segments in table order,
 // and takes the decision.  No sum depends on which warp scored which chunk.
-template <int V, int NC>
+template <int V>
 __device__ __forceinline__ bool close_sweep(const SearchZ& p, int n_chunks, const float* __restrict__ dinv, const float4* scratch,
                                             const float4* __restrict__ Hn, const float4* __restrict__ Zn, int ld4) {
-  constexpr int PER = NC;
+  constexpr int PER = kCand;
   const int lane = threadIdx.x & 31;
   const int gwarp = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), n_warps = (int)((gridDim.x * blockDim.x) >> 5);
   const auto nothing = [] {};
@@ -1339,7 +1323,7 @@ __device__ __forceinline__ bool close_sweep(const SearchZ& p, int n_chunks, cons
           for (int q = 0; q < sp.w; ++q) k[v] = vadd(k[v], __ldcg(scratch + (long long)(sp.z + q) * ld4 + f));
         }
       }
-      score_segment<V, NC>(k, dinv[sp.x], a, b, p.ctl[sp.y].inv_cand, lane, p.split_scores + (size_t)s * PER, false);
+      score_segment<V>(k, dinv[sp.x], a, b, p.ctl[sp.y].inv_cand, lane, p.split_scores + (size_t)s * PER, false);
     }
     const int width = p.n_comm * PER;
     for (int g = blockIdx.x; g < p.n_groups; g += gridDim.x) {
@@ -1404,13 +1388,13 @@ __device__ __forceinline__ void move_blocks(const SearchZ& p, long long n) {
 // One sweep over all chunks by the warps of the grid.  Dynamic shared memory: per warp the row's a, b (2 V float4 per
 // lane; parked there during the walk so that the registers hold gathered rows instead), the candidates of every community
 // (one float4; negative when its search is closed), then the per-warp sums; the last two only with use_smem.
-template <int V, int UN, int NC>
+template <int V, int UN>
 __device__ __forceinline__ void score_sweep(const int* __restrict__ row_ptr, const int* __restrict__ col,
           const unsigned short* __restrict__ col_comm, const float* __restrict__ dinv,
           const float4* __restrict__ T, const float4* __restrict__ Hn, const float4* __restrict__ Zn, int ld4, const SearchCtl* ctl, int n_comm, double* chunk_part, int use_smem,
           const int* __restrict__ chunk_ptr, int n_chunks, int* chunk_counter,
           const int4* __restrict__ items, int n_items, int long_len, float4* scratch) {
-  constexpr int PER = NC;
+  constexpr int PER = kCand;
   extern __shared__ float4 s_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int warps_per_block = blockDim.x >> 5;
@@ -1517,7 +1501,7 @@ __device__ __forceinline__ void score_sweep(const int* __restrict__ row_ptr, con
         a[v] = row_ab[32 * v];
         b[v] = row_ab[32 * (V + v)];
       }
-      score_segment<V, NC>(k, di, a, b, use_smem ? reinterpret_cast<const float*>(s_cand + cur) : ctl[cur].inv_cand, lane,
+      score_segment<V>(k, di, a, b, use_smem ? reinterpret_cast<const float*>(s_cand + cur) : ctl[cur].inv_cand, lane,
                                 mine + cur * PER, true);
     };
 
@@ -1595,7 +1579,7 @@ __device__ __forceinline__ void score_sweep(const int* __restrict__ row_ptr, con
   }
 }
 
-template <int V, int UN, int NC>
+template <int V, int UN>
 __global__ void __launch_bounds__(256, (V <= 1 ? 4 : V <= 2 ? 3 : 1))
 k_score_z(const int* __restrict__ row_ptr, const int* __restrict__ col,
           const unsigned short* __restrict__ col_comm, const float* __restrict__ dinv,
@@ -1604,7 +1588,7 @@ k_score_z(const int* __restrict__ row_ptr, const int* __restrict__ col,
           const int* __restrict__ chunk_ptr, int n_chunks, int* __restrict__ chunk_counter,
           const int4* __restrict__ items, int n_items, int long_len, float4* __restrict__ scratch) {
   if (*n_active <= 0) return;
-  score_sweep<V, UN, NC>(row_ptr, col, col_comm, dinv, T, Hn, Zn, ld4, ctl, n_comm, chunk_part, use_smem, chunk_ptr, n_chunks,
+  score_sweep<V, UN>(row_ptr, col, col_comm, dinv, T, Hn, Zn, ld4, ctl, n_comm, chunk_part, use_smem, chunk_ptr, n_chunks,
                               chunk_counter, items, n_items, long_len, scratch);
 }
 
@@ -1613,7 +1597,7 @@ k_score_z(const int* __restrict__ row_ptr, const int* __restrict__ col,
 // kernel of its own because, compiled together with this one, its walk spills registers (2.4 M rows x 256: 14.9 against 13.6 ms).
 // The searches of a launch start together, so the sweep that scores the last of max_trials is the last one: *n_active alone
 // would not end the loop where a launch before this one gave up and left it too high.
-template <int V, int UN, int NC>
+template <int V, int UN>
 __global__ void __launch_bounds__(256, (V <= 2 ? 3 : 1))
 k_close_z(const int* __restrict__ row_ptr, const int* __restrict__ col,
           const unsigned short* __restrict__ col_comm, const float* __restrict__ dinv,
@@ -1622,9 +1606,9 @@ k_close_z(const int* __restrict__ row_ptr, const int* __restrict__ col,
   if (__ldcg(sz.err) != 0) return;   // see GridBar
   if (__ldcg(sz.n_active) > 0) {
     for (int scored = sz.a.cand;; scored += sz.a.cand) {
-      if (!close_sweep<V, NC>(sz, n_chunks, dinv, scratch, Hn, Zn, ld4)) return;
+      if (!close_sweep<V>(sz, n_chunks, dinv, scratch, Hn, Zn, ld4)) return;
       if (__ldcg(sz.n_active) <= 0 || scored >= sz.a.max_trials) break;   // *n_active changes only between the meetings of close_sweep
-      score_sweep<V, UN, NC>(row_ptr, col, col_comm, dinv, T, Hn, Zn, ld4, sz.ctl, sz.n_comm, sz.chunk_part, use_smem, chunk_ptr,
+      score_sweep<V, UN>(row_ptr, col, col_comm, dinv, T, Hn, Zn, ld4, sz.ctl, sz.n_comm, sz.chunk_part, use_smem, chunk_ptr,
                                   n_chunks, sz.chunk_counter, items, n_items, long_len, scratch);
       if (!grid_meet(sz.bar, sz.err, [] {})) return;
     }
