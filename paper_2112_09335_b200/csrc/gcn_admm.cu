@@ -753,8 +753,13 @@ struct gcn_admm {
       a.segs = d_segs; a.chunks = d_seg_chunks; a.n_chunks = n_seg_chunks; a.chunk_counter = chunk_counter;
       a.slot_ptr = d_slot_ptr; a.slots = slots; a.comm_done = comm_done; a.split_done = split_done; a.items = d_items; a.split = d_split;
       a.ctl = ctl; a.own = sums_z; a.n_active = n_active; a.status = status; a.a = decide;
-      // one wave of chunks: the longest segment is the critical path, so long ones get a whole warp
-      a.share_from = ld4 <= 4 ? 24 : n_seg_chunks <= 2 * kSmCount * 24 ? 64 : INT_MAX;
+      // The longest segments are the critical path.  A warp shared by 32 / CL sets walks one in as many fewer steps, a short one in
+      // none fewer but with its sets half empty, so the line lies the higher the fewer sets there are.  us at 6 / 24 / 48 / 128 /
+      // never: 3 columns (19.7 k rows, 2 entries each) 21.0 / 20.8 / 21.5 / 22.6 / 22.5, 10 (13.8 k, 30) 36.9 / 35.1 / 36.6 / 41.2 /
+      // 52.2, 4 (600 k, 40) 456 / 314 / 305 / 304 / 305; 23 (30 k, 16) 34.2 / 32.2 / 32.9 / 35.4 / 44.6, 23 (20 k, 50) 47.1 / 41.2 /
+      // 40.8 / 43.3 / 51.6; 40 (169 k, 14) 113 / 104 / 103 / 103 / 105, 47 (600 k, 50) 1032 / 934 / 915 / 899 / 896, 47 (2.45 M, 51)
+      // 4181 / 3850 / 3771 / 3743 / 3756.  With CL = 32 there is one set and no difference.
+      a.share_from = ld4 <= 4 ? 24 : ld4 <= 8 ? 48 : 128;
       std::snprintf(zname, sizeof zname, "search_z_out@%d", ldn);
       {
         Scope sc(this, zname, 1, 4.0 * gi.nnz + 12.0 * n + 8.0 * (double)n * ldn, 2.0 * (double)gi.nnz * ldn);

@@ -1628,8 +1628,7 @@ k_close_z(const int* __restrict__ row_ptr, const int* __restrict__ col,
 // (Walking the rows instead, with a ballot per group of entries to find the segments and a shared-memory slot per
 // community: 45 us at 20 k rows x 3 classes, 146 us at 169 k x 40, 4.6 ms at 2.45 M x 47; this form: 21 us, 99 us, 3.8 ms.)
 // CL lanes hold a row of T (ld4 <= CL float4), 32 / CL segments at a time per warp; segments of `share_from` entries or more
-// are shared by all lanes of the warp, entry e going to set e mod (32 / CL): where the chunks are few and the longest
-// segment sets the time, and with CL <= 4.  The warp that finishes a community's last slot adds
+// are shared by all lanes of the warp, entry e going to set e mod (32 / CL).  The warp that finishes a community's last slot adds
 // its slots up in slot order and takes the decision.
 // ------------------------------------------------------------------------------------------
 struct SegRef {

@@ -1,10 +1,11 @@
-"""The launches of a step-size search where their dispatch changes: the lane groups of the narrow output layer (4, 8, 16
-float4 per row, then a whole warp) and their fall back to larger ones when the communities' sums do not fit, sweeps with few
-and with many chunks, gradients with few and with many splits, all class widths of the output rows; against the oracle."""
+"""The launches of a step-size search where their dispatch changes: the lane groups of the last hidden layer's search (4, 8, 16,
+32 float4 per row of the output) and the segment lengths at which their walk changes, the hidden layers' sums in shared memory
+and, with more communities, in global memory, sweeps with few and with many chunks, gradients with few and with many splits,
+all class widths of the output rows; against the oracle."""
 import numpy as np
 import pytest
 
-from conftest import tiny_problem
+from conftest import dense_to_csr, tiny_problem
 from paper_2112_09335_b200 import binding
 from test_gpu_edge_cases import run_pair
 
@@ -16,9 +17,31 @@ def test_output_widths(classes):
     run_pair(tiny_problem(20 + classes, n=90, widths=(6, 9, classes), n_comm=3), n_it=3)
 
 
-@pytest.mark.parametrize("n_comm,classes", [(96, 5), (97, 5), (192, 20), (193, 20)])
-def test_communities_around_the_limits_of_the_lane_groups(n_comm, classes):
-    run_pair(tiny_problem(60, n=800, widths=(5, 7, classes), n_comm=n_comm, p=0.01), n_it=3)
+@pytest.mark.parametrize("n_comm", [384, 385])
+def test_communities_around_the_shared_memory_of_a_sweep(n_comm):
+    """8 warps x 32 bytes per community are kept in shared memory up to 96 KB: 384 communities."""
+    run_pair(tiny_problem(60, n=800, widths=(5, 7, 6, 5), n_comm=n_comm, p=0.01), n_it=3)
+
+
+@pytest.mark.parametrize("classes", [3, 7, 16, 23, 40, 70])
+@pytest.mark.parametrize("entries", [2, 4, 23, 47, 127, 300])
+def test_lengths_of_segments(classes, entries):
+    """The closed form walks segments of 1, 2 and 3 entries, longer ones by a group of lanes, and those of 24 entries or more
+    (up to 16 columns), 48 (up to 32) or 128 by a whole warp.  Communities of `entries` fully connected nodes, one more or one
+    less, and single edges between them; at 300 the rows are cut and their long segments go in pieces."""
+    n_comm = 9 if entries < 100 else 4
+    sizes = [max(1, entries + (m % 3) - 1) for m in range(n_comm)]
+    comm = np.repeat(np.arange(n_comm), sizes)
+    n = len(comm)
+    rng = np.random.default_rng(entries)
+    cross = np.triu(rng.random((n, n)) < 1.0 / n, 1)
+    A = ((comm[:, None] == comm[None, :]) | cross | cross.T).astype(np.float64)
+    np.fill_diagonal(A, 0.0)
+    pr = tiny_problem(64, n=n, widths=(6, 9, classes), n_comm=n_comm)
+    order = rng.permutation(n)
+    row_ptr, col_idx = dense_to_csr(A[np.ix_(order, order)])
+    pr.update(A=A, row_ptr=row_ptr, col_idx=col_idx, community=comm[order])
+    run_pair(pr, n_it=3)
 
 
 def test_many_chunks_and_a_search_of_several_sweeps():
