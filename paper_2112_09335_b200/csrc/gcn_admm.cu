@@ -1560,7 +1560,7 @@ int gcn_admm_step(gcn_admm* h, int n_iters) {
       cudaGraph_t graph = nullptr;
       CU(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
       const long long launches_before = h->launches, log_before = h->log_count;
-      h->capturing = true;          // the recorded pass is replayed many times: it forms every product
+      h->capturing = true;          // it launches every product; the device leaves H_1's out while H_1 is kept (see refresh)
       try {
         h->iterate();
         h->capturing = false;

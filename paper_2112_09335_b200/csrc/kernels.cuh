@@ -185,7 +185,8 @@ __device__ __forceinline__ void finish_item(const ItemRows& ir, int unit, T* __r
 // (1000 columns on 14 k rows 195 -> 142 us).  Lane t of a group of 32
 // stored entries holds column and weight of entry t, handed to the warp by shuffles.  UN neighbours in flight per
 // lane: the kernel is bound by the L2-to-SM traffic of the gathered rows, and by how the compiler orders its loads (the plain
-// loop measured faster than one that fetches columns ahead: 138 against 160 us at 128 columns on 169 k rows).
+// loop measured faster than one that fetches columns ahead: 138 against 160 us at 128 columns on 169 k rows).  At the 40
+// registers of 24 blocks per SM the form of 256 columns spills 8 bytes, the sliced one 32.
 template <int VEC, int NV, int UN, bool MAPPED, bool SLICED, bool RELU>
 __global__ void __launch_bounds__(64, VEC == 4 ? 24 : 16)
 k_spmm_wide(const int* __restrict__ row_ptr, const int* __restrict__ col, const float* __restrict__ dinv,
@@ -914,7 +915,8 @@ __device__ __forceinline__ void weight_tile(int tile, int rows, int cols, int pa
 // Weight gradient from its split partial sums, and the start of the W_l search, in one launch:
 //   grad[e] = sum over splits of part[s][e] (fp64, in split order), its transpose and its image for P grad, ||grad||^2, ||W||^2.
 // SG = 1: a block owns a tile of 32 x 32 elements (grid: tiles over rows x ldp).  SG = 8 (many splits): 32 consecutive elements,
-// eight threads per element, each adding its own run of consecutive splits.  The last block to finish adds the
+// eight threads per element, each adding its own run of consecutive splits; the transpose and the image are then written one
+// float at a time (a tile of 32 x 32 would leave one block where there are 32 now).  The last block to finish adds the
 // blocks' sums of squares up in block order and starts the search.  W = NULL: only the sum over the splits.
 template <int SG>
 __global__ void __launch_bounds__(256)
@@ -1629,7 +1631,8 @@ k_close_z(const int* __restrict__ row_ptr, const int* __restrict__ col,
 // community: 45 us at 20 k rows x 3 classes, 146 us at 169 k x 40, 4.6 ms at 2.45 M x 47; this form: 21 us, 99 us, 3.8 ms.)
 // CL lanes hold a row of T (ld4 <= CL float4), 32 / CL segments at a time per warp; segments of `share_from` entries or more
 // are shared by all lanes of the warp, entry e going to set e mod (32 / CL).  The warp that finishes a community's last slot adds
-// its slots up in slot order and takes the decision.
+// its slots up in slot order and takes the decision.  At the 80 registers of three blocks per SM every instantiation spills
+// (100 to 332 bytes of stores); two blocks, and the decision as a function of its own, have not been measured.
 // ------------------------------------------------------------------------------------------
 struct SegRef {
   int begin;

@@ -3,7 +3,9 @@
 //
 // A handle has about sixty device buffers.  Allocated one by one they cost 5 ms to create and 2 ms to free on a quiet
 // machine, more than the twenty passes of a small training run, and ten times that where other processes use the
-// driver too.  Copies between the device and pageable host memory go through the driver's own staging on one core at
+// driver too.  create and destroy of a handle of 2.7 k nodes, 1433-16-7: 1.6 ms on memory an earlier handle left, 8 to 15
+// without (slab, 12 MB of page-locked memory), 26 as the first of a process; 169 k nodes, 128-256-256-40: 14, 22 to 29, 45.
+// Copies between the device and pageable host memory go through the driver's own staging on one core at
 // 5-10 GB/s; here several cores fill or drain one part of the staging buffer while the copy engine works on the next.
 //
 // Slabs, staging buffers and streams of destroyed handles are kept for later ones up to a fixed amount (kIdleSlabBytes,
