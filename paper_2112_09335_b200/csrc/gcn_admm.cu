@@ -1130,6 +1130,7 @@ int guarded(gcn_admm* h, F&& body) {
     body();
     return GCN_ADMM_OK;
   } catch (const Fail& f) {
+    cudaGetLastError();   // reported here: the next call of this thread, on whichever handle, is not to find it again
     h->err = f.msg;
     return f.code;
   } catch (const std::bad_alloc&) {

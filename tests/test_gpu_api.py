@@ -84,6 +84,27 @@ def test_two_handles_do_not_interfere_and_launches_are_counted():
         ref.destroy()
 
 
+def test_a_failed_allocation_is_reported_once():
+    """A wide propagation whose workspace no device holds (items x 2^24 floats) fails before anything is launched; the next
+    calls of the thread, on another handle and on the same one, are not to meet that error again."""
+    import torch
+    wl = inputs.make_workload(0)
+    a, b = make(wl, long_row=1), make(wl)
+    try:
+        width = 1 << 24
+        assert 4 * width * wl.col_idx.size > 2 * torch.cuda.mem_get_info()[1]
+        x = torch.zeros(2, 16, device="cuda")
+        with pytest.raises(binding.GcnAdmmError) as e:
+            a.propagate(x[0].data_ptr(), width, x[1].data_ptr())
+        assert e.value.code == -5, str(e.value)
+        b.step(1)
+        a.step(1)
+        assert np.array_equal(a.weights(1), b.weights(1))
+    finally:
+        a.destroy()
+        b.destroy()
+
+
 def splitmix64(x):
     """Output function of the splitmix64 generator at state x + 0x9E3779B97F4A7C15 (Steele, Lea, Flood 2014)."""
     m = (1 << 64) - 1
