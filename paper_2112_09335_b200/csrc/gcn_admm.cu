@@ -180,6 +180,7 @@ struct gcn_admm {
   };
   void collect_profile() {
     cudaStreamSynchronize(stream);
+    event_pool.reserve(event_pool.size() + 2 * pending.size());
     for (ProfPending& q : pending) {
       float ms = 0.f;
       if (cudaEventElapsedTime(&ms, q.a, q.b) == cudaSuccess) q.stat->ms += ms;
@@ -1516,7 +1517,8 @@ void gcn_admm_destroy(gcn_admm* h) {
   if (!h) return;
   if (cudaSetDevice(h->p.device) == cudaSuccess) {
     cudaStreamSynchronize(h->stream);
-    h->collect_profile();
+    for (const ProfPending& q : h->pending)
+      for (cudaEvent_t e : {q.a, q.b}) cudaEventDestroy(e);
     if (h->pass_graph) cudaGraphExecDestroy(h->pass_graph);
     if (h->side.stream) {
       cudaStreamSynchronize(h->side.stream);

@@ -20,6 +20,7 @@
 #include <cstddef>
 #include <cstring>
 #include <mutex>
+#include <new>
 #include <utility>
 #include <vector>
 
@@ -73,25 +74,27 @@ class Pool {
     }
     return e;
   }
+  // What follows is called where a handle ends and throws nothing: what cannot be noted down for keeping is freed.
   // The slab's device is current and no work uses the slab any more.
-  void give(const Slab& s) {
+  void give(const Slab& s) noexcept {
     if (!s.base) return;
-    std::vector<Slab> out;   // the oldest make room; their work has finished too
-    {
-      std::lock_guard<std::mutex> lock(mutex_);
-      if (s.size <= kIdleSlabBytes) {
-        while (idle_bytes_ + s.size > kIdleSlabBytes) {
-          out.push_back(idle_.front());
-          idle_bytes_ -= idle_.front().size;
-          idle_.erase(idle_.begin());
+    for (;;) {   // the oldest make room; their work has finished too
+      Slab oldest;
+      {
+        std::lock_guard<std::mutex> lock(mutex_);
+        if (s.size > kIdleSlabBytes) break;
+        if (idle_bytes_ + s.size <= kIdleSlabBytes) {
+          if (!note(idle_, s)) break;
+          idle_bytes_ += s.size;
+          return;
         }
-        idle_bytes_ += s.size;
-        idle_.push_back(s);
-      } else {
-        out.push_back(s);
+        oldest = idle_.front();
+        idle_bytes_ -= oldest.size;
+        idle_.erase(idle_.begin());
       }
+      cudaFree(oldest.base);
     }
-    for (const Slab& o : out) cudaFree(o.base);
+    cudaFree(s.base);
   }
   char* take_stage() {
     {
@@ -106,11 +109,11 @@ class Pool {
     if (cudaHostAlloc(&p, kSlot * kSlots, cudaHostAllocPortable) != cudaSuccess) { cudaGetLastError(); return nullptr; }
     return static_cast<char*>(p);
   }
-  void give_stage(char* p) {
+  void give_stage(char* p) noexcept {
     if (!p) return;
     {
       std::lock_guard<std::mutex> lock(mutex_);
-      if (stages_.size() < kIdleStages) { stages_.push_back(p); return; }
+      if (stages_.size() < kIdleStages && note(stages_, p)) return;
     }
     cudaFreeHost(p);
   }
@@ -127,15 +130,15 @@ class Pool {
     }
     return cudaStreamCreateWithFlags(out, cudaStreamNonBlocking);
   }
-  void give_stream(int device, cudaStream_t s) {
+  void give_stream(int device, cudaStream_t s) noexcept {
     {
       std::lock_guard<std::mutex> lock(mutex_);
-      if (streams_.size() < kIdleStages) { streams_.push_back({device, s}); return; }
+      if (streams_.size() < kIdleStages && note(streams_, std::make_pair(device, s))) return;
     }
     cudaStreamDestroy(s);
   }
   // Gives everything idle back to the driver.
-  void release() {
+  void release() noexcept {
     release_slabs(kAnyDevice);
     std::vector<char*> stages;
     std::vector<std::pair<int, cudaStream_t>> streams;
@@ -152,16 +155,23 @@ class Pool {
  private:
   static constexpr int kAnyDevice = -1;
   // Whether there was anything to give back.
-  bool release_slabs(int device) {
-    std::vector<Slab> out;
-    {
-      std::lock_guard<std::mutex> lock(mutex_);
-      for (auto it = idle_.begin(); it != idle_.end();)
-        if (device == kAnyDevice || it->device == device) { out.push_back(*it); idle_bytes_ -= it->size; it = idle_.erase(it); }
-        else ++it;
+  bool release_slabs(int device) noexcept {
+    for (bool any = false;; any = true) {
+      Slab s;
+      {
+        std::lock_guard<std::mutex> lock(mutex_);
+        const auto it = std::find_if(idle_.begin(), idle_.end(), [&](const Slab& q) { return device == kAnyDevice || q.device == device; });
+        if (it == idle_.end()) return any;
+        s = *it;
+        idle_bytes_ -= s.size;
+        idle_.erase(it);
+      }
+      cudaFree(s.base);
     }
-    for (const Slab& s : out) cudaFree(s.base);
-    return !out.empty();
+  }
+  template <typename T>
+  static bool note(std::vector<T>& list, const T& x) noexcept {
+    try { list.push_back(x); return true; } catch (const std::bad_alloc&) { return false; }
   }
   std::mutex mutex_;
   std::vector<Slab> idle_;

@@ -3,6 +3,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <map>
+#include <new>
 #include <vector>
 
 #include "memory.hpp"
@@ -26,6 +27,15 @@ cudaError_t CUDARTAPI cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { ++s
 cudaError_t CUDARTAPI cudaStreamDestroy(cudaStream_t) { --streams; return cudaSuccess; }
 cudaError_t CUDARTAPI cudaGetLastError() { return cudaSuccess; }
 }
+
+static bool no_memory = false;   // every allocation of the host's fails
+void* operator new(std::size_t n) {
+  void* p = no_memory ? nullptr : std::malloc(n);
+  if (!p) throw std::bad_alloc();
+  return p;
+}
+void operator delete(void* p) noexcept { std::free(p); }
+void operator delete(void* p, std::size_t) noexcept { std::free(p); }
 
 #define NEED(c) \
   if (!(c)) { std::printf("line %d: %s\n", __LINE__, #c); return 1; }
@@ -74,6 +84,22 @@ int main(int argc, char** argv) {
   NEED(pool.allocate(0, 3 * GB, &p) == cudaSuccess && failures == 1 && device_bytes == 4 * GB);
   NEED(pool.allocate(0, GB, &p) == cudaErrorMemoryAllocation && failures == 2 && device_bytes == 4 * GB);   // nothing of device 0 is idle: no second try
   NEED(pool.take(1, GB, &c) == cudaSuccess && c.base == b.base);
+
+  // a handle ends without host memory: nothing is thrown, what cannot be kept goes back
+  pool.release();
+  limit = 8 * GB;
+  device_bytes = 0;
+  std::vector<Slab> many(64);
+  for (Slab& s : many) NEED(pool.take(0, GB / 32, &s) == cudaSuccess);
+  stage[0] = pool.take_stage();
+  NEED(pool.take_stream(0, &st) == cudaSuccess);
+  no_memory = true;
+  for (const Slab& s : many) pool.give(s);
+  pool.give_stage(stage[0]);
+  pool.give_stream(0, st);
+  pool.release();
+  no_memory = false;
+  NEED(device_bytes == 0 && host_bytes == 0 && streams == 0);
   std::printf("ok\n");
   return 0;
 }
