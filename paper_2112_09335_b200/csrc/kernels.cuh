@@ -1047,8 +1047,9 @@ k_search_w_hidden(const SearchW p) {
   __shared__ double sh[kCand * 8], total[kCand];
   SearchCtl* const ctl = p.ctl;
   const long long first = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
-  if (__ldcg(p.err) != 0) return;   // see GridBar
-  if (ctl->done) {                  // skipped: the same in every block
+  const int gave_up = __ldcg(p.err), skipped = ctl->done;   // side by side: one latency
+  if (gave_up != 0) return;         // see GridBar
+  if (skipped) {                    // the same in every block
     if (first == 0) log_decision(p.log, 0, ctl);
   } else {
     bool open = true;
@@ -1605,8 +1606,9 @@ k_close_z(const int* __restrict__ row_ptr, const int* __restrict__ col,
           const unsigned short* __restrict__ col_comm, const float* __restrict__ dinv,
           const float4* __restrict__ T, const float4* __restrict__ Hn, const float4* __restrict__ Zn, int ld4, int n, int use_smem, const int* __restrict__ chunk_ptr, int n_chunks,
           const int4* __restrict__ items, int n_items, int long_len, float4* scratch, const SearchZ sz) {
-  if (__ldcg(sz.err) != 0) return;   // see GridBar
-  if (__ldcg(sz.n_active) > 0) {
+  const int gave_up = __ldcg(sz.err), active = __ldcg(sz.n_active);   // side by side: one latency
+  if (gave_up != 0) return;   // see GridBar
+  if (active > 0) {
     for (int scored = sz.a.cand;; scored += sz.a.cand) {
       if (!close_sweep<V>(sz, n_chunks, dinv, scratch, Hn, Zn, ld4)) return;
       if (__ldcg(sz.n_active) <= 0 || scored >= sz.a.max_trials) break;   // *n_active changes only between the meetings of close_sweep
