@@ -76,7 +76,8 @@ enum {
  *                  this many entries, each walked by a warp of its own, and the items' sums are added up
  *                  in a fixed order afterwards (the paper's graphs have power-law degrees; a hub row
  *                  walked by one warp would outlast the rest of the launch).  Same sums up to fp32
- *                  rounding order.  0: the default, 256; a value above the longest row switches it off
+ *                  rounding order.  0: a length chosen by the size of the graph, 48 to 256; a value above the
+ *                  longest row switches it off
  *  w_init          L host pointers to row-major C_{l-1} x C_l matrices, or NULL: then every W_l is drawn
  *                  Glorot-uniform, entry (i, j) of W_l = a (2 u - 1) with a = sqrt(6 / (C_{l-1} + C_l)) and
  *                  u = (top 24 bits of splitmix64(seed + 2^32 l + i C_l + j)) / 2^24, where splitmix64(x) is

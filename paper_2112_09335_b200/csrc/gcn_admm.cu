@@ -43,7 +43,19 @@ constexpr int kZBlockRows = 32;      // rows per block of the hidden-layer gradi
 constexpr int kChunkGroups = 512;    // groups the sums of a scoring sweep's chunks are first added up in, when there are more chunks
 constexpr size_t kDirectBytes = (size_t)256 << 10;   // matrices up to this size cross the bus inside the permuting kernel (one copy and its latency less)
 constexpr long long kSmallProblem = 1LL << 27;   // nodes x widest layer: below it launch gaps show in a pass
-constexpr int kDefaultLongRow = 256;   // stored entries one warp walks before a row is cut into items
+// Stored entries one warp walks before a row is cut into items, where the caller leaves it open.  A warp that walks a long row alone
+// outlasts a launch whose warps have few entries each, and every cut costs an item's sums written, read and added up; the line
+// lies where the two meet, the lower the fewer entries a resident warp has, and well above the mean row (at twice it few rows are
+// cut).  us at 32 / 48 / 64 / 96 / 128 / 256 entries: 13 k rows, 0.15 M entries, six passes 2761 / 2757 / 2761 / 2806 / 2867 / 3099;
+// 23 k, 0.12 M, objective curve 769 / 782 / 788 / 815 / 833 / 935; 30 k, 0.51 M, serial 2270 / 2244 / 2247 / 2255 / 2289 / 2454;
+// 47 k, 1.6 M 3891 / 3762 / 3691 / 3688 / 3730 / 3921; 169 k, 2.5 M 10983 / 10834 / 10689 / 10689 / 10826 / 10868; 239 k, 6.7 M
+// 2631 / 2474 / 2380 / 2327 / 2325 / 2330; 409 k, 12.4 M 3720 / 3358 / 3185 / 3019 / 2956 / 2867.  127 k rows of 46 entries lose at 64.
+// Under 4,096 rows a launch is a wave of short chains and no length differs from 256 by more than its runs do.
+int default_long_row(long long n, long long nnz) {
+  if (n < 4096 || nnz > 8000000) return 256;
+  const int line = nnz <= 300000 ? 48 : nnz <= 2000000 ? 64 : 96;
+  return (int)std::min<long long>(256, std::max<long long>(line, 2 * nnz / n));
+}
 
 thread_local std::string g_create_error;
 
@@ -1245,7 +1257,7 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
     }
   }
   h->want_table(h->d_fista_momentum, mom);
-  h->long_len = p.long_row > 0 ? p.long_row : kDefaultLongRow;
+  h->long_len = p.long_row > 0 ? p.long_row : default_long_row(n, g.nnz);
   gcn_admm_host::LongRowTables lt;
   gcn_admm_host::build_long_row_tables(g, h->long_len, lt);
   h->n_items = (int)lt.items.size();

@@ -131,3 +131,20 @@ def test_workspace_of_wide_propagations():
     check(300)                                       # loads the kernels
     grown, workspace = check(3000)
     assert workspace <= grown <= 1.25 * workspace    # (1000 + 1400) / 2000 more with all three kept; the driver takes some MB of its own
+
+
+@pytest.mark.parametrize("index,scale", [(3, 0.03), (3, 0.2), (4, 0.01), (3, 1.0)])   # 48, 64, twice the mean row, 96
+def test_default_length_of_items(index, scale):
+    """The length a handle chooses from its graph's size: every row as the oracle's, rounding of partial sums apart."""
+    wl = inputs.make_workload(index, scale=scale)
+    g = handle(wl)
+    try:
+        At = orc.normalized_adjacency(wl.n, wl.row_ptr, wl.col_idx)
+        for width in (3, 40, 137):
+            x = np.random.default_rng(width).standard_normal((wl.n, width)).astype(np.float32)
+            got, want = g.propagate(x), At @ x.astype(np.float64)
+            # pieces and items of at most 256 entries each: sums of fp32 roundings, far below 2^-24 times a row's entries
+            scale_of = abs(At) @ np.abs(x.astype(np.float64)) + 1e-30
+            assert np.max(np.abs(got - want) / scale_of) < 1e-6
+    finally:
+        g.destroy()
