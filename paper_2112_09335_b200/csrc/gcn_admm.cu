@@ -17,6 +17,7 @@
 #include <string>
 #include <vector>
 
+#include "gemm_half.cuh"
 #include "gemm_tc.cuh"
 #include "graph_index.hpp"
 #include "kernels.cuh"
@@ -38,7 +39,7 @@ namespace {
 
 constexpr int kLogPasses = 256;
 constexpr int kSmCount = 148;
-constexpr long long kImageMinRows = 16384;   // row count from which the weight operand is pre-split
+constexpr long long kHalfMinRows = 16384;    // row count from which products of any width go by split halves
 constexpr int kZBlockRows = 32;      // rows per block of the hidden-layer gradient's closing sweep
 constexpr int kChunkGroups = 512;    // groups the sums of a scoring sweep's chunks are first added up in, when there are more chunks
 constexpr size_t kDirectBytes = (size_t)256 << 10;   // matrices up to this size cross the bus inside the permuting kernel (one copy and its latency less)
@@ -113,8 +114,8 @@ EncodeTiledFn encode_tiled() {
 }
 
 // Tensor map of a row-major rows x ld fp32 matrix for 128-row x 32-column tiles written with the 128-byte
-// swizzle; elements outside the matrix read as zero.  False when the map cannot be made (the caller then
-// stages the operand through registers).
+// swizzle; elements outside the matrix read as zero.  False when the map cannot be made (the product then takes the
+// form that stages the operand through registers).
 bool make_a_tile_map(const float* A, long long rows, int ld, CUtensorMap* map) {
   EncodeTiledFn fn = encode_tiled();
   if (fn == nullptr || ld < gtc::kChunkK) return false;
@@ -234,7 +235,9 @@ struct gcn_admm {
   float* grad = nullptr;     // max over l of C_{l-1} x ld_l
   float* grad_t = nullptr;   // its transpose, C_l x ld_{l-1} (K-major operand of the tensor-core product)
   int* tc_error = nullptr;   // &report->error: raised by a tensor-core product (1) or a search (2) whose bounded wait ran out
-  std::vector<gtc::Image> img_H, img_G, img_D;   // 1..L: kept images of W_l for P_l W_l, of W_l for S W_l^T, of the gradient for P_l grad
+  std::vector<gtc::Image> img_H, img_G, img_D;   // 1..L: images of W_l for P_l W_l, of W_l for S W_l^T, of the gradient for P_l grad
+  std::vector<float*> P_max;                     // 1..L: row maxima of P_l; NULL where no product of it takes them
+  float *B1_max = nullptr, *B2_max = nullptr;    // of S and G (B1, B2) while a Z update uses them, of the forward pass's operands
   float* part = nullptr;     // split partial sums of the transposed product
   size_t part_elems = 0;
   SearchCtl *ctl_w = nullptr, *ctl_z = nullptr;   // [L+1], [(L+1) * M]
@@ -334,12 +337,18 @@ struct gcn_admm {
   }
 
   // ---- launches -----------------------------------------------------------------------
-  void spmm(const float* x, float* out, int ldx, bool relu = false) {
+  // out_max: where the row maxima of the result go, or NULL
+  void spmm(const float* x, float* out, int ldx, float* out_max, bool relu = false) {
     char name[48];
     std::snprintf(name, sizeof name, "spmm@%d", ldx);
     Scope sc(this, name, 1, 4.0 * gi.nnz + 8.0 * n + 8.0 * (double)n * ldx, 2.0 * (double)gi.nnz * ldx);
-    if (relu) spmm_tables<4, false, true>(gather_graph(ldx), x, out, ldx / 4);
-    else spmm_tables<4, false>(gather_graph(ldx), x, out, ldx / 4);
+    if (relu) spmm_tables<4, false, true>(gather_graph(ldx), x, out, ldx / 4, out_max);
+    else spmm_tables<4, false>(gather_graph(ldx), x, out, ldx / 4, out_max);
+    if (out_max != nullptr && ldx > 256) {   // its rows are shared by blocks
+      launch_alone(gk::k_row_max, grid_for(32 * n), 256, 0, (const float4*)out, ldx / 4, n, out_max);
+      CU(cudaGetLastError());
+      ++launches;
+    }
   }
 
   // out = A~ x for dense n x width device matrices in the caller's row order, in vectors as wide as the width and
@@ -423,7 +432,7 @@ struct gcn_admm {
   // The propagation kernels on a graph given by its tables (the handle's own, or a rank's local part of it); x and
   // out have ldv vectors of VEC floats per row.
   template <int VEC, bool MAPPED, bool RELU = false>
-  void spmm_tables(const GatherGraph& g, const float* xf, float* outf, int ldv) {
+  void spmm_tables(const GatherGraph& g, const float* xf, float* outf, int ldv, float* row_max = nullptr) {
     using T = typename gk::Vec<VEC>::T;
     const T* x = reinterpret_cast<const T*>(xf);
     T *out = reinterpret_cast<T*>(outf), *scratch = reinterpret_cast<T*>(g.item_sums);
@@ -433,10 +442,10 @@ struct gcn_admm {
 #define WIDE(NV4, UN, SLICED)                                                                                             \
   launch_alone(gk::k_spmm_wide<VEC, 4 / VEC * (NV4), UN, MAPPED, SLICED, RELU>, dim3((unsigned)cdiv(units * 32, 64), (unsigned)std::min<long long>(32768, cdiv(ld4, 32 * (NV4))),                \
               (unsigned)cdiv(ld4, 32768LL * 32 * (NV4))), 64, 0,                                                \
-      g.row_ptr, g.col, g.dinv, g.perm, g.items, g.n, g.n_items, g.long_len, x, out, ldv, scratch)
+      g.row_ptr, g.col, g.dinv, g.perm, g.items, g.n, g.n_items, g.long_len, x, out, ldv, scratch, row_max)
 #define SETS(CL, EP, UN)                                                                                                  \
   launch(gk::k_spmm_sets<VEC, 4 / VEC, CL, EP, UN, MAPPED, RELU>, (unsigned)cdiv(units * ((CL) * (EP)), 128), 128, 0,  \
-      g.row_ptr, g.col, g.dinv, g.perm, g.items, g.n, g.n_items, g.long_len, x, out, ldv, scratch, g.row_order, gk::ItemRows{g.rows, g.item_row, g.row_done})
+      g.row_ptr, g.col, g.dinv, g.perm, g.items, g.n, g.n_items, g.long_len, x, out, ldv, scratch, g.row_order, gk::ItemRows{g.rows, g.item_row, g.row_done}, row_max)
     // Sets of entries per row: as many as the warp holds while the grid is then still small (latency counts), fewer
     // where the rows alone fill the chip several times over and the lanes of half-empty sets would only cost issue
     // slots.  Lines between the measured sizes 0.2 / 1.4 / 20 M lanes (columns x rows); the rule reads the handle's n, so a
@@ -460,79 +469,79 @@ struct gcn_admm {
     in_pass = true;
     CU(cudaGetLastError());
     if (ld4 > 16 && g.n_long > 0) {
-      launch(gk::k_spmm_long_rows<T, MAPPED>, (unsigned)g.n_long, 64, 0, g.rows, scratch, out, ldv, g.perm);
+      launch(gk::k_spmm_long_rows<T, MAPPED>, (unsigned)g.n_long, 64, 0, g.rows, scratch, out, ldv, g.perm, row_max);
       CU(cudaGetLastError());
       ++launches;   // booked with the propagation it completes
     }
   }
 
   // Whether C = A B with these sizes runs on the tensor cores (K capped at 2048 because the accumulator error grows with K,
-  // about 2.5e-9 K of the magnitude), and how: columns per group, and whether B is taken from an image of the staged layout.
+  // about 2.5e-9 K of the magnitude), and how: columns per group, and whether by split halves (B then comes as an image).
   bool on_tensor_cores(long long Mr, int K) const { return p.tensor_cores && K >= 8 && K <= 2048 && Mr >= 512; }
-  int group_width(long long Mr, int N, int K, int lda) const {
-    if (N <= 16) return 16;
-    if (N <= 32) return 32;
-    if (N <= 48) return 48;
-    if (N <= 64) return 64;
-    if (N <= 128) return 128;
-    // 129..256 columns with a short reduction (K <= 128: a tile has at most four chunks of MMAs, so the epilogue
-    // that the single accumulator set of the 256-column form leaves uncovered dominates): two groups of 128 columns
-    // in the tensor-copy form instead, whose two accumulator sets put the epilogue under the next tile's MMAs
-    // (measured on 1.2 M rows: 0.372 -> 0.326 ms at K = 47, 0.560 -> 0.463 at 100, 0.518 -> 0.456 at 128; no gain at 256)
-    return K <= 128 && lda >= gtc::kChunkK && Mr >= kImageMinRows ? 128 : 256;
+  static int group_width(int N, bool halves) {
+    return N <= 16 ? 16 : N <= 32 ? 32 : N <= 48 ? 48 : N <= 64 ? 64 : halves && N <= 96 ? 96 : N <= 128 ? 128 : halves && N <= 192 ? 192 : 256;
   }
-  // With many row tiles the producers would split the same weights again for every tile; with at most one tile per CTA, or
-  // with few chunks, that costs nothing (13.8 k rows, 767 x 1000, three tiles per CTA: 130 -> 98 us; 10 x 1000: no gain).
-  bool takes_image(long long Mr, int N, int K, int nt) const {
-    return p.tensor_cores == 2 || Mr >= kImageMinRows || (K >= 128 && cdiv(Mr, gtc::kBlockM) > kSmCount / cdiv(N, nt));
+  // With many row tiles k_gemm_tc_ws would split the same weights again for every tile; with at most one tile per CTA, or
+  // with few chunks, that costs nothing, and the launch that makes the image would (13.8 k rows, 767 x 1000, three tiles per CTA:
+  // 130 -> 98 us by an image; 10 x 1000: no gain).  A's tensor copies want rows of at least one chunk.
+  bool by_halves(long long Mr, int N, int K, int lda) const {
+    if (!on_tensor_cores(Mr, K) || lda < gtc::kChunkK || encode_tiled() == nullptr) return false;
+    return p.tensor_cores == 2 || Mr >= kHalfMinRows || (K >= 128 && cdiv(Mr, gtc::kBlockM) > kSmCount / cdiv(N, group_width(N, true)));
   }
-  static size_t image_bytes(int N, int K, int nt) { return (size_t)cdiv(N, nt) * cdiv(K, gtc::kChunkK) * 2 * nt * gtc::kChunkK * 4; }
-  // Asks for a kept image of the operand of an n x K by K x N product, where that product takes one.
+  static size_t image_bytes(int N, const gtc::Image& im) {
+    const int groups = (int)cdiv(N, im.nt);
+    return gtc::image_blocks_bytes(groups, im.nt, im.kc) + (size_t)groups * im.nt * sizeof(float);
+  }
+  // Asks for an image of the operand of an n x K by K x N product, where that product takes one.
   void want_image(gtc::Image& im, int N, int K, int lda) {
-    im = gtc::Image{nullptr, group_width(n, N, K, lda), (int)cdiv(K, gtc::kChunkK)};
-    if (on_tensor_cores(n, K) && takes_image(n, N, K, im.nt)) want(im.data, image_bytes(N, K, im.nt), kZero);
+    im = gtc::Image{nullptr, group_width(N, true), (int)cdiv(K, gtc::kChunkK)};
+    if (by_halves(n, N, K, lda)) want(im.data, image_bytes(N, im), kZero);
+  }
+  void split_b(const gtc::SplitB& b) {
+    const int rows = (int)(cdiv(b.N, b.image.nt) * b.image.nt);
+    Scope sc(this, "split_b", 1, 8.0 * (double)b.N * b.K, 0.0);
+    launch(gtc::k_split_b, (unsigned)cdiv(rows, 8), 256, 0, b, rows);
+    CU(cudaGetLastError());
   }
 
   // C = A B.  B is handed over twice: row-major K x N (ldb) for the fp32-ALU kernels and K-major N x K (Bk, ldbk; may be
-  // NULL) for the tensor-core kernel, which is used whenever it applies; `kept`: its image, where the product takes one.
-  void gemm_nn(const float* A, int lda, const float* B, int ldb, const float* Bk, int ldbk, float* Cm, int ldc,
-               long long Mr, int N, int K, const gtc::Image* kept = nullptr, const int* skip = nullptr) {
+  // NULL) for the tensor-core kernels, which are used whenever they apply; a_max, image: the row maxima of A and the image of B,
+  // for the product by split halves.
+  void gemm_nn(const float* A, int lda, const float* a_max, const float* B, int ldb, const float* Bk, int ldbk, float* Cm, int ldc,
+               long long Mr, int N, int K, const gtc::Image& image, const int* skip = nullptr) {
     char name[48];
     if (Bk != nullptr && on_tensor_cores(Mr, K)) {
-      std::snprintf(name, sizeof name, "gemm_tc@%dx%d", K, N);
-      Scope sc(this, name, 1, 4.0 * ((double)Mr * (lda + ldc) + (double)K * ldb), 2.0 * (double)Mr * N * K);
-      const int tiles = (int)cdiv(Mr, gtc::kBlockM), nt = group_width(Mr, N, K, lda), groups = (int)cdiv(N, nt), kc = (int)cdiv(K, gtc::kChunkK);
-      dim3 grid((unsigned)std::max(1, std::min(tiles, kSmCount / groups)), (unsigned)groups);
       CUtensorMap tmap;
-      std::memset(&tmap, 0, sizeof tmap);
-      const uint8_t* const image = takes_image(Mr, N, K, nt) && kept != nullptr ? kept->data : nullptr;
+      const bool halves = by_halves(Mr, N, K, lda) && a_max != nullptr && image.data != nullptr && make_a_tile_map(A, Mr, lda, &tmap);
+      const int tiles = (int)cdiv(Mr, gtc::kBlockM), nt = group_width(N, halves), groups = (int)cdiv(N, nt), kc = (int)cdiv(K, gtc::kChunkK);
+      std::snprintf(name, sizeof name, halves ? "gemm_half@%dx%d" : "gemm_tc@%dx%d", K, N);
+      Scope sc(this, name, 1, 4.0 * ((double)Mr * (lda + ldc) + (double)K * ldb), 2.0 * (double)Mr * N * K);
+      dim3 grid((unsigned)std::max(1, std::min(tiles, kSmCount / groups)), (unsigned)groups);
       // few row tiles and a long reduction: several CTAs share a tile's K chunks, at least four chunks each
       // (2.7 k rows, K = 1433, 16 columns: 34 -> 13 us)
-      if (image == nullptr)
+      if (!halves)
         grid.z = (unsigned)std::max<long long>(1, std::min<long long>({kSmCount / ((long long)tiles * groups), kc / 4,
                                                                        (long long)(part_elems / ((size_t)Mr * ldc))}));
-      // an image and up to 128 columns: A tiles by tensor copies into a ring of their own (at 256 columns shared memory
-      // leaves no room for it, and the form measured no faster there)
-      const bool copies = image != nullptr && nt <= 128 && make_a_tile_map(A, Mr, lda, &tmap);
-      auto run = [&](auto kernel, int threads, size_t smem) {
-        CU(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        launch_alone(kernel, grid, threads, smem, A, lda, Bk, ldbk, Cm, ldc, (int)Mr, N, K, skip, tc_error, image, tmap, part, tile_tickets);
-      };
       auto with_width = [&](auto width) {
         constexpr int NT = decltype(width)::value;
-        using Cfg = gtc::WsCfg<NT>;
-        if constexpr (NT <= 128) {
-          if (copies) { run(gtc::k_gemm_tc_ws<NT, true, true>, Cfg::kThreads + 32, Cfg::kSmemRing); return; }
+        if (halves) {
+          using Cfg = gtc::HalfCfg<NT>;
+          CU(cudaFuncSetAttribute(gtc::k_gemm_half<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::kSmem));
+          launch_alone(gtc::k_gemm_half<NT>, grid, Cfg::kThreads, Cfg::kSmem, a_max, Cm, ldc, (int)Mr, N, K, skip, tc_error, image.data, tmap);
+        } else if constexpr (NT != 96 && NT != 192) {
+          using Cfg = gtc::WsCfg<NT>;
+          CU(cudaFuncSetAttribute(gtc::k_gemm_tc_ws<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::kSmem));
+          launch_alone(gtc::k_gemm_tc_ws<NT>, grid, Cfg::kThreads, Cfg::kSmem, A, lda, Bk, ldbk, Cm, ldc, (int)Mr, N, K, skip, tc_error, part, tile_tickets);
         }
-        if (image != nullptr) run(gtc::k_gemm_tc_ws<NT, true, false>, Cfg::kThreads, Cfg::kSmem);
-        else run(gtc::k_gemm_tc_ws<NT, false, false>, Cfg::kThreads, Cfg::kSmem);
       };
       switch (nt) {
         case 16: with_width(std::integral_constant<int, 16>()); break;
         case 32: with_width(std::integral_constant<int, 32>()); break;
         case 48: with_width(std::integral_constant<int, 48>()); break;
         case 64: with_width(std::integral_constant<int, 64>()); break;
+        case 96: with_width(std::integral_constant<int, 96>()); break;
         case 128: with_width(std::integral_constant<int, 128>()); break;
+        case 192: with_width(std::integral_constant<int, 192>()); break;
         default: with_width(std::integral_constant<int, 256>());
       }
       CU(cudaGetLastError());
@@ -556,10 +565,11 @@ struct gcn_admm {
   // Whether P^T R runs on the tensor cores (that form can also build a hidden layer's R itself).
   bool tn_on_tensor_cores(long long rows) const { return p.tensor_cores != 0 && rows >= 4096; }
 
+  // part_max (tensor-core form only): raised to the largest magnitude among the partial sums, as bits.
   // With `zres` (tensor-core form only) B holds pre-activations H and the operand is
   // h > 0 ? nu (h - z) : 0, formed while staging: the residual matrix is never stored.
   int gemm_tn(const float* A, int lda, const float* B, int ldb, int ldp, long long rows, int Ka, int Nb,
-              const float* zres = nullptr, float nu = 0.f) {
+              const float* zres = nullptr, float nu = 0.f, unsigned* part_max = nullptr) {
     int splits = 1;
     long long rps = rows;
     char name[48];
@@ -587,10 +597,10 @@ struct gcn_admm {
     dim3 grid((unsigned)groups, (unsigned)splits, (unsigned)nb_groups);                                        \
     if (zres) {                                                                                                \
       CU(cudaFuncSetAttribute(gtc::k_gemm_tn_tc<NT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
-      launch_alone(gtc::k_gemm_tn_tc<NT, true>, grid, gtc::kTnThreads, smem, A, lda, B, ldb, part, ldp, rows, rps, Ka, Nb, tc_error, zres, nu); \
+      launch_alone(gtc::k_gemm_tn_tc<NT, true>, grid, gtc::kTnThreads, smem, A, lda, B, ldb, part, ldp, rows, rps, Ka, Nb, tc_error, zres, nu, part_max); \
     } else {                                                                                                   \
       CU(cudaFuncSetAttribute(gtc::k_gemm_tn_tc<NT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
-      launch_alone(gtc::k_gemm_tn_tc<NT, false>, grid, gtc::kTnThreads, smem, A, lda, B, ldb, part, ldp, rows, rps, Ka, Nb, tc_error, nullptr, 0.f); \
+      launch_alone(gtc::k_gemm_tn_tc<NT, false>, grid, gtc::kTnThreads, smem, A, lda, B, ldb, part, ldp, rows, rps, Ka, Nb, tc_error, nullptr, 0.f, part_max); \
     }                                                                                                          \
   }
       if (Nb <= 16) TN_TC(16)
@@ -696,13 +706,15 @@ struct gcn_admm {
     float *const R = resid_of(l), *const D = l == L && DL != nullptr ? DL : B1;
     int splits;
     if (l < L && tn_on_tensor_cores(n)) {                               // grad = P_l^T R_l, R_l formed inside the product
-      splits = gemm_tn(P[l], ld[l - 1], H[l], ldc, ldc, n, Kp, Cn, Z[l], p.nu);
+      splits = gemm_tn(P[l], ld[l - 1], H[l], ldc, ldc, n, Kp, Cn, Z[l], p.nu, &ctl->part_max);
     } else {
       resid(l, R);                                                      // R_l
-      splits = gemm_tn(P[l], ld[l - 1], R, ldc, ldc, n, Kp, Cn);        // grad = P_l^T R_l
+      splits = gemm_tn(P[l], ld[l - 1], R, ldc, ldc, n, Kp, Cn, nullptr, 0.f, &ctl->part_max);   // grad = P_l^T R_l
     }
-    finish_grad(splits, Kp, Cn, ldc, grad, grad_t, ld[l - 1], W[l], ctl, img_D[l]);
-    gemm_nn(P[l], ld[l - 1], grad, ldc, grad_t, ld[l - 1], D, ldc, n, Cn, Kp, &img_D[l], &ctl->done);   // D = P_l grad
+    const bool bounded = tn_on_tensor_cores(n);   // by the largest partial sum; else the image is made from the gradient itself
+    finish_grad(splits, Kp, Cn, ldc, grad, grad_t, ld[l - 1], W[l], ctl, bounded ? img_D[l] : gtc::Image{nullptr, 16, 1});
+    if (!bounded && img_D[l].data != nullptr) split_b(gtc::SplitB{grad_t, ld[l - 1], Cn, Kp, img_D[l]});
+    gemm_nn(P[l], ld[l - 1], P_max[l], grad, ldc, grad_t, ld[l - 1], D, ldc, n, Cn, Kp, img_D[l], &ctl->done);   // D = P_l grad
     gk::SearchW a{};
     a.H = (float4*)H[l]; a.D = (const float4*)D; a.Z = (const float4*)Z[l]; a.U = (const float4*)U; a.R = (const float4*)R;
     a.Rn = resid_next ? (float4*)R : nullptr;
@@ -725,9 +737,11 @@ struct gcn_admm {
         launch(gk::k_score_w_out, grid_for(n4), 256, 0, a);
         CU(cudaGetLastError());
       }
-      Scope sc(this, "move_w_out", 1, 16.0 * (3 + (resid_next ? 3 : 0)) * n4, 0.0);
-      launch(gk::k_move_w_out, grid_for(n4), 256, 0, a);
-      CU(cudaGetLastError());
+      {
+        Scope sc(this, "move_w_out", 1, 16.0 * (3 + (resid_next ? 3 : 0)) * n4, 0.0);
+        launch(gk::k_move_w_out, grid_for(n4), 256, 0, a);
+        CU(cudaGetLastError());
+      }
     } else {
       Scope sc(this, "search_w_hidden", 1, 16.0 * (6 + (resid_next ? 2 : 0)) * n4, 0.0);
       launch_together(gk::k_search_w_hidden, cdiv(n4, 256), 256, 0, a);
@@ -742,12 +756,16 @@ struct gcn_admm {
     SearchCtl* ctl = ctl_z + (size_t)l * M;
     float* const Rn = resid_of(l + 1);
     if (!resid_ready) resid(l + 1, Rn);                                  // R'_{l+1}
-    spmm(Rn, B1, ldn);                                                   // S = A~ R'
-    gemm_nn(B1, ldn, Wt[l + 1], ldl, W[l + 1], ldn, B2, ldl, n, C[l], C[l + 1], &img_G[l + 1]);        // S W_{l+1}^T
+    spmm(Rn, B1, ldn, img_G[l + 1].data != nullptr ? B1_max : nullptr);                                // S = A~ R'
+    gemm_nn(B1, ldn, B1_max, Wt[l + 1], ldl, W[l + 1], ldn, B2, ldl, n, C[l], C[l + 1], img_G[l + 1]); // S W_{l+1}^T
     {
       Scope sc(this, "zgrad_finish", 1, 16.0 * 4.0 * (double)n * (ldl / 4), 0.0);
-      launch(gk::k_zgrad_finish, (unsigned)n_zblocks, 256, 0, (float4*)B2, (const float4*)Z[l], (const float4*)H[l], ldl / 4, d_zblocks, p.nu, red_part, d_comm_block_ptr, comm_tickets, ctl, sums_z,
-          p.bt_shrink, p.bt_growth, n_active, status);
+      const auto finish = [&](auto kernel) {
+        launch(kernel, (unsigned)n_zblocks, 256, 0, (float4*)B2, (const float4*)Z[l], (const float4*)H[l], ldl / 4, d_zblocks, p.nu, red_part, d_comm_block_ptr, comm_tickets, ctl, sums_z,
+               p.bt_shrink, p.bt_growth, n_active, status, img_H[l + 1].data != nullptr ? B2_max : nullptr);
+      };
+      if (ldl <= 16) finish(gk::k_zgrad_finish<4>);
+      else finish(gk::k_zgrad_finish<8>);   // whole lines still, and few idle lanes at any width
       CU(cudaGetLastError());
     }
     const int ld4 = ldn / 4, warps = 8;
@@ -759,7 +777,7 @@ struct gcn_admm {
     decide.max_trials = p.bt_max_trials;
     decide.own_nu = p.nu;
     if (l + 1 == L) {   // closed form
-      gemm_nn(B2, ldl, W[L], ldn, Wt[L], ldl, B0, ldn, n, C[L], C[l], &img_H[L]);   // T = G W_L; S stays in B1
+      gemm_nn(B2, ldl, B2_max, W[L], ldn, Wt[L], ldl, B0, ldn, n, C[L], C[l], img_H[L]);   // T = G W_L; S stays in B1
       decide.mode = 1;
       decide.quad_coef = 0.5 * p.rho;
       gk::SearchOut a{};
@@ -797,7 +815,7 @@ struct gcn_admm {
       CU(cudaGetLastError());
       return;
     }
-    gemm_nn(B2, ldl, W[l + 1], ldn, Wt[l + 1], ldl, B1, ldn, n, C[l + 1], C[l], &img_H[l + 1]);         // T = G W_{l+1}
+    gemm_nn(B2, ldl, B2_max, W[l + 1], ldn, Wt[l + 1], ldl, B1, ldn, n, C[l + 1], C[l], img_H[l + 1]);         // T = G W_{l+1}
     decide.cand = gk::kCand;   // steady-state searches close at trial 0..2
     decide.scale = 0.5 * p.nu;
     gk::SearchZ a{};
@@ -882,13 +900,13 @@ struct gcn_admm {
   bool capturing = false;
   void refresh(bool keep_h1 = false) {
     Range range("gcn_admm: refresh P_l, H_l");
-    for (int l = 2; l <= L; ++l) spmm(Z[l - 1], P[l], ld[l - 1]);
+    for (int l = 2; l <= L; ++l) spmm(Z[l - 1], P[l], ld[l - 1], P_max[l]);
     refresh_H1(keep_h1);
     for (int l = 2; l <= L; ++l) refresh_H(l);
     fresh = true;
   }
   void refresh_H(int l, const int* skip = nullptr) {
-    gemm_nn(P[l], ld[l - 1], W[l], ld[l], Wt[l], ld[l - 1], H[l], ld[l], n, C[l], C[l - 1], &img_H[l], skip);
+    gemm_nn(P[l], ld[l - 1], P_max[l], W[l], ld[l], Wt[l], ld[l - 1], H[l], ld[l], n, C[l], C[l - 1], img_H[l], skip);
   }
   void refresh_H1(bool keep_h1) {
     const bool skip = keep_h1 && !capturing && h1_age + 1 < kH1RefreshEvery;
@@ -908,7 +926,7 @@ struct gcn_admm {
     if (!fresh) refresh();
     for (int l = 1; l <= L; ++l) {
       if (l >= 2) {   // Z_{l-1} has just moved: P_l and H_l follow it (H_{l+1} still matches the untouched Z_l)
-        spmm(Z[l - 1], P[l], ld[l - 1]);
+        spmm(Z[l - 1], P[l], ld[l - 1], P_max[l]);
         refresh_H(l);
       }
       update_W(l, false);
@@ -989,7 +1007,7 @@ struct gcn_admm {
         end_pass();
         CU(cudaEventRecord(side.done, stream));
       });
-      for (int l = 2; l <= L; ++l) spmm(Z[l - 1], P[l], ld[l - 1]);
+      for (int l = 2; l <= L; ++l) spmm(Z[l - 1], P[l], ld[l - 1], P_max[l]);
       join(stream, side.out_done);   // its rows of H_L have been read
       for (int l = 2; l <= L; ++l) refresh_H(l);
       join(stream, side.done);
@@ -1000,10 +1018,9 @@ struct gcn_admm {
     end_pass();
   }
 
-  void relu(const float* x, float* out, int ldx) {
-    const long long n4 = n * ldx / 4;
-    Scope sc(this, "relu", 1, 32.0 * n4, 0.0);
-    gk::k_relu<<<grid_for(n4), 256, 0, stream>>>((const float4*)x, (float4*)out, n4);
+  void relu(const float* x, float* out, int ldx, float* out_max = nullptr) {
+    Scope sc(this, "relu", 1, 8.0 * (double)n * ldx, 0.0);
+    gk::k_relu<<<grid_for(32 * n), 256, 0, stream>>>((const float4*)x, (float4*)out, ldx / 4, n, out_max);
     CU(cudaGetLastError());
   }
 
@@ -1015,18 +1032,19 @@ struct gcn_admm {
   const float* forward_logits() {
     const float* h = H[1];
     if (!fresh) {
-      gemm_nn(P[1], ld[0], W[1], ld[1], Wt[1], ld[0], B0, ld[1], n, C[1], C[0], &img_H[1]);
+      gemm_nn(P[1], ld[0], P_max[1], W[1], ld[1], Wt[1], ld[0], B0, ld[1], n, C[1], C[0], img_H[1]);
       h = B0;
     }
     for (int l = 1; l < L; ++l) {
       float *const out = h == B0 ? B1 : B0, *const mid = out == B0 ? B1 : B0;
+      float* const max = img_H[l + 1].data != nullptr ? B2_max : nullptr;
       if (gi.nnz * (long long)(ld[l] - ld[l + 1]) >= 8 * n * ld[l]) {
-        relu(h, B2, ld[l]);
-        gemm_nn(B2, ld[l], W[l + 1], ld[l + 1], Wt[l + 1], ld[l], mid, ld[l + 1], n, C[l + 1], C[l], &img_H[l + 1]);
-        spmm(mid, out, ld[l + 1]);
+        relu(h, B2, ld[l], max);
+        gemm_nn(B2, ld[l], max, W[l + 1], ld[l + 1], Wt[l + 1], ld[l], mid, ld[l + 1], n, C[l + 1], C[l], img_H[l + 1]);
+        spmm(mid, out, ld[l + 1], nullptr);
       } else {
-        spmm(h, B2, ld[l], true);
-        gemm_nn(B2, ld[l], W[l + 1], ld[l + 1], Wt[l + 1], ld[l], out, ld[l + 1], n, C[l + 1], C[l], &img_H[l + 1]);
+        spmm(h, B2, ld[l], max, true);
+        gemm_nn(B2, ld[l], max, W[l + 1], ld[l + 1], Wt[l + 1], ld[l], out, ld[l + 1], n, C[l + 1], C[l], img_H[l + 1]);
       }
       h = out;
     }
@@ -1103,7 +1121,9 @@ struct gcn_admm {
     CU(stage.put(grad, host_w, sizeof(float) * (size_t)r * c, stream));
     CU(stage.finish(stream));
     const long long cells = std::max((long long)r * ld[l], (long long)c * ld[l - 1]);
-    gk::k_load_weight<<<grid_for(cells), 256, 0, stream>>>(grad, r, c, W[l], ld[l], Wt[l], ld[l - 1], img_H[l], img_G[l]);
+    float most = 0.f;
+    for (long long e = 0; e < (long long)r * c; ++e) most = std::max(most, std::fabs(host_w[e]));
+    gk::k_load_weight<<<grid_for(cells), 256, 0, stream>>>(grad, r, c, W[l], ld[l], Wt[l], ld[l - 1], img_H[l], img_G[l], most);
     CU(cudaGetLastError());
   }
   // Step parameters (t_prev) of `count` searches in a row, to and from the host.
@@ -1362,7 +1382,7 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
     h->want(h->side.part, h->side.part_elems);
     h->want(h->side.grad, ge);
     h->want(h->side.grad_t, (size_t)h->C[L] * h->ld[L - 1], gcn_admm::kZero);
-    h->want(h->side.red_part, std::max<size_t>((size_t)kSmCount * 8 * gk::kCand, (size_t)cdiv((long long)ge, 32) * 2));
+    h->want(h->side.red_part, std::max<size_t>((size_t)kSmCount * 8 * gk::kCand, (size_t)cdiv((long long)ge, 32) * 3));
     h->want_counter(h->side.ticket, 1);
     h->want_counter(h->side.tile_tickets, kSmCount);
     CU(gcn_admm_mem::Pool::get().take_stream(p.device, &h->side.stream));
@@ -1373,11 +1393,15 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
   h->want(h->grad, grad_elems);
   h->want(h->grad_t, grad_t_elems, gcn_admm::kZero);
   h->img_H.assign(L + 1, gtc::Image{nullptr, 16, 1}); h->img_G = h->img_D = h->img_H;
+  h->P_max.assign(L + 1, nullptr);
   for (int l = 1; l <= L; ++l) {
-    h->want_image(h->img_H[l], h->C[l], h->C[l - 1], h->ld[l - 1]);
+    h->want_image(h->img_H[l], h->C[l], h->C[l - 1], h->ld[l - 1]);   // P_l W_l, G W_l; P_l grad has its shape
     h->want_image(h->img_D[l], h->C[l], h->C[l - 1], h->ld[l - 1]);
     if (l >= 2) h->want_image(h->img_G[l], h->C[l - 1], h->C[l], h->ld[l]);
+    if (h->by_halves(n, h->C[l], h->C[l - 1], h->ld[l - 1])) h->want(h->P_max[l], rows);
   }
+  h->want(h->B1_max, rows);
+  h->want(h->B2_max, rows);
   h->want(h->part, h->part_elems);
   std::vector<SearchCtl> cw(L + 1), cz((size_t)(L + 1) * n_comm);
   std::memset(cw.data(), 0, cw.size() * sizeof(SearchCtl));
@@ -1408,7 +1432,7 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
   h->want_counter(h->comm_tickets, n_comm);
   h->want_counter(h->grid_bar, 1);
   h->want(h->red_part, std::max<size_t>({(size_t)kSmCount * 8 * gk::kCand, (size_t)h->n_zblocks * 3,
-                                         (size_t)cdiv(n, 8) * 2, grad_blocks * 2}));
+                                         (size_t)cdiv(n, 8) * 2, grad_blocks * 3}));
   h->want_counter(h->n_active, 1);
   h->want(h->d_pass, 1, gcn_admm::kZero);
   h->want(h->d_h1_age, 1, gcn_admm::kZero);
@@ -1433,7 +1457,7 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
       gk::k_permute_rows<<<h->grid_for(n * h->ld[0]), 256, 0, h->stream>>>(on_device ? X : h->B0, h->B1, h->d_inv, n, h->C[0], h->ld[0], 1);
       CU(cudaGetLastError());
     }
-    h->spmm(h->B1, h->P[1], h->ld[0]);
+    h->spmm(h->B1, h->P[1], h->ld[0], h->P_max[1]);
   }
 
   for (int l = 1; l <= L; ++l) {
@@ -1451,7 +1475,7 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
   // forward pass of Problem 1 with the same kernels that later recompute H_l, so that the
   // initial residuals are exactly zero
   for (int l = 1; l <= L; ++l) {
-    if (l >= 2) h->spmm(h->Z[l - 1], h->P[l], h->ld[l - 1]);
+    if (l >= 2) h->spmm(h->Z[l - 1], h->P[l], h->ld[l - 1], h->P_max[l]);
     h->refresh_H(l);
     if (l < L) h->relu(h->H[l], h->Z[l], h->ld[l]);
     else CU(cudaMemcpyAsync(h->Z[l], h->H[l], rows * h->ld[l] * sizeof(float), cudaMemcpyDeviceToDevice, h->stream));
@@ -1739,7 +1763,7 @@ int gcn_admm_dense_product(gcn_admm* h, const float* A, const float* B, float* C
     if (!is_device_pointer(A) || !is_device_pointer(B) || !is_device_pointer(C))
       throw Fail{GCN_ADMM_ERR_ARG, "A, B and C must be device pointers"};
     const int lda = ldpad(k), ldb = ldpad(n), ldc = ldpad(n), ldbk = ldpad(k);
-    float *a = nullptr, *b = nullptr, *bk = nullptr, *c = nullptr;
+    float *a = nullptr, *b = nullptr, *bk = nullptr, *c = nullptr, *a_max = nullptr;
     gtc::Image image{nullptr, 16, 1};
     const int saved = h->p.tensor_cores;
     try {
@@ -1755,24 +1779,26 @@ int gcn_admm_dense_product(gcn_admm* h, const float* A, const float* B, float* C
       gk::k_transpose_small<<<(unsigned)cdiv((long long)k * n, 256), 256, 0, h->stream>>>(b, ldb, bk, ldbk, k, n);
       CU(cudaGetLastError());
       h->p.tensor_cores = tensor_cores;
-      const int nt = h->group_width(m, n, k, lda);
-      if (h->on_tensor_cores(m, k) && h->takes_image(m, n, k, nt)) {
-        const long long units = cdiv(n, nt) * cdiv(k, gtc::kChunkK) * nt * 8;   // threads of k_split_b
-        image = gtc::Image{dalloc<uint8_t>(gcn_admm::image_bytes(n, k, nt)), nt, (int)cdiv(k, gtc::kChunkK)};
-        gtc::k_split_b<<<(unsigned)std::min<long long>(cdiv(units, 256), 4 * kSmCount), 256, 0, h->stream>>>(bk, ldbk, n, k, nt, image.data);
+      if (tensor_cores && h->by_halves(m, n, k, lda)) {
+        image.nt = gcn_admm::group_width(n, true);
+        image.kc = (int)cdiv(k, gtc::kChunkK);
+        image.data = dalloc<uint8_t>(gcn_admm::image_bytes(n, image));
+        a_max = dalloc<float>((size_t)m);
+        h->split_b(gtc::SplitB{bk, ldbk, n, k, image});
+        gk::k_row_max<<<h->grid_for(32 * m), 256, 0, h->stream>>>(reinterpret_cast<const float4*>(a), lda / 4, m, a_max);
         CU(cudaGetLastError());
         ++h->launches;
       }
-      h->gemm_nn(a, lda, b, ldb, tensor_cores ? bk : nullptr, ldbk, c, ldc, m, n, k, &image);
+      h->gemm_nn(a, lda, a_max, b, ldb, tensor_cores ? bk : nullptr, ldbk, c, ldc, m, n, k, image);
       h->p.tensor_cores = saved;
       CU(cudaMemcpy2DAsync(C, (size_t)n * 4, c, (size_t)ldc * 4, (size_t)n * 4, (size_t)m, cudaMemcpyDeviceToDevice, h->stream));
       CU(cudaStreamSynchronize(h->stream));
     } catch (...) {
       h->p.tensor_cores = saved;
-      cudaFree(a); cudaFree(b); cudaFree(bk); cudaFree(c); cudaFree(image.data);
+      cudaFree(a); cudaFree(b); cudaFree(bk); cudaFree(c); cudaFree(a_max); cudaFree(image.data);
       throw;
     }
-    cudaFree(a); cudaFree(b); cudaFree(bk); cudaFree(c); cudaFree(image.data);
+    cudaFree(a); cudaFree(b); cudaFree(bk); cudaFree(c); cudaFree(a_max); cudaFree(image.data);
     h->check_status();
   });
 }

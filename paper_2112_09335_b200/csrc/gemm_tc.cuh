@@ -203,76 +203,14 @@ struct WsCfg {
   static constexpr int kAccCols = kSets * 2 * NT;
   static constexpr uint32_t kTmemCols = kAccCols <= 64 ? 64 : kAccCols <= 128 ? 128 : kAccCols <= 256 ? 256 : 512;
   static constexpr size_t kSmem = (size_t)kStagesWs * kStage + kEpiWarps * 4096 + 1024;   // + the epilogue warps' buffers
-  // Tensor-copy form (NT <= 128): a ring of R slots {raw A tile (read in place as the hi operand), B_hi, B_lo},
-  // filled by copies alone and therefore a DRAM latency ahead of the MMAs, and a ring of S A_lo tiles that the
-  // producers fill from the raw tiles; a lo tile is held only from the producers' stores to the end of its MMAs.
-  static constexpr int kRawSlots = NT > 64 ? 3 : 5;
-  static constexpr int kLoStages = 3;
-  static constexpr int kRawSlot = kATileBytes + 2 * kBTile;
-  static constexpr size_t kSmemRing = (size_t)kRawSlots * kRawSlot + (size_t)kLoStages * kATileBytes + kEpiWarps * 4096 + 1024;
 };
 
-// The weight operand split once, in the layout the MMA descriptors read: for column group g and K
-// chunk kc, the 128-byte-swizzled NT x 32 tile of B_hi followed by that of B_lo, one contiguous block
-// of 2 * NT * 128 bytes at block index g * chunks + kc.  With it (IMG = true) a stage's B tiles arrive
-// by one bulk copy issued by one thread, and the producers stage A only; without it they load, split
-// and store B again for every 128-row tile.
-__global__ void k_split_b(const float* __restrict__ Bk, int ldbk, int N, int K, int nt, uint8_t* __restrict__ image) {
-  const int kc_count = (K + kChunkK - 1) / kChunkK;
-  const int groups = (N + nt - 1) / nt;
-  const long long total = (long long)groups * kc_count * nt * 8;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-    const int c16 = (int)(i & 7);
-    const int nrow = (int)((i >> 3) % nt);
-    const long long blk = i / (8LL * nt);
-    const int kc = (int)(blk % kc_count), g = (int)(blk / kc_count);
-    const int k0 = kc * kChunkK + c16 * 4, n = g * nt + nrow;
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (n < N && k0 < K) v = *reinterpret_cast<const float4*>(Bk + (long long)n * ldbk + k0);
-    float4 h, l;
-    split_tf32(v.x, h.x, l.x); split_tf32(v.y, h.y, l.y); split_tf32(v.z, h.z, l.z); split_tf32(v.w, h.w, l.w);
-    uint8_t* dst = image + (size_t)blk * (size_t)(2 * nt * kChunkK * 4) + swz(nrow, c16);
-    *reinterpret_cast<float4*>(dst) = h;
-    *reinterpret_cast<float4*>(dst + (size_t)nt * kChunkK * 4) = l;
-  }
-}
-
-// Such an image kept up to date by whoever writes the operand (the weights and their gradients: a launch of k_split_b and
-// its gap before every product otherwise, 4 us each).  nt: column group width, kc: K chunks; data = NULL: no image is kept.
-// The padding of the image is zero from the start and never written.
-struct Image {
-  uint8_t* data;
-  int nt, kc;
-};
-__device__ __forceinline__ void put_split(const Image& im, int n, int k, float x) {
-  if (im.data == nullptr) return;
-  const int g = n / im.nt, r = n - g * im.nt, c = k / kChunkK, kk = k - c * kChunkK;
-  uint8_t* const at = im.data + (size_t)(g * im.kc + c) * (size_t)(2 * im.nt * kChunkK * 4) + swz(r, kk >> 2) + (kk & 3) * 4;
-  float h, l;
-  split_tf32(x, h, l);
-  *reinterpret_cast<float*>(at) = h;
-  *reinterpret_cast<float*>(at + (size_t)im.nt * kChunkK * 4) = l;
-}
-
-// TMA = true (needs IMG): the A operand is not loaded by the producers at all.  One more warp (its lane 0)
-// fetches each 128 x 32 tile of A with a tensor copy (cp.async.bulk.tensor, 128-byte swizzle: the copy
-// engine writes exactly the K-major layout the MMA descriptors read) and the chunk's two weight tiles with
-// a bulk copy into slot j mod R of a ring that only copies fill, up to R chunks ahead of the MMAs.  The
-// tensor core reads a 32-bit operand as TF32 by dropping its 13 low mantissa bits, so the raw tile IS the
-// hi operand, hi = x with those bits cleared, and the producers only form lo = x - hi from the tile in
-// shared memory (exact) and store it into stage j mod S of a second ring: no global loads and half the
-// stores, and the A stream no longer passes through L1.  A slot is freed by the commit of its chunk's
-// MMAs (raw_empty), a lo stage likewise (empty).  Rows past M and columns past the matrix are filled with
-// zeros by the copy.
-template <int NT, bool IMG, bool TMA = false>
-__global__ void __launch_bounds__(WsCfg<NT>::kThreads + (TMA ? 32 : 0), 1)
+template <int NT>
+__global__ void __launch_bounds__(WsCfg<NT>::kThreads, 1)
 k_gemm_tc_ws(const float* __restrict__ A, int lda, const float* __restrict__ Bk, int ldbk, float* __restrict__ C, int ldc,
-             int M, int N, int K, const int* __restrict__ skip, int* __restrict__ error_flag,
-             const uint8_t* __restrict__ b_image, const __grid_constant__ CUtensorMap tmap_a, float* partial, unsigned* tickets) {
-  static_assert(!TMA || IMG, "the tensor-copy form stages no B tile");
+             int M, int N, int K, const int* __restrict__ skip, int* __restrict__ error_flag, float* partial, unsigned* tickets) {
   using Cfg = WsCfg<NT>;
-  constexpr int S = TMA ? Cfg::kLoStages : Cfg::kStagesWs;   // stages of the ring the producers fill
-  constexpr int R = TMA ? Cfg::kRawSlots : 1;                // slots of the ring the copies fill (tensor-copy form only)
+  constexpr int S = Cfg::kStagesWs;
   constexpr int B_PASSES = (NT + 31) / 32;
   constexpr int A_PASSES = kBlockM / 32;
   constexpr int SETS = Cfg::kSets;
@@ -280,27 +218,21 @@ k_gemm_tc_ws(const float* __restrict__ A, int lda, const float* __restrict__ Bk,
   if (skip != nullptr && *skip) return;
 
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t bars[2 * S + 5 + 2 * R];      // full[S], empty[S], acc_full[2], acc_empty[2], raw_full[R], raw_empty[R], drain
+  __shared__ __align__(8) uint64_t bars[2 * S + 5];      // full[S], empty[S], acc_full[2], acc_empty[2], drain
   __shared__ uint32_t tmem_base_slot;
-  __shared__ int abort_flag, last_part, copies;   // copies: chunks whose bulk copies have been started
+  __shared__ int abort_flag, last_part;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t smem_base = smem_u32(smem);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t bar_full = smem_u32(&bars[0]), bar_empty = smem_u32(&bars[S]);
   const uint32_t bar_acc_full = smem_u32(&bars[2 * S]), bar_acc_empty = smem_u32(&bars[2 * S + 2]);
-  const uint32_t bar_raw_full = smem_u32(&bars[2 * S + 4]), bar_raw_empty = smem_u32(&bars[2 * S + 4 + R]);
-  // shared-memory map of the tensor-copy form: R slots of {raw A, B_hi, B_lo}, then S tiles of A_lo
-  constexpr uint32_t kRawSlot = (uint32_t)Cfg::kRawSlot;
-  constexpr uint32_t kLoBase = (uint32_t)R * kRawSlot;
-  constexpr uint32_t kStageBytes = TMA ? (uint32_t)kATileBytes : (uint32_t)Cfg::kStage;
-  constexpr uint32_t kRingBytes = TMA ? kLoBase + (uint32_t)S * kStageBytes : (uint32_t)S * kStageBytes;
+  constexpr uint32_t kStageBytes = (uint32_t)Cfg::kStage, kRingBytes = (uint32_t)S * kStageBytes;
 
   if (tid == 0) {
     for (int s = 0; s < S; ++s) { mbar_init(bar_full + 8 * s, 8); mbar_init(bar_empty + 8 * s, 1); }   // full: one arrival per producer warp
-    for (int r = 0; r < R; ++r) { mbar_init(bar_raw_full + 8 * r, 1); mbar_init(bar_raw_empty + 8 * r, 1); }
     for (int a = 0; a < 2; ++a) { mbar_init(bar_acc_full + 8 * a, 1); mbar_init(bar_acc_empty + 8 * a, Cfg::kEpiWarps); }
-    mbar_init(bar_raw_empty + 8 * R, 1);
-    abort_flag = copies = 0;
+    mbar_init(bar_full + 8 * (2 * S + 4), 1);
+    abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == Cfg::kMmaWarp) {
@@ -328,10 +260,10 @@ k_gemm_tc_ws(const float* __restrict__ A, int lda, const float* __restrict__ Bk,
   if (warp < 8) {
     // ---------------- producers ----------------
     const int ld_c16 = tid & 7, ld_row = tid >> 3;
-    constexpr int DEPTH = IMG ? 4 : (NT > 128 ? 1 : 2);   // chunks a thread holds in registers ahead of the one it stores
-    float4 ra[DEPTH][A_PASSES], rb[DEPTH][IMG ? 1 : B_PASSES];
+    constexpr int DEPTH = NT > 128 ? 1 : 2;   // chunks a thread holds in registers ahead of the one it stores
+    float4 ra[DEPTH][A_PASSES], rb[DEPTH][B_PASSES];
     // chunks are loaded strictly in order, so tile and K chunk of the next load are counters (no division per chunk)
-    int ld_j = 0, ld_kc = 0, st_kc = 0;
+    int ld_j = 0, ld_kc = 0;
     long long ld_row0 = (long long)blockIdx.x * kBlockM;
     auto load_chunk = [&](float4* pa, float4* pb) {
       if (ld_j >= total) return;
@@ -348,16 +280,14 @@ k_gemm_tc_ws(const float* __restrict__ A, int lda, const float* __restrict__ Bk,
         }
         pa[i] = v;
       }
-      if (!IMG) {
 #pragma unroll
-        for (int i = 0; i < B_PASSES; ++i) {
-          const int nrow = ld_row + 32 * i;
-          float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (nrow < n_loc && k0 < K) {
-            v = *reinterpret_cast<const float4*>(Bk + (long long)(n0 + nrow) * ldbk + k0);
-          }
-          pb[i] = v;
+      for (int i = 0; i < B_PASSES; ++i) {
+        const int nrow = ld_row + 32 * i;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (nrow < n_loc && k0 < K) {
+          v = *reinterpret_cast<const float4*>(Bk + (long long)(n0 + nrow) * ldbk + k0);
         }
+        pb[i] = v;
       }
     };
     auto store_chunk = [&](int stage, const float4* pa, const float4* pb) {
@@ -371,47 +301,19 @@ k_gemm_tc_ws(const float* __restrict__ A, int lda, const float* __restrict__ Bk,
         *reinterpret_cast<float4*>(st + off) = h;
         *reinterpret_cast<float4*>(st + kATileBytes + off) = l;
       }
-      if (!IMG) {
 #pragma unroll
-        for (int i = 0; i < B_PASSES; ++i) {
-          const int nrow = ld_row + 32 * i;
-          if (nrow < NT) {
-            float4 h, l;
-            split_tf32(pb[i].x, h.x, l.x); split_tf32(pb[i].y, h.y, l.y);
-            split_tf32(pb[i].z, h.z, l.z); split_tf32(pb[i].w, h.w, l.w);
-            const uint32_t off = swz(nrow, ld_c16);
-            *reinterpret_cast<float4*>(st + 2 * kATileBytes + off) = h;
-            *reinterpret_cast<float4*>(st + 2 * kATileBytes + Cfg::kBTile + off) = l;
-          }
+      for (int i = 0; i < B_PASSES; ++i) {
+        const int nrow = ld_row + 32 * i;
+        if (nrow < NT) {
+          float4 h, l;
+          split_tf32(pb[i].x, h.x, l.x); split_tf32(pb[i].y, h.y, l.y);
+          split_tf32(pb[i].z, h.z, l.z); split_tf32(pb[i].w, h.w, l.w);
+          const uint32_t off = swz(nrow, ld_c16);
+          *reinterpret_cast<float4*>(st + 2 * kATileBytes + off) = h;
+          *reinterpret_cast<float4*>(st + 2 * kATileBytes + Cfg::kBTile + off) = l;
         }
       }
     };
-    if (TMA) {
-      // chunk j: raw tile and weight tiles in slot j mod R (see the copy warp below), lo in stage j mod S
-      int stage = 0, slot = 0;
-      uint32_t empty_parity = 1, raw_parity = 0;   // a fresh barrier passes a wait on parity 1
-      for (int j = 0; j < total; ++j) {
-        if (!__all_sync(0xffffffffu, mbar_wait_abortable(bar_empty + 8 * stage, empty_parity, abortp))) break;   // warp-uniform: the arrival below is per warp
-        if (!__all_sync(0xffffffffu, mbar_wait_abortable(bar_raw_full + 8 * slot, raw_parity, abortp))) break;
-        const uint8_t* raw = smem + (size_t)slot * kRawSlot;
-        uint8_t* st = smem + kLoBase + (size_t)stage * kStageBytes;
-#pragma unroll
-        for (int i = 0; i < A_PASSES; ++i) {
-          const uint32_t off = swz(ld_row + 32 * i, ld_c16);
-          const float4 x = *reinterpret_cast<const float4*>(raw + off);
-          float4 l;
-          l.x = x.x - __uint_as_float(__float_as_uint(x.x) & 0xffffe000u);
-          l.y = x.y - __uint_as_float(__float_as_uint(x.y) & 0xffffe000u);
-          l.z = x.z - __uint_as_float(__float_as_uint(x.z) & 0xffffe000u);
-          l.w = x.w - __uint_as_float(__float_as_uint(x.w) & 0xffffe000u);
-          *reinterpret_cast<float4*>(st + off) = l;
-        }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        mbar_arrive_warp(bar_full + 8 * stage);
-        if (++stage == S) { stage = 0; empty_parity ^= 1u; }
-        if (++slot == R) { slot = 0; raw_parity ^= 1u; }
-      }
-    } else {
 #pragma unroll
     for (int d = 0; d < DEPTH; ++d) load_chunk(ra[d], rb[d]);
     bool stop = false;
@@ -422,47 +324,10 @@ k_gemm_tc_ws(const float* __restrict__ A, int lda, const float* __restrict__ Bk,
         if (j >= total) break;
         const int stage = j % S;
         if (j >= S && !__all_sync(0xffffffffu, mbar_wait_abortable(bar_empty + 8 * stage, ((j / S) - 1) & 1, abortp))) { stop = true; break; }
-        if (IMG && tid == 0) {
-          // the stage is free (its MMAs have retired): fetch both B tiles of this chunk with one bulk copy
-          // that reports its bytes to the stage's full barrier; this thread's own arrival comes below
-          const uint32_t bytes = 2u * (uint32_t)Cfg::kBTile;
-          const uint8_t* src = b_image + ((size_t)blockIdx.y * kc_all + (size_t)(kc0 + st_kc)) * bytes;
-          const uint32_t dst = smem_base + (uint32_t)stage * Cfg::kStage + 2u * kATileBytes;
-          asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar_full + 8 * stage), "r"(bytes) : "memory");
-          asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                       ::"r"(dst), "l"(src), "r"(bytes), "r"(bar_full + 8 * stage)
-                       : "memory");
-          copies = j + 1;
-        }
-        if (++st_kc == kc_count) st_kc = 0;
         store_chunk(stage, ra[d], rb[d]);
         load_chunk(ra[d], rb[d]);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         mbar_arrive_warp(bar_full + 8 * stage);
-      }
-    }
-    }
-  } else if (TMA && warp == Cfg::kMmaWarp + 1) {
-    // ---------------- copies (tensor-copy form only): A tile and weight tiles of chunk j as soon as slot j mod R is free ----------------
-    if (lane == 0) {
-      const uint32_t b_bytes = 2u * (uint32_t)Cfg::kBTile;
-      const uint8_t* const b_src = b_image + ((size_t)blockIdx.y * kc_all + (size_t)kc0) * b_bytes;
-      int kc = 0, tile = blockIdx.x, slot = 0;
-      uint32_t empty_parity = 1;   // a fresh barrier passes a wait on parity 1
-      for (int j = 0; j < total; ++j) {
-        if (!mbar_wait_abortable(bar_raw_empty + 8 * slot, empty_parity, abortp)) break;
-        const uint32_t dst_a = smem_base + (uint32_t)slot * kRawSlot;
-        const uint32_t raw_bar = bar_raw_full + 8 * slot;
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(raw_bar), "r"((uint32_t)kATileBytes + b_bytes) : "memory");
-        asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-                     ::"r"(dst_a), "l"(&tmap_a), "r"((kc0 + kc) * kChunkK), "r"(tile * kBlockM), "r"(raw_bar)
-                     : "memory");
-        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                     ::"r"(dst_a + (uint32_t)kATileBytes), "l"(b_src + (size_t)kc * b_bytes), "r"(b_bytes), "r"(raw_bar)
-                     : "memory");
-        copies = j + 1;
-        if (++kc == kc_count) { kc = 0; tile += gridDim.x; }
-        if (++slot == R) { slot = 0; empty_parity ^= 1u; }
       }
     }
   } else if (warp == Cfg::kMmaWarp) {
@@ -471,7 +336,7 @@ k_gemm_tc_ws(const float* __restrict__ A, int lda, const float* __restrict__ Bk,
     // (no division by kc_count, no 64-bit descriptor arithmetic: counters that wrap, one addition per operand).
     if (lane == 0) {
       const uint32_t idesc = instr_desc(NT), idesc2 = instr_desc(NT <= 128 ? 2 * NT : NT);
-      int stage = 0, kc = 0, tile_i = 0, slot = 0;
+      int stage = 0, kc = 0, tile_i = 0;
       uint32_t full_parity = 0;
       for (int j = 0; j < total; ++j) {
         const int set = SETS == 1 ? 0 : (tile_i & 1);
@@ -479,9 +344,8 @@ k_gemm_tc_ws(const float* __restrict__ A, int lda, const float* __restrict__ Bk,
         if (!mbar_wait_abortable(bar_full + 8 * stage, full_parity, abortp)) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         // shared memory ends below 2^18, so additions to a descriptor's low word never carry out of the address field
-        const uint32_t a_hi = operand_desc_lo(TMA ? smem_base + slot * kRawSlot : smem_base + stage * kStageBytes);
-        const uint32_t a_lo = TMA ? operand_desc_lo(smem_base + kLoBase + stage * kStageBytes) : a_hi + (kATileBytes >> 4);
-        const uint32_t b_hi = TMA ? a_hi + (kATileBytes >> 4) : a_hi + (2 * kATileBytes >> 4), b_lo = b_hi + (Cfg::kBTile >> 4);
+        const uint32_t a_hi = operand_desc_lo(smem_base + stage * kStageBytes), a_lo = a_hi + (kATileBytes >> 4);
+        const uint32_t b_hi = a_hi + (2 * kATileBytes >> 4), b_lo = b_hi + (Cfg::kBTile >> 4);
         const uint32_t acc = tmem_base + (uint32_t)(set * 2 * NT);
 #pragma unroll
         for (int ks = 0; ks < kChunkK / 8; ++ks) {
@@ -501,10 +365,6 @@ k_gemm_tc_ws(const float* __restrict__ A, int lda, const float* __restrict__ Bk,
           }
         }
         mma_commit(bar_empty + 8 * stage);
-        if (TMA) {
-          mma_commit(bar_raw_empty + 8 * slot);
-          if (++slot == R) slot = 0;
-        }
         if (++kc == kc_count) {
           mma_commit(bar_acc_full + 8 * set);
           kc = 0;
@@ -595,11 +455,8 @@ k_gemm_tc_ws(const float* __restrict__ A, int lda, const float* __restrict__ Bk,
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (abort_flag) {
-    if (tid == 0) {
-      atomicOr(error_flag, 1);
-      if (IMG) drain_copies(TMA ? bar_raw_full : bar_full, TMA ? R : S, copies);
-    }
-    if (tid == Cfg::kMmaWarp * 32) drain_mmas(bar_raw_empty + 8 * R);
+    if (tid == 0) atomicOr(error_flag, 1);
+    if (tid == Cfg::kMmaWarp * 32) drain_mmas(bar_full + 8 * (2 * S + 4));
     __syncthreads();
   }
   if (warp == Cfg::kMmaWarp) {
@@ -654,11 +511,12 @@ struct TnCfg {
 // its pre-activation, formed while staging from the pre-activation H (passed as B) and the layer's
 // Z (Zres, same leading dimension):  b = h > 0 ? nu (h - z) : 0.  Both rows are fetched one chunk
 // ahead (A stays two chunks ahead), so the second matrix costs no further registers.
+// part_max (may be NULL): raised to the largest magnitude among the partial sums.
 template <int NT, bool RESID>
 __global__ void __launch_bounds__(kTnThreads, 1)
 k_gemm_tn_tc(const float* __restrict__ A, int lda, const float* __restrict__ B, int ldb, float* __restrict__ part, int ldp,
              long long rows, long long rows_per_split, int Ka, int Nb, int* __restrict__ error_flag,
-             const float* __restrict__ Zres, float nu) {
+             const float* __restrict__ Zres, float nu, unsigned* part_max) {
   using Cfg = TnCfg<NT>;
   constexpr int S = Cfg::kStagesTn;
   constexpr int A_PASSES = 4;                              // 1024 float4 / 256 threads
@@ -819,6 +677,7 @@ k_gemm_tn_tc(const float* __restrict__ A, int lda, const float* __restrict__ B, 
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const int ka = ka0 + warp * 32 + lane;
     float* dst = part + ((long long)blockIdx.y * Ka + ka) * ldp;
+    float big = 0.f;
 #pragma unroll 1
     for (int cchunk = 0; cchunk < NT / 16; ++cchunk) {
       uint32_t v[16], w[16];
@@ -834,14 +693,18 @@ k_gemm_tn_tc(const float* __restrict__ A, int lda, const float* __restrict__ B, 
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const int col = nb0 + cchunk * 16 + q * 4;
-          if (col < ldp)
-            *reinterpret_cast<float4*>(dst + col) =
-                make_float4(__uint_as_float(v[q * 4]) + __uint_as_float(w[q * 4]),
-                            __uint_as_float(v[q * 4 + 1]) + __uint_as_float(w[q * 4 + 1]),
-                            __uint_as_float(v[q * 4 + 2]) + __uint_as_float(w[q * 4 + 2]),
-                            __uint_as_float(v[q * 4 + 3]) + __uint_as_float(w[q * 4 + 3]));
+          const float4 sum = make_float4(__uint_as_float(v[q * 4]) + __uint_as_float(w[q * 4]),
+                                         __uint_as_float(v[q * 4 + 1]) + __uint_as_float(w[q * 4 + 1]),
+                                         __uint_as_float(v[q * 4 + 2]) + __uint_as_float(w[q * 4 + 2]),
+                                         __uint_as_float(v[q * 4 + 3]) + __uint_as_float(w[q * 4 + 3]));
+          big = fmaxf(fmaxf(big, fmaxf(fabsf(sum.x), fabsf(sum.y))), fmaxf(fabsf(sum.z), fabsf(sum.w)));
+          if (col < ldp) *reinterpret_cast<float4*>(dst + col) = sum;
         }
       }
+    }
+    if (part_max != nullptr) {   // magnitudes: their order is that of their bits
+      const unsigned most = __reduce_max_sync(0xffffffffu, __float_as_uint(big));
+      if (lane == 0) atomicMax(part_max, most);
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");

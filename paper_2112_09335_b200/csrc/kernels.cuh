@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "gemm_half.cuh"
 #include "gemm_tc.cuh"
 
 namespace gk {
@@ -27,6 +28,10 @@ struct SearchCtl {
   int trial;       // accepted trial index, -1 skipped, -2 exhausted
   int pass;        // passes already scored
   float inv_cand[kCand];  // 1/t of the candidates of the current pass
+  // W blocks, for the scales of the split images: largest magnitude of the gradient and of W (k_finish_grad); of the gradient's
+  // partial sums, as bits (raised by the transposed product, left at zero by k_finish_grad)
+  float g_max, w_max;
+  unsigned part_max;
 };
 
 // Numbers and flags the host reads back together.
@@ -118,6 +123,7 @@ __device__ __forceinline__ void add_block_sums(const double* partial, int count,
 // MAPPED: x and out are dense matrices in the caller's row order; node c's row is perm[c] (a 4-byte load in
 // parallel with that of its weight), so that no copy of the operand in community order and none back is made.
 // RELU: out = A~ max(x, 0), so that a forward pass needs no sweep for its activations.
+// row_max (may be NULL): the largest magnitude of every row of `out`, which a product of `out` by split halves scales the row by.
 // Values are moved in vectors of VEC floats: four wherever rows start on 16-byte boundaries (always inside the
 // library), fewer for a caller's matrix of odd width.
 // ------------------------------------------------------------------------------------------
@@ -145,6 +151,9 @@ __device__ __forceinline__ float4 vxor(unsigned m, float4 a, int o) {
 __device__ __forceinline__ float vrelu(float a) { return relu(a); }
 __device__ __forceinline__ float2 vrelu(float2 a) { return make_float2(relu(a.x), relu(a.y)); }
 __device__ __forceinline__ float4 vrelu(float4 a) { return make_float4(relu(a.x), relu(a.y), relu(a.z), relu(a.w)); }
+__device__ __forceinline__ float vabsmax(float a) { return fabsf(a); }
+__device__ __forceinline__ float vabsmax(float2 a) { return fmaxf(fabsf(a.x), fabsf(a.y)); }
+__device__ __forceinline__ float vabsmax(float4 a) { return fmaxf(fmaxf(fabsf(a.x), fabsf(a.y)), fmaxf(fabsf(a.z), fabsf(a.w))); }
 __device__ __forceinline__ void vzero(float& a) { a = 0.f; }
 __device__ __forceinline__ void vzero(float2& a) { a = make_float2(0.f, 0.f); }
 __device__ __forceinline__ void vzero(float4& a) { a = make_float4(0.f, 0.f, 0.f, 0.f); }
@@ -160,7 +169,7 @@ struct ItemRows {
 // Called by the G lanes (mask `gmask`, lane `gl`) that have just written item `unit`'s sums to scratch.
 template <typename T, int G>
 __device__ __forceinline__ void finish_item(const ItemRows& ir, int unit, T* __restrict__ row_out, const T* scratch, int ldv,
-                                            unsigned gmask, int gl) {
+                                            unsigned gmask, int gl, float* row_max) {
   const int lr = ir.item_row[unit];
   const int4 whole = ir.rows[lr];
   __threadfence();
@@ -170,12 +179,19 @@ __device__ __forceinline__ void finish_item(const ItemRows& ir, int unit, T* __r
   done = __shfl_sync(gmask, done, 0, G);
   if (done + 1 < whole.z) return;
   __threadfence();
+  float m = 0.f;
   for (int f = gl; f < ldv; f += G) {
     T s;
     vzero(s);
 #pragma unroll 4
     for (int k = 0; k < whole.z; ++k) s = vadd(s, __ldcg(scratch + (long long)(whole.y + k) * ldv + f));
     row_out[f] = s;
+    m = fmaxf(m, vabsmax(s));
+  }
+  if (row_max != nullptr) {
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(gmask, m, o));
+    if (gl == 0) row_max[whole.x] = m;
   }
   if (gl == 0) ir.done[lr] = 0;
 }
@@ -184,15 +200,17 @@ __device__ __forceinline__ void finish_item(const ItemRows& ir, int unit, T* __r
 // (blockIdx.y and, past the limit of that, .z): more warps, and one slice of the operand at a time is what L2 has to hold
 // (1000 columns on 14 k rows 195 -> 142 us).  Lane t of a group of 32
 // stored entries holds column and weight of entry t, handed to the warp by shuffles.  UN neighbours in flight per
-// lane: the kernel is bound by the L2-to-SM traffic of the gathered rows, and by how the compiler orders its loads (the plain
-// loop measured faster than one that fetches columns ahead: 138 against 160 us at 128 columns on 169 k rows).  At the 40
-// registers of 24 blocks per SM the form of 256 columns spills 8 bytes, the sliced one 32.
+// lane: the kernel is bound by what L1 and L2 deliver of the gathered rows (about a third of the bytes are L1 hits on the hub rows of
+// a community: with loads that do not allocate in L1 10.4 instead of 6.8 ms, 2.45 M rows at 256 columns) and by how the compiler
+// orders its loads (the plain loop is faster than one that fetches columns ahead: 118 against 143 us at 128 columns on 169 k rows).
+// The bound of 21 blocks gives the 40 registers of 24 and an order of loads that the row maxima at the end do not disturb: 6.81 ms with
+// them, 6.75 without; under a bound of 24 blocks 8.78.  With ReLU on the gathered rows it is a bound of 20 (9.0 against 9.4 ms).
 template <int VEC, int NV, int UN, bool MAPPED, bool SLICED, bool RELU>
-__global__ void __launch_bounds__(64, VEC == 4 ? 24 : 16)
+__global__ void __launch_bounds__(64, VEC == 4 ? (RELU ? 20 : 21) : 16)
 k_spmm_wide(const int* __restrict__ row_ptr, const int* __restrict__ col, const float* __restrict__ dinv,
             const int* __restrict__ perm, const int4* __restrict__ items, int n, int n_items, int long_len,
             const typename Vec<VEC>::T* __restrict__ x, typename Vec<VEC>::T* __restrict__ out, int ldv,
-            typename Vec<VEC>::T* __restrict__ scratch) {
+            typename Vec<VEC>::T* __restrict__ scratch, float* __restrict__ row_max) {
   using T = typename Vec<VEC>::T;
   const int lane = threadIdx.x & 31;
   const int off = SLICED ? (blockIdx.y + gridDim.y * blockIdx.z) * (32 * NV) : 0;
@@ -214,6 +232,13 @@ k_spmm_wide(const int* __restrict__ row_ptr, const int* __restrict__ col, const 
     dst = out + (long long)(MAPPED ? perm[row] : row) * ldv;
   }
   const float di = dinv[row];
+  // The unit once more, behind the compiler's back: kept from above it is a register too many during the walk.
+  const auto again = [] {
+    unsigned block, thread;
+    asm volatile("mov.u32 %0, %%ctaid.x;" : "=r"(block));
+    asm volatile("mov.u32 %0, %%tid.x;" : "=r"(thread));
+    return (int)((block * 64ull + thread) >> 5);
+  };
   // One turn only, but the compiler is not to know: it then issues all loads of a step before the first sum (+20 % at 256 columns).
   for (int cb = 0; cb < wv; cb += 32 * NV) {
     T acc[NV];
@@ -254,24 +279,42 @@ k_spmm_wide(const int* __restrict__ row_ptr, const int* __restrict__ col, const 
       const int f = cb + lane + 32 * v;
       if (f < wv) dst[f] = vscale(di, acc[v]);
     }
+    if (!MAPPED && !SLICED && row_max != nullptr) {
+      float m = 0.f;
+#pragma unroll
+      for (int v = 0; v < NV; ++v)
+        if (cb + lane + 32 * v < wv) m = fmaxf(m, vabsmax(acc[v]));
+      m = di * __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m)));
+      const int own = again() - n_items;
+      if (lane == 0 && own >= 0) row_max[own] = m;
+    }
   }
 }
 
 // Rows that k_spmm_wide handled as items (a kernel of its own: with finish_item at its end k_spmm_wide takes more
 // registers and was 4 % slower): out[row] = sum of the row's item sums, in item order, one block per row.
 template <typename T, bool MAPPED>
-__global__ void k_spmm_long_rows(const int4* __restrict__ rows, const T* __restrict__ scratch, T* __restrict__ out, int ldv,
-                                 const int* __restrict__ perm) {
+__global__ void __launch_bounds__(64)
+k_spmm_long_rows(const int4* __restrict__ rows, const T* __restrict__ scratch, T* __restrict__ out, int ldv,
+                                 const int* __restrict__ perm, float* __restrict__ row_max) {
   gtc::enter_kernel();
   const int4 r = rows[blockIdx.x];
   const long long row = MAPPED ? perm[r.x] : r.x;
+  float m = 0.f;
   for (int f = threadIdx.x; f < ldv; f += blockDim.x) {
     T s;
     vzero(s);
 #pragma unroll 4
     for (int k = 0; k < r.z; ++k) s = vadd(s, scratch[(long long)(r.y + k) * ldv + f]);
     out[row * ldv + f] = s;
+    m = fmaxf(m, vabsmax(s));
   }
+  if (MAPPED || row_max == nullptr) return;
+  __shared__ float s_max;
+  m = warp_max(m);
+  if (threadIdx.x == 32) s_max = m;
+  __syncthreads();
+  if (threadIdx.x == 0) row_max[row] = fmaxf(m, s_max);
 }
 
 // Narrow operands.  G = CL * EP lanes share a row: CL of them side by side over its columns (NV vectors each), EP
@@ -288,7 +331,7 @@ __global__ void __launch_bounds__(128, CL >= 8 && VEC == 4 ? 10 : 8)
 k_spmm_sets(const int* __restrict__ row_ptr, const int* __restrict__ col, const float* __restrict__ dinv,
             const int* __restrict__ perm, const int4* __restrict__ items, int n, int n_items, int long_len,
             const typename Vec<VEC>::T* __restrict__ x, typename Vec<VEC>::T* __restrict__ out, int ldv,
-            typename Vec<VEC>::T* __restrict__ scratch, const int* __restrict__ row_order, const ItemRows ir) {
+            typename Vec<VEC>::T* __restrict__ scratch, const int* __restrict__ row_order, const ItemRows ir, float* __restrict__ row_max) {
   gtc::enter_kernel();
   using T = typename Vec<VEC>::T;
   constexpr int G = CL * EP;
@@ -312,6 +355,7 @@ k_spmm_sets(const int* __restrict__ row_ptr, const int* __restrict__ col, const 
   const float di = dinv[row];
   T* const row_out = out + (long long)(MAPPED ? perm[row] : row) * ldv;
   T* const dst = item ? scratch + (long long)unit * ldv : row_out;
+  float m = 0.f;
   for (int cb = 0; cb < ldv; cb += CL * NV) {
     T acc[NV];
 #pragma unroll
@@ -388,11 +432,21 @@ k_spmm_sets(const int* __restrict__ row_ptr, const int* __restrict__ col, const 
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         const int f = cb + cl + CL * v;
-        if (f < ldv) dst[f] = vscale(di, acc[v]);
+        if (f < ldv) {
+          const T s = vscale(di, acc[v]);
+          dst[f] = s;
+          m = fmaxf(m, vabsmax(s));
+        }
       }
     }
   }
-  if (item) finish_item<T, G>(ir, unit, row_out, scratch, ldv, gmask, gl);
+  if (item) {
+    finish_item<T, G>(ir, unit, row_out, scratch, ldv, gmask, gl, MAPPED ? nullptr : row_max);
+  } else if (!MAPPED && row_max != nullptr) {
+#pragma unroll
+    for (int o = CL / 2; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(gmask, m, o));
+    if (gl == 0) row_max[row] = m;
+  }
 }
 
 // ------------------------------------------------------------------------------------------
@@ -880,14 +934,14 @@ __device__ __forceinline__ void log_decision(const DecisionLog& lg, int i, const
   lg.q[at] = c->q;
 }
 
-// Weight matrices are written in two orders at once (themselves and their transpose, an image for either): in tiles of 32 x
+// Weight matrices are written in two orders at once (themselves and their transpose, a split image for either): in tiles of 32 x
 // 32 that turn through shared memory, because a column of single floats costs a memory sector per element.
 // `value(r, c)` is called once per element of the tile, padding columns included, and gives its new value; t may be NULL.
 // Blocks of 256 threads, all of them.
 using WeightTile = float[32][33];
 template <typename F>
 __device__ __forceinline__ void weight_tile(int tile, int rows, int cols, int padded, WeightTile& turn, float* __restrict__ t, int ldt,
-                                            const gtc::Image& image, const gtc::Image& image_t, F&& value) {
+                                            const gtc::Image& image, float scale, const gtc::Image& image_t, float scale_t, F&& value) {
   const int x = threadIdx.x & 31, y = threadIdx.x >> 5, col_tiles = (padded + 31) / 32;
   const int r0 = tile / col_tiles * 32, c0 = tile % col_tiles * 32;
   __syncthreads();   // the tile before this one has been read
@@ -897,7 +951,7 @@ __device__ __forceinline__ void weight_tile(int tile, int rows, int cols, int pa
     if (r < rows && c < padded) {
       const float v = value(r, c);
       turn[y + k][x] = v;
-      if (c < cols) gtc::put_split(image_t, r, c, v);
+      if (c < cols) gtc::put_half(image_t, r, c, v * scale_t);
     }
   }
   __syncthreads();
@@ -907,15 +961,17 @@ __device__ __forceinline__ void weight_tile(int tile, int rows, int cols, int pa
     if (r < rows && c < cols) {
       const float v = turn[x][y + k];
       if (t != nullptr) t[(long long)c * ldt + r] = v;
-      gtc::put_split(image, c, r, v);
+      gtc::put_half(image, c, r, v * scale);
     }
   }
 }
 
 // Weight gradient from its split partial sums, and the start of the W_l search, in one launch:
-//   grad[e] = sum over splits of part[s][e] (fp64, in split order), its transpose and its image for P grad, ||grad||^2, ||W||^2.
+//   grad[e] = sum over splits of part[s][e] (fp64, in split order), its transpose for P grad, ||grad||^2, ||W||^2, and where one is
+//   kept the transpose's image, scaled by the bound splits * (largest partial sum): the split holds an element to 2^-23 of its
+//   magnitude down to 2^-29 of the bound, which is at most `splits` times too large where all partial sums are alike.
 // SG = 1: a block owns a tile of 32 x 32 elements (grid: tiles over rows x ldp).  SG = 8 (many splits): 32 consecutive elements,
-// eight threads per element, each adding its own run of consecutive splits; the transpose and the image are then written one
+// eight threads per element, each adding its own run of consecutive splits; the transpose is then written one
 // float at a time (a tile of 32 x 32 would leave one block where there are 32 now).  The last block to finish adds the
 // blocks' sums of squares up in block order and starts the search.  W = NULL: only the sum over the splits.
 template <int SG>
@@ -929,6 +985,10 @@ k_finish_grad(const float* __restrict__ part, int splits, int rows, int cols, in
   __shared__ int s_last;
   const long long elems = (long long)rows * ldp;
   double sq[2] = {0.0, 0.0};   // of grad, of W
+  float most[2] = {0.f, 0.f};
+  const float bound = W != nullptr && image.data != nullptr ? (float)splits * __uint_as_float(__ldcg(&ctl->part_max)) : 0.f;
+  const float scale = gtc::scale_of(bound);
+  if (W != nullptr && blockIdx.x == 0) gtc::put_scales(image, cols, bound);
   const auto sum_splits = [&](long long e, int k0, int k1) {
     double s = 0.0;
 #pragma unroll 8
@@ -936,11 +996,15 @@ k_finish_grad(const float* __restrict__ part, int splits, int rows, int cols, in
     return s;
   };
   if (SG == 1) {
-    weight_tile((int)blockIdx.x, rows, cols, ldp, turn, W != nullptr ? grad_t : nullptr, ldt, image, gtc::Image{nullptr, 16, 1}, [&](int r, int c) {
+    weight_tile((int)blockIdx.x, rows, cols, ldp, turn, W != nullptr ? grad_t : nullptr, ldt, image, scale, gtc::Image{nullptr, 16, 1}, 1.f, [&](int r, int c) {
       const long long e = (long long)r * ldp + c;
       const float g = (float)sum_splits(e, 0, splits);
       grad[e] = g;
-      if (W != nullptr) { const double w = W[e]; sq[0] += (double)g * (double)g; sq[1] += w * w; }
+      if (W != nullptr) {
+        const float w = W[e];
+        sq[0] += (double)g * (double)g; sq[1] += (double)w * (double)w;
+        most[0] = fmaxf(most[0], fabsf(g)); most[1] = fmaxf(most[1], fabsf(w));
+      }
       return g;
     });
   } else {
@@ -960,18 +1024,33 @@ k_finish_grad(const float* __restrict__ part, int splits, int rows, int cols, in
         const int r = (int)(e / ldp), c = (int)(e - (long long)r * ldp);
         if (c < cols) {
           grad_t[(long long)c * ldt + r] = g;
-          gtc::put_split(image, c, r, g);
+          gtc::put_half(image, c, r, g * scale);
         }
         sq[0] = (double)g * (double)g;
         sq[1] = (double)w * (double)w;
+        most[0] = fabsf(g);
+        most[1] = fabsf(w);
       }
     }
   }
   if (W == nullptr) return;
+  __shared__ unsigned s_most[2];   // magnitudes: their order is that of their bits
+  const auto block_most = [&] {
+    if (threadIdx.x < 2) s_most[threadIdx.x] = 0u;
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(most[j]));
+      if ((threadIdx.x & 31) == 0) atomicMax(&s_most[j], m);
+    }
+    __syncthreads();
+  };
   block_sums(sq, sh);
+  block_most();
   if (threadIdx.x == 0) {
-    partial[2 * (size_t)blockIdx.x] = sq[0];
-    partial[2 * (size_t)blockIdx.x + 1] = sq[1];
+    partial[3 * (size_t)blockIdx.x] = sq[0];
+    partial[3 * (size_t)blockIdx.x + 1] = sq[1];
+    reinterpret_cast<uint2*>(partial)[3 * (size_t)blockIdx.x + 2] = make_uint2(s_most[0], s_most[1]);
     __threadfence();
     s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
   }
@@ -979,13 +1058,21 @@ k_finish_grad(const float* __restrict__ part, int splits, int rows, int cols, in
   if (!s_last) return;
   __threadfence();
   sq[0] = sq[1] = 0.0;
+  most[0] = most[1] = 0.f;
   for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x) {
-    sq[0] += __ldcg(partial + 2 * (size_t)b);
-    sq[1] += __ldcg(partial + 2 * (size_t)b + 1);
+    sq[0] += __ldcg(partial + 3 * (size_t)b);
+    sq[1] += __ldcg(partial + 3 * (size_t)b + 1);
+    const uint2 m = __ldcg(reinterpret_cast<const uint2*>(partial) + 3 * (size_t)b + 2);
+    most[0] = fmaxf(most[0], __uint_as_float(m.x));
+    most[1] = fmaxf(most[1], __uint_as_float(m.y));
   }
   block_sums(sq, sh);
+  block_most();
   if (threadIdx.x == 0) {
     *ticket = 0;
+    ctl->g_max = __uint_as_float(s_most[0]);
+    ctl->w_max = __uint_as_float(s_most[1]);
+    ctl->part_max = 0u;   // every block has read it
     begin_one(ctl, sq[0], sq[1], shrink, growth, nullptr, status);
   }
 }
@@ -1023,8 +1110,13 @@ __device__ __forceinline__ void move_w(const SearchW& p, float step) {
   if (step != 0.f) {
     __shared__ WeightTile turn;
     const int tiles = ((p.rows + 31) / 32) * ((p.cols + 31) / 32);
+    const float bound = fmaf(step, __ldcg(&p.ctl->g_max), __ldcg(&p.ctl->w_max)), scale = gtc::scale_of(bound);   // |W - step grad| elementwise
+    if (blockIdx.x == 0) {
+      gtc::put_scales(p.image, p.cols, bound);
+      gtc::put_scales(p.image_t, p.rows, bound);
+    }
     for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x)
-      weight_tile(tile, p.rows, p.cols, p.cols, turn, p.Wt, p.ldwt, p.image, p.image_t, [&](int r, int c) {
+      weight_tile(tile, p.rows, p.cols, p.cols, turn, p.Wt, p.ldwt, p.image, scale, p.image_t, scale, [&](int r, int c) {
         const long long e = (long long)r * p.ldw + c;
         const float w = fmaf(-p.grad[e], step, p.W[e]);
         p.W[e] = w;
@@ -1159,27 +1251,41 @@ __global__ void k_log_clear(int* __restrict__ trial_base, const int* __restrict_
 // community, { ||G||^2, ||Z_l||^2, <Z_l - f(H_l), G> }.  blocks[b] = {first row, one past the last, community, 0}: a
 // block never crosses a community boundary and leaves the sums of its rows in partial[b*3 + ..]; the last block of a
 // community to finish (tickets[m], left at zero) adds the community's blocks block_ptr[m] .. block_ptr[m+1]-1 up in a
-// fixed order and starts its search.
+// fixed order and starts its search.  A group of LPR lanes takes a row; row_max (may be NULL): the largest magnitude of every row of G.
 // ------------------------------------------------------------------------------------------
+template <int LPR>
 __global__ void __launch_bounds__(256)
 k_zgrad_finish(float4* __restrict__ G, const float4* __restrict__ Z, const float4* __restrict__ H, int ld4,
                const int4* __restrict__ blocks, float nu, double* partial, const int* __restrict__ block_ptr, unsigned* tickets,
-               SearchCtl* ctl, double* __restrict__ sums, double shrink, double growth, int* n_active, int* status) {
+               SearchCtl* ctl, double* __restrict__ sums, double shrink, double growth, int* n_active, int* status, float* __restrict__ row_max) {
   gtc::enter_kernel();
   __shared__ double sh[24];
   __shared__ int s_last;
   const int4 rb = blocks[blockIdx.x];
   double t[3] = {0.0, 0.0, 0.0};
-  const long long e0 = (long long)rb.x * ld4, e1 = (long long)rb.y * ld4;
-  for (long long e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
-    const float4 z = Z[e], h = H[e];
-    float4 g = G[e];
-    const float ax = z.x - relu(h.x), ay = z.y - relu(h.y), az = z.z - relu(h.z), aw = z.w - relu(h.w);
-    g.x = fmaf(nu, ax, g.x); g.y = fmaf(nu, ay, g.y); g.z = fmaf(nu, az, g.z); g.w = fmaf(nu, aw, g.w);
-    G[e] = g;
-    t[0] += (double)(g.x * g.x + g.y * g.y + g.z * g.z + g.w * g.w);
-    t[1] += (double)(z.x * z.x + z.y * z.y + z.z * z.z + z.w * z.w);
-    t[2] += (double)(ax * g.x + ay * g.y + az * g.z + aw * g.w);
+  const int sub = threadIdx.x & (LPR - 1);
+  for (int row = rb.x + (int)(threadIdx.x / LPR); __any_sync(0xffffffffu, row < rb.y); row += 256 / LPR) {
+    const long long at = (long long)row * ld4;
+    float big = 0.f;
+    if (row < rb.y) {
+#pragma unroll 2
+      for (int f = sub; f < ld4; f += LPR) {
+        const float4 z = Z[at + f], h = H[at + f];
+        float4 g = G[at + f];
+        const float ax = z.x - relu(h.x), ay = z.y - relu(h.y), az = z.z - relu(h.z), aw = z.w - relu(h.w);
+        g.x = fmaf(nu, ax, g.x); g.y = fmaf(nu, ay, g.y); g.z = fmaf(nu, az, g.z); g.w = fmaf(nu, aw, g.w);
+        G[at + f] = g;
+        big = fmaxf(big, vabsmax(g));
+        t[0] += (double)(g.x * g.x + g.y * g.y + g.z * g.z + g.w * g.w);
+        t[1] += (double)(z.x * z.x + z.y * z.y + z.z * z.z + z.w * z.w);
+        t[2] += (double)(ax * g.x + ay * g.y + az * g.z + aw * g.w);
+      }
+    }
+    if (row_max != nullptr) {
+#pragma unroll
+      for (int o = LPR / 2; o > 0; o >>= 1) big = fmaxf(big, __shfl_xor_sync(0xffffffffu, big, o));
+      if (sub == 0 && row < rb.y) row_max[row] = big;
+    }
   }
   block_sums(t, sh);
   const int m = rb.z, b0 = block_ptr[m], b1 = block_ptr[m + 1];
@@ -2126,13 +2232,34 @@ k_row_loss_argmax(const float* __restrict__ Zrows, const float* __restrict__ log
   }
 }
 
-// Y = relu(X).
-__global__ void k_relu(const float4* __restrict__ X, float4* __restrict__ Y, long long n4) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n4;
-       i += (long long)gridDim.x * blockDim.x) {
-    float4 y = X[i];
-    y.x = relu(y.x); y.y = relu(y.y); y.z = relu(y.z); y.w = relu(y.w);
-    Y[i] = y;
+// Y = relu(X) for n rows of ld4 float4, a warp per row.  row_max (may be NULL): the largest element of every row of Y.
+__global__ void __launch_bounds__(256)
+k_relu(const float4* __restrict__ X, float4* __restrict__ Y, int ld4, long long n, float* __restrict__ row_max) {
+  const int lane = threadIdx.x & 31;
+  for (long long row = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; row < n; row += ((long long)gridDim.x * blockDim.x) >> 5) {
+    float m = 0.f;
+#pragma unroll 2
+    for (int f = lane; f < ld4; f += 32) {
+      const float4 y = vrelu(X[row * ld4 + f]);
+      Y[row * ld4 + f] = y;
+      m = fmaxf(m, vabsmax(y));
+    }
+    if (row_max == nullptr) continue;
+    m = warp_max(m);
+    if (lane == 0) row_max[row] = m;
+  }
+}
+
+// out[row] = the largest magnitude of the row, a warp per row of ld4 float4.
+__global__ void __launch_bounds__(256)
+k_row_max(const float4* __restrict__ X, int ld4, long long n, float* __restrict__ out) {
+  const int lane = threadIdx.x & 31;
+  for (long long row = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; row < n; row += ((long long)gridDim.x * blockDim.x) >> 5) {
+    float m = 0.f;
+#pragma unroll 4
+    for (int f = lane; f < ld4; f += 32) m = fmaxf(m, vabsmax(X[row * ld4 + f]));
+    m = warp_max(m);
+    if (lane == 0) out[row] = m;
   }
 }
 
@@ -2159,17 +2286,23 @@ __global__ void k_transpose_small(const float* __restrict__ src, int lds, float*
   dst[c * ldd + r] = src[r * lds + c];
 }
 
-// W (rows x cols, leading dimension ldw), its transpose and its images from a dense matrix; padding columns become zero.
+// W (rows x cols, leading dimension ldw), its transpose and its images from a dense matrix whose largest magnitude is `bound`; padding
+// columns become zero.
 __global__ void k_load_weight(const float* __restrict__ src, int rows, int cols, float* __restrict__ W, int ldw,
-                              float* __restrict__ Wt, int ldwt, const gtc::Image image, const gtc::Image image_t) {
+                              float* __restrict__ Wt, int ldwt, const gtc::Image image, const gtc::Image image_t, float bound) {
+  const float scale = gtc::scale_of(bound);
+  if (blockIdx.x == 0) {
+    gtc::put_scales(image, cols, bound);
+    gtc::put_scales(image_t, rows, bound);
+  }
   const long long first = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
   for (long long i = first; i < (long long)rows * ldw; i += stride) {
     const long long r = i / ldw, c = i - r * ldw;
     const float w = c < cols ? src[r * cols + c] : 0.f;
     W[i] = w;
     if (c < cols) {
-      gtc::put_split(image, (int)c, (int)r, w);
-      gtc::put_split(image_t, (int)r, (int)c, w);
+      gtc::put_half(image, (int)c, (int)r, w * scale);
+      gtc::put_half(image_t, (int)r, (int)c, w * scale);
     }
   }
   for (long long i = first; i < (long long)cols * ldwt; i += stride) {

@@ -1,0 +1,87 @@
+"""The product by split halves (rows of A scaled to a common exponent, columns of B likewise, each element a pair of fp16 numbers)
+at the edges of its tiles, column groups and K chunks, over the fp32 range, and on values no scale can hold."""
+import pytest
+
+from paper_2112_09335_b200 import binding, inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def handle():
+    wl = inputs.make_workload(0)
+    g = binding.GcnAdmm(wl.n, wl.row_ptr, wl.col_idx, wl.X, wl.y, wl.train_mask, wl.widths, wl.n_comm, wl.community, wl.w_init)
+    yield g
+    g.destroy()
+
+
+def product(g, a, b, tensor_cores=1):
+    import torch
+    c = torch.full((a.shape[0], b.shape[1]), float("nan"), device="cuda")
+    torch.cuda.synchronize()
+    g.dense_product(a.data_ptr(), b.data_ptr(), c.data_ptr(), a.shape[0], b.shape[1], a.shape[1], tensor_cores)
+    return c
+
+
+def bound(k):
+    """Relative to sum |a||b|: both operands to 2^-23, the dropped product of the low parts 2^-24, and an accumulator that is rounded
+    toward zero (2^-23) at each of ceil(k / 16) matrix instructions and once at the end."""
+    return (2.5 + -(-k // 16) + 1) * 2.0 ** -23
+
+
+@pytest.mark.parametrize("m", [16384, 16385, 19071])                                   # whole tiles, one row more, a tile less one row
+@pytest.mark.parametrize("n,k", [(1, 32), (16, 33), (17, 63), (33, 64), (49, 65), (65, 96), (97, 40), (129, 47), (193, 128), (257, 100), (8, 2048)])
+def test_edges(handle, m, n, k):
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(m + n + k)
+    a = torch.randn(m, k, generator=gen, device="cuda")
+    b = torch.randn(k, n, generator=gen, device="cuda")
+    got = product(handle, a, b).double()
+    want, size = a.double() @ b.double(), a.double().abs() @ b.double().abs()
+    assert float(((got - want).abs() / size).max()) < bound(k)
+
+
+def test_scales(handle):
+    """Rows between 2^-60 and 2^60, columns between 2^-50 and 2^50, some of either zero: the error is relative to each element's own terms."""
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    m, n, k = 16500, 130, 100
+    a = torch.randn(m, k, generator=gen, device="cuda") * torch.exp2(torch.randint(-60, 61, (m, 1), generator=gen, device="cuda").float())
+    b = torch.randn(k, n, generator=gen, device="cuda") * torch.exp2(torch.randint(-50, 51, (1, n), generator=gen, device="cuda").float())
+    a[::97] = 0
+    b[:, ::13] = 0
+    got = product(handle, a, b).double()
+    want, size = a.double() @ b.double(), a.double().abs() @ b.double().abs()
+    assert bool((got[size == 0] == 0).all())
+    assert float(((got - want).abs() / size)[size > 0].max()) < bound(k)
+
+
+@pytest.mark.parametrize("spread", [20, 28])
+def test_elements_far_below_the_largest_of_their_row(handle, spread):
+    """A row and a column whose largest elements meet zeros: what is left is `spread` bits below them and still held to 2^-23 of itself."""
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(spread)
+    m, n, k = 16400, 48, 64
+    a = torch.randn(m, k, generator=gen, device="cuda").clamp(-2, 2)
+    b = torch.randn(k, n, generator=gen, device="cuda")
+    a[:, 0], b[0] = 2.0 ** (spread + 1), 0.0
+    got = product(handle, a, b).double()
+    want, size = a.double() @ b.double(), a.double().abs() @ b.double().abs()
+    # elements of A reach far below the normal ones drawn here: 2^-51 of the row's largest is what a pair can hold of them
+    floor = 2.0 ** (spread + 1 - 51) * b.double().abs().sum(0)
+    assert bool(((got - want).abs() <= bound(k) * size + floor).all())
+
+
+def test_values_without_a_scale_stay_in_their_row(handle):
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(7)
+    m, n, k = 16384, 40, 64
+    a = torch.randn(m, k, generator=gen, device="cuda")
+    b = torch.randn(k, n, generator=gen, device="cuda")
+    clean = product(handle, a, b)
+    a[5, 3], a[700, 9] = float("inf"), float("nan")
+    got = product(handle, a, b)
+    assert not bool(torch.isfinite(got[5]).any()) and not bool(torch.isfinite(got[700]).any())
+    keep = torch.ones(m, dtype=torch.bool, device="cuda")
+    keep[5] = keep[700] = False
+    assert torch.equal(got[keep], clean[keep])
