@@ -42,6 +42,7 @@ constexpr int kSmCount = 148;
 constexpr long long kHalfMinRows = 16384;    // row count from which products of any width go by split halves
 constexpr int kZBlockRows = 32;      // rows per block of the hidden-layer gradient's closing sweep
 constexpr int kChunkGroups = 512;    // groups the sums of a scoring sweep's chunks are first added up in, when there are more chunks
+constexpr long long kUserColumns = 16 << 20;  // entries up to which a handle keeps the caller's column numbers too (64 MB)
 constexpr size_t kDirectBytes = (size_t)256 << 10;   // matrices up to this size cross the bus inside the permuting kernel (one copy and its latency less)
 constexpr long long kSmallProblem = 1LL << 27;   // nodes x widest layer: below it launch gaps show in a pass
 // Stored entries one warp walks before a row is cut into items, where the caller leaves it open.  A warp that walks a long row alone
@@ -255,6 +256,8 @@ struct gcn_admm {
   // Z scoring: units in chunks of about equally many stored entries, dealt to the warps of the grid in a fixed order
   int* d_chunk_ptr = nullptr;
   int* d_row_order = nullptr;               // rows per community by falling length: the order of the kernels that put several rows in a warp
+  int4* d_row_table = nullptr;              // the same order with what those kernels want of a row (see k_spmm_sets)
+  int* d_user_col = nullptr;                // the caller's row of every column; NULL on graphs of more than kUserColumns entries
   // closed-form search of the last hidden layer (gcn_admm_host::SegmentTables)
   gk::SegRef* d_segs = nullptr;
   gk::SegChunk* d_seg_chunks = nullptr;
@@ -368,9 +371,9 @@ struct gcn_admm {
   // wider than the item buffer (a caller's matrix wider than every layer, where nothing may be allocated): then
   // they are walked whole, slower but the same sums.
   struct GatherGraph {
-    const int *row_ptr, *col, *row_order, *perm;
+    const int *row_ptr, *col, *perm, *user_col;
     const float* dinv;
-    const int4 *items, *rows;
+    const int4 *row_table, *items, *rows;
     const int* item_row;
     int* row_done;
     int n, n_items, n_long, long_len;
@@ -380,7 +383,7 @@ struct gcn_admm {
     const size_t need = (size_t)n_items * ldw;
     float* const room = need <= item_sums_elems ? item_sums : wide && need * sizeof(float) <= wide_sums.size ? reinterpret_cast<float*>(wide_sums.base) : nullptr;
     const bool cut = n_items > 0 && room != nullptr;
-    return GatherGraph{d_row_ptr, d_col, d_row_order, d_perm, d_dinv, d_items, d_long_rows, d_item_row, d_row_done,
+    return GatherGraph{d_row_ptr, d_col, d_perm, d_user_col, d_dinv, d_row_table, d_items, d_long_rows, d_item_row, d_row_done,
                        (int)n, cut ? n_items : 0, cut ? n_long : 0, cut ? long_len : INT_MAX, room};
   }
   // Room for the items' sums at ldw padded columns.  Passes, recorded ones too, and callers under capture hold item_sums, which
@@ -443,9 +446,10 @@ struct gcn_admm {
   launch_alone(gk::k_spmm_wide<VEC, 4 / VEC * (NV4), UN, MAPPED, SLICED, RELU>, dim3((unsigned)cdiv(units * 32, 64), (unsigned)std::min<long long>(32768, cdiv(ld4, 32 * (NV4))),                \
               (unsigned)cdiv(ld4, 32768LL * 32 * (NV4))), 64, 0,                                                \
       g.row_ptr, g.col, g.dinv, g.perm, g.items, g.n, g.n_items, g.long_len, x, out, ldv, scratch, row_max)
-#define SETS(CL, EP, UN)                                                                                                  \
-  launch(gk::k_spmm_sets<VEC, 4 / VEC, CL, EP, UN, MAPPED, RELU>, (unsigned)cdiv(units * ((CL) * (EP)), 128), 128, 0,  \
-      g.row_ptr, g.col, g.dinv, g.perm, g.items, g.n, g.n_items, g.long_len, x, out, ldv, scratch, g.row_order, gk::ItemRows{g.rows, g.item_row, g.row_done}, row_max)
+#define SETS(CL, EP, UN) SETS_OF(1, CL, EP, UN)
+#define SETS_OF(NV4, CL, EP, UN)                                                                                          \
+  launch(gk::k_spmm_sets<VEC, 4 / VEC * (NV4), CL, EP, UN, MAPPED, RELU>, (unsigned)cdiv(units * ((CL) * (EP)), 128), 128, 0,  \
+      g.row_ptr, g.col, g.dinv, g.perm, g.user_col, g.items, g.n, g.n_items, g.long_len, x, out, ldv, scratch, g.row_table, gk::ItemRows{g.rows, g.item_row, g.row_done}, row_max)
     // Sets of entries per row: as many as the warp holds while the grid is then still small (latency counts), fewer
     // where the rows alone fill the chip several times over and the lanes of half-empty sets would only cost issue
     // slots.  Lines between the measured sizes 0.2 / 1.4 / 20 M lanes (columns x rows); the rule reads the handle's n, so a
@@ -458,7 +462,11 @@ struct gcn_admm {
     } else if (ld4 <= 4) {
       if (lanes <= 240000) SETS(4, 8, 4); else SETS(4, 2, 4);
     } else if (ld4 <= 8) {
-      if (lanes <= 480000) SETS(8, 4, 8); else SETS(8, 1, 8);
+      if (VEC == 4 && lanes <= 160000) SETS_OF(2, 4, 4, 4); else if (lanes <= 480000) SETS(8, 4, 8); else SETS(8, 1, 8);
+    } else if (VEC == 4 && ld4 <= 12) {
+      // four lanes of three vectors leave none idle (us, against 16 lanes: 13.0 -> 11.0 at 12 k rows, 76 -> 63 at 169 k, 2469 -> 2149
+      // at 2.45 M); of twelve single floats, for a matrix of odd width, they are slower (13.6 -> 17.4 at 10 k rows)
+      if (lanes <= 640000) SETS_OF(3, 4, 4, 4); else SETS_OF(3, 4, 2, 4);
     } else if (ld4 <= 16) {
       if (lanes <= 960000) SETS(16, 2, 8); else SETS(16, 1, 8);
     } else if (ld4 <= 32) WIDE(1, 4, false);
@@ -466,6 +474,7 @@ struct gcn_admm {
     else WIDE(2, 2, false);   // two neighbours in flight per lane beat four (fewer registers, more warps): measured
 #undef WIDE
 #undef SETS
+#undef SETS_OF
     in_pass = true;
     CU(cudaGetLastError());
     if (ld4 > 16 && g.n_long > 0) {
@@ -1305,6 +1314,8 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
   gcn_admm_host::Table<int> row_order;
   gcn_admm_host::order_rows_by_length(g, row_order);
   h->want_table(h->d_row_order, row_order);
+  h->want(h->d_row_table, (size_t)n);
+  if ((long long)g.nnz <= kUserColumns) h->want(h->d_user_col, (size_t)g.nnz);
   // work lists of the two forms of the Z search: the closed form's segments by community (at least two layers), and chunks
   // of units (items first, then rows) holding about the same number of stored entries each (at least three layers)
   gcn_admm_host::SegmentTables seg;
@@ -1445,6 +1456,12 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
   { gcn_admm_host::Table<unsigned short>().swap(h->gi.col_comm); }   // needed on the device only
   h->status = &h->report->status;
   h->tc_error = &h->report->error;
+  {
+    gcn_admm::Scope sc(h, "gather_tables", 1, 24.0 * n + 12.0 * g.nnz, 0.0);
+    gk::k_gather_tables<<<h->grid_for(std::max<long long>(n, h->d_user_col ? g.nnz : 0)), 256, 0, h->stream>>>(
+        h->d_row_order, h->d_row_ptr, h->d_dinv, (int)n, h->d_row_table, h->d_col, h->d_perm, g.nnz, h->d_user_col);
+    CU(cudaGetLastError());
+  }
 
   // Z_0 in community order, then P_1 = A~ Z_0 (Z_0 never changes, so neither does P_1)
   {
@@ -1964,15 +1981,22 @@ int gcn_admm_propagate_sharded(gcn_admm* h, int n_ranks, const float* x, int wid
         }
         for (int i = 0; i < n_own; ++i) order[(size_t)i] = i;
         std::stable_sort(order.begin(), order.end(), [&](int p_, int q_) { return rp[p_ + 1] - rp[p_] > rp[q_ + 1] - rp[q_]; });
+        std::vector<int4> table((size_t)n_own);
+        for (int i = 0; i < n_own; ++i) {
+          const int r_ = order[(size_t)i];
+          int bits;
+          std::memcpy(&bits, &dv[(size_t)r_], sizeof bits);
+          table[(size_t)i] = make_int4(r_, rp[r_], rp[r_ + 1], bits);
+        }
         int* d_rp = static_cast<int*>(take(rp.size() * sizeof(int)));
         int* d_cl = static_cast<int*>(take(cl.size() * sizeof(int)));
-        int* d_order = static_cast<int*>(take(order.size() * sizeof(int)));
+        int4* d_table = static_cast<int4*>(take(table.size() * sizeof(int4)));
         int* d_held = static_cast<int*>(take(held.size() * sizeof(int)));
         float* d_dv = static_cast<float*>(take(dv.size() * sizeof(float)));
         float* xl = static_cast<float*>(take((size_t)n_held * ldw * sizeof(float)));
         CU(cudaMemcpyAsync(d_rp, rp.data(), rp.size() * sizeof(int), cudaMemcpyHostToDevice, h->stream));
         if (!cl.empty()) CU(cudaMemcpyAsync(d_cl, cl.data(), cl.size() * sizeof(int), cudaMemcpyHostToDevice, h->stream));
-        if (n_own > 0) CU(cudaMemcpyAsync(d_order, order.data(), order.size() * sizeof(int), cudaMemcpyHostToDevice, h->stream));
+        if (n_own > 0) CU(cudaMemcpyAsync(d_table, table.data(), table.size() * sizeof(int4), cudaMemcpyHostToDevice, h->stream));
         if (n_held > 0) {
           CU(cudaMemcpyAsync(d_held, held.data(), held.size() * sizeof(int), cudaMemcpyHostToDevice, h->stream));
           CU(cudaMemcpyAsync(d_dv, dv.data(), dv.size() * sizeof(float), cudaMemcpyHostToDevice, h->stream));
@@ -1985,7 +2009,7 @@ int gcn_admm_propagate_sharded(gcn_admm* h, int n_ranks, const float* x, int wid
         }
         if (n_own > 0) {
           gcn_admm::Scope sc(h, "spmm.sharded", 1, 0.0, 0.0);
-          h->spmm_tables<4, false>(gcn_admm::GatherGraph{d_rp, d_cl, d_order, nullptr, d_dv, nullptr, nullptr, nullptr, nullptr, n_own, 0, 0, INT_MAX, nullptr},
+          h->spmm_tables<4, false>(gcn_admm::GatherGraph{d_rp, d_cl, nullptr, nullptr, d_dv, d_table, nullptr, nullptr, nullptr, nullptr, n_own, 0, 0, INT_MAX, nullptr},
                          xl, b + (size_t)lo * ldw, ldw / 4);
         }
         CU(cudaStreamSynchronize(h->stream));   // the host vectors of this rank go out of scope

@@ -120,8 +120,10 @@ __device__ __forceinline__ void add_block_sums(const double* partial, int count,
 // therefore not handled as rows: they come as `n_items` items {row, first entry, one past the last} (first in
 // the grid), whose sums go to `scratch` (one row per item).  The row's items are then added up in
 // item order: by the last of them to finish (one counter per long row, left at zero), or by k_spmm_long_rows.
-// MAPPED: x and out are dense matrices in the caller's row order; node c's row is perm[c] (a 4-byte load in
-// parallel with that of its weight), so that no copy of the operand in community order and none back is made.
+// MAPPED: x and out are dense matrices in the caller's row order; node c's row is perm[c], so that no copy of the operand in
+// community order and none back is made.  user_col (may be NULL): perm[col[e]] for every entry, for k_spmm_sets one dependent load
+// less on the way to the rows of x (24 k rows of 36 entries, 6 columns: 14.9 -> 13.4 us; in k_spmm_wide it disturbed the order of
+// the loads: 135 -> 143 us at 128 columns on 169 k rows).
 // RELU: out = A~ max(x, 0), so that a forward pass needs no sweep for its activations.
 // row_max (may be NULL): the largest magnitude of every row of `out`, which a product of `out` by split halves scales the row by.
 // Values are moved in vectors of VEC floats: four wherever rows start on 16-byte boundaries (always inside the
@@ -320,18 +322,19 @@ k_spmm_long_rows(const int4* __restrict__ rows, const T* __restrict__ scratch, T
 // Narrow operands.  G = CL * EP lanes share a row: CL of them side by side over its columns (NV vectors each), EP
 // such sets over its stored entries (entry e goes to set (e - first) mod EP), so that a row of k entries costs
 // k / EP dependent steps instead of k and a narrow row still fills the lanes of a warp; a shuffle tree adds the
-// sets at the end.  The order of a row's sum depends on EP alone: all layouts of a width agree bit for bit.
+// sets at the end.  The order of a row's sum depends on EP alone.
 // CL <= 4: every lane loads column and weight of its own entries (one word for the CL lanes of a set), one step
 // ahead of the operand rows.  CL >= 8: the G lanes load one entry each, columns two groups ahead and weights one,
 // and hand them to the sets by shuffles (with more lanes per set the repeated loads cost more than the shuffles).
-// Rows sharing a warp are taken by falling length.  Measured at 4 / 16 / 48 columns against one set per row:
+// Rows sharing a warp are taken by falling length, from row_table[k] = {row, first entry, one past the last, dinv}: one load where
+// order, row pointers and weight would be two that wait for each other.  Measured at 4 / 16 / 48 columns against one set per row:
 // 2.4 M rows, 126 M entries: 5.5 -> 1.1 ms, 2.2 -> 1.0, 2.7 -> 2.7; 13.8 k rows, 0.43 M entries: 293 -> 15 us, 85 -> 15, 37 -> 25.
 template <int VEC, int NV, int CL, int EP, int UN, bool MAPPED, bool RELU>
 __global__ void __launch_bounds__(128, CL >= 8 && VEC == 4 ? 10 : 8)
 k_spmm_sets(const int* __restrict__ row_ptr, const int* __restrict__ col, const float* __restrict__ dinv,
-            const int* __restrict__ perm, const int4* __restrict__ items, int n, int n_items, int long_len,
+            const int* __restrict__ perm, const int* __restrict__ user_col, const int4* __restrict__ items, int n, int n_items, int long_len,
             const typename Vec<VEC>::T* __restrict__ x, typename Vec<VEC>::T* __restrict__ out, int ldv,
-            typename Vec<VEC>::T* __restrict__ scratch, const int* __restrict__ row_order, const ItemRows ir, float* __restrict__ row_max) {
+            typename Vec<VEC>::T* __restrict__ scratch, const int4* __restrict__ row_table, const ItemRows ir, float* __restrict__ row_max) {
   gtc::enter_kernel();
   using T = typename Vec<VEC>::T;
   constexpr int G = CL * EP;
@@ -342,17 +345,22 @@ k_spmm_sets(const int* __restrict__ row_ptr, const int* __restrict__ col, const 
   const int unit = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) / G);
   if (unit >= n + n_items) return;
   int row, rs, re;
+  float di;
   const bool item = unit < n_items;
   if (item) {
     const int4 it = items[unit];
     row = it.x; rs = it.y; re = it.z;
+    di = dinv[row];
+  } else if (G < 32) {
+    const int4 it = row_table[unit - n_items];
+    row = it.x; rs = it.y; re = it.z;
+    di = __int_as_float(it.w);
   } else {
     row = unit - n_items;
-    if (G < 32) row = row_order[row];
     rs = row_ptr[row]; re = row_ptr[row + 1];
-    if (re - rs > long_len) return;
+    di = dinv[row];
   }
-  const float di = dinv[row];
+  if (!item && re - rs > long_len) return;
   T* const row_out = out + (long long)(MAPPED ? perm[row] : row) * ldv;
   T* const dst = item ? scratch + (long long)unit * ldv : row_out;
   float m = 0.f;
@@ -361,20 +369,24 @@ k_spmm_sets(const int* __restrict__ row_ptr, const int* __restrict__ col, const 
 #pragma unroll
     for (int v = 0; v < NV; ++v) vzero(acc[v]);
     if constexpr (CL <= 4) {
-      int c[UN];
+      int c[UN], ru[UN];
+      const auto fetch = [&](int e) {
 #pragma unroll
-      for (int u = 0; u < UN; ++u) c[u] = (rs + set + u * EP < re) ? col[rs + set + u * EP] : -1;
+        for (int u = 0; u < UN; ++u) {
+          c[u] = (e + u * EP < re) ? col[e + u * EP] : -1;
+          if (MAPPED && user_col != nullptr) ru[u] = (e + u * EP < re) ? user_col[e + u * EP] : -1;
+        }
+      };
+      fetch(rs + set);
       for (int e = rs + set; e < re; e += EP * UN) {
         float w[UN];
         int r[UN];
 #pragma unroll
         for (int u = 0; u < UN; ++u) {
           w[u] = c[u] >= 0 ? dinv[c[u]] : 0.f;
-          r[u] = c[u] >= 0 ? (MAPPED ? perm[c[u]] : c[u]) : -1;
+          r[u] = c[u] < 0 || !MAPPED ? c[u] : user_col != nullptr ? ru[u] : perm[c[u]];
         }
-        const int en = e + EP * UN;
-#pragma unroll
-        for (int u = 0; u < UN; ++u) c[u] = (en + u * EP < re) ? col[en + u * EP] : -1;
+        fetch(e + EP * UN);
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
           const int f = cb + cl + CL * v;
@@ -391,15 +403,16 @@ k_spmm_sets(const int* __restrict__ row_ptr, const int* __restrict__ col, const 
       }
     } else {
       int c_n = rs + gl < re ? col[rs + gl] : -1, c_n2 = rs + G + gl < re ? col[rs + G + gl] : -1;
+      const auto row_of = [&](int c, int e) { return c < 0 ? 0 : !MAPPED ? c : user_col != nullptr ? user_col[e] : perm[c]; };
       float w_n = c_n >= 0 ? dinv[c_n] : 0.f;
-      int r_n = c_n >= 0 ? (MAPPED ? perm[c_n] : c_n) : 0;
+      int r_n = row_of(c_n, rs + gl);
       for (int base = rs; base < re; base += G) {
         const float w = w_n;
         const int r = r_n;
         c_n = c_n2;
         c_n2 = base + 2 * G + gl < re ? col[base + 2 * G + gl] : -1;
         w_n = c_n >= 0 ? dinv[c_n] : 0.f;
-        r_n = c_n >= 0 ? (MAPPED ? perm[c_n] : c_n) : 0;
+        r_n = row_of(c_n, base + G + gl);
         const int steps = (min(G, re - base) + EP - 1) / EP;
         for (int t = 0; t < steps; t += UN) {
           int rj[UN];
@@ -2275,6 +2288,19 @@ __global__ void k_dual(float4* __restrict__ U, const float4* __restrict__ Z, con
     u.z = fmaf(rho, z.z - h.z, u.z); u.w = fmaf(rho, z.w - h.w, u.w);
     U[i] = u;
   }
+}
+
+// The tables of k_spmm_sets' rows and of the caller's columns (may be NULL) from those of the graph.
+__global__ void k_gather_tables(const int* __restrict__ order, const int* __restrict__ row_ptr, const float* __restrict__ dinv, int n,
+                                int4* __restrict__ row_table, const int* __restrict__ col, const int* __restrict__ perm, long long nnz,
+                                int* __restrict__ user_col) {
+  const long long first = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
+  for (long long i = first; i < n; i += stride) {
+    const int row = order[i];
+    row_table[i] = make_int4(row, row_ptr[row], row_ptr[row + 1], __float_as_int(dinv[row]));
+  }
+  if (user_col == nullptr) return;
+  for (long long e = first; e < nnz; e += stride) user_col[e] = perm[col[e]];
 }
 
 // dst[c][r] = src[r][c] for a small rows x cols matrix (weights and their gradients).

@@ -39,3 +39,17 @@ def test_device_propagation(case, width, shift):
         got = buf[1, shift:shift + wl.n * width].reshape(wl.n, width).cpu().numpy()
         assert np.max(np.abs(got - want) / scale) < 1e-6
         assert float(buf[1, shift + wl.n * width]) == -7.0
+
+
+@pytest.mark.parametrize("width", [20, 21, 30, 35, 36, 42, 47, 48, 49])
+def test_lane_splits_of_narrow_operands(case, width):
+    """Two and three vectors per lane, whole and ragged; rows of vectors of one, two and four floats."""
+    import torch
+    wl, g, At = case
+    x = np.random.default_rng(width).standard_normal((wl.n, width)).astype(np.float32)
+    src, dst = torch.from_numpy(x).cuda(), torch.full((wl.n, width), -7.0, device="cuda")
+    torch.cuda.synchronize()
+    g.propagate(src.data_ptr(), width, dst.data_ptr())
+    want = At @ x.astype(np.float64)
+    scale = abs(At) @ np.abs(x.astype(np.float64)) + 1e-30
+    assert np.max(np.abs(dst.cpu().numpy() - want) / scale) < 1e-6
