@@ -119,7 +119,7 @@ EncodeTiledFn encode_tiled() {
 // form that stages the operand through registers).
 bool make_a_tile_map(const float* A, long long rows, int ld, CUtensorMap* map) {
   EncodeTiledFn fn = encode_tiled();
-  if (fn == nullptr || ld < gtc::kChunkK) return false;
+  if (fn == nullptr) return false;
   const cuuint64_t dims[2] = {(cuuint64_t)ld, (cuuint64_t)rows};
   const cuuint64_t strides[1] = {(cuuint64_t)ld * sizeof(float)};
   const cuuint32_t box[2] = {(cuuint32_t)gtc::kChunkK, (cuuint32_t)gtc::kBlockM};
@@ -492,9 +492,9 @@ struct gcn_admm {
   }
   // With many row tiles k_gemm_tc_ws would split the same weights again for every tile; with at most one tile per CTA, or
   // with few chunks, that costs nothing, and the launch that makes the image would (13.8 k rows, 767 x 1000, three tiles per CTA:
-  // 130 -> 98 us by an image; 10 x 1000: no gain).  A's tensor copies want rows of at least one chunk.
-  bool by_halves(long long Mr, int N, int K, int lda) const {
-    if (!on_tensor_cores(Mr, K) || lda < gtc::kChunkK || encode_tiled() == nullptr) return false;
+  // 130 -> 98 us by an image; 10 x 1000: no gain).
+  bool by_halves(long long Mr, int N, int K) const {
+    if (!on_tensor_cores(Mr, K) || encode_tiled() == nullptr) return false;
     return p.tensor_cores == 2 || Mr >= kHalfMinRows || (K >= 128 && cdiv(Mr, gtc::kBlockM) > kSmCount / cdiv(N, group_width(N, true)));
   }
   static size_t image_bytes(int N, const gtc::Image& im) {
@@ -502,9 +502,9 @@ struct gcn_admm {
     return gtc::image_blocks_bytes(groups, im.nt, im.kc) + (size_t)groups * im.nt * sizeof(float);
   }
   // Asks for an image of the operand of an n x K by K x N product, where that product takes one.
-  void want_image(gtc::Image& im, int N, int K, int lda) {
+  void want_image(gtc::Image& im, int N, int K) {
     im = gtc::Image{nullptr, group_width(N, true), (int)cdiv(K, gtc::kChunkK)};
-    if (by_halves(n, N, K, lda)) want(im.data, image_bytes(N, im), kZero);
+    if (by_halves(n, N, K)) want(im.data, image_bytes(N, im), kZero);
   }
   void split_b(const gtc::SplitB& b) {
     const int rows = (int)(cdiv(b.N, b.image.nt) * b.image.nt);
@@ -521,7 +521,7 @@ struct gcn_admm {
     char name[48];
     if (Bk != nullptr && on_tensor_cores(Mr, K)) {
       CUtensorMap tmap;
-      const bool halves = by_halves(Mr, N, K, lda) && a_max != nullptr && image.data != nullptr && make_a_tile_map(A, Mr, lda, &tmap);
+      const bool halves = by_halves(Mr, N, K) && a_max != nullptr && image.data != nullptr && make_a_tile_map(A, Mr, lda, &tmap);
       const int tiles = (int)cdiv(Mr, gtc::kBlockM), nt = group_width(N, halves), groups = (int)cdiv(N, nt), kc = (int)cdiv(K, gtc::kChunkK);
       std::snprintf(name, sizeof name, halves ? "gemm_half@%dx%d" : "gemm_tc@%dx%d", K, N);
       Scope sc(this, name, 1, 4.0 * ((double)Mr * (lda + ldc) + (double)K * ldb), 2.0 * (double)Mr * N * K);
@@ -645,15 +645,15 @@ struct gcn_admm {
 
   // grad (and grad_t) from the `splits` partial sums gemm_tn left in `part`; with `ctl` the start of the W_l search too.
   void finish_grad(int splits, int Ka, int Nb, int ldp, float* out, float* out_t, int ldt, const float* w, SearchCtl* ctl,
-                   const gtc::Image& image) {
+                   const gtc::Image& image, bool maxima) {
     Scope sc(this, "finish_grad", 1, 4.0 * (double)Ka * ldp * (splits + (w ? 3 : 1)), 0.0);
     const long long elems = (long long)Ka * ldp;
     if (splits >= 16)
       launch(gk::k_finish_grad<8>, (unsigned)cdiv(elems, 32), 256, 0, part, splits, Ka, Nb, ldp, out, out_t, ldt, w, red_part,
-                                                                            ticket, ctl, p.bt_shrink, p.bt_growth, status, image);
+                                                                            ticket, ctl, p.bt_shrink, p.bt_growth, status, image, maxima);
     else
       launch(gk::k_finish_grad<1>, (unsigned)(cdiv(Ka, 32) * cdiv(ldp, 32)), 256, 0, part, splits, Ka, Nb, ldp, out, out_t, ldt, w, red_part,
-                                                                                     ticket, ctl, p.bt_shrink, p.bt_growth, status, image);
+                                                                                     ticket, ctl, p.bt_shrink, p.bt_growth, status, image, maxima);
     CU(cudaGetLastError());
   }
 
@@ -721,7 +721,8 @@ struct gcn_admm {
       splits = gemm_tn(P[l], ld[l - 1], R, ldc, ldc, n, Kp, Cn, nullptr, 0.f, &ctl->part_max);   // grad = P_l^T R_l
     }
     const bool bounded = tn_on_tensor_cores(n);   // by the largest partial sum; else the image is made from the gradient itself
-    finish_grad(splits, Kp, Cn, ldc, grad, grad_t, ld[l - 1], W[l], ctl, bounded ? img_D[l] : gtc::Image{nullptr, 16, 1});
+    finish_grad(splits, Kp, Cn, ldc, grad, grad_t, ld[l - 1], W[l], ctl, bounded ? img_D[l] : gtc::Image{nullptr, 16, 1},
+                img_H[l].data != nullptr || img_G[l].data != nullptr);
     if (!bounded && img_D[l].data != nullptr) split_b(gtc::SplitB{grad_t, ld[l - 1], Cn, Kp, img_D[l]});
     gemm_nn(P[l], ld[l - 1], P_max[l], grad, ldc, grad_t, ld[l - 1], D, ldc, n, Cn, Kp, img_D[l], &ctl->done);   // D = P_l grad
     gk::SearchW a{};
@@ -1131,7 +1132,10 @@ struct gcn_admm {
     CU(stage.finish(stream));
     const long long cells = std::max((long long)r * ld[l], (long long)c * ld[l - 1]);
     float most = 0.f;
-    for (long long e = 0; e < (long long)r * c; ++e) most = std::max(most, std::fabs(host_w[e]));
+    if (img_H[l].data != nullptr || img_G[l].data != nullptr) {
+#pragma omp simd reduction(max : most)
+      for (long long e = 0; e < (long long)r * c; ++e) most = std::max(most, std::fabs(host_w[e]));
+    }
     gk::k_load_weight<<<grid_for(cells), 256, 0, stream>>>(grad, r, c, W[l], ld[l], Wt[l], ld[l - 1], img_H[l], img_G[l], most);
     CU(cudaGetLastError());
   }
@@ -1406,10 +1410,10 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
   h->img_H.assign(L + 1, gtc::Image{nullptr, 16, 1}); h->img_G = h->img_D = h->img_H;
   h->P_max.assign(L + 1, nullptr);
   for (int l = 1; l <= L; ++l) {
-    h->want_image(h->img_H[l], h->C[l], h->C[l - 1], h->ld[l - 1]);   // P_l W_l, G W_l; P_l grad has its shape
-    h->want_image(h->img_D[l], h->C[l], h->C[l - 1], h->ld[l - 1]);
-    if (l >= 2) h->want_image(h->img_G[l], h->C[l - 1], h->C[l], h->ld[l]);
-    if (h->by_halves(n, h->C[l], h->C[l - 1], h->ld[l - 1])) h->want(h->P_max[l], rows);
+    h->want_image(h->img_H[l], h->C[l], h->C[l - 1]);   // P_l W_l, G W_l; P_l grad has its shape
+    h->want_image(h->img_D[l], h->C[l], h->C[l - 1]);
+    if (l >= 2) h->want_image(h->img_G[l], h->C[l - 1], h->C[l]);
+    if (h->by_halves(n, h->C[l], h->C[l - 1])) h->want(h->P_max[l], rows);
   }
   h->want(h->B1_max, rows);
   h->want(h->B2_max, rows);
@@ -1796,7 +1800,7 @@ int gcn_admm_dense_product(gcn_admm* h, const float* A, const float* B, float* C
       gk::k_transpose_small<<<(unsigned)cdiv((long long)k * n, 256), 256, 0, h->stream>>>(b, ldb, bk, ldbk, k, n);
       CU(cudaGetLastError());
       h->p.tensor_cores = tensor_cores;
-      if (tensor_cores && h->by_halves(m, n, k, lda)) {
+      if (tensor_cores && h->by_halves(m, n, k)) {
         image.nt = gcn_admm::group_width(n, true);
         image.kc = (int)cdiv(k, gtc::kChunkK);
         image.data = dalloc<uint8_t>(gcn_admm::image_bytes(n, image));
@@ -1840,7 +1844,7 @@ int gcn_admm_dense_product_tn(gcn_admm* h, const float* A, const float* B, float
       CU(cudaMemcpy2DAsync(b, (size_t)ldb * 4, B, (size_t)nb * 4, (size_t)nb * 4, (size_t)rows, cudaMemcpyDeviceToDevice, h->stream));
       h->p.tensor_cores = tensor_cores;
       const int splits = h->gemm_tn(a, lda, b, ldb, ldp, rows, ka, nb);
-      h->finish_grad(splits, ka, nb, ldp, c, nullptr, 0, nullptr, nullptr, gtc::Image{nullptr, 16, 1});
+      h->finish_grad(splits, ka, nb, ldp, c, nullptr, 0, nullptr, nullptr, gtc::Image{nullptr, 16, 1}, false);
       h->p.tensor_cores = saved;
       CU(cudaMemcpy2DAsync(C, (size_t)nb * 4, c, (size_t)ldp * 4, (size_t)nb * 4, (size_t)ka, cudaMemcpyDeviceToDevice, h->stream));
       CU(cudaStreamSynchronize(h->stream));

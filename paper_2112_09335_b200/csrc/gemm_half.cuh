@@ -11,11 +11,11 @@
 // accumulator is rounded half as often: errors against fp64 halve, 6.4e-7 -> 3.4e-7 of ||C|| at K = 256), and the operands take
 // half the shared memory and half of its bandwidth, which bounded the TF32 form at 256 columns.
 //
-// 1.2 M rows, launched alone, TF32 pairs -> this form in ms (HBM alone): 256 x 256 0.81 -> 0.61 (0.38), 128 x 256 0.46 -> 0.40 (0.28),
-// 256 x 128 0.43 -> 0.36 (0.28), 256 x 47 0.31 -> 0.26 (0.22).  At 256 columns shared memory is what is left: a K chunk of 32 moves
+// 1.2 M rows, launched alone, TF32 pairs -> this form in ms (HBM alone): 256 x 256 0.81 -> 0.59 (0.38), 128 x 256 0.46 -> 0.38 (0.28),
+// 256 x 128 0.43 -> 0.36 (0.28), 47 x 256 0.33 -> 0.31 (0.22), 256 x 47 0.31 -> 0.26 (0.22).  At 256 columns shared memory is what is left: a K chunk of 32 moves
 // 72 KB of MMA operands, 48 KB of copies, 32 KB of splitting and 48 KB of the epilogue through it, 1,560 clocks at 128 B a clock
 // against 768 of MMAs; leaving out the copies of B, the splitting or the stores alone saves 4, 13 and 10 %.  Columns in one group
-// of 256 instead of two of 128 (every A tile read and split twice): 0.61 against 0.71 ms.
+// of 256 instead of two of 128 (every A tile read and split twice): 0.59 against 0.67 ms.
 //
 // The row maxima of A come with A: whoever writes the matrix leaves them (row_max).  B comes as an image of the staged layout, kept
 // by whoever writes the weights (put_half: every column by one scale, from a bound of the matrix) or made by k_split_b.
@@ -137,8 +137,10 @@ k_split_b(const SplitB p, int rows) {
 template <int NT>
 struct HalfCfg {
   static constexpr int kSets = NT > 128 ? 1 : 2;        // accumulator sets (main + correction each)
-  // With one set the MMAs of the next tile wait for the epilogue: eight warps then, which leaves room for four producer warps.
-  static constexpr int kProdWarps = NT > 128 ? 4 : 8, kEpiWarps = NT > 128 ? 8 : 4;
+  // Eight epilogue warps where the column steps divide by two per quarter: with one set the MMAs of the next tile wait for them (and
+  // four producer warps leave them the registers), with two and a short reduction they are what a tile takes longest for (1.2 M rows,
+  // 128 columns, four -> eight: 201 -> 152 us at K = 12, 207 -> 159 at 47, 238 -> 212 at 128, 358 -> 358 at 256).
+  static constexpr int kProdWarps = NT > 128 ? 4 : 8, kEpiWarps = NT >= 64 && NT != 96 ? 8 : 4;
   static constexpr int kMmaWarp = kProdWarps + kEpiWarps;
   static constexpr int kThreads = (kMmaWarp + 2) * 32;
   static constexpr int kBBytes = 2 * NT * kHalfRow;     // hi and lo of a chunk
@@ -169,6 +171,7 @@ k_gemm_half(const float* __restrict__ row_max, float* __restrict__ C, int ldc, i
   __shared__ __align__(8) uint64_t bars[3 * R + 5];           // raw[R], ready[R], empty[R], acc_full[2], acc_empty[2], drain
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag, copies;                          // copies: chunks whose copies have been started
+  __shared__ unsigned col_range[2];                           // bits of the largest and, inverted, of the smallest column factor
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t smem_base = smem_u32(smem);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -185,8 +188,7 @@ k_gemm_half(const float* __restrict__ row_max, float* __restrict__ C, int ldc, i
     abort_flag = copies = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  for (int c = tid; c < NT; c += Cfg::kThreads)
-    col_factor[c] = reinterpret_cast<const float*>(b_image + image_blocks_bytes(gridDim.y, NT, kc_count))[blockIdx.y * NT + c];
+  if (tid < 2) col_range[tid] = 0u;
   if (warp == Cfg::kMmaWarp) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)),
                  "r"(Cfg::kTmemCols)
@@ -198,6 +200,14 @@ k_gemm_half(const float* __restrict__ row_max, float* __restrict__ C, int ldc, i
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem_base = tmem_base_slot;
   volatile int* abortp = &abort_flag;
+  if (warp >= Cfg::kProdWarps && warp < Cfg::kMmaWarp) {   // the epilogue's own; it waits at a barrier of its own below
+    for (int c = tid - Cfg::kProdWarps * 32; c < NT; c += Cfg::kEpiWarps * 32) {
+      const float f = reinterpret_cast<const float*>(b_image + image_blocks_bytes(gridDim.y, NT, kc_count))[blockIdx.y * NT + c];
+      col_factor[c] = f;
+      atomicMax(&col_range[0], __float_as_uint(f));
+      atomicMax(&col_range[1], ~__float_as_uint(f));
+    }
+  }
 
   const int n_tiles = (M + kBlockM - 1) / kBlockM;
   const int my_tiles = (n_tiles > (int)blockIdx.x) ? (n_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
@@ -317,6 +327,9 @@ k_gemm_half(const float* __restrict__ row_max, float* __restrict__ C, int ldc, i
     constexpr int SLOTS = CW / 4;
     constexpr int ROWS_PER_STORE = 32 / SLOTS;
     constexpr int WARPS_PER_QUARTER = Cfg::kEpiWarps / 4, STEPS = NT / CW / WARPS_PER_QUARTER;
+    static_assert(NT == STEPS * CW * WARPS_PER_QUARTER, "every column has its step");
+    asm volatile("bar.sync 1, %0;" ::"n"(Cfg::kEpiWarps * 32) : "memory");   // the column factors are there
+    const float col_most = __uint_as_float(col_range[0]), col_least = __uint_as_float(~col_range[1]);
     const int turn = (warp - Cfg::kProdWarps) >> 2;   // which of the quarter's warps this is: they take the column steps in turn
     uint8_t* tbuf = smem + kEpiBase + (size_t)(warp - Cfg::kProdWarps) * 4096;
     for (int tile_i = 0; tile_i < my_tiles; ++tile_i) {
@@ -325,6 +338,8 @@ k_gemm_half(const float* __restrict__ row_max, float* __restrict__ C, int ldc, i
       const float row_factor = inverse_scale_of(row0 + lane < M ? __ldg(row_max + row0 + lane) : 0.f);
       if (!__all_sync(0xffffffffu, mbar_wait_abortable(bar_acc_full + 8 * set, (tile_i / SETS) & 1, abortp))) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      // whether row and column factors may be joined: normal numbers for every pair of the warp's
+      const bool joined = __all_sync(0xffffffffu, row_factor * col_most <= 0x1p126f && row_factor * col_least >= 0x1p-126f);
       uint32_t v[16], w[16];   // main product and corrections of 16 columns; with one accumulator set read ahead, beside the stores of those before
       constexpr bool AHEAD = SETS == 1;
       const auto fetch = [&](int part) {   // part of this warp's columns: CW / 16 of them make a step
@@ -353,10 +368,14 @@ k_gemm_half(const float* __restrict__ row_max, float* __restrict__ C, int ldc, i
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
             const float4 f = *reinterpret_cast<const float4*>(col_factor + at + half * 16 + q * 4);
-            // the smaller factor first: the product of the two alone may leave the range, and so may the sum times the larger
-            const auto scaled = [&](float x, float c) { return x * fminf(row_factor, c) * fmaxf(row_factor, c); };
-            *reinterpret_cast<float4*>(tbuf + lane * 128 + (((half * 4 + q) ^ (lane & (SLOTS - 1))) * 16)) =
-                make_float4(scaled(sum[q * 4], f.x), scaled(sum[q * 4 + 1], f.y), scaled(sum[q * 4 + 2], f.z), scaled(sum[q * 4 + 3], f.w));
+            float4 x = make_float4(sum[q * 4], sum[q * 4 + 1], sum[q * 4 + 2], sum[q * 4 + 3]);
+            if (joined) {
+              x.x *= row_factor * f.x; x.y *= row_factor * f.y; x.z *= row_factor * f.z; x.w *= row_factor * f.w;
+            } else {   // the smaller factor first: the sum times the larger one may leave the range too
+              const auto scaled = [&](float y, float c) { return y * fminf(row_factor, c) * fmaxf(row_factor, c); };
+              x = make_float4(scaled(x.x, f.x), scaled(x.y, f.y), scaled(x.z, f.z), scaled(x.w, f.w));
+            }
+            *reinterpret_cast<float4*>(tbuf + lane * 128 + (((half * 4 + q) ^ (lane & (SLOTS - 1))) * 16)) = x;
           }
         }
         __syncwarp();

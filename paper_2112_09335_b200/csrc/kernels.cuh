@@ -982,7 +982,8 @@ __device__ __forceinline__ void weight_tile(int tile, int rows, int cols, int pa
 // Weight gradient from its split partial sums, and the start of the W_l search, in one launch:
 //   grad[e] = sum over splits of part[s][e] (fp64, in split order), its transpose for P grad, ||grad||^2, ||W||^2, and where one is
 //   kept the transpose's image, scaled by the bound splits * (largest partial sum): the split holds an element to 2^-23 of its
-//   magnitude down to 2^-29 of the bound, which is at most `splits` times too large where all partial sums are alike.
+//   magnitude down to 2^-29 of the bound.  `maxima`: the largest magnitudes of grad and W go to the control block, for the images of
+//   W after its move.
 // SG = 1: a block owns a tile of 32 x 32 elements (grid: tiles over rows x ldp).  SG = 8 (many splits): 32 consecutive elements,
 // eight threads per element, each adding its own run of consecutive splits; the transpose is then written one
 // float at a time (a tile of 32 x 32 would leave one block where there are 32 now).  The last block to finish adds the
@@ -991,7 +992,7 @@ template <int SG>
 __global__ void __launch_bounds__(256)
 k_finish_grad(const float* __restrict__ part, int splits, int rows, int cols, int ldp, float* __restrict__ grad,
               float* __restrict__ grad_t, int ldt, const float* __restrict__ W, double* partial, unsigned* ticket,
-              SearchCtl* ctl, double shrink, double growth, int* status, const gtc::Image image) {
+              SearchCtl* ctl, double shrink, double growth, int* status, const gtc::Image image, bool maxima) {
   gtc::enter_kernel();
   __shared__ double sh[16], s_part[SG == 1 ? 1 : SG][32];
   __shared__ WeightTile turn;
@@ -1047,23 +1048,28 @@ k_finish_grad(const float* __restrict__ part, int splits, int rows, int cols, in
     }
   }
   if (W == nullptr) return;
-  __shared__ unsigned s_most[2];   // magnitudes: their order is that of their bits
-  const auto block_most = [&] {
-    if (threadIdx.x < 2) s_most[threadIdx.x] = 0u;
-    __syncthreads();
+  // The sums, and in passing the maxima: a warp's go to shared memory before block_sums, whose barriers hand them to thread 0.
+  __shared__ unsigned s_most[8][2];   // magnitudes: their order is that of their bits
+  const auto block_totals = [&](uint2& top) {
+    if (maxima) {
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(most[j]));
-      if ((threadIdx.x & 31) == 0) atomicMax(&s_most[j], m);
+      for (int j = 0; j < 2; ++j) {
+        const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(most[j]));
+        if ((threadIdx.x & 31) == 0) s_most[threadIdx.x >> 5][j] = m;
+      }
     }
-    __syncthreads();
+    block_sums(sq, sh);
+    top = make_uint2(0u, 0u);
+    if (maxima && threadIdx.x == 0)
+#pragma unroll
+      for (int w = 0; w < 8; ++w) top = make_uint2(max(top.x, s_most[w][0]), max(top.y, s_most[w][1]));
   };
-  block_sums(sq, sh);
-  block_most();
+  uint2 top;
+  block_totals(top);
   if (threadIdx.x == 0) {
     partial[3 * (size_t)blockIdx.x] = sq[0];
     partial[3 * (size_t)blockIdx.x + 1] = sq[1];
-    reinterpret_cast<uint2*>(partial)[3 * (size_t)blockIdx.x + 2] = make_uint2(s_most[0], s_most[1]);
+    if (maxima) reinterpret_cast<uint2*>(partial)[3 * (size_t)blockIdx.x + 2] = top;
     __threadfence();
     s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
   }
@@ -1072,19 +1078,19 @@ k_finish_grad(const float* __restrict__ part, int splits, int rows, int cols, in
   __threadfence();
   sq[0] = sq[1] = 0.0;
   most[0] = most[1] = 0.f;
+#pragma unroll 4
   for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x) {
     sq[0] += __ldcg(partial + 3 * (size_t)b);
     sq[1] += __ldcg(partial + 3 * (size_t)b + 1);
+    if (!maxima) continue;
     const uint2 m = __ldcg(reinterpret_cast<const uint2*>(partial) + 3 * (size_t)b + 2);
     most[0] = fmaxf(most[0], __uint_as_float(m.x));
     most[1] = fmaxf(most[1], __uint_as_float(m.y));
   }
-  block_sums(sq, sh);
-  block_most();
+  block_totals(top);
   if (threadIdx.x == 0) {
     *ticket = 0;
-    ctl->g_max = __uint_as_float(s_most[0]);
-    ctl->w_max = __uint_as_float(s_most[1]);
+    if (maxima) { ctl->g_max = __uint_as_float(top.x); ctl->w_max = __uint_as_float(top.y); }
     ctl->part_max = 0u;   // every block has read it
     begin_one(ctl, sq[0], sq[1], shrink, growth, nullptr, status);
   }

@@ -30,7 +30,7 @@ def bound(k):
 
 
 @pytest.mark.parametrize("m", [16384, 16385, 19071])                                   # whole tiles, one row more, a tile less one row
-@pytest.mark.parametrize("n,k", [(1, 32), (16, 33), (17, 63), (33, 64), (49, 65), (65, 96), (97, 40), (129, 47), (193, 128), (257, 100), (8, 2048)])
+@pytest.mark.parametrize("n,k", [(1, 32), (16, 33), (17, 63), (33, 64), (49, 65), (65, 96), (97, 40), (129, 47), (193, 128), (257, 100), (8, 2048), (40, 8), (256, 11), (64, 31)])
 def test_edges(handle, m, n, k):
     import torch
     gen = torch.Generator(device="cuda").manual_seed(m + n + k)
