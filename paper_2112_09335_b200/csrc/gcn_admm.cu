@@ -129,14 +129,15 @@ bool make_a_tile_map(const float* A, long long rows, int ld, CUtensorMap* map) {
 }
 
 // Lets `kernel` be launched on the current device (`device`) with `smem` bytes of dynamic shared memory.  The limit belongs to the
-// function, not to a handle, and handles of other sizes are stepped in between: it is only ever raised.
+// function, not to a handle, and handles of other sizes are stepped in between: it is only ever raised.  (What needs no leave is 48
+// KB, the kernel's static shared memory among them.)
 void allow_shared(int device, const void* kernel, size_t smem) {
   static std::mutex mutex;
   static std::map<std::pair<int, const void*>, size_t> most;
   std::lock_guard<std::mutex> lock(mutex);
   size_t& limit = most[{device, kernel}];
   limit = std::max(limit, smem);
-  if (limit > 48 * 1024) CU(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit));
+  if (limit > 40 * 1024) CU(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit));
 }
 
 bool is_device_pointer(const void* p) {
@@ -758,6 +759,18 @@ struct gcn_admm {
     }
   }
 
+  // Whether the update of Z_l forms its gradient and T in one launch (k_zgrad_products).  What it saves is launches and passes of G
+  // through memory, what it costs is the rate of fp32 FMA out of shared memory, so the line lies by the next layer's width against
+  // this one's and by n.  us a pass, separate / joined: 64-128-4 at 4 k, 170 k and 600 k rows 110 / 101, 657 / 602, 2024 / 1927;
+  // 64-256-16 149 / 139, 1124 / 1102, 3700 / 3596; 64-128-16 112 / 102, 697 / 708, 2156 / 2274; 64-32-8 84 / 75, 346 / 351, 1009 / 1048;
+  // 64-64-31 at 1 k, 4 k, 8 k, 16 k 75 / 69, 92 / 85, 100 / 98, 132 / 138; 64-64-47 78 / 74, 97 / 91, 107 / 112, 142 / 162.
+  bool joins_products(int l) const {
+    const long long ldl = ld[l], ldn = ld[l + 1];
+    if (ldn > 48 || (ldn + 12) * ldl * sizeof(float) > 96 * 1024) return false;
+    if (ldn > 16) return n <= (ldn <= 32 ? 8192 : 4096);
+    return n <= 65536 || ldn <= 4 || ldl >= 16 * ldn;
+  }
+
   // ---- Z_{l,m}, l < L, every community (Appendix A, Eq. 5/6 and 8-10) ------------------
   // resid_ready: resid_of(l + 1) holds the derivative of phi_{l+1} at the stored H_{l+1}.
   void update_Z_hidden(int l, bool resid_ready) {
@@ -766,9 +779,28 @@ struct gcn_admm {
     SearchCtl* ctl = ctl_z + (size_t)l * M;
     float* const Rn = resid_of(l + 1);
     if (!resid_ready) resid(l + 1, Rn);                                  // R'_{l+1}
-    spmm(Rn, B1, ldn, img_G[l + 1].data != nullptr ? B1_max : nullptr);                                // S = A~ R'
-    gemm_nn(B1, ldn, B1_max, Wt[l + 1], ldl, W[l + 1], ldn, B2, ldl, n, C[l], C[l + 1], img_G[l + 1]); // S W_{l+1}^T
-    {
+    spmm(Rn, B1, ldn, !joins_products(l) && img_G[l + 1].data != nullptr ? B1_max : nullptr);                      // S = A~ R'
+    // G = S W_{l+1}^T + nu (Z_l - f(H_l)) and T = G W_{l+1}: in one launch where the next layer is narrow (see k_zgrad_products)
+    const bool joined = joins_products(l);
+    if (joined) {
+      Scope sc(this, "zgrad_products", 1, 4.0 * (double)n * (3.0 * ldl + 2.0 * ldn), 4.0 * (double)n * C[l] * C[l + 1]);
+      const auto finish = [&](auto kernel, int kv, int rows) {
+        static_assert(kZBlockRows == 32, "a block's groups of eight lanes take 32 rows");
+        const size_t smem = (size_t)kv * 4 * ldl * sizeof(float);
+        const int blocks = std::min(n_zblocks, resident_blocks((const void*)kernel, 256 / rows, smem));
+        launch(kernel, (unsigned)blocks, 256 / rows, smem, (float4*)B2, (const float4*)Z[l], (const float4*)H[l], (const float4*)B1, (const float4*)Wt[l + 1], (float4*)B0,
+               ldl / 4, C[l + 1], d_zblocks, n_zblocks, p.nu, red_part, d_comm_block_ptr, comm_tickets, ctl, sums_z, p.bt_shrink, p.bt_growth, n_active, status);
+      };
+      if (ldn <= 4) finish(gk::k_zgrad_products<1, 2>, 1, 2);
+      else if (ldn <= 8) finish(gk::k_zgrad_products<2, 2>, 2, 2);
+      else if (ldn <= 12) finish(gk::k_zgrad_products<3, 2>, 3, 2);
+      else if (ldn <= 16) finish(gk::k_zgrad_products<4, 2>, 4, 2);
+      else if (ldn <= 24) finish(gk::k_zgrad_products<6, 1>, 6, 1);
+      else if (ldn <= 32) finish(gk::k_zgrad_products<8, 1>, 8, 1);
+      else finish(gk::k_zgrad_products<12, 1>, 12, 1);
+      CU(cudaGetLastError());
+    } else {
+      gemm_nn(B1, ldn, B1_max, Wt[l + 1], ldl, W[l + 1], ldn, B2, ldl, n, C[l], C[l + 1], img_G[l + 1]);
       Scope sc(this, "zgrad_finish", 1, 16.0 * 4.0 * (double)n * (ldl / 4), 0.0);
       const auto finish = [&](auto kernel) {
         launch(kernel, (unsigned)n_zblocks, 256, 0, (float4*)B2, (const float4*)Z[l], (const float4*)H[l], ldl / 4, d_zblocks, p.nu, red_part, d_comm_block_ptr, comm_tickets, ctl, sums_z,
@@ -787,7 +819,7 @@ struct gcn_admm {
     decide.max_trials = p.bt_max_trials;
     decide.own_nu = p.nu;
     if (l + 1 == L) {   // closed form
-      gemm_nn(B2, ldl, B2_max, W[L], ldn, Wt[L], ldl, B0, ldn, n, C[L], C[l], img_H[L]);   // T = G W_L; S stays in B1
+      if (!joined) gemm_nn(B2, ldl, B2_max, W[L], ldn, Wt[L], ldl, B0, ldn, n, C[L], C[l], img_H[L]);   // T = G W_L; S stays in B1
       decide.mode = 1;
       decide.quad_coef = 0.5 * p.rho;
       gk::SearchOut a{};
@@ -825,7 +857,7 @@ struct gcn_admm {
       CU(cudaGetLastError());
       return;
     }
-    gemm_nn(B2, ldl, B2_max, W[l + 1], ldn, Wt[l + 1], ldl, B1, ldn, n, C[l + 1], C[l], img_H[l + 1]);         // T = G W_{l+1}
+    if (!joined) gemm_nn(B2, ldl, B2_max, W[l + 1], ldn, Wt[l + 1], ldl, B0, ldn, n, C[l + 1], C[l], img_H[l + 1]);   // T = G W_{l+1}
     decide.cand = gk::kCand;   // steady-state searches close at trial 0..2
     decide.scale = 0.5 * p.nu;
     gk::SearchZ a{};
@@ -840,7 +872,7 @@ struct gcn_admm {
     a.log = log_z(l);
     a.Z = (float4*)Z[l]; a.G = (const float4*)B2; a.ldz4 = ldl / 4; a.row_comm = d_row_comm;
     std::snprintf(zname, sizeof zname, "score_z_hidden@%d", ldn);
-    const float4 *T = (const float4*)B1, *Hn = (const float4*)H[l + 1], *Zn = (const float4*)Z[l + 1];
+    const float4 *T = (const float4*)B0, *Hn = (const float4*)H[l + 1], *Zn = (const float4*)Z[l + 1];
     const size_t sums = (size_t)warps * M * gk::kCand * sizeof(double);
     const int use_smem = sums <= 96 * 1024;
     auto score = [&](auto kernel, auto close, int V) {
@@ -1412,7 +1444,7 @@ void create_impl(gcn_admm* h, long long n, const long long* row_ptr, const int* 
   for (int l = 1; l <= L; ++l) {
     h->want_image(h->img_H[l], h->C[l], h->C[l - 1]);   // P_l W_l, G W_l; P_l grad has its shape
     h->want_image(h->img_D[l], h->C[l], h->C[l - 1]);
-    if (l >= 2) h->want_image(h->img_G[l], h->C[l - 1], h->C[l]);
+    if (l >= 2 && !h->joins_products(l - 1)) h->want_image(h->img_G[l], h->C[l - 1], h->C[l]);   // (narrower: k_zgrad_products)
     if (h->by_halves(n, h->C[l], h->C[l - 1])) h->want(h->P_max[l], rows);
   }
   h->want(h->B1_max, rows);

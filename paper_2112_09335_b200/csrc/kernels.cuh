@@ -1272,6 +1272,36 @@ __global__ void k_log_clear(int* __restrict__ trial_base, const int* __restrict_
 // community to finish (tickets[m], left at zero) adds the community's blocks block_ptr[m] .. block_ptr[m+1]-1 up in a
 // fixed order and starts its search.  A group of LPR lanes takes a row; row_max (may be NULL): the largest magnitude of every row of G.
 // ------------------------------------------------------------------------------------------
+// The sums t of row block `block` of community m, and what follows when it is the community's last to finish; the whole block.
+__device__ __forceinline__ void close_zgrad(double (&t)[3], int block, int m, double* sh, double* partial, const int* __restrict__ block_ptr,
+                                            unsigned* tickets, SearchCtl* ctl, double* __restrict__ sums, double shrink, double growth,
+                                            int* n_active, int* status) {
+  __shared__ int s_last;
+  block_sums(t, sh);
+  const int b0 = block_ptr[m], b1 = block_ptr[m + 1];
+  if (threadIdx.x == 0) {
+#pragma unroll
+    for (int j = 0; j < 3; ++j) partial[(size_t)block * 3 + j] = t[j];
+    __threadfence();
+    s_last = atomicAdd(tickets + m, 1u) == (unsigned)(b1 - b0) - 1u;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+#pragma unroll
+  for (int j = 0; j < 3; ++j) t[j] = 0.0;
+  for (int b = b0 + threadIdx.x; b < b1; b += blockDim.x)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) t[j] += __ldcg(partial + (size_t)b * 3 + j);
+  block_sums(t, sh);
+  if (threadIdx.x == 0) {
+    tickets[m] = 0;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) sums[m * 3 + j] = t[j];
+    begin_one(ctl + m, t[0], t[1], shrink, growth, n_active, status);
+  }
+}
+
 template <int LPR>
 __global__ void __launch_bounds__(256)
 k_zgrad_finish(float4* __restrict__ G, const float4* __restrict__ Z, const float4* __restrict__ H, int ld4,
@@ -1279,7 +1309,6 @@ k_zgrad_finish(float4* __restrict__ G, const float4* __restrict__ Z, const float
                SearchCtl* ctl, double* __restrict__ sums, double shrink, double growth, int* n_active, int* status, float* __restrict__ row_max) {
   gtc::enter_kernel();
   __shared__ double sh[24];
-  __shared__ int s_last;
   const int4 rb = blocks[blockIdx.x];
   double t[3] = {0.0, 0.0, 0.0};
   const int sub = threadIdx.x & (LPR - 1);
@@ -1306,28 +1335,86 @@ k_zgrad_finish(float4* __restrict__ G, const float4* __restrict__ Z, const float
       if (sub == 0 && row < rb.y) row_max[row] = big;
     }
   }
-  block_sums(t, sh);
-  const int m = rb.z, b0 = block_ptr[m], b1 = block_ptr[m + 1];
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int j = 0; j < 3; ++j) partial[(size_t)blockIdx.x * 3 + j] = t[j];
-    __threadfence();
-    s_last = atomicAdd(tickets + m, 1u) == (unsigned)(b1 - b0) - 1u;
-  }
+  close_zgrad(t, (int)blockIdx.x, rb.z, sh, partial, block_ptr, tickets, ctl, sums, shrink, growth, n_active, status);
+}
+
+// The same with both products beside it, for a narrow next layer: G[i] = S[i] W^T + nu (Z[i] - f(H[i])) and T[i] = G[i] W are rows of
+// their own, so that G is written once and not read again (three launches and G through memory three times otherwise).  fp32 FMA.
+// W^T lies in shared memory, 4 KV rows of ld4 float4 (those past the layer's width zero).  Eight lanes take R rows of G, so that a
+// value of W serves R; shared memory is read 4 KV times per R float4 of G for each product, which with the registers of a row's S
+// and T is what bounds it where HBM does not (see the rule in update_Z_hidden).
+template <int KV, int R>
+__global__ void __launch_bounds__(256 / R)
+k_zgrad_products(float4* __restrict__ G, const float4* __restrict__ Z, const float4* __restrict__ H, const float4* __restrict__ S,
+                 const float4* __restrict__ Wt, float4* __restrict__ T, int ld4, int next_cols, const int4* __restrict__ blocks,
+                 int n_blocks, float nu, double* partial, const int* __restrict__ block_ptr, unsigned* tickets, SearchCtl* ctl,
+                 double* __restrict__ sums, double shrink, double growth, int* n_active, int* status) {
+  gtc::enter_kernel();
+  extern __shared__ float4 s_wt[];
+  __shared__ double sh[24];
+  for (int i = threadIdx.x; i < 4 * KV * ld4; i += blockDim.x) s_wt[i] = i < next_cols * ld4 ? Wt[i] : make_float4(0.f, 0.f, 0.f, 0.f);
   __syncthreads();
-  if (!s_last) return;
-  __threadfence();
+  const int sub = threadIdx.x & 7, group = threadIdx.x >> 3, next4 = (next_cols + 3) / 4;
+  for (int blk = blockIdx.x; blk < n_blocks; blk += gridDim.x) {
+    const int4 rb = blocks[blk];
+    double t[3] = {0.0, 0.0, 0.0};
+    const int row = rb.x + R * group;   // the first of this group's rows: a block has R for each of its groups
+    bool in[R];
+    float s[R][4 * KV], out[R][4 * KV];
 #pragma unroll
-  for (int j = 0; j < 3; ++j) t[j] = 0.0;
-  for (int b = b0 + threadIdx.x; b < b1; b += blockDim.x)
+    for (int j = 0; j < R; ++j) {
+      in[j] = row + j < rb.y;
 #pragma unroll
-    for (int j = 0; j < 3; ++j) t[j] += __ldcg(partial + (size_t)b * 3 + j);
-  block_sums(t, sh);
-  if (threadIdx.x == 0) {
-    tickets[m] = 0;
+      for (int k = 0; k < KV; ++k) {
+        const float4 v = in[j] && k < next4 ? S[(long long)(row + j) * next4 + k] : make_float4(0.f, 0.f, 0.f, 0.f);
+        s[j][4 * k] = v.x; s[j][4 * k + 1] = v.y; s[j][4 * k + 2] = v.z; s[j][4 * k + 3] = v.w;
+        out[j][4 * k] = out[j][4 * k + 1] = out[j][4 * k + 2] = out[j][4 * k + 3] = 0.f;
+      }
+    }
+    for (int f = sub; f < ld4; f += 8) {
+      float4 z[R], h[R], g[R];
 #pragma unroll
-    for (int j = 0; j < 3; ++j) sums[m * 3 + j] = t[j];
-    begin_one(ctl + m, t[0], t[1], shrink, growth, n_active, status);
+      for (int j = 0; j < R; ++j) {
+        z[j] = h[j] = g[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (in[j]) { z[j] = Z[(long long)(row + j) * ld4 + f]; h[j] = H[(long long)(row + j) * ld4 + f]; }
+      }
+#pragma unroll
+      for (int k = 0; k < 4 * KV; ++k) {
+        const float4 w = s_wt[k * ld4 + f];
+#pragma unroll
+        for (int j = 0; j < R; ++j) g[j] = vfma(s[j][k], w, g[j]);
+      }
+#pragma unroll
+      for (int j = 0; j < R; ++j) {
+        const float ax = z[j].x - relu(h[j].x), ay = z[j].y - relu(h[j].y), az = z[j].z - relu(h[j].z), aw = z[j].w - relu(h[j].w);
+        g[j].x = fmaf(nu, ax, g[j].x); g[j].y = fmaf(nu, ay, g[j].y); g[j].z = fmaf(nu, az, g[j].z); g[j].w = fmaf(nu, aw, g[j].w);
+        if (in[j]) G[(long long)(row + j) * ld4 + f] = g[j];
+        t[0] += (double)(g[j].x * g[j].x + g[j].y * g[j].y + g[j].z * g[j].z + g[j].w * g[j].w);
+        t[1] += (double)(z[j].x * z[j].x + z[j].y * z[j].y + z[j].z * z[j].z + z[j].w * z[j].w);
+        t[2] += (double)(ax * g[j].x + ay * g[j].y + az * g[j].z + aw * g[j].w);
+      }
+#pragma unroll
+      for (int k = 0; k < 4 * KV; ++k) {
+        const float4 w = s_wt[k * ld4 + f];
+#pragma unroll
+        for (int j = 0; j < R; ++j)
+          out[j][k] = fmaf(g[j].w, w.w, fmaf(g[j].z, w.z, fmaf(g[j].y, w.y, fmaf(g[j].x, w.x, out[j][k]))));
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < R; ++j)
+#pragma unroll
+      for (int k = 0; k < 4 * KV; ++k)
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) out[j][k] += __shfl_xor_sync(0xffffffffu, out[j][k], o);
+#pragma unroll
+    for (int j = 0; j < R; ++j)
+#pragma unroll
+      for (int k = 0; k < KV; ++k)
+        if (in[j] && k < next4 && sub == ((j * KV + k) & 7))
+          T[(long long)(row + j) * next4 + k] = make_float4(out[j][4 * k], out[j][4 * k + 1], out[j][4 * k + 2], out[j][4 * k + 3]);
+    close_zgrad(t, blk, rb.z, sh, partial, block_ptr, tickets, ctl, sums, shrink, growth, n_active, status);
+    __syncthreads();   // its shared memory is free again
   }
 }
 
