@@ -465,9 +465,9 @@ struct gcn_admm {
     } else if (ld4 <= 8) {
       if (VEC == 4 && lanes <= 160000) SETS_OF(2, 4, 4, 4); else if (lanes <= 480000) SETS(8, 4, 8); else SETS(8, 1, 8);
     } else if (VEC == 4 && ld4 <= 12) {
-      // four lanes of three vectors leave none idle (us, against 16 lanes: 13.0 -> 11.0 at 12 k rows, 76 -> 63 at 169 k, 2469 -> 2149
-      // at 2.45 M); of twelve single floats, for a matrix of odd width, they are slower (13.6 -> 17.4 at 10 k rows)
-      if (lanes <= 640000) SETS_OF(3, 4, 4, 4); else SETS_OF(3, 4, 2, 4);
+      // four lanes of three vectors leave none idle (us, against 16 lanes: 76 -> 65 at 169 k rows, 2469 -> 2115 at 2.45 M); of twelve
+      // single floats, for a matrix of odd width, they are slower.  As many sets as there: all layouts of a width agree bit for bit.
+      if (lanes <= 960000) SETS_OF(3, 4, 2, 4); else SETS_OF(3, 4, 1, 4);
     } else if (ld4 <= 16) {
       if (lanes <= 960000) SETS(16, 2, 8); else SETS(16, 1, 8);
     } else if (ld4 <= 32) WIDE(1, 4, false);

@@ -322,7 +322,7 @@ k_spmm_long_rows(const int4* __restrict__ rows, const T* __restrict__ scratch, T
 // Narrow operands.  G = CL * EP lanes share a row: CL of them side by side over its columns (NV vectors each), EP
 // such sets over its stored entries (entry e goes to set (e - first) mod EP), so that a row of k entries costs
 // k / EP dependent steps instead of k and a narrow row still fills the lanes of a warp; a shuffle tree adds the
-// sets at the end.  The order of a row's sum depends on EP alone.
+// sets at the end.  The order of a row's sum depends on EP alone: all layouts of a width agree bit for bit.
 // CL <= 4: every lane loads column and weight of its own entries (one word for the CL lanes of a set), one step
 // ahead of the operand rows.  CL >= 8: the G lanes load one entry each, columns two groups ahead and weights one,
 // and hand them to the sets by shuffles (with more lanes per set the repeated loads cost more than the shuffles).
