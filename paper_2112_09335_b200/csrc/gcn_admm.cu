@@ -576,14 +576,13 @@ struct gcn_admm {
   bool tn_on_tensor_cores(long long rows) const { return p.tensor_cores != 0 && rows >= 4096; }
 
   // part_max (tensor-core form only): raised to the largest magnitude among the partial sums, as bits.
-  // With `zres` (tensor-core form only) B holds pre-activations H and the operand is
+  // With `zres` B holds pre-activations H and the operand is
   // h > 0 ? nu (h - z) : 0, formed while staging: the residual matrix is never stored.
   int gemm_tn(const float* A, int lda, const float* B, int ldb, int ldp, long long rows, int Ka, int Nb,
               const float* zres = nullptr, float nu = 0.f, unsigned* part_max = nullptr) {
     int splits = 1;
     long long rps = rows;
     char name[48];
-    if (zres && !tn_on_tensor_cores(rows)) throw Fail{GCN_ADMM_ERR_ARG, "fused residual needs the tensor-core product"};
     if (tn_on_tensor_cores(rows)) {
       std::snprintf(name, sizeof name, zres ? "gemm_tn_tc.resid@%dx%d" : "gemm_tn_tc@%dx%d", Ka, Nb);
       Scope sc(this, name, 1, 4.0 * ((double)rows * (lda + (zres ? 2 : 1) * ldb) + (double)Ka * ldp), 2.0 * (double)rows * Ka * Nb);
@@ -623,8 +622,8 @@ struct gcn_admm {
       CU(cudaGetLastError());
       return splits;
     }
-    std::snprintf(name, sizeof name, "gemm_tn@%dx%d", Ka, Nb);
-    Scope sc(this, name, 1, 4.0 * ((double)rows * (lda + ldb) + (double)Ka * ldp), 2.0 * (double)rows * Ka * Nb);
+    std::snprintf(name, sizeof name, zres ? "gemm_tn.resid@%dx%d" : "gemm_tn@%dx%d", Ka, Nb);
+    Scope sc(this, name, 1, 4.0 * ((double)rows * (lda + (zres ? 2 : 1) * ldb) + (double)Ka * ldp), 2.0 * (double)rows * Ka * Nb);
 #define TN_CASE(BM, BN, BK, TM, TN)                                                             \
   {                                                                                             \
     const long long tiles = cdiv(Ka, BM) * cdiv(ldp, BN);                                        \
@@ -633,7 +632,8 @@ struct gcn_admm {
     rps = cdiv(rows, splits);                                                                    \
     splits = (int)cdiv(rows, rps);                                                               \
     dim3 grid((unsigned)cdiv(Ka, BM), (unsigned)cdiv(ldp, BN), (unsigned)splits);                \
-    launch_alone(gk::k_gemm_tn<BM, BN, BK, TM, TN>, grid, (BM / TM) * (BN / TN), 0, A, lda, B, ldb, part, ldp, rows, rps, Ka, Nb); \
+    if (zres) launch_alone(gk::k_gemm_tn<BM, BN, BK, TM, TN, true>, grid, (BM / TM) * (BN / TN), 0, A, lda, B, ldb, part, ldp, rows, rps, Ka, Nb, zres, nu); \
+    else launch_alone(gk::k_gemm_tn<BM, BN, BK, TM, TN, false>, grid, (BM / TM) * (BN / TN), 0, A, lda, B, ldb, part, ldp, rows, rps, Ka, Nb, nullptr, 0.f); \
   }
     if (Nb > 64) TN_CASE(128, 128, 16, 8, 8)
     else if (Nb > 16) TN_CASE(128, 64, 16, 8, 4)
@@ -715,7 +715,7 @@ struct gcn_admm {
     SearchCtl* ctl = ctl_w + l;
     float *const R = resid_of(l), *const D = l == L && DL != nullptr ? DL : B1;
     int splits;
-    if (l < L && tn_on_tensor_cores(n)) {                               // grad = P_l^T R_l, R_l formed inside the product
+    if (l < L) {                                                        // grad = P_l^T R_l, R_l formed inside the product
       splits = gemm_tn(P[l], ld[l - 1], H[l], ldc, ldc, n, Kp, Cn, Z[l], p.nu, &ctl->part_max);
     } else {
       resid(l, R);                                                      // R_l

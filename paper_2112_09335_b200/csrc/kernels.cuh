@@ -600,12 +600,24 @@ k_gemm_nn(const float* __restrict__ A, int lda, const float* __restrict__ B, int
   }
 }
 
+// Residuals with respect to the pre-activation H (derivatives of phi, Section 3):
+//   hidden layer  R = nu (f(H) - Z) * f'(H)
+//   last layer    R = -(U + rho (Z - H))
+__device__ __forceinline__ float4 resid_hidden(const float4& h, const float4& z, float nu) {
+  return make_float4(h.x > 0.f ? nu * (h.x - z.x) : 0.f, h.y > 0.f ? nu * (h.y - z.y) : 0.f,
+                     h.z > 0.f ? nu * (h.z - z.z) : 0.f, h.w > 0.f ? nu * (h.w - z.w) : 0.f);
+}
+__device__ __forceinline__ float4 resid_out(const float4& h, const float4& z, const float4& u, float rho) {
+  return make_float4(-(u.x + rho * (z.x - h.x)), -(u.y + rho * (z.y - h.y)), -(u.z + rho * (z.z - h.z)), -(u.w + rho * (z.w - h.w)));
+}
+
+// RESID: B is not stored; it is the hidden layer's R, formed from H (passed as B) and Z (Zres) as they are loaded.
 // part[(split * Ka + ka) * ldp + nb].  A: rows x Ka (lda), B: rows x Nb (ldb).
 // Split s owns rows [s * rows_per_split, min(rows, (s+1) * rows_per_split)).
-template <int BM, int BN, int BK, int TM, int TN>
+template <int BM, int BN, int BK, int TM, int TN, bool RESID>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN), 2)
 k_gemm_tn(const float* __restrict__ A, int lda, const float* __restrict__ B, int ldb,
-          float* __restrict__ part, int ldp, long long rows, long long rows_per_split, int Ka, int Nb) {
+          float* __restrict__ part, int ldp, long long rows, long long rows_per_split, int Ka, int Nb, const float* __restrict__ Zres, float nu) {
   constexpr int NT = (BM / TM) * (BN / TN);
   constexpr int TX = BN / TN;
   constexpr int A_F4 = BK * BM / 4, B_F4 = BK * BN / 4;
@@ -649,6 +661,7 @@ k_gemm_tn(const float* __restrict__ A, int lda, const float* __restrict__ B, int
         const int gc = b0 + c;
         if (gr < r_end && gc < Nb) {
           v = *reinterpret_cast<const float4*>(B + gr * ldb + gc);
+          if (RESID) v = resid_hidden(v, *reinterpret_cast<const float4*>(Zres + gr * ldb + gc), nu);
           if (gc + 1 >= Nb) v.y = 0.f;
           if (gc + 2 >= Nb) v.z = 0.f;
           if (gc + 3 >= Nb) v.w = 0.f;
@@ -735,18 +748,8 @@ k_gemm_tn(const float* __restrict__ A, int lda, const float* __restrict__ B, int
 }
 
 // ------------------------------------------------------------------------------------------
-// Residuals with respect to the pre-activation H (derivatives of phi, Section 3):
-//   hidden layer  R = nu (f(H) - Z) * f'(H)
-//   last layer    R = -(U + rho (Z - H))
+// Residuals where they are stored.
 // ------------------------------------------------------------------------------------------
-__device__ __forceinline__ float4 resid_hidden(const float4& h, const float4& z, float nu) {
-  return make_float4(h.x > 0.f ? nu * (h.x - z.x) : 0.f, h.y > 0.f ? nu * (h.y - z.y) : 0.f,
-                     h.z > 0.f ? nu * (h.z - z.z) : 0.f, h.w > 0.f ? nu * (h.w - z.w) : 0.f);
-}
-__device__ __forceinline__ float4 resid_out(const float4& h, const float4& z, const float4& u, float rho) {
-  return make_float4(-(u.x + rho * (z.x - h.x)), -(u.y + rho * (z.y - h.y)), -(u.z + rho * (z.z - h.z)), -(u.w + rho * (z.w - h.w)));
-}
-
 __global__ void k_resid_hidden(const float4* __restrict__ H, const float4* __restrict__ Z,
                                float4* __restrict__ R, long long n4, float nu) {
   gtc::enter_kernel();
@@ -1352,11 +1355,12 @@ k_zgrad_products(float4* __restrict__ G, const float4* __restrict__ Z, const flo
   gtc::enter_kernel();
   extern __shared__ float4 s_wt[];
   __shared__ double sh[24];
+  int4 rb = blocks[blockIdx.x];   // beside the first loads of W
   for (int i = threadIdx.x; i < 4 * KV * ld4; i += blockDim.x) s_wt[i] = i < next_cols * ld4 ? Wt[i] : make_float4(0.f, 0.f, 0.f, 0.f);
   __syncthreads();
   const int sub = threadIdx.x & 7, group = threadIdx.x >> 3, next4 = (next_cols + 3) / 4;
   for (int blk = blockIdx.x; blk < n_blocks; blk += gridDim.x) {
-    const int4 rb = blocks[blk];
+    if (blk != (int)blockIdx.x) rb = blocks[blk];
     double t[3] = {0.0, 0.0, 0.0};
     const int row = rb.x + R * group;   // the first of this group's rows: a block has R for each of its groups
     bool in[R];
@@ -2026,17 +2030,22 @@ __device__ __forceinline__ float4 add_sets(float4 k) {
   return k;
 }
 
+// The next chunk of a sweep whose `warps` warps began with one each.
+__device__ __forceinline__ int next_chunk(int* counter, int warps, int lane) {
+  int ch = 0;
+  if (lane == 0) ch = warps + atomicAdd(counter, 1);
+  return __shfl_sync(0xffffffffu, ch, 0);
+}
+
 template <int CL>
 __global__ void __launch_bounds__(256, 3)
 k_search_z_out(const int* __restrict__ col, const float* __restrict__ dinv, const float4* __restrict__ T, const float4* __restrict__ S,
                int ld4, float4* scratch, const SearchOut p) {
   constexpr int GROUPS = 32 / CL;
   const int lane = threadIdx.x & 31, grp = lane / CL, cl = lane & (CL - 1);
-  for (;;) {
-    int ch = 0;
-    if (lane == 0) ch = atomicAdd(p.chunk_counter, 1);
-    ch = __shfl_sync(0xffffffffu, ch, 0);
-    if (ch >= p.n_chunks) return;
+  // every warp's first chunk is its own number, the others come from the counter
+  const int warps = (int)(gridDim.x * (blockDim.x >> 5));
+  for (int ch = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); ch < p.n_chunks; ch = next_chunk(p.chunk_counter, warps, lane)) {
     const SegChunk c = p.chunks[ch];
     if (__ldcg(&p.ctl[c.comm].done)) continue;   // skipped: none of its slots is filled
     double lin = 0.0, quad = 0.0;
