@@ -282,6 +282,49 @@ class Stage {
     return e;
   }
 
+  // Device -> host: `count` dense arrays one after the other, the bus moving on to the next while the host still empties the parts of
+  // the one before.  Returns with the host buffers filled.
+  struct Part {
+    void* dst;
+    const void* src;
+    std::size_t bytes;
+  };
+  cudaError_t get_all(const Part* parts, int count, cudaStream_t stream) {
+    if (const cudaError_t e = flush(stream)) return e;
+    bool direct = false;
+    int p_begun = 0, p_done = 0;             // array and offset of the next piece to start and of the next to empty
+    std::size_t at_begun = 0, at_done = 0, begun = 0, done = 0;
+    const auto staged = [&](int p) { return parts[p].bytes > 0 && !(parts[p].bytes >= kSlot / 4 && page_locked(parts[p].dst)); };
+    for (int p = 0; p < count; ++p)
+      if (parts[p].bytes > 0 && !staged(p)) {
+        direct = true;
+        if (const cudaError_t e = cudaMemcpyAsync(parts[p].dst, parts[p].src, parts[p].bytes, cudaMemcpyDeviceToHost, stream)) return e;
+      }
+    const auto skip = [&](int& p) { while (p < count && !staged(p)) ++p; };
+    skip(p_begun);
+    skip(p_done);
+    while (p_done < count) {
+      while (p_begun < count && begun < done + kSlots) {
+        const std::size_t k = (slot_ + begun) % kSlots, len = std::min(kSlot, parts[p_begun].bytes - at_begun);
+        cudaError_t e = cudaEventSynchronize(used_[k]);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(base_ + k * kSlot, static_cast<const char*>(parts[p_begun].src) + at_begun, len, cudaMemcpyDeviceToHost, stream);
+        if (e == cudaSuccess) e = cudaEventRecord(used_[k], stream);
+        if (e != cudaSuccess) return e;
+        ++begun;
+        at_begun += len;
+        if (at_begun == parts[p_begun].bytes) { at_begun = 0; ++p_begun; skip(p_begun); }
+      }
+      const std::size_t k = (slot_ + done) % kSlots, len = std::min(kSlot, parts[p_done].bytes - at_done);
+      if (const cudaError_t e = cudaEventSynchronize(used_[k])) return e;
+      copy_bytes(static_cast<char*>(parts[p_done].dst) + at_done, base_ + k * kSlot, len);
+      ++done;
+      at_done += len;
+      if (at_done == parts[p_done].bytes) { at_done = 0; ++p_done; skip(p_done); }
+    }
+    slot_ = (int)((slot_ + done) % kSlots);
+    return direct ? cudaStreamSynchronize(stream) : cudaSuccess;
+  }
+
   // Device -> host: `rows` rows of `width` bytes, `pitch` bytes apart on the device, dense on the host.  Returns with the
   // host buffer filled.
   cudaError_t get(void* dst, const void* src, std::size_t width, std::size_t pitch, std::size_t rows, cudaStream_t stream) {

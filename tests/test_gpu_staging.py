@@ -97,3 +97,34 @@ def test_idle_memory_goes_back_on_request():
     live.step(1)
     assert np.isfinite(live.objective()).all()
     live.destroy()
+
+
+@pytest.mark.parametrize("n,classes", [(70, 3), (1598, 40), (1599, 40), (30000, 35), (40000, 104)])   # either side of 256 KB together, one part and a bit, five
+@pytest.mark.parametrize("pinned", [False, True])
+def test_predictions_together_and_apart(n, classes, pinned):
+    """Labels and logits in one call, either alone, into pageable and page-locked memory: the same values."""
+    import torch
+    pr = tiny_problem(73, n=min(n, 2000), widths=(5, 6, classes), n_comm=4, p=0.002)
+    if n > 2000:                                    # a ring: a dense adjacency of that size would not fit
+        pr["n"] = n
+        pr["row_ptr"] = np.arange(0, 2 * n + 1, 2, dtype=np.int64)
+        i = np.arange(n)
+        pr["col_idx"] = np.sort(np.stack([(i - 1) % n, (i + 1) % n], 1), 1).reshape(-1).astype(np.int32)
+        rng = np.random.default_rng(1)
+        pr["X"], pr["y"], pr["community"] = rng.standard_normal((n, 5)), rng.integers(0, classes, n), rng.integers(0, 4, n)
+        pr["mask"] = (rng.random(n) < 0.3).astype(np.uint8)
+    g = handle(pr)
+    try:
+        lib = binding.load()
+        def buf(shape, dt):
+            t = torch.full(shape, -1, dtype=dt)
+            return (t.pin_memory() if pinned else t).numpy()
+        logits, labels = buf((n, classes), torch.float32), buf((n,), torch.int32)
+        assert lib.gcn_admm_predict(g._h, binding._ptr(logits), binding._ptr(labels)) == 0
+        assert np.array_equal(labels, logits.argmax(axis=1))
+        only = buf((n, classes), torch.float32), buf((n,), torch.int32)
+        assert lib.gcn_admm_predict(g._h, binding._ptr(only[0]), None) == 0 and lib.gcn_admm_predict(g._h, None, binding._ptr(only[1])) == 0
+        assert np.array_equal(only[0], logits) and np.array_equal(only[1], labels)
+        assert abs(g.objective()[5] - (labels == pr["y"])[pr["mask"] != 0].mean()) < 1e-12
+    finally:
+        g.destroy()
