@@ -602,7 +602,7 @@ struct gcn_admm {
       splits = (int)cdiv(rows, rps);
 #define TN_TC(NT)                                                                                              \
   {                                                                                                            \
-    const size_t smem = gtc::TnCfg<NT>::kSmem;                                                                 \
+    const size_t smem = zres ? gtc::TnCfg<NT, true>::kSmem : gtc::TnCfg<NT, false>::kSmem;                     \
     dim3 grid((unsigned)groups, (unsigned)splits, (unsigned)nb_groups);                                        \
     if (zres) {                                                                                                \
       CU(cudaFuncSetAttribute(gtc::k_gemm_tn_tc<NT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \

@@ -470,9 +470,9 @@ k_gemm_tc_ws(const float* __restrict__ A, int lda, const float* __restrict__ Bk,
 // A[r,:]^T B[r,:]  (the weight gradient P^T R, reduction over the node dimension).
 // Here the reduction index r is the MMA's K, and both operands are stored with their own index
 // (ka, nb) contiguous: "MN-major" operands, for which 32-bit elements have exactly one shared-memory
-// form: 128-byte rows swizzled at 32-byte granularity.  A chunk is 32 rows; atom (g, q) holds rows
+// form: 128-byte rows swizzled at 32-byte granularity.  A chunk is 16 or 32 rows; atom (g, q) holds rows
 // 4q..4q+3 of column group g (32 columns = 128 bytes per row), 512 bytes, and inside it the 32-byte
-// unit u of row r sits at unit u ^ (r mod 4); successive column groups are 4096 bytes apart (the
+// unit u of row r sits at unit u ^ (r mod 4); successive column groups are 128 bytes per row of the chunk apart (the
 // descriptor's leading byte offset), successive groups of 4 rows 512 bytes apart (its stride byte
 // offset).  One MMA consumes 8 rows (K = 8), i.e. two atoms.  Same hi/lo split, same separate correction accumulator, same roles as
 // above (8 producer warps, one MMA warp); a CTA owns 128 columns of A (blockIdx.x), NT columns of B
@@ -481,46 +481,54 @@ k_gemm_tc_ws(const float* __restrict__ A, int lda, const float* __restrict__ Bk,
 // together, and the second one finds them in L2.
 // ------------------------------------------------------------------------------------------------
 constexpr int kTnThreads = 9 * 32;
-constexpr int kTnRows = 32;                       // rows (reduction steps) per chunk
 
-// MN-major tile: LBO = 4096, SBO = 512, version 1, 128-byte swizzle with 32-byte base (low / high word as above)
+// MN-major tile: LBO = bytes of a column group, SBO = 512, version 1, 128-byte swizzle with 32-byte base (low / high word as above)
 constexpr uint32_t kOperandDescMnHi = (512u >> 4) | (1u << 14) | (1u << 29);
-__device__ __forceinline__ uint32_t operand_desc_mn_lo(uint32_t smem_addr) { return ((smem_addr >> 4) & 0x3fffu) | ((4096u >> 4) << 16); }
+template <int GROUP>
+__device__ __forceinline__ uint32_t operand_desc_mn_lo(uint32_t smem_addr) { return ((smem_addr >> 4) & 0x3fffu) | ((uint32_t)(GROUP >> 4) << 16); }
 __device__ __forceinline__ uint32_t instr_desc_mn(int nt) {
   return (1u << 4) | (2u << 7) | (2u << 10) | (1u << 15) | (1u << 16) | ((uint32_t)(nt >> 3) << 17) |
          ((uint32_t)(kBlockM >> 4) << 24);
 }
-// byte offset of float4 number c4 (columns 4 c4 .. 4 c4 + 3) of chunk row r in an MN-major tile
+// byte offset of float4 number c4 (columns 4 c4 .. 4 c4 + 3) of chunk row r in an MN-major tile of column groups of GROUP bytes
+template <int GROUP>
 __device__ __forceinline__ uint32_t swz_mn(int r, int c4) {
-  return (uint32_t)(c4 >> 3) * 4096u + (uint32_t)(r >> 2) * 512u + (uint32_t)(r & 3) * 128u +
+  return (uint32_t)(c4 >> 3) * (uint32_t)GROUP + (uint32_t)(r >> 2) * 512u + (uint32_t)(r & 3) * 128u +
          (uint32_t)(((((c4 & 7) >> 1) ^ (r & 3)) << 5) | ((c4 & 1) << 4));
 }
 
-template <int NT>
+// The producers are bound by the latency of their loads: what counts is the bytes they hold in flight, in registers.  Chunks of 32
+// rows, several ahead, where a row is short; of 16 rows where it is long (the same registers hold more of them: three chunks of
+// 16 rows where two of 32 spilled).  1.2 M rows, chunks of 32 and one (R) or two (P) ahead before: 256 x 256 with R formed
+// 1084 -> 934 us, 128 x 256 579 -> 512, 256 x 128 722 -> 615, 126 x 51 294 -> 229; 256 x 47 without 517 -> 394, 128 x 11 243 -> 191
+// (from HBM alone 564, 470, 376, 167; 222, 102).
+template <int NT, bool RESID>
 struct TnCfg {
+  static constexpr int kRows = NT >= 128 ? 16 : 32;       // rows (reduction steps) per chunk
+  static constexpr int kAhead = NT > 128 ? (RESID ? 3 : 4) : NT > 64 ? (RESID ? 4 : 6) : 4;   // chunks held in registers
+  static constexpr int kGroup = kRows * 128;              // bytes of a group of 32 columns
   static constexpr int kGroupsB = (NT + 31) / 32;
-  static constexpr int kATile = 4 * 4096;                 // 128 columns x 32 rows, one of hi / lo
-  static constexpr int kBTile = kGroupsB * 4096;
+  static constexpr int kATile = 4 * kGroup;               // 128 columns, one of hi / lo
+  static constexpr int kBTile = kGroupsB * kGroup;
   static constexpr int kStage = 2 * kATile + 2 * kBTile;
-  static constexpr int kStagesTn = kStage > 72 * 1024 ? 2 : 3;
+  static constexpr int kStagesTn = kStage > 72 * 1024 ? 2 : kStage > 50 * 1024 ? 3 : kStage > 40 * 1024 ? 4 : 5;
   static constexpr uint32_t kTmemCols = 2 * NT <= 32 ? 32 : 2 * NT <= 64 ? 64 : 2 * NT <= 128 ? 128 : 2 * NT <= 256 ? 256 : 512;
   static constexpr size_t kSmem = (size_t)kStagesTn * kStage + 1024;
 };
 
 // RESID: B is not stored.  The operand is the derivative of a hidden layer's penalty with respect to
 // its pre-activation, formed while staging from the pre-activation H (passed as B) and the layer's
-// Z (Zres, same leading dimension):  b = h > 0 ? nu (h - z) : 0.  Both rows are fetched one chunk
-// ahead (A stays two chunks ahead), so the second matrix costs no further registers.
+// Z (Zres, same leading dimension):  b = h > 0 ? nu (h - z) : 0.
 // part_max (may be NULL): raised to the largest magnitude among the partial sums.
 template <int NT, bool RESID>
 __global__ void __launch_bounds__(kTnThreads, 1)
 k_gemm_tn_tc(const float* __restrict__ A, int lda, const float* __restrict__ B, int ldb, float* __restrict__ part, int ldp,
              long long rows, long long rows_per_split, int Ka, int Nb, int* __restrict__ error_flag,
              const float* __restrict__ Zres, float nu, unsigned* part_max) {
-  using Cfg = TnCfg<NT>;
-  constexpr int S = Cfg::kStagesTn;
-  constexpr int A_PASSES = 4;                              // 1024 float4 / 256 threads
-  constexpr int B_F4 = kTnRows * (NT / 4);
+  using Cfg = TnCfg<NT, RESID>;
+  constexpr int S = Cfg::kStagesTn, ROWS = Cfg::kRows, GROUP = Cfg::kGroup;
+  constexpr int A_PASSES = ROWS * 32 / 256;
+  constexpr int B_F4 = ROWS * (NT / 4);
   constexpr int B_PASSES = (B_F4 + 255) / 256;
   static_assert(NT % 16 == 0 && NT <= 256, "NT");
 
@@ -554,16 +562,17 @@ k_gemm_tn_tc(const float* __restrict__ A, int lda, const float* __restrict__ B, 
 
   const long long r_begin = (long long)blockIdx.y * rows_per_split;
   const long long r_end = min(rows, r_begin + rows_per_split);
-  const int total = r_end > r_begin ? (int)((r_end - r_begin + kTnRows - 1) / kTnRows) : 0;
+  const int total = r_end > r_begin ? (int)((r_end - r_begin + ROWS - 1) / ROWS) : 0;
   const int ka0 = blockIdx.x * kBlockM;
   const int nb0 = blockIdx.z * NT;                 // first column of B (and of the partial sum) of this CTA
 
   if (warp < 8) {
     // ---------------- producers ----------------
-    float4 ra[2][A_PASSES], rb[2][B_PASSES];
+    constexpr int AHEAD = Cfg::kAhead;
+    float4 ra[AHEAD][A_PASSES], rb[AHEAD][B_PASSES], rz[RESID ? AHEAD : 1][B_PASSES];
     auto load_a = [&](int j, float4* pa) {
       if (j >= total) return;
-      const long long r0 = r_begin + (long long)j * kTnRows;
+      const long long r0 = r_begin + (long long)j * ROWS;
 #pragma unroll
       for (int i = 0; i < A_PASSES; ++i) {
         const int f = tid + 256 * i, rr = f >> 5, c4 = f & 31;
@@ -576,7 +585,7 @@ k_gemm_tn_tc(const float* __restrict__ A, int lda, const float* __restrict__ B, 
     };
     auto load_b = [&](int j, const float* __restrict__ src, float4* pb) {
       if (j >= total) return;
-      const long long r0 = r_begin + (long long)j * kTnRows;
+      const long long r0 = r_begin + (long long)j * ROWS;
 #pragma unroll
       for (int i = 0; i < B_PASSES; ++i) {
         const int f = tid + 256 * i;
@@ -595,7 +604,7 @@ k_gemm_tn_tc(const float* __restrict__ A, int lda, const float* __restrict__ B, 
         float4 h, l;
         split_tf32(pa[i].x, h.x, l.x); split_tf32(pa[i].y, h.y, l.y);
         split_tf32(pa[i].z, h.z, l.z); split_tf32(pa[i].w, h.w, l.w);
-        const uint32_t off = swz_mn(rr, c4);
+        const uint32_t off = swz_mn<GROUP>(rr, c4);
         *reinterpret_cast<float4*>(st + off) = h;
         *reinterpret_cast<float4*>(st + Cfg::kATile + off) = l;
       }
@@ -615,35 +624,33 @@ k_gemm_tn_tc(const float* __restrict__ A, int lda, const float* __restrict__ B, 
           float4 h, l;
           split_tf32(b.x, h.x, l.x); split_tf32(b.y, h.y, l.y);
           split_tf32(b.z, h.z, l.z); split_tf32(b.w, h.w, l.w);
-          const uint32_t off = swz_mn(rr, c4);
+          const uint32_t off = swz_mn<GROUP>(rr, c4);
           *reinterpret_cast<float4*>(st + 2 * Cfg::kATile + off) = h;
           *reinterpret_cast<float4*>(st + 2 * Cfg::kATile + Cfg::kBTile + off) = l;
         }
       }
     };
-    load_a(0, ra[0]);
-    load_a(1, ra[1]);
-    if (RESID) {   // rb[0] = rows of H, rb[1] = rows of Z, both of the next chunk
-      load_b(0, B, rb[0]);
-      load_b(0, Zres, rb[1]);
-    } else {
-      load_b(0, B, rb[0]);
-      load_b(1, B, rb[1]);
-    }
-    for (int j = 0; j < total; ++j) {
-      const int stage = j % S;
-      if (j >= S && !__all_sync(0xffffffffu, mbar_wait_abortable(bar_empty + 8 * stage, ((j / S) - 1) & 1, abortp))) break;
-      if (RESID) {
-        if (j & 1) { store_chunk(stage, ra[1], rb[0], rb[1]); load_a(j + 2, ra[1]); }
-        else       { store_chunk(stage, ra[0], rb[0], rb[1]); load_a(j + 2, ra[0]); }
-        load_b(j + 1, B, rb[0]);
-        load_b(j + 1, Zres, rb[1]);
-      } else {
-        if (j & 1) { store_chunk(stage, ra[1], rb[1], nullptr); load_a(j + 2, ra[1]); load_b(j + 2, B, rb[1]); }
-        else       { store_chunk(stage, ra[0], rb[0], nullptr); load_a(j + 2, ra[0]); load_b(j + 2, B, rb[0]); }
+    auto load = [&](int j, int d) {
+      load_a(j, ra[d]);
+      load_b(j, B, rb[d]);
+      if (RESID) load_b(j, Zres, rz[RESID ? d : 0]);
+    };
+#pragma unroll
+    for (int d = 0; d < AHEAD; ++d) load(d, d);
+    int stage = 0;
+    uint32_t empty_parity = 1;   // a fresh barrier passes a wait on parity 1
+    bool stop = false;
+    for (int j0 = 0; j0 < total && !stop; j0 += AHEAD) {
+#pragma unroll
+      for (int d = 0; d < AHEAD; ++d) {
+        if (j0 + d >= total) break;
+        if (!__all_sync(0xffffffffu, mbar_wait_abortable(bar_empty + 8 * stage, empty_parity, abortp))) { stop = true; break; }
+        store_chunk(stage, ra[d], rb[d], rz[RESID ? d : 0]);
+        load(j0 + d + AHEAD, d);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        mbar_arrive_warp(bar_full + 8 * stage);
+        if (++stage == S) { stage = 0; empty_parity ^= 1u; }
       }
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      mbar_arrive_warp(bar_full + 8 * stage);
     }
   } else if (lane == 0) {
     // ---------------- MMA issue ----------------
@@ -654,10 +661,10 @@ k_gemm_tn_tc(const float* __restrict__ A, int lda, const float* __restrict__ B, 
     for (int j = 0; j < total; ++j) {
       if (!mbar_wait_abortable(bar_full + 8 * stage, full_parity, abortp)) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t a_hi = operand_desc_mn_lo(smem_base + stage * Cfg::kStage), a_lo = a_hi + (Cfg::kATile >> 4);
+      const uint32_t a_hi = operand_desc_mn_lo<GROUP>(smem_base + stage * Cfg::kStage), a_lo = a_hi + (Cfg::kATile >> 4);
       const uint32_t b_hi = a_hi + (2 * Cfg::kATile >> 4), b_lo = b_hi + (Cfg::kBTile >> 4);
 #pragma unroll
-      for (int ks = 0; ks < kTnRows / 8; ++ks) {
+      for (int ks = 0; ks < ROWS / 8; ++ks) {
         const uint32_t o = ks * (1024 >> 4);       // the next group of 8 rows, in 16-byte units
         const uint32_t first = (ks > 0) ? 1u : (j > 0 ? 1u : 0u);
         mma_tf32_lo(tmem_base + NT, a_lo + o, b_hi + o, idesc, first, kOperandDescMnHi);   // corrections
