@@ -340,6 +340,8 @@ def run_ours(args):
 
     def bound_of(row):
         k = row["kernel"]
+        if k.startswith("gemm_half"):     # three fp16 products of the split operands
+            return "tensor", row["tflops"], peaks["bf16_tflops"] / 3.0, "TFLOP/s"
         if k.startswith("gemm_tc") or k.startswith("gemm_tn_tc"):
             return "tensor", row["tflops"], tc_peak, "TFLOP/s"
         if k.startswith("gemm"):
