@@ -2,6 +2,7 @@
 // kernels.cuh.  See include/gcn_admm.h for the contract of every entry point.
 #include "../../include/gcn_admm.h"
 
+#include <cfloat>
 #include <climits>
 #include <cmath>
 #include <cuda_runtime.h>
@@ -492,7 +493,7 @@ struct gcn_admm {
     return N <= 16 ? 16 : N <= 32 ? 32 : N <= 48 ? 48 : N <= 64 ? 64 : halves && N <= 96 ? 96 : N <= 128 ? 128 : halves && N <= 192 ? 192 : 256;
   }
   // With many row tiles k_gemm_tc_ws would split the same weights again for every tile; with at most one tile per CTA, or
-  // with few chunks, that costs nothing, and the launch that makes the image would (13.8 k rows, 767 x 1000, three tiles per CTA:
+  // with few chunks, that costs nothing, and the image would (13.8 k rows, 767 x 1000, three tiles per CTA:
   // 130 -> 98 us by an image; 10 x 1000: no gain).
   bool by_halves(long long Mr, int N, int K) const {
     if (!on_tensor_cores(Mr, K) || encode_tiled() == nullptr) return false;
@@ -1166,7 +1167,10 @@ struct gcn_admm {
     float most = 0.f;
     if (img_H[l].data != nullptr || img_G[l].data != nullptr) {
 #pragma omp simd reduction(max : most)
-      for (long long e = 0; e < (long long)r * c; ++e) most = std::max(most, std::fabs(host_w[e]));
+      for (long long e = 0; e < (long long)r * c; ++e) {   // of the finite elements: an infinity or NaN stays in its column
+        const float size = std::fabs(host_w[e]);
+        most = size <= FLT_MAX ? std::max(most, size) : most;
+      }
     }
     gk::k_load_weight<<<grid_for(cells), 256, 0, stream>>>(grad, r, c, W[l], ld[l], Wt[l], ld[l - 1], img_H[l], img_G[l], most);
     CU(cudaGetLastError());

@@ -91,12 +91,13 @@ __device__ __forceinline__ void put_half(const Image& im, int n, int k, float x)
   *reinterpret_cast<__half*>(at) = h;
   *reinterpret_cast<__half*>(at + (size_t)im.nt * kHalfRow) = __float2half_rn(fmaf(-kLoScale, __half2float(h), kLoScale * x));
 }
-// The inverse scales of an image whose `n` columns share the scale of m, by the threads of one block.
+// The inverse scales of an image whose `n` columns share the scale of m, by the threads of one block.  No scale holds the finite
+// elements beside an infinite one: where m is not finite every column of the product becomes NaN, rather than some of them zero.
 __device__ __forceinline__ void put_scales(const Image& im, int n, float m) {
   if (im.data == nullptr) return;
   const int groups = (n + im.nt - 1) / im.nt;
   float* const at = reinterpret_cast<float*>(im.data + image_blocks_bytes(groups, im.nt, im.kc));
-  for (int c = threadIdx.x; c < groups * im.nt; c += blockDim.x) at[c] = inverse_scale_of(m);
+  for (int c = threadIdx.x; c < groups * im.nt; c += blockDim.x) at[c] = fabsf(m) < INFINITY ? inverse_scale_of(m) : __int_as_float(0x7fffffff);
 }
 
 struct SplitB {
@@ -153,7 +154,7 @@ struct HalfCfg {
 
 // Roles (see k_gemm_tc_ws; the waits, the abort flag and the way out are the same):
 //   copy warp   one thread: raw tile of A by a tensor copy, B's chunk by a bulk copy, into slot j mod R as soon as it is free
-//   warps 0-7   producers: scale and split the raw tile of A where it lies (a pair of halves takes the room of its float, and a
+//   producers   four or eight warps: scale and split the raw tile of A where it lies (a pair of halves takes the room of its float, and a
 //               warp's 16 rows become its own two groups of A_hi and A_lo); arrive on ready[slot]
 //   MMA warp    one thread issues; its commit frees the slot
 //   epilogue    accumulators -> scales taken off -> C

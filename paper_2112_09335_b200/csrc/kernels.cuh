@@ -2446,8 +2446,8 @@ __global__ void k_transpose_small(const float* __restrict__ src, int lds, float*
   dst[c * ldd + r] = src[r * lds + c];
 }
 
-// W (rows x cols, leading dimension ldw), its transpose and its images from a dense matrix whose largest magnitude is `bound`; padding
-// columns become zero.
+// W (rows x cols, leading dimension ldw), its transpose and its images from a dense matrix whose largest finite magnitude is `bound`;
+// padding columns become zero.
 __global__ void k_load_weight(const float* __restrict__ src, int rows, int cols, float* __restrict__ W, int ldw,
                               float* __restrict__ Wt, int ldwt, const gtc::Image image, const gtc::Image image_t, float bound) {
   const float scale = gtc::scale_of(bound);

@@ -85,3 +85,25 @@ def test_values_without_a_scale_stay_in_their_row(handle):
     keep = torch.ones(m, dtype=torch.bool, device="cuda")
     keep[5] = keep[700] = False
     assert torch.equal(got[keep], clean[keep])
+
+
+@pytest.mark.parametrize("bad", [float("inf"), float("nan")])
+def test_a_weight_without_a_scale_stays_in_its_column(bad):
+    """The columns of a layer's weights share one scale: that of the finite ones."""
+    import numpy as np
+    wl = inputs.make_workload(3, scale=0.05)
+    assert wl.n >= 4096
+    w = [np.array(x, dtype=np.float32) for x in wl.w_init]
+    r = int(np.argmin(np.abs(w[-1][:, 2])))          # not the element the scale comes from
+    logits = []
+    for value in (w[-1][r, 2], bad):
+        w[-1][r, 2] = value
+        g = binding.GcnAdmm(wl.n, wl.row_ptr, wl.col_idx, wl.X, wl.y, wl.train_mask, wl.widths, wl.n_comm, wl.community, w, tensor_cores=2)
+        try:
+            logits.append(g.predict()[0])
+        finally:
+            g.destroy()
+    clean, got = logits
+    others = [c for c in range(clean.shape[1]) if c != 2]
+    assert np.isfinite(clean).all() and not np.isfinite(got[:, 2]).any()
+    assert np.array_equal(got[:, others], clean[:, others])
