@@ -837,19 +837,23 @@ struct gcn_admm {
       std::snprintf(zname, sizeof zname, "search_z_out@%d", ldn);
       {
         Scope sc(this, zname, 1, 4.0 * gi.nnz + 12.0 * n + 8.0 * (double)n * ldn, 2.0 * (double)gi.nnz * ldn);
-#define SEARCH_OUT(CL)                                                                                                      \
-  {                                                                                                                         \
-    const auto kernel = gk::k_search_z_out<CL>;                                                                             \
-    const int grid = (int)std::min<long long>(cdiv(n_seg_chunks, warps), resident_blocks((const void*)kernel, warps * 32, 0)); \
-    launch_alone(kernel, grid, warps * 32, 0, d_col, d_dinv, (const float4*)B0, (const float4*)B1, ld4, scratch, a);          \
+        const auto search = [&](auto kernel, int grid, int block) {
+          launch_alone(kernel, grid, block, 0, d_col, d_dinv, (const float4*)B0, (const float4*)B1, ld4, scratch, a);
+        };
+        const int dealt = (int)cdiv(n_seg_chunks, 2);
+#define NARROW(CL)                                                                                     \
+  {                                                                                                    \
+    const int grid = resident_blocks((const void*)gk::k_search_z_out<CL, false>, warps * 32, 0);       \
+    if (n_seg_chunks <= grid * warps) search(gk::k_search_z_out<CL, true>, dealt, 64);                 \
+    else search(gk::k_search_z_out<CL, false>, grid, warps * 32);                                      \
   }
-        if (ld4 <= 1) SEARCH_OUT(1)
-        else if (ld4 <= 2) SEARCH_OUT(2)
-        else if (ld4 <= 4) SEARCH_OUT(4)
-        else if (ld4 <= 8) SEARCH_OUT(8)
-        else if (ld4 <= 16) SEARCH_OUT(16)
-        else SEARCH_OUT(32)
-#undef SEARCH_OUT
+        if (ld4 <= 1) NARROW(1)
+        else if (ld4 <= 2) NARROW(2)
+        else if (ld4 <= 4) NARROW(4)
+        else if (ld4 <= 8) search(gk::k_search_z_out<8, true>, dealt, 64);
+        else if (ld4 <= 16) search(gk::k_search_z_out<16, true>, dealt, 64);
+        else search(gk::k_search_z_out<32, true>, dealt, 64);
+#undef NARROW
         CU(cudaGetLastError());
       }
       Scope sc(this, "move_z", 1, move_bytes, 0.0);

@@ -2030,22 +2030,25 @@ __device__ __forceinline__ float4 add_sets(float4 k) {
   return k;
 }
 
-// The next chunk of a sweep whose `warps` warps began with one each.
-__device__ __forceinline__ int next_chunk(int* counter, int warps, int lane) {
-  int ch = 0;
-  if (lane == 0) ch = warps + atomicAdd(counter, 1);
-  return __shfl_sync(0xffffffffu, ch, 0);
-}
-
-template <int CL>
-__global__ void __launch_bounds__(256, 3)
+// DEALT: a warp of its own for every chunk, the one of its number, in blocks of 64 threads; else as many warps as the chip holds, which
+// take chunks from the counter.  The loop over chunks keeps so many values alive across a chunk that it spills 100 to 332 bytes at the 80
+// registers of 24 warps per SM; without it nothing spills (2.45 M rows, 47 columns: 4.95 -> 3.36 ms, 3.53 in blocks of 256, 3.31 at 64
+// registers with spills; 169 k, 40 columns 118 -> 94 us, 100, 97).  Chunks of narrow rows are too little work for a block's start
+// (19.7 k rows, 3 columns: 20.8 by the counter, 23.2 dealt) unless the chip holds all of them at once.
+template <int CL, bool DEALT>
+__global__ void __launch_bounds__(DEALT ? 64 : 256, DEALT ? 12 : 3)
 k_search_z_out(const int* __restrict__ col, const float* __restrict__ dinv, const float4* __restrict__ T, const float4* __restrict__ S,
                int ld4, float4* scratch, const SearchOut p) {
   constexpr int GROUPS = 32 / CL;
   const int lane = threadIdx.x & 31, grp = lane / CL, cl = lane & (CL - 1);
-  // every warp's first chunk is its own number, the others come from the counter
-  const int warps = (int)(gridDim.x * (blockDim.x >> 5));
-  for (int ch = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); ch < p.n_chunks; ch = next_chunk(p.chunk_counter, warps, lane)) {
+  do {
+    int ch = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    if (!DEALT) {
+      ch = 0;
+      if (lane == 0) ch = atomicAdd(p.chunk_counter, 1);
+      ch = __shfl_sync(0xffffffffu, ch, 0);
+    }
+    if (ch >= p.n_chunks) return;
     const SegChunk c = p.chunks[ch];
     if (__ldcg(&p.ctl[c.comm].done)) continue;   // skipped: none of its slots is filled
     double lin = 0.0, quad = 0.0;
@@ -2116,7 +2119,7 @@ k_search_z_out(const int* __restrict__ col, const float* __restrict__ dinv, cons
     sums[0] = warp_sum(sums[0]);
     sums[1] = warp_sum(sums[1]);
     decide_one(p.ctl + c.comm, sums, p.own[c.comm * 3 + 2], p.a, p.n_active, p.status);
-  }
+  } while (!DEALT);
 }
 
 // The move of the blocks after it: Z_l[i,:] <- Z_l[i,:] - G[i,:] / theta_{comm(i)} (Eq. 10), and the log entries.

@@ -49,6 +49,12 @@ def test_many_chunks_and_a_search_of_several_sweeps():
     run_pair(tiny_problem(61, n=2600, widths=(6, 10, 8, 4), n_comm=5, p=0.012), n_it=3, tau0=1e-3, theta0=1e-5, bt_max_trials=64)
 
 
+@pytest.mark.parametrize("classes", [3, 7, 16, 23])
+def test_closed_form_with_more_chunks_than_warps(classes):
+    """155 k stored entries in chunks of at most 32: more than the 3,552 warps the chip holds, so narrow rows take chunks from the counter."""
+    run_pair(tiny_problem(65, n=5000, widths=(6, 9, classes), n_comm=5, p=0.006), n_it=2)
+
+
 @pytest.mark.parametrize("n", [900, 1100, 5000])
 def test_few_and_many_splits_of_the_weight_gradient(n):
     run_pair(tiny_problem(62, n=n, widths=(33, 9, 4), n_comm=4, p=3.0 / n), n_it=2)
