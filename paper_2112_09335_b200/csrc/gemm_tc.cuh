@@ -1,6 +1,7 @@
 // Dense product C[M x N] = A[M x K] * B on the 5th-generation tensor cores (tcgen05, accumulator
-// in tensor memory), used for the feature-by-weight contractions of every layer:
-//   H_l = P_l W_l,  D = P_l grad,  G = S W_{l+1}^T,  T = G W_{l+1}.
+// in tensor memory), used for the feature-by-weight contractions of small graphs (gemm_half.cuh has those of larger ones):
+//   H_l = P_l W_l,  D = P_l grad,  G = S W_{l+1}^T,  T = G W_{l+1},
+// and the transposed product P_l^T R of every graph of 4,096 rows or more (k_gemm_tn_tc).
 //
 // fp32 accuracy from TF32 hardware: each operand x is split into x_hi + x_lo with both halves held
 // at TF32 resolution (x_hi = x rounded to 10 mantissa bits, x_lo = x - x_hi, at most 2^-11 of x), and
