@@ -20,6 +20,7 @@
 // The row maxima of A come with A: whoever writes the matrix leaves them (row_max).  B comes as an image of the staged layout, kept
 // by whoever writes the weights (put_half: every column by one scale, from a bound of the matrix) or made by k_split_b.
 #pragma once
+#include <cfloat>
 #include <cuda_fp16.h>
 
 #include "gemm_tc.cuh"
@@ -91,13 +92,15 @@ __device__ __forceinline__ void put_half(const Image& im, int n, int k, float x)
   *reinterpret_cast<__half*>(at) = h;
   *reinterpret_cast<__half*>(at + (size_t)im.nt * kHalfRow) = __float2half_rn(fmaf(-kLoScale, __half2float(h), kLoScale * x));
 }
-// The inverse scales of an image whose `n` columns share the scale of m, by the threads of one block.  No scale holds the finite
-// elements beside an infinite one: where m is not finite every column of the product becomes NaN, rather than some of them zero.
+// A bound formed from others may leave the range while every element it bounds is finite: the largest number bounds those too.
+// Elements that are not finite stay in their column of the product under any finite scale.
+__device__ __forceinline__ float finite_bound(float m) { return fminf(m, FLT_MAX); }
+// The inverse scales of an image whose `n` columns share the scale of m, a finite number, by the threads of one block.
 __device__ __forceinline__ void put_scales(const Image& im, int n, float m) {
   if (im.data == nullptr) return;
   const int groups = (n + im.nt - 1) / im.nt;
   float* const at = reinterpret_cast<float*>(im.data + image_blocks_bytes(groups, im.nt, im.kc));
-  for (int c = threadIdx.x; c < groups * im.nt; c += blockDim.x) at[c] = fabsf(m) < INFINITY ? inverse_scale_of(m) : __int_as_float(0x7fffffff);
+  for (int c = threadIdx.x; c < groups * im.nt; c += blockDim.x) at[c] = inverse_scale_of(m);
 }
 
 struct SplitB {

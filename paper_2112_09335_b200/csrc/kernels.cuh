@@ -1003,7 +1003,7 @@ k_finish_grad(const float* __restrict__ part, int splits, int rows, int cols, in
   const long long elems = (long long)rows * ldp;
   double sq[2] = {0.0, 0.0};   // of grad, of W
   float most[2] = {0.f, 0.f};
-  const float bound = W != nullptr && image.data != nullptr ? (float)splits * __uint_as_float(__ldcg(&ctl->part_max)) : 0.f;
+  const float bound = W != nullptr && image.data != nullptr ? gtc::finite_bound((float)splits * __uint_as_float(__ldcg(&ctl->part_max))) : 0.f;
   const float scale = gtc::scale_of(bound);
   if (W != nullptr && blockIdx.x == 0) gtc::put_scales(image, cols, bound);
   const auto sum_splits = [&](long long e, int k0, int k1) {
@@ -1132,7 +1132,7 @@ __device__ __forceinline__ void move_w(const SearchW& p, float step) {
   if (step != 0.f) {
     __shared__ WeightTile turn;
     const int tiles = ((p.rows + 31) / 32) * ((p.cols + 31) / 32);
-    const float bound = fmaf(step, __ldcg(&p.ctl->g_max), __ldcg(&p.ctl->w_max)), scale = gtc::scale_of(bound);   // |W - step grad| elementwise
+    const float bound = gtc::finite_bound(fmaf(step, __ldcg(&p.ctl->g_max), __ldcg(&p.ctl->w_max))), scale = gtc::scale_of(bound);   // |W - step grad| elementwise
     if (blockIdx.x == 0) {
       gtc::put_scales(p.image, p.cols, bound);
       gtc::put_scales(p.image_t, p.rows, bound);

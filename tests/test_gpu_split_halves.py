@@ -107,3 +107,34 @@ def test_a_weight_without_a_scale_stays_in_its_column(bad):
     others = [c for c in range(clean.shape[1]) if c != 2]
     assert np.isfinite(clean).all() and not np.isfinite(got[:, 2]).any()
     assert np.array_equal(got[:, others], clean[:, others])
+
+
+def test_partial_sums_whose_bound_leaves_the_range():
+    """The image of a weight gradient is scaled by (number of partial sums) x (largest of them).  Here that product is above the
+    largest float while the gradient is finite: 64 splits of 256 rows hold 1.1e37 each in the rows of half of the features, of one
+    sign in one half of the nodes and of the other in the rest, and what is left is 7e30.  One W block, against fp32 FMA."""
+    import numpy as np
+    n, hidden, classes = 16384, 64, 8
+    X = np.ones((n, 16), dtype=np.float32)
+    X[:, :8] = 1e8
+    X[n // 2:, :8] *= -1
+    rng = np.random.default_rng(0)
+    W1 = np.zeros((16, hidden), dtype=np.float32)
+    W1[8:] = rng.uniform(0.5, 1.0, (8, hidden)) / 8
+    W2 = rng.standard_normal((hidden, classes)).astype(np.float32)
+    Z1 = np.broadcast_to(-4.3e26 * (1 + np.arange(hidden) / hidden), (n, hidden)).astype(np.float32)
+    found = []
+    for tensor_cores in (0, 1):
+        g = binding.GcnAdmm(n, np.zeros(n + 1, np.int64), np.zeros(0, np.int32), X, np.zeros(n, np.int32), np.zeros(n, np.uint8), [16, hidden, classes],
+                            2, np.arange(n, dtype=np.int32) // (n // 2), [W1, W2], nu=1.0, rho=1.0, tau0=2e34, tensor_cores=tensor_cores)
+        try:
+            g.set_state(binding.ST_Z, 1, Z1)
+            g.step_block(binding.PHASE_W, 1)
+            d = g.decisions()
+            found.append((d["trial_w"][0, 0], d["q_w"][0, 0], g.get_state(binding.ST_W, 1), g.predict()[0]))
+        finally:
+            g.destroy()
+    (trial, q, w, logits), (trial_tc, q_tc, w_tc, logits_tc) = found
+    assert trial == 0 and np.abs(w - W1).max() > 1e-4                       # the block moves
+    assert trial_tc == trial and abs(q_tc - q) < 1e-4 * abs(q)
+    assert np.abs(w_tc - w).max() < 1e-6 and np.abs(logits_tc - logits).max() < 1e-5 * np.abs(logits).max()
