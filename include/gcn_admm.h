@@ -55,15 +55,15 @@ enum {
  *                  1/(loss_scale/2 + rho), t_1 = 1, warm start, no early exit)
  *  loss_scale      R = loss_scale * sum over training rows of the softmax cross-entropy
  *  dual_mode       0: Eq. 3 as printed (Z_L^k, Z_{L-1}^k, W_L^{k+1}); 1: the k+1 iterates
- *  tensor_cores    1: dense products with 8 <= K <= 2048 and at least 512 rows run on the tensor cores as an
- *                  error-compensated TF32 product (three passes, fp32 accumulation, relative error of a few
- *                  1e-7 of sum |a||b|); products of 16384 rows or more (or with several row tiles per SM
- *                  and K >= 128) take the weight operand from an image of the staged layout, kept by the
- *                  kernels that write the weights, and fetch it with bulk copies (smaller ones split it per
- *                  row tile), and with at most 128 output columns they also
- *                  fetch the tiles of the row operand by tensor copies (products with 129 to 256 output columns
- *                  and K <= 128 run in that form as two groups of 128 columns); 2: the same kernels, pre-split
- *                  at every size; 0: fp32 FMA kernels everywhere
+ *  tensor_cores    1: dense products with 8 <= K <= 2048 and at least 512 rows run on the tensor cores, each
+ *                  operand element as the sum of two numbers of 11 bits (fp32 accumulation, relative error of a
+ *                  few 1e-7 of sum |a||b|).  Products of 16384 rows or more (or with several row tiles per SM and
+ *                  K >= 128) use pairs of fp16 numbers under a power of two per row of the first operand and per
+ *                  matrix or column of the second; rows whose elements span too much of the fp32 range for that
+ *                  (2^27 in one operand while the other spans 2^22 or has zeros, or 2^27 in the second) are formed
+ *                  again by pairs of TF32 numbers, which have an exponent per element, in up to four times
+ *                  the time.  Smaller products, and the transposed ones of 4096 rows or more, use TF32 pairs throughout;
+ *                  2: the same kernels, fp16 pairs at every size; 0: fp32 FMA kernels everywhere
  *  use_graph       1: gcn_admm_step records one pass as a CUDA graph on first use and replays it (only when
  *                  the handle's stream is not the default stream and profiling is off; for calls of one
  *                  pass from the third on); 2: the same, but

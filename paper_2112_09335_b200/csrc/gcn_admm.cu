@@ -501,7 +501,7 @@ struct gcn_admm {
   }
   static size_t image_bytes(int N, const gtc::Image& im) {
     const int groups = (int)cdiv(N, im.nt);
-    return gtc::image_blocks_bytes(groups, im.nt, im.kc) + (size_t)groups * im.nt * sizeof(float);
+    return gtc::image_blocks_bytes(groups, im.nt, im.kc) + (size_t)groups * im.nt * sizeof(float) + (size_t)gtc::image_marks(groups, im.nt, im.kc) * sizeof(int);
   }
   // Asks for an image of the operand of an n x K by K x N product, where that product takes one.
   void want_image(gtc::Image& im, int N, int K) {
@@ -538,7 +538,7 @@ struct gcn_admm {
         if (halves) {
           using Cfg = gtc::HalfCfg<NT>;
           CU(cudaFuncSetAttribute(gtc::k_gemm_half<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::kSmem));
-          launch_alone(gtc::k_gemm_half<NT>, grid, Cfg::kThreads, Cfg::kSmem, a_max, Cm, ldc, (int)Mr, N, K, skip, tc_error, image.data, tmap);
+          launch_alone(gtc::k_gemm_half<NT>, grid, Cfg::kThreads, Cfg::kSmem, A, lda, a_max, Bk, ldbk, Cm, ldc, (int)Mr, N, K, skip, tc_error, image.data, tmap);
         } else if constexpr (NT != 96 && NT != 192) {
           using Cfg = gtc::WsCfg<NT>;
           CU(cudaFuncSetAttribute(gtc::k_gemm_tc_ws<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::kSmem));
@@ -576,11 +576,10 @@ struct gcn_admm {
   // Whether P^T R runs on the tensor cores (that form can also build a hidden layer's R itself).
   bool tn_on_tensor_cores(long long rows) const { return p.tensor_cores != 0 && rows >= 4096; }
 
-  // part_max (tensor-core form only): raised to the largest magnitude among the partial sums, as bits.
   // With `zres` B holds pre-activations H and the operand is
   // h > 0 ? nu (h - z) : 0, formed while staging: the residual matrix is never stored.
   int gemm_tn(const float* A, int lda, const float* B, int ldb, int ldp, long long rows, int Ka, int Nb,
-              const float* zres = nullptr, float nu = 0.f, unsigned* part_max = nullptr) {
+              const float* zres = nullptr, float nu = 0.f) {
     int splits = 1;
     long long rps = rows;
     char name[48];
@@ -607,10 +606,10 @@ struct gcn_admm {
     dim3 grid((unsigned)groups, (unsigned)splits, (unsigned)nb_groups);                                        \
     if (zres) {                                                                                                \
       CU(cudaFuncSetAttribute(gtc::k_gemm_tn_tc<NT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
-      launch_alone(gtc::k_gemm_tn_tc<NT, true>, grid, gtc::kTnThreads, smem, A, lda, B, ldb, part, ldp, rows, rps, Ka, Nb, tc_error, zres, nu, part_max); \
+      launch_alone(gtc::k_gemm_tn_tc<NT, true>, grid, gtc::kTnThreads, smem, A, lda, B, ldb, part, ldp, rows, rps, Ka, Nb, tc_error, zres, nu); \
     } else {                                                                                                   \
       CU(cudaFuncSetAttribute(gtc::k_gemm_tn_tc<NT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
-      launch_alone(gtc::k_gemm_tn_tc<NT, false>, grid, gtc::kTnThreads, smem, A, lda, B, ldb, part, ldp, rows, rps, Ka, Nb, tc_error, nullptr, 0.f, part_max); \
+      launch_alone(gtc::k_gemm_tn_tc<NT, false>, grid, gtc::kTnThreads, smem, A, lda, B, ldb, part, ldp, rows, rps, Ka, Nb, tc_error, nullptr, 0.f); \
     }                                                                                                          \
   }
       if (Nb <= 16) TN_TC(16)
@@ -647,15 +646,15 @@ struct gcn_admm {
 
   // grad (and grad_t) from the `splits` partial sums gemm_tn left in `part`; with `ctl` the start of the W_l search too.
   void finish_grad(int splits, int Ka, int Nb, int ldp, float* out, float* out_t, int ldt, const float* w, SearchCtl* ctl,
-                   const gtc::Image& image, bool maxima) {
+                   bool maxima) {
     Scope sc(this, "finish_grad", 1, 4.0 * (double)Ka * ldp * (splits + (w ? 3 : 1)), 0.0);
     const long long elems = (long long)Ka * ldp;
     if (splits >= 16)
       launch(gk::k_finish_grad<8>, (unsigned)cdiv(elems, 32), 256, 0, part, splits, Ka, Nb, ldp, out, out_t, ldt, w, red_part,
-                                                                            ticket, ctl, p.bt_shrink, p.bt_growth, status, image, maxima);
+                                                                            ticket, ctl, p.bt_shrink, p.bt_growth, status, maxima);
     else
       launch(gk::k_finish_grad<1>, (unsigned)(cdiv(Ka, 32) * cdiv(ldp, 32)), 256, 0, part, splits, Ka, Nb, ldp, out, out_t, ldt, w, red_part,
-                                                                                     ticket, ctl, p.bt_shrink, p.bt_growth, status, image, maxima);
+                                                                                     ticket, ctl, p.bt_shrink, p.bt_growth, status, maxima);
     CU(cudaGetLastError());
   }
 
@@ -717,15 +716,14 @@ struct gcn_admm {
     float *const R = resid_of(l), *const D = l == L && DL != nullptr ? DL : B1;
     int splits;
     if (l < L) {                                                        // grad = P_l^T R_l, R_l formed inside the product
-      splits = gemm_tn(P[l], ld[l - 1], H[l], ldc, ldc, n, Kp, Cn, Z[l], p.nu, &ctl->part_max);
+      splits = gemm_tn(P[l], ld[l - 1], H[l], ldc, ldc, n, Kp, Cn, Z[l], p.nu);
     } else {
       resid(l, R);                                                      // R_l
-      splits = gemm_tn(P[l], ld[l - 1], R, ldc, ldc, n, Kp, Cn, nullptr, 0.f, &ctl->part_max);   // grad = P_l^T R_l
+      splits = gemm_tn(P[l], ld[l - 1], R, ldc, ldc, n, Kp, Cn);   // grad = P_l^T R_l
     }
-    const bool bounded = tn_on_tensor_cores(n);   // by the largest partial sum; else the image is made from the gradient itself
-    finish_grad(splits, Kp, Cn, ldc, grad, grad_t, ld[l - 1], W[l], ctl, bounded ? img_D[l] : gtc::Image{nullptr, 16, 1},
-                img_H[l].data != nullptr || img_G[l].data != nullptr);
-    if (!bounded && img_D[l].data != nullptr) split_b(gtc::SplitB{grad_t, ld[l - 1], Cn, Kp, img_D[l]});
+    finish_grad(splits, Kp, Cn, ldc, grad, grad_t, ld[l - 1], W[l], ctl, img_H[l].data != nullptr || img_G[l].data != nullptr);
+    // in a launch of its own, for the scales: only a finished gradient gives each column its largest element
+    if (img_D[l].data != nullptr) split_b(gtc::SplitB{grad_t, ld[l - 1], Cn, Kp, img_D[l]});
     gemm_nn(P[l], ld[l - 1], P_max[l], grad, ldc, grad_t, ld[l - 1], D, ldc, n, Cn, Kp, img_D[l], &ctl->done);   // D = P_l grad
     gk::SearchW a{};
     a.H = (float4*)H[l]; a.D = (const float4*)D; a.Z = (const float4*)Z[l]; a.U = (const float4*)U; a.R = (const float4*)R;
@@ -1168,15 +1166,21 @@ struct gcn_admm {
     CU(stage.put(grad, host_w, sizeof(float) * (size_t)r * c, stream));
     CU(stage.finish(stream));
     const long long cells = std::max((long long)r * ld[l], (long long)c * ld[l - 1]);
-    float most = 0.f;
+    float most = 0.f, least = FLT_MAX;
+    int zeros = 0;
     if (img_H[l].data != nullptr || img_G[l].data != nullptr) {
-#pragma omp simd reduction(max : most)
+#pragma omp simd reduction(max : most) reduction(min : least) reduction(| : zeros)
       for (long long e = 0; e < (long long)r * c; ++e) {   // of the finite elements: an infinity or NaN stays in its column
         const float size = std::fabs(host_w[e]);
         most = size <= FLT_MAX ? std::max(most, size) : most;
+        least = size > 0.f ? std::min(least, size) : least;
+        zeros |= size == 0.f;
       }
     }
-    gk::k_load_weight<<<grid_for(cells), 256, 0, stream>>>(grad, r, c, W[l], ld[l], Wt[l], ld[l - 1], img_H[l], img_G[l], most);
+    // most is scaled to 2^14 at least: elements below 2^-27 of it may be too small for a pair, below 2^-22 they make the matrix wide
+    const int marks = ((double)least < std::ldexp((double)most, -27) || least < FLT_MIN ? gtc::kBelowPairs : 0) |
+                      (zeros || (double)least < std::ldexp((double)most, -22) ? gtc::kWide : 0);
+    gk::k_load_weight<<<grid_for(cells), 256, 0, stream>>>(grad, r, c, W[l], ld[l], Wt[l], ld[l - 1], img_H[l], img_G[l], most, marks);
     CU(cudaGetLastError());
   }
   // Step parameters (t_prev) of `count` searches in a row, to and from the host.
@@ -1850,6 +1854,7 @@ int gcn_admm_dense_product(gcn_admm* h, const float* A, const float* B, float* C
         image.nt = gcn_admm::group_width(n, true);
         image.kc = (int)cdiv(k, gtc::kChunkK);
         image.data = dalloc<uint8_t>(gcn_admm::image_bytes(n, image));
+        CU(cudaMemsetAsync(image.data, 0, gcn_admm::image_bytes(n, image), h->stream));
         a_max = dalloc<float>((size_t)m);
         h->split_b(gtc::SplitB{bk, ldbk, n, k, image});
         gk::k_row_max<<<h->grid_for(32 * m), 256, 0, h->stream>>>(reinterpret_cast<const float4*>(a), lda / 4, m, a_max);
@@ -1890,7 +1895,7 @@ int gcn_admm_dense_product_tn(gcn_admm* h, const float* A, const float* B, float
       CU(cudaMemcpy2DAsync(b, (size_t)ldb * 4, B, (size_t)nb * 4, (size_t)nb * 4, (size_t)rows, cudaMemcpyDeviceToDevice, h->stream));
       h->p.tensor_cores = tensor_cores;
       const int splits = h->gemm_tn(a, lda, b, ldb, ldp, rows, ka, nb);
-      h->finish_grad(splits, ka, nb, ldp, c, nullptr, 0, nullptr, nullptr, gtc::Image{nullptr, 16, 1}, false);
+      h->finish_grad(splits, ka, nb, ldp, c, nullptr, 0, nullptr, nullptr, false);
       h->p.tensor_cores = saved;
       CU(cudaMemcpy2DAsync(C, (size_t)nb * 4, c, (size_t)ldp * 4, (size_t)nb * 4, (size_t)ka, cudaMemcpyDeviceToDevice, h->stream));
       CU(cudaStreamSynchronize(h->stream));

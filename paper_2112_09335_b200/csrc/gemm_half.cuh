@@ -3,8 +3,13 @@
 //
 // fp32 accuracy from fp16 hardware: a row of A is scaled by a power of two that brings its largest element into [2^14, 2^15)
 // (exact), so is a column of B (or all of B by a bound of its elements), and each scaled element x is split into x_hi = half(x) and x_lo = half(2^11 (x - x_hi)).  Both
-// hold 11 bits and are rounded to nearest, so x_hi + 2^-11 x_lo is x to 2^-23 of its magnitude for every element down to 2^-29 of
-// the largest of its row, and to 2^-51 of that one below.  As with TF32 pairs,
+// hold 11 bits and are rounded to nearest, so x_hi + 2^-11 x_lo is x to 2^-23 of its magnitude where that is 2^-13 or more, that is for
+// elements down to 2^-27 of the largest of their row; below, bits of x_lo fall under the smallest half and the element is held to
+// 2^-51 of that largest one only.  Where that could show, rows are formed by TF32 pairs instead (redo_rows): all of them where B holds
+// such an element (its image says); where B is wide, those whose row of A does (the producers look).  B is wide where an element,
+// zero included, is below 2^-8 (the largest is 2^14 or more).  Beside a B that is not, K elements held to 2^-36 (2^15 is the largest)
+// cost at most K 2^-36 2^15 against sum |a||b| >= 2^14 2^-8: K 2^-27, and with the accumulator's (K / 16 + 3.5) 2^-23 that
+// is within the bound of TF32 pairs, (K / 8 + 11) 2^-23.  As with TF32 pairs,
 //   A B ~= A_hi B_hi + 2^-11 (A_lo B_hi + A_hi B_lo)
 // is accumulated in fp32, the main product and the corrections apart (the tensor core rounds an accumulator toward zero at every
 // MMA); the scales come off in the epilogue.  Against TF32 pairs an MMA covers twice the reduction in the same time (and the
@@ -18,7 +23,9 @@
 // of 256 instead of two of 128 (every A tile read and split twice): 0.59 against 0.67 ms.
 //
 // The row maxima of A come with A: whoever writes the matrix leaves them (row_max).  B comes as an image of the staged layout, kept
-// by whoever writes the weights (put_half: every column by one scale, from a bound of the matrix) or made by k_split_b.
+// by whoever writes the weights (put_half: every column by one scale, from a bound of the matrix) or made by k_split_b from a finished
+// gradient (every column by its own: a bound kept with the partial sums, in the writer itself, is 2^5 to 2^7 above the largest element, and
+// with it a 767 x 1000 gradient always held elements too small for a pair; the launch takes 6 to 8 us under a profiler).
 #pragma once
 #include <cfloat>
 #include <cuda_fp16.h>
@@ -59,6 +66,27 @@ __device__ __forceinline__ uint32_t scale_field(float m) { return (uint32_t)min(
 __device__ __forceinline__ float scale_of(float m) { return __uint_as_float(scale_field(m) << 23); }
 __device__ __forceinline__ float inverse_scale_of(float m) { return __uint_as_float((254u - scale_field(m)) << 23); }
 
+// Elements too small for a pair.  Keys order magnitudes with zero, which every pair holds, behind all others; below_pairs(scale) is the
+// key below which a scaled element lies under 2^-13, marks_for the marks an element of B makes.  Where the largest element is not
+// finite (scale 2^-114) there is no such key: the row is NaN in any form.  Under a scale of 2^114 or more (largest element below
+// 2^-98) subnormal elements count as too small.
+__host__ __device__ __forceinline__ uint32_t size_key(uint32_t bits) { return (bits << 1) - 1u; }
+__device__ __forceinline__ uint32_t size_key(float x) { return size_key(__float_as_uint(x)); }
+__device__ __forceinline__ uint32_t below_pairs(float scale) {
+  const int field = (int)(__float_as_uint(scale) >> 23);
+  return field == 13 ? 0u : size_key((uint32_t)max(1, 241 - field) << 23);
+}
+constexpr int kBelowPairs = 1, kWide = 2;
+__device__ __forceinline__ int marks_for(float x, float scale) {
+  return (size_key(x) < below_pairs(scale) ? kBelowPairs : 0) | (fabsf(x * scale) < 0x1p-8f ? kWide : 0);
+}
+__device__ __forceinline__ uint32_t least_key(const float4& a) {
+  return min(__vimin3_u32(size_key(a.x), size_key(a.y), size_key(a.z)), size_key(a.w));
+}
+__device__ __forceinline__ uint32_t least_key(const float4& a, const float4& b) {
+  return __vimin3_u32(least_key(a), __vimin3_u32(size_key(b.x), size_key(b.y), size_key(b.z)), size_key(b.w));
+}
+
 // Eight scaled elements as halves: hi rounded to nearest, lo = half(2^11 (x - hi)), the difference exact.
 __device__ __forceinline__ void split_pair(float x0, float x1, float scale, uint32_t& hi, uint32_t& lo) {
   const float y0 = x0 * scale, y1 = x1 * scale;
@@ -77,12 +105,25 @@ __device__ __forceinline__ void split_unit(const float4& a, const float4& b, flo
 
 // The weight operand, split in the layout the MMA descriptors read.  For column group g (nt columns) and K chunk kc: the nt x 32
 // tile of B_hi followed by that of B_lo, one contiguous block of 2 * nt * 64 bytes at block index g * kc_count + kc, which a stage
-// gets by one bulk copy; behind all blocks the inverse scale of every column, nt per group.
+// gets by one bulk copy; behind all blocks the inverse scale of every column, nt per group, and the marks: words that hold kBelowPairs or
+// kWide where elements ask for it.  A writer has a word of its own for each column or each 32 x 32 elements it
+// writes, or writes them all, so that none has to be cleared beforehand; a word nobody writes stays zero.
 struct Image {
   uint8_t* data;   // NULL: no image is kept
   int nt, kc;      // column group width, K chunks
 };
 __host__ __device__ inline size_t image_blocks_bytes(int groups, int nt, int kc) { return (size_t)groups * kc * 2 * nt * kHalfRow; }
+__host__ __device__ inline int image_marks(int groups, int nt, int kc) { return max(groups * nt, kc * ((groups * nt + 31) / 32)); }
+__device__ __forceinline__ int* marks_of(const Image& im, int n) {
+  const int groups = (n + im.nt - 1) / im.nt;
+  return reinterpret_cast<int*>(im.data + image_blocks_bytes(groups, im.nt, im.kc)) + groups * im.nt;
+}
+// All marks of an image of `n` columns alike, by the threads of one block.
+__device__ __forceinline__ void put_marks(const Image& im, int n, int marks) {
+  if (im.data == nullptr) return;
+  int* const at = marks_of(im, n);
+  for (int i = threadIdx.x; i < image_marks((n + im.nt - 1) / im.nt, im.nt, im.kc); i += blockDim.x) at[i] = marks;
+}
 // One element of an image: B[k][n] = x, already scaled.  The padding of an image is zero from the start and never written.
 __device__ __forceinline__ void put_half(const Image& im, int n, int k, float x) {
   if (im.data == nullptr) return;
@@ -118,13 +159,20 @@ k_split_b(const SplitB p, int rows) {
   const float* const src = p.Bk + (long long)n * p.ldbk;
   const auto load = [&](int k) { return n < p.N && k < p.K ? *reinterpret_cast<const float4*>(src + k) : make_float4(0.f, 0.f, 0.f, 0.f); };
   float m = 0.f;
+  float least = INFINITY;   // zeros count
+  uint32_t key = 0xffffffffu;
   for (int k = lane * 4; k < p.K; k += 128) {
     const float4 v = load(k);
     m = fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
+    key = min(key, least_key(v));
+    const float size[4] = {fabsf(v.x), fabsf(v.y), fabsf(v.z), fabsf(v.w)};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) least = k + i < p.K ? fminf(least, size[i]) : least;
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
   const float scale = scale_of(m);
+  const int marks = n >= p.N ? 0 : (__any_sync(0xffffffffu, key < below_pairs(scale)) ? kBelowPairs : 0) | (__any_sync(0xffffffffu, least * scale < 0x1p-8f) ? kWide : 0);
   const int g = n / nt, r = n - g * nt;
   uint8_t* const at = p.image.data + image_blocks_bytes(g, nt, p.image.kc);
   for (int q = lane; q < units; q += 32) {
@@ -135,7 +183,10 @@ k_split_b(const SplitB p, int rows) {
     *reinterpret_cast<uint4*>(dst + (size_t)nt * kHalfRow) = lo;
   }
   const int groups = (p.N + nt - 1) / nt;
-  if (lane == 0) reinterpret_cast<float*>(p.image.data + image_blocks_bytes(groups, nt, p.image.kc))[n] = inverse_scale_of(m);
+  if (lane == 0) {
+    reinterpret_cast<float*>(p.image.data + image_blocks_bytes(groups, nt, p.image.kc))[n] = inverse_scale_of(m);
+    marks_of(p.image, p.N)[n] = marks;
+  }
 }
 
 template <int NT>
@@ -153,7 +204,117 @@ struct HalfCfg {
   static constexpr int kAccCols = kSets * 2 * NT;
   static constexpr uint32_t kTmemCols = kAccCols <= 64 ? 64 : kAccCols <= 128 ? 128 : kAccCols <= 256 ? 256 : 512;
   static constexpr size_t kSmem = (size_t)kSlots * kSlot + kEpiWarps * 4096 + NT * sizeof(float) + 1024;
+  static constexpr int kRedoStage = 2 * kATileBytes + 2 * NT * kChunkK * 4;   // a chunk of both operands as TF32 pairs
+  static_assert(2 * kRedoStage <= kSlots * kSlot && kRedoStage % 1024 == 0, "two of them lie where the slots were");
 };
+
+// Row tiles of this block whose rows may hold elements too small for a pair: bit i for its i-th tile, the last bit for all from there on.
+constexpr int kRedoBits = 2048;
+
+// Rows with elements too small for a pair, or all rows (`all`), of this block's tiles once more, by TF32 pairs: each element has an
+// exponent of its own there.  By all threads of the block, after its pipeline has come to rest; shared memory and tensor memory are the
+// pipeline's.  Which rows are stored is decided by the rows themselves, so a row's value does not depend on the others of its tile.
+// Ordinary data rarely comes here, so this is two stages between barriers and not a pipeline of its own.  us, nothing to redo / one row in
+// 100 k / every row: 256 x 256 on 169 k rows 91 / 114 / 341, on 1.2 M 603 / 646 / 2298, 256 x 47 on 1.2 M 271 / 308 / 1079 (all rows by
+// k_gemm_tc_ws's pipeline: 0.81 ms, 0.31).  False: a wait ran out.
+template <int NT>
+__device__ __noinline__ bool redo_rows(const float* __restrict__ A, int lda, const float* __restrict__ row_max, const float* __restrict__ Bk, int ldbk,
+                                       float* __restrict__ C, int ldc, int M, int N, int K, const uint32_t* marked, bool all, uint8_t* smem, uint32_t tmem_base,
+                                       uint32_t bars, volatile int* abortp) {
+  using Cfg = HalfCfg<NT>;
+  constexpr int kRows = Cfg::kThreads / 8;   // rows a turn of the block's threads covers, eight 16-byte units each
+  constexpr int kPassesA = (kBlockM + kRows - 1) / kRows, kPassesB = (NT + kRows - 1) / kRows;
+  constexpr uint32_t kBTile = NT * kChunkK * 4;
+  int* const row_marks = reinterpret_cast<int*>(smem + (size_t)Cfg::kSlots * Cfg::kSlot);   // of the tile's rows, where the epilogue's buffers were
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, unit = tid & 7;
+  const int n_tiles = (M + kBlockM - 1) / kBlockM, kc_count = (K + kChunkK - 1) / kChunkK, n0 = blockIdx.y * NT;
+  int chunk = 0;                             // chunks staged so far: stage chunk & 1, whose commits complete its barrier in turn
+  for (int tile = blockIdx.x, tile_i = 0; tile < n_tiles; tile += gridDim.x, ++tile_i) {
+    const int bit = min(tile_i, kRedoBits - 1);
+    if (!all && !(marked[bit >> 5] >> (bit & 31) & 1u)) continue;
+    const long long row0 = (long long)tile * kBlockM;
+    if (tid < kBlockM) row_marks[tid] = all;
+    float4 va[kPassesA], vb[kPassesB];   // the next chunk's elements, on their way while the one before it is multiplied
+    const auto load = [&](int kc) {
+      const int k = kc * kChunkK + unit * 4;
+      const auto at = [&](const float* p, bool in) { return in && k < K ? *reinterpret_cast<const float4*>(p + k) : make_float4(0.f, 0.f, 0.f, 0.f); };
+#pragma unroll
+      for (int i = 0; i < kPassesA; ++i) {
+        const int r = (tid >> 3) + i * kRows;
+        va[i] = at(A + (row0 + r) * lda, r < kBlockM && row0 + r < M);
+      }
+#pragma unroll
+      for (int i = 0; i < kPassesB; ++i) {
+        const int r = (tid >> 3) + i * kRows;
+        vb[i] = at(Bk + (long long)(n0 + r) * ldbk, r < NT && n0 + r < N);
+      }
+    };
+    load(0);
+    for (int kc = 0; kc < kc_count; ++kc, ++chunk) {
+      const int stage = chunk & 1;
+      const bool ok = chunk < 2 || mbar_wait_abortable(bars + 8 * stage, (uint32_t)((chunk >> 1) - 1) & 1u, abortp);
+      if (!__syncthreads_and(ok)) return false;   // and the row marks are set
+      uint8_t* const st = smem + (size_t)stage * Cfg::kRedoStage;
+      const auto put = [&](uint8_t* at, uint32_t lo_at, const float4& v) {
+        float4 h, l;
+        split_tf32(v.x, h.x, l.x); split_tf32(v.y, h.y, l.y); split_tf32(v.z, h.z, l.z); split_tf32(v.w, h.w, l.w);
+        *reinterpret_cast<float4*>(at) = h;
+        *reinterpret_cast<float4*>(at + lo_at) = l;
+      };
+#pragma unroll
+      for (int i = 0; i < kPassesA; ++i) {
+        const int r = (tid >> 3) + i * kRows;
+        if (r >= kBlockM) break;
+        if (row0 + r < M && least_key(va[i]) < below_pairs(scale_of(__ldg(row_max + row0 + r)))) row_marks[r] = 1;
+        put(st + swz(r, unit), kATileBytes, va[i]);
+      }
+#pragma unroll
+      for (int i = 0; i < kPassesB; ++i) {
+        const int r = (tid >> 3) + i * kRows;
+        if (r < NT) put(st + 2 * kATileBytes + swz(r, unit), kBTile, vb[i]);
+      }
+      if (kc + 1 < kc_count) load(kc + 1);
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncthreads();
+      if (tid == Cfg::kMmaWarp * 32) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t idesc = instr_desc(NT), a_hi = operand_desc_lo(smem_u32(st)), a_lo = a_hi + (kATileBytes >> 4);
+        const uint32_t b_hi = a_hi + (2 * kATileBytes >> 4), b_lo = b_hi + (kBTile >> 4);
+#pragma unroll
+        for (int ks = 0; ks < kChunkK / 8; ++ks) {
+          const uint32_t o = ks * 2, more = kc > 0 || ks > 0;
+          mma_tf32_lo(tmem_base + NT, a_lo + o, b_hi + o, idesc, more);
+          mma_tf32_lo(tmem_base + NT, a_hi + o, b_lo + o, idesc, 1u);
+          mma_tf32_lo(tmem_base, a_hi + o, b_hi + o, idesc, more);
+        }
+        mma_commit(bars + 8 * stage);
+      }
+    }
+    const bool ok = mbar_wait_abortable(bars + 8 * ((chunk - 1) & 1), (uint32_t)((chunk - 1) >> 1) & 1u, abortp);   // every MMA before it is done too
+    if (!__syncthreads_and(ok)) return false;
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (warp < 8) {   // two warps per quarter of the lanes, 16 columns in turn
+      const int r = (warp & 3) * 32 + lane;
+      const bool mine = row0 + r < M && row_marks[r];
+      for (int at = (warp >> 2) * 16; at < NT; at += 32) {
+        uint32_t v[16], w[16];
+        const uint32_t taddr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)at;
+        GTC_TMEM_LD16(v, taddr);
+        GTC_TMEM_LD16(w, taddr + (uint32_t)NT);
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+        for (int q = 0; q < 16; q += 4)
+          if (mine && n0 + at + q < ldc)
+            *reinterpret_cast<float4*>(C + (row0 + r) * ldc + n0 + at + q) =
+                make_float4(__uint_as_float(v[q]) + __uint_as_float(w[q]), __uint_as_float(v[q + 1]) + __uint_as_float(w[q + 1]),
+                            __uint_as_float(v[q + 2]) + __uint_as_float(w[q + 2]), __uint_as_float(v[q + 3]) + __uint_as_float(w[q + 3]));
+      }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();   // the sums and the row marks have been read
+  }
+  return true;
+}
 
 // Roles (see k_gemm_tc_ws; the waits, the abort flag and the way out are the same):
 //   copy warp   one thread: raw tile of A by a tensor copy, B's chunk by a bulk copy, into slot j mod R as soon as it is free
@@ -163,8 +324,8 @@ struct HalfCfg {
 //   epilogue    accumulators -> scales taken off -> C
 template <int NT>
 __global__ void __launch_bounds__(HalfCfg<NT>::kThreads, 1)
-k_gemm_half(const float* __restrict__ row_max, float* __restrict__ C, int ldc, int M, int N, int K, const int* __restrict__ skip,
-            int* __restrict__ error_flag, const uint8_t* __restrict__ b_image, const __grid_constant__ CUtensorMap tmap_a) {
+k_gemm_half(const float* __restrict__ A, int lda, const float* __restrict__ row_max, const float* __restrict__ Bk, int ldbk, float* C, int ldc, int M, int N,
+            int K, const int* __restrict__ skip, int* __restrict__ error_flag, const uint8_t* __restrict__ b_image, const __grid_constant__ CUtensorMap tmap_a) {
   using Cfg = HalfCfg<NT>;
   constexpr int R = Cfg::kSlots, SETS = Cfg::kSets;
   static_assert(NT <= 256 && NT % 16 == 0, "NT");
@@ -172,15 +333,17 @@ k_gemm_half(const float* __restrict__ row_max, float* __restrict__ C, int ldc, i
   if (skip != nullptr && *skip) return;
 
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t bars[3 * R + 5];           // raw[R], ready[R], empty[R], acc_full[2], acc_empty[2], drain
+  __shared__ __align__(8) uint64_t bars[3 * R + 7];           // raw[R], ready[R], empty[R], acc_full[2], acc_empty[2], drain, redo[2]
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag, copies;                          // copies: chunks whose copies have been started
+  __shared__ int redo_some, image_marked;                     // elements too small for a pair in the marked tiles; the image's marks
+  __shared__ uint32_t marked[kRedoBits / 32];                 // row tiles with elements too small for a pair
   __shared__ unsigned col_range[2];                           // bits of the largest and, inverted, of the smallest column factor
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t smem_base = smem_u32(smem);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t bar_raw = smem_u32(&bars[0]), bar_ready = smem_u32(&bars[R]), bar_empty = smem_u32(&bars[2 * R]);
-  const uint32_t bar_acc_full = smem_u32(&bars[3 * R]), bar_acc_empty = smem_u32(&bars[3 * R + 2]), bar_drain = smem_u32(&bars[3 * R + 4]);
+  const uint32_t bar_acc_full = smem_u32(&bars[3 * R]), bar_acc_empty = smem_u32(&bars[3 * R + 2]), bar_drain = smem_u32(&bars[3 * R + 4]), bar_redo = smem_u32(&bars[3 * R + 5]);
   constexpr uint32_t kSlot = (uint32_t)Cfg::kSlot, kEpiBase = (uint32_t)R * kSlot;
   float* const col_factor = reinterpret_cast<float*>(smem + kEpiBase + Cfg::kEpiWarps * 4096);   // inverse scales of this CTA's columns
 
@@ -189,10 +352,12 @@ k_gemm_half(const float* __restrict__ row_max, float* __restrict__ C, int ldc, i
     for (int r = 0; r < R; ++r) { mbar_init(bar_raw + 8 * r, 1); mbar_init(bar_ready + 8 * r, Cfg::kProdWarps); mbar_init(bar_empty + 8 * r, 1); }   // ready: one arrival per producer warp
     for (int a = 0; a < 2; ++a) { mbar_init(bar_acc_full + 8 * a, 1); mbar_init(bar_acc_empty + 8 * a, Cfg::kEpiWarps); }
     mbar_init(bar_drain, 1);
-    abort_flag = copies = 0;
+    for (int i = 0; i < 2; ++i) mbar_init(bar_redo + 8 * i, 1);
+    abort_flag = copies = redo_some = image_marked = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (tid < 2) col_range[tid] = 0u;
+  if (tid < kRedoBits / 32) marked[tid] = 0u;
   if (warp == Cfg::kMmaWarp) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)),
                  "r"(Cfg::kTmemCols)
@@ -204,9 +369,10 @@ k_gemm_half(const float* __restrict__ row_max, float* __restrict__ C, int ldc, i
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem_base = tmem_base_slot;
   volatile int* abortp = &abort_flag;
+  const float* const factors = reinterpret_cast<const float*>(b_image + image_blocks_bytes(gridDim.y, NT, kc_count));
   if (warp >= Cfg::kProdWarps && warp < Cfg::kMmaWarp) {   // the epilogue's own; it waits at a barrier of its own below
     for (int c = tid - Cfg::kProdWarps * 32; c < NT; c += Cfg::kEpiWarps * 32) {
-      const float f = reinterpret_cast<const float*>(b_image + image_blocks_bytes(gridDim.y, NT, kc_count))[blockIdx.y * NT + c];
+      const float f = factors[blockIdx.y * NT + c];
       col_factor[c] = f;
       atomicMax(&col_range[0], __float_as_uint(f));
       atomicMax(&col_range[1], ~__float_as_uint(f));
@@ -233,7 +399,13 @@ k_gemm_half(const float* __restrict__ row_max, float* __restrict__ C, int ldc, i
       }
     };
     fetch_max(0);
+    int marks = 0;         // the image's, while the first copies are under way
+    for (int i = lane; i < image_marks(gridDim.y, NT, kc_count); i += 32) marks |= __ldg(reinterpret_cast<const int*>(factors) + gridDim.y * NT + i);
+    marks = (int)__reduce_or_sync(0xffffffffu, (unsigned)marks);
+    if (tid == 0) image_marked = marks;
+    const bool look = (marks & kWide) != 0;   // always looking takes 256 x 256 on 169 k rows from 88.5 to 92.0 us, 256 x 47 on 2.45 M from 640 to 686
     float scale[GROUPS];
+    bool small = false;    // an element of this tile is too small for a pair
     int slot = 0, kc = 0, tile_i = 0;
     uint32_t raw_parity = 0;
     for (int j = 0; j < total; ++j) {
@@ -255,13 +427,22 @@ k_gemm_half(const float* __restrict__ row_max, float* __restrict__ C, int ldc, i
       for (int i = 0; i < GROUPS; ++i) {
         uint4 hi, lo;
         split_unit(a[i], b[i], scale[i], hi, lo);
+        if (look) small |= least_key(a[i], b[i]) < below_pairs(scale[i]);
         uint8_t* const at = tile + (size_t)(warp * GROUPS + i) * (2 * kHalfGroup) + swz_half(lane >> 2, u);
         *reinterpret_cast<uint4*>(at) = hi;
         *reinterpret_cast<uint4*>(at + kHalfGroup) = lo;
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       mbar_arrive_warp(bar_ready + 8 * slot);
-      if (++kc == kc_count) kc = 0;
+      if (++kc == kc_count) {
+        kc = 0;
+        if (small) {
+          const int bit = min(tile_i - 1, kRedoBits - 1);
+          atomicOr(&marked[bit >> 5], 1u << (bit & 31));
+          redo_some = 1;
+          small = false;
+        }
+      }
       if (++slot == R) { slot = 0; raw_parity ^= 1u; }
     }
   } else if (warp == Cfg::kMmaWarp + 1) {
@@ -396,7 +577,12 @@ k_gemm_half(const float* __restrict__ row_max, float* __restrict__ C, int ldc, i
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
+  const bool gave_up = __syncthreads_or(*abortp);
+  const bool all = (image_marked & kBelowPairs) != 0;
+  if (!gave_up && (all || redo_some)) {
+    redo_rows<NT>(A, lda, row_max, Bk, ldbk, C, ldc, M, N, K, marked, all, smem, tmem_base, bar_redo, abortp);
+    __syncthreads();
+  }
   if (abort_flag) {
     if (tid == 0) {
       atomicOr(error_flag, 1);

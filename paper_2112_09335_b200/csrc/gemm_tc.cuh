@@ -520,12 +520,11 @@ struct TnCfg {
 // RESID: B is not stored.  The operand is the derivative of a hidden layer's penalty with respect to
 // its pre-activation, formed while staging from the pre-activation H (passed as B) and the layer's
 // Z (Zres, same leading dimension):  b = h > 0 ? nu (h - z) : 0.
-// part_max (may be NULL): raised to the largest magnitude among the partial sums.
 template <int NT, bool RESID>
 __global__ void __launch_bounds__(kTnThreads, 1)
 k_gemm_tn_tc(const float* __restrict__ A, int lda, const float* __restrict__ B, int ldb, float* __restrict__ part, int ldp,
              long long rows, long long rows_per_split, int Ka, int Nb, int* __restrict__ error_flag,
-             const float* __restrict__ Zres, float nu, unsigned* part_max) {
+             const float* __restrict__ Zres, float nu) {
   using Cfg = TnCfg<NT, RESID>;
   constexpr int S = Cfg::kStagesTn, ROWS = Cfg::kRows, GROUP = Cfg::kGroup;
   constexpr int A_PASSES = ROWS * 32 / 256;
@@ -685,7 +684,6 @@ k_gemm_tn_tc(const float* __restrict__ A, int lda, const float* __restrict__ B, 
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const int ka = ka0 + warp * 32 + lane;
     float* dst = part + ((long long)blockIdx.y * Ka + ka) * ldp;
-    float big = 0.f;
 #pragma unroll 1
     for (int cchunk = 0; cchunk < NT / 16; ++cchunk) {
       uint32_t v[16], w[16];
@@ -701,18 +699,14 @@ k_gemm_tn_tc(const float* __restrict__ A, int lda, const float* __restrict__ B, 
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const int col = nb0 + cchunk * 16 + q * 4;
-          const float4 sum = make_float4(__uint_as_float(v[q * 4]) + __uint_as_float(w[q * 4]),
-                                         __uint_as_float(v[q * 4 + 1]) + __uint_as_float(w[q * 4 + 1]),
-                                         __uint_as_float(v[q * 4 + 2]) + __uint_as_float(w[q * 4 + 2]),
-                                         __uint_as_float(v[q * 4 + 3]) + __uint_as_float(w[q * 4 + 3]));
-          big = fmaxf(fmaxf(big, fmaxf(fabsf(sum.x), fabsf(sum.y))), fmaxf(fabsf(sum.z), fabsf(sum.w)));
-          if (col < ldp) *reinterpret_cast<float4*>(dst + col) = sum;
+          if (col < ldp)
+            *reinterpret_cast<float4*>(dst + col) =
+                make_float4(__uint_as_float(v[q * 4]) + __uint_as_float(w[q * 4]),
+                            __uint_as_float(v[q * 4 + 1]) + __uint_as_float(w[q * 4 + 1]),
+                            __uint_as_float(v[q * 4 + 2]) + __uint_as_float(w[q * 4 + 2]),
+                            __uint_as_float(v[q * 4 + 3]) + __uint_as_float(w[q * 4 + 3]));
         }
       }
-    }
-    if (part_max != nullptr) {   // magnitudes: their order is that of their bits
-      const unsigned most = __reduce_max_sync(0xffffffffu, __float_as_uint(big));
-      if (lane == 0) atomicMax(part_max, most);
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");

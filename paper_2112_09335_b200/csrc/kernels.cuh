@@ -28,10 +28,8 @@ struct SearchCtl {
   int trial;       // accepted trial index, -1 skipped, -2 exhausted
   int pass;        // passes already scored
   float inv_cand[kCand];  // 1/t of the candidates of the current pass
-  // W blocks, for the scales of the split images: largest magnitude of the gradient and of W (k_finish_grad); of the gradient's
-  // partial sums, as bits (raised by the transposed product, left at zero by k_finish_grad)
+  // W blocks, for the scale of the weights' split images: largest magnitude of the gradient and of W (k_finish_grad)
   float g_max, w_max;
-  unsigned part_max;
 };
 
 // Numbers and flags the host reads back together.
@@ -957,7 +955,7 @@ __device__ __forceinline__ void log_decision(const DecisionLog& lg, int i, const
 using WeightTile = float[32][33];
 template <typename F>
 __device__ __forceinline__ void weight_tile(int tile, int rows, int cols, int padded, WeightTile& turn, float* __restrict__ t, int ldt,
-                                            const gtc::Image& image, float scale, const gtc::Image& image_t, float scale_t, F&& value) {
+                                            const gtc::Image& image, const gtc::Image& image_t, float scale, F&& value) {
   const int x = threadIdx.x & 31, y = threadIdx.x >> 5, col_tiles = (padded + 31) / 32;
   const int r0 = tile / col_tiles * 32, c0 = tile % col_tiles * 32;
   __syncthreads();   // the tile before this one has been read
@@ -967,7 +965,7 @@ __device__ __forceinline__ void weight_tile(int tile, int rows, int cols, int pa
     if (r < rows && c < padded) {
       const float v = value(r, c);
       turn[y + k][x] = v;
-      if (c < cols) gtc::put_half(image_t, r, c, v * scale_t);
+      if (c < cols) gtc::put_half(image_t, r, c, v * scale);
     }
   }
   __syncthreads();
@@ -983,10 +981,8 @@ __device__ __forceinline__ void weight_tile(int tile, int rows, int cols, int pa
 }
 
 // Weight gradient from its split partial sums, and the start of the W_l search, in one launch:
-//   grad[e] = sum over splits of part[s][e] (fp64, in split order), its transpose for P grad, ||grad||^2, ||W||^2, and where one is
-//   kept the transpose's image, scaled by the bound splits * (largest partial sum): the split holds an element to 2^-23 of its
-//   magnitude down to 2^-29 of the bound.  `maxima`: the largest magnitudes of grad and W go to the control block, for the images of
-//   W after its move.
+//   grad[e] = sum over splits of part[s][e] (fp64, in split order), its transpose for P grad, ||grad||^2 and ||W||^2.  `maxima`: the
+//   largest magnitudes of grad and W go to the control block, for the images of W after its move.
 // SG = 1: a block owns a tile of 32 x 32 elements (grid: tiles over rows x ldp).  SG = 8 (many splits): 32 consecutive elements,
 // eight threads per element, each adding its own run of consecutive splits; the transpose is then written one
 // float at a time (a tile of 32 x 32 would leave one block where there are 32 now).  The last block to finish adds the
@@ -995,7 +991,7 @@ template <int SG>
 __global__ void __launch_bounds__(256)
 k_finish_grad(const float* __restrict__ part, int splits, int rows, int cols, int ldp, float* __restrict__ grad,
               float* __restrict__ grad_t, int ldt, const float* __restrict__ W, double* partial, unsigned* ticket,
-              SearchCtl* ctl, double shrink, double growth, int* status, const gtc::Image image, bool maxima) {
+              SearchCtl* ctl, double shrink, double growth, int* status, bool maxima) {
   gtc::enter_kernel();
   __shared__ double sh[16], s_part[SG == 1 ? 1 : SG][32];
   __shared__ WeightTile turn;
@@ -1003,9 +999,6 @@ k_finish_grad(const float* __restrict__ part, int splits, int rows, int cols, in
   const long long elems = (long long)rows * ldp;
   double sq[2] = {0.0, 0.0};   // of grad, of W
   float most[2] = {0.f, 0.f};
-  const float bound = W != nullptr && image.data != nullptr ? gtc::finite_bound((float)splits * __uint_as_float(__ldcg(&ctl->part_max))) : 0.f;
-  const float scale = gtc::scale_of(bound);
-  if (W != nullptr && blockIdx.x == 0) gtc::put_scales(image, cols, bound);
   const auto sum_splits = [&](long long e, int k0, int k1) {
     double s = 0.0;
 #pragma unroll 8
@@ -1013,7 +1006,7 @@ k_finish_grad(const float* __restrict__ part, int splits, int rows, int cols, in
     return s;
   };
   if (SG == 1) {
-    weight_tile((int)blockIdx.x, rows, cols, ldp, turn, W != nullptr ? grad_t : nullptr, ldt, image, scale, gtc::Image{nullptr, 16, 1}, 1.f, [&](int r, int c) {
+    weight_tile((int)blockIdx.x, rows, cols, ldp, turn, W != nullptr ? grad_t : nullptr, ldt, gtc::Image{nullptr, 16, 1}, gtc::Image{nullptr, 16, 1}, 1.f, [&](int r, int c) {
       const long long e = (long long)r * ldp + c;
       const float g = (float)sum_splits(e, 0, splits);
       grad[e] = g;
@@ -1039,10 +1032,7 @@ k_finish_grad(const float* __restrict__ part, int splits, int rows, int cols, in
       grad[e] = g;
       if (W != nullptr) {
         const int r = (int)(e / ldp), c = (int)(e - (long long)r * ldp);
-        if (c < cols) {
-          grad_t[(long long)c * ldt + r] = g;
-          gtc::put_half(image, c, r, g * scale);
-        }
+        if (c < cols) grad_t[(long long)c * ldt + r] = g;
         sq[0] = (double)g * (double)g;
         sq[1] = (double)w * (double)w;
         most[0] = fabsf(g);
@@ -1094,7 +1084,6 @@ k_finish_grad(const float* __restrict__ part, int splits, int rows, int cols, in
   if (threadIdx.x == 0) {
     *ticket = 0;
     if (maxima) { ctl->g_max = __uint_as_float(top.x); ctl->w_max = __uint_as_float(top.y); }
-    ctl->part_max = 0u;   // every block has read it
     begin_one(ctl, sq[0], sq[1], shrink, growth, nullptr, status);
   }
 }
@@ -1137,13 +1126,23 @@ __device__ __forceinline__ void move_w(const SearchW& p, float step) {
       gtc::put_scales(p.image, p.cols, bound);
       gtc::put_scales(p.image_t, p.rows, bound);
     }
-    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x)
-      weight_tile(tile, p.rows, p.cols, p.cols, turn, p.Wt, p.ldwt, p.image, scale, p.image_t, scale, [&](int r, int c) {
+    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+      int marks = 0;
+      weight_tile(tile, p.rows, p.cols, p.cols, turn, p.Wt, p.ldwt, p.image, p.image_t, scale, [&](int r, int c) {
         const long long e = (long long)r * p.ldw + c;
         const float w = fmaf(-p.grad[e], step, p.W[e]);
         p.W[e] = w;
+        marks |= gtc::marks_for(w, scale);
         return w;
       });
+      if (p.image.data != nullptr || p.image_t.data != nullptr) {
+        marks = (__syncthreads_or(marks & gtc::kBelowPairs) ? gtc::kBelowPairs : 0) | (__syncthreads_or(marks & gtc::kWide) ? gtc::kWide : 0);
+        if (threadIdx.x == 0) {   // a mark per tile, in both images: as many tiles in one as in the other
+          if (p.image.data != nullptr) gtc::marks_of(p.image, p.cols)[tile] = marks;
+          if (p.image_t.data != nullptr) gtc::marks_of(p.image_t, p.rows)[tile] = marks;
+        }
+      }
+    }
   }
   if (step == 0.f && p.Rn == nullptr) return;
   for (long long i = first; i < p.n4; i += stride) {
@@ -2450,13 +2449,15 @@ __global__ void k_transpose_small(const float* __restrict__ src, int lds, float*
 }
 
 // W (rows x cols, leading dimension ldw), its transpose and its images from a dense matrix whose largest finite magnitude is `bound`;
-// padding columns become zero.
+// padding columns become zero.  marks: what its elements make the marks of the images.
 __global__ void k_load_weight(const float* __restrict__ src, int rows, int cols, float* __restrict__ W, int ldw,
-                              float* __restrict__ Wt, int ldwt, const gtc::Image image, const gtc::Image image_t, float bound) {
+                              float* __restrict__ Wt, int ldwt, const gtc::Image image, const gtc::Image image_t, float bound, int marks) {
   const float scale = gtc::scale_of(bound);
   if (blockIdx.x == 0) {
     gtc::put_scales(image, cols, bound);
     gtc::put_scales(image_t, rows, bound);
+    gtc::put_marks(image, cols, marks);
+    gtc::put_marks(image_t, rows, marks);
   }
   const long long first = (long long)blockIdx.x * blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
   for (long long i = first; i < (long long)rows * ldw; i += stride) {

@@ -109,10 +109,9 @@ def test_a_weight_without_a_scale_stays_in_its_column(bad):
     assert np.array_equal(got[:, others], clean[:, others])
 
 
-def test_partial_sums_whose_bound_leaves_the_range():
-    """The image of a weight gradient is scaled by (number of partial sums) x (largest of them).  Here that product is above the
-    largest float while the gradient is finite: 64 splits of 256 rows hold 1.1e37 each in the rows of half of the features, of one
-    sign in one half of the nodes and of the other in the rest, and what is left is 7e30.  One W block, against fp32 FMA."""
+def test_partial_sums_far_above_their_gradient():
+    """64 splits of 256 rows hold 1.1e37 each in the rows of half of the features, of one sign in one half of the nodes and of the other
+    in the rest: their magnitudes add up to more than the largest float, what is left of the gradient is 7e30.  One W block, against fp32 FMA."""
     import numpy as np
     n, hidden, classes = 16384, 64, 8
     X = np.ones((n, 16), dtype=np.float32)
