@@ -245,9 +245,9 @@ int gcn_admm_shard_plan(gcn_admm* h, int n_ranks, int which, int receiver, int s
  * the first-order rows of every sender are gathered into a local matrix (on several devices that second
  * part is what the receives from the rows' owners fill), the rank's rows of A + I are renumbered to
  * positions in that local matrix, and the propagation kernel runs on those local tables alone and writes
- * the rank's rows of the result.  Entry order inside a row is kept, so a row is summed in the same order
- * as by gcn_admm_propagate (rows longer than `long_row` excepted: there the unsharded call adds partial
- * sums of pieces).  x, out: n x width, original node order, both host or both device; staged_rows (may be
+ * the rank's rows of the result.  Entry order inside a row is kept and rows longer than `long_row` are cut at
+ * the same entries, so a row is summed in the same order as by gcn_admm_propagate and comes out with the same
+ * bits.  x, out: n x width, original node order, both host or both device; staged_rows (may be
  * NULL) receives the number of copied first-order rows summed over the ranks.  Allocates per rank and
  * synchronises; a check of the plan on the device, not a fast path.  No collective is issued. */
 int gcn_admm_propagate_sharded(gcn_admm* h, int n_ranks, const float* x, int width, float* out,

@@ -1991,6 +1991,9 @@ int gcn_admm_propagate_sharded(gcn_admm* h, int n_ranks, const float* x, int wid
     const size_t rows = (size_t)h->n;
     const bool dev_in = is_device_pointer(x), dev_out = is_device_pointer(out);
     if (dev_in != dev_out) throw Fail{GCN_ADMM_ERR_ARG, "x and out must both be host or both be device pointers"};
+    // Long rows are cut into the items of the unsharded kernel, so that every row is the same sum.
+    gcn_admm_host::LongRowTables lt;
+    gcn_admm_host::build_long_row_tables(g, h->long_len, lt);
     std::vector<void*> mine;   // freed on every way out
     auto take = [&](size_t bytes) { void* q = dalloc<char>(std::max<size_t>(bytes, 16)); mine.push_back(q); return q; };
     auto release = [&] { for (void* q : mine) cudaFree(q); mine.clear(); };
@@ -2015,8 +2018,7 @@ int gcn_admm_propagate_sharded(gcn_admm* h, int n_ranks, const float* x, int wid
         }
         const int n_held = (int)held.size();
         staged += n_held - n_own;
-        // local tables: the rank's rows of A + I with columns renumbered to positions in `held`
-        // (entry order kept, so every row is summed in the order of the unsharded kernel)
+        // local tables: the rank's rows of A + I with columns renumbered to positions in `held`, entry order kept
         std::vector<int> rp((size_t)n_own + 1), order((size_t)n_own);
         const long long e0 = g.row_ptr[lo], e1 = g.row_ptr[hi];
         std::vector<int> cl((size_t)(e1 - e0));
@@ -2043,6 +2045,32 @@ int gcn_admm_propagate_sharded(gcn_admm* h, int n_ranks, const float* x, int wid
           std::memcpy(&bits, &dv[(size_t)r_], sizeof bits);
           table[(size_t)i] = make_int4(r_, rp[r_], rp[r_ + 1], bits);
         }
+        // the rank's long rows, and their items behind one another
+        const auto below = [](const gcn_admm_host::Quad& q, int row) { return q.x < row; };
+        const auto row_lo = std::lower_bound(lt.rows.begin(), lt.rows.end(), lo, below), row_hi = std::lower_bound(row_lo, lt.rows.end(), hi, below);
+        const int first_item = row_lo < row_hi ? row_lo->y : 0;
+        std::vector<int4> items, long_rows;
+        std::vector<int> item_row;
+        for (auto it = row_lo; it < row_hi; ++it) {
+          for (int k = it->y; k < it->y + it->z; ++k) {
+            const gcn_admm_host::Quad& q = lt.items[(size_t)k];
+            items.push_back(make_int4(q.x - lo, (int)(q.y - e0), (int)(q.z - e0), -1));
+            item_row.push_back((int)long_rows.size());
+          }
+          long_rows.push_back(make_int4(it->x - lo, it->y - first_item, it->z, 0));
+        }
+        const int n_items = (int)items.size(), n_long = (int)long_rows.size();
+        int4* d_items = static_cast<int4*>(take(items.size() * sizeof(int4)));
+        int4* d_long = static_cast<int4*>(take(long_rows.size() * sizeof(int4)));
+        int* d_item_row = static_cast<int*>(take(item_row.size() * sizeof(int)));
+        int* d_done = static_cast<int*>(take(long_rows.size() * sizeof(int)));
+        float* item_sums = static_cast<float*>(take(items.size() * ldw * sizeof(float)));
+        if (n_items > 0) {
+          CU(cudaMemcpyAsync(d_items, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice, h->stream));
+          CU(cudaMemcpyAsync(d_long, long_rows.data(), long_rows.size() * sizeof(int4), cudaMemcpyHostToDevice, h->stream));
+          CU(cudaMemcpyAsync(d_item_row, item_row.data(), item_row.size() * sizeof(int), cudaMemcpyHostToDevice, h->stream));
+          CU(cudaMemsetAsync(d_done, 0, long_rows.size() * sizeof(int), h->stream));
+        }
         int* d_rp = static_cast<int*>(take(rp.size() * sizeof(int)));
         int* d_cl = static_cast<int*>(take(cl.size() * sizeof(int)));
         int4* d_table = static_cast<int4*>(take(table.size() * sizeof(int4)));
@@ -2064,7 +2092,7 @@ int gcn_admm_propagate_sharded(gcn_admm* h, int n_ranks, const float* x, int wid
         }
         if (n_own > 0) {
           gcn_admm::Scope sc(h, "spmm.sharded", 1, 0.0, 0.0);
-          h->spmm_tables<4, false>(gcn_admm::GatherGraph{d_rp, d_cl, nullptr, nullptr, d_dv, d_table, nullptr, nullptr, nullptr, nullptr, n_own, 0, 0, INT_MAX, nullptr},
+          h->spmm_tables<4, false>(gcn_admm::GatherGraph{d_rp, d_cl, nullptr, nullptr, d_dv, d_table, d_items, d_long, d_item_row, d_done, n_own, n_items, n_long, h->long_len, item_sums},
                          xl, b + (size_t)lo * ldw, ldw / 4);
         }
         CU(cudaStreamSynchronize(h->stream));   // the host vectors of this rank go out of scope
