@@ -107,7 +107,8 @@ __device__ __forceinline__ void split_unit(const float4& a, const float4& b, flo
 // tile of B_hi followed by that of B_lo, one contiguous block of 2 * nt * 64 bytes at block index g * kc_count + kc, which a stage
 // gets by one bulk copy; behind all blocks the inverse scale of every column, nt per group, and the marks: words that hold kBelowPairs or
 // kWide where elements ask for it.  A writer has a word of its own for each column or each 32 x 32 elements it
-// writes, or writes them all, so that none has to be cleared beforehand; a word nobody writes stays zero.
+// writes, the first of them among these; one that marks the whole image (put_marks) sets that first word and clears the others, so that
+// whoever writes the image next, by tiles, leaves none of its marks behind.
 struct Image {
   uint8_t* data;   // NULL: no image is kept
   int nt, kc;      // column group width, K chunks
@@ -118,11 +119,11 @@ __device__ __forceinline__ int* marks_of(const Image& im, int n) {
   const int groups = (n + im.nt - 1) / im.nt;
   return reinterpret_cast<int*>(im.data + image_blocks_bytes(groups, im.nt, im.kc)) + groups * im.nt;
 }
-// All marks of an image of `n` columns alike, by the threads of one block.
+// The marks of a whole image of `n` columns, by the threads of one block.
 __device__ __forceinline__ void put_marks(const Image& im, int n, int marks) {
   if (im.data == nullptr) return;
   int* const at = marks_of(im, n);
-  for (int i = threadIdx.x; i < image_marks((n + im.nt - 1) / im.nt, im.nt, im.kc); i += blockDim.x) at[i] = marks;
+  for (int i = threadIdx.x; i < image_marks((n + im.nt - 1) / im.nt, im.nt, im.kc); i += blockDim.x) at[i] = i == 0 ? marks : 0;
 }
 // One element of an image: B[k][n] = x, already scaled.  The padding of an image is zero from the start and never written.
 __device__ __forceinline__ void put_half(const Image& im, int n, int k, float x) {

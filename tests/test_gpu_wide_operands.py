@@ -221,3 +221,27 @@ def test_hidden_gradient_with_weights_of_wide_range(spread):
     moved, error = z[:, dead] - Z1[:, dead], z_tc[:, dead] - z[:, dead]
     # sums of 64 products; in S both sides form H_2 - Z_2, from sums of 64 products as well: ten times the bound of one of them
     assert np.abs(moved).max() > 0 and np.linalg.norm(error) < 10 * bound(C2) * np.linalg.norm(moved)
+
+
+def test_a_weight_step_leaves_no_mark_of_the_weights_before_it():
+    """Weights of wide range are loaded and moved to where they are not; logits from the images the move left have the bits of those from
+    images of the same weights loaded anew."""
+    rng, X, W1, W2 = problem(4)
+    moved = W1 + 0.5 * rng.uniform(-1, 1, W1.shape) * np.sqrt(6.0 / (C0 + C1))
+    W1[:, ::7] *= 2.0 ** -40
+    Z1 = np.maximum(X @ moved, 0)
+    X, W1, W2, Z1 = f32(X, W1, W2, Z1)
+    g = trainer(X, W1, W2, nu=1.0, rho=1.0, tau0=4e4)
+    try:
+        g.set_state(binding.ST_Z, 1, Z1)
+        g.step_block(binding.PHASE_W, 1)
+        assert g.decisions()["trial_w"][0, 0] >= 0
+        W = g.get_state(binding.ST_W, 1)
+        assert np.abs(W).min() > 2.0 ** -18 * np.abs(W).max()          # no element small under either scale
+        g.set_state(binding.ST_Z, 1, Z1)                               # H_1 has to be formed anew
+        after_step = g.predict()[0]
+        g.set_state(binding.ST_W, 1, W)
+        after_load = g.predict()[0]
+    finally:
+        g.destroy()
+    assert np.array_equal(after_step, after_load)
