@@ -950,7 +950,8 @@ __device__ __forceinline__ void log_decision(const DecisionLog& lg, int i, const
 
 // Weight matrices are written in two orders at once (themselves and their transpose, a split image for either): in tiles of 32 x
 // 32 that turn through shared memory, because a column of single floats costs a memory sector per element.
-// `value(r, c)` is called once per element of the tile, padding columns included, and gives its new value; t may be NULL.
+// `value(r, c)` is called once per element of the tile, padding columns included, and gives its new value; t may be NULL.  The
+// transpose's padding columns are written too: layers of other sizes share the buffer of the gradient's.
 // Blocks of 256 threads, all of them.
 using WeightTile = float[32][33];
 template <typename F>
@@ -972,10 +973,13 @@ __device__ __forceinline__ void weight_tile(int tile, int rows, int cols, int pa
 #pragma unroll
   for (int k = 0; k < 32; k += 8) {
     const int r = r0 + x, c = c0 + y + k;
-    if (r < rows && c < cols) {
+    if (c >= cols) continue;
+    if (r < rows) {
       const float v = turn[x][y + k];
       if (t != nullptr) t[(long long)c * ldt + r] = v;
       gtc::put_half(image, c, r, v * scale);
+    } else if (t != nullptr && r < ldt) {
+      t[(long long)c * ldt + r] = 0.f;
     }
   }
 }
@@ -1032,7 +1036,11 @@ k_finish_grad(const float* __restrict__ part, int splits, int rows, int cols, in
       grad[e] = g;
       if (W != nullptr) {
         const int r = (int)(e / ldp), c = (int)(e - (long long)r * ldp);
-        if (c < cols) grad_t[(long long)c * ldt + r] = g;
+        if (c < cols) {
+          grad_t[(long long)c * ldt + r] = g;
+          if (r == rows - 1)
+            for (int pad = rows; pad < ldt; ++pad) grad_t[(long long)c * ldt + pad] = 0.f;
+        }
         sq[0] = (double)g * (double)g;
         sq[1] = (double)w * (double)w;
         most[0] = fabsf(g);

@@ -245,3 +245,31 @@ def test_a_weight_step_leaves_no_mark_of_the_weights_before_it():
     finally:
         g.destroy()
     assert np.array_equal(after_step, after_load)
+
+
+@pytest.mark.parametrize("n", [600, 5000, 20000])
+def test_a_gradient_beside_a_far_larger_one(n):
+    """Layer widths that are no multiples of four: what a W block decides does not depend on the gradient, 2^40 times as large, that another
+    layer's block has formed before it."""
+    rng = np.random.default_rng(5)
+    widths = [9, 21, 16, 3]
+    X = rng.standard_normal((n, 9)).astype(np.float32)
+    W = f32(*(rng.uniform(-1, 1, (a, b)) for a, b in zip(widths, widths[1:])))
+    Z1 = np.maximum(X @ W[0], 0) + 0.1 * rng.standard_normal((n, 21))
+    Z2 = 2.0 ** 40 * rng.standard_normal((n, 16))
+    found = []
+    for first in (None, 2):
+        g = binding.GcnAdmm(n, np.zeros(n + 1, np.int64), np.zeros(0, np.int32), X, np.zeros(n, np.int32), np.zeros(n, np.uint8), widths, 2,
+                            np.arange(n, dtype=np.int32) // ((n + 1) // 2), W, tensor_cores=2)
+        try:
+            g.set_state(binding.ST_Z, 1, Z1.astype(np.float32))
+            g.set_state(binding.ST_Z, 2, Z2.astype(np.float32))
+            if first is not None:
+                g.step_block(binding.PHASE_W, first)
+            g.step_block(binding.PHASE_W, 1)
+            d = g.decisions()
+            found.append((d["trial_w"][0, 0], d["q_w"][0, 0], g.get_state(binding.ST_W, 1)))
+        finally:
+            g.destroy()
+    (trial, q, w), (trial_after, q_after, w_after) = found
+    assert trial >= 0 and trial_after == trial and q_after == q and np.array_equal(w_after, w)
