@@ -58,7 +58,7 @@ def test_scales(handle):
 
 @pytest.mark.parametrize("spread", [20, 28])
 def test_elements_far_below_the_largest_of_their_row(handle, spread):
-    """A row and a column whose largest elements meet zeros: what is left is `spread` bits below them and still held to 2^-23 of itself."""
+    """A row and a column whose largest elements meet zeros: the sum of what is left, `spread` bits below them, is as good as any other."""
     import torch
     gen = torch.Generator(device="cuda").manual_seed(spread)
     m, n, k = 16400, 48, 64
@@ -67,9 +67,39 @@ def test_elements_far_below_the_largest_of_their_row(handle, spread):
     a[:, 0], b[0] = 2.0 ** (spread + 1), 0.0
     got = product(handle, a, b).double()
     want, size = a.double() @ b.double(), a.double().abs() @ b.double().abs()
-    # elements of A reach far below the normal ones drawn here: 2^-51 of the row's largest is what a pair can hold of them
+    # the elements of A that are smallest of all may be off by 2^-51 of the row's largest
     floor = 2.0 ** (spread + 1 - 51) * b.double().abs().sum(0)
     assert bool(((got - want).abs() <= bound(k) * size + floor).all())
+
+
+@pytest.mark.parametrize("spread", [0, 20, 26, 27, 28, 30, 34, 60, 100])
+def test_each_element_by_itself(handle, spread):
+    """Every column of B picks one element of each row of A, `spread` bits below the row's largest: no sum hides how it is held.  By halves
+    to 2^-23 down to 27 bits below, then, in rows that are formed again, by TF32 pairs to 2^-21; and half a unit (2^-24) for the sum of the pair."""
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(spread)
+    m, n, k = 16400, 48, 64
+    a = (1 + torch.rand(m, k, generator=gen, device="cuda")) * 2.0 ** -spread
+    a[:, ::3] *= -1
+    a[:, 0] = 1
+    b = torch.zeros(k, n, device="cuda")
+    b[torch.arange(1, n + 1), torch.arange(n)] = 1
+    want = a[:, 1:n + 1].double()
+    off = float(((product(handle, a, b).double() - want).abs() / want.abs()).max())
+    assert off <= (2.0 ** -23 if spread <= 27 else 2.0 ** -21) + 2.0 ** -24
+
+
+@pytest.mark.parametrize("n,k", [(8, 2048), (100, 767), (256, 256), (40, 32)])
+def test_errors_of_random_signs_do_not_add_up(handle, n, k):
+    """Root mean squares, against that of the result: after j of J matrix instructions a sum of random signs has grown to sqrt(j / J) of it,
+    and each cuts off 2^-23 of what is there (2/3 J + 1 of them in all); the pairs' errors, 2.5 x 2^-23 a term, have random signs too."""
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(k)
+    a = torch.randn(16384, k, generator=gen, device="cuda")
+    b = torch.randn(k, n, generator=gen, device="cuda")
+    want = a.double() @ b.double()
+    off = float((product(handle, a, b).double() - want).norm() / want.norm())
+    assert off < (2 / 3 * -(-k // 16) + 1 + 2.5 + 1) * 2.0 ** -23
 
 
 def test_values_without_a_scale_stay_in_their_row(handle):
