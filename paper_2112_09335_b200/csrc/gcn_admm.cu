@@ -257,7 +257,7 @@ struct gcn_admm {
   int *n_active = nullptr, *status = nullptr, *d_pass = nullptr;   // status = &report->status
   // Z scoring: units in chunks of about equally many stored entries, dealt to the warps of the grid in a fixed order
   int* d_chunk_ptr = nullptr;
-  int* d_row_order = nullptr;               // rows per community by falling length: the order of the kernels that put several rows in a warp
+  int* d_row_order = nullptr;               // rows per community by falling length, for d_row_table at create
   int4* d_row_table = nullptr;              // the same order with what those kernels want of a row (see k_spmm_sets)
   int* d_user_col = nullptr;                // the caller's row of every column; NULL on graphs of more than kUserColumns entries
   // closed-form search of the last hidden layer (gcn_admm_host::SegmentTables)

@@ -5,7 +5,7 @@
 // (exact), so is a column of B (or all of B by a bound of its elements), and each scaled element x is split into x_hi = half(x) and x_lo = half(2^11 (x - x_hi)).  Both
 // hold 11 bits and are rounded to nearest, so x_hi + 2^-11 x_lo is x to 2^-23 of its magnitude where that is 2^-13 or more, that is for
 // elements down to 2^-27 of the largest of their row; below, bits of x_lo fall under the smallest half and the element is held to
-// 2^-51 of that largest one only.  Where that could show, rows are formed by TF32 pairs instead (redo_rows): all of them where B holds
+// 2^-50 of that largest one only.  Where that could show, rows are formed by TF32 pairs instead (redo_rows): all of them where B holds
 // such an element (its image says); where B is wide, those whose row of A does (the producers look).  B is wide where an element,
 // zero included, is below 2^-8 (the largest is 2^14 or more).  Beside a B that is not, K elements held to 2^-36 (2^15 is the largest)
 // cost at most K 2^-36 2^15 against sum |a||b| >= 2^14 2^-8: K 2^-27, and with the accumulator's (K / 16 + 3.5) 2^-23 that

@@ -89,11 +89,6 @@ __device__ __forceinline__ void block_sums(double (&v)[N], double* sh) {
       for (int j = 0; j < N; ++j) v[j] += __shfl_xor_sync(0xffffffffu, v[j], o);
   }
 }
-__device__ __forceinline__ double block_sum(double v, double* sh) {
-  double a[1] = {v};
-  block_sums(a, sh);
-  return a[0];
-}
 
 // Sums over the `count` blocks that left N values each in partial[b * N + ..], by one block: warp j adds value j, lanes strided,
 // then the shuffle tree.  total[0 .. N-1] (shared memory) is valid after the barrier at the end.
@@ -200,9 +195,10 @@ __device__ __forceinline__ void finish_item(const ItemRows& ir, int unit, T* __r
 // (blockIdx.y and, past the limit of that, .z): more warps, and one slice of the operand at a time is what L2 has to hold
 // (1000 columns on 14 k rows 195 -> 142 us).  Lane t of a group of 32
 // stored entries holds column and weight of entry t, handed to the warp by shuffles.  UN neighbours in flight per
-// lane: the kernel is bound by what L1 and L2 deliver of the gathered rows (about a third of the bytes are L1 hits on the hub rows of
-// a community: with loads that do not allocate in L1 10.4 instead of 6.8 ms, 2.45 M rows at 256 columns) and by how the compiler
-// orders its loads (the plain loop is faster than one that fetches columns ahead: 118 against 143 us at 128 columns on 169 k rows).
+// lane: the kernel is bound by load latency at what its 40 or so resident warps keep in flight (256 columns, 47 entries a row: half of
+// the L2-to-SM fabric's peak, L2 58 %, issue slots 46 %; 128 columns, 15 a row: 28, 35 and 54 %), on operands far larger than L2 by DRAM.
+// 11 % of the sectors are L1 hits, and yet loads that do not allocate there take 10.4 instead of 6.8 ms (2.45 M rows at 256 columns).
+// How the compiler orders the loads counts for as much (the plain loop is faster than one that fetches columns ahead: 118 against 143 us at 128 columns on 169 k rows).
 // The bound of 21 blocks gives the 40 registers of 24 and an order of loads that the row maxima at the end do not disturb: 6.81 ms with
 // them, 6.75 without; under a bound of 24 blocks 8.78.  With ReLU on the gathered rows it is a bound of 20 (9.0 against 9.4 ms).
 template <int VEC, int NV, int UN, bool MAPPED, bool SLICED, bool RELU>
@@ -1352,7 +1348,8 @@ k_zgrad_finish(float4* __restrict__ G, const float4* __restrict__ Z, const float
 // their own, so that G is written once and not read again (three launches and G through memory three times otherwise).  fp32 FMA.
 // W^T lies in shared memory, 4 KV rows of ld4 float4 (those past the layer's width zero).  Eight lanes take R rows of G, so that a
 // value of W serves R; shared memory is read 4 KV times per R float4 of G for each product, which with the registers of a row's S
-// and T is what bounds it where HBM does not (see the rule in update_Z_hidden).
+// and T is what bounds it where HBM does not (see joins_products).  At KV = 12 these do not fit: 255 registers and 540 bytes of spills, on
+// graphs of up to 4,096 rows only.
 template <int KV, int R>
 __global__ void __launch_bounds__(256 / R)
 k_zgrad_products(float4* __restrict__ G, const float4* __restrict__ Z, const float4* __restrict__ H, const float4* __restrict__ S,
