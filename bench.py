@@ -37,15 +37,15 @@ SM_COUNT = 148
 
 # DRAM bytes (read + write) per stored entry of A + I moved by one launch of the propagation at leading dimension
 # 256, from ncu (dram__bytes_read.sum + dram__bytes_write.sum) on this workload's recipe.  FULL: a one-pass capture
-# of a launch at full size (126,404,737 stored entries); SCALED: a capture at scale 0.25 (30,189,629 stored entries),
+# of a launch at full size (126,404,737 stored entries); SCALED: a capture at scale 0.1 (11,551,755 stored entries),
 # used for other sizes in proportion to the stored entries (the share of neighbour rows that miss L2 grows with
-# the size, so scaling up from 0.25 understates the traffic).
+# the size, so scaling up from 0.1 understates the traffic).
 NCU_SPMM256 = dict(
-    scaled=dict(dram_bytes=5066328832.0 + 715988992.0, nnz=30189629, scale=0.25),
-    full=dict(dram_bytes=34.20e9 + 3.03e9, nnz=126404737),
+    scaled=dict(dram_bytes=1460091904.0 + 271882752.0, nnz=11551755, scale=0.1),
+    full=dict(dram_bytes=34.22e9 + 3.04e9, nnz=126404737),
 )
-# SM-to-L2 fabric: ncu reports l1tex__m_xbar2l1tex_read_bytes at 51.2 % of its peak for 29.15 GB in 1.578 ms at
-# 1.906 GHz, i.e. a peak of 128 bytes per clock per SM
+# SM-to-L2 fabric: ncu reports l1tex__m_xbar2l1tex_read_bytes at 50.8 % of its peak for 11.06 GB in 0.616 ms, i.e. a
+# peak of 35.3 TB/s: 128 bytes per clock per SM at 1.86 GHz
 XBAR_BYTES_PER_CLK_PER_SM = 128.0
 
 
