@@ -185,7 +185,8 @@ k_split_b(const SplitB p, int rows) {
   }
   const int groups = (p.N + nt - 1) / nt;
   if (lane == 0) {
-    reinterpret_cast<float*>(p.image.data + image_blocks_bytes(groups, nt, p.image.kc))[n] = inverse_scale_of(m);
+    // a column of zeros, padding among them, takes any: 1 joins with the factor of every row that others join with
+    reinterpret_cast<float*>(p.image.data + image_blocks_bytes(groups, nt, p.image.kc))[n] = m > 0.f ? inverse_scale_of(m) : 1.f;
     marks_of(p.image, p.N)[n] = marks;
   }
 }
