@@ -511,7 +511,7 @@ struct gcn_admm {
   void split_b(const gtc::SplitB& b) {
     const int rows = (int)(cdiv(b.N, b.image.nt) * b.image.nt);
     Scope sc(this, "split_b", 1, 8.0 * (double)b.N * b.K, 0.0);
-    launch(gtc::k_split_b, (unsigned)cdiv(rows, 8), 256, 0, b, rows);
+    launch(gtc::k_split_b, (unsigned)cdiv(rows, gtc::kSplitColumns), 256, 0, b, rows);
     CU(cudaGetLastError());
   }
 
