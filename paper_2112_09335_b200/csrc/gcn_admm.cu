@@ -2,7 +2,6 @@
 // kernels.cuh.  See include/gcn_admm.h for the contract of every entry point.
 #include "../../include/gcn_admm.h"
 
-#include <cfloat>
 #include <climits>
 #include <cmath>
 #include <cuda_runtime.h>
@@ -1166,21 +1165,13 @@ struct gcn_admm {
     CU(stage.put(grad, host_w, sizeof(float) * (size_t)r * c, stream));
     CU(stage.finish(stream));
     const long long cells = std::max((long long)r * ld[l], (long long)c * ld[l - 1]);
-    float most = 0.f, least = FLT_MAX;
-    int zeros = 0;
+    gk::WeightRange* const ranges = reinterpret_cast<gk::WeightRange*>(red_part);
+    int n_ranges = 0;
     if (img_H[l].data != nullptr || img_G[l].data != nullptr) {
-#pragma omp simd reduction(max : most) reduction(min : least) reduction(| : zeros)
-      for (long long e = 0; e < (long long)r * c; ++e) {   // of the finite elements: an infinity or NaN stays in its column
-        const float size = std::fabs(host_w[e]);
-        most = size <= FLT_MAX ? std::max(most, size) : most;
-        least = size > 0.f ? std::min(least, size) : least;
-        zeros |= size == 0.f;
-      }
+      n_ranges = (int)std::min<long long>(kSmCount, cdiv((long long)r * c, 256));
+      gk::k_weight_range<<<n_ranges, 256, 0, stream>>>(grad, (long long)r * c, ranges);
     }
-    // most is scaled to 2^14 at least: elements below 2^-27 of it may be too small for a pair, below 2^-22 they make the matrix wide
-    const int marks = ((double)least < std::ldexp((double)most, -27) || least < FLT_MIN ? gtc::kBelowPairs : 0) |
-                      (zeros || (double)least < std::ldexp((double)most, -22) ? gtc::kWide : 0);
-    gk::k_load_weight<<<grid_for(cells), 256, 0, stream>>>(grad, r, c, W[l], ld[l], Wt[l], ld[l - 1], img_H[l], img_G[l], most, marks);
+    gk::k_load_weight<<<grid_for(cells), 256, 0, stream>>>(grad, r, c, W[l], ld[l], Wt[l], ld[l - 1], img_H[l], img_G[l], ranges, n_ranges);
     CU(cudaGetLastError());
   }
   // Step parameters (t_prev) of `count` searches in a row, to and from the host.

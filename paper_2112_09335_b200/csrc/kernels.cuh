@@ -2453,12 +2453,55 @@ __global__ void k_transpose_small(const float* __restrict__ src, int lds, float*
   dst[c * ldd + r] = src[r * lds + c];
 }
 
-// W (rows x cols, leading dimension ldw), its transpose and its images from a dense matrix whose largest finite magnitude is `bound`;
-// padding columns become zero.  marks: what its elements make the marks of the images.
-__global__ void k_load_weight(const float* __restrict__ src, int rows, int cols, float* __restrict__ W, int ldw,
-                              float* __restrict__ Wt, int ldwt, const gtc::Image image, const gtc::Image image_t, float bound, int marks) {
-  const float scale = gtc::scale_of(bound);
+// What the images of a weight matrix are scaled and marked by: {largest finite magnitude, smallest above zero, both as bits, whether there is
+// a zero}.  An infinity or NaN stays in its column of the product under any scale and counts for nothing.
+struct WeightRange {
+  unsigned most, least;
+  int zero, pad;
+};
+// All threads of a block of 256: the range of what they hold.
+__device__ __forceinline__ WeightRange block_range(WeightRange w) {
+  __shared__ WeightRange s_range[8];
+  w.most = __reduce_max_sync(0xffffffffu, w.most);
+  w.least = __reduce_min_sync(0xffffffffu, w.least);
+  w.zero = __any_sync(0xffffffffu, w.zero);
+  if ((threadIdx.x & 31) == 0) s_range[threadIdx.x >> 5] = w;
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    w.most = max(w.most, s_range[k].most);
+    w.least = min(w.least, s_range[k].least);
+    w.zero |= s_range[k].zero;
+  }
+  return w;
+}
+constexpr unsigned kLargestBits = 0x7f7fffffu;   // of FLT_MAX
+// One range per block of at most 256, added up by k_load_weight (on the host, before: 64,000 elements 51 to 118 us).
+__global__ void __launch_bounds__(256)
+k_weight_range(const float* __restrict__ src, long long count, WeightRange* __restrict__ out) {
+  WeightRange w{0u, kLargestBits, 0, 0};
+#pragma unroll 4
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (long long)gridDim.x * blockDim.x) {
+    const unsigned size = __float_as_uint(src[i]) & 0x7fffffffu;
+    w.most = max(w.most, size <= kLargestBits ? size : 0u);
+    w.least = min(w.least, size > 0u ? size : kLargestBits);
+    w.zero |= size == 0u;
+  }
+  w = block_range(w);
+  if (threadIdx.x == 0) out[blockIdx.x] = w;
+}
+
+// W (rows x cols, leading dimension ldw), its transpose and its images from a dense matrix; padding columns become zero.  ranges:
+// what k_weight_range left of it, where an image is kept.
+__global__ void __launch_bounds__(256)
+k_load_weight(const float* __restrict__ src, int rows, int cols, float* __restrict__ W, int ldw,
+              float* __restrict__ Wt, int ldwt, const gtc::Image image, const gtc::Image image_t, const WeightRange* __restrict__ ranges, int n_ranges) {
+  const WeightRange own = (int)threadIdx.x < n_ranges ? ranges[threadIdx.x] : WeightRange{0u, kLargestBits, 0, 0}, range = block_range(own);
+  const float bound = __uint_as_float(range.most), least = __uint_as_float(range.least), scale = gtc::scale_of(bound);
   if (blockIdx.x == 0) {
+    // the bound is scaled to 2^14 at least: elements below 2^-27 of it may be too small for a pair, below 2^-22 they make the matrix wide
+    const int marks = ((double)least < (double)bound * 0x1p-27 || least < FLT_MIN ? gtc::kBelowPairs : 0) |
+                      (range.zero || (double)least < (double)bound * 0x1p-22 ? gtc::kWide : 0);
     gtc::put_scales(image, cols, bound);
     gtc::put_scales(image_t, rows, bound);
     gtc::put_marks(image, cols, marks);

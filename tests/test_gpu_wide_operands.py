@@ -171,6 +171,24 @@ def test_predictions_with_units_near_dead(spread, loaded):
     assert np.max(np.abs(got - want) / size) < FORWARD
 
 
+@pytest.mark.parametrize("at", [0, 255, 148 * 256 - 1, 148 * 256, 200 * 256 - 1])
+def test_one_large_weight_anywhere(at):
+    """The scale of a layer's weights comes from one element of 51,200 (148 blocks of 256 look at them), 2^30 above the others."""
+    rng = np.random.default_rng(6)
+    X, W1, W2 = rng.standard_normal((N, 200)), rng.uniform(-1, 1, (200, 256)), rng.uniform(-1, 1, (256, 16))
+    W1.flat[at] = 2.0 ** 30
+    X[:, at // 256] *= 2.0 ** -30
+    X, W1, W2 = f32(X, W1, W2)
+    g = binding.GcnAdmm(N, np.zeros(N + 1, np.int64), np.zeros(0, np.int32), X, np.zeros(N, np.int32), np.zeros(N, np.uint8), [200, 256, 16], 2,
+                        np.arange(N, dtype=np.int32) // (N // 2), [W1, W2])
+    try:
+        got = g.predict()[0].astype(np.float64)
+    finally:
+        g.destroy()
+    want, size = forward(X, W1, W2)
+    assert np.max(np.abs(got - want) / size) < bound(200) + bound(256)
+
+
 @pytest.mark.parametrize("spread", SPREADS)
 def test_weight_step_with_units_near_dead(spread):
     """Gradient columns and weight columns 2^-spread of the others: the W_1 block moves H_1 by the product with the gradient and leaves images
